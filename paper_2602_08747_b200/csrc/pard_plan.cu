@@ -1301,12 +1301,6 @@ __device__ __forceinline__ SegVal unpack_val(unsigned long long w) {
   return a;
 }
 
-/* X = deadline - A of a request from its deadline offset: offsets of a queue served high
- * budget first count down from the ctx's largest deadline, and A_rel is that deadline - A */
-__device__ __forceinline__ long long slack_of(unsigned long long off, const PardSegConst& K) {
-  return (K.narrow & kSegHighFirst) ? K.A_rel - (long long)off : (long long)off - K.A_rel;
-}
-
 /* First half of the decision pass for one thread's kDecItems consecutive
  * sorted elements: decode, admission threshold u, position r inside the own
  * queue, and the thread's running segmented reduction (admitted mode: minimum
@@ -3261,6 +3255,18 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   if (rc != PARD_OK) return rc;
   const uint4* req4 = (const uint4*)d_requests;
 
+  /* the decision by a walk of every queue (pard_policy.cu), between the sort and the outputs */
+  auto decide_by_walk = [&](PolicyArgs& pa) -> int {
+    pa.rounds = win_cnt; pa.tail = win_off; pa.tile_x = (uint32_t*)tile_carry;
+    pa.out_keep = out->d_keep; pa.out_est = (long long*)out->d_est_us; pa.out_perm = out->d_perm;
+    pa.out_kept_idx = out->d_kept_idx; pa.kept_base = kept_base; pa.seg_kept = seg_kept;
+    int wrc = launch_policy_walk(pa, stream);
+    if (wrc != PARD_OK) return wrc;
+    launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
+               (unsigned long long*)out->d_n_kept);
+    return launch_policy_emit(pa, stream);
+  };
+
   /* ---- keys wider than one sort element: see k_wide_reset.  Run only when a finished call has
    * reported that width (the host cannot know the deadline span beforehand), hence not for
    * PARD_MODE_NOWAIT, whose caller gets PARD_ERANGE from pard_plan_status as before. ---- */
@@ -3310,17 +3316,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     pa.n = n32; pa.ibits = ibits; pa.n_seg = L.n_seg; pa.mode = mode;
     pa.ktab = ktab; pa.seg_off = seg_off; pa.req = req4; pa.arrivals = d_arrivals;
     pa.pipes = pipe_table; pa.n_pipelines = n_pipelines; pa.st = *state;
-    pa.out_keep = out->d_keep; pa.out_est = (long long*)out->d_est_us; pa.out_perm = out->d_perm;
-    pa.kept_tmp = out->d_kept_idx ? kept_tmp : nullptr; pa.seg_kept = seg_kept;
-    int wrc = launch_policy_decision(pa, sms, stream);
+    const int wrc = decide_by_walk(pa);
     if (wrc != PARD_OK) return wrc;
-    launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
-               (unsigned long long*)out->d_n_kept);
-    if (out->d_kept_idx)
-      launch_pdl(k_kept_move, std::min<uint32_t>(((uint32_t)((n + kCompactChunk - 1) / kCompactChunk) + L.n_seg + 7) / 8,
-                                                 (uint32_t)sms * 8), 256, 0, stream,
-                 kept_tmp, seg_off, seg_kept, kept_base, chunk_base, L.n_seg, out->d_kept_idx);
-    PARD_CUDA_OK(cudaGetLastError());
     return pard_plan_status(d_workspace, cuda_stream);
   };
 
@@ -3495,10 +3492,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     pa.n = n32; pa.ibits = ibits; pa.n_seg = L.n_seg; pa.mode = mode;
     pa.ktab = ktab; pa.seg_off = seg_off; pa.req = req4; pa.arrivals = d_arrivals;
     pa.pipes = pipe_table; pa.n_pipelines = n_pipelines; pa.st = *state;
-    pa.out_keep = out->d_keep; pa.out_est = (long long*)out->d_est_us; pa.out_perm = out->d_perm;
-    pa.kept_tmp = out->d_kept_idx ? kept_tmp : nullptr; pa.seg_kept = seg_kept;
     mark();
-    rc = launch_policy_decision(pa, sms, stream);
+    rc = decide_by_walk(pa);
     if (rc != PARD_OK) return rc;
   } else if (n > 0) {
     uint32_t* tmp = out->d_kept_idx ? kept_tmp : nullptr;
@@ -3530,14 +3525,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   }
   if (n == 0) mark();
   mark();
-  if (rule_walk || n == 0) {                       /* the queue walk leaves per-queue lists; an empty call still owes its zeros */
+  if (n == 0)                                      /* an empty call still owes its zeros */
     launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
                (unsigned long long*)out->d_n_kept);
-    if (n > 0 && out->d_kept_idx)
-      launch_pdl(k_kept_move, std::min<uint32_t>(((uint32_t)((n + kCompactChunk - 1) / kCompactChunk) + L.n_seg + 7) / 8,
-                                                 (uint32_t)sms * 8), 256, 0, stream,
-          kept_tmp, seg_off, seg_kept, kept_base, chunk_base, L.n_seg, out->d_kept_idx);
-  }
   mark();
   PARD_CUDA_OK(cudaGetLastError());
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;

@@ -103,6 +103,12 @@ __device__ __forceinline__ uint32_t threshold_u(int64_t X, const PardSegConst& K
   return u > kUClamp ? kUClamp : (uint32_t)u;
 }
 
+/* X = deadline - A of a request from its deadline offset: offsets of a queue served high
+ * budget first count down from the ctx's largest deadline, and A_rel is that deadline - A */
+__device__ __forceinline__ long long slack_of(unsigned long long off, const PardSegConst& K) {
+  return (K.narrow & kSegHighFirst) ? K.A_rel - (long long)off : (long long)off - K.A_rel;
+}
+
 /* 32 bytes with one access; p is 32-byte aligned */
 __device__ __forceinline__ void load4(const unsigned long long* p, unsigned long long* v) {
   asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];"
@@ -130,13 +136,20 @@ struct PolicyArgs {
   PipeTable pipes;
   uint32_t n_pipelines;
   pard_queue_state_t st;
+  uint32_t* rounds;               /* [n_seg] batch rounds the walk has closed */
+  uint32_t* tail;                 /* [n_seg] Nexus: requests of the last, partly filled window */
+  uint32_t* tile_x;               /* [tiles of kDecTile] kept requests ahead of the tile's first one, in its queue */
   uint8_t* out_keep;
   long long* out_est;
   uint32_t* out_perm;
-  uint32_t* kept_tmp;
+  uint32_t* out_kept_idx;
+  const uint32_t* kept_base;      /* [n_seg] output offset of every queue's survivors, known after the walk */
   uint32_t* seg_kept;
 };
-int launch_policy_decision(const PolicyArgs& a, int sms, cudaStream_t stream);
+/* thresholds and walk: every queue's rounds and kept count (seg_kept) */
+int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream);
+/* estimates, flags, order and survivors, once the output offsets are known */
+int launch_policy_emit(const PolicyArgs& a, cudaStream_t stream);
 
 }  // namespace pard_plan_detail
 

@@ -7,19 +7,21 @@
  *   - in arrival order (Table 1 and Sec. 5.3, PARD-FCFS);
  *   - for Clipper++'s per-module share of the objective (Sec. 5.1, Baseline), arrival order;
  *   - for Nexus' window scan (Sec. 5.1, Baseline), a rule of its own.
- * For the first three the loop is  x <- x + [x < u_r]  with u_r the number of requests that may
- * be admitted ahead of or at r while r still makes its (own) deadline; x is the admitted count.
- * Three kernels over the sorted elements:
- *   k_policy_terms   every request on its own: gathers the request (and its arrival record),
- *                    computes u_r (Nexus: the number of batch rounds r still fits)    -> T[n]
- *   k_policy_walk    one warp per queue walks T in queue order, 32 requests per step: the
- *                    admitted positions of a step are the fixed point of
- *                    keep_i = [x + #kept among lanes below i < u_i], found by iterating from
- *                    "all kept" (bit i is final after i + 1 rounds; a few rounds in practice)
- *                                                                      -> C[n] = position | keep << 31
- *   k_policy_emit    every request on its own again: estimate from its position, outputs,
- *                    survivor lists
- * T and C live in the sort buffer that does not hold the elements. */
+ * For the first three the loop is  x <- x + [x < u_r]  with x the admitted count and u_r a multiple
+ * of the batch round's size: u_r = cap * v_r, v_r the number of rounds r still fits.  So r is
+ * admitted iff floor(x / cap) < v_r, and while one round fills up -- until cap more requests are
+ * admitted -- the test is the same for every request: v_r > b, b the number of the round.  A walk
+ * is therefore a chain of rounds, not of requests: in round b, count the requests with v_r > b
+ * until there are cap of them, which any number of threads can do side by side.  Nexus' scan has
+ * the same shape (find the first cap consecutive requests with v_r > b).
+ *   k_policy_terms   every request on its own: v_r                                -> T[n]
+ *   k_policy_walk    a group of threads per queue (16 requests each and step) closes round after
+ *                    round; round b's end goes to C[first position of the queue + b]
+ *   k_policy_emit    every request on its own again: its round by a search in the ends, estimate,
+ *                    decision, survivors straight to their final place
+ * T and C live in the sort buffer that does not hold the elements.
+ * Nexus on 16 queues of 2^20 requests: the walk takes 0.2 ms where one warp per queue, 32 requests
+ * per step, took 23.8 ms. */
 #include "pard_plan_internal.cuh"
 
 using namespace pard_plan_detail;
@@ -29,15 +31,15 @@ namespace {
 constexpr int kPolThreads = 128;
 constexpr int kPolItems = 8;
 constexpr int kPolTile = kPolThreads * kPolItems;
-constexpr int kStageSegs = 4;            /* queues whose path sums a block keeps in shared memory */
+constexpr int kStageSegs = 16;           /* queues whose path sums a block keeps in shared memory */
 constexpr int kMaskPaths = 16;           /* bits of pard_request_t.flags */
-constexpr uint32_t kKeepBit = 0x80000000u;
 
 struct SortedView {
   const unsigned long long* src;
   uint32_t* T;
   uint32_t* C;
   uint32_t kshift, imask;
+  unsigned long long dmask;
 };
 
 __device__ __forceinline__ SortedView sorted_view(const PolicyArgs& a) {
@@ -49,6 +51,7 @@ __device__ __forceinline__ SortedView sorted_view(const PolicyArgs& a) {
   v.C = spare + a.n;                     /* 8 bytes per request: two 32-bit arrays */
   v.kshift = a.ibits + a.hdr->dbits;
   v.imask = (1u << a.ibits) - 1;
+  v.dmask = a.hdr->dbits >= 64 ? ~0ull : ((1ull << a.hdr->dbits) - 1);
   return v;
 }
 
@@ -78,10 +81,13 @@ struct StagedPaths {
   uint32_t seg0;
 };
 
-__device__ void stage_paths(const PolicyArgs& a, uint32_t seg0, StagedPaths& sp) {
+__device__ void stage_paths(const PolicyArgs& a, const SortedView& v, uint64_t tile0, StagedPaths& sp) {
   const uint32_t S = (uint32_t)a.st.stage_stride;
+  const uint64_t end = tile0 + kPolTile < a.n ? tile0 + kPolTile : a.n;
+  const uint32_t seg0 = (uint32_t)(v.src[tile0] >> v.kshift);
+  const uint32_t segs = (uint32_t)(v.src[end - 1] >> v.kshift) - seg0 + 1;
   if (threadIdx.x == 0) sp.seg0 = seg0;
-  for (uint32_t t = threadIdx.x; t < kStageSegs * kMaskPaths; t += blockDim.x) {
+  for (uint32_t t = threadIdx.x; t < min(segs, (uint32_t)kStageSegs) * kMaskPaths; t += blockDim.x) {
     const uint32_t q = t / kMaskPaths, j = t % kMaskPaths, seg = seg0 + q;
     if (seg >= a.n_seg) { if (j == 0) sp.n_paths[q] = 0; continue; }
     const uint32_t c = seg / S, k = seg % S;
@@ -97,62 +103,31 @@ __device__ void stage_paths(const PolicyArgs& a, uint32_t seg0, StagedPaths& sp)
   __syncthreads();
 }
 
-/* What the rule needs of one request: with A the completion estimate at admitted position 0 and
- * D the instant it is compared with, the request at admitted position c completes (by the rule's
- * own account) at A + floor(c / cap) * d and is kept iff that is <= D. */
-struct Terms {
-  long long A, D;
-};
-
-__device__ Terms request_terms(const PolicyArgs& a, const StagedPaths& sp, uint32_t seg, uint32_t idx,
-                               const PardSegConst& K) {
-  Terms t;
-  const uint4 r = __ldg(&a.req[idx]);
-  t.D = (long long)(((unsigned long long)r.y << 32) | r.x);
-  t.A = K.A;
-  if (a.mode & (PARD_MODE_NEXUS | PARD_MODE_CLIPPER)) t.A = K.A - K.lsub;     /* the current module only: base + d */
-  if (a.mode & PARD_MODE_CLIPPER) {
-    /* the module's share of the request's objective, counted from its arrival at the module; the
-     * request is kept iff its batch starts within the share: start <= arrive + share, i.e.
-     * start + d <= arrive + share + d */
-    const pard_arrival_t ar = a.arrivals[idx];
-    long long share = 0;
-    if (ar.arrive_us < 0 || ar.arrive_us >= PARD_TIME_LIMIT_US || ar.slo_us < 0 || ar.slo_us >= (1ll << 31) ||
-        K.d >= (1ll << 32)) {
-      set_status(a.hdr, PARD_EDATA);
-      t.D = 0;
-    } else {
-      share = (long long)((unsigned long long)ar.slo_us * (unsigned long long)K.d / (unsigned long long)K.dsum);
-      t.D = ar.arrive_us + share + K.d;
-    }
+/* The downstream estimate of a request whose path is known: the maximum over the paths its mask
+ * names; K.lsub when the mask names none of the stage's (input error) or the stage is a sink. */
+__device__ long long masked_lsub(const PolicyArgs& a, const StagedPaths& sp, uint32_t seg, uint32_t flags,
+                                 const PardSegConst& K) {
+  const uint32_t q = seg - sp.seg0;
+  long long best = -1;
+  int32_t np;
+  if (q < (uint32_t)kStageSegs) {
+    np = sp.n_paths[q];
+    for (int32_t j = 0; j < np && j < kMaskPaths; ++j)
+      if ((flags >> j) & 1u) best = sp.sum[q][j] > best ? sp.sum[q][j] : best;
+  } else {                                       /* a queue beyond the staged ones: straight from the tables */
+    const uint32_t S = (uint32_t)a.st.stage_stride, c = seg / S, k = seg % S;
+    const PardPipeDev* p = pipe_of(a, c);
+    const int32_t s0 = p->stage_slot_off[k];
+    np = p->stage_slot_off[k + 1] - s0;
+    for (int32_t j = 0; j < np && j < kMaskPaths; ++j)
+      if ((flags >> j) & 1u) {
+        const long long v = path_sum(a, p, c, s0 + j);
+        best = v > best ? v : best;
+      }
   }
-  const uint32_t flags = r.w >> 16;
-  if ((a.mode & PARD_MODE_PATH_MASK) && flags != 0 && !(K.narrow & kSegNoStage)) {
-    /* the request's downstream path is known: the maximum runs over the named paths only */
-    const uint32_t q = seg - sp.seg0;
-    long long best = -1;
-    int32_t np;
-    if (q < (uint32_t)kStageSegs) {
-      np = sp.n_paths[q];
-      for (int32_t j = 0; j < np && j < kMaskPaths; ++j)
-        if ((flags >> j) & 1u) best = sp.sum[q][j] > best ? sp.sum[q][j] : best;
-    } else {                                     /* a queue beyond the staged ones: straight from the tables */
-      const uint32_t S = (uint32_t)a.st.stage_stride, c = seg / S, k = seg % S;
-      const PardPipeDev* p = pipe_of(a, c);
-      const int32_t s0 = p->stage_slot_off[k];
-      np = p->stage_slot_off[k + 1] - s0;
-      for (int32_t j = 0; j < np && j < kMaskPaths; ++j)
-        if ((flags >> j) & 1u) {
-          const long long v = path_sum(a, p, c, s0 + j);
-          best = v > best ? v : best;
-        }
-    }
-    if (np > 0) {                                /* a sink has nothing downstream whatever the mask says */
-      if (best < 0) set_status(a.hdr, PARD_EDATA);   /* the mask names no path of this stage */
-      else t.A = K.A - K.lsub + best;
-    }
-  }
-  return t;
+  if (np <= 0) return K.lsub;                    /* a sink has nothing downstream whatever the mask says */
+  if (best < 0) { set_status(a.hdr, PARD_EDATA); return K.lsub; }   /* the mask names no path of this stage */
+  return best;
 }
 
 /* number of batch rounds b for which a request still fits, b < v: Nexus tests "base + b*d + d <= D" */
@@ -164,167 +139,474 @@ __device__ __forceinline__ uint32_t rounds_fit(long long X, const PardSegConst& 
   return q >= kUClamp ? kUClamp : (uint32_t)q + 1;
 }
 
+/* One request's rounds and, for PARD_MODE_PATH_MASK, its own downstream estimate. */
 __global__ void __launch_bounds__(kPolThreads)
 k_policy_terms(const PolicyArgs a) {
   pdl_wait();
   __shared__ StagedPaths sp;
   if (a.hdr->wide || a.hdr->aborted) return;
   const SortedView v = sorted_view(a);
+  const bool lookup = a.hdr->lookup != 0;
   const uint64_t tile0 = (uint64_t)blockIdx.x * kPolTile;
-  if (a.mode & PARD_MODE_PATH_MASK) stage_paths(a, (uint32_t)(v.src[tile0] >> v.kshift), sp);
-  else if (threadIdx.x == 0) sp.seg0 = 0;
-  for (int i = 0; i < kPolItems; ++i) {
-    const uint64_t j = tile0 + (uint64_t)i * kPolThreads + threadIdx.x;
-    if (j >= a.n) break;
-    const unsigned long long e = v.src[j];
-    const uint32_t seg = (uint32_t)(e >> v.kshift), idx = (uint32_t)e & v.imask;
-    const PardSegConst K = a.ktab[seg];
-    if (K.narrow & kSegNoStage) { set_status(a.hdr, PARD_EDATA); v.T[j] = 0; continue; }
-    const Terms t = request_terms(a, sp, seg, idx, K);
-    v.T[j] = (a.mode & PARD_MODE_NEXUS) ? rounds_fit(t.D - t.A, K) : threshold_u(t.D - t.A, K);
-  }
-}
-
-/* One warp per queue.  General rule: x <- x + [x < u_r]. */
-__device__ void walk_admit(const uint32_t* __restrict__ T, uint32_t* __restrict__ C, uint32_t lo, uint32_t hi,
-                           uint32_t lane, uint32_t* kept_out, bool raw) {
-  const uint32_t below = (1u << lane) - 1;
-  uint32_t x = 0;
-  if (raw) {
-    /* every queued request ahead takes a batch slot: a request is kept iff its own queue position
-     * is below its threshold, whatever happened before it; what is walked is only the count of
-     * kept requests ahead (the survivor's slot) */
-    for (uint32_t b0 = lo; b0 < hi; b0 += 32) {
-      const uint32_t j = b0 + lane;
-      const bool keep = j < hi && (j - lo) < T[j];
-      const uint32_t m = __ballot_sync(0xffffffffu, keep);
-      if (j < hi) C[j] = (x + __popc(m & below)) | (keep ? kKeepBit : 0u);
-      x += __popc(m);
-    }
-    *kept_out = x;
-    return;
-  }
-  constexpr int kAhead = 4;                        /* steps whose thresholds are requested together */
-  for (uint32_t b0 = lo; b0 < hi; b0 += 32 * kAhead) {
-    uint32_t u[kAhead];
+  if (a.mode & PARD_MODE_PATH_MASK) stage_paths(a, v, tile0, sp);
+  constexpr int kUn = 4;                           /* elements, then their records, requested together */
+#pragma unroll 1
+  for (int i0 = 0; i0 < kPolItems; i0 += kUn) {
+    unsigned long long e[kUn], D[kUn];
+    uint32_t flags[kUn];
 #pragma unroll
-    for (int k = 0; k < kAhead; ++k) {
-      const uint32_t j = b0 + 32 * k + lane;
-      u[k] = j < hi ? T[j] : 0u;                   /* beyond the queue: never kept */
+    for (int u = 0; u < kUn; ++u) {
+      const uint64_t j = tile0 + (uint64_t)(i0 + u) * kPolThreads + threadIdx.x;
+      e[u] = j < a.n ? v.src[j] : 0ull;
     }
 #pragma unroll
-    for (int k = 0; k < kAhead; ++k) {
-      if (b0 + 32 * k >= hi) break;                /* uniform */
-      uint32_t m = __ballot_sync(0xffffffffu, x < u[k]);        /* as if nobody in the step were kept before */
-      for (int round = 0; round < 34; ++round) {   /* bit i is final after i + 1 rounds */
-        const uint32_t m2 = __ballot_sync(0xffffffffu, x + __popc(m & below) < u[k]);
-        if (m2 == m) break;
-        m = m2;
+    for (int u = 0; u < kUn; ++u) {
+      const uint64_t j = tile0 + (uint64_t)(i0 + u) * kPolThreads + threadIdx.x;
+      const uint32_t idx = (uint32_t)e[u] & v.imask;
+      D[u] = 0;
+      flags[u] = 0;
+      if (j >= a.n) continue;
+      if (lookup) D[u] = __ldg(reinterpret_cast<const unsigned long long*>(&a.req[idx]));
+      if (a.mode & PARD_MODE_PATH_MASK) flags[u] = __ldg(&reinterpret_cast<const uint32_t*>(&a.req[idx])[3]) >> 16;
+    }
+#pragma unroll
+    for (int u = 0; u < kUn; ++u) {
+      const uint64_t j = tile0 + (uint64_t)(i0 + u) * kPolThreads + threadIdx.x;
+      if (j >= a.n) continue;
+      const uint32_t seg = (uint32_t)(e[u] >> v.kshift), idx = (uint32_t)e[u] & v.imask;
+      const PardSegConst& K = a.ktab[seg];
+      if (K.narrow & kSegNoStage) { set_status(a.hdr, PARD_EDATA); v.T[j] = 0; continue; }
+      long long X = lookup ? (long long)D[u] - K.A : slack_of((e[u] >> a.ibits) & v.dmask, K);   /* deadline - A */
+      if (a.mode & PARD_MODE_NEXUS) X += K.lsub;   /* the current module only: base + d */
+      if (a.mode & PARD_MODE_CLIPPER) {
+        /* the module's share of the request's objective, counted from its arrival at the module; the
+         * request is kept iff its batch starts within the share: start <= arrive + share, i.e.
+         * start + d <= arrive + share + d */
+        const pard_arrival_t ar = a.arrivals[idx];
+        if (ar.arrive_us < 0 || ar.arrive_us >= PARD_TIME_LIMIT_US || ar.slo_us < 0 || ar.slo_us >= (1ll << 31) ||
+            K.d >= (1ll << 32)) {
+          set_status(a.hdr, PARD_EDATA);
+          X = -1;
+        } else {
+          const long long share = (long long)((unsigned long long)ar.slo_us * (unsigned long long)K.d / (unsigned long long)K.dsum);
+          X = ar.arrive_us + share + K.d - (K.A - K.lsub);
+        }
       }
-      const uint32_t j = b0 + 32 * k + lane;
-      if (j < hi) C[j] = (x + __popc(m & below)) | (((m >> lane) & 1u) ? kKeepBit : 0u);
-      x += __popc(m);
+      if (flags[u]) X += K.lsub - masked_lsub(a, sp, seg, flags[u], K);
+      v.T[j] = rounds_fit(X, K);
     }
   }
-  *kept_out = x;
 }
 
-/* Nexus: a window of one batch round (W requests) slides over the queue; the batch is the first
- * window whose requests all still fit the round b being formed (b < v_r); everything before it
- * is dropped; b advances; the scan resumes behind the window.  A request's position is
- * b * W + its offset in the run of fitting requests it belongs to, so floor(position / W) = the
- * round it was tested against, and for the kept ones it is also the number kept before them. */
-__device__ void walk_nexus(const uint32_t* __restrict__ T, uint32_t* __restrict__ C, uint32_t lo, uint32_t hi,
-                           uint32_t W, uint32_t lane, uint32_t* kept_out) {
+/* What a group of WARPS warps that walks one queue together exchanges: running sums and maxima
+ * over its threads, in thread order.  One barrier each; the slots are used in turn. */
+template <int WARPS>
+struct WalkGroup {
+  struct Shared {
+    uint32_t sum[2][WARPS];
+    int32_t top[2][WARPS];
+    uint32_t first[2][WARPS];
+    uint32_t pos;
+  };
+  Shared& sh;
+  uint32_t lane, warp;
+  uint32_t turn;
+  __device__ void sync() const {
+    if (WARPS > 1) __syncthreads();
+    else __syncwarp();
+  }
+  /* sum over the earlier threads; *total: over all */
+  __device__ uint32_t sum_before(uint32_t x, uint32_t* total) {
+    uint32_t incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    if (WARPS == 1) {
+      *total = __shfl_sync(0xffffffffu, incl, 31);
+      return incl - x;
+    }
+    turn ^= 1;
+    if (lane == 31) sh.sum[turn][warp] = incl;
+    sync();
+    const uint32_t w = lane < (uint32_t)WARPS ? sh.sum[turn][lane] : 0u;
+    *total = __reduce_add_sync(0xffffffffu, w);
+    return incl - x + __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+  }
+  /* maximum over the earlier threads (at least `floor`); *total: over all */
+  __device__ int32_t max_before(int32_t x, int32_t floor, int32_t* total) {
+    int32_t incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= (uint32_t)o) incl = max(incl, y);
+    }
+    int32_t before = __shfl_up_sync(0xffffffffu, incl, 1);
+    if (lane == 0) before = floor;
+    if (WARPS == 1) {
+      *total = max(floor, __shfl_sync(0xffffffffu, incl, 31));
+      return max(floor, before);
+    }
+    turn ^= 1;
+    if (lane == 31) sh.top[turn][warp] = incl;
+    sync();
+    const int32_t w = lane < (uint32_t)WARPS ? sh.top[turn][lane] : floor;
+    *total = max(floor, __reduce_max_sync(0xffffffffu, w));
+    return max(max(floor, before), __reduce_max_sync(0xffffffffu, lane < warp ? w : floor));
+  }
+  /* smallest x of the group */
+  __device__ uint32_t min_all(uint32_t x) {
+    const uint32_t m = __reduce_min_sync(0xffffffffu, x);
+    if (WARPS == 1) return m;
+    turn ^= 1;
+    if (lane == 0) sh.first[turn][warp] = m;
+    sync();
+    return __reduce_min_sync(0xffffffffu, lane < (uint32_t)WARPS ? sh.first[turn][lane] : 0xffffffffu);
+  }
+};
+
+constexpr int kWalkItems = 16;                     /* consecutive requests per thread and step */
+constexpr uint32_t kWalkWarps = 16;                /* warps of a group that walks a long queue */
+constexpr uint32_t kWalkLong = 2048;               /* requests per queue on average from which a block, not a warp, walks one:
+                                                      a quarter of the 8,192 requests a block takes in one step */
+constexpr uint32_t kWalkSmallRound = 64;           /* rounds below this size are walked by one warp, 32 requests per step: a step
+                                                      closes several of them, where a group needs a barrier for each */
+
+/* this thread's 16 thresholds; the array may be read up to the next multiple of 16 (workspace) */
+__device__ __forceinline__ void walk_load(const uint32_t* __restrict__ T, uint32_t at, uint32_t hi, uint32_t (&v)[kWalkItems]) {
+#pragma unroll
+  for (int q = 0; q < kWalkItems / 4; ++q) {
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+    if (at + 4 * q < hi) x = *reinterpret_cast<const uint4*>(T + at + 4 * q);
+    v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+  }
+}
+
+/* bits of this thread's requests that fit round b */
+__device__ __forceinline__ uint32_t walk_fit(const uint32_t (&v)[kWalkItems], uint32_t b) {
+  uint32_t g = 0;
+#pragma unroll
+  for (int i = 0; i < kWalkItems; ++i) g |= (v[i] > b ? 1u : 0u) << i;
+  return g;
+}
+
+/* bits of the positions at .. at+15 that lie in [from, hi) */
+__device__ __forceinline__ uint32_t walk_range(uint32_t at, uint32_t from, uint32_t hi) {
+  uint32_t m = 0xffffu;
+  if (from > at) m = from - at >= 16 ? 0u : m & (0xffffu << (from - at));
+  if (hi < at + 16) m = hi <= at ? 0u : m & (0xffffu >> (at + 16 - hi));
+  return m;
+}
+
+/* The general rule in rounds of at least kWalkSmallRound.  RAW: every request ahead takes a slot,
+ * so a request's round is its position's and no round has to be waited for. */
+template <int WARPS, bool RAW>
+__device__ void walk_admit(WalkGroup<WARPS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
+                           uint32_t hi, const PardSegConst& K) {
+  constexpr uint32_t kStep = WARPS * 32 * kWalkItems;
+  const uint32_t cap = K.cap, t = G.warp * 32 + G.lane;
+  uint32_t x = 0, b = 0, left = cap;
+  uint32_t next[kWalkItems];
+  uint32_t at = (lo & ~(uint32_t)(kWalkItems - 1)) + t * kWalkItems;
+  walk_load(v.T, at, hi, next);
+  for (uint32_t step = lo & ~(uint32_t)(kWalkItems - 1); step < hi; step += kStep, at += kStep) {
+    uint32_t u[kWalkItems];
+#pragma unroll
+    for (int i = 0; i < kWalkItems; ++i) u[i] = next[i];
+    walk_load(v.T, at + kStep, hi, next);          /* the next step's, while this one is decided */
+    uint32_t open = walk_range(at, lo, hi), kept = 0, before = 0, total = 0;
+    const uint32_t x0 = x;
+    bool several = false;
+    for (;;) {
+      uint32_t fit = 0;
+      if (RAW) {
+#pragma unroll
+        for (int i = 0; i < kWalkItems; ++i) {
+          const uint32_t r = at + i - lo, round = K.cap_magic ? div_magic32(r, K.cap_magic) : r;
+          fit |= (u[i] > round ? 1u : 0u) << i;
+        }
+      } else {
+        fit = walk_fit(u, b);
+      }
+      fit &= open;
+      const uint32_t mine = __popc(fit);
+      before = G.sum_before(mine, &total);
+      if (RAW || total < left) {                   /* the round does not close in this step */
+        kept |= fit;
+        x += total;
+        left -= total;
+        break;
+      }
+      several = true;
+      if (before < left && left <= before + mine) {     /* it closes here, behind this thread's (left - before)-th fitting request */
+        uint32_t m = fit;
+        for (uint32_t k = left - before; k > 1; --k) m &= m - 1;
+        const uint32_t end = at + __ffs(m);        /* position behind it */
+        kept |= fit & (0xffffu >> (at + 16 - end));
+        v.C[lo + b] = end;
+        G.sh.pos = end;
+      } else if (before + mine < left) {
+        kept |= fit;
+      }
+      G.sync();
+      const uint32_t end = G.sh.pos;
+      x += left;
+      left = cap;
+      ++b;
+      open = walk_range(at, end, hi);
+      if (end >= hi) { G.sync(); break; }          /* (the slot may be written again) */
+    }
+    if (several) before = G.sum_before(__popc(kept), &total);
+    if ((at & (kPolTile - 1)) == 0 && at >= lo && at < hi) a.tile_x[at / kPolTile] = x0 + before;
+  }
+  if (t == 0) { a.seg_kept[s] = x; a.rounds[s] = b; }
+}
+
+/* The same in small rounds, by one warp: the keep mask of a step of 32 is the fixed point of
+ * keep_i = [x + #kept among lanes below i < u_i] (bit i is final after i + 1 iterations). */
+__device__ void walk_admit_small(const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo, uint32_t hi,
+                                 const PardSegConst& K, uint32_t lane) {
+  const uint32_t below = (1u << lane) - 1, cap = K.cap;
+  uint32_t x = 0;
+  uint32_t next = lo + lane < hi ? v.T[lo + lane] : 0u;
+  for (uint32_t b0 = lo; b0 < hi; b0 += 32) {
+    const uint32_t j = b0 + lane;
+    const unsigned long long u64 = (unsigned long long)next * cap;
+    const uint32_t u = u64 > kUClamp ? kUClamp : (uint32_t)u64;       /* beyond the queue: 0, never kept */
+    next = j + 32 < hi ? v.T[j + 32] : 0u;
+    uint32_t m = __ballot_sync(0xffffffffu, x < u);        /* as if nobody in the step were kept before */
+    for (int round = 0; round < 34; ++round) {
+      const uint32_t m2 = __ballot_sync(0xffffffffu, x + __popc(m & below) < u);
+      if (m2 == m) break;
+      m = m2;
+    }
+    const uint32_t c = x + __popc(m & below);
+    if ((j & (kPolTile - 1)) == 0 && j < hi) a.tile_x[j / kPolTile] = c;
+    if ((m >> lane) & 1u) {                        /* the c-th admitted request closes a round when c + 1 fills it */
+      const uint32_t q = K.cap_magic ? div_magic32(c + 1, K.cap_magic) : c + 1;
+      if (q * cap == c + 1) v.C[lo + q - 1] = j + 1;
+    }
+    x += __popc(m);
+  }
+  if (lane == 0) { a.seg_kept[s] = x; a.rounds[s] = K.cap_magic ? div_magic32(x, K.cap_magic) : x; }
+}
+
+/* Nexus: the batch is the first window of W = cap requests that all fit the round b being formed
+ * (b < v_r), everything before it is dropped, b advances, the scan goes on behind it.  With `bad`
+ * the last position that does not fit (or that ends the window before), a window closes at
+ * bad + W, the first time that lies before the next misfit. */
+template <int WARPS>
+__device__ void walk_nexus(WalkGroup<WARPS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
+                           uint32_t hi, uint32_t W) {
+  constexpr uint32_t kStep = WARPS * 32 * kWalkItems;
+  constexpr uint32_t kNone = 0xffffffffu;
+  const uint32_t t = G.warp * 32 + G.lane;
+  uint32_t b = 0;
+  int32_t bad = (int32_t)lo - 1;
+  uint32_t next[kWalkItems];
+  uint32_t at = (lo & ~(uint32_t)(kWalkItems - 1)) + t * kWalkItems;
+  walk_load(v.T, at, hi, next);
+  for (uint32_t step = lo & ~(uint32_t)(kWalkItems - 1); step < hi; step += kStep, at += kStep) {
+    uint32_t u[kWalkItems];
+#pragma unroll
+    for (int i = 0; i < kWalkItems; ++i) u[i] = next[i];
+    walk_load(v.T, at + kStep, hi, next);
+    uint32_t from = lo;
+    for (;;) {
+      const uint32_t open = walk_range(at, from, hi);
+      const uint32_t miss = ~walk_fit(u, b) & open;
+      int32_t top;
+      int32_t last = G.max_before(miss ? (int32_t)at + 31 - __clz(miss) : -1, bad, &top);
+      uint32_t found = kNone;
+      for (uint32_t m = miss; open;) {             /* stretches of fitting requests between this thread's misfits */
+        const uint32_t end = m ? at + __ffs(m) - 1 : min(at + 16, hi);     /* where the stretch ends */
+        const unsigned long long full = (unsigned long long)((long long)last + W);   /* where a window would close */
+        if (full < end && full >= max(at, from)) { found = (uint32_t)full; break; }
+        if (!m) break;
+        last = (int32_t)end;
+        m &= m - 1;
+      }
+      found = G.min_all(found);
+      if (found == kNone) { bad = top; break; }
+      if (t == 0) v.C[lo + b] = found + 1;
+      ++b;
+      bad = (int32_t)found;
+      from = found + 1;
+      if (from >= hi) break;
+    }
+  }
+  if (t == 0) {
+    const uint32_t run = (uint32_t)((int32_t)hi - 1 - bad);          /* a last, partly filled window runs as it is */
+    a.rounds[s] = b;
+    a.tail[s] = run;
+    a.seg_kept[s] = b * W + run;
+  }
+}
+
+/* Nexus in small windows, by one warp, 32 requests per step. */
+__device__ void walk_nexus_small(const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo, uint32_t hi,
+                                 uint32_t W, uint32_t lane) {
   uint32_t b = 0, run = 0;                         /* batches formed; length of the current run of fitting requests */
+  uint32_t next = lo + lane < hi ? v.T[lo + lane] : 0u;
   for (uint32_t p0 = lo; p0 < hi; p0 += 32) {
     const uint32_t nvalid = min(32u, hi - p0);
-    const uint32_t v = lane < nvalid ? T[p0 + lane] : 0u;
+    const uint32_t x = next;
+    next = p0 + 32 + lane < hi ? v.T[p0 + 32 + lane] : 0u;
     const uint32_t valid = nvalid == 32 ? 0xffffffffu : ((1u << nvalid) - 1);
-    uint32_t cval = 0;
     uint32_t pos = 0;
     while (pos < nvalid) {                         /* uniform */
-      const uint32_t fit = __ballot_sync(0xffffffffu, b < v) & valid;
-      const uint32_t from = ~((1u << pos) - 1);    /* lanes >= pos */
-      const uint32_t bad = ~fit & valid & from;
-      const uint32_t firstbad = bad ? (uint32_t)__ffs(bad) - 1 : nvalid;
+      const uint32_t fit = __ballot_sync(0xffffffffu, b < x) & valid;
+      const uint32_t misfit = ~fit & valid & ~((1u << pos) - 1);
+      const uint32_t firstbad = misfit ? (uint32_t)__ffs(misfit) - 1 : nvalid;
       const uint32_t fitlen = firstbad - pos, need = W - run;
       if (fitlen >= need) {                        /* the window is full at lane pos + need - 1 */
-        if (lane >= pos && lane < pos + need) cval = (b * W + run + (lane - pos)) | kKeepBit;
+        pos += need;
+        if (lane == 0) v.C[lo + b] = p0 + pos;
         ++b;
         run = 0;
-        pos += need;
       } else if (firstbad < nvalid) {              /* a request that does not fit: the run before it goes too */
-        if (lane >= pos && lane < firstbad) cval = b * W + run + (lane - pos);
-        if (lane == firstbad) cval = b * W;
-        /* the part of the run met in earlier steps (a run only grows across a step's end, so none
-         * of it lies in this step): those positions lose their provisional keep */
-        if (run > 0) {
-          __syncwarp();
-          const uint32_t first = p0 + pos - run;   /* >= lo; pos is 0 here */
-          for (uint32_t q = first + lane; q < p0 + pos; q += 32) C[q] &= ~kKeepBit;
-          __syncwarp();
-        }
         run = 0;
         pos = firstbad + 1;
       } else {                                     /* everything up to the end of the step fits: the run goes on */
-        if (lane >= pos && lane < nvalid) cval = (b * W + run + (lane - pos)) | kKeepBit;
         run += fitlen;
         pos = nvalid;
       }
     }
-    if (lane < nvalid) C[p0 + lane] = cval;
   }
-  *kept_out = b * W + run;                         /* a last, partly filled window runs as it is */
+  if (lane == 0) { a.rounds[s] = b; a.tail[s] = run; a.seg_kept[s] = b * W + run; }
 }
 
-__global__ void __launch_bounds__(kPolThreads)
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS == 1 ? kPolThreads : WARPS * 32)
 k_policy_walk(const PolicyArgs a) {
   pdl_wait();
+  constexpr int kGroups = WARPS == 1 ? kPolThreads / 32 : 1;
+  __shared__ typename WalkGroup<WARPS>::Shared sh[kGroups];
   if (a.hdr->wide || a.hdr->aborted) return;
-  const uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (s >= a.n_seg) return;                        /* whole warps leave together */
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t s = WARPS == 1 ? blockIdx.x * kGroups + warp : blockIdx.x;
+  if (s >= a.n_seg) return;                        /* whole groups leave together */
   const SortedView v = sorted_view(a);
   const uint32_t lo = a.seg_off[s], hi = a.seg_off[s + 1];
-  uint32_t kept = 0;
-  if (hi > lo) {
-    if (a.mode & PARD_MODE_NEXUS) walk_nexus(v.T, v.C, lo, hi, a.ktab[s].cap, lane, &kept);
-    else walk_admit(v.T, v.C, lo, hi, lane, &kept, (a.mode & PARD_MODE_RAW) != 0);
+  if (hi <= lo) {
+    if (lane == 0 && (WARPS == 1 || warp == 0)) { a.rounds[s] = 0; a.tail[s] = 0; a.seg_kept[s] = 0; }
+    return;
   }
-  if (lane == 0) a.seg_kept[s] = kept;
+  const PardSegConst K = a.ktab[s];
+  const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
+  if (K.cap < kWalkSmallRound && !raw) {
+    if (WARPS > 1 && warp != 0) return;
+    if (nexus) walk_nexus_small(a, v, s, lo, hi, K.cap, lane);
+    else walk_admit_small(a, v, s, lo, hi, K, lane);
+    return;
+  }
+  WalkGroup<WARPS> G{sh[WARPS == 1 ? warp : 0], lane, WARPS == 1 ? 0u : warp, 0u};
+  if (nexus) walk_nexus<WARPS>(G, a, v, s, lo, hi, K.cap);
+  else if (raw) walk_admit<WARPS, true>(G, a, v, s, lo, hi, K);
+  else walk_admit<WARPS, false>(G, a, v, s, lo, hi, K);
 }
 
+/* Estimates, decisions and survivors.  A request's round is the number of rounds of its queue that
+ * ended at or before it (a search in the ends, starting at the round of the thread's request
+ * before); its place among the survivors is, for Nexus, given by its window, else the kept requests
+ * ahead of it: those ahead of the tile (a.tile_x) and, by ballots, those inside it. */
 __global__ void __launch_bounds__(kPolThreads)
 k_policy_emit(const PolicyArgs a) {
   pdl_wait();
+  constexpr int kWarps = kPolThreads / 32, kRows = kPolItems * kWarps;
+  static_assert(kRows == 32, "one warp scans the rows");
   __shared__ StagedPaths sp;
+  __shared__ uint32_t s_keep[kRows], s_before[kRows + 1];
   if (a.hdr->wide || a.hdr->aborted) return;
   const SortedView v = sorted_view(a);
-  const uint64_t tile0 = (uint64_t)blockIdx.x * kPolTile;
-  if (a.mode & PARD_MODE_PATH_MASK) stage_paths(a, (uint32_t)(v.src[tile0] >> v.kshift), sp);
-  else if (threadIdx.x == 0) sp.seg0 = 0;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t tile0 = blockIdx.x * kPolTile;
+  const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW, mask = a.mode & PARD_MODE_PATH_MASK;
+  if (mask) stage_paths(a, v, tile0, sp);
+  unsigned long long e[kPolItems];
+  uint32_t t[kPolItems], round[kPolItems], flags[kPolItems];
+#pragma unroll
   for (int i = 0; i < kPolItems; ++i) {
-    const uint64_t j = tile0 + (uint64_t)i * kPolThreads + threadIdx.x;
-    if (j >= a.n) break;
-    const unsigned long long e = v.src[j];
-    const uint32_t seg = (uint32_t)(e >> v.kshift), idx = (uint32_t)e & v.imask;
-    const PardSegConst K = a.ktab[seg];
-    uint32_t c = 0, keep = 0;
-    long long est = K.A;
-    if (!(K.narrow & kSegNoStage)) {
-      const Terms t = request_terms(a, sp, seg, idx, K);
-      const uint32_t w = v.C[j];
-      c = w & ~kKeepBit;                           /* kept requests ahead in the queue */
-      keep = w >> 31;
-      /* the batch-slot position: the kept requests ahead, or, when every request ahead takes a slot, all of them */
-      const uint32_t slot = (a.mode & PARD_MODE_RAW) ? (uint32_t)j - a.seg_off[seg] : c;
-      const uint32_t round = K.cap_magic ? div_magic32(slot, K.cap_magic) : slot;     /* floor(slot / cap) */
-      est = t.A + (long long)round * K.d;
+    const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
+    e[i] = j < a.n ? v.src[j] : 0ull;
+    t[i] = j < a.n && !nexus ? v.T[j] : 0u;
+  }
+  if (mask) {
+#pragma unroll
+    for (int i = 0; i < kPolItems; ++i) {
+      const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
+      flags[i] = j < a.n ? __ldg(&reinterpret_cast<const uint32_t*>(&a.req[(uint32_t)e[i] & v.imask])[3]) >> 16 : 0u;
     }
+  }
+  uint32_t cur = 0xffffffffu, lo = 0, hi = 0, nb = 0, b = 0, keepbits = 0;
+#pragma unroll
+  for (int i = 0; i < kPolItems; ++i) {
+    const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
+    bool keep = false;
+    round[i] = 0;
+    if (j < a.n) {
+      const uint32_t seg = (uint32_t)(e[i] >> v.kshift);
+      if (seg != cur) {
+        cur = seg;
+        lo = a.seg_off[seg];
+        hi = a.seg_off[seg + 1];
+        nb = a.rounds[seg];
+        b = 0;
+      }
+      const PardSegConst& K = a.ktab[seg];
+      if (raw) {
+        b = K.cap_magic ? div_magic32(j - lo, K.cap_magic) : j - lo;
+      } else {
+        uint32_t z = nb;                           /* ends b .. nb-1: how many are <= j */
+        while (b < z) {
+          const uint32_t mid = b + (z - b) / 2;
+          if (v.C[lo + mid] <= j) b = mid + 1; else z = mid;
+        }
+      }
+      if (nexus) keep = b < nb ? j + K.cap >= v.C[lo + b] : j + a.tail[seg] >= hi;
+      else keep = t[i] > b;
+      keep = keep && !(K.narrow & kSegNoStage);
+      round[i] = b;
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, keep);
+    if (lane == 0) s_keep[i * kWarps + warp] = m;
+    keepbits |= (keep ? 1u : 0u) << i;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t x = __popc(s_keep[lane]);
+    uint32_t incl = x;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    s_before[lane] = incl - x;
+  }
+  __syncthreads();
+  /* kept requests of the tile ahead of its position p */
+  auto kept_before = [&](uint32_t p) { return s_before[p >> 5] + __popc(s_keep[p >> 5] & ((1u << (p & 31)) - 1)); };
+#pragma unroll
+  for (int i = 0; i < kPolItems; ++i) {
+    const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
+    if (j >= a.n) break;
+    const uint32_t seg = (uint32_t)(e[i] >> v.kshift), idx = (uint32_t)e[i] & v.imask;
+    const PardSegConst& K = a.ktab[seg];
+    const uint32_t keep = (keepbits >> i) & 1u;
+    long long A = K.A;
+    if (a.mode & (PARD_MODE_NEXUS | PARD_MODE_CLIPPER)) A -= K.lsub;     /* the current module only */
+    if (mask && flags[i] && !(K.narrow & kSegNoStage)) A += masked_lsub(a, sp, seg, flags[i], K) - K.lsub;
     if (a.out_keep) a.out_keep[j] = (uint8_t)keep;
-    if (a.out_est) a.out_est[j] = est;
+    if (a.out_est) a.out_est[j] = (K.narrow & kSegNoStage) ? K.A : A + (long long)round[i] * K.d;
     if (a.out_perm) a.out_perm[j] = idx;
-    if (keep && a.kept_tmp) a.kept_tmp[a.seg_off[seg] + c] = idx;                /* c = kept requests ahead in the queue */
+    if (keep && a.out_kept_idx) {
+      const uint32_t first = a.seg_off[seg];
+      uint32_t c;
+      if (nexus) c = round[i] * K.cap + (round[i] < a.rounds[seg] ? j + K.cap - v.C[first + round[i]] : j + a.tail[seg] - a.seg_off[seg + 1]);
+      else if (first <= tile0) c = a.tile_x[blockIdx.x] + kept_before(j - tile0);
+      else c = kept_before(j - tile0) - kept_before(first - tile0);
+      a.out_kept_idx[a.kept_base[seg] + c] = idx;
+    }
   }
 }
 
@@ -332,11 +614,19 @@ k_policy_emit(const PolicyArgs a) {
 
 namespace pard_plan_detail {
 
-int launch_policy_decision(const PolicyArgs& a, int sms, cudaStream_t stream) {
-  (void)sms;
+int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
+  static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
   launch_pdl(k_policy_terms, tiles, kPolThreads, 0, stream, a);
-  launch_pdl(k_policy_walk, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
+  if (a.n / a.n_seg >= kWalkLong)
+    launch_pdl(k_policy_walk<kWalkWarps>, a.n_seg, kWalkWarps * 32, 0, stream, a);
+  else
+    launch_pdl(k_policy_walk<1>, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
+  return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
+}
+
+int launch_policy_emit(const PolicyArgs& a, cudaStream_t stream) {
+  const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
   launch_pdl(k_policy_emit, tiles, kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
 }

@@ -1,0 +1,95 @@
+"""The variants a dispatch chooses from, at the sizes where they can go wrong, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2602_08747_b200 import binding as pb
+from paper_2602_08747_b200 import inputs
+from tests import util
+from tests.gpu_util import assert_identical, run_library
+
+pytestmark = pytest.mark.gpu
+
+FCFS, NEXUS = pb.PARD_MODE_FCFS, pb.PARD_MODE_NEXUS
+RULES = pb.PARD_MODE_PATH_MASK | FCFS | NEXUS | pb.PARD_MODE_CLIPPER
+
+
+def check(wl, mode=0):
+    want = oracle.plan(wl.pipelines, wl.requests, wl.state, wl.n_ctx, mode & (RULES | pb.PARD_MODE_RAW))
+    rc, got = run_library(wl, mode)
+    assert rc == 0
+    assert_identical(got, want)
+    return got
+
+
+def several_ctx(n_ctx, sizes, seed=0, S=3, span=3000, sort=True, mix=False, B=2, m=1):
+    """Contexts of the given sizes on one chain; deadlines in order inside every ctx when `sort`."""
+    rng = np.random.default_rng(seed)
+    p = util.pipeline(inputs.chain_edges(S), S, list(rng.integers(5, 40, size=S)), bmax=max(B, 4))
+    ctx = np.repeat(np.arange(n_ctx), sizes)
+    d = 1000 + rng.integers(0, span, size=ctx.size)
+    if sort:
+        d = d[np.lexsort((d, ctx))]
+    if mix:
+        k = rng.permutation(ctx.size)
+        ctx, d = ctx[k], d[k]
+    st = util.state(n_ctx, S, inputs.n_slots(p), 1000, B, workers=m, w=rng.integers(0, 50, size=(n_ctx, inputs.n_slots(p))))
+    return inputs.Workload("variants", [p], util.requests(d, rng.integers(0, S, size=ctx.size), ctx), st, n_ctx)
+
+
+# ---- rounds closed by a warp, by a block, or 32 requests per step --------------------------------
+@pytest.mark.parametrize("rule", [FCFS, NEXUS])
+@pytest.mark.parametrize("cap", [63, 64, 65, 1000, 8191, 8193])
+@pytest.mark.parametrize("n", [15, 2047, 2049, 8192, 8193, 30_011])
+def test_walk_rounds_against_steps_and_queue_lengths(rule, cap, n):
+    rng = np.random.default_rng(n + cap)
+    p = util.pipeline([], 1, [13], bmax=4096)
+    st = util.state(1, 1, 0, 0, cap // 2 if cap > 4096 else cap, workers=2 if cap > 4096 else 1)
+    real = int(st.batch[0, 0] * st.workers[0, 0])
+    for top in (1.0, 3.0):                                 # rounds the queue needs, and well beyond
+        dl = rng.integers(0, int(13 * (n / real + 2) * top), size=n)
+        if rule == NEXUS:                                  # mostly fitting, so that windows do fill
+            dl[rng.random(n) < 0.999] = 10**6
+        check(inputs.Workload("edge", [p], util.requests(dl), st, 1), rule)
+
+
+@pytest.mark.parametrize("sizes", [[5000, 0, 1, 4099], [200] * 40, [2100, 2048, 1]])
+@pytest.mark.parametrize("mode", [FCFS, NEXUS, pb.PARD_MODE_PATH_MASK])
+def test_walk_of_several_queues_with_heads_inside_tiles(sizes, mode):
+    for m in (1, 40):
+        check(several_ctx(len(sizes), sizes, sort=False, mix=True, m=m), mode)
+
+
+# ---- requests that come in deadline order --------------------------------------------------------
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_GROUPED, pb.PARD_MODE_RAW, pb.PARD_MODE_SCAN])
+@pytest.mark.parametrize("sizes", [[1], [8192], [8193], [20_011], [3000, 1, 0, 8192], [9000, 10_001, 8193, 8200]])
+def test_requests_in_deadline_order(sizes, mode):
+    if mode == pb.PARD_MODE_GROUPED and max(sizes) > 8192 >= sum(sizes) / len(sizes):
+        pytest.skip("breaks the promise")
+    wl = several_ctx(len(sizes), sizes, S=4, m=20)
+    check(wl, mode)
+    for at in (1, wl.n // 2, wl.n - 1):                    # in order but for one request
+        if 0 < at < wl.n:
+            w2 = several_ctx(len(sizes), sizes, S=4, m=20)
+            w2.requests["deadline_us"][at] = 990
+            check(w2, mode)
+    wl.state.priority = np.ones((wl.n_ctx, 4), np.uint8)    # order of deadlines is not the queues' order then
+    check(wl, mode)
+
+
+def test_requests_in_deadline_order_across_mixed_contexts():
+    wl = several_ctx(7, [3000] * 7, sort=False, mix=True)
+    wl.requests["deadline_us"].sort()
+    check(wl)
+    wl.requests["deadline_us"][[5, 9000]] = wl.requests["deadline_us"][[9000, 5]]
+    check(wl)
+
+
+# ---- ranges of mixed contexts --------------------------------------------------------------------
+@pytest.mark.parametrize("n_ctx,n", [(2, 3000), (500, 740_000), (4096, 9_000), (4097, 30_000)])
+def test_ranges_of_contexts_in_mixed_order(n_ctx, n):
+    rng = np.random.default_rng(n_ctx)
+    wl = several_ctx(n_ctx, np.bincount(rng.integers(0, n_ctx, size=n), minlength=n_ctx), S=2, sort=False, mix=True, m=3)
+    check(wl)
+    wl.requests["deadline_us"][rng.integers(0, n, size=5)] += 1 << 33      # beyond 32-bit offsets from the first request
+    check(wl)
