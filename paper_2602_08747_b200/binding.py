@@ -3,11 +3,14 @@
 Argument marshalling only: every step of the planner runs in the library's
 kernels.  PyTorch is used for device memory and streams.  The functions carry
 the names of the C entry points declared in include/pard.h.  There is no CPU
-fallback: a missing library raises at the first call.
+fallback: a missing library raises at the first call.  The calls of a control
+loop go through a small native module (csrc/pard_pycall.c), the others through
+ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import List, Optional, Sequence
@@ -16,6 +19,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libpard.so")
+CALL_PATH = os.path.join(_HERE, "_pardcall.so")
 
 PARD_OK = 0
 PARD_EINVAL, PARD_ECYCLE, PARD_ERANGE, PARD_ENOMEM = -1, -2, -3, -4
@@ -128,6 +132,24 @@ def library() -> C.CDLL:
     return _lib
 
 
+_calls = None
+
+
+def _native():
+    """The marshalling module, bound to the library."""
+    global _calls
+    if _calls is None:
+        library()
+        if not os.path.exists(CALL_PATH):
+            raise RuntimeError("_pardcall.so is missing: run `python -m paper_2602_08747_b200.build`")
+        spec = importlib.util.spec_from_file_location("_pardcall", CALL_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.bind(LIB_PATH)
+        _calls = mod
+    return _calls
+
+
 def pard_strerror(status: int) -> str:
     return library().pard_strerror(int(status)).decode()
 
@@ -147,10 +169,11 @@ def _ptr(t) -> Optional[int]:
 
 
 class Pipeline:
-    """Owns one pard_pipeline_t handle."""
+    """Owns one pard_pipeline_t handle (`addr`: its address, 0 once freed)."""
 
     def __init__(self, handle: int):
         self._h = C.c_void_p(handle)
+        self.addr = handle or 0
 
     def __del__(self):
         try:
@@ -162,6 +185,7 @@ class Pipeline:
         if getattr(self, "_h", None) is not None and self._h.value:
             library().pard_free_pipeline(self._h)
             self._h = C.c_void_p(None)
+            self.addr = 0
 
     @property
     def handle(self) -> int:
@@ -255,19 +279,11 @@ def pard_plan_host_workspace_bytes(n: int, n_ctx: int, stage_stride: int, slot_s
     return v.value
 
 
-def _handles(pipelines: Sequence[Pipeline]):
-    return (C.c_void_p * len(pipelines))(*[p.handle for p in pipelines])
-
-
 def pard_plan(pipelines: Sequence[Pipeline], d_requests, n: int, state: QueueStateArrays,
               n_ctx: int, mode: int, out: PlanOut, d_workspace, workspace_bytes: Optional[int] = None,
               stream: int = 0, check: bool = True) -> int:
-    hs = _handles(pipelines)
-    st, o = state.c_struct(), out.c_struct()
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_plan(hs, len(pipelines), _ptr(d_requests), n, C.byref(st), n_ctx, mode,
-                             C.byref(o), _ptr(d_workspace), wb, stream or None)
-    if check:
+    rc = (_calls or _native()).plan(0, pipelines, d_requests, None, n, state, n_ctx, mode, out, d_workspace, workspace_bytes, stream)
+    if rc and check:
         _check(rc, "pard_plan")
     return rc
 
@@ -275,12 +291,9 @@ def pard_plan(pipelines: Sequence[Pipeline], d_requests, n: int, state: QueueSta
 def pard_plan_policy(pipelines: Sequence[Pipeline], d_requests, d_arrivals, n: int, state: QueueStateArrays,
                      n_ctx: int, mode: int, out: PlanOut, d_workspace, workspace_bytes: Optional[int] = None,
                      stream: int = 0, check: bool = True) -> int:
-    hs = _handles(pipelines)
-    st, o = state.c_struct(), out.c_struct()
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_plan_policy(hs, len(pipelines), _ptr(d_requests), _ptr(d_arrivals), n, C.byref(st), n_ctx,
-                                    mode, C.byref(o), _ptr(d_workspace), wb, stream or None)
-    if check:
+    rc = (_calls or _native()).plan(1, pipelines, d_requests, d_arrivals, n, state, n_ctx, mode, out, d_workspace, workspace_bytes,
+                                    stream)
+    if rc and check:
         _check(rc, "pard_plan_policy")
     return rc
 
@@ -288,12 +301,8 @@ def pard_plan_policy(pipelines: Sequence[Pipeline], d_requests, d_arrivals, n: i
 def pard_plan_host(pipelines: Sequence[Pipeline], requests, n: int, state: QueueStateArrays,
                    n_ctx: int, mode: int, out: PlanOut, d_workspace,
                    workspace_bytes: Optional[int] = None, stream: int = 0, check: bool = True) -> int:
-    hs = _handles(pipelines)
-    st, o = state.c_struct(), out.c_struct()
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_plan_host(hs, len(pipelines), _ptr(requests), n, C.byref(st), n_ctx, mode,
-                                  C.byref(o), _ptr(d_workspace), wb, stream or None)
-    if check:
+    rc = (_calls or _native()).plan(2, pipelines, requests, None, n, state, n_ctx, mode, out, d_workspace, workspace_bytes, stream)
+    if rc and check:
         _check(rc, "pard_plan_host")
     return rc
 
@@ -304,18 +313,15 @@ def pard_plan_static(pipelines: Sequence[Pipeline], d_requests, n: int, state: Q
     fixed device array, for callers that must not allocate device memory
     (problems up to PARD_STATIC_SCRATCH_BYTES of scratch; larger ones return
     PARD_ESTATIC).  Calls on one device share that array and must not overlap."""
-    hs = _handles(pipelines)
-    st, o = state.c_struct(), out.c_struct()
-    rc = library().pard_plan_static(hs, len(pipelines), _ptr(d_requests), n, C.byref(st), n_ctx, mode,
-                                    C.byref(o), stream or None)
-    if check:
+    rc = (_calls or _native()).plan(3, pipelines, d_requests, None, n, state, n_ctx, mode, out, None, None, stream)
+    if rc and check:
         _check(rc, "pard_plan_static")
     return rc
 
 
 def pard_plan_status(d_workspace, stream: int = 0, check: bool = True) -> int:
-    rc = library().pard_plan_status(_ptr(d_workspace), stream or None)
-    if check:
+    rc = (_calls or _native()).status(d_workspace, stream)
+    if rc and check:
         _check(rc, "pard_plan_status")
     return rc
 
@@ -342,9 +348,8 @@ def pard_profile_end() -> dict:
 
 def pard_goodput(d_keep, d_seg_offsets, d_seg_kept, n: int, n_ctx: int, stage_stride: int, d_out_total,
                  d_out_kept, stream: int = 0, check: bool = True) -> int:
-    rc = library().pard_goodput(_ptr(d_keep), _ptr(d_seg_offsets), _ptr(d_seg_kept), n, n_ctx, stage_stride,
-                                _ptr(d_out_total), _ptr(d_out_kept), stream or None)
-    if check:
+    rc = (_calls or _native()).goodput(d_keep, d_seg_offsets, d_seg_kept, n, n_ctx, stage_stride, d_out_total, d_out_kept, stream)
+    if rc and check:
         _check(rc, "pard_goodput")
     return rc
 
@@ -359,13 +364,9 @@ def pard_estimate_w(pipelines: Sequence[Pipeline], d_pipeline_of_ctx, n_ctx: int
                     slot_stride: int, d_wait_samples, n_samples: int, lambda_num: int, lambda_den: int,
                     seed: int, mode: int, d_w_us, d_workspace, workspace_bytes: Optional[int] = None,
                     stream: int = 0, check: bool = True) -> int:
-    hs = _handles(pipelines)
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_estimate_w(hs, len(pipelines), _ptr(d_pipeline_of_ctx), n_ctx, stage_stride,
-                                   slot_stride, _ptr(d_wait_samples), n_samples, lambda_num, lambda_den,
-                                   seed & (2**64 - 1), mode, _ptr(d_w_us), _ptr(d_workspace),
-                                   wb, stream or None)
-    if check:
+    rc = (_calls or _native()).estimate_w(pipelines, d_pipeline_of_ctx, n_ctx, stage_stride, slot_stride, d_wait_samples, n_samples,
+                                          lambda_num, lambda_den, seed, mode, d_w_us, d_workspace, workspace_bytes, stream)
+    if rc and check:
         _check(rc, "pard_estimate_w")
     return rc
 
@@ -381,13 +382,9 @@ def pard_update_priority(pipelines: Sequence[Pipeline], d_pipeline_of_ctx, n_ctx
                          d_batch, d_workers, d_arrivals, n_hist: int, window: int, interval_us: int,
                          mode: int, d_priority, d_workspace, workspace_bytes: Optional[int] = None,
                          stream: int = 0, check: bool = True) -> int:
-    hs = _handles(pipelines)
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_update_priority(hs, len(pipelines), _ptr(d_pipeline_of_ctx), n_ctx, stage_stride,
-                                        _ptr(d_batch), _ptr(d_workers), _ptr(d_arrivals), n_hist, window,
-                                        interval_us, mode, _ptr(d_priority), _ptr(d_workspace), wb,
-                                        stream or None)
-    if check:
+    rc = (_calls or _native()).update_priority(pipelines, d_pipeline_of_ctx, n_ctx, stage_stride, d_batch, d_workers, d_arrivals,
+                                               n_hist, window, interval_us, mode, d_priority, d_workspace, workspace_bytes, stream)
+    if rc and check:
         _check(rc, "pard_update_priority")
     return rc
 
@@ -401,11 +398,9 @@ def pard_update_queue_delay_workspace_bytes() -> int:
 def pard_update_queue_delay(n_ctx: int, stage_stride: int, d_now_us, d_sample_time_us, d_sample_delay_us,
                             n_samples: int, window_us: int, mode: int, d_q_us, d_workspace,
                             workspace_bytes: Optional[int] = None, stream: int = 0, check: bool = True) -> int:
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_update_queue_delay(n_ctx, stage_stride, _ptr(d_now_us), _ptr(d_sample_time_us),
-                                           _ptr(d_sample_delay_us), n_samples, window_us, mode, _ptr(d_q_us),
-                                           _ptr(d_workspace), wb, stream or None)
-    if check:
+    rc = (_calls or _native()).update_queue_delay(n_ctx, stage_stride, d_now_us, d_sample_time_us, d_sample_delay_us, n_samples,
+                                                  window_us, mode, d_q_us, d_workspace, workspace_bytes, stream)
+    if rc and check:
         _check(rc, "pard_update_queue_delay")
     return rc
 
@@ -420,13 +415,10 @@ def pard_advance_state(pipelines: Sequence[Pipeline], d_pipeline_of_ctx, n_ctx: 
                        d_batch, d_workers, d_seg_kept, d_free_at_us, d_sample_time_us, d_sample_delay_us,
                        n_samples: int, slot: int, mode: int, d_workspace, workspace_bytes: Optional[int] = None,
                        stream: int = 0, check: bool = True) -> int:
-    hs = _handles(pipelines)
-    wb = workspace_bytes if workspace_bytes is not None else d_workspace.numel() * d_workspace.element_size()
-    rc = library().pard_advance_state(hs, len(pipelines), _ptr(d_pipeline_of_ctx), n_ctx, stage_stride,
-                                      _ptr(d_now_us), _ptr(d_batch), _ptr(d_workers), _ptr(d_seg_kept),
-                                      _ptr(d_free_at_us), _ptr(d_sample_time_us), _ptr(d_sample_delay_us),
-                                      n_samples, slot, mode, _ptr(d_workspace), wb, stream or None)
-    if check:
+    rc = (_calls or _native()).advance_state(pipelines, d_pipeline_of_ctx, n_ctx, stage_stride, d_now_us, d_batch, d_workers,
+                                             d_seg_kept, d_free_at_us, d_sample_time_us, d_sample_delay_us, n_samples, slot, mode,
+                                             d_workspace, workspace_bytes, stream)
+    if rc and check:
         _check(rc, "pard_advance_state")
     return rc
 
