@@ -77,6 +77,28 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+/* Status of a waiting call (pard_report.cu): where in pinned host memory the device answers.
+ * word == NULL: nowhere, the status is copied. */
+struct PardTicket {
+  unsigned long long* word;
+  uint32_t ticket;
+};
+void pard_report_init();
+PardTicket pard_report_ticket();
+/* waits for the answer to `t` (given by the work already enqueued on `stream`); the call's status */
+int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream);
+/* the same behind everything enqueued so far: answers `t` with a kernel of its own */
+int pard_wait_status(const uint32_t* d_status, cudaStream_t stream);
+
+#ifdef __CUDACC__
+/* by one thread, once every write of the call is visible to it */
+__device__ __forceinline__ void pard_report(const uint32_t* status, unsigned long long* word, uint32_t ticket) {
+  const unsigned long long w = ((unsigned long long)ticket << 32) | __ldcg(status);
+  __threadfence_system();
+  asm volatile("st.release.sys.global.u64 [%0], %1;" :: "l"(word), "l"(w) : "memory");
+}
+#endif
+
 /* see pard_profile_begin: lets pard_goodput count as the end of the planner's last phase */
 void pard_profile_extend_last(cudaStream_t stream);
 

@@ -159,6 +159,7 @@ extern "C" int pard_load_pipeline(const pard_dag_t* dag, const pard_profile_t* p
     int dev = -1;
     char* d = nullptr;
     if (cudaGetDevice(&dev) != cudaSuccess) { delete p; return PARD_ECUDA; }
+    pard_report_init();
     if (cudaMalloc((void**)&d, total) != cudaSuccess) {
       cudaGetLastError();
       delete p;

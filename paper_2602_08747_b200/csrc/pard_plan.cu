@@ -446,7 +446,7 @@ __device__ PardSegConst seg_const_warp(const PipeTable& pipes, uint32_t n_pipeli
 
 /* Per-segment constants; one warp per (ctx, stage). */
 __global__ void __launch_bounds__(128)
-k_seg_const(const PipeTable pipes, uint32_t n_pipelines,
+k_seg_const(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
             pard_queue_state_t st, uint32_t n_ctx,
             const unsigned long long* __restrict__ ctx_dmin_inv,
             const unsigned long long* __restrict__ ctx_dmax, PardSegConst* __restrict__ ktab,
@@ -2466,6 +2466,7 @@ struct LocalArgs {
   unsigned long long* dst;
   unsigned long long* ctx_dmin_inv;
   unsigned long long* ctx_dmax;
+  PardTicket answer;               /* the call's only kernel, and its caller waits: the status goes out from here */
 };
 
 template <int THREADS>
@@ -2517,9 +2518,7 @@ __device__ __forceinline__ LocalElem local_decode(unsigned long long e, uint32_t
  * half as many ranking rounds per warp, twice the warps -- measured the same 28 us at 4,096
  * requests: the time is the chain of barriers and dependent shared-memory steps, not the warps.) */
 template <bool RAW, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1)
-k_plan_local(PlanHeader* __restrict__ hdr, const LocalArgs a) {
-  pdl_wait();
+__device__ __forceinline__ void plan_local(PlanHeader* __restrict__ hdr, const LocalArgs& a) {
   constexpr int WARPS = THREADS / 32;
   constexpr int kItems = kSortTile / THREADS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2930,6 +2929,17 @@ k_plan_local(PlanHeader* __restrict__ hdr, const LocalArgs a) {
       const uint32_t nk = Sm.stage_kept[k], from = Sm.stage_first[k], to = Sm.kept_base[k];
       for (uint32_t i = tid; i < nk; i += THREADS) a.out_kept_idx[to + i] = a.kept_tmp[from + i];
     }
+}
+
+template <bool RAW, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1)
+k_plan_local(PlanHeader* __restrict__ hdr, const __grid_constant__ LocalArgs a) {
+  pdl_wait();
+  plan_local<RAW, THREADS>(hdr, a);
+  if (a.answer.word) {
+    __syncthreads();
+    if (threadIdx.x == 0) pard_report(&hdr->status, a.answer.word, a.answer.ticket);
+  }
 }
 
 /* ------------------------------------------------------------------------ */
@@ -3344,6 +3354,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
       launch_pdl(k_seg_const, (L.n_seg + 3) / 4, 128, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax,
                  ktab, hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
     }
+    const bool answered = fused_single && !(mode & PARD_MODE_NOWAIT);
+    if (answered) la.answer = pard_report_ticket();
     launch_pdl((mode & PARD_MODE_RAW) ? k_plan_local<true, 512> : k_plan_local<false, 512>, n_ctx, 512,
                sizeof(LocalSmem<512>), stream, hdr, la);
     if (fused_grouped) {
@@ -3357,7 +3369,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     while (phase <= PARD_N_PHASES) mark();             /* the phases are those of the other path: all of this counts as the first */
     PARD_CUDA_OK(cudaGetLastError());
     if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-    rc = pard_plan_status(d_workspace, cuda_stream);
+    rc = answered ? pard_report_wait(la.answer, &hdr->status, stream) : pard_plan_status(d_workspace, cuda_stream);
     return rc == PARD_ERANGE ? plan_wide() : rc;
   }
 
@@ -3537,12 +3549,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
 
 extern "C" int pard_plan_status(const void* d_workspace, void* cuda_stream) {
   if (!d_workspace) return PARD_EINVAL;
-  cudaStream_t stream = (cudaStream_t)cuda_stream;
-  uint32_t h_status = 0;
-  PARD_CUDA_OK(cudaMemcpyAsync(&h_status, &((const PlanHeader*)d_workspace)->status, 4,
-                               cudaMemcpyDeviceToHost, stream));
-  PARD_CUDA_OK(cudaStreamSynchronize(stream));
-  return h_status ? -(int)h_status : PARD_OK;
+  return pard_wait_status(&((const PlanHeader*)d_workspace)->status, (cudaStream_t)cuda_stream);
 }
 
 extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t stage_stride,

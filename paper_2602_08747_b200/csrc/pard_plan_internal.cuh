@@ -66,8 +66,9 @@ __device__ __forceinline__ void set_status(PlanHeader* hdr, int status) {
 }
 
 /* The device tables of the call's pipelines: handed over inside the kernel arguments when they
- * are few (no copy to enqueue), else through a table in the workspace. */
-constexpr int kFewPipelines = 8;
+ * fit there (2 KB; no copy to enqueue, which also holds the first kernel up), else through a table
+ * in the workspace. */
+constexpr int kFewPipelines = 256;
 struct PipeTable {
   const PardPipeDev* few[kFewPipelines];
   const PardPipeDev* const* many;

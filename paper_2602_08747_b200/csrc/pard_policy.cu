@@ -141,7 +141,7 @@ __device__ __forceinline__ uint32_t rounds_fit(long long X, const PardSegConst& 
 
 /* One request's rounds and, for PARD_MODE_PATH_MASK, its own downstream estimate. */
 __global__ void __launch_bounds__(kPolThreads)
-k_policy_terms(const PolicyArgs a) {
+k_policy_terms(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   __shared__ StagedPaths sp;
   if (a.hdr->wide || a.hdr->aborted) return;
@@ -479,7 +479,7 @@ __device__ void walk_nexus_small(const PolicyArgs& a, const SortedView& v, uint3
 
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS == 1 ? kPolThreads : WARPS * 32)
-k_policy_walk(const PolicyArgs a) {
+k_policy_walk(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   constexpr int kGroups = WARPS == 1 ? kPolThreads / 32 : 1;
   __shared__ typename WalkGroup<WARPS>::Shared sh[kGroups];
@@ -512,7 +512,7 @@ k_policy_walk(const PolicyArgs a) {
  * before); its place among the survivors is, for Nexus, given by its window, else the kept requests
  * ahead of it: those ahead of the tile (a.tile_x) and, by ballots, those inside it. */
 __global__ void __launch_bounds__(kPolThreads)
-k_policy_emit(const PolicyArgs a) {
+k_policy_emit(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   constexpr int kWarps = kPolThreads / 32, kRows = kPolItems * kWarps;
   static_assert(kRows == 32, "one warp scans the rows");

@@ -182,8 +182,5 @@ extern "C" int pard_update_priority(const pard_pipeline_t* const* pipelines, uin
                           (uint32_t)stage_stride, d_batch, d_workers, d_arrivals, n_hist, window, interval_us,
                           d_priority, hdr));
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-  uint32_t h_status = 0;
-  PARD_CUDA_OK(cudaMemcpyAsync(&h_status, &hdr->status, 4, cudaMemcpyDeviceToHost, stream));
-  PARD_CUDA_OK(cudaStreamSynchronize(stream));
-  return h_status ? -(int)h_status : PARD_OK;
+  return pard_wait_status(&hdr->status, stream);
 }

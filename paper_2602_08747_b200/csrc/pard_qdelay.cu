@@ -91,8 +91,5 @@ extern "C" int pard_update_queue_delay(uint32_t n_ctx, int32_t stage_stride, con
                           (const long long*)d_now_us, (const long long*)d_sample_time_us, d_sample_delay_us,
                           n_samples, window_us, (long long*)d_q_us, hdr));
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-  uint32_t h_status = 0;
-  PARD_CUDA_OK(cudaMemcpyAsync(&h_status, &hdr->status, 4, cudaMemcpyDeviceToHost, stream));
-  PARD_CUDA_OK(cudaStreamSynchronize(stream));
-  return h_status ? -(int)h_status : PARD_OK;
+  return pard_wait_status(&hdr->status, stream);
 }

@@ -106,8 +106,5 @@ extern "C" int pard_advance_state(const pard_pipeline_t* const* pipelines, uint3
                           (long long*)d_free_at_us, (long long*)d_sample_time_us, d_sample_delay_us, n_samples,
                           slot, hdr));
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-  uint32_t h_status = 0;
-  PARD_CUDA_OK(cudaMemcpyAsync(&h_status, &hdr->status, 4, cudaMemcpyDeviceToHost, stream));
-  PARD_CUDA_OK(cudaStreamSynchronize(stream));
-  return h_status ? -(int)h_status : PARD_OK;
+  return pard_wait_status(&hdr->status, stream);
 }

@@ -218,8 +218,5 @@ extern "C" int pard_estimate_w(const pard_pipeline_t* const* pipelines, uint32_t
                           (uint32_t)stage_stride, (uint32_t)slot_stride, d_wait_samples, n_samples,
                           (uint32_t)rank, (unsigned long long)seed, (long long*)d_w_us, hdr));
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-  uint32_t h_status = 0;
-  PARD_CUDA_OK(cudaMemcpyAsync(&h_status, &hdr->status, 4, cudaMemcpyDeviceToHost, stream));
-  PARD_CUDA_OK(cudaStreamSynchronize(stream));
-  return h_status ? -(int)h_status : PARD_OK;
+  return pard_wait_status(&hdr->status, stream);
 }
