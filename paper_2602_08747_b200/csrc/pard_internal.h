@@ -85,6 +85,8 @@ struct PardTicket {
 };
 void pard_report_init();
 PardTicket pard_report_ticket();
+/* zeroes the status header (256 bytes) of a call, by a kernel that the next one need not wait for to be placed */
+cudaError_t pard_clear_status(void* hdr, cudaStream_t stream);
 /* waits for the answer to `t` (given by the work already enqueued on `stream`); the call's status */
 int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream);
 /* the same behind everything enqueued so far: answers `t` with a kernel of its own */

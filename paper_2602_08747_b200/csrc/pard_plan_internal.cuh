@@ -74,6 +74,22 @@ struct PipeTable {
   const PardPipeDev* const* many;
 };
 
+/* Fills the table for a call whose pipelines have been checked; d_many: room for their addresses in
+ * the workspace, used when they do not fit the arguments. */
+inline int pard_pipe_table(const pard_pipeline_t* const* pipelines, uint32_t n_pipelines, void* d_many, cudaStream_t stream,
+                           PipeTable* out) {
+  out->many = (const PardPipeDev* const*)d_many;
+  if (n_pipelines <= (uint32_t)kFewPipelines) {
+    for (uint32_t i = 0; i < (uint32_t)kFewPipelines; ++i)
+      out->few[i] = i < n_pipelines ? (const PardPipeDev*)pipelines[i]->d_blob : nullptr;
+    return PARD_OK;
+  }
+  std::vector<const PardPipeDev*> h(n_pipelines);
+  for (uint32_t i = 0; i < n_pipelines; ++i) h[i] = (const PardPipeDev*)pipelines[i]->d_blob;
+  PARD_CUDA_OK(cudaMemcpyAsync(d_many, h.data(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
+  return PARD_OK;
+}
+
 /* floor(2^64 / d) + 1 for d >= 2 */
 __device__ __forceinline__ unsigned long long magic64(unsigned long long d) {
   unsigned long long q = ~0ull / d;

@@ -9,7 +9,9 @@
  * window (the same row read `window` places back), so the work is linear in
  * the history length for any window.  All quantities are integers; the two
  * threshold tests are done cross-multiplied in 128 bits. */
-#include "pard_internal.h"
+#include "pard_plan_internal.cuh"
+
+using namespace pard_plan_detail;
 
 namespace {
 
@@ -36,7 +38,7 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
 }
 
 __global__ void __launch_bounds__(256)
-k_update_priority(const PardPipeDev* const* __restrict__ pipes, uint32_t n_pipelines,
+k_update_priority(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
                   const int32_t* __restrict__ pipeline_of_ctx, uint32_t n_ctx, uint32_t S,
                   const int32_t* __restrict__ batch, const int32_t* __restrict__ workers,
                   const uint32_t* __restrict__ arrivals, uint32_t H, uint32_t W, uint32_t interval_us,
@@ -51,7 +53,7 @@ k_update_priority(const PardPipeDev* const* __restrict__ pipes, uint32_t n_pipel
     if (lane == 0) atomicMax(&hdr->status, (uint32_t)(-PARD_EDATA));
     return;
   }
-  const PardPipeDev* p = pipes[pi];
+  const PardPipeDev* p = n_pipelines <= (uint32_t)kFewPipelines ? pipes.few[pi] : pipes.many[pi];
   if (k >= (uint32_t)p->n_stages) return;        /* padding column of the row: left untouched */
   const int32_t B = batch[seg];
   const long long m = workers ? workers[seg] : 1;
@@ -159,12 +161,10 @@ extern "C" int pard_update_priority(const pard_pipeline_t* const* pipelines, uin
     return PARD_ERANGE;
   int dev = -1;
   PARD_CUDA_OK(cudaGetDevice(&dev));
-  std::vector<const PardPipeDev*> h_pipes(n_pipelines);
   for (uint32_t i = 0; i < n_pipelines; ++i) {
     const pard_pipeline_t* p = pipelines[i];
     if (!p || !p->d_blob || p->device != dev) return PARD_EINVAL;
     if (p->n_stages > stage_stride) return PARD_EINVAL;
-    h_pipes[i] = (const PardPipeDev*)p->d_blob;
   }
   if (!d_workspace || ((uintptr_t)d_workspace & 255)) return PARD_EINVAL;
   uint64_t need = 0;
@@ -173,12 +173,13 @@ extern "C" int pard_update_priority(const pard_pipeline_t* const* pipelines, uin
 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   PrioHeader* hdr = (PrioHeader*)d_workspace;
-  const PardPipeDev** d_pipes = (const PardPipeDev**)((char*)d_workspace + sizeof(PrioHeader));
-  PARD_CUDA_OK(cudaMemsetAsync(hdr, 0, sizeof(PrioHeader), stream));
-  PARD_CUDA_OK(cudaMemcpyAsync(d_pipes, h_pipes.data(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
+  PipeTable table;
+  const int trc = pard_pipe_table(pipelines, n_pipelines, (char*)d_workspace + sizeof(PrioHeader), stream, &table);
+  if (trc != PARD_OK) return trc;
+  PARD_CUDA_OK(pard_clear_status(hdr, stream));
   const uint32_t n_seg = n_ctx * (uint32_t)stage_stride;
   PARD_CUDA_OK(launch_pdl(k_update_priority, (n_seg + 7) / 8, 256, 0, stream,
-                          (const PardPipeDev* const*)d_pipes, n_pipelines, d_pipeline_of_ctx, n_ctx,
+                          table, n_pipelines, d_pipeline_of_ctx, n_ctx,
                           (uint32_t)stage_stride, d_batch, d_workers, d_arrivals, n_hist, window, interval_us,
                           d_priority, hdr));
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;

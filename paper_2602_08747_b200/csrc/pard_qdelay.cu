@@ -85,7 +85,7 @@ extern "C" int pard_update_queue_delay(uint32_t n_ctx, int32_t stage_stride, con
   if (workspace_bytes < sizeof(QdHeader)) return PARD_EWORKSPACE;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   QdHeader* hdr = (QdHeader*)d_workspace;
-  PARD_CUDA_OK(cudaMemsetAsync(hdr, 0, sizeof(QdHeader), stream));
+  PARD_CUDA_OK(pard_clear_status(hdr, stream));
   const uint32_t n_rows = n_ctx * (uint32_t)stage_stride;
   PARD_CUDA_OK(launch_pdl(k_queue_delay, (n_rows + 7) / 8, 256, 0, stream, n_rows, (uint32_t)stage_stride,
                           (const long long*)d_now_us, (const long long*)d_sample_time_us, d_sample_delay_us,

@@ -3,7 +3,9 @@
  * planner's own reading of paper Sec. 4.2 (t_e, the expected end of the
  * previous batch; batches run back to back) and records the queueing-delay
  * sample that pard_update_queue_delay averages.  One thread per (ctx, stage). */
-#include "pard_internal.h"
+#include "pard_plan_internal.cuh"
+
+using namespace pard_plan_detail;
 
 namespace {
 
@@ -14,7 +16,7 @@ struct AdvHeader {
 static_assert(sizeof(AdvHeader) == 256, "header is 256 bytes");
 
 __global__ void __launch_bounds__(256)
-k_advance_state(const PardPipeDev* const* __restrict__ pipes, uint32_t n_pipelines,
+k_advance_state(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
                 const int32_t* __restrict__ pipeline_of_ctx, uint32_t n_ctx, uint32_t S,
                 const long long* __restrict__ now_us, const int32_t* __restrict__ batch,
                 const int32_t* __restrict__ workers, const uint32_t* __restrict__ seg_kept,
@@ -29,7 +31,7 @@ k_advance_state(const PardPipeDev* const* __restrict__ pipes, uint32_t n_pipelin
     atomicMax(&hdr->status, (uint32_t)(-PARD_EDATA));
     return;
   }
-  const PardPipeDev* p = pipes[pi];
+  const PardPipeDev* p = n_pipelines <= (uint32_t)kFewPipelines ? pipes.few[pi] : pipes.many[pi];
   if (k >= (uint32_t)p->n_stages) return;        /* padding column of the row: left untouched */
   const int32_t B = batch[seg];
   const long long m = workers ? workers[seg] : 1;
@@ -82,12 +84,10 @@ extern "C" int pard_advance_state(const pard_pipeline_t* const* pipelines, uint3
     return PARD_ERANGE;
   int dev = -1;
   PARD_CUDA_OK(cudaGetDevice(&dev));
-  std::vector<const PardPipeDev*> h_pipes(n_pipelines);
   for (uint32_t i = 0; i < n_pipelines; ++i) {
     const pard_pipeline_t* p = pipelines[i];
     if (!p || !p->d_blob || p->device != dev) return PARD_EINVAL;
     if (p->n_stages > stage_stride) return PARD_EINVAL;
-    h_pipes[i] = (const PardPipeDev*)p->d_blob;
   }
   if (!d_workspace || ((uintptr_t)d_workspace & 255)) return PARD_EINVAL;
   uint64_t need = 0;
@@ -96,12 +96,13 @@ extern "C" int pard_advance_state(const pard_pipeline_t* const* pipelines, uint3
 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   AdvHeader* hdr = (AdvHeader*)d_workspace;
-  const PardPipeDev** d_pipes = (const PardPipeDev**)((char*)d_workspace + sizeof(AdvHeader));
-  PARD_CUDA_OK(cudaMemsetAsync(hdr, 0, sizeof(AdvHeader), stream));
-  PARD_CUDA_OK(cudaMemcpyAsync(d_pipes, h_pipes.data(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
+  PipeTable table;
+  const int trc = pard_pipe_table(pipelines, n_pipelines, (char*)d_workspace + sizeof(AdvHeader), stream, &table);
+  if (trc != PARD_OK) return trc;
+  PARD_CUDA_OK(pard_clear_status(hdr, stream));
   const uint32_t n_seg = n_ctx * (uint32_t)stage_stride;
   PARD_CUDA_OK(launch_pdl(k_advance_state, (n_seg + 255) / 256, 256, 0, stream,
-                          (const PardPipeDev* const*)d_pipes, n_pipelines, d_pipeline_of_ctx, n_ctx,
+                          table, n_pipelines, d_pipeline_of_ctx, n_ctx,
                           (uint32_t)stage_stride, (const long long*)d_now_us, d_batch, d_workers, d_seg_kept,
                           (long long*)d_free_at_us, (long long*)d_sample_time_us, d_sample_delay_us, n_samples,
                           slot, hdr));

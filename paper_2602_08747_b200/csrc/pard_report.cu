@@ -48,7 +48,16 @@ __global__ void k_report(const uint32_t* status, unsigned long long* word, uint3
   pard_report(status, word, ticket);
 }
 
+__global__ void k_clear_status(uint32_t* hdr) {
+  pdl_wait();
+  hdr[threadIdx.x] = 0;
+}
+
 }  // namespace
+
+cudaError_t pard_clear_status(void* hdr, cudaStream_t stream) {
+  return launch_pdl(k_clear_status, 1, 64, 0, stream, (uint32_t*)hdr);
+}
 
 void pard_report_init() {
   if (g_page.load(std::memory_order_acquire)) return;

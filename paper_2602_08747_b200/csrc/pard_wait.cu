@@ -3,19 +3,27 @@
  * samples of the batch wait aggregated over the path's stages, and the sample
  * of rank floor(lambda * M).
  *
- * One block per (ctx, slot).  The block writes its M sums into shared memory
- * (every thread draws the recorded waits of its samples with a counter-based
- * generator, so no state is carried between samples), then finds the rank-th
- * smallest by a radix select over the sums: four rounds of 8 bits from the
- * top, each a shared-memory histogram and a scan of 256 bins by one warp. */
+ * A block takes every G-th slot of one ctx.  The recorded waits of one stage at a time are copied
+ * into shared memory, asynchronously and one row ahead (across slots too), and the draws gather
+ * from there; a thread keeps the sums of its samples in registers.  The rank-th smallest sum: a
+ * histogram over the top 11 of the bits that occur, a scan of it, then the few sums of the one bin
+ * that holds the rank are compared with each other (or, if they are many, split again).
+ * Bound by the integer pipes (multiplications and logic both near 60 % of their cycles, issue slots
+ * at 69 %): of some 35 instructions per draw two thirds are splitmix64.  M = 10,000 on the
+ * 4,500 slots of 256 pipelines (262 M draws): 635 us with a block of its own for every slot of the
+ * stride -- most of them padding, each paying five dependent loads to find its path --, the sums
+ * in shared memory and four rounds of selection over all of them; 425 us like this. */
+#include <algorithm>
 #include <mutex>
 
-#include "pard_internal.h"
+#include "pard_plan_internal.cuh"
+
+using namespace pard_plan_detail;
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr uint32_t kSampleLimit = 1u << 24;      /* recorded waits lie in [0, 2^24) us */
+constexpr uint32_t kSampleBits = 24;             /* recorded waits lie in [0, 2^24) us */
+constexpr uint32_t kSelBits = 11, kSelBins = 1u << kSelBits;
 
 struct WaitHeader {
   uint32_t status;                               /* 0, or the positive value of a pard_status */
@@ -23,144 +31,258 @@ struct WaitHeader {
 };
 static_assert(sizeof(WaitHeader) == 256, "header is 256 bytes");
 
-/* splitmix64 (Steele, Lea, Flood 2014): the finaliser applied to counter + gamma */
-__device__ __forceinline__ unsigned long long splitmix64(unsigned long long x) {
-  unsigned long long z = x + 0x9E3779B97F4A7C15ull;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
+struct WaitArgs {
+  uint32_t n_pipelines;
+  const int32_t* pipeline_of_ctx;
+  uint32_t S, R, M, G, rank;
+  const int32_t* samples;
+  unsigned long long seed;
+  long long* w_out;
+  WaitHeader* hdr;
+};
+
+/* High word of splitmix64 (Steele, Lea, Flood 2014): the finaliser applied to counter + gamma, given
+ * as two words that already hold the sum.  The counters of one slot are neighbours: unless their low
+ * words wrap around inside the slot (SAME_HI is false then) the high word is the same for all draws,
+ * and so is its part of the first product, `fixed`. */
+constexpr unsigned long long kMixA = 0xBF58476D1CE4E5B9ull, kMixB = 0x94D049BB133111EBull;
+__device__ __forceinline__ unsigned long long splitmix_fixed(uint32_t hi) {
+  return (unsigned long long)((hi ^ (hi >> 30)) * (uint32_t)kMixA) << 32;
+}
+__device__ __forceinline__ uint32_t splitmix_hi(uint32_t lo, uint32_t hi, unsigned long long fixed) {
+  const uint32_t l = lo ^ __funnelshift_r(lo, hi, 30);
+  unsigned long long z = (unsigned long long)l * (uint32_t)kMixA + fixed;
+  z += (unsigned long long)(l * (uint32_t)(kMixA >> 32)) << 32;
+  z = (z ^ (z >> 27)) * kMixB;
+  const uint32_t h = (uint32_t)(z >> 32);
+  return h ^ (h >> 31);
 }
 
-/* STAGED: the recorded waits of one stage at a time are copied into shared
- * memory (coalesced) and the draws gather from there, so a slot reads every
- * row of its path once instead of one 32-byte sector per draw.  Needs 8 bytes
- * of shared memory per sample; the direct form needs 4 and gathers from
- * global memory. */
-template <bool STAGED>
-__global__ void __launch_bounds__(kThreads)
-k_estimate_w(const PardPipeDev* const* __restrict__ pipes, uint32_t n_pipelines,
-             const int32_t* __restrict__ pipeline_of_ctx, uint32_t S, uint32_t R,
-             const int32_t* __restrict__ samples, uint32_t M, uint32_t rank, unsigned long long seed,
-             long long* __restrict__ w_out, WaitHeader* __restrict__ hdr) {
-  pdl_wait();
-  extern __shared__ uint32_t s_sum[];            /* [M] aggregated waits of this slot's samples, then
-                                                    (STAGED) [M] recorded waits of the current stage */
-  __shared__ uint32_t s_hist[256];
-  __shared__ int32_t s_path[PARD_MAX_STAGES];
-  __shared__ uint32_t s_prefix, s_rank, s_bad;
+__device__ __forceinline__ void copy_async_16(uint32_t smem, const void* g) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem), "l"(g) : "memory");
+}
+__device__ __forceinline__ void copy_async_4(uint32_t smem, const void* g) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem), "l"(g) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-  const uint32_t c = blockIdx.x / R, slot = blockIdx.x % R;
-  const int32_t pi = pipeline_of_ctx ? pipeline_of_ctx[c] : 0;
-  if (pi < 0 || (uint32_t)pi >= n_pipelines) {
-    if (threadIdx.x == 0) atomicMax(&hdr->status, (uint32_t)(-PARD_EDATA));
-    return;
-  }
-  const PardPipeDev* P = pipes[pi];
-  if ((uint32_t)P->n_slots > R || (uint32_t)P->n_stages > S) {
-    if (threadIdx.x == 0) atomicMax(&hdr->status, (uint32_t)(-PARD_EDATA));
-    return;
-  }
-  if (slot >= (uint32_t)P->n_slots) return;      /* padding of the slot stride: left untouched */
-  const int32_t p0 = P->path_off[slot];
-  const uint32_t L = (uint32_t)(P->path_off[slot + 1] - p0);
-  if (threadIdx.x < L) s_path[threadIdx.x] = P->path_stage[p0 + threadIdx.x];
-  if (threadIdx.x == 0) { s_bad = 0; s_prefix = 0; s_rank = rank; }
-  __syncthreads();
-
-  /* ---- the M samples: one recorded wait per stage of the path, picked at random ---- */
-  const int32_t* ctx_samples = samples + (size_t)c * S * M;
-  const unsigned long long slot_counter = ((unsigned long long)c * R + slot) * M;
-  uint32_t bad = 0;
-  if (STAGED) {
-    uint32_t* s_stage = s_sum + M;
-    for (uint32_t m = threadIdx.x; m < M; m += kThreads) s_sum[m] = 0;
-    for (uint32_t j = 0; j < L; ++j) {
-      const int32_t* row = ctx_samples + (size_t)s_path[j] * M;
-      for (uint32_t m = threadIdx.x; m < M; m += kThreads) s_stage[m] = (uint32_t)__ldg(&row[m]);
-      __syncthreads();
-      for (uint32_t m = threadIdx.x; m < M; m += kThreads) {
-        const uint32_t hi = (uint32_t)(splitmix64(seed + (slot_counter + m) * 64ull + j) >> 32);
-        const uint32_t v = s_stage[__umulhi(hi, M)];
-        bad |= v >= kSampleLimit;
-        s_sum[m] += v;                           /* < 64 * 2^24 = 2^30 when no value is bad */
-      }
-      __syncthreads();
-    }
+/* one row of M recorded waits into shared memory; 16 bytes at a time where rows start on such a boundary */
+template <int THREADS>
+__device__ __forceinline__ void copy_row(uint32_t* dst, const int32_t* row, uint32_t M) {
+  const uint32_t s = (uint32_t)__cvta_generic_to_shared(dst);
+  if (((uintptr_t)row & 15) == 0) {
+    for (uint32_t q = threadIdx.x; q < M / 4; q += THREADS) copy_async_16(s + 16 * q, row + 4 * q);
+    for (uint32_t m = (M & ~3u) + threadIdx.x; m < M; m += THREADS) copy_async_4(s + 4 * m, row + m);
   } else {
-    for (uint32_t m = threadIdx.x; m < M; m += kThreads) {
-      const unsigned long long counter = seed + (slot_counter + m) * 64ull;
-      uint32_t sum = 0;
-      for (uint32_t j = 0; j < L; ++j) {
-        const uint32_t hi = (uint32_t)(splitmix64(counter + j) >> 32);
-        const uint32_t v = (uint32_t)__ldg(&ctx_samples[(size_t)s_path[j] * M + __umulhi(hi, M)]);
-        bad |= v >= kSampleLimit;
-        sum += v;
-      }
-      s_sum[m] = sum;
-    }
+    for (uint32_t m = threadIdx.x; m < M; m += THREADS) copy_async_4(s + 4 * m, row + m);
   }
-  if (bad) s_bad = 1;
-  __syncthreads();
-  if (s_bad) {
-    if (threadIdx.x == 0) atomicMax(&hdr->status, (uint32_t)(-PARD_EDATA));
+}
+
+/* THREADS * PER >= M.  DOUBLE: two row buffers, the next row is copied while this one is drawn from. */
+template <int THREADS, int PER, bool DOUBLE>
+__global__ void __launch_bounds__(THREADS, THREADS >= 1024 ? 1 : 1024 / THREADS)
+k_estimate_w(const __grid_constant__ PipeTable pipes, const WaitArgs a) {
+  pdl_wait();
+  constexpr int WARPS = THREADS / 32, kGroup = 4;
+  static_assert(PER % kGroup == 0, "whole groups");
+  extern __shared__ __align__(16) uint32_t s_rows[];         /* one or two rows, each padded to 16 bytes */
+  __shared__ uint32_t s_hist[kSelBins];
+  __shared__ int32_t s_path[2][PARD_MAX_STAGES];
+  __shared__ uint32_t s_len[2], s_warp[WARPS], s_bin, s_left, s_count;
+  __shared__ uint32_t s_cand[THREADS];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t c = blockIdx.x / a.G, g = blockIdx.x % a.G, M = a.M;
+  const int32_t pi = a.pipeline_of_ctx ? a.pipeline_of_ctx[c] : 0;
+  if (pi < 0 || (uint32_t)pi >= a.n_pipelines) {
+    if (tid == 0) atomicMax(&a.hdr->status, (uint32_t)(-PARD_EDATA));
     return;
   }
-
-  /* ---- radix select: the element of rank s_rank among those that match s_prefix ---- */
+  const PardPipeDev* P = a.n_pipelines <= (uint32_t)kFewPipelines ? pipes.few[pi] : pipes.many[pi];
+  const uint32_t n_slots = (uint32_t)P->n_slots;             /* slots beyond it are padding: left untouched */
+  if (n_slots > a.R || (uint32_t)P->n_stages > a.S) {
+    if (tid == 0) atomicMax(&a.hdr->status, (uint32_t)(-PARD_EDATA));
+    return;
+  }
+  if (g >= n_slots) return;
+  const int32_t* __restrict__ path_off = P->path_off;
+  const int32_t* __restrict__ path_stage = P->path_stage;
+  const int32_t* ctx_samples = a.samples + (size_t)c * a.S * M;
+  const uint32_t row_words = (M + 3) & ~3u;
+  auto load_path = [&](uint32_t slot, uint32_t to) {         /* by one warp */
+    const int32_t p0 = path_off[slot];
+    const uint32_t len = (uint32_t)(path_off[slot + 1] - p0);
+    for (uint32_t k = lane; k < len; k += 32) s_path[to][k] = path_stage[p0 + k];
+    if (lane == 0) s_len[to] = len;
+  };
+  if (warp == 0) load_path(g, 0);
+  __syncthreads();
+  if (DOUBLE) copy_row<THREADS>(s_rows, ctx_samples + (size_t)s_path[0][0] * M, M);
+  uint32_t pb = 0, buf = 0;
 #pragma unroll 1
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    if (threadIdx.x < 256) s_hist[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t prefix = s_prefix;
-    const uint32_t himask = shift == 24 ? 0u : ~0u << (shift + 8);
-    for (uint32_t m = threadIdx.x; m < M; m += kThreads) {
-      const uint32_t v = s_sum[m];
-      if ((v & himask) == prefix) atomicAdd(&s_hist[(v >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {                      /* one warp: bin whose running count passes the rank */
-      const uint32_t lane = threadIdx.x, want = s_rank;
-      uint32_t cnt[8], tot = 0;
+  for (uint32_t slot = g; slot < n_slots; slot += a.G, pb ^= 1) {
+    const uint32_t len = s_len[pb];
+    const bool more = slot + a.G < n_slots;
+    if (more && warp == 0) load_path(slot + a.G, pb ^ 1);    /* read behind the next barrier */
+
+    /* ---- the M samples: one recorded wait per stage of the path, picked at random ---- */
+    uint32_t sum[PER];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) { cnt[i] = s_hist[lane * 8 + i]; tot += cnt[i]; }
-      uint32_t incl = tot;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += t;
+    for (int i = 0; i < PER; ++i) sum[i] = 0;
+    uint32_t seen = 0;
+    const unsigned long long x0 = a.seed + 0x9E3779B97F4A7C15ull + ((unsigned long long)c * a.R + slot) * M * 64ull;
+    const bool same_hi = (uint32_t)x0 <= ~0u - (THREADS * PER + 1u) * 64u;       /* uniform */
+    unsigned long long x = x0 + tid * 64ull;
+#pragma unroll 1
+    for (uint32_t j = 0; j < len; ++j, ++x) {
+      if (!DOUBLE) {
+        __syncthreads();
+        copy_row<THREADS>(s_rows, ctx_samples + (size_t)s_path[pb][j] * M, M);
       }
-      uint32_t before = incl - tot;              /* elements in bins of lower lanes */
-      if (want >= before && want < incl) {       /* exactly one lane holds the rank */
+      copy_async_wait();
+      __syncthreads();
+      if (DOUBLE) {
+        uint32_t* next = s_rows + (buf ^ 1) * row_words;
+        if (j + 1 < len) copy_row<THREADS>(next, ctx_samples + (size_t)s_path[pb][j + 1] * M, M);
+        else if (more) copy_row<THREADS>(next, ctx_samples + (size_t)s_path[pb ^ 1][0] * M, M);
+      }
+      const uint32_t* row = s_rows + (DOUBLE ? buf * row_words : 0u);
+      const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
+      const unsigned long long fixed = splitmix_fixed(hi);
+      auto draw = [&](int i) {
+        const uint32_t step = (uint32_t)i * THREADS * 64u;
+        if (same_hi) return row[__umulhi(splitmix_hi(lo + step, hi, fixed), M)];
+        const uint32_t h = hi + (lo + step < lo ? 1u : 0u);
+        return row[__umulhi(splitmix_hi(lo + step, h, splitmix_fixed(h)), M)];
+      };
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (want >= before && want < before + cnt[i]) {
-            s_prefix = prefix | ((uint32_t)(lane * 8 + i) << shift);
-            s_rank = want - before;
+      for (int i0 = 0; i0 < PER; i0 += kGroup) {
+        if (i0 * THREADS >= (int)M) break;                   /* uniform */
+        if (same_hi && (i0 + kGroup) * THREADS <= (int)M) {  /* every lane has all of the group's samples */
+#pragma unroll
+          for (int i = i0; i < i0 + kGroup; ++i) {
+            const uint32_t v = row[__umulhi(splitmix_hi(lo + (uint32_t)i * THREADS * 64u, hi, fixed), M)];
+            seen |= v;
+            sum[i] += v;                                     /* < 64 * 2^24 = 2^30 when no value is bad */
           }
-          before += cnt[i];
+        } else {
+#pragma unroll
+          for (int i = i0; i < i0 + kGroup; ++i) {
+            const uint32_t v = draw(i);
+            if (tid + i * THREADS < M) seen |= v;
+            sum[i] += v;
+          }
         }
       }
+      if (DOUBLE) buf ^= 1;
     }
-    __syncthreads();
+
+    /* ---- the sum of rank a.rank ---- */
+    uint32_t top = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+      if (tid + i * THREADS < M) top |= sum[i];
+    top = __reduce_or_sync(0xffffffffu, top);
+    if (lane == 0) s_warp[warp] = top;
+    if (__syncthreads_or((int)(seen >> kSampleBits))) {
+      if (tid == 0) atomicMax(&a.hdr->status, (uint32_t)(-PARD_EDATA));
+      copy_async_wait();
+      return;
+    }
+    for (int w = 0; w < WARPS; ++w) top |= s_warp[w];
+    int hi = 32 - __clz((int)top);                           /* bits not settled yet: [0, hi) */
+    uint32_t prefix = 0, left = a.rank;                      /* settled bits of the answer; its rank among the sums that share them */
+    uint32_t answer = 0;
+#pragma unroll 1
+    for (;;) {
+      const int shift = hi > (int)kSelBits ? hi - (int)kSelBits : 0;
+      for (uint32_t b = tid; b < kSelBins; b += THREADS) s_hist[b] = 0;
+      if (tid == 0) s_count = 0;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if ((uint32_t)i * THREADS >= M) break;
+        if (tid + i * THREADS < M && ((sum[i] ^ prefix) >> hi) == 0) atomicAdd(&s_hist[(sum[i] >> shift) & (kSelBins - 1)], 1u);
+      }
+      __syncthreads();
+      /* which bin holds the rank: a thread owns kSelBins / THREADS bins in a row */
+      constexpr int kOwn = kSelBins / THREADS;
+      uint32_t mine = 0;
+#pragma unroll
+      for (int b = 0; b < kOwn; ++b) mine += s_hist[tid * kOwn + b];
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+      }
+      if (lane == 31) s_warp[warp] = incl;
+      __syncthreads();
+      const uint32_t w = lane < (uint32_t)WARPS ? s_warp[lane] : 0u;
+      uint32_t before = incl - mine + __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+      if (left >= before && left < before + mine) {          /* exactly one thread */
+#pragma unroll
+        for (int b = 0; b < kOwn; ++b) {
+          const uint32_t k = s_hist[tid * kOwn + b];
+          if (left >= before && left < before + k) { s_bin = tid * kOwn + b; s_left = left - before; s_count = k; }
+          before += k;
+        }
+      }
+      __syncthreads();
+      const uint32_t count = s_count;
+      prefix |= s_bin << shift;
+      left = s_left;
+      hi = shift;
+      __syncthreads();
+      if (hi == 0) { answer = prefix; break; }
+      if (count > (uint32_t)THREADS) continue;               /* many in one bin: split it */
+      /* few: list them, every one counts those before it */
+      if (tid == 0) s_count = 0;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < PER; ++i) {
+        if ((uint32_t)i * THREADS >= M) break;
+        if (tid + i * THREADS < M && ((sum[i] ^ prefix) >> hi) == 0) s_cand[atomicAdd(&s_count, 1u)] = sum[i];
+      }
+      __syncthreads();
+      if (tid < count) {
+        const uint32_t v = s_cand[tid];
+        uint32_t less = 0, same = 0;
+        for (uint32_t k = 0; k < count; ++k) {
+          less += s_cand[k] < v ? 1u : 0u;
+          same += s_cand[k] == v ? 1u : 0u;
+        }
+        if (left >= less && left < less + same) s_bin = v;   /* equal values write the same */
+      }
+      __syncthreads();
+      answer = s_bin;
+      break;
+    }
+    if (tid == 0) a.w_out[(size_t)c * a.R + slot] = (long long)answer;
   }
-  if (threadIdx.x == 0) w_out[(size_t)c * R + slot] = (long long)s_prefix;
 }
 
-constexpr int kStagedSmemLimit = 112 * 1024;    /* two blocks per multiprocessor */
-constexpr uint32_t kDirectMaxSamples = 2048;    /* rows this short stay in the first-level cache */
+/* Threads and samples per thread by M: the smallest block whose threads keep all sums in 20
+ * registers each (more, smaller blocks hide each other's barriers); beyond 20,480 samples 32
+ * registers and a single row buffer (two rows would not fit). */
+struct WaitShape {
+  void (*kernel)(const PipeTable, const WaitArgs);
+  int threads, rows;
+};
+constexpr int kShapes = 5;
+const WaitShape kShape[kShapes] = {{k_estimate_w<128, 20, true>, 128, 2},  {k_estimate_w<256, 20, true>, 256, 2},
+                                   {k_estimate_w<512, 20, true>, 512, 2},  {k_estimate_w<1024, 20, true>, 1024, 2},
+                                   {k_estimate_w<1024, 32, false>, 1024, 1}};
+inline int shape_of(uint32_t M) { return M <= 2560 ? 0 : M <= 5120 ? 1 : M <= 10240 ? 2 : M <= 20480 ? 3 : 4; }
 
 std::mutex g_attr_mutex;
-int g_attr_bytes[2][64];                         /* per form and device: dynamic shared memory already allowed */
+int g_attr_bytes[kShapes][64];                   /* per shape and device: dynamic shared memory already allowed */
 
-int allow_wait_smem(int dev, bool staged, int bytes) {
-  if (bytes <= 48 * 1024) return PARD_OK;
+int allow_wait_smem(int dev, int shape, int bytes) {
+  if (bytes <= 32 * 1024) return PARD_OK;        /* static and dynamic shared memory together stay below 48 KB */
   std::lock_guard<std::mutex> lock(g_attr_mutex);
-  if (dev >= 0 && dev < 64 && g_attr_bytes[staged][dev] >= bytes) return PARD_OK;
-  if (staged)
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_estimate_w<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  else
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_estimate_w<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  if (dev >= 0 && dev < 64) g_attr_bytes[staged][dev] = bytes;
+  if (dev >= 0 && dev < 64 && g_attr_bytes[shape][dev] >= bytes) return PARD_OK;
+  PARD_CUDA_OK(cudaFuncSetAttribute(kShape[shape].kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  if (dev >= 0 && dev < 64) g_attr_bytes[shape][dev] = bytes;
   return PARD_OK;
 }
 
@@ -190,12 +312,10 @@ extern "C" int pard_estimate_w(const pard_pipeline_t* const* pipelines, uint32_t
     return PARD_ERANGE;
   int dev = -1;
   PARD_CUDA_OK(cudaGetDevice(&dev));
-  std::vector<const PardPipeDev*> h_pipes(n_pipelines);
   for (uint32_t i = 0; i < n_pipelines; ++i) {
     const pard_pipeline_t* p = pipelines[i];
     if (!p || !p->d_blob || p->device != dev) return PARD_EINVAL;
     if (p->n_stages > stage_stride || p->n_slots > slot_stride) return PARD_EINVAL;
-    h_pipes[i] = (const PardPipeDev*)p->d_blob;
   }
   if (!d_workspace || ((uintptr_t)d_workspace & 255)) return PARD_EINVAL;
   uint64_t need = 0;
@@ -204,19 +324,27 @@ extern "C" int pard_estimate_w(const pard_pipeline_t* const* pipelines, uint32_t
 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   WaitHeader* hdr = (WaitHeader*)d_workspace;
-  const PardPipeDev** d_pipes = (const PardPipeDev**)((char*)d_workspace + sizeof(WaitHeader));
-  const bool staged = n_samples > kDirectMaxSamples && 8ull * n_samples <= (uint64_t)kStagedSmemLimit;
-  const int smem = (int)((staged ? 8ull : 4ull) * n_samples);
-  int rc = allow_wait_smem(dev, staged, smem);
+  const int shape = shape_of(n_samples);
+  const int smem = (int)(4u * ((n_samples + 3) & ~3u)) * kShape[shape].rows;
+  int rc = allow_wait_smem(dev, shape, smem);
   if (rc != PARD_OK) return rc;
-  PARD_CUDA_OK(cudaMemsetAsync(hdr, 0, sizeof(WaitHeader), stream));
-  PARD_CUDA_OK(cudaMemcpyAsync(d_pipes, h_pipes.data(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
-  uint64_t rank = (uint64_t)lambda_num * n_samples / lambda_den;
-  if (rank > n_samples - 1) rank = n_samples - 1;
-  PARD_CUDA_OK(launch_pdl(staged ? k_estimate_w<true> : k_estimate_w<false>, n_ctx * (uint32_t)slot_stride, kThreads, (size_t)smem, stream,
-                          (const PardPipeDev* const*)d_pipes, n_pipelines, d_pipeline_of_ctx,
-                          (uint32_t)stage_stride, (uint32_t)slot_stride, d_wait_samples, n_samples,
-                          (uint32_t)rank, (unsigned long long)seed, (long long*)d_w_us, hdr));
+  PipeTable table;
+  rc = pard_pipe_table(pipelines, n_pipelines, (char*)d_workspace + sizeof(WaitHeader), stream, &table);
+  if (rc != PARD_OK) return rc;
+  PARD_CUDA_OK(pard_clear_status(hdr, stream));
+  WaitArgs a = {};
+  a.n_pipelines = n_pipelines; a.pipeline_of_ctx = d_pipeline_of_ctx;
+  a.S = (uint32_t)stage_stride; a.R = (uint32_t)slot_stride; a.M = n_samples;
+  a.samples = d_wait_samples; a.seed = (unsigned long long)seed; a.w_out = (long long*)d_w_us; a.hdr = hdr;
+  const uint64_t rank = (uint64_t)lambda_num * n_samples / lambda_den;
+  a.rank = (uint32_t)std::min<uint64_t>(rank, n_samples - 1);
+  /* blocks per ctx: about thirty rounds of resident blocks in all, so that uneven paths even out;
+   * with few contexts a block per slot */
+  int sms = 148;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const uint64_t blocks = 32ull * (uint64_t)sms * (1024 / kShape[shape].threads);
+  a.G = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)slot_stride, (blocks + n_ctx - 1) / n_ctx));
+  PARD_CUDA_OK(launch_pdl(kShape[shape].kernel, n_ctx * a.G, kShape[shape].threads, (size_t)smem, stream, table, a));
   if (mode & PARD_MODE_NOWAIT) return PARD_OK;
   return pard_wait_status(&hdr->status, stream);
 }

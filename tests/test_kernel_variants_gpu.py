@@ -93,3 +93,20 @@ def test_ranges_of_contexts_in_mixed_order(n_ctx, n):
     check(wl)
     wl.requests["deadline_us"][rng.integers(0, n, size=5)] += 1 << 33      # beyond 32-bit offsets from the first request
     check(wl)
+
+
+# ---- batch-wait estimate: block shapes, ranks inside crowded and sparse bins, counters that wrap ---
+@pytest.mark.parametrize("M", [1, 127, 2560, 2561, 5121, 10_240, 10_241, 20_481, 32_768])
+def test_estimate_w_shapes(M):
+    from tests.gpu_util import run_estimate_w
+    rng = np.random.default_rng(M)
+    wl = inputs.make("C2", n=10)
+    S = wl.state.stage_stride
+    for kind in range(3):
+        s = (rng.integers(0, 1 << 24, size=(1, S, M)) if kind == 0 else np.full((1, S, M), 7) if kind == 1
+             else rng.integers(0, 3, size=(1, S, M)) * 100_000)
+        for num, den, seed in ((1, 10, 5), (0, 1, 2**64 - 1), (1, 1, 2**32 - 0x7F4A7C15 - 100_000)):
+            want = oracle.estimate_w(wl.pipelines, None, 1, S, wl.state.slot_stride, s.astype(np.int32), num, den, seed)
+            rc, got = run_estimate_w(wl, s.astype(np.int32), num, den, seed, fill=0)
+            assert rc == 0
+            assert np.array_equal(got, np.asarray(want).reshape(got.shape))
