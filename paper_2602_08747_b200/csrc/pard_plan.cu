@@ -159,7 +159,7 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     for (uint32_t i = threadIdx.x; i < 2 * n_ctx; i += blockDim.x) s_range[i] = 0;
     __syncthreads();
   }
-  bool time_back = false, pair_back = false;     /* see PlanHeader; looked for until both have been met */
+  bool time_back = false, pair_back = false, pair_seen = false;   /* see PlanHeader; looked for until both have been met */
   uint32_t run_ctx = kNone;
   unsigned long long lmin = ~0ull, lmax = 0;
   bool bad_seen = false;
@@ -208,23 +208,23 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     if (!(time_back && pair_back)) {
       uint4 p = make_uint4(0u, 0u, 0u, 0u);      /* the request before the warp's first one */
       if (first > 0 && first < n) p = __ldg(&req[first - 1]);
-      unsigned long long lastD = ((unsigned long long)p.y << 32) | p.x;
-      uint32_t lastc = p.z;
+      /* one shuffle per row and word: lane 31 hands out the row before, whose last request precedes
+       * lane 0's (rows beyond the array compare as in order) */
 #pragma unroll
       for (int i = 0; i < kPreUn; ++i) {
-        const unsigned long long D = ((unsigned long long)r[i].y << 32) | r[i].x;
-        unsigned long long pD = __shfl_up_sync(0xffffffffu, D, 1);
-        uint32_t pc = __shfl_up_sync(0xffffffffu, r[i].z, 1);
-        if (lane == 0) { pD = lastD; pc = lastc; }
-        if (first + i * 32 + lane < n) {
-          time_back |= D < pD;
-          pair_back |= r[i].z < pc || (r[i].z == pc && D < pD);
+        const uint4 q = i == 0 ? p : r[i > 0 ? i - 1 : 0];
+        const bool give = lane == 31;
+        const unsigned long long D = ((unsigned long long)r[i].y << 32) | r[i].x, qD = ((unsigned long long)q.y << 32) | q.x;
+        const unsigned long long pD = __shfl_sync(0xffffffffu, give ? qD : D, (lane - 1) & 31);
+        const bool in = first + i * 32 + lane < n;
+        time_back |= in && D < pD;
+        if (!pair_back) {                        /* (uniform) */
+          const uint32_t pc = __shfl_sync(0xffffffffu, give ? q.z : r[i].z, (lane - 1) & 31);
+          pair_seen |= in && (r[i].z < pc || (r[i].z == pc && D < pD));
         }
-        lastD = __shfl_sync(0xffffffffu, D, 31);
-        lastc = __shfl_sync(0xffffffffu, r[i].z, 31);
       }
       time_back = __any_sync(0xffffffffu, time_back);
-      pair_back = __any_sync(0xffffffffu, pair_back);
+      pair_back = pair_back || __any_sync(0xffffffffu, pair_seen);
     }
     /* a new chunk usually lies in another ctx than the last one: hand the old one over together */
     if (__any_sync(0xffffffffu, run_ctx != kNone && r[0].z != run_ctx)) warp_flush();
@@ -704,6 +704,29 @@ __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
 }
 
+/* The grid (resident as a whole) meets: every block's writes before are visible to every block
+ * after.  `bar` counts arrivals from zero.  Bounded: about half a second, then PARD_ETIMEOUT and false
+ * in every block. */
+__device__ bool grid_barrier(PlanHeader* hdr, uint32_t* bar, bool withhold = false) {
+  __shared__ uint32_t s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (!withhold) atomicAdd(bar, 1u);      /* (testing aid: a block that never arrives) */
+    uint32_t spins = 0;
+    bool ok = true;
+    while (ld_relaxed(bar) < gridDim.x) {     /* up to about half a second: other work may hold multiprocessors for a while */
+      if (++spins > 8 * kSpinLimit || hdr->aborted) { ok = false; break; }
+      __nanosleep(200);
+    }
+    if (!ok) set_aborted(hdr);
+    __threadfence();
+    s_ok = ok ? 1u : 0u;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
 struct SortSmem {
   unsigned long long keys[kSortTile];
   uint32_t slot[kSortThreads / 32][kBins];    /* counts, then next free tile-local slot per (warp, digit) */
@@ -717,14 +740,14 @@ struct SortSmem {
 };
 
 /* one warp's share of step 1: ITEMS rounds of 32 consecutive elements */
-template <int ITEMS>
+template <int ITEMS, bool L2>
 __device__ __forceinline__ void sort_load_count(unsigned long long (&key)[kItemsHi], const unsigned long long* src,
                                                 uint64_t first, uint32_t n, uint32_t shift, uint32_t* slot_row,
                                                 uint32_t lane, uint32_t dig_mask = 255u) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     const uint64_t j = first + i * 32 + lane;
-    key[i] = j < n ? src[j] : ~0ull;
+    key[i] = j < n ? (L2 ? __ldcg(src + j) : src[j]) : ~0ull;
   }
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) atomicAdd(&slot_row[(uint32_t)(key[i] >> shift) & dig_mask], 1u);
@@ -771,11 +794,11 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, const uint32_t (&bal
   return m;
 }
 
-template <int ITEMS, int BITS>
+template <int ITEMS, int BITS, bool L2>
 __device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[kItemsHi], const unsigned long long* src,
                                                     uint64_t first, uint32_t shift, uint32_t* slot_row, uint32_t lane) {
 #pragma unroll
-  for (int i = 0; i < ITEMS; ++i) key[i] = src[first + i * 32 + lane];
+  for (int i = 0; i < ITEMS; ++i) key[i] = L2 ? __ldcg(src + first + i * 32 + lane) : src[first + i * 32 + lane];
   uint32_t mine = 0;                                     /* lane j: keys of this warp with digit j */
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
@@ -807,13 +830,13 @@ __device__ __forceinline__ void sort_rank_drop_few(const unsigned long long (&ke
 }
 
 /* digit width known at run time only: one instantiation per width */
-template <int ITEMS>
+template <int ITEMS, bool L2>
 __device__ __forceinline__ void sort_load_count_few_n(unsigned long long (&key)[kItemsHi], const unsigned long long* src,
                                                       uint64_t first, uint32_t shift, uint32_t bits, uint32_t* slot_row,
                                                       uint32_t lane) {
   switch (bits) {
-    case 1: sort_load_count_few<ITEMS, 1>(key, src, first, shift, slot_row, lane); break;
-    default: sort_load_count_few<ITEMS, 2>(key, src, first, shift, slot_row, lane); break;
+    case 1: sort_load_count_few<ITEMS, 1, L2>(key, src, first, shift, slot_row, lane); break;
+    default: sort_load_count_few<ITEMS, 2, L2>(key, src, first, shift, slot_row, lane); break;
   }
 }
 template <int ITEMS, int CAP>
@@ -836,28 +859,21 @@ struct CtxTiles {
   uint32_t n_ctx;
 };
 
+/* PERSIST: the block takes tile after tile, and the elements may have been written by other blocks
+ * of the same kernel (they are read from L2).  False: given up, a bounded wait ran out. */
 template <bool PERSIST, bool CTX>
-__global__ void __launch_bounds__(kSortThreads, 2)
-k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf_a,
+__device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf_a,
             unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ hist,
             uint32_t* __restrict__ lookback, uint32_t* __restrict__ lookback_next, uint32_t n,
-            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct) {
-  pdl_wait();
+            uint32_t ibits, uint32_t stall, const CtxTiles& ct) {
   constexpr int WARPS = kSortThreads / 32;
   static_assert(kLoWarps * 32 == kBins, "one look-back thread per digit");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  SortSmem& S = *reinterpret_cast<SortSmem*>(smem_raw);
-
-  if (pass >= hdr->npass || hdr->aborted || sort_is_local(hdr, local_candidate)) return;
   const unsigned long long* src = (pass & 1) ? buf_b : buf_a;
   unsigned long long* dst = (pass & 1) ? buf_a : buf_b;
   hist += pass * kBins;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t lanebit = 1u << lane;
   const uint32_t n_tiles = (uint32_t)(((uint64_t)n + kSortTile - 1) / kSortTile);
-  /* PERSIST: a small grid whose blocks take tile after tile (used where the pass is launched
-   * only as the fallback of the block-local sort and will almost always return at once);
-   * otherwise one tile per block */
   for (;;) {
   if (tid == 0) {
     const uint32_t t = atomicAdd(&hdr->ticket[pass], 1u);
@@ -883,8 +899,8 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   uint32_t gh = (!CTX && tid < kBins) ? hist[tid] : 0; /* count of digit tid in the whole array (in the ctx), needed in step 2 */
   __syncthreads();
   const uint32_t tile = S.tile;
-  if (PERSIST && tile >= n_tiles) return;
-  if (CTX && S.ctx == 0xffffffffu) return;
+  if (!CTX && PERSIST && tile >= n_tiles) return true;
+  if (CTX && S.ctx == 0xffffffffu) return true;
   if (CTX && tid < kBins) gh = ct.hist[((size_t)S.ctx * kMaxPasses + pass) * kBins + tid];
   const uint64_t base = CTX ? (uint64_t)S.base : (uint64_t)tile * kSortTile;
   const uint32_t limit = CTX ? S.limit : n;            /* end of the range the tile belongs to */
@@ -905,10 +921,10 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   const uint32_t dig_mask = CTX ? (1u << dig_bits) - 1 : 255u;
   const bool few = dig_bits <= 2 && base + kSortTile <= (uint64_t)limit;
   if (few) {
-    if (lo_warp) sort_load_count_few_n<kItemsLo>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane);
-    else sort_load_count_few_n<kItemsHi>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane);
-  } else if (lo_warp) sort_load_count<kItemsLo>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask);
-  else sort_load_count<kItemsHi>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask);
+    if (lo_warp) sort_load_count_few_n<kItemsLo, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane);
+    else sort_load_count_few_n<kItemsHi, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane);
+  } else if (lo_warp) sort_load_count<kItemsLo, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask);
+  else sort_load_count<kItemsHi, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask);
   __syncthreads();
 
   /* 2. thread d owns digit d */
@@ -986,7 +1002,7 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   __syncthreads();
   if (S.abort) {
     if (tid == 0) set_aborted(hdr);
-    return;
+    return false;
   }
 
   /* 5. write out */
@@ -997,10 +1013,48 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
     const uint32_t d = (uint32_t)(k >> shift) & dig_mask;
     dst[S.gofs[d] + pos] = k;
   }
-  if (!PERSIST) return;
+  if (!PERSIST) return true;
   __syncthreads();                                     /* the tile buffer and the tables are reused */
   }
 }
+
+/* One pass, one tile per block. */
+template <bool CTX>
+__global__ void __launch_bounds__(kSortThreads, 2)
+k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf_a,
+            unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ hist,
+            uint32_t* __restrict__ lookback, uint32_t* __restrict__ lookback_next, uint32_t n,
+            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (pass >= hdr->npass || hdr->aborted || sort_is_local(hdr, local_candidate)) return;
+  sort_tiles<false, CTX>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
+                         stall, ct);
+}
+
+/* All passes from `pass` on, by a grid that is resident as a whole and meets between them (bounded
+ * waits as in grid_barrier).  How many passes a key needs is only known on the device, and a pass
+ * that finds nothing to do still costs a launch: 2.5 to 4.5 us each, up to seven per call.  At
+ * 2^24 elements a resident grid takes 9 us more per pass than one block per tile (the blocks' loads
+ * no longer start under the write-out of others), so the passes that large calls usually need keep
+ * launches of their own; calls whose tiles are all resident at once do all passes here. */
+template <bool CTX>
+__global__ void __launch_bounds__(kSortThreads, 2)
+k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned long long* buf_b,
+            const uint32_t* __restrict__ hist, uint32_t* lookback, size_t lb_words, uint32_t n,
+            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (hdr->aborted || sort_is_local(hdr, local_candidate)) return;
+  const uint32_t npass = hdr->npass;
+  for (uint32_t p = pass; p < npass; ++p) {
+    if (!sort_tiles<true, CTX>(*reinterpret_cast<SortSmem*>(smem_raw), p, hdr, buf_a, buf_b, hist, lookback + (p & 1) * lb_words,
+                               lookback + ((p + 1) & 1) * lb_words, n, ibits, p == 0 ? stall : 0u, ct))
+      return;
+    if (p + 1 < npass && !grid_barrier(hdr, &hdr->sort_bar[p])) return;
+  }
+}
+
 
 /* First tile of every ctx when the tiles are cut at ctx boundaries: the running sum of
  * ceil(requests of the ctx / kSortTile).  One block. */
@@ -2384,26 +2438,6 @@ k_kept_move(const uint32_t* __restrict__ kept_tmp, const uint32_t* __restrict__ 
  * blocks of 128 threads per multiprocessor), and its blocks meet at counters in the workspace
  * header, each wait bounded like the sort's (PARD_ETIMEOUT, every block gives up, nothing hangs;
  * the bound only bites when other streams keep the multiprocessors full for that long). */
-__device__ bool grid_barrier(PlanHeader* hdr, int k, bool withhold = false) {
-  __shared__ uint32_t s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (!withhold) atomicAdd(&hdr->bar[k], 1u);      /* (testing aid: a block that never arrives) */
-    uint32_t spins = 0;
-    bool ok = true;
-    while (ld_relaxed(&hdr->bar[k]) < gridDim.x) {     /* up to about half a second: other work may hold multiprocessors for a while */
-      if (++spins > 8 * kSpinLimit || hdr->aborted) { ok = false; break; }
-      __nanosleep(200);
-    }
-    if (!ok) set_aborted(hdr);
-    __threadfence();
-    s_ok = ok ? 1u : 0u;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
 template <bool RAW>
 __global__ void __launch_bounds__(kDecThreads, 3)
 k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
@@ -2418,13 +2452,13 @@ k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
   if (hdr->wide || hdr->aborted || !hdr->use_scan) return;
   const uint32_t n_tiles = (n + kDecTile - 1) / kDecTile;
   tile_agg_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, tile_agg);
-  if (!grid_barrier(hdr, 0, stall && blockIdx.x == 0)) return;
+  if (!grid_barrier(hdr, &hdr->bar[0], stall && blockIdx.x == 0)) return;
   if (blockIdx.x == 0) tile_scan_block<RAW, kDecThreads>(tile_agg, n_tiles, carry);
-  if (!grid_barrier(hdr, 1)) return;
+  if (!grid_barrier(hdr, &hdr->bar[1])) return;
   decide_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, carry, out_keep, out_est, out_perm, kept_tmp, seg_kept);
-  if (!grid_barrier(hdr, 2)) return;
+  if (!grid_barrier(hdr, &hdr->bar[2])) return;
   if (blockIdx.x == 0) kept_scan_block<kDecThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
-  if (!grid_barrier(hdr, 3)) return;
+  if (!grid_barrier(hdr, &hdr->bar[3])) return;
   if (out_kept_idx) kept_move_jobs(kept_tmp, seg_off, seg_kept, kept_base, chunk_base, n_seg, out_kept_idx);
 }
 
@@ -3101,12 +3135,10 @@ int allow_sort_smem(int dev) {
   if (done[dev].load(std::memory_order_acquire)) return PARD_OK;    /* every call but the first on a device */
   std::lock_guard<std::mutex> lock(mu);
   if (!done[dev].load(std::memory_order_relaxed)) {
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(SortSmem)));
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(SortSmem)));
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<false, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -3116,6 +3148,14 @@ int allow_sort_smem(int dev) {
     done[dev].store(true, std::memory_order_release);
   }
   return PARD_OK;
+}
+
+/* Passes of the sort that get a launch of their own: none when all tiles are resident at once (or
+ * the sort is only there in case the block-local one does not apply), else three, the 24 bits that
+ * a queue id and the deadlines of about a second take. */
+uint32_t sort_own_passes(uint32_t tiles, uint32_t max_passes, int sms, uint32_t local_cand) {
+  if (local_cand || tiles <= 2u * (uint32_t)sms) return 0;
+  return std::min(3u, max_passes);
 }
 
 bool local_sort_candidate(uint64_t n, uint32_t n_ctx) {
@@ -3306,7 +3346,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
       launch_pdl(k_wide_pack, grid_n, 256, 0, stream, req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, state->d_priority, sbits, ibits,
                  sp, (const PlanHeader*)hdr, (const uint32_t*)order, buf_a, hist);
       for (uint32_t p = 0; p < chunk_passes; ++p)
-        launch_pdl(k_sort_pass<false, false>, L.sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
+        launch_pdl(k_sort_pass<false>, L.sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
                    lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, CtxTiles{});
       launch_pdl(k_wide_chase, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a, buf_b, n32,
                  ibits, sp, (const uint32_t*)order);
@@ -3474,17 +3514,22 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  (mode & PARD_MODE_RAW) ? 1u : 0u, seg_kept, out->d_seg_kept, kept_base, (unsigned long long*)out->d_n_kept,
                  (const uint32_t*)hist, sbits);
   }
+  /* passes with a launch of their own, then the rest in one kernel (see k_sort_rest) */
+  const uint32_t sort_tiles = ctx_sort ? L.lb_tiles : L.sort_tiles;
+  const uint32_t max_passes = ctx_sort ? std::min<uint32_t>(kMaxPasses, (key_sbits + 60 + 7) / 8) : L.max_passes;
+  const uint32_t own_passes = sort_own_passes(sort_tiles, max_passes, sms, local_cand);
+  const uint32_t rest_grid = std::min<uint32_t>(sort_tiles, 2u * (uint32_t)sms);
+  const uint32_t stall = (mode & PARD_MODE_TEST_STALL) && !ctx_sort ? 1u : 0u;
   for (uint32_t p = 0; p < (uint32_t)kMaxPasses; ++p) {
     mark();
-    if (ctx_sort) {
-      if (p < std::min<uint32_t>(kMaxPasses, (key_sbits + 60 + 7) / 8))
-        launch_pdl(k_sort_pass<false, true>, L.lb_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
-                   lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, ctx_tiles);
-    } else if (n > 0 && p < L.max_passes && !local_sure)
-      launch_pdl(local_cand ? k_sort_pass<true, false> : k_sort_pass<false, false>,
-                 local_cand ? std::min<uint32_t>(L.sort_tiles, 2u * (uint32_t)sms) : L.sort_tiles, kSortThreads, sizeof(SortSmem), stream,
-          p, hdr, buf_a, buf_b, hist, lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words,
-          n32, ibits, (p == 0 && (mode & PARD_MODE_TEST_STALL)) ? 1u : 0u, local_cand, CtxTiles{});
+    if (n == 0 || local_sure || p >= max_passes) continue;
+    if (p < own_passes)
+      launch_pdl(ctx_sort ? k_sort_pass<true> : k_sort_pass<false>, sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
+                 buf_b, hist, lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, p == 0 ? stall : 0u,
+                 local_cand, ctx_tiles);
+    else if (p == own_passes)
+      launch_pdl(ctx_sort ? k_sort_rest<true> : k_sort_rest<false>, rest_grid, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
+                 buf_b, hist, lookback, lb_words, n32, ibits, stall, local_cand, ctx_tiles);
   }
   mark();
   if (win_hist) {
@@ -3568,7 +3613,14 @@ extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t sta
   const uint32_t width_kernels = n_seg <= kFoldSegs ? 0 : 1;   /* key_width (+ ctx_span when n > 0) */
   const bool local_cand = local_sort_candidate(n, n_ctx);
   const uint32_t local_kernels = local_cand ? 2 : 0;            /* ctx_ranges, sort_local */
-  const uint32_t passes = make_layout(n, n_ctx, stage_stride).max_passes;
+  const Layout L = make_layout(n, n_ctx, stage_stride);
+  int dev = 0, sms = 148;                                       /* without a device: as on the full chip */
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    sms = 148;
+  }
+  const uint32_t own = sort_own_passes(L.sort_tiles, L.max_passes, sms, local_cand ? 1u : 0u);
+  const uint32_t passes = own + (own < L.max_passes ? 1 : 0);   /* and the kernel that does the rest */
   const bool counted = n > 0 && n_seg <= kHistSegs && !local_cand;
   if (n_ctx == 1 && n > 0 && n <= (uint64_t)kSortTile) *launches = 1;
   else if (n == 0) *launches = 4 + width_kernels;               /* clear, (key_width,) seg_const, seg_win, kept_scan */
