@@ -363,107 +363,22 @@ __global__ void k_key_width(uint32_t sbits, uint32_t ibits, PlanHeader* hdr, uin
   set_key_width(hdr, hdr->span_max, sbits, ibits, key_sbits, arrival_order, priority != 0);
 }
 
-/* The constants of one queue (ctx c, stage k), by one whole warp: lanes over the stage's
- * downstream paths (the path table of the pipeline lists, for every stage, each stage sequence
- * from a successor to a sink).  dmin / dmax: smallest and largest deadline of the ctx, the
- * origins of the queue's deadline offsets.  Every lane returns the same value; *bad is set in
- * the lanes that met an input out of range. */
-__device__ PardSegConst seg_const_warp(const PipeTable& pipes, uint32_t n_pipelines, const pard_queue_state_t& st,
-                                       uint32_t c, uint32_t k, unsigned long long dmin, unsigned long long dmax,
-                                       uint32_t lane, bool* bad_out) {
-  const uint32_t S = (uint32_t)st.stage_stride;
-  PardSegConst out;
-  out.A = 0; out.A_rel = 0; out.d = 1; out.cap = 1; out.d_magic = 0; out.cap_magic = 0;
-  out.narrow = 0; out.lsub = 0; out.dsum = 1;
-  int32_t pi = st.d_pipeline_of_ctx ? st.d_pipeline_of_ctx[c] : 0;
-  bool bad = false;
-  if (pi < 0 || (uint32_t)pi >= n_pipelines) {
-    bad = true;
-  } else {
-    const PardPipeDev* p = n_pipelines <= (uint32_t)kFewPipelines ? pipes.few[pi] : pipes.many[pi];
-    const int64_t* qrow = st.d_q_us + (size_t)c * S;
-    const int32_t* brow = st.d_batch + (size_t)c * S;
-    if (k >= (uint32_t)p->n_stages) {
-      out.narrow = 2;            /* no such stage: a request found in this queue is an input error */
-    } else {
-      int32_t B = brow[k];
-      int64_t m = st.d_workers ? st.d_workers[(size_t)c * S + k] : 1;
-      int64_t now = st.d_now_us[c], fa = st.d_free_at_us[(size_t)c * S + k];
-      if (B < 1 || B > p->bmax[k] || m < 1 || now < 0 || now >= PARD_TIME_LIMIT_US || fa < 0 ||
-          fa >= PARD_TIME_LIMIT_US) {
-        bad = true;
-      } else {
-        const int64_t d = p->lat_us[p->lat_offsets[k] + B - 1];
-        const int32_t s0 = p->stage_slot_off[k], s1 = p->stage_slot_off[k + 1];
-        long long lsub = -1;                              /* every path sum is >= 1 */
-        for (int32_t s = s0 + (int32_t)lane; s < s1; s += 32) {
-          int64_t acc = st.d_w_us ? st.d_w_us[(size_t)c * st.slot_stride + s] : 0;
-          if (acc < 0 || acc >= PARD_TIME_LIMIT_US) { bad = true; acc = 0; }
-          for (int32_t e = p->path_off[s]; e < p->path_off[s + 1]; ++e) {
-            int32_t i = p->path_stage[e];
-            int32_t Bi = brow[i];
-            int64_t qi = qrow[i];
-            if (Bi < 1 || Bi > p->bmax[i] || qi < 0 || qi >= PARD_TIME_LIMIT_US) { bad = true; Bi = 1; qi = 0; }
-            acc += qi + p->lat_us[p->lat_offsets[i] + Bi - 1];
-          }
-          lsub = acc > lsub ? acc : lsub;
-        }
-        for (int o = 16; o; o >>= 1) {                    /* maximum over the paths */
-          long long t = __shfl_xor_sync(0xffffffffu, lsub, o);
-          lsub = t > lsub ? t : lsub;
-        }
-        if (lsub < 0) lsub = 0;                           /* a sink: nothing downstream */
-        int64_t base = now > fa ? now : fa;
-        int64_t cap = (int64_t)B * m;
-        out.d = d;
-        out.cap = (uint32_t)(cap > (int64_t)(1u << 30) ? (int64_t)(1u << 30) : cap);
-        out.A = base + d + lsub;
-        /* A against the origin of the queue's deadline offsets: offsets count up from the ctx's
-         * smallest deadline, or, for a queue served high budget first, down from its largest */
-        const bool high_first = st.d_priority && st.d_priority[(size_t)c * S + k] != 0;
-        out.A_rel = high_first ? (int64_t)dmax - out.A : out.A - (int64_t)dmin;
-        out.d_magic = (d >= 2 && d < ((int64_t)1 << 32)) ? magic64((uint64_t)d) : 0;
-        out.cap_magic = out.cap >= 2 ? magic64(out.cap) : 0;
-        const int64_t lim = (int64_t)1 << 29;
-        out.narrow = (out.d_magic != 0 && d < ((int64_t)1 << 31) && out.A_rel > -lim && out.A_rel < lim) ? 1u : 0u;
-        if (high_first) out.narrow |= kSegHighFirst;
-        out.lsub = lsub;
-        /* all stages' durations at their current batch sizes, for the rule that splits the objective
-         * in proportion to them (a batch size out of range is reported by that stage's own warp) */
-        long long dsum = 0;
-        for (int32_t i = (int32_t)lane; i < p->n_stages; i += 32) {
-          const int32_t Bi = brow[i];
-          dsum += p->lat_us[p->lat_offsets[i] + ((Bi >= 1 && Bi <= p->bmax[i]) ? Bi : 1) - 1];
-        }
-        for (int o = 16; o; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-        out.dsum = dsum;
-      }
-    }
-  }
-  *bad_out = bad;
-  return out;
-}
-
-/* Per-segment constants; one warp per (ctx, stage). */
-__global__ void __launch_bounds__(128)
+/* Per-segment constants; one block per ctx. */
+__global__ void __launch_bounds__(kConstThreads)
 k_seg_const(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
-            pard_queue_state_t st, uint32_t n_ctx,
+            const __grid_constant__ pard_queue_state_t st, uint32_t n_ctx,
             const unsigned long long* __restrict__ ctx_dmin_inv,
             const unsigned long long* __restrict__ ctx_dmax, PardSegConst* __restrict__ ktab,
             PlanHeader* hdr, uint32_t sbits, uint32_t ibits, uint32_t with_key_width, uint32_t arrival_order,
             uint32_t win_hist, uint32_t force_scan, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
             uint32_t key_sbits) {
   pdl_wait();
+  __shared__ CtxScratch scratch;
   const uint32_t S = (uint32_t)st.stage_stride;
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t seg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (seg < n_ctx * S) {                                 /* whole warps take the same side */
-    const uint32_t c = seg / S, k = seg % S;
-    bool bad = false;
-    const PardSegConst out = seg_const_warp(pipes, n_pipelines, st, c, k, ~ctx_dmin_inv[c], ctx_dmax[c], lane, &bad);
-    if (bad) set_status(hdr, PARD_EDATA);
-    if (lane == 0) ktab[seg] = out;
-  }
+  if (ctx_constants(pipes, n_pipelines, st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
+                    ktab + (size_t)blockIdx.x * S, scratch))
+    set_status(hdr, PARD_EDATA);
   /* With few queues the block that finishes last also finds the widest deadline span and with
    * it the width of the sort key (the work of k_ctx_span and k_key_width, without their launches). */
   if (!with_key_width) return;
@@ -2632,19 +2547,15 @@ __device__ __forceinline__ void plan_local(PlanHeader* __restrict__ hdr, const L
   }
   if (Sm.flag_bad && tid == 0) set_status(hdr, PARD_EDATA);
 
-  /* 2. constants of the ctx's queues: worked out here, a warp per stage, when the call is this
+  /* 2. constants of the ctx's queues: worked out here when the call is this
    * one block; else taken from the table k_seg_const has filled for all queues at once (a chain
    * of dependent loads that every block would otherwise wait for) and completed with what hangs
    * on the ctx's deadline range */
   if (a.sort_only) {
     /* the constants come later, from k_seg_const, once every ctx's range is known */
   } else if (single) {
-    for (uint32_t k = warp; k < S; k += WARPS) {
-      bool kbad = false;
-      const PardSegConst K = seg_const_warp(a.pipes, a.n_pipelines, a.st, c, k, dmin, dmax, lane, &kbad);
-      if (kbad) set_status(hdr, PARD_EDATA);
-      if (lane == 0) Sm.K[k] = K;
-    }
+    if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, dmin, dmax, Sm.K, *reinterpret_cast<CtxScratch*>(&Sm.match[0][0])))
+      set_status(hdr, PARD_EDATA);
   } else {
     for (uint32_t k = tid; k < S; k += THREADS) {
       PardSegConst K = a.ktab[(size_t)c * S + k];
@@ -3334,7 +3245,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, sms, stream);
     launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
     launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, 0u, sbits, 1u);
-    launch_pdl(k_seg_const, (L.n_seg + 3) / 4, 128, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
+    launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
                hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
     const uint32_t cw = 64 - ibits;                         /* key bits per super-pass */
     const uint32_t supers = (sbits + 60 + cw - 1) / cw;     /* for the widest legal span; chunks beyond the key are empty */
@@ -3391,7 +3302,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
       launch_pdl(k_clear, 4, 256, 0, stream, (uint4*)(ws + L.hdr), (unsigned long long)(L.hist / 16));
       launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr, 0u, 0u);
       /* the queues' constants; what depends on a ctx's deadline range is added by the ctx's block */
-      launch_pdl(k_seg_const, (L.n_seg + 3) / 4, 128, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax,
+      launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax,
                  ktab, hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
     }
     const bool answered = fused_single && !(mode & PARD_MODE_NOWAIT);
@@ -3429,7 +3340,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     launch_pdl(k_clear, 8, 256, 0, stream, (uint4*)(ws + L.hdr), (unsigned long long)(L.hist / 16));
     launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr, fmt_dbits, sbits);
     launch_pdl(k_plan_local<false, 512>, n_ctx, 512, sizeof(LocalSmem<512>), stream, hdr, la);
-    launch_pdl(k_seg_const, (L.n_seg + 3) / 4, 128, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
+    launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
                hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
     if (L.n_seg >= kManyQueues)
       launch_pdl(k_seg_win_many, ((L.n_seg + 31) / 31 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab,
@@ -3489,7 +3400,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   /* few queues, decided by the planner's own rule in budget order from the start of every queue:
    * the window tables are counted while the requests are packed */
   const bool win_hist = n > 0 && L.n_seg <= kHistSegs && !rule_walk && !state->d_priority && !local_cand && !ctx_sort;
-  launch_pdl(k_seg_const, (L.n_seg + 3) / 4, 128, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
+  launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
              hdr, sbits, ibits, fold_width ? 1u : 0u, arrival_order ? 1u : 0u, win_hist ? 1u : 0u,
              (mode & PARD_MODE_SCAN) ? 1u : 0u, win_off, win_cnt, key_sbits);
   if ((local_cand && !local_sure) || ctx_sort)

@@ -98,6 +98,100 @@ __device__ __forceinline__ unsigned long long magic64(unsigned long long d) {
   return q + 1;
 }
 
+/* The constants of all queues of ctx c, by one block: threads over the stages, then over the (stage,
+ * downstream path) slots, then over the stages again.  dmin / dmax: smallest and largest deadline of
+ * the ctx, the origins of the queues' deadline offsets.  True in the threads that met an input out
+ * of range.  Bound by dependent loads (pipeline -> profile offsets -> durations; slot -> path ->
+ * durations): with the durations of all stages fetched side by side first, a path costs one load
+ * per stage instead of a chain of three.  One warp per queue that walked its paths on its own took
+ * 10 us for 16 queues and 37 us for 32,768. */
+constexpr int kConstThreads = 64;                  /* k_seg_const's blocks; any number of threads will do */
+struct CtxScratch {
+  long long delay[PARD_MAX_STAGES];                /* q_i + d_i(B_i), -1: out of range */
+  long long dur[PARD_MAX_STAGES];                  /* d_i(B_i); d_i(1) for a batch size out of range */
+  unsigned long long lsub[PARD_MAX_STAGES];
+  int32_t slot_off[PARD_MAX_STAGES + 1];
+};
+__device__ __forceinline__ unsigned long long magic64(unsigned long long d);
+
+__device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n_pipelines, const pard_queue_state_t& st, uint32_t c,
+                                              unsigned long long dmin, unsigned long long dmax, PardSegConst* K_out,
+                                              CtxScratch& sc) {
+  const uint32_t S = (uint32_t)st.stage_stride, tid = threadIdx.x, nt = blockDim.x;
+  const int32_t pi = st.d_pipeline_of_ctx ? st.d_pipeline_of_ctx[c] : 0;
+  const PardPipeDev* p = nullptr;
+  if (pi >= 0 && (uint32_t)pi < n_pipelines) p = n_pipelines <= (uint32_t)kFewPipelines ? pipes.few[pi] : pipes.many[pi];
+  bool bad = p == nullptr;
+  const uint32_t stages = p ? (uint32_t)p->n_stages : 0u;   /* <= S: checked on the host */
+  const int32_t n_slots = p ? p->n_slots : 0;
+  const size_t row = (size_t)c * S;
+  for (uint32_t k = tid; k < stages; k += nt) {
+    const int32_t B = st.d_batch[row + k];
+    const int64_t q = st.d_q_us[row + k];
+    const bool ok = B >= 1 && B <= p->bmax[k];
+    const long long d = p->lat_us[p->lat_offsets[k] + (ok ? B : 1) - 1];
+    sc.dur[k] = d;
+    sc.delay[k] = ok && q >= 0 && q < PARD_TIME_LIMIT_US ? q + d : -1;
+    sc.lsub[k] = 0;
+    sc.slot_off[k] = p->stage_slot_off[k];
+  }
+  __syncthreads();
+  for (int32_t s = (int32_t)tid; s < n_slots; s += (int32_t)nt) {
+    int64_t acc = st.d_w_us ? st.d_w_us[(size_t)c * st.slot_stride + s] : 0;
+    if (acc < 0 || acc >= PARD_TIME_LIMIT_US) { bad = true; acc = 0; }
+    const int32_t e1 = p->path_off[s + 1];
+    for (int32_t e = p->path_off[s]; e < e1; ++e) {
+      const long long t = sc.delay[p->path_stage[e]];
+      if (t < 0) bad = true;
+      else acc += t;
+    }
+    uint32_t lo = 0, hi = stages;                  /* the slot's stage: the last whose slots begin at or before s */
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) / 2;
+      if (sc.slot_off[mid] <= s) lo = mid; else hi = mid;
+    }
+    atomicMax(&sc.lsub[lo], (unsigned long long)acc);      /* maximum over the stage's paths; a sink has none: 0 */
+  }
+  __syncthreads();
+  for (uint32_t k = tid; k < S; k += nt) {
+    PardSegConst out;
+    out.A = 0; out.A_rel = 0; out.d = 1; out.cap = 1; out.d_magic = 0; out.cap_magic = 0;
+    out.narrow = 0; out.lsub = 0; out.dsum = 1;
+    if (p && k >= stages) {
+      out.narrow = kSegNoStage;                    /* no such stage: a request found in this queue is an input error */
+    } else if (p) {
+      const int32_t B = st.d_batch[row + k];
+      const int64_t m = st.d_workers ? st.d_workers[row + k] : 1;
+      const int64_t now = st.d_now_us[c], fa = st.d_free_at_us[row + k];
+      if (B < 1 || B > p->bmax[k] || m < 1 || now < 0 || now >= PARD_TIME_LIMIT_US || fa < 0 || fa >= PARD_TIME_LIMIT_US) {
+        bad = true;
+      } else {
+        const int64_t d = sc.dur[k], lsub = (int64_t)sc.lsub[k], base = now > fa ? now : fa, cap = (int64_t)B * m;
+        out.d = d;
+        out.cap = (uint32_t)(cap > (int64_t)(1u << 30) ? (int64_t)(1u << 30) : cap);
+        out.A = base + d + lsub;
+        /* A against the origin of the queue's deadline offsets: offsets count up from the ctx's
+         * smallest deadline, or, for a queue served high budget first, down from its largest */
+        const bool high_first = st.d_priority && st.d_priority[row + k] != 0;
+        out.A_rel = high_first ? (int64_t)dmax - out.A : out.A - (int64_t)dmin;
+        out.d_magic = (d >= 2 && d < ((int64_t)1 << 32)) ? magic64((uint64_t)d) : 0;
+        out.cap_magic = out.cap >= 2 ? magic64(out.cap) : 0;
+        const int64_t lim = (int64_t)1 << 29;
+        out.narrow = (out.d_magic != 0 && d < ((int64_t)1 << 31) && out.A_rel > -lim && out.A_rel < lim) ? kSegNarrow : 0u;
+        if (high_first) out.narrow |= kSegHighFirst;
+        out.lsub = lsub;
+        /* all stages' durations at their current batch sizes, for the rule that splits the objective
+         * in proportion to them */
+        long long dsum = 0;
+        for (uint32_t i = 0; i < stages; ++i) dsum += sc.dur[i];
+        out.dsum = dsum;
+      }
+    }
+    K_out[k] = out;
+  }
+  return bad;
+}
+
 /* floor(x / d) for 32-bit x, with M = floor(2^64 / d) + 1 (d >= 2): exact
  * whenever x * d < 2^64, i.e. for every 32-bit x and d */
 __device__ __forceinline__ uint32_t div_magic32(uint32_t x, unsigned long long M) {
