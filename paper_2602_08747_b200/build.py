@@ -13,7 +13,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpard.so")
 CALL = os.path.join(HERE, "_pardcall.so")
 CALL_SOURCE = os.path.join(CSRC, "pard_pycall.c")
-SOURCES = ["pard_pipeline.cu", "pard_plan.cu", "pard_policy.cu", "pard_goodput.cu", "pard_host.cu",
+SOURCES = ["pard_pipeline.cu", "pard_plan.cu", "pard_local.cu", "pard_policy.cu", "pard_goodput.cu", "pard_host.cu",
            "pard_static.cu", "pard_wait.cu", "pard_priority.cu", "pard_qdelay.cu", "pard_replay.cu",
            "pard_report.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -1,0 +1,1031 @@
+/* One block plans one ctx from start to end.
+ *
+ * For calls whose requests come grouped by ascending ctx with no ctx above 8,192 requests -- one
+ * module's queue planned every few milliseconds, or thousands of decision epochs in one call -- a
+ * block does the whole job for "its" ctx without leaving shared memory:
+ *   1. reads the ctx's requests once into registers; deadline range, input checks, and whether the
+ *      deadlines ever step back;
+ *   2. gets the constants of the ctx's queues (Eq. 3);
+ *   3. sorts (stage | deadline offset | index) in shared memory -- by the stage alone when the
+ *      deadlines are in order already (arrival order, one objective), by up to 16 stages with
+ *      ballots and without counters in shared memory;
+ *   4. finds the batch-window tables (see pard_plan.cu) in the sorted elements: an element whose
+ *      window differs from its neighbour's knows the P of the windows between them;
+ *   5. the tables give every queue's kept count, a look-back over the ctxs before gives the place of
+ *      the ctx's survivors in the output;
+ *   6. decides every request on its own and writes the outputs.
+ * 16 bytes are read and 13 + 4f written per request and nothing else touches global memory.
+ * Queues with more windows than the block's tables hold are decided by the segmented prefix-min
+ * scan over the elements instead.
+ * Bound by shared-memory work and barriers, not by memory.  @@NUM@@ */
+#include <cstddef>
+
+#include "pard_plan_internal.cuh"
+
+using namespace pard_plan_detail;
+
+namespace {
+
+constexpr int kLocThreads = 512;
+constexpr int kLocWarps = kLocThreads / 32;
+constexpr int kLocItems = kLocalTile / kLocThreads;      /* rounds of 32 consecutive requests per warp */
+static_assert(kLocItems == 16 && kLocItems * kLocThreads == kLocalTile, "16 items per thread");
+constexpr uint32_t kTabEntries = 2048;                   /* window-table entries of one ctx */
+constexpr uint32_t kNoWindow = 0xffffu;                  /* window of a request with deadline < A */
+
+struct Tables {                                          /* 4. to 6., in the room of the sort's counters */
+  uint32_t P[kTabEntries];                               /* requests of the queue in earlier windows */
+  int32_t E[kTabEntries];                                /* min of u_t - t over them */
+  uint32_t Kp[kTabEntries];                              /* raw positions: kept requests among them */
+  uint16_t win[kLocalTile];                              /* windows of the sorted elements */
+};
+
+/* The usual ctx after its sort: nothing served high budget first, offsets and A within 31 bits, at most
+ * 32 stages.  The elements fall apart into arrays, queue after queue. */
+struct Split {
+  uint32_t off[kLocalTile];                              /* deadline offsets */
+  uint16_t idx[kLocalTile];                              /* index inside the ctx */
+  uint16_t win[kLocalTile];                              /* window */
+  uint32_t P[kTabEntries];
+  int32_t EK[kTabEntries];                               /* E, or Kp for raw positions */
+  uint32_t U[kTabEntries];                               /* u of the window */
+};
+
+/* Requests that come in order, on their way into the Split form: beside its off and idx. */
+struct Ordered {
+  uint32_t off[kLocalTile];                              /* Split's */
+  uint16_t idx[kLocalTile];
+  uint32_t D[kLocalTile];                                /* low words of the deadlines */
+  uint8_t code[kLocalTile];                              /* stage, then stage | rank << 4 among the 16 requests of one thread */
+  uint16_t place[16][kLocThreads];                       /* [stage][thread]: first place of the thread's requests */
+};
+
+struct LocalSmem {
+  unsigned long long keys[kLocalTile];
+  union {
+    struct {
+      uint32_t slot[kLocWarps][kBins];                   /* running counts, then first place of every (warp, digit) */
+      uint32_t match[kLocWarps][kBins];                  /* lanes currently holding the digit */
+    };
+    Tables tab;
+  };
+  PardSegConst K[PARD_MAX_STAGES];
+  uint32_t stage_first[PARD_MAX_STAGES + 2];
+  uint32_t stage_kept[PARD_MAX_STAGES];
+  uint32_t kept_base[PARD_MAX_STAGES];
+  uint32_t hb_kept[PARD_MAX_STAGES];                     /* high budget first: length of the kept prefix */
+  uint32_t win_off[PARD_MAX_STAGES], win_cnt[PARD_MAX_STAGES];
+  uint32_t row_first[PARD_MAX_STAGES + 1];               /* Split: first row of 32 positions of every queue */
+  uint32_t scan[kLocWarps];
+  uint32_t few[8][kLocWarps];
+  unsigned long long red_min[kLocWarps], red_max[kLocWarps];
+  int32_t wm[kLocWarps];
+  uint32_t wh[kLocWarps];
+  uint32_t ctx, first, cnt, flags, use_scan, base, abort;
+};
+
+static_assert(sizeof(Ordered) <= offsetof(LocalSmem, K) && sizeof(Split) <= offsetof(LocalSmem, K), "inside keys and counters");
+
+/* a thread's sorted element, decoded */
+struct Elem {
+  uint32_t stage, idx, r;
+  long long X;                                           /* deadline - A */
+};
+
+struct Format {                                          /* of the ctx's elements: stage | deadline offset | index */
+  uint32_t ibits, dbits, imask;
+  unsigned long long dmask;
+};
+
+__device__ __forceinline__ Elem decode(unsigned long long e, uint32_t pos, const LocalSmem& Sm, const Format& f) {
+  Elem x;
+  x.stage = (uint32_t)(e >> (f.ibits + f.dbits));
+  x.idx = (uint32_t)e & f.imask;
+  x.r = pos - Sm.stage_first[x.stage];
+  x.X = slack_of((e >> f.ibits) & f.dmask, Sm.K[x.stage]);
+  return x;
+}
+
+/* window of a request of a queue that has a table */
+__device__ __forceinline__ uint32_t window_of(long long X, const PardSegConst& K) {
+  if (X < 0) return kNoWindow;
+  if (((unsigned long long)X >> 32) == 0 && K.d_magic) return div_magic32((uint32_t)X, K.d_magic);
+  return (uint32_t)((unsigned long long)X / (unsigned long long)K.d);
+}
+
+/* 16-bit values of a thread's items, two to a register */
+__device__ __forceinline__ void put16(uint32_t (&v)[kLocItems / 2], int i, uint32_t x) {
+  v[i / 2] = (i & 1) ? (v[i / 2] & 0xffffu) | (x << 16) : x;
+}
+__device__ __forceinline__ uint32_t get16(const uint32_t (&v)[kLocItems / 2], int i) {
+  return (i & 1) ? v[i / 2] >> 16 : v[i / 2] & 0xffffu;
+}
+
+/* One stable pass over 8 bits: ranks first -- the lanes that hold the same digit find each other
+ * through a shared word (atomic OR), the warp's running count gives the rank inside the warp --,
+ * then the counts of all warps become places, then the elements move.  Every warp's counters are
+ * zero at the start and again at the end. */
+__device__ __forceinline__ void pass_byte(unsigned long long (&key)[kLocItems], uint32_t shift, int items, LocalSmem& Sm, uint32_t tid,
+                                          bool reload) {
+  const uint32_t lane = tid & 31, warp = tid >> 5, lanebit = 1u << lane;
+  uint32_t* slot = Sm.slot[warp];
+  uint32_t* match = Sm.match[warp];
+  uint32_t rank[kLocItems / 2];
+#pragma unroll
+  for (int i = 0; i < kLocItems; ++i) {
+    if (i >= items) break;                               /* uniform */
+    const uint32_t d = (uint32_t)(key[i] >> shift) & 255u;
+    atomicOr(&match[d], lanebit);
+    __syncwarp();
+    const uint32_t grp = match[d], below = grp & (lanebit - 1), first = slot[d];
+    __syncwarp();
+    if (below == 0) {                                    /* lowest lane of the group */
+      slot[d] = first + __popc(grp);
+      match[d] = 0;
+    }
+    put16(rank, i, first + __popc(below));
+    __syncwarp();
+  }
+  __syncthreads();
+  uint32_t count = 0, x = 0;
+  if (tid < kBins) {                                     /* thread d owns digit d */
+#pragma unroll
+    for (int w = 0; w < kLocWarps; ++w) count += Sm.slot[w][tid];
+    x = count;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane == 31) Sm.scan[warp] = x;
+  }
+  __syncthreads();
+  if (tid < kBins) {
+    uint32_t place = x - count;
+#pragma unroll
+    for (int w = 0; w < kBins / 32; ++w)
+      if (w < (int)warp) place += Sm.scan[w];
+#pragma unroll
+    for (int w = 0; w < kLocWarps; ++w) {
+      const uint32_t t = Sm.slot[w][tid];
+      Sm.slot[w][tid] = place;
+      place += t;
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kLocItems; ++i) {
+    if (i >= items) break;
+    Sm.keys[slot[(uint32_t)(key[i] >> shift) & 255u] + get16(rank, i)] = key[i];
+  }
+  __syncthreads();
+  if (reload) {
+    const uint32_t wfirst = warp * 32 * (uint32_t)items;
+#pragma unroll
+    for (int i = 0; i < kLocItems; ++i)
+      if (i < items) key[i] = Sm.keys[wfirst + i * 32 + lane];
+    for (uint32_t b = lane; b < kBins; b += 32) slot[b] = 0;
+    __syncwarp();
+  }
+}
+
+/* A stable counting sort by stage of requests that come in order: a thread owns 16 consecutive
+ * requests and counts its stages in the bytes of registers, which also yields every request's rank
+ * among them; the counts, two to a word, are scanned over the block.  HALVES: 8 stages each.  (By
+ * ballots, row after row, the same took three times the instructions.)  Leaves the queues' first
+ * positions in Sm.stage_first. */
+template <int HALVES>
+__device__ __forceinline__ void order_few(LocalSmem& Sm, Ordered& T, uint32_t cnt, uint32_t S) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWords = 2 * HALVES;                     /* 4 stages each */
+  uint32_t n[kWords];
+#pragma unroll
+  for (int h = 0; h < kWords; ++h) n[h] = 0;
+  const uint32_t mine = cnt > tid * 16 ? min(cnt - tid * 16, 16u) : 0u;
+  if (mine) {
+    uint4* codes = reinterpret_cast<uint4*>(&T.code[tid * 16]);
+    const uint4 s = *codes;
+    uint32_t out[4];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t w = i < 4 ? s.x : i < 8 ? s.y : i < 12 ? s.z : s.w;
+      const uint32_t k = (w >> (8 * (i & 3))) & 15u, sh = (k & 3u) * 8, inc = (i < (int)mine ? 1u : 0u) << sh;
+      uint32_t have = n[0];
+#pragma unroll
+      for (int h = 1; h < kWords; ++h) have = (k >> 2) == (uint32_t)h ? n[h] : have;
+      const uint32_t r = (have >> sh) & 0xffu;
+#pragma unroll
+      for (int h = 0; h < kWords; ++h) n[h] += (k >> 2) == (uint32_t)h ? inc : 0u;
+      out[i / 4] = (i & 3) ? out[i / 4] | ((k | r << 4) << (8 * (i & 3))) : (k | r << 4);
+    }
+    *codes = make_uint4(out[0], out[1], out[2], out[3]);
+  }
+  /* stages 4h, 4h+2 in c[2h], 4h+1, 4h+3 in c[2h+1]; counts of at most 8,192 in 16 bits */
+  uint32_t c[2 * kWords], own[2 * kWords];
+#pragma unroll
+  for (int h = 0; h < kWords; ++h) {
+    own[2 * h] = c[2 * h] = n[h] & 0x00ff00ffu;
+    own[2 * h + 1] = c[2 * h + 1] = (n[h] >> 8) & 0x00ff00ffu;
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+    for (int q = 0; q < 2 * kWords; ++q) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, c[q], o);
+      if (lane >= (uint32_t)o) c[q] += y;
+    }
+  if (lane == 31)
+#pragma unroll
+    for (int q = 0; q < 2 * kWords; ++q) Sm.few[q][warp] = c[q];
+  __syncthreads();
+  uint32_t run = 0;                                      /* first position of the stage at hand */
+  uint32_t total[2 * kWords];
+#pragma unroll
+  for (int q = 0; q < 2 * kWords; ++q) {
+    const uint32_t w = lane < (uint32_t)kLocWarps ? Sm.few[q][lane] : 0u;
+    total[q] = __reduce_add_sync(0xffffffffu, w);
+    c[q] += __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) - own[q];     /* before this thread */
+  }
+#pragma unroll
+  for (int k = 0; k < 8 * HALVES; ++k) {
+    const int q = 2 * (k / 4) + (k & 1), sh = (k & 2) ? 16 : 0;
+    T.place[k][tid] = (uint16_t)(run + ((c[q] >> sh) & 0xffffu));
+    if (tid == 0 && k < (int)S) Sm.stage_first[k] = run;
+    run += (total[q] >> sh) & 0xffffu;
+  }
+  if (tid == 0) Sm.stage_first[S] = cnt;
+  __syncthreads();
+}
+
+/* E and, for raw positions, Kp of one queue's table, by one warp; returns the queue's kept count,
+ * which follows from the complete table: n - 1 + min(E, 1), or the running Kp. */
+template <bool RAW>
+__device__ uint32_t table_prefix(Tables& t, uint32_t off, uint32_t cnt, uint32_t cap, uint32_t lane) {
+  uint32_t* P = t.P + off;
+  const uint32_t P0 = P[0];
+  int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;       /* the requests with deadline < A: u = 0 */
+  uint32_t k_carry = 0;
+  if (lane == 0) { t.E[off] = e_carry; if (RAW) t.Kp[off] = 0; }
+  for (uint32_t b0 = 0; b0 + 1 < cnt; b0 += 32) {                /* windows b0.. -> entries b0+1.. */
+    const uint32_t b = b0 + lane;
+    int32_t val = kWinInf;
+    uint32_t kept = 0;
+    if (b + 1 < cnt) {
+      const uint32_t p = P[b], q = P[b + 1];
+      if (q > p) {
+        const uint32_t u = win_u(b, cap);
+        val = (int32_t)u - (int32_t)(q - 1);
+        if (RAW) { const uint32_t top = u < q ? u : q; kept = top > p ? top - p : 0; }
+      }
+    }
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t v2 = __shfl_up_sync(0xffffffffu, val, o);
+      if (lane >= (uint32_t)o) val = min(val, v2);
+      if (RAW) {
+        const uint32_t k2 = __shfl_up_sync(0xffffffffu, kept, o);
+        if (lane >= (uint32_t)o) kept += k2;
+      }
+    }
+    const int32_t e_inc = min(e_carry, val);
+    const uint32_t k_inc = k_carry + kept;
+    if (b + 1 < cnt) { t.E[off + b + 1] = e_inc; if (RAW) t.Kp[off + b + 1] = k_inc; }
+    e_carry = __shfl_sync(0xffffffffu, e_inc, 31);
+    if (RAW) k_carry = __shfl_sync(0xffffffffu, k_inc, 31);
+  }
+  const uint32_t n_q = P[cnt - 1];
+  return n_q == 0 ? 0u : (RAW ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1)));
+}
+
+/* Kept requests of all ctxs before this one: ctxs are taken in ticket order, so a block only waits
+ * for blocks that run already; 32 ctxs per round trip, bounded.  One warp. */
+__device__ bool look_back(PlanHeader* hdr, uint32_t* words, uint32_t c, uint32_t mine, uint32_t lane, uint32_t* before) {
+  if (lane == 0) st_relaxed(words + c, mine | (c == 0 ? kLbIncl : kLbAgg));
+  uint32_t sum = 0, spins = 0;
+  int64_t t = (int64_t)c - 1;
+  while (t >= 0) {
+    const uint32_t v = t - (int64_t)lane >= 0 ? ld_relaxed(words + (t - lane)) : (uint32_t)kLbIncl;
+    const uint32_t unset = __ballot_sync(0xffffffffu, (v >> 30) == 0), incl = __ballot_sync(0xffffffffu, (v & kLbIncl) != 0);
+    const uint32_t stop = incl ? (uint32_t)__ffs(incl) : 32u;      /* lanes 0 .. stop-1 count */
+    const uint32_t ready = unset ? (uint32_t)__ffs(unset) - 1 : 32u;
+    const uint32_t use = min(stop, ready);
+    sum += __reduce_add_sync(0xffffffffu, lane < use ? v & kLbMask : 0u);
+    if (use == stop && incl) break;
+    t -= use;
+    if (use < 32) {
+      if (++spins > kSpinLimit || ld_relaxed(&hdr->aborted)) return false;
+      __nanosleep(40);
+    }
+  }
+  if (lane == 0 && c > 0) st_relaxed(words + c, ((sum + mine) & kLbMask) | kLbIncl);
+  *before = sum;
+  return true;
+}
+
+/* Where the survivors of the ctx's queues go: behind those of the ctxs before (one warp; the others
+ * wait).  False: a wait ran out, here or in another block. */
+__device__ __forceinline__ bool place_survivors(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, uint32_t c) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, S = (uint32_t)a.st.stage_stride;
+  if (tid < 32) {
+    uint32_t run = 0;
+    for (uint32_t k0 = 0; k0 < S; k0 += 32) {
+      const uint32_t k = k0 + lane;
+      const uint32_t v = k < S ? Sm.stage_kept[k] : 0u;
+      uint32_t y = v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= (uint32_t)o) y += z;
+      }
+      if (k < S) {
+        Sm.kept_base[k] = run + y - v;
+        if (a.out_seg_kept) a.out_seg_kept[(size_t)c * S + k] = v;
+      }
+      run += __shfl_sync(0xffffffffu, y, 31);
+    }
+    uint32_t before = 0;
+    if (a.ctx_start && !look_back(hdr, a.kept_words, c, run, lane, &before) && lane == 0) Sm.abort = 1;
+    if (lane == 0) {
+      Sm.base = before;
+      if (c + 1 == a.n_ctx && a.out_n_kept) *a.out_n_kept = before + run;
+    }
+  }
+  __syncthreads();
+  if (Sm.abort && tid == 0 && !ld_relaxed(&hdr->aborted)) {          /* the wait ran out (not: another block gave up) */
+    hdr->aborted = 1;
+    __threadfence();
+    atomicExch(&hdr->status, (uint32_t)(-PARD_ETIMEOUT));
+  }
+  return Sm.abort == 0;
+}
+
+/* Whether the constants allow the Split form; by all threads. */
+__device__ __forceinline__ bool split_fits(const LocalArgs& a, const LocalSmem& Sm, unsigned long long span) {
+  const uint32_t S = (uint32_t)a.st.stage_stride, k = threadIdx.x;
+  bool ok = S <= 32 && !a.st.d_priority && !a.force_scan && (span >> 31) == 0;
+  if (k < S) {
+    const PardSegConst& K = Sm.K[k];
+    const bool none = Sm.stage_first[k] == Sm.stage_first[k + 1];
+    ok = ok && (none || (!(K.narrow & kSegNoStage) && K.d_magic != 0 && K.A_rel > -(1ll << 31) && K.A_rel < (1ll << 31)));
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+/* 4. to 6. in the Split form.  Work is dealt out in rows of 32 positions of one queue, so that the
+ * queue's constants are the same for a whole row.  False: more windows than the tables hold,
+ * nothing has been written. */
+template <bool RAW>
+__device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, uint32_t c, uint32_t first) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t S = (uint32_t)a.st.stage_stride;
+  Split& T = *reinterpret_cast<Split*>(Sm.keys);
+  if (warp == 0) {                                       /* extents: windows up to every queue's last request, rows */
+    uint32_t w = 0, rows = 0;
+    if (lane < S) {
+      const uint32_t lo = Sm.stage_first[lane], hi = Sm.stage_first[lane + 1];
+      const PardSegConst& K = Sm.K[lane];
+      if (hi > lo) {
+        const long long X = (long long)T.off[hi - 1] - K.A_rel;
+        w = X < 0 ? 1u : min(div_magic32((uint32_t)X, K.d_magic), kTabEntries) + 2u;
+        rows = (hi - lo + 31) / 32;
+      }
+    }
+    uint32_t x = w, y = rows;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= (uint32_t)o) { x += p; y += q; }
+    }
+    if (lane < S) {
+      Sm.win_off[lane] = x - w;
+      Sm.win_cnt[lane] = w;
+      Sm.row_first[lane] = y - rows;
+      if (w && x <= kTabEntries) T.P[x - 1] = Sm.stage_first[lane + 1] - Sm.stage_first[lane];   /* the end marker */
+    }
+    if (lane == 31) {
+      Sm.row_first[S] = y;
+      Sm.use_scan = x > kTabEntries ? 1u : 0u;
+    }
+  }
+  __syncthreads();
+  if (Sm.use_scan) return false;
+  /* a warp takes consecutive rows; lane j holds queue j's first row */
+  const uint32_t n_rows = Sm.row_first[S], my_row_first = lane < S ? Sm.row_first[lane] : 0xffffffffu;
+  const uint32_t per = (n_rows + kLocWarps - 1) / kLocWarps, row0 = min(warp * per, n_rows), row1 = min(row0 + per, n_rows);
+  for (uint32_t row = row0; row < row1;) {
+    const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, my_row_first <= row));   /* the queue of the row */
+    const uint32_t lo = Sm.stage_first[k], n = Sm.stage_first[k + 1] - lo, rf = Sm.row_first[k];
+    const uint32_t rows = min(row1, Sm.row_first[k + 1]);
+    const int32_t A = (int32_t)Sm.K[k].A_rel;
+    const unsigned long long magic = Sm.K[k].d_magic;
+    uint32_t* P = T.P + Sm.win_off[k];
+    uint32_t r = (row - rf) * 32 + lane;
+    uint32_t before = kNoWindow;                         /* window of the request ahead of the row */
+    if (row > rf) {
+      const int32_t off = (int32_t)T.off[lo + r - lane - 1];
+      before = off < A ? kNoWindow : div_magic32((uint32_t)off - (uint32_t)A, magic);
+    }
+#pragma unroll 2
+    for (; row < rows; ++row, r += 32) {
+      const bool in = r < n;
+      const int32_t off = in ? (int32_t)T.off[lo + r] : A;
+      const uint32_t b = off < A ? kNoWindow : div_magic32((uint32_t)off - (uint32_t)A, magic);
+      const uint32_t pb = __shfl_sync(0xffffffffu, lane == 31 ? before : b, (lane - 1) & 31);
+      before = b;
+      if (in) {
+        T.win[lo + r] = (uint16_t)b;
+        if (b != pb || r == 0) {                         /* (b == kNoWindow: no entry begins here) */
+          if (b != kNoWindow)
+            for (uint32_t e = r == 0 || pb == kNoWindow ? 0u : pb + 1; e <= b; ++e) P[e] = r;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  /* E (Kp), u and every queue's kept count */
+  for (uint32_t k = warp; k < S; k += kLocWarps) {
+    uint32_t kept = 0;
+    const uint32_t at = Sm.win_off[k], cnt = Sm.win_cnt[k], cap = Sm.K[k].cap;
+    if (cnt) {
+      const uint32_t P0 = T.P[at];
+      int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;       /* the requests with deadline < A: u = 0 */
+      uint32_t k_carry = 0;
+      if (lane == 0) T.EK[at] = RAW ? 0 : e_carry;
+      for (uint32_t b0 = 0; b0 + 1 < cnt; b0 += 32) {                /* windows b0.. -> entries b0+1.. */
+        const uint32_t b = b0 + lane;
+        int32_t val = kWinInf;
+        uint32_t more = 0;
+        if (b + 1 < cnt) {
+          const uint32_t p = T.P[at + b], q = T.P[at + b + 1], u = win_u(b, cap);
+          T.U[at + b] = u;
+          if (q > p) {
+            val = (int32_t)u - (int32_t)(q - 1);
+            const uint32_t top = u < q ? u : q;
+            more = top > p ? top - p : 0;
+          }
+        }
+        for (int o = 1; o < 32; o <<= 1) {
+          if (RAW) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, more, o);
+            if (lane >= (uint32_t)o) more += y;
+          } else {
+            const int32_t y = __shfl_up_sync(0xffffffffu, val, o);
+            if (lane >= (uint32_t)o) val = min(val, y);
+          }
+        }
+        const int32_t out = RAW ? (int32_t)(k_carry + more) : min(e_carry, val);
+        if (b + 1 < cnt) T.EK[at + b + 1] = out;
+        const int32_t last = __shfl_sync(0xffffffffu, out, 31);
+        if (RAW) k_carry = (uint32_t)last; else e_carry = last;
+      }
+      const uint32_t n_q = T.P[at + cnt - 1];
+      kept = RAW ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1));
+    }
+    if (lane == 0) {
+      Sm.stage_kept[k] = kept;
+      if (a.out_seg_off) a.out_seg_off[(size_t)c * S + k] = first + Sm.stage_first[k];
+    }
+  }
+  if (tid == 0 && c + 1 == a.n_ctx && a.out_seg_off) a.out_seg_off[(size_t)a.n_ctx * S] = a.n;
+  __syncthreads();
+  if (!place_survivors(hdr, a, Sm, c)) return true;
+  const uint32_t base = Sm.base;
+  for (uint32_t row = row0; row < row1;) {
+    const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, my_row_first <= row));
+    const uint32_t lo = Sm.stage_first[k], n = Sm.stage_first[k + 1] - lo, rf = Sm.row_first[k];
+    const uint32_t rows = min(row1, Sm.row_first[k + 1]);
+    const PardSegConst& K = Sm.K[k];
+    const long long A = K.A;
+    const unsigned long long cap_magic = K.cap_magic;
+    const uint32_t d = (uint32_t)K.d, woff = Sm.win_off[k];          /* d fits 32 bits: it has a magic number */
+    uint32_t* kept_out = a.out_kept_idx ? a.out_kept_idx + base + Sm.kept_base[k] : nullptr;
+    uint32_t r = (row - rf) * 32 + lane;
+    const size_t g0 = (size_t)first + lo + r;
+    uint8_t* keep_p = a.out_keep + g0;
+    long long* est_p = a.out_est + g0;
+    uint32_t* perm_p = a.out_perm + g0;
+#pragma unroll 2
+    for (; row < rows; ++row, r += 32, keep_p += 32, est_p += 32, perm_p += 32) {
+      if (r >= n) continue;
+      const uint32_t b = T.win[lo + r], idx = first + T.idx[lo + r];
+      uint32_t cpos = RAW ? r : 0u, ahead = 0, u = 0;    /* batch-slot position; kept requests ahead in the queue */
+      if (b != kNoWindow) {
+        const uint32_t P = T.P[woff + b];
+        u = T.U[woff + b];
+        if (RAW) {
+          const uint32_t top = r < u ? r : u;
+          ahead = (uint32_t)T.EK[woff + b] + (top > P ? top - P : 0);
+        } else {
+          int32_t m = T.EK[woff + b];                    /* min over t < r of (u_t - t); values above 1 cannot lower the position */
+          if (r > P) m = min(m, (int32_t)u - (int32_t)(r - 1));
+          cpos = ahead = r == 0 ? 0u : r - 1 + (uint32_t)min(m, 1);
+        }
+      }
+      const bool keep = cpos < u;
+      const uint32_t round = cap_magic ? div_magic32(cpos, cap_magic) : cpos;
+      if (keep && kept_out) kept_out[ahead] = idx;
+      if (a.out_keep) *keep_p = keep ? 1 : 0;
+      if (a.out_est) *est_p = A + (long long)((unsigned long long)round * d);
+      if (a.out_perm) *perm_p = idx;
+    }
+  }
+  return true;
+}
+
+/* 4. to 6. for every other ctx, from the sorted elements as they are. */
+template <bool RAW>
+__device__ __noinline__ void finish_ctx(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, const Format& f, uint32_t c,
+                                        uint32_t first, uint32_t cnt, int items) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t S = (uint32_t)a.st.stage_stride, wfirst = warp * (32 * (uint32_t)items), kshift = f.ibits + f.dbits;
+  const uint32_t n_good = Sm.stage_first[S];             /* requests that passed the checks; the others follow them */
+
+  /* 4. window tables.  Their extents: a queue has windows up to its last element's. */
+  if (warp == 0) {
+    uint32_t run = 0;
+    for (uint32_t k0 = 0; k0 < S; k0 += 32) {
+      const uint32_t k = k0 + lane;
+      uint32_t w = 0;
+      if (k < S) {
+        const uint32_t lo = Sm.stage_first[k], hi = Sm.stage_first[k + 1];
+        const PardSegConst& K = Sm.K[k];
+        if (a.out_seg_off) a.out_seg_off[(size_t)c * S + k] = first + lo;
+        Sm.stage_kept[k] = 0;
+        Sm.hb_kept[k] = hi - lo;
+        if (hi > lo && (K.narrow & kSegNoStage)) set_status(hdr, PARD_EDATA);   /* requests queued at a stage the pipeline lacks */
+        if (hi > lo && !(K.narrow & (kSegNoStage | kSegHighFirst))) {
+          const long long X = slack_of((Sm.keys[hi - 1] >> f.ibits) & f.dmask, K);
+          const unsigned long long nb = X < 0 ? 0ull : (unsigned long long)X / (unsigned long long)K.d + 1;
+          if (nb >= kTabEntries) Sm.use_scan = 1;
+          else w = (uint32_t)nb + 1;
+        }
+      }
+      uint32_t x = w;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+      }
+      if (k < S) { Sm.win_off[k] = run + x - w; Sm.win_cnt[k] = w; }
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0 && (run > kTabEntries || a.force_scan)) Sm.use_scan = 1;
+    if (c + 1 == a.n_ctx && lane == 0 && a.out_seg_off) a.out_seg_off[(size_t)a.n_ctx * S] = a.n;
+  }
+  __syncthreads();
+  /* a queue served high budget first keeps a prefix: its length is the first position r with r >= u_r */
+  if (a.st.d_priority) {
+#pragma unroll 1
+    for (int i = 0; i < items; ++i) {
+      const uint32_t pos = wfirst + i * 32 + lane;
+      if (pos >= n_good) break;
+      const Elem x = decode(Sm.keys[pos], pos, Sm, f);
+      const PardSegConst& K = Sm.K[x.stage];
+      if ((K.narrow & (kSegHighFirst | kSegNoStage)) == kSegHighFirst && x.r >= threshold_u(x.X, K)) atomicMin(&Sm.hb_kept[x.stage], x.r);
+    }
+    __syncthreads();
+  }
+  const bool tables = !Sm.use_scan;
+  if (tables) {
+#pragma unroll 1
+    for (int i = 0; i < items; ++i) {
+      const uint32_t pos = wfirst + i * 32 + lane;
+      const bool in = pos < n_good;
+      Elem x = {};
+      uint32_t b = kNoWindow;
+      bool has = false;
+      if (in) {
+        x = decode(Sm.keys[pos], pos, Sm, f);
+        has = Sm.win_cnt[x.stage] != 0;
+        if (has) b = window_of(x.X, Sm.K[x.stage]);
+      }
+      if (in) Sm.tab.win[pos] = (uint16_t)b;
+      uint32_t pb = __shfl_up_sync(0xffffffffu, b, 1);   /* the neighbour's window, when it is of the same queue */
+      if (lane == 0 && in && has && x.r > 0) pb = window_of(decode(Sm.keys[pos - 1], pos - 1, Sm, f).X, Sm.K[x.stage]);
+      if (has) {
+        const uint32_t off = Sm.win_off[x.stage];
+        const uint32_t from = x.r == 0 || pb == kNoWindow ? 0u : pb + 1;
+        if (b != kNoWindow)
+          for (uint32_t e = from; e <= b; ++e) Sm.tab.P[off + e] = x.r;
+        if (pos + 1 == Sm.stage_first[x.stage + 1]) Sm.tab.P[off + Sm.win_cnt[x.stage] - 1] = x.r + 1;
+      }
+    }
+    __syncthreads();
+    for (uint32_t k = warp; k < S; k += kLocWarps) {
+      uint32_t kept = 0;
+      if (Sm.win_cnt[k]) kept = table_prefix<RAW>(Sm.tab, Sm.win_off[k], Sm.win_cnt[k], Sm.K[k].cap, lane);
+      else if ((Sm.K[k].narrow & (kSegHighFirst | kSegNoStage)) == kSegHighFirst) kept = Sm.hb_kept[k];
+      if (lane == 0) Sm.stage_kept[k] = kept;
+    }
+    __syncthreads();
+  }
+
+  if (tables) {
+    if (!place_survivors(hdr, a, Sm, c)) return;
+    const uint32_t base = Sm.base;
+    /* 6. every request on its own */
+#pragma unroll 2
+    for (int i = 0; i < items; ++i) {
+      const uint32_t pos = wfirst + i * 32 + lane;
+      if (pos >= cnt) break;
+      const unsigned long long e = Sm.keys[pos];
+      const uint32_t idx = (uint32_t)e & f.imask;
+      uint32_t keep = 0;
+      long long est = 0;
+      if (pos < n_good) {
+        const uint32_t stage = (uint32_t)(e >> kshift), r = pos - Sm.stage_first[stage];
+        const PardSegConst& K = Sm.K[stage];
+        uint32_t cpos = RAW ? r : 0u, ahead = 0, u = 0;  /* batch-slot position; kept requests ahead in the queue */
+        const uint32_t b = Sm.tab.win[pos];
+        if (b != kNoWindow) {
+          const uint32_t at = Sm.win_off[stage] + b, P = Sm.tab.P[at];
+          u = win_u(b, K.cap);
+          if (RAW) {
+            const uint32_t top = r < u ? r : u;
+            ahead = Sm.tab.Kp[at] + (top > P ? top - P : 0);
+          } else {
+            int32_t m = Sm.tab.E[at];                    /* min over t < r of (u_t - t); values above 1 cannot lower the position */
+            if (r > P) m = min(m, (int32_t)u - (int32_t)(r - 1));
+            cpos = ahead = r == 0 ? 0u : r - 1 + (uint32_t)min(m, 1);
+          }
+        } else if ((K.narrow & (kSegHighFirst | kSegNoStage)) == kSegHighFirst) {
+          u = threshold_u(slack_of((e >> f.ibits) & f.dmask, K), K);
+          ahead = min(r, Sm.hb_kept[stage]);
+          cpos = RAW ? r : ahead;
+        }
+        keep = cpos < u ? 1u : 0u;
+        const uint32_t round = K.cap_magic ? div_magic32(cpos, K.cap_magic) : cpos;
+        est = K.A + (long long)((unsigned long long)round * (unsigned long long)K.d);
+        if (keep && a.out_kept_idx) a.out_kept_idx[base + Sm.kept_base[stage] + ahead] = idx;
+      }
+      const uint32_t g = first + pos;
+      if (a.out_keep) a.out_keep[g] = (uint8_t)keep;
+      if (a.out_est) a.out_est[g] = est;
+      if (a.out_perm) a.out_perm[g] = idx;
+    }
+    return;
+  }
+
+  /* Too many windows: the segmented scan over the elements, first what every warp's add up to, then
+   * positions and decisions; the survivors' list is packed afterwards. */
+  SegVal run = seg_identity<RAW>();
+  for (int pass = 0; pass < 2; ++pass) {
+    SegVal carry = seg_identity<RAW>();
+    if (pass == 1)
+      for (uint32_t w = 0; w < warp; ++w) {
+        SegVal t; t.m = Sm.wm[w]; t.head = Sm.wh[w];
+        carry = seg_combine<RAW>(carry, t);
+      }
+#pragma unroll 1
+    for (int i = 0; i < items; ++i) {
+      const uint32_t pos = wfirst + i * 32 + lane;
+      const bool in = pos < n_good;
+      Elem x = {};
+      SegVal v = seg_identity<RAW>();
+      uint32_t u = 0;
+      if (in) {
+        x = decode(Sm.keys[pos], pos, Sm, f);
+        const PardSegConst& K = Sm.K[x.stage];
+        u = (K.narrow & kSegNoStage) ? 0u : threshold_u(x.X, K);
+        v.head = x.r == 0 ? 1u : 0u;
+        v.m = RAW ? (x.r < u ? 1 : 0) : (int32_t)u - (int32_t)x.r;
+      }
+      const SegVal inc = warp_scan<RAW>(v, lane);
+      SegVal exc, all;
+      exc.m = __shfl_up_sync(0xffffffffu, inc.m, 1);
+      exc.head = __shfl_up_sync(0xffffffffu, inc.head, 1);
+      if (lane == 0) exc = seg_identity<RAW>();
+      all.m = __shfl_sync(0xffffffffu, inc.m, 31);
+      all.head = __shfl_sync(0xffffffffu, inc.head, 31);
+      if (pass == 0) { run = seg_combine<RAW>(run, all); continue; }
+      const SegVal pre = seg_combine<RAW>(carry, exc);   /* over the earlier requests of the same queue */
+      carry = seg_combine<RAW>(carry, all);
+      if (pos >= cnt) continue;
+      uint32_t keep = 0;
+      long long est = 0;
+      if (in) {
+        const PardSegConst& K = Sm.K[x.stage];
+        uint32_t cpos, ahead;
+        if (RAW) {
+          cpos = x.r;
+          ahead = x.r == 0 ? 0u : (uint32_t)pre.m;
+        } else {
+          const long long cc = (long long)x.r - 1 + pre.m;
+          cpos = x.r == 0 ? 0u : (cc < (long long)x.r ? (uint32_t)cc : x.r);
+          if (K.narrow & kSegHighFirst) cpos = min(x.r, Sm.hb_kept[x.stage]);
+          ahead = cpos;
+        }
+        const uint32_t round = K.cap_magic ? div_magic32(cpos, K.cap_magic) : cpos;
+        est = K.A + (long long)((unsigned long long)round * (unsigned long long)K.d);
+        keep = cpos < u ? 1u : 0u;
+        if (keep && a.kept_tmp) a.kept_tmp[first + Sm.stage_first[x.stage] + ahead] = x.idx;
+        if (pos + 1 == Sm.stage_first[x.stage + 1]) Sm.stage_kept[x.stage] = ahead + keep;     /* the queue's last request */
+      }
+      const uint32_t g = first + pos;
+      if (a.out_keep) a.out_keep[g] = (uint8_t)keep;
+      if (a.out_est) a.out_est[g] = est;
+      if (a.out_perm) a.out_perm[g] = (uint32_t)Sm.keys[pos] & f.imask;
+    }
+    if (pass == 0) {
+      if (lane == 0) { Sm.wm[warp] = run.m; Sm.wh[warp] = run.head; }
+      __syncthreads();
+    }
+  }
+  __threadfence_block();
+  __syncthreads();
+  if (!place_survivors(hdr, a, Sm, c)) return;
+  if (a.out_kept_idx && a.kept_tmp)
+    for (uint32_t k = 0; k < S; ++k) {
+      const uint32_t nk = Sm.stage_kept[k], from = first + Sm.stage_first[k], to = Sm.base + Sm.kept_base[k];
+      for (uint32_t i = tid; i < nk; i += kLocThreads) a.out_kept_idx[to + i] = a.kept_tmp[from + i];
+    }
+}
+
+template <bool RAW>
+__device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t S = (uint32_t)a.st.stage_stride;
+  const bool single = a.ctx_start == nullptr;
+  if (single) {                                          /* the only kernel of the call: the header starts here */
+    if (tid < sizeof(PlanHeader) / 4) reinterpret_cast<uint32_t*>(hdr)[tid] = 0;
+    if (tid == 0) { Sm.ctx = 0; Sm.first = 0; Sm.cnt = a.n; }
+  } else {
+    if (hdr->unsorted || hdr->ctx_too_big) {             /* k_ctx_prep found the promised grouping broken */
+      if (tid == 0 && blockIdx.x == 0) { set_status(hdr, PARD_EDATA); hdr->aborted = 1; }
+      return;
+    }
+    if (tid == 0) {
+      const uint32_t t = atomicAdd(&hdr->ticket[0], 1u);
+      Sm.ctx = t;
+      Sm.first = a.ctx_start[t];
+      Sm.cnt = a.ctx_start[t + 1] - Sm.first;
+    }
+  }
+  if (tid == 0) { Sm.flags = a.st.d_priority ? 4u : 0u; Sm.use_scan = 0; Sm.abort = 0; }
+  __syncthreads();
+  const uint32_t c = Sm.ctx, first = Sm.first, cnt = Sm.cnt;
+  /* every warp owns `items` rounds of 32 consecutive requests: as few as the ctx needs */
+  const int items = (int)((cnt + kLocThreads - 1) / kLocThreads);
+  const uint32_t wfirst = warp * (32 * (uint32_t)items);
+
+  /* 1. the ctx's requests: deadline range, input checks, order.  As long as a warp finds its requests
+   * in order (and the deadlines share their high word: no 71-minute boundary inside the ctx) it only
+   * looks at low words, and leaves them and the stages in shared memory. */
+  Ordered& O = *reinterpret_cast<Ordered*>(Sm.keys);
+  const bool few = S <= 16 && !a.st.d_priority;          /* (queues served high budget first want descending deadlines) */
+  unsigned long long lmin = ~0ull, lmax = 0;
+  uint32_t seen = few ? 0u : 4u;                         /* 1: a request of another ctx, 2: out of range, 4: not in order */
+  if (wfirst < cnt) {
+    const uint4* req = a.req + first;
+    const uint4 p = __ldg(&req[wfirst > 0 ? wfirst - 1 : 0]);
+    const uint32_t high = p.y;
+    uint32_t last = p.x;                                 /* low words of the row before this one, first the request before the warp's */
+    constexpr int kUn = 4;                               /* requests in flight per thread */
+    const uint32_t wend = min(cnt, wfirst + 32 * (uint32_t)items);
+#pragma unroll 1
+    for (uint32_t p0 = wfirst + lane; p0 - lane < wend; p0 += 32 * kUn) {
+      uint4 r[kUn];
+      const bool full = p0 - lane + 32 * kUn <= wend;    /* uniform */
+#pragma unroll
+      for (int u = 0; u < kUn; ++u) {
+        r[u] = make_uint4(0xffffffffu, high, c, 0u);     /* behind every request */
+        if (full || p0 + u * 32 < wend) r[u] = __ldg(&req[p0 + u * 32]);
+      }
+      uint32_t other = 0, top = 0, hi = 0;
+      bool back = false;
+#pragma unroll
+      for (int u = 0; u < kUn; ++u) {
+        const uint32_t px = __shfl_sync(0xffffffffu, lane == 31 ? last : r[u].x, (lane - 1) & 31);
+        last = r[u].x;
+        back |= r[u].x < px;
+        other |= r[u].z ^ c;
+        hi |= r[u].y ^ high;
+        top = max(top, r[u].w & 0xffffu);
+        if (full || p0 + u * 32 < wend) {
+          O.D[p0 + u * 32] = r[u].x;
+          O.code[p0 + u * 32] = (uint8_t)(r[u].w & 15u);
+        }
+      }
+      const bool fine = !back && (other | hi) == 0 && top < S && high < (uint32_t)(PARD_TIME_LIMIT_US >> 32);
+      if (__all_sync(0xffffffffu, fine) && !(seen & 4u)) {
+        /* in order: the lane's range is that of its first and its last request */
+        uint32_t x1 = r[0].x;
+#pragma unroll
+        for (int u = 1; u < kUn; ++u)
+          if (full || p0 + u * 32 < wend) x1 = r[u].x;
+        if (p0 < wend) {
+          const unsigned long long D0 = ((unsigned long long)high << 32) | r[0].x, D1 = ((unsigned long long)high << 32) | x1;
+          lmin = D0 < lmin ? D0 : lmin;
+          lmax = D1 > lmax ? D1 : lmax;
+        }
+      } else {
+        seen |= 4u;
+#pragma unroll
+        for (int u = 0; u < kUn; ++u) {
+          const unsigned long long D = ((unsigned long long)r[u].y << 32) | r[u].x;
+          if (p0 + u * 32 < wend) {
+            if (r[u].z == c && (r[u].w & 0xffffu) < S && D < (unsigned long long)PARD_TIME_LIMIT_US) {
+              lmin = D < lmin ? D : lmin;
+              lmax = D > lmax ? D : lmax;
+            } else {
+              seen |= r[u].z != c ? 3u : 2u;
+            }
+          }
+        }
+      }
+    }
+  }
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, lmin, o), y = __shfl_xor_sync(0xffffffffu, lmax, o);
+    lmin = x < lmin ? x : lmin;
+    lmax = y > lmax ? y : lmax;
+  }
+  seen = __reduce_or_sync(0xffffffffu, seen);
+  if (lane == 0) {
+    Sm.red_min[warp] = lmin;
+    Sm.red_max[warp] = lmax;
+    if (seen) atomicOr(&Sm.flags, seen);
+  }
+  __syncthreads();
+  const uint32_t flags = Sm.flags;
+  if (flags & 1u) {                                      /* not grouped by ctx after all (or, with one ctx, a request of another) */
+    if (tid == 0) { hdr->unsorted = 1; set_status(hdr, PARD_EDATA); hdr->aborted = 1; }
+    return;
+  }
+  unsigned long long dmin = ~0ull, dmax = 0;
+#pragma unroll
+  for (int w = 0; w < kLocWarps; ++w) {
+    dmin = Sm.red_min[w] < dmin ? Sm.red_min[w] : dmin;
+    dmax = Sm.red_max[w] > dmax ? Sm.red_max[w] : dmax;
+  }
+  const bool flagged = flags & 2u;
+  const unsigned long long span = dmin <= dmax ? dmax - dmin : 0ull;
+  const bool in_order = cnt > 0 && !(flags & 6u) && (span >> 31) == 0;
+  Format f;
+  f.ibits = a.ibits;
+  f.dbits = span ? 64u - (uint32_t)__clzll((long long)span) : 0u;
+  f.imask = (1u << a.ibits) - 1;
+  f.dmask = f.dbits >= 64 ? ~0ull : ((1ull << f.dbits) - 1);
+  /* stage field of the elements: requests that failed the checks carry the value S there, so
+   * that they sort behind the ctx's queues; they are reported, never decided */
+  const uint32_t sb = 32u - __clz(flagged ? S : S - 1);  /* bit width of the largest value; __clz(0) = 32 */
+  if (flagged && tid == 0) set_status(hdr, PARD_EDATA);
+
+  /* 2. constants of the ctx's queues: worked out here when the call is this one block; else taken
+   * from the table filled for all queues at once (a chain of dependent loads that every block
+   * would otherwise wait for) and completed with what hangs on the ctx's deadline range */
+  if (single) {
+    if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, dmin, dmax, Sm.K, *reinterpret_cast<CtxScratch*>(Sm.keys))) set_status(hdr, PARD_EDATA);
+  } else {
+    for (uint32_t k = tid; k < S; k += kLocThreads) {
+      PardSegConst K = a.ktab[(size_t)c * S + k];
+      K.A_rel = (K.narrow & kSegHighFirst) ? (int64_t)dmax - K.A : K.A - (int64_t)dmin;
+      Sm.K[k] = K;
+    }
+  }
+
+  /* 3. elements, sorted */
+  if (in_order) {
+    if (S <= 8) order_few<1>(Sm, O, cnt, S);
+    else order_few<2>(Sm, O, cnt, S);
+    if (split_fits(a, Sm, span)) {
+#pragma unroll 4
+      for (int i = 0; i < items; ++i) {
+        const uint32_t pos = wfirst + i * 32 + lane;
+        if (pos < cnt) {
+          const uint32_t code = O.code[pos], at = O.place[code & 15u][pos >> 4] + (code >> 4);
+          O.off[at] = O.D[pos] - (uint32_t)dmin;
+          O.idx[at] = (uint16_t)pos;
+        }
+      }
+      __syncthreads();
+      if (finish_split<RAW>(hdr, a, Sm, c, first)) return;
+    }
+  }
+  if (sb + f.dbits + f.ibits > 64) {         /* the element does not fit 64 bits */
+    if (tid == 0) { hdr->wide = 1; set_status(hdr, PARD_ERANGE); hdr->aborted = 1; }
+    return;
+  }
+  {
+    unsigned long long key[kLocItems];
+#pragma unroll
+    for (int i = 0; i < kLocItems; ++i) {
+      if (i >= items) break;
+      const uint32_t pos = wfirst + i * 32 + lane;
+      key[i] = ~0ull;                                    /* padding sorts last */
+      if (pos < cnt) {
+        const uint4 r = __ldg(&a.req[first + pos]);
+        const unsigned long long D = ((unsigned long long)r.y << 32) | r.x;
+        const uint32_t stage = r.w & 0xffffu, j = first + pos;
+        if (stage < S && D < (unsigned long long)PARD_TIME_LIMIT_US) {
+          const bool high_first = a.st.d_priority && a.st.d_priority[(size_t)c * S + stage] != 0;
+          key[i] = ((((unsigned long long)stage << f.dbits) | ((high_first ? dmax - D : D - dmin) & f.dmask)) << f.ibits) | j;
+        } else {
+          key[i] = (((unsigned long long)S << f.dbits) << f.ibits) | j;
+        }
+      }
+    }
+    __syncthreads();                                     /* the room of the counters has been in use */
+    for (uint32_t i = tid; i < 2 * kLocWarps * kBins; i += kLocThreads) (&Sm.slot[0][0])[i] = 0;
+    __syncthreads();
+    const uint32_t skip = (flags & 4u) ? 0u : f.dbits, passes = (f.dbits - skip + sb + 7) / 8;
+    for (uint32_t p = 0; p < passes; ++p) pass_byte(key, f.ibits + skip + 8 * p, items, Sm, tid, p + 1 < passes);
+    if (passes == 0) {
+#pragma unroll
+      for (int i = 0; i < kLocItems; ++i)
+        if (i < items) Sm.keys[wfirst + i * 32 + lane] = key[i];
+      __syncthreads();
+    }
+  }
+
+  /* queue boundaries: where the stage changes between neighbours */
+  const uint32_t kshift = f.ibits + f.dbits;
+#pragma unroll 1
+  for (int i = 0; i < items; ++i) {
+    const uint32_t pos = wfirst + i * 32 + lane;
+    if (pos >= cnt) break;
+    const uint32_t k1 = (uint32_t)(Sm.keys[pos] >> kshift);
+    const uint32_t k0 = pos ? (uint32_t)(Sm.keys[pos - 1] >> kshift) + 1 : 0u;
+    for (uint32_t k = k0; k <= k1; ++k) Sm.stage_first[k] = pos;
+    if (pos + 1 == cnt)
+      for (uint32_t k = k1 + 1; k <= S; ++k) Sm.stage_first[k] = cnt;
+  }
+  if (cnt == 0)
+    for (uint32_t k = tid; k <= S; k += kLocThreads) Sm.stage_first[k] = 0;
+  __syncthreads();
+  if (Sm.stage_first[S] == cnt && split_fits(a, Sm, span)) {
+    /* the elements apart, in place */
+    Split& T = *reinterpret_cast<Split*>(Sm.keys);
+    unsigned long long e[kLocItems];
+#pragma unroll
+    for (int i = 0; i < kLocItems; ++i)
+      if (i < items) e[i] = Sm.keys[wfirst + i * 32 + lane];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kLocItems; ++i) {
+      if (i >= items) break;
+      const uint32_t pos = wfirst + i * 32 + lane;
+      if (pos < cnt) {
+        T.off[pos] = (uint32_t)((e[i] >> f.ibits) & f.dmask);
+        T.idx[pos] = (uint16_t)(((uint32_t)e[i] & f.imask) - first);
+      }
+    }
+    __syncthreads();
+    if (finish_split<RAW>(hdr, a, Sm, c, first)) return;
+#pragma unroll
+    for (int i = 0; i < kLocItems; ++i)                  /* too many windows: as they were */
+      if (i < items) Sm.keys[wfirst + i * 32 + lane] = e[i];
+    __syncthreads();
+  }
+  finish_ctx<RAW>(hdr, a, Sm, f, c, first, cnt, items);
+}
+
+template <bool RAW>
+__global__ void __launch_bounds__(kLocThreads, 2)
+k_plan_local(PlanHeader* __restrict__ hdr, const __grid_constant__ LocalArgs a) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  plan_ctx<RAW>(hdr, a, *reinterpret_cast<LocalSmem*>(smem_raw));
+  if (a.answer.word) {
+    __syncthreads();
+    if (threadIdx.x == 0) pard_report(&hdr->status, a.answer.word, a.answer.ticket);
+  }
+}
+
+/* What the blocks of a grouped call need beforehand: the constants of all queues (a block per ctx)
+ * and where every ctx begins (a warp per ctx, in further blocks of the same launch): the first request
+ * whose ctx is >= c, by a 32-ary search.  Whether the requests do come in ctx order is settled by
+ * k_plan_local, where every block checks that its range holds requests of its ctx only; that test is
+ * complete as long as the boundaries never step back and the ranges cover all requests, which is
+ * checked here. */
+__global__ void __launch_bounds__(kConstThreads)
+k_ctx_prep(const __grid_constant__ LocalArgs a, PardSegConst* __restrict__ ktab, uint32_t* __restrict__ ctx_start, PlanHeader* hdr) {
+  pdl_wait();
+  __shared__ CtxScratch scratch;
+  if (blockIdx.x < a.n_ctx) {
+    if (ctx_constants(a.pipes, a.n_pipelines, a.st, blockIdx.x, 0, 0, ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch))
+      set_status(hdr, PARD_EDATA);
+    return;
+  }
+  const uint32_t c = (blockIdx.x - a.n_ctx) * (kConstThreads / 32) + (threadIdx.x >> 5);
+  if (c <= a.n_ctx) ctx_range_search(a.req, a.n, a.n_ctx, c, ctx_start, hdr, kLocalTile);
+}
+
+}  // namespace
+
+namespace pard_plan_detail {
+
+int allow_local_smem() {
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
+  return PARD_OK;
+}
+
+int launch_ctx_prep(const LocalArgs& a, PardSegConst* ktab, uint32_t* ctx_start, PlanHeader* hdr, cudaStream_t stream) {
+  const uint32_t per = kConstThreads / 32;
+  PARD_CUDA_OK(launch_pdl(k_ctx_prep, a.n_ctx + (a.n_ctx + 1 + per - 1) / per, kConstThreads, 0, stream, a, ktab, ctx_start, hdr));
+  return PARD_OK;
+}
+
+int launch_plan_local(const LocalArgs& a, PlanHeader* hdr, bool raw, cudaStream_t stream) {
+  PARD_CUDA_OK(launch_pdl(raw ? k_plan_local<true> : k_plan_local<false>, a.ctx_start ? a.n_ctx : 1u, kLocThreads, sizeof(LocalSmem),
+                          stream, hdr, a));
+  return PARD_OK;
+}
+
+}  // namespace pard_plan_detail

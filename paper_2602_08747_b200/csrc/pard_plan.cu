@@ -609,16 +609,6 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
  *   5. the buffer is written out, run by run, to the digit's global range.
  * Large tiles keep the number of tiles in flight, and with it the depth of the
  * look-back, small. */
-/* loads and stores of look-back words: relaxed, device scope (other blocks write them) */
-__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
-}
-
 /* The grid (resident as a whole) meets: every block's writes before are visible to every block
  * after.  `bar` counts arrivals from zero.  Bounded: about half a second, then PARD_ETIMEOUT and false
  * in every block. */
@@ -1081,46 +1071,15 @@ k_pack_ctx(const uint4* __restrict__ req, uint32_t S, const unsigned long long* 
  * the device adds what only it can see.  A call with a single ctx of at most kSortTile requests
  * needs no test at all: its one block is certain, and neither the range search nor the global
  * passes are launched -- the case of one module's queue planned every few milliseconds. */
-/* Where every ctx would begin if the requests came in ascending ctx order: the first request
- * whose ctx is >= c, by a 32-ary search, one warp per ctx.  Whether they do come in that order
- * is settled by k_sort_local, where every block checks that its range holds requests of its ctx
- * only; that test is complete as long as the boundaries never step back and the ranges cover
- * all requests, which is checked here. */
+/* Where every ctx would begin if the requests came in ascending ctx order, one warp per ctx.  Whether
+ * they do is settled by k_sort_local (k_pack_ctx), where every block checks that its range holds
+ * requests of its ctx only. */
 __global__ void __launch_bounds__(256)
 k_ctx_ranges(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t* __restrict__ ctx_start,
-             PlanHeader* hdr, uint32_t fmt_dbits, uint32_t sbits) {
+             PlanHeader* hdr) {
   pdl_wait();
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t lane = threadIdx.x & 31;
-  if (c > n_ctx) return;                         /* whole warps leave together */
-  if (c == 0 && lane == 0 && fmt_dbits) {        /* the element format is fixed by the host: no key-width step */
-    hdr->dbits = fmt_dbits;
-    hdr->keybits = sbits + fmt_dbits;
-    hdr->npass = 0;                              /* the sorted elements are in the first buffer */
-  }
-  uint32_t lo[2] = {0, 0}, hi[2] = {n, n};       /* first request whose ctx is >= c, >= c + 1 */
-  while (lo[0] < hi[0] || lo[1] < hi[1]) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      if (lo[q] < hi[q]) {                       /* uniform across the warp */
-        const uint32_t span = hi[q] - lo[q];
-        const uint32_t p = lo[q] + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* lo <= p < hi */
-        const bool less = __ldg(&req[p]).z < c + q;
-        const uint32_t k = __popc(__ballot_sync(0xffffffffu, less));
-        const uint32_t p_below = __shfl_sync(0xffffffffu, p, k > 0 ? k - 1 : 0);
-        const uint32_t p_at = __shfl_sync(0xffffffffu, p, k < 32 ? k : 31);
-        if (k > 0) lo[q] = p_below + 1;
-        if (k < 32) hi[q] = p_at;
-      }
-    }
-  }
-  if (lane != 0) return;
-  ctx_start[c] = lo[0];
-  if (c == n_ctx && lo[0] != n) hdr->unsorted = 1;      /* requests past the last ctx's range (ctx out of range) */
-  if (c < n_ctx) {
-    if (lo[1] < lo[0]) hdr->unsorted = 1;
-    else if (lo[1] - lo[0] > (uint32_t)kSortTile) hdr->ctx_too_big = 1;
-  }
+  if (c <= n_ctx) ctx_range_search(req, n, n_ctx, c, ctx_start, hdr, (uint32_t)kSortTile);   /* whole warps stay together */
 }
 
 /* One block per ctx: the ctx's requests, read from the caller's array, turned into the sort
@@ -1238,28 +1197,6 @@ k_sort_local(PlanHeader* __restrict__ hdr, uint32_t candidate, const uint4* __re
 /* ------------------------------------------------------------------------ */
 /* decision pass over the sorted elements                                    */
 /* ------------------------------------------------------------------------ */
-struct SegVal {            /* value of a segmented running reduction */
-  int32_t m;               /* admitted mode: minimum of u_t - t; raw mode: number of kept requests;
-                              over the elements since the last queue head (or since the span's start) */
-  uint32_t head;           /* a queue head lies inside the span */
-};
-
-template <bool RAW>
-__device__ __forceinline__ SegVal seg_identity() {
-  SegVal a;
-  a.m = RAW ? 0 : 0x7fffffff;
-  a.head = 0;
-  return a;
-}
-
-template <bool RAW>
-__device__ __forceinline__ SegVal seg_combine(SegVal left, SegVal right) {
-  SegVal r;
-  r.m = right.head ? right.m : (RAW ? left.m + right.m : min(left.m, right.m));
-  r.head = left.head | right.head;
-  return r;
-}
-
 __device__ __forceinline__ unsigned long long pack_val(SegVal a, unsigned long long state) {
   return state | ((unsigned long long)a.head << 32) | (uint32_t)a.m;
 }
@@ -1375,19 +1312,6 @@ __device__ __forceinline__ TileCtx make_tile_ctx(const PlanHeader* hdr, const un
   T.narrow = dbits <= 29 || (hdr->span_max >> 29) == 0;
   T.hdr = const_cast<PlanHeader*>(hdr);
   return T;
-}
-
-/* Inclusive segmented warp scan of the threads' values (in lane order). */
-template <bool RAW>
-__device__ __forceinline__ SegVal warp_scan(SegVal v, uint32_t lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    SegVal l;
-    l.m = __shfl_up_sync(0xffffffffu, v.m, o);
-    l.head = __shfl_up_sync(0xffffffffu, v.head, o);
-    if (lane >= (uint32_t)o) v = seg_combine<RAW>(l, v);
-  }
-  return v;
 }
 
 /* Exclusive segmented scan of the tile aggregates by one block, eight tiles
@@ -1756,17 +1680,10 @@ struct __align__(16) WinEntry {
   uint32_t Kp;     /* raw mode: kept requests among them                          */
   uint32_t pad;
 };
-constexpr int32_t kWinInf = 0x7fffffff;
 constexpr uint32_t kWinMaxPerSeg = 4096;
 constexpr uint32_t kManyQueues = 8192;     /* from this many queues on a lane, not a warp, handles a queue in k_seg_win_many */
 constexpr uint32_t kWinLongQueue = 8192;   /* above this a window boundary is searched by a whole warp, else by one lane */
 
-
-/* u of window b (the saturation of threshold_u) */
-__device__ __forceinline__ uint32_t win_u(uint32_t b, uint32_t cap) {
-  const unsigned long long u = (unsigned long long)(b + 1) * cap;
-  return u > kUClamp ? kUClamp : (uint32_t)u;
-}
 
 /* window of a non-negative X = D - A */
 __device__ __forceinline__ unsigned long long win_of(unsigned long long X, const PardSegConst& K) {
@@ -2336,14 +2253,6 @@ __device__ __forceinline__ void kept_move_jobs(const uint32_t* __restrict__ kept
   }
 }
 
-__global__ void __launch_bounds__(256)
-k_kept_move(const uint32_t* __restrict__ kept_tmp, const uint32_t* __restrict__ seg_off,
-            const uint32_t* __restrict__ seg_kept, const uint32_t* __restrict__ kept_base,
-            const uint32_t* __restrict__ chunk_base, uint32_t n_seg, uint32_t* __restrict__ out_kept_idx) {
-  pdl_wait();
-  kept_move_jobs(kept_tmp, seg_off, seg_kept, kept_base, chunk_base, n_seg, out_kept_idx);
-}
-
 /* The decision by scanning, from the sorted elements to the packed survivors, as ONE kernel: the
  * fallback for calls whose queues have too many batch windows for the tables (and what
  * PARD_MODE_SCAN asks for).  Launched on every call; returns at once when the tables did the
@@ -2375,516 +2284,6 @@ k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
   if (blockIdx.x == 0) kept_scan_block<kDecThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
   if (!grid_barrier(hdr, &hdr->bar[3])) return;
   if (out_kept_idx) kept_move_jobs(kept_tmp, seg_off, seg_kept, kept_base, chunk_base, n_seg, out_kept_idx);
-}
-
-/* ------------------------------------------------------------------------ */
-/* one block plans one ctx from start to end                                 */
-/* ------------------------------------------------------------------------ */
-/* For calls whose requests come grouped by ascending ctx with no ctx above a sort tile -- one
- * module's queue planned every few milliseconds, or many decision epochs in one call -- a block
- * does the whole job for "its" ctx without leaving shared memory: it reads the ctx's requests
- * once, finds the ctx's deadline range, computes the constants of the ctx's queues (Eq. 3),
- * sorts (radix passes over the stage and deadline bits, as k_sort_local), finds every request's
- * admitted position by a segmented scan over the sorted elements, and writes the outputs: 16
- * bytes read and 13 + 4f written per request, no element ever stored to global memory, no window
- * table, no search.  The scan runs twice over the elements, which stay in shared memory: once
- * for the warps' aggregates, once for the positions.  With a single ctx the block also packs the
- * survivors (the whole call is one launch); with several, k_kept_scan and k_kept_move follow. */
-struct LocalArgs {
-  const uint4* req;
-  const uint32_t* ctx_start;       /* NULL: the call has one ctx */
-  uint32_t n, n_ctx, ibits, raw;
-  PipeTable pipes;
-  uint32_t n_pipelines;
-  pard_queue_state_t st;
-  uint8_t* out_keep;
-  long long* out_est;
-  uint32_t* out_perm;
-  uint32_t* out_kept_idx;          /* used directly only with one ctx */
-  unsigned long long* out_n_kept;
-  uint32_t* out_seg_off;
-  uint32_t* out_seg_kept;
-  const PardSegConst* ktab;        /* several ctx: the queues' constants, from k_seg_const */
-  uint32_t* seg_off;               /* workspace copies, read by k_kept_scan / k_kept_move */
-  uint32_t* seg_kept;
-  uint32_t* kept_tmp;
-  /* sort only (large grouped calls): the block stops behind the sort, hands the elements over in
-   * the call's format -- fmt_dbits deadline bits, whatever the ctx's own span -- and publishes the
-   * ctx's deadline range; the kernels of the general path take it from there */
-  uint32_t sort_only, fmt_dbits;
-  unsigned long long* dst;
-  unsigned long long* ctx_dmin_inv;
-  unsigned long long* ctx_dmax;
-  PardTicket answer;               /* the call's only kernel, and its caller waits: the status goes out from here */
-};
-
-template <int THREADS>
-struct LocalSmem {
-  unsigned long long keys[kSortTile];
-  uint32_t slot[THREADS / 32][kBins];      /* counts, then next free slot per (warp, digit) */
-  uint32_t match[THREADS / 32][kBins];     /* lanes currently holding the digit */
-  uint32_t scan[THREADS / 32];
-  PardSegConst K[PARD_MAX_STAGES];
-  uint32_t stage_cnt[PARD_MAX_STAGES];
-  uint32_t stage_first[PARD_MAX_STAGES + 1];
-  uint32_t stage_kept[PARD_MAX_STAGES];
-  uint32_t kept_base[PARD_MAX_STAGES + 1];
-  uint32_t hb_kept[PARD_MAX_STAGES];       /* high budget first: length of the kept prefix */
-  unsigned long long red_min[THREADS / 32], red_max[THREADS / 32];
-  int32_t wm[THREADS / 32];
-  uint32_t wh[THREADS / 32];
-  uint32_t flag_foreign, flag_bad, flag_back;
-};
-
-/* decoded view of one sorted element inside a block of k_plan_local */
-struct LocalElem {
-  uint32_t stage, idx, r, u;
-  bool high_first;
-};
-
-template <class SMEM>
-__device__ __forceinline__ LocalElem local_decode(unsigned long long e, uint32_t pos, const SMEM& Sm,
-                                                  uint32_t ibits, uint32_t dbits, unsigned long long dmask,
-                                                  uint32_t imask) {
-  LocalElem x;
-  x.stage = (uint32_t)(e >> (ibits + dbits));
-  x.idx = (uint32_t)e & imask;
-  const PardSegConst& K = Sm.K[x.stage];
-  x.high_first = K.narrow & kSegHighFirst;
-  x.r = pos - Sm.stage_first[x.stage];
-  const unsigned long long off = (e >> ibits) & dmask;
-  if ((K.narrow & kSegNarrow) && dbits <= 29) {
-    const int32_t X = x.high_first ? (int32_t)K.A_rel - (int32_t)off : (int32_t)off - (int32_t)K.A_rel;
-    const unsigned long long uu = (unsigned long long)(div_magic32((uint32_t)X, K.d_magic) + 1u) * K.cap;
-    x.u = X < 0 ? 0u : (uu > kUClamp ? kUClamp : (uint32_t)uu);
-  } else {
-    x.u = (K.narrow & kSegNoStage) ? 0u : threshold_u(slack_of(off, K), K);
-  }
-  return x;
-}
-
-/* THREADS: 512, two blocks per multiprocessor.  (1,024 threads for a call that is this one block --
- * half as many ranking rounds per warp, twice the warps -- measured the same 28 us at 4,096
- * requests: the time is the chain of barriers and dependent shared-memory steps, not the warps.) */
-template <bool RAW, int THREADS>
-__device__ __forceinline__ void plan_local(PlanHeader* __restrict__ hdr, const LocalArgs& a) {
-  constexpr int WARPS = THREADS / 32;
-  constexpr int kItems = kSortTile / THREADS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  LocalSmem<THREADS>& Sm = *reinterpret_cast<LocalSmem<THREADS>*>(smem_raw);
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t lanebit = 1u << lane;
-  const uint32_t S = (uint32_t)a.st.stage_stride;
-  const uint32_t c = blockIdx.x;
-  const bool single = a.ctx_start == nullptr;
-  if (single) {                                          /* the only kernel of the call: the header starts here */
-    if (tid < sizeof(PlanHeader) / 4) reinterpret_cast<uint32_t*>(hdr)[tid] = 0;
-    __syncthreads();
-  } else if (hdr->unsorted || hdr->ctx_too_big) {      /* k_ctx_ranges found the promised grouping broken */
-    if (tid == 0 && c == 0) { set_status(hdr, PARD_EDATA); hdr->aborted = 1; }   /* nothing is sorted: later kernels return */
-    return;
-  }
-  const uint32_t first = single ? 0u : a.ctx_start[c];
-  const uint32_t cnt = single ? a.n : a.ctx_start[c + 1] - first;
-  /* every warp owns `items` rounds of 32 consecutive requests: as few as the ctx needs */
-  const int items = (int)((cnt + THREADS - 1) / THREADS);
-  const uint32_t wfirst = warp * (32 * (uint32_t)items);
-  uint16_t* stage16 = reinterpret_cast<uint16_t*>(&Sm.slot[0][0]);     /* 16 KB: the stages until the elements are built */
-
-  /* 1. the ctx's requests: deadlines into the tile buffer, stages beside them; deadline range,
-   * queue lengths, input checks */
-  for (uint32_t i = tid; i < S; i += THREADS) { Sm.stage_cnt[i] = 0; Sm.stage_kept[i] = 0; }
-  if (tid == 0) { Sm.flag_foreign = 0; Sm.flag_bad = 0; Sm.flag_back = a.st.d_priority ? 1u : 0u; }
-  __syncthreads();
-  unsigned long long lmin = ~0ull, lmax = 0;
-  bool foreign = false, bad = false;
-#pragma unroll 4
-  for (int i = 0; i < kItems; ++i) {
-    if (i >= items) break;
-    const uint32_t pos = wfirst + i * 32 + lane;
-    if (pos < cnt) {
-      const uint4 r = __ldg(&a.req[first + pos]);
-      const unsigned long long D = ((unsigned long long)r.y << 32) | r.x;
-      const uint32_t stage = r.w & 0xffffu;
-      foreign |= r.z != c;
-      const bool ok = r.z == c && stage < S && D < (unsigned long long)PARD_TIME_LIMIT_US;
-      bad |= !ok;
-      Sm.keys[pos] = D;
-      stage16[pos] = ok ? (uint16_t)stage : (uint16_t)0xffffu;
-      if (ok) {
-        lmin = D < lmin ? D : lmin;
-        lmax = D > lmax ? D : lmax;
-        atomicAdd(&Sm.stage_cnt[stage], 1u);
-      }
-    }
-  }
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long x = __shfl_xor_sync(0xffffffffu, lmin, o), y = __shfl_xor_sync(0xffffffffu, lmax, o);
-    lmin = x < lmin ? x : lmin;
-    lmax = y > lmax ? y : lmax;
-  }
-  if (lane == 0) { Sm.red_min[warp] = lmin; Sm.red_max[warp] = lmax; }
-  if (foreign) Sm.flag_foreign = 1;
-  if (bad) Sm.flag_bad = 1;
-  __syncthreads();
-  if (Sm.flag_foreign) {                                 /* not grouped by ctx after all (or, with one ctx, a request of another) */
-    if (tid == 0) { hdr->unsorted = 1; set_status(hdr, PARD_EDATA); hdr->aborted = 1; }
-    return;
-  }
-  unsigned long long dmin = ~0ull, dmax = 0;
-#pragma unroll
-  for (int w = 0; w < WARPS; ++w) {
-    dmin = Sm.red_min[w] < dmin ? Sm.red_min[w] : dmin;
-    dmax = Sm.red_max[w] > dmax ? Sm.red_max[w] : dmax;
-  }
-  const uint32_t dbits = dmin <= dmax ? bit_width64(dmax - dmin) : 0u;
-  /* stage field of the elements: requests that failed the checks carry the value S there, so
-   * that they sort behind the ctx's queues; they are reported, never decided */
-  const uint32_t sb = 32u - __clz(Sm.flag_bad ? S : S - 1);    /* bit width of the largest value; __clz(0) = 32 */
-  if (sb + dbits + a.ibits > 64) {                       /* the element does not fit 64 bits */
-    if (tid == 0) { hdr->wide = 1; set_status(hdr, PARD_ERANGE); }
-    return;
-  }
-  if (Sm.flag_bad && tid == 0) set_status(hdr, PARD_EDATA);
-
-  /* 2. constants of the ctx's queues: worked out here when the call is this
-   * one block; else taken from the table k_seg_const has filled for all queues at once (a chain
-   * of dependent loads that every block would otherwise wait for) and completed with what hangs
-   * on the ctx's deadline range */
-  if (a.sort_only) {
-    /* the constants come later, from k_seg_const, once every ctx's range is known */
-  } else if (single) {
-    if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, dmin, dmax, Sm.K, *reinterpret_cast<CtxScratch*>(&Sm.match[0][0])))
-      set_status(hdr, PARD_EDATA);
-  } else {
-    for (uint32_t k = tid; k < S; k += THREADS) {
-      PardSegConst K = a.ktab[(size_t)c * S + k];
-      const bool high_first = K.narrow & kSegHighFirst;
-      K.A_rel = high_first ? (int64_t)dmax - K.A : K.A - (int64_t)dmin;
-      const int64_t lim = (int64_t)1 << 29;
-      const bool fits32 = K.d_magic != 0 && K.d < ((int64_t)1 << 31) && K.A_rel > -lim && K.A_rel < lim;
-      K.narrow = (K.narrow & ~kSegNarrow) | (fits32 && !(K.narrow & kSegNoStage) ? kSegNarrow : 0u);
-      Sm.K[k] = K;
-    }
-  }
-  if (warp == 0) {                                       /* first position of every queue inside the ctx */
-    uint32_t run = 0;
-    for (uint32_t k0 = 0; k0 < S; k0 += 32) {
-      const uint32_t k = k0 + lane;
-      const uint32_t v = k < S ? Sm.stage_cnt[k] : 0u;
-      uint32_t x = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= (uint32_t)o) x += y;
-      }
-      if (k < S) Sm.stage_first[k] = run + x - v;
-      run += __shfl_sync(0xffffffffu, x, 31);
-    }
-    if (lane == 0) Sm.stage_first[S] = run;
-  }
-  __syncthreads();
-  const unsigned long long dmask = dbits >= 64 ? ~0ull : ((1ull << dbits) - 1);
-  const uint32_t imask = (1u << a.ibits) - 1;
-
-  /* 3. sort elements (stage | deadline offset | index), built from the tile buffer.  Deadlines that
-   * never step back along the ctx's requests (arrival order, one objective) are in order inside
-   * every queue as they come: only the stage is sorted then (4,096 contexts of 8,192 requests:
-   * one pass instead of three). */
-  unsigned long long key[kItems];
-  bool back = false;
-#pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    if (i >= items) break;
-    const uint32_t pos = wfirst + i * 32 + lane;
-    key[i] = ~0ull;                                      /* padding sorts last */
-    if (pos < cnt) {
-      const unsigned long long D = Sm.keys[pos];
-      back |= pos > 0 && D < Sm.keys[pos - 1];
-      const uint32_t stage = stage16[pos];
-      const uint32_t j = first + pos;
-      if (stage != 0xffffu) {
-        const bool high_first = a.st.d_priority && a.st.d_priority[(size_t)c * S + stage] != 0;
-        const unsigned long long off = (high_first ? dmax - D : D - dmin) & dmask;
-        key[i] = ((((unsigned long long)stage << dbits) | off) << a.ibits) | j;
-      } else {
-        key[i] = (((unsigned long long)S << dbits) << a.ibits) | j;
-      }
-    }
-  }
-  if (back) Sm.flag_back = 1;
-  __syncthreads();                                       /* the stages have been read: their room becomes the counters again */
-  const uint32_t pshift = Sm.flag_back ? 0u : dbits;
-  const uint32_t local_bits = dbits - pshift + sb;
-  const uint32_t passes = (local_bits + 7) / 8;
-  for (uint32_t i = tid; i < WARPS * kBins; i += THREADS) (&Sm.match[0][0])[i] = 0;
-  for (uint32_t p = 0; p < passes; ++p) {
-    const uint32_t shift = a.ibits + pshift + 8 * p;
-    for (uint32_t i = tid; i < WARPS * kBins; i += THREADS) (&Sm.slot[0][0])[i] = 0;
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kItems; ++i)
-      if (i < items) atomicAdd(&Sm.slot[warp][(uint32_t)(key[i] >> shift) & 255u], 1u);
-    __syncthreads();
-    uint32_t count = 0, x = 0;
-    if (tid < kBins) {
-#pragma unroll
-      for (int w = 0; w < WARPS; ++w) {
-        const uint32_t t = Sm.slot[w][tid];
-        Sm.slot[w][tid] = count;
-        count += t;
-      }
-      x = count;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= (uint32_t)o) x += y;
-      }
-      if (lane == 31) Sm.scan[warp] = x;
-    }
-    __syncthreads();
-    if (tid < kBins) {
-      uint32_t wx = 0;
-#pragma unroll
-      for (int w = 0; w < kBins / 32; ++w)
-        if (w < (int)warp) wx += Sm.scan[w];
-      const uint32_t dstart = wx + x - count;
-#pragma unroll
-      for (int w = 0; w < WARPS; ++w) Sm.slot[w][tid] += dstart;
-    }
-    __syncthreads();
-    sort_rank_drop<kItems, kItems>(key, shift, Sm.slot[warp], Sm.match[warp], Sm.keys, lanebit, items);
-    __syncthreads();
-    if (p + 1 < passes) {
-#pragma unroll
-      for (int i = 0; i < kItems; ++i)
-        if (i < items) key[i] = Sm.keys[wfirst + i * 32 + lane];
-      __syncthreads();
-    }
-  }
-  if (passes == 0) {
-#pragma unroll
-    for (int i = 0; i < kItems; ++i)
-      if (i < items) Sm.keys[wfirst + i * 32 + lane] = key[i];
-    __syncthreads();
-  }
-
-  if (a.sort_only) {
-    if (Sm.flag_bad) {                                   /* a flagged request has no place in the general path's order */
-      if (tid == 0) hdr->aborted = 1;
-      return;
-    }
-    if (dbits > a.fmt_dbits) {                           /* this ctx's span does not fit the call's element */
-      if (tid == 0) { hdr->wide = 1; set_status(hdr, PARD_ERANGE); }
-      return;
-    }
-    if (tid == 0 && dmin <= dmax) {
-      a.ctx_dmin_inv[c] = ~dmin;
-      a.ctx_dmax[c] = dmax;
-      atomicMax(&hdr->span_max, dmax - dmin);
-    }
-    const uint32_t kshift = a.ibits + dbits;
-    for (uint32_t pos = tid; pos < cnt; pos += THREADS) {
-      const unsigned long long e = Sm.keys[pos];
-      const unsigned long long seg = (unsigned long long)c * S + (uint32_t)(e >> kshift);
-      a.dst[first + pos] = ((seg << a.fmt_dbits | ((e >> a.ibits) & dmask)) << a.ibits) | (e & imask);
-    }
-    return;
-  }
-
-  /* 4. queue boundaries of the ctx */
-  const uint32_t n_good = Sm.stage_first[S];             /* requests that passed the checks; the others follow them */
-  for (uint32_t k = tid; k < S; k += THREADS) {
-    const uint32_t v = first + Sm.stage_first[k];
-    a.seg_off[(size_t)c * S + k] = v;
-    if (a.out_seg_off) a.out_seg_off[(size_t)c * S + k] = v;
-    Sm.hb_kept[k] = Sm.stage_cnt[k];
-  }
-  if (c + 1 == a.n_ctx && tid == 0) {
-    a.seg_off[(size_t)a.n_ctx * S] = a.n;
-    if (a.out_seg_off) a.out_seg_off[(size_t)a.n_ctx * S] = a.n;
-  }
-  __syncthreads();
-  /* a queue served high budget first keeps a prefix: its length is the first position r with r >= u_r */
-  if (a.st.d_priority) {
-#pragma unroll 1
-    for (int i = 0; i < kItems; ++i) {
-      if (i >= items) break;
-      const uint32_t pos = wfirst + i * 32 + lane;
-      if (pos < n_good) {
-        const LocalElem x = local_decode(Sm.keys[pos], pos, Sm, a.ibits, dbits, dmask, imask);
-        if (x.high_first && x.r >= x.u) atomicMin(&Sm.hb_kept[x.stage], x.r);
-      }
-    }
-    __syncthreads();
-  }
-
-  /* 5. segmented scan, first time: what every warp's elements add up to.  kGroup rounds are
-   * scanned side by side (their shuffles do not wait for each other), then chained. */
-  constexpr int kGroup = 4;
-  static_assert(kItems % kGroup == 0, "whole groups");
-  SegVal run = seg_identity<RAW>();
-#pragma unroll 1                                         /* (see 6.) */
-  for (int i0 = 0; i0 < kItems; i0 += kGroup) {
-    if (i0 >= items) break;
-    SegVal v[kGroup];
-#pragma unroll
-    for (int g = 0; g < kGroup; ++g) {
-      const uint32_t pos = wfirst + (i0 + g) * 32 + lane;
-      v[g] = seg_identity<RAW>();
-      if (i0 + g < items && pos < n_good) {
-        const LocalElem x = local_decode(Sm.keys[pos], pos, Sm, a.ibits, dbits, dmask, imask);
-        v[g].head = x.r == 0 ? 1u : 0u;
-        v[g].m = RAW ? (x.r < x.u ? 1 : 0) : (int32_t)x.u - (int32_t)x.r;
-      }
-    }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-      for (int g = 0; g < kGroup; ++g) {
-        SegVal l;
-        l.m = __shfl_up_sync(0xffffffffu, v[g].m, o);
-        l.head = __shfl_up_sync(0xffffffffu, v[g].head, o);
-        if (lane >= (uint32_t)o) v[g] = seg_combine<RAW>(l, v[g]);
-      }
-    }
-#pragma unroll
-    for (int g = 0; g < kGroup; ++g) {
-      SegVal all;
-      all.m = __shfl_sync(0xffffffffu, v[g].m, 31);
-      all.head = __shfl_sync(0xffffffffu, v[g].head, 31);
-      run = seg_combine<RAW>(run, all);
-    }
-  }
-  if (lane == 0) { Sm.wm[warp] = run.m; Sm.wh[warp] = run.head; }
-  __syncthreads();
-  SegVal carry = seg_identity<RAW>();
-#pragma unroll
-  for (int w = 0; w < WARPS; ++w) {
-    SegVal t; t.m = Sm.wm[w]; t.head = Sm.wh[w];
-    if (w < (int)warp) carry = seg_combine<RAW>(carry, t);
-  }
-
-  /* 6. second time: every request's position, estimate and decision; outputs.  The loop is kept a
-   * loop: a block that is alone on the device (one small ctx) waits for its instructions more than
-   * for anything else (ncu: "no instruction" is its first stall reason), so code that runs once
-   * per group is not unrolled over the groups. */
-#pragma unroll 1
-  for (int i0 = 0; i0 < kItems; i0 += kGroup) {
-    if (i0 >= items) break;
-    SegVal v[kGroup];
-    LocalElem x[kGroup];
-    unsigned long long e[kGroup];
-#pragma unroll
-    for (int g = 0; g < kGroup; ++g) {
-      const uint32_t pos = wfirst + (i0 + g) * 32 + lane;
-      v[g] = seg_identity<RAW>();
-      x[g].stage = 0; x[g].idx = 0; x[g].r = 0; x[g].u = 0; x[g].high_first = false;
-      e[g] = 0;
-      if (i0 + g < items && pos < cnt) e[g] = Sm.keys[pos];
-      if (i0 + g < items && pos < n_good) {
-        x[g] = local_decode(e[g], pos, Sm, a.ibits, dbits, dmask, imask);
-        v[g].head = x[g].r == 0 ? 1u : 0u;
-        v[g].m = RAW ? (x[g].r < x[g].u ? 1 : 0) : (int32_t)x[g].u - (int32_t)x[g].r;
-      }
-    }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-      for (int g = 0; g < kGroup; ++g) {
-        SegVal l;
-        l.m = __shfl_up_sync(0xffffffffu, v[g].m, o);
-        l.head = __shfl_up_sync(0xffffffffu, v[g].head, o);
-        if (lane >= (uint32_t)o) v[g] = seg_combine<RAW>(l, v[g]);
-      }
-    }
-#pragma unroll
-    for (int g = 0; g < kGroup; ++g) {
-      const uint32_t pos = wfirst + (i0 + g) * 32 + lane;
-      const bool valid = i0 + g < items && pos < n_good;
-      SegVal exc;
-      exc.m = __shfl_up_sync(0xffffffffu, v[g].m, 1);
-      exc.head = __shfl_up_sync(0xffffffffu, v[g].head, 1);
-      if (lane == 0) exc = seg_identity<RAW>();
-      const SegVal pre = seg_combine<RAW>(carry, exc);   /* over the earlier requests of the same queue */
-      SegVal all;
-      all.m = __shfl_sync(0xffffffffu, v[g].m, 31);
-      all.head = __shfl_sync(0xffffffffu, v[g].head, 31);
-      carry = seg_combine<RAW>(carry, all);
-      if (i0 + g < items && pos < cnt) {
-        const uint32_t gpos = first + pos;
-        uint32_t keep = 0;
-        long long est = 0;
-        if (valid) {
-          const PardSegConst& K = Sm.K[x[g].stage];
-          uint32_t cpos, ahead;                          /* batch-slot position; kept requests ahead in the queue */
-          if (RAW) {
-            cpos = x[g].r;
-            ahead = x[g].r == 0 ? 0u : (uint32_t)pre.m;
-          } else {
-            if (x[g].r == 0) cpos = 0;
-            else {
-              const long long cc = (long long)x[g].r - 1 + pre.m;
-              cpos = cc < (long long)x[g].r ? (uint32_t)cc : x[g].r;
-            }
-            if (x[g].high_first) cpos = min(x[g].r, Sm.hb_kept[x[g].stage]);
-            ahead = cpos;
-          }
-          const uint32_t round = K.cap_magic ? div_magic32(cpos, K.cap_magic) : cpos;
-          est = K.A + (long long)round * K.d;
-          keep = (cpos < x[g].u && !(K.narrow & kSegNoStage)) ? 1u : 0u;
-          if (K.narrow & kSegNoStage) set_status(hdr, PARD_EDATA);
-          if (keep && a.kept_tmp) a.kept_tmp[first + Sm.stage_first[x[g].stage] + ahead] = x[g].idx;
-          if (x[g].r + 1 == Sm.stage_cnt[x[g].stage]) Sm.stage_kept[x[g].stage] = ahead + keep;   /* the queue's last request */
-        }
-        if (a.out_keep) a.out_keep[gpos] = (uint8_t)keep;
-        if (a.out_est) a.out_est[gpos] = est;
-        if (a.out_perm) a.out_perm[gpos] = (uint32_t)e[g] & imask;
-      }
-    }
-  }
-  __syncthreads();
-  for (uint32_t k = tid; k < S; k += THREADS) {
-    a.seg_kept[(size_t)c * S + k] = Sm.stage_kept[k];
-    if (single && a.out_seg_kept) a.out_seg_kept[k] = Sm.stage_kept[k];
-  }
-  if (!single) return;
-
-  /* 7. one ctx: pack the survivors here (queue after queue) and finish the call */
-  if (warp == 0) {
-    uint32_t run_k = 0;
-    for (uint32_t k0 = 0; k0 < S; k0 += 32) {
-      const uint32_t k = k0 + lane;
-      const uint32_t v = k < S ? Sm.stage_kept[k] : 0u;
-      uint32_t y = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= (uint32_t)o) y += z;
-      }
-      if (k < S) Sm.kept_base[k] = run_k + y - v;
-      run_k += __shfl_sync(0xffffffffu, y, 31);
-    }
-    if (lane == 0) {
-      Sm.kept_base[S] = run_k;
-      if (a.out_n_kept) *a.out_n_kept = run_k;
-    }
-  }
-  __threadfence_block();
-  __syncthreads();
-  if (a.out_kept_idx && a.kept_tmp)
-    for (uint32_t k = 0; k < S; ++k) {
-      const uint32_t nk = Sm.stage_kept[k], from = Sm.stage_first[k], to = Sm.kept_base[k];
-      for (uint32_t i = tid; i < nk; i += THREADS) a.out_kept_idx[to + i] = a.kept_tmp[from + i];
-    }
-}
-
-template <bool RAW, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 512 ? 2 : 1)
-k_plan_local(PlanHeader* __restrict__ hdr, const __grid_constant__ LocalArgs a) {
-  pdl_wait();
-  plan_local<RAW, THREADS>(hdr, a);
-  if (a.answer.word) {
-    __syncthreads();
-    if (threadIdx.x == 0) pard_report(&hdr->status, a.answer.word, a.answer.ticket);
-  }
 }
 
 /* ------------------------------------------------------------------------ */
@@ -3052,10 +2451,8 @@ int allow_sort_smem(int dev) {
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(SortSmem)));
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<false, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(LocalSmem<512>)));
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sizeof(LocalSmem<512>)));
+    const int rc = allow_local_smem();
+    if (rc != PARD_OK) return rc;
     done[dev].store(true, std::memory_order_release);
   }
   return PARD_OK;
@@ -3282,95 +2679,32 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     return pard_plan_status(d_workspace, cuda_stream);
   };
 
-  /* ---- a block per ctx does everything (k_plan_local): a single ctx within one tile, or the
+  /* ---- a block per ctx does everything (pard_local.cu): a single ctx within one tile, or the
    * caller's word that the requests come grouped by ctx with no ctx beyond a tile ---- */
-  const bool fused_single = n_ctx == 1 && n > 0 && n <= (uint64_t)kSortTile && !rule_walk;
-  /* worth it while the blocks fit a few waves: beyond that the streaming decision kernel of the
-   * general path (which finds the grouping by itself) does the positions cheaper than the blocks' scans */
-  const bool fused_grouped = (mode & PARD_MODE_GROUPED) && n_ctx > 1 && n > 0 && !rule_walk && n_ctx <= 4u * (uint32_t)sms &&
-                             !L.ctx_passes;
-  if (fused_single || fused_grouped) {
+  const bool local_single = local_sure && !rule_walk;
+  if (local_single || ((mode & PARD_MODE_GROUPED) && n_ctx > 1 && n > 0 && !rule_walk && !L.ctx_passes)) {
     LocalArgs la = {};
-    la.req = req4; la.ctx_start = fused_single ? nullptr : ctx_start;
-    la.n = n32; la.n_ctx = n_ctx; la.ibits = ibits; la.raw = (mode & PARD_MODE_RAW) ? 1u : 0u;
+    la.req = req4; la.ctx_start = local_single ? nullptr : ctx_start;
+    la.n = n32; la.n_ctx = n_ctx; la.ibits = ibits; la.force_scan = (mode & PARD_MODE_SCAN) ? 1u : 0u;
     la.pipes = pipe_table; la.n_pipelines = n_pipelines; la.st = *state;
     la.out_keep = out->d_keep; la.out_est = (long long*)out->d_est_us; la.out_perm = out->d_perm;
     la.out_kept_idx = out->d_kept_idx; la.out_n_kept = (unsigned long long*)out->d_n_kept;
     la.out_seg_off = out->d_seg_offsets; la.out_seg_kept = out->d_seg_kept;
-    la.ktab = ktab; la.seg_off = seg_off; la.seg_kept = seg_kept; la.kept_tmp = out->d_kept_idx ? kept_tmp : nullptr;
-    if (fused_grouped) {
-      launch_pdl(k_clear, 4, 256, 0, stream, (uint4*)(ws + L.hdr), (unsigned long long)(L.hist / 16));
-      launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr, 0u, 0u);
-      /* the queues' constants; what depends on a ctx's deadline range is added by the ctx's block */
-      launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax,
-                 ktab, hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
-    }
-    const bool answered = fused_single && !(mode & PARD_MODE_NOWAIT);
+    la.ktab = ktab; la.kept_words = (uint32_t*)ctx_dmin; la.kept_tmp = out->d_kept_idx ? kept_tmp : nullptr;
+    const bool answered = local_single && !(mode & PARD_MODE_NOWAIT);
     if (answered) la.answer = pard_report_ticket();
-    launch_pdl((mode & PARD_MODE_RAW) ? k_plan_local<true, 512> : k_plan_local<false, 512>, n_ctx, 512,
-               sizeof(LocalSmem<512>), stream, hdr, la);
-    if (fused_grouped) {
-      launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
-                 (unsigned long long*)out->d_n_kept);
-      if (out->d_kept_idx)
-        launch_pdl(k_kept_move, std::min<uint32_t>(((uint32_t)((n + kCompactChunk - 1) / kCompactChunk) + L.n_seg + 7) / 8,
-                                                   (uint32_t)sms * 8), 256, 0, stream,
-                   kept_tmp, seg_off, seg_kept, kept_base, chunk_base, L.n_seg, out->d_kept_idx);
+    if (!local_single) {
+      launch_pdl(k_clear, std::min<uint32_t>((n_ctx + 1023) / 1024 + 1, (uint32_t)sms), 256, 0, stream, (uint4*)(ws + L.hdr),
+                 (unsigned long long)((L.ctx_dmin + 4ull * n_ctx + 15) / 16));
+      rc = launch_ctx_prep(la, ktab, ctx_start, hdr, stream);
+      if (rc != PARD_OK) return rc;
     }
+    rc = launch_plan_local(la, hdr, (mode & PARD_MODE_RAW) != 0, stream);
+    if (rc != PARD_OK) return rc;
     while (phase <= PARD_N_PHASES) mark();             /* the phases are those of the other path: all of this counts as the first */
     PARD_CUDA_OK(cudaGetLastError());
     if (mode & PARD_MODE_NOWAIT) return PARD_OK;
     rc = answered ? pard_report_wait(la.answer, &hdr->status, stream) : pard_plan_status(d_workspace, cuda_stream);
-    return rc == PARD_ERANGE ? plan_wide() : rc;
-  }
-
-  /* ---- the same promise for more contexts than that: a block per ctx still reads, checks and
-   * sorts its ctx (k_plan_local, stopping behind the sort) and publishes the ctx's deadline range,
-   * so that neither the prepass over all requests nor the packing and radix kernels (launched
-   * otherwise in case the device finds the requests not grouped) are needed; the element format
-   * is fixed here (all bits the queue id and the index leave), tables and decision as in the
-   * general path ---- */
-  if ((mode & PARD_MODE_GROUPED) && n_ctx > 1 && n > 0 && !rule_walk && !L.ctx_passes) {
-    const uint32_t fmt_dbits = std::min(60u, 64u - ibits - sbits);
-    LocalArgs la = {};
-    la.req = req4; la.ctx_start = ctx_start;
-    la.n = n32; la.n_ctx = n_ctx; la.ibits = ibits;
-    la.pipes = pipe_table; la.n_pipelines = n_pipelines; la.st = *state;
-    la.sort_only = 1; la.fmt_dbits = fmt_dbits; la.dst = buf_a; la.ctx_dmin_inv = ctx_dmin; la.ctx_dmax = ctx_dmax;
-    launch_pdl(k_clear, 8, 256, 0, stream, (uint4*)(ws + L.hdr), (unsigned long long)(L.hist / 16));
-    launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr, fmt_dbits, sbits);
-    launch_pdl(k_plan_local<false, 512>, n_ctx, 512, sizeof(LocalSmem<512>), stream, hdr, la);
-    launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
-               hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
-    if (L.n_seg >= kManyQueues)
-      launch_pdl(k_seg_win_many, ((L.n_seg + 31) / 31 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab,
-                 seg_off, out->d_seg_offsets, win_off, win_cnt, win_own, win_big, L.win_capacity,
-                 (mode & PARD_MODE_SCAN) ? 1u : 0u, 1u, seg_kept);
-    else
-      launch_pdl(k_seg_win, (L.n_seg + 1 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab, seg_off,
-                 out->d_seg_offsets, win_off, win_cnt, win_own, win_big, L.win_capacity,
-                 (mode & PARD_MODE_SCAN) ? 1u : 0u, (const uint32_t*)hist, sbits, 1u, 1u, seg_kept);
-    uint32_t* tmp = out->d_kept_idx ? kept_tmp : nullptr;
-    long long* est = (long long*)out->d_est_us;
-    const bool raw = mode & PARD_MODE_RAW;
-    launch_pdl(k_win_bounds, std::min<uint32_t>((L.win_capacity + 7) / 8, (uint32_t)sms * 8), 256, 0, stream,
-        hdr, buf_a, buf_b, ibits, L.n_seg, ktab, seg_off, win_off, win_cnt, win_own, win_big, win_done, wtab, raw ? 1u : 0u, seg_kept);
-    launch_pdl(k_win_prefix, (L.n_seg + 7) / 8, 256, 0, stream, hdr, L.n_seg, ktab, seg_off, win_off, win_cnt, wtab, raw ? 1u : 0u, seg_kept);
-    launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
-               (unsigned long long*)out->d_n_kept);
-    auto decide_win = raw ? (state->d_priority ? k_decide_win<true, true> : k_decide_win<true, false>)
-                          : (state->d_priority ? k_decide_win<false, true> : k_decide_win<false, false>);
-    launch_pdl(decide_win, (uint32_t)((n + (uint64_t)kDecTile - 1) / kDecTile), kDecThreads, 0, stream, hdr, buf_a, buf_b, n32,
-               ibits, ktab, seg_off, win_off, win_cnt, wtab, out->d_keep, est, out->d_perm, out->d_kept_idx,
-               (const uint32_t*)kept_base, (uint32_t*)nullptr);
-    launch_pdl(raw ? k_scan_path<true> : k_scan_path<false>, std::min<uint32_t>(L.dec_tiles, (uint32_t)sms * 2), kDecThreads, 0,
-               stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab, seg_off, win_off, tile_agg, tile_carry, out->d_keep, est,
-               out->d_perm, tmp, seg_kept, kept_base, chunk_base, out->d_seg_kept, (unsigned long long*)out->d_n_kept,
-               out->d_kept_idx, 0u);
-    while (phase <= PARD_N_PHASES) mark();
-    PARD_CUDA_OK(cudaGetLastError());
-    if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-    rc = pard_plan_status(d_workspace, cuda_stream);
     return rc == PARD_ERANGE ? plan_wide() : rc;
   }
 
@@ -3404,7 +2738,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
              hdr, sbits, ibits, fold_width ? 1u : 0u, arrival_order ? 1u : 0u, win_hist ? 1u : 0u,
              (mode & PARD_MODE_SCAN) ? 1u : 0u, win_off, win_cnt, key_sbits);
   if ((local_cand && !local_sure) || ctx_sort)
-    launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr, 0u, 0u);
+    launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr);
   if (ctx_sort) launch_pdl(k_tile_table, 1, 1024, 0, stream, (const uint32_t*)ctx_start, n_ctx, (uint32_t*)(ws + L.tile_first));
   mark();
   if (local_cand)                                /* every ctx inside one tile: sorted block by block, straight from the requests */

@@ -232,6 +232,115 @@ __device__ __forceinline__ void store4(void* p, unsigned long long a, unsigned l
 }
 
 
+/* loads and stores of look-back words: relaxed, device scope (other blocks write them) */
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
+}
+
+struct SegVal {            /* value of a segmented running reduction */
+  int32_t m;               /* admitted mode: minimum of u_t - t; raw mode: number of kept requests;
+                              over the elements since the last queue head (or since the span's start) */
+  uint32_t head;           /* a queue head lies inside the span */
+};
+
+template <bool RAW>
+__device__ __forceinline__ SegVal seg_identity() {
+  SegVal a;
+  a.m = RAW ? 0 : 0x7fffffff;
+  a.head = 0;
+  return a;
+}
+
+template <bool RAW>
+__device__ __forceinline__ SegVal seg_combine(SegVal left, SegVal right) {
+  SegVal r;
+  r.m = right.head ? right.m : (RAW ? left.m + right.m : min(left.m, right.m));
+  r.head = left.head | right.head;
+  return r;
+}
+
+/* Inclusive segmented warp scan of the threads' values (in lane order). */
+template <bool RAW>
+__device__ __forceinline__ SegVal warp_scan(SegVal v, uint32_t lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    SegVal l;
+    l.m = __shfl_up_sync(0xffffffffu, v.m, o);
+    l.head = __shfl_up_sync(0xffffffffu, v.head, o);
+    if (lane >= (uint32_t)o) v = seg_combine<RAW>(l, v);
+  }
+  return v;
+}
+
+constexpr int32_t kWinInf = 0x7fffffff;
+
+/* u of window b (the saturation of threshold_u) */
+__device__ __forceinline__ uint32_t win_u(uint32_t b, uint32_t cap) {
+  const unsigned long long u = (unsigned long long)(b + 1) * cap;
+  return u > kUClamp ? kUClamp : (uint32_t)u;
+}
+
+/* The first request whose ctx is >= c, by one warp's 32-ary search, into ctx_start[c].  That the
+ * boundaries never step back and the ranges cover all requests is checked here; the planner's
+ * blocks check that their ranges hold requests of their ctx only: both together prove the grouping. */
+__device__ __forceinline__ void ctx_range_search(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t c,
+                                                 uint32_t* __restrict__ ctx_start, PlanHeader* hdr, uint32_t limit) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t lo[2] = {0, 0}, hi[2] = {n, n};       /* first request whose ctx is >= c, >= c + 1 */
+  while (lo[0] < hi[0] || lo[1] < hi[1]) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      if (lo[q] < hi[q]) {                       /* uniform across the warp */
+        const uint32_t span = hi[q] - lo[q];
+        const uint32_t p = lo[q] + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* lo <= p < hi */
+        const bool less = __ldg(&req[p]).z < c + q;
+        const uint32_t k = __popc(__ballot_sync(0xffffffffu, less));
+        const uint32_t p_below = __shfl_sync(0xffffffffu, p, k > 0 ? k - 1 : 0);
+        const uint32_t p_at = __shfl_sync(0xffffffffu, p, k < 32 ? k : 31);
+        if (k > 0) lo[q] = p_below + 1;
+        if (k < 32) hi[q] = p_at;
+      }
+    }
+  }
+  if (lane != 0) return;
+  ctx_start[c] = lo[0];
+  if (c == n_ctx && lo[0] != n) hdr->unsorted = 1;      /* requests past the last ctx's range (ctx out of range) */
+  if (c < n_ctx) {
+    if (lo[1] < lo[0]) hdr->unsorted = 1;
+    else if (lo[1] - lo[0] > limit) hdr->ctx_too_big = 1;
+  }
+}
+
+/* ---- one block plans one ctx (pard_local.cu) ---- */
+constexpr uint32_t kLocalTile = 8192;             /* requests of one ctx a block can take */
+struct LocalArgs {
+  const uint4* req;
+  const uint32_t* ctx_start;       /* NULL: the call has one ctx */
+  uint32_t n, n_ctx, ibits, force_scan;
+  PipeTable pipes;
+  uint32_t n_pipelines;
+  pard_queue_state_t st;
+  uint8_t* out_keep;
+  long long* out_est;
+  uint32_t* out_perm;
+  uint32_t* out_kept_idx;
+  unsigned long long* out_n_kept;
+  uint32_t* out_seg_off;
+  uint32_t* out_seg_kept;
+  const PardSegConst* ktab;        /* several ctx: the queues' constants, from k_ctx_prep */
+  uint32_t* kept_words;            /* several ctx: look-back words over the ctxs' kept counts, zero at the start */
+  uint32_t* kept_tmp;
+  PardTicket answer;               /* the call's only kernel, and its caller waits: the status goes out from here */
+};
+int allow_local_smem();            /* once per device, by the planner's set-up */
+int launch_ctx_prep(const LocalArgs& a, PardSegConst* ktab, uint32_t* ctx_start, PlanHeader* hdr, cudaStream_t stream);
+int launch_plan_local(const LocalArgs& a, PlanHeader* hdr, bool raw, cudaStream_t stream);
+
 /* Decision by a sequential walk of every queue (requests whose downstream path is known, arrival
  * order, the Nexus and Clipper++ rules): defined in pard_policy.cu, enqueued by pard_plan after
  * the sort and the queue boundaries.  The sorted elements are in buf_b when hdr->npass is odd,
