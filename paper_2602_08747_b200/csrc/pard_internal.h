@@ -89,6 +89,12 @@ PardTicket pard_report_ticket();
 cudaError_t pard_clear_status(void* hdr, cudaStream_t stream);
 /* waits for the answer to `t` (given by the work already enqueued on `stream`); the call's status */
 int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream);
+/* enqueues the answer to `t`, and *d_count (may be NULL) beside it in t.word[1] */
+int pard_report_enqueue(const PardTicket& t, const uint32_t* d_status, const unsigned long long* d_count, cudaStream_t stream);
+/* kStagingBytes of pinned memory of the calling thread's own, or NULL; free again when the call that
+ * uses it has waited for its copies */
+constexpr size_t kStagingBytes = 64 * 1024;
+char* pard_staging();
 /* the same behind everything enqueued so far: answers `t` with a kernel of its own */
 int pard_wait_status(const uint32_t* d_status, cudaStream_t stream);
 

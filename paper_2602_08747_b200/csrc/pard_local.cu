@@ -7,8 +7,8 @@
  *      deadlines ever step back;
  *   2. gets the constants of the ctx's queues (Eq. 3);
  *   3. sorts (stage | deadline offset | index) in shared memory -- by the stage alone when the
- *      deadlines are in order already (arrival order, one objective), by up to 16 stages with
- *      ballots and without counters in shared memory;
+ *      deadlines are in order already (arrival order, one objective), for up to 16 stages a
+ *      counting sort in registers;
  *   4. finds the batch-window tables (see pard_plan.cu) in the sorted elements: an element whose
  *      window differs from its neighbour's knows the P of the windows between them;
  *   5. the tables give every queue's kept count, a look-back over the ctxs before gives the place of
@@ -17,7 +17,11 @@
  * 16 bytes are read and 13 + 4f written per request and nothing else touches global memory.
  * Queues with more windows than the block's tables hold are decided by the segmented prefix-min
  * scan over the elements instead.
- * Bound by shared-memory work and barriers, not by memory.  @@NUM@@ */
+ * Bound by the chain of steps between barriers, two blocks per multiprocessor covering for each other:
+ * of 400 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the copy bandwidth) 120 go to the
+ * requests, 75 to the counting sort, 50 to the tables and 110 to the outputs.  The form before,
+ * two segmented scans instead of tables, took 762 us there, three radix passes without a look at the
+ * order 865. */
 #include <cstddef>
 
 #include "pard_plan_internal.cuh"
@@ -49,6 +53,7 @@ struct Split {
   uint32_t P[kTabEntries];
   int32_t EK[kTabEntries];                               /* E, or Kp for raw positions */
   uint32_t U[kTabEntries];                               /* u of the window */
+  uint16_t kept[kLocalTile];                             /* survivors, queue after queue */
 };
 
 /* Requests that come in order, on their way into the Split form: beside its off and idx. */
@@ -81,7 +86,7 @@ struct LocalSmem {
   unsigned long long red_min[kLocWarps], red_max[kLocWarps];
   int32_t wm[kLocWarps];
   uint32_t wh[kLocWarps];
-  uint32_t ctx, first, cnt, flags, use_scan, base, abort;
+  uint32_t ctx, first, cnt, flags, use_scan, kept, base, abort;
 };
 
 static_assert(sizeof(Ordered) <= offsetof(LocalSmem, K) && sizeof(Split) <= offsetof(LocalSmem, K), "inside keys and counters");
@@ -295,16 +300,42 @@ __device__ uint32_t table_prefix(Tables& t, uint32_t off, uint32_t cnt, uint32_t
   return n_q == 0 ? 0u : (RAW ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1)));
 }
 
+/* Places of the survivors of the ctx's queues inside the ctx, the queues' kept counts to the caller, the
+ * ctx's count to the blocks behind.  One warp. */
+__device__ __forceinline__ void publish_kept(const LocalArgs& a, LocalSmem& Sm, uint32_t c, uint32_t lane) {
+  const uint32_t S = (uint32_t)a.st.stage_stride;
+  uint32_t run = 0;
+  for (uint32_t k0 = 0; k0 < S; k0 += 32) {
+    const uint32_t k = k0 + lane;
+    const uint32_t v = k < S ? Sm.stage_kept[k] : 0u;
+    uint32_t y = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= (uint32_t)o) y += z;
+    }
+    if (k < S) {
+      Sm.kept_base[k] = run + y - v;
+      if (a.out_seg_kept) a.out_seg_kept[(size_t)c * S + k] = v;
+    }
+    run += __shfl_sync(0xffffffffu, y, 31);
+  }
+  if (lane == 0) {
+    Sm.kept = run;
+    if (a.ctx_start) st_relaxed(a.kept_words + c, run | (c == 0 ? kLbIncl : kLbAgg));
+  }
+}
+
 /* Kept requests of all ctxs before this one: ctxs are taken in ticket order, so a block only waits
- * for blocks that run already; 32 ctxs per round trip, bounded.  One warp. */
-__device__ bool look_back(PlanHeader* hdr, uint32_t* words, uint32_t c, uint32_t mine, uint32_t lane, uint32_t* before) {
-  if (lane == 0) st_relaxed(words + c, mine | (c == 0 ? kLbIncl : kLbAgg));
+ * for blocks that run already; 32 ctxs per round trip, bounded.  Called as late as possible: the
+ * blocks in flight are mostly at the same point, and a block that asks right after publishing its own
+ * count waits for the slowest of those before it (92 us of 468 at 4,096 ctxs). */
+__device__ __forceinline__ bool look_back(PlanHeader* hdr, uint32_t* words, uint32_t c, uint32_t mine, uint32_t lane, uint32_t* before) {
   uint32_t sum = 0, spins = 0;
   int64_t t = (int64_t)c - 1;
   while (t >= 0) {
     const uint32_t v = t - (int64_t)lane >= 0 ? ld_relaxed(words + (t - lane)) : (uint32_t)kLbIncl;
     const uint32_t unset = __ballot_sync(0xffffffffu, (v >> 30) == 0), incl = __ballot_sync(0xffffffffu, (v & kLbIncl) != 0);
-    const uint32_t stop = incl ? (uint32_t)__ffs(incl) : 32u;      /* lanes 0 .. stop-1 count */
+    const uint32_t stop = incl ? (uint32_t)__ffs(incl) : 32u;        /* lanes 0 .. stop-1 count */
     const uint32_t ready = unset ? (uint32_t)__ffs(unset) - 1 : 32u;
     const uint32_t use = min(stop, ready);
     sum += __reduce_add_sync(0xffffffffu, lane < use ? v & kLbMask : 0u);
@@ -320,31 +351,16 @@ __device__ bool look_back(PlanHeader* hdr, uint32_t* words, uint32_t c, uint32_t
   return true;
 }
 
-/* Where the survivors of the ctx's queues go: behind those of the ctxs before (one warp; the others
- * wait).  False: a wait ran out, here or in another block. */
+/* The ctx's place in the list of survivors (one warp; the others wait).  False: a wait ran out, here or
+ * in another block. */
 __device__ __forceinline__ bool place_survivors(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, uint32_t c) {
-  const uint32_t tid = threadIdx.x, lane = tid & 31, S = (uint32_t)a.st.stage_stride;
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
   if (tid < 32) {
-    uint32_t run = 0;
-    for (uint32_t k0 = 0; k0 < S; k0 += 32) {
-      const uint32_t k = k0 + lane;
-      const uint32_t v = k < S ? Sm.stage_kept[k] : 0u;
-      uint32_t y = v;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= (uint32_t)o) y += z;
-      }
-      if (k < S) {
-        Sm.kept_base[k] = run + y - v;
-        if (a.out_seg_kept) a.out_seg_kept[(size_t)c * S + k] = v;
-      }
-      run += __shfl_sync(0xffffffffu, y, 31);
-    }
     uint32_t before = 0;
-    if (a.ctx_start && !look_back(hdr, a.kept_words, c, run, lane, &before) && lane == 0) Sm.abort = 1;
+    if (a.ctx_start && !look_back(hdr, a.kept_words, c, Sm.kept, lane, &before) && lane == 0) Sm.abort = 1;
     if (lane == 0) {
       Sm.base = before;
-      if (c + 1 == a.n_ctx && a.out_n_kept) *a.out_n_kept = before + run;
+      if (c + 1 == a.n_ctx && a.out_n_kept) *a.out_n_kept = before + Sm.kept;
     }
   }
   __syncthreads();
@@ -484,8 +500,8 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
   }
   if (tid == 0 && c + 1 == a.n_ctx && a.out_seg_off) a.out_seg_off[(size_t)a.n_ctx * S] = a.n;
   __syncthreads();
-  if (!place_survivors(hdr, a, Sm, c)) return true;
-  const uint32_t base = Sm.base;
+  if (warp == 0) publish_kept(a, Sm, c, lane);
+  __syncthreads();
   for (uint32_t row = row0; row < row1;) {
     const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, my_row_first <= row));
     const uint32_t lo = Sm.stage_first[k], n = Sm.stage_first[k + 1] - lo, rf = Sm.row_first[k];
@@ -494,7 +510,7 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
     const long long A = K.A;
     const unsigned long long cap_magic = K.cap_magic;
     const uint32_t d = (uint32_t)K.d, woff = Sm.win_off[k];          /* d fits 32 bits: it has a magic number */
-    uint32_t* kept_out = a.out_kept_idx ? a.out_kept_idx + base + Sm.kept_base[k] : nullptr;
+    uint16_t* kept_out = T.kept + Sm.kept_base[k];
     uint32_t r = (row - rf) * 32 + lane;
     const size_t g0 = (size_t)first + lo + r;
     uint8_t* keep_p = a.out_keep + g0;
@@ -503,7 +519,7 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
 #pragma unroll 2
     for (; row < rows; ++row, r += 32, keep_p += 32, est_p += 32, perm_p += 32) {
       if (r >= n) continue;
-      const uint32_t b = T.win[lo + r], idx = first + T.idx[lo + r];
+      const uint32_t b = T.win[lo + r], local = T.idx[lo + r];
       uint32_t cpos = RAW ? r : 0u, ahead = 0, u = 0;    /* batch-slot position; kept requests ahead in the queue */
       if (b != kNoWindow) {
         const uint32_t P = T.P[woff + b];
@@ -519,12 +535,15 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
       }
       const bool keep = cpos < u;
       const uint32_t round = cap_magic ? div_magic32(cpos, cap_magic) : cpos;
-      if (keep && kept_out) kept_out[ahead] = idx;
+      if (keep) kept_out[ahead] = (uint16_t)local;
       if (a.out_keep) *keep_p = keep ? 1 : 0;
       if (a.out_est) *est_p = A + (long long)((unsigned long long)round * d);
-      if (a.out_perm) *perm_p = idx;
+      if (a.out_perm) *perm_p = first + local;
     }
   }
+  if (!place_survivors(hdr, a, Sm, c)) return true;      /* (its barrier also completes the list) */
+  if (a.out_kept_idx)
+    for (uint32_t i = tid; i < Sm.kept; i += kLocThreads) a.out_kept_idx[Sm.base + i] = first + T.kept[i];
   return true;
 }
 
@@ -616,6 +635,7 @@ __device__ __noinline__ void finish_ctx(PlanHeader* __restrict__ hdr, const Loca
   }
 
   if (tables) {
+    if (warp == 0) publish_kept(a, Sm, c, lane);
     if (!place_survivors(hdr, a, Sm, c)) return;
     const uint32_t base = Sm.base;
     /* 6. every request on its own */
@@ -728,6 +748,7 @@ __device__ __noinline__ void finish_ctx(PlanHeader* __restrict__ hdr, const Loca
   }
   __threadfence_block();
   __syncthreads();
+  if (warp == 0) publish_kept(a, Sm, c, lane);
   if (!place_survivors(hdr, a, Sm, c)) return;
   if (a.out_kept_idx && a.kept_tmp)
     for (uint32_t k = 0; k < S; ++k) {

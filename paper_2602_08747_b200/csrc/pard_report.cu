@@ -18,10 +18,13 @@ namespace {
 constexpr int kSlots = 64;
 struct alignas(64) Slot {
   unsigned long long word;                       /* ticket << 32 | status */
-  unsigned long long pad[7];
+  unsigned long long count;                      /* a number that goes with it */
+  unsigned long long pad[6];
 };
 std::mutex g_mu;
 std::atomic<Slot*> g_page{nullptr};
+std::atomic<char*> g_staging{nullptr};           /* kStagingBytes for each of the first kStagingSlots slots */
+constexpr int kStagingSlots = 8;
 std::atomic<uint64_t> g_taken{0};
 uint32_t g_ticket[kSlots];                       /* of the slot's owner */
 
@@ -43,8 +46,9 @@ int own_slot() {
   return -1;
 }
 
-__global__ void k_report(const uint32_t* status, unsigned long long* word, uint32_t ticket) {
+__global__ void k_report(const uint32_t* status, unsigned long long* word, uint32_t ticket, const unsigned long long* count) {
   pdl_wait();
+  if (count) word[1] = __ldcg(count);
   pard_report(status, word, ticket);
 }
 
@@ -69,6 +73,11 @@ void pard_report_init() {
     return;
   }
   for (int i = 0; i < kSlots; ++i) ((Slot*)p)[i].word = 0;
+  void* s = nullptr;
+  if (cudaHostAlloc(&s, (size_t)kStagingSlots * kStagingBytes, cudaHostAllocPortable) == cudaSuccess)
+    g_staging.store((char*)s, std::memory_order_release);
+  else
+    cudaGetLastError();
   g_page.store((Slot*)p, std::memory_order_release);
 }
 
@@ -103,8 +112,19 @@ int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t
   return h_status ? -(int)h_status : PARD_OK;
 }
 
+int pard_report_enqueue(const PardTicket& t, const uint32_t* d_status, const unsigned long long* d_count, cudaStream_t stream) {
+  if (t.word) PARD_CUDA_OK(launch_pdl(k_report, 1, 1, 0, stream, d_status, t.word, t.ticket, d_count));
+  return PARD_OK;
+}
+
 int pard_wait_status(const uint32_t* d_status, cudaStream_t stream) {
   const PardTicket t = pard_report_ticket();
-  if (t.word) PARD_CUDA_OK(launch_pdl(k_report, 1, 1, 0, stream, d_status, t.word, t.ticket));
-  return pard_report_wait(t, d_status, stream);
+  const int rc = pard_report_enqueue(t, d_status, nullptr, stream);
+  return rc != PARD_OK ? rc : pard_report_wait(t, d_status, stream);
+}
+
+char* pard_staging() {
+  const int k = own_slot();
+  char* s = g_staging.load(std::memory_order_acquire);
+  return k >= 0 && k < kStagingSlots && s ? s + (size_t)k * kStagingBytes : nullptr;
 }
