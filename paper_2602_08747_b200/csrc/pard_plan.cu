@@ -25,8 +25,8 @@ namespace {
 struct Layout {
   /* [hdr, zero_end) must be zero when the first kernel starts: cleared by k_clear (of the two
    * look-back arrays only the first: every sort pass clears the array of the pass after it) */
-  uint64_t hdr, ctx_dmin, ctx_dmax, seg_off, seg_kept, win_done, hist, whist, hist_ctx, lookback, zero_end, tile_first,
-      ctx_start, pipes, ktab, kept_base, chunk_base, tile_agg, tile_carry, win_off, win_cnt, win_own, win_big, wtab, kept_tmp,
+  uint64_t hdr, ctx_dmin, ctx_dmax, seg_off, seg_kept, hist, whist, hist_ctx, lookback, zero_end, tile_first,
+      ctx_start, pipes, ktab, kept_base, chunk_base, tile_agg, tile_carry, win_off, win_cnt, wtab, kept_tmp,
       buf_a, buf_b, total;
   uint32_t n_seg, sort_tiles, dec_tiles, max_passes, win_capacity;
   uint32_t lb_tiles;          /* tiles the look-back arrays are sized for */
@@ -60,7 +60,6 @@ Layout make_layout(uint64_t n, uint32_t n_ctx, int32_t stage_stride) {
   L.ctx_dmax = o;  o = al(o + 8ull * n_ctx);
   L.seg_off = o;   o = al(o + 4ull * (L.n_seg + 1));
   L.seg_kept = o;  o = al(o + 4ull * L.n_seg);
-  L.win_done = o;  o = al(o + 4ull * L.n_seg);
   L.hist = o;      o = al(o + 4ull * kMaxPasses * kBins);
   L.whist = o;     o = al(o + (L.n_seg <= kHistSegs ? 4ull * kHistCap : 0ull));   /* window counts of calls with few queues */
   /* passes kept inside the contexts' ranges cut the tiles at ctx boundaries: at most one more
@@ -82,8 +81,6 @@ Layout make_layout(uint64_t n, uint32_t n_ctx, int32_t stage_stride) {
   if (L.n_seg <= kHistSegs) L.win_capacity = std::max(L.win_capacity, kHistCap);   /* counted tables: see k_seg_const */
   L.win_off = o;   o = al(o + 4ull * (L.n_seg + 1));
   L.win_cnt = o;   o = al(o + 4ull * (L.n_seg + 1));
-  L.win_own = o;   o = al(o + 4ull * L.win_capacity);
-  L.win_big = o;   o = al(o + 4ull * L.win_capacity);
   L.wtab = o;      o = al(o + 16ull * L.win_capacity);
   L.kept_tmp = o;  o = al(o + 4ull * n);
   L.buf_a = o;     o = al(o + 8ull * n);
@@ -475,7 +472,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     my_copy = (threadIdx.x & (copies - 1)) * win_total;
     if (win_shared) for (uint32_t i = threadIdx.x; i < win_total * copies; i += blockDim.x) s_win[i] = 0;
     /* When the queue id lies inside the last pass's digit the queues' lengths can be read off that
-     * pass's digit counts (see k_seg_win), and entry 0 of a queue -- its requests with deadline < A,
+     * pass's digit counts (see k_windows), and entry 0 of a queue -- its requests with deadline < A,
      * often most of an overloaded queue -- is its length minus its other entries: such requests
      * are then not counted here at all. */
     win_derive = npass > 0 && hdr->keybits - (dbits - pshift) <= hdr->keybits - 8 * (npass - 1);
@@ -1681,221 +1678,16 @@ struct __align__(16) WinEntry {
   uint32_t pad;
 };
 constexpr uint32_t kWinMaxPerSeg = 4096;
-constexpr uint32_t kManyQueues = 8192;     /* from this many queues on a lane, not a warp, handles a queue in k_seg_win_many */
-constexpr uint32_t kWinLongQueue = 8192;   /* above this a window boundary is searched by a whole warp, else by one lane */
-
-
 /* window of a non-negative X = D - A */
 __device__ __forceinline__ unsigned long long win_of(unsigned long long X, const PardSegConst& K) {
   if ((X >> 32) == 0 && K.d_magic) return div_magic32((uint32_t)X, K.d_magic);
   return X / (unsigned long long)K.d;
 }
 
-/* One warp per queue: its first and last sorted position (a 32-ary search for
- * the segment id in the elements' upper bits), the number of its batch windows
- * (from its latest deadline), and a range of table entries for them, taken
- * from a shared counter; every entry is labelled with its queue.  If the
- * table cannot hold the windows the call falls back to the scan kernels. */
-__global__ void __launch_bounds__(256)
-k_seg_win(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
-          const unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t ibits, uint32_t n_seg,
-          const PardSegConst* __restrict__ ktab, uint32_t* __restrict__ seg_off,
-          uint32_t* __restrict__ out_seg_off, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
-          uint32_t* __restrict__ win_own, uint32_t* __restrict__ win_big, uint32_t capacity,
-          uint32_t force_scan, const uint32_t* __restrict__ hist, uint32_t sbits, uint32_t local_candidate,
-          uint32_t tables, uint32_t* __restrict__ seg_kept) {
-  pdl_wait();
-  const uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t lane = threadIdx.x & 31;
-  if (s > n_seg) return;                         /* whole warps leave together */
-  if (s == 0 && lane == 0 && force_scan) hdr->use_scan = 1;
-  uint32_t lo[2] = {0, 0};
-  const bool wide = hdr->wide != 0 || hdr->aborted != 0;   /* nothing usable was sorted */
-  const unsigned long long* src = (hdr->npass & 1) ? buf_b : buf_a;
-  const uint32_t dbits = hdr->dbits;
-  const uint32_t npass = hdr->npass;
-  const uint32_t top_bits = npass ? hdr->keybits - 8 * (npass - 1) : 0;   /* width of the last pass's digit */
-  if (!wide && n > 0 && npass && sbits <= top_bits && !sort_is_local(hdr, local_candidate)) {
-    /* the segment id is the upper part of the last pass's digit: the queue starts where the
-     * digits below (s << (top_bits - sbits)) end, and the digit counts of that pass are known */
-    const uint32_t* h = hist + (npass - 1) * kBins;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const uint32_t limit = min((s + q) << (top_bits - sbits), (uint32_t)kBins);
-      uint32_t sum = 0;
-      for (uint32_t d = lane; d < limit; d += 32) sum += h[d];
-      for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      lo[q] = sum;
-    }
-  } else if (!wide && n > 0) {
-    const uint32_t kshift = ibits + dbits;
-    uint32_t hi[2] = {n, n};                     /* answers: first element whose segment id is >= s, >= s+1 */
-    while (lo[0] < hi[0] || lo[1] < hi[1]) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        if (lo[q] < hi[q]) {                     /* uniform across the warp */
-          const uint32_t span = hi[q] - lo[q];
-          const uint32_t p = lo[q] + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* lo <= p < hi */
-          const bool less = (uint32_t)(__ldg(src + p) >> kshift) < s + q;
-          const uint32_t k = __popc(__ballot_sync(0xffffffffu, less));   /* lanes 0..k-1 saw a smaller id */
-          const uint32_t p_below = __shfl_sync(0xffffffffu, p, k > 0 ? k - 1 : 0);
-          const uint32_t p_at = __shfl_sync(0xffffffffu, p, k < 32 ? k : 31);
-          if (k > 0) lo[q] = p_below + 1;
-          if (k < 32) hi[q] = p_at;
-        }
-      }
-    }
-  }
-  if (lane == 0) {
-    seg_off[s] = lo[0];
-    if (out_seg_off) out_seg_off[s] = lo[0];
-  }
-  if (s == n_seg || !tables) return;             /* the boundaries are all the sequential rules need */
-  /* A queue served high budget first needs no window table: its thresholds fall along the
-   * queue while the positions rise, so the kept requests are a prefix of it.  The prefix
-   * length (first position r with r >= u_r) is found by a 32-ary search and handed to the
-   * decision kernels in win_off. */
-  if (lo[1] > lo[0] && !wide && (ktab[s].narrow & (kSegHighFirst | kSegNoStage)) == kSegHighFirst) {
-    const PardSegConst K = ktab[s];
-    const unsigned long long dmask = dbits >= 64 ? ~0ull : ((1ull << dbits) - 1);
-    uint32_t a = lo[0], b = lo[1];
-    while (a < b) {                                /* uniform across the warp */
-      const uint32_t span = b - a;
-      const uint32_t p = a + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* a <= p < b */
-      const bool kept = p - lo[0] < threshold_u(slack_of((__ldg(src + p) >> ibits) & dmask, K), K);
-      const uint32_t k = __popc(__ballot_sync(0xffffffffu, kept));   /* lanes 0..k-1 probe kept requests */
-      const uint32_t p_below = __shfl_sync(0xffffffffu, p, k > 0 ? k - 1 : 0);
-      const uint32_t p_at = __shfl_sync(0xffffffffu, p, k < 32 ? k : 31);
-      if (k > 0) a = p_below + 1;
-      if (k < 32) b = p_at;
-    }
-    if (lane == 0) { win_off[s] = a - lo[0]; win_cnt[s] = 0; seg_kept[s] = a - lo[0]; }   /* the kept prefix is the queue's kept count */
-    return;
-  }
-  /* batch windows of the queue: 0..b_last of its requests, plus the end marker */
-  uint32_t w = 0, first = 0;
-  if (lane == 0 && lo[1] > lo[0] && !wide) {
-    const PardSegConst K = ktab[s];
-    if (K.narrow & kSegNoStage) {
-      set_status(hdr, PARD_EDATA);               /* requests queued at a stage the pipeline lacks */
-    } else {
-      const unsigned long long dmask = dbits >= 64 ? ~0ull : ((1ull << dbits) - 1);
-      const long long X = (long long)((src[lo[1] - 1] >> ibits) & dmask) - K.A_rel;   /* latest deadline of the queue */
-      const unsigned long long nb = X < 0 ? 0 : win_of((unsigned long long)X, K) + 1;
-      if (nb >= kWinMaxPerSeg) {
-        hdr->use_scan = 1;
-      } else {
-        w = (uint32_t)nb + 1;
-        const unsigned long long at = atomicAdd(&hdr->win_total, (unsigned long long)w);
-        if (at + w > (unsigned long long)capacity) { hdr->use_scan = 1; w = 0; }
-        else first = (uint32_t)at;
-      }
-    }
-  }
-  w = __shfl_sync(0xffffffffu, w, 0);
-  first = __shfl_sync(0xffffffffu, first, 0);
-  if (lane == 0) { win_off[s] = first; win_cnt[s] = w; }
-  for (uint32_t e = lane; e < w; e += 32) win_own[first + e] = s;
-  if (w && lo[1] - lo[0] > kWinLongQueue) {      /* long queue: list its entries for the warp-wide search */
-    uint32_t at = 0;
-    if (lane == 0) at = atomicAdd(&hdr->big_total, w);
-    at = __shfl_sync(0xffffffffu, at, 0);
-    for (uint32_t e = lane; e < w; e += 32) win_big[at + e] = first + e;
-  }
-}
-
-/* The same for calls with thousands of queues, where a warp per queue means more probes than a
- * pass over the elements: here a LANE owns a queue.  Lane i of a warp finds the first element
- * of queue s0 + i by a plain binary search (the lanes' early probes coincide, so they cost one
- * sector), takes the end of its queue from lane i + 1, and the warp draws its queues' table
- * entries from the shared counter with one addition. */
-__global__ void __launch_bounds__(256)
-k_seg_win_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
-               const unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t ibits, uint32_t n_seg,
-               const PardSegConst* __restrict__ ktab, uint32_t* __restrict__ seg_off,
-               uint32_t* __restrict__ out_seg_off, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
-               uint32_t* __restrict__ win_own, uint32_t* __restrict__ win_big, uint32_t capacity,
-               uint32_t force_scan, uint32_t tables, uint32_t* __restrict__ seg_kept) {
-  pdl_wait();
-  const uint32_t warp_g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t s0 = warp_g * 31u;              /* queues s0 .. s0+30, boundaries s0 .. s0+31 */
-  if (s0 > n_seg) return;                        /* whole warps leave together */
-  if (warp_g == 0 && lane == 0 && force_scan) hdr->use_scan = 1;
-  const uint32_t s = s0 + lane;
-  const bool wide = hdr->wide != 0 || hdr->aborted != 0;   /* nothing usable was sorted */
-  const unsigned long long* src = (hdr->npass & 1) ? buf_b : buf_a;
-  const uint32_t dbits = hdr->dbits;
-  const unsigned long long dmask = dbits >= 64 ? ~0ull : ((1ull << dbits) - 1);
-  uint32_t lo = 0;                               /* first element whose segment id is >= s */
-  if (!wide && n > 0 && s <= n_seg) {
-    const uint32_t kshift = ibits + dbits;
-    uint32_t hi = n;
-    while (lo < hi) {
-      const uint32_t mid = lo + (hi - lo) / 2;
-      if ((uint32_t)(__ldg(src + mid) >> kshift) < s) lo = mid + 1; else hi = mid;
-    }
-  }
-  if (lane < 31 && s <= n_seg) {                 /* boundary s0+31 belongs to the next warp */
-    seg_off[s] = lo;
-    if (out_seg_off) out_seg_off[s] = lo;
-  }
-  const uint32_t end = __shfl_down_sync(0xffffffffu, lo, 1);
-  if (!tables) return;                           /* the boundaries are all the sequential rules need */
-  const bool mine = lane < 31 && s < n_seg;
-  uint32_t w = 0;
-  bool high_first = false;
-  if (mine && end > lo && !wide) {
-    const PardSegConst K = ktab[s];
-    if (K.narrow & kSegNoStage) {
-      set_status(hdr, PARD_EDATA);               /* requests queued at a stage the pipeline lacks */
-    } else if (K.narrow & kSegHighFirst) {       /* length of the kept prefix (see k_seg_win) */
-      high_first = true;
-      uint32_t a = lo, b = end;
-      while (a < b) {
-        const uint32_t mid = a + (b - a) / 2;
-        if (mid - lo < threshold_u(slack_of((__ldg(src + mid) >> ibits) & dmask, K), K)) a = mid + 1; else b = mid;
-      }
-      win_off[s] = a - lo;
-      seg_kept[s] = a - lo;                      /* the kept prefix is the queue's kept count */
-      win_cnt[s] = 0;
-    } else {
-      const long long X = (long long)((src[end - 1] >> ibits) & dmask) - K.A_rel;   /* latest deadline of the queue */
-      const unsigned long long nb = X < 0 ? 0 : win_of((unsigned long long)X, K) + 1;
-      if (nb >= kWinMaxPerSeg) hdr->use_scan = 1;
-      else w = (uint32_t)nb + 1;
-    }
-  }
-  uint32_t incl = w;                             /* the warp's queues take consecutive table entries */
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= (uint32_t)o) incl += t;
-  }
-  unsigned long long base = 0;
-  if (lane == 31 && incl) base = atomicAdd(&hdr->win_total, (unsigned long long)incl);
-  base = __shfl_sync(0xffffffffu, base, 31);
-  const unsigned long long first64 = base + incl - w;        /* 64 bits: the counter may pass 2^32 on legal input */
-  if (w && first64 + w > (unsigned long long)capacity) { hdr->use_scan = 1; w = 0; }
-  const uint32_t first = w ? (uint32_t)first64 : 0u;
-  if (mine && !high_first) { win_off[s] = w ? first : 0u; win_cnt[s] = w; }
-  for (uint32_t e = 0; e < w; ++e) win_own[first + e] = s;
-  if (w && end - lo > kWinLongQueue) {           /* long queue: list its entries for the warp-wide search */
-    const uint32_t at = atomicAdd(&hdr->big_total, w);
-    for (uint32_t e = 0; e < w; ++e) win_big[at + e] = first + e;
-  }
-}
-
-/* E and Kp of the table entries of one queue: the warp runs over the queue's windows, 32 at a
+/* E and Kp of the table of one queue (cnt >= 1 entries): the warp runs over the queue's windows, 32 at a
  * time. */
-__device__ __forceinline__ uint32_t win_prefix_warp(uint32_t s, const PardSegConst* __restrict__ ktab,
-                                                const uint32_t* __restrict__ win_off,
-                                                const uint32_t* __restrict__ win_cnt, WinEntry* __restrict__ wtab,
-                                                uint32_t lane, uint32_t raw) {
-  const uint32_t w0 = win_off[s], cnt = win_cnt[s];
-  if (cnt == 0) return 0xffffffffu;              /* no table (served high budget first, or no such stage) */
-  const uint32_t cap = ktab[s].cap;
-  WinEntry* tab = wtab + w0;
-  const uint32_t P0 = __ldcg(&tab[0].P);          /* other blocks may have written the P (long queues) */
+__device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __restrict__ tab, uint32_t cnt, uint32_t lane, uint32_t raw) {
+  const uint32_t P0 = __ldcg(&tab[0].P);
   int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;     /* the expired run: u = 0 */
   uint32_t k_carry = 0;
   if (lane == 0) { tab[0].E = e_carry; tab[0].Kp = 0; }
@@ -1931,90 +1723,277 @@ __device__ __forceinline__ uint32_t win_prefix_warp(uint32_t s, const PardSegCon
   return n_q == 0 ? 0u : (raw ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1)));
 }
 
-/* The window tables.  P of every entry: a search in the queue's sorted elements, by one lane
- * (short queue) or by a whole warp with 32 probes per step (long queue).  (Counting finished
- * entries per queue so that the last finisher could run the queue's prefix pass in the same
- * kernel was tried: the fence and the atomic per entry cost more than the launch they saved
- * once there are thousands of queues.) */
-__global__ void __launch_bounds__(256)
-k_win_bounds(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a,
-             const unsigned long long* __restrict__ buf_b, uint32_t ibits, uint32_t n_seg,
-             const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off,
-             const uint32_t* __restrict__ win_off, const uint32_t* __restrict__ win_cnt,
-             const uint32_t* __restrict__ win_own, const uint32_t* __restrict__ win_big,
-             uint32_t* __restrict__ win_done, WinEntry* __restrict__ wtab, uint32_t raw, uint32_t* __restrict__ seg_kept) {
+/* Queue boundaries, window tables and output offsets of kWinQueues queues per block, from the sorted
+ * elements:
+ *   - every queue's first position: read off the last pass's digit counts when the queue id lies inside
+ *     that digit, else a warp's 32-ary search for it in the elements' upper bits;
+ *   - its number of windows, from its latest deadline, and a range of table entries for the block's
+ *     queues from a shared counter (none left, or a queue with thousands: the scan path decides);
+ *   - P of every entry, a lane each: four-way search of the window's first deadline in the queue;
+ *   - E, Kp and the queue's kept count, a warp per queue; for a queue served high budget first the
+ *     length of its kept prefix instead (win_off), by a warp's 32-ary search: its thresholds fall along
+ *     the queue while the positions rise;
+ *   - in the last block to finish, the output offsets of all queues' survivors.
+ * Bound by dependent loads.  As four launches (boundaries, entries of short queues by a lane and of long
+ * ones by a warp each, prefixes, offsets) the same took 9 us more for 256 queues of 4,096 requests (a
+ * replay epoch: 73 -> 64 us) and 12 more for 4,096 of them. */
+constexpr int kWinQueues = 16;
+constexpr int kWinThreads = 32 * kWinQueues;
+__global__ void __launch_bounds__(kWinThreads, 2)
+k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
+          uint32_t ibits, uint32_t n_seg, const PardSegConst* __restrict__ ktab, uint32_t* __restrict__ seg_off,
+          uint32_t* __restrict__ out_seg_off, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
+          WinEntry* __restrict__ wtab, uint32_t capacity, uint32_t force_scan, const uint32_t* __restrict__ hist, uint32_t sbits,
+          uint32_t local_candidate, uint32_t tables, uint32_t raw, uint32_t* __restrict__ seg_kept,
+          uint32_t* __restrict__ kept_base, uint32_t* __restrict__ chunk_base, uint32_t* __restrict__ out_seg_kept,
+          unsigned long long* __restrict__ out_n_kept) {
   pdl_wait();
-  if (hdr->use_scan || hdr->wide || hdr->aborted) return;
-  const uint32_t lane = threadIdx.x & 31;
-  const unsigned long long* src = (hdr->npass & 1) ? buf_b : buf_a;
-  const uint32_t dbits = hdr->dbits;
+  __shared__ uint32_t s_lo[kWinQueues + 1], s_w[kWinQueues], s_first[kWinQueues + 1];
+  __shared__ long long s_A[kWinQueues], s_d[kWinQueues];
+  __shared__ uint32_t s_base, s_scan;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
+  const uint32_t s0 = blockIdx.x * kWinQueues, s = s0 + q;
+  const bool usable = hdr->wide == 0 && hdr->aborted == 0 && n > 0;       /* else nothing was sorted */
+  const uint32_t npass = hdr->npass, dbits = hdr->dbits;
+  const unsigned long long* src = (npass & 1) ? buf_b : buf_a;
   const unsigned long long dmask = dbits >= 64 ? ~0ull : ((1ull << dbits) - 1);
-  /* entries of short queues: one lane each, plain binary search */
-  {
-    /* without use_scan every request for entries was granted, so the counter is within the table */
-    const uint32_t total = (uint32_t)hdr->win_total, step = gridDim.x * blockDim.x;
-    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += step) {
-      const uint32_t s = win_own[e];
-      uint32_t lo = seg_off[s], hi = seg_off[s + 1];
-      if (hi - lo > kWinLongQueue) continue;
-      const uint32_t first = lo;
-      const long long thr = ktab[s].A_rel + (long long)(e - win_off[s]) * ktab[s].d;
-      while (lo < hi) {
-        const uint32_t mid = lo + (hi - lo) / 2;
-        if ((long long)((__ldg(src + mid) >> ibits) & dmask) < thr) lo = mid + 1; else hi = mid;
+  /* first element whose queue id is >= s (warp 0 also: >= s0 + kWinQueues) */
+  uint32_t lo[2] = {0, 0};
+  const uint32_t want[2] = {s, q == 0 ? s0 + kWinQueues : s};
+  if (usable) {
+    const uint32_t top_bits = npass ? hdr->keybits - 8 * (npass - 1) : 0;   /* width of the last pass's digit */
+    if (npass && sbits <= top_bits && !sort_is_local(hdr, local_candidate)) {
+      /* the queue id is the upper part of that digit: the queue starts where the digits below
+       * (s << (top_bits - sbits)) end */
+      const uint32_t* h = hist + (npass - 1) * kBins;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t limit = (uint32_t)min((unsigned long long)want[k] << (top_bits - sbits), (unsigned long long)kBins);
+        uint32_t sum = 0;
+        for (uint32_t d = lane; d < limit; d += 32) sum += h[d];
+        lo[k] = __reduce_add_sync(0xffffffffu, sum);
       }
-      wtab[e].P = lo - first;
+    } else {
+      const uint32_t kshift = ibits + dbits;
+      uint32_t hi[2] = {n, q == 0 ? n : 0u};
+      while (lo[0] < hi[0] || lo[1] < hi[1]) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (lo[k] < hi[k]) {                     /* uniform across the warp */
+            const uint32_t span = hi[k] - lo[k];
+            const uint32_t p = lo[k] + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* lo <= p < hi */
+            const bool less = (uint32_t)(__ldg(src + p) >> kshift) < want[k];
+            const uint32_t c = __popc(__ballot_sync(0xffffffffu, less));   /* lanes 0..c-1 saw a smaller id */
+            const uint32_t p_below = __shfl_sync(0xffffffffu, p, c > 0 ? c - 1 : 0);
+            const uint32_t p_at = __shfl_sync(0xffffffffu, p, c < 32 ? c : 31);
+            if (c > 0) lo[k] = p_below + 1;
+            if (c < 32) hi[k] = p_at;
+          }
+        }
+      }
     }
   }
-  /* entries of long queues: one warp each, 32 probes per step */
-  const uint32_t total = hdr->big_total, step = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < total; i += step) {   /* whole warps stay together */
-    const uint32_t e = win_big[i];
-    const uint32_t s = win_own[e], b = e - win_off[s];
-    const PardSegConst K = ktab[s];
-    const long long thr = K.A_rel + (long long)b * K.d;     /* window >= b  <=>  deadline offset >= thr */
-    uint32_t lo = seg_off[s], hi = seg_off[s + 1];
-    const uint32_t first = lo;
-    while (lo < hi) {
-      const uint32_t span = hi - lo;
-      const uint32_t p = lo + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);
-      const bool less = (long long)((__ldg(src + p) >> ibits) & dmask) < thr;
-      const uint32_t k = __popc(__ballot_sync(0xffffffffu, less));
-      const uint32_t p_below = __shfl_sync(0xffffffffu, p, k > 0 ? k - 1 : 0);
-      const uint32_t p_at = __shfl_sync(0xffffffffu, p, k < 32 ? k : 31);
-      if (k > 0) lo = p_below + 1;
-      if (k < 32) hi = p_at;
+  if (lane == 0) {
+    s_lo[q] = lo[0];
+    if (q == 0) s_lo[kWinQueues] = lo[1];
+    if (s <= n_seg) {
+      seg_off[s] = lo[0];
+      if (out_seg_off) out_seg_off[s] = lo[0];
     }
-    /* a long queue has few hundred entries at most, spread over as many warps: they are counted,
-     * and the warp that stores the last one goes on to the queue's prefix pass */
-    uint32_t last = 0;
-    if (lane == 0) {
-      wtab[e].P = lo - first;
-      __threadfence();
-      last = atomicAdd(&win_done[s], 1u) + 1 == win_cnt[s] ? 1u : 0u;
-    }
-    if (__shfl_sync(0xffffffffu, last, 0)) {
-      __threadfence();
-      const uint32_t kept = win_prefix_warp(s, ktab, win_off, win_cnt, wtab, lane, raw);
-      if (lane == 0 && kept != 0xffffffffu) seg_kept[s] = kept;
+    if (q == 0 && s0 + kWinQueues == n_seg) {
+      seg_off[n_seg] = lo[1];
+      if (out_seg_off) out_seg_off[n_seg] = lo[1];
     }
   }
+  if (!tables) return;                             /* the boundaries are all the sequential rules need */
+  if (tid == 0) s_scan = force_scan;
+  __syncthreads();
+  const uint32_t begin = s_lo[q], end = s_lo[q + 1];
+  const bool mine = s < n_seg && usable && end > begin;
+  bool high_first = false;
+  {
+    uint32_t w = 0;
+    if (mine) {                                    /* whole warps */
+      const PardSegConst K = ktab[s];
+      if (K.narrow & kSegNoStage) {
+        if (lane == 0) set_status(hdr, PARD_EDATA);   /* requests queued at a stage the pipeline lacks */
+      } else if (K.narrow & kSegHighFirst) {
+        high_first = true;
+        uint32_t a = begin, b = end;
+        while (a < b) {                            /* uniform across the warp */
+          const uint32_t span = b - a;
+          const uint32_t p = a + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* a <= p < b */
+          const bool kept = p - begin < threshold_u(slack_of((__ldg(src + p) >> ibits) & dmask, K), K);
+          const uint32_t c = __popc(__ballot_sync(0xffffffffu, kept));   /* lanes 0..c-1 probe kept requests */
+          const uint32_t p_below = __shfl_sync(0xffffffffu, p, c > 0 ? c - 1 : 0);
+          const uint32_t p_at = __shfl_sync(0xffffffffu, p, c < 32 ? c : 31);
+          if (c > 0) a = p_below + 1;
+          if (c < 32) b = p_at;
+        }
+        if (lane == 0) { win_off[s] = a - begin; win_cnt[s] = 0; seg_kept[s] = a - begin; }   /* the kept prefix is the queue's kept count */
+      } else {
+        const long long X = (long long)((src[end - 1] >> ibits) & dmask) - K.A_rel;   /* latest deadline of the queue */
+        const unsigned long long nb = X < 0 ? 0 : win_of((unsigned long long)X, K) + 1;
+        if (nb >= kWinMaxPerSeg) { if (lane == 0) s_scan = 1; }
+        else w = (uint32_t)nb + 1;                 /* windows 0..nb-1 and the end marker */
+        if (lane == 0) { s_A[q] = K.A_rel; s_d[q] = K.d; }
+      }
+    }
+    if (lane == 0) s_w[q] = w;
+  }
+  __syncthreads();
+  if (tid < 32) {
+    const uint32_t w = lane < kWinQueues ? s_w[lane] : 0u;
+    uint32_t x = w;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane < kWinQueues) s_first[lane] = x - w;
+    if (lane == 31) {
+      s_first[kWinQueues] = x;
+      const unsigned long long at = x && !s_scan ? atomicAdd(&hdr->win_total, (unsigned long long)x) : 0ull;
+      if (at + x > (unsigned long long)capacity) s_scan = 1;
+      s_base = (uint32_t)at;
+      if (s_scan) hdr->use_scan = 1;
+    }
+  }
+  __syncthreads();
+  const uint32_t total = s_scan ? 0u : s_first[kWinQueues], base = s_base;
+  if (lane == 0 && s < n_seg && !high_first) {
+    win_off[s] = base + s_first[q];
+    win_cnt[s] = total ? s_w[q] : 0u;
+  }
+  for (uint32_t e = tid; e < total; e += kWinThreads) {
+    uint32_t k = 0;
+#pragma unroll
+    for (int b = kWinQueues / 2; b; b >>= 1)
+      if (s_first[k + b] <= e) k += b;             /* last queue whose entries begin at or before e */
+    const long long thr = s_A[k] + (long long)(e - s_first[k]) * s_d[k];     /* window >= b  <=>  deadline offset >= thr */
+    const uint32_t first = s_lo[k];
+    uint32_t a = first, b = s_lo[k + 1];
+    while (a < b) {                                /* first position whose offset is >= thr; three probes per step */
+      const uint32_t quarter = (b - a) / 4, m1 = a + quarter, m2 = a + 2 * quarter, m3 = a + 3 * quarter;   /* a <= m1 <= m2 <= m3 < b */
+      const bool l1 = (long long)((__ldg(src + m1) >> ibits) & dmask) < thr, l2 = (long long)((__ldg(src + m2) >> ibits) & dmask) < thr,
+                 l3 = (long long)((__ldg(src + m3) >> ibits) & dmask) < thr;
+      if (l3) a = m3 + 1;
+      else if (l2) { a = m2 + 1; b = m3; }
+      else if (l1) { a = m1 + 1; b = m2; }
+      else b = m1;
+    }
+    wtab[base + e].P = a - first;
+  }
+  __syncthreads();
+  if (total && mine && !high_first && s_w[q]) {
+    const uint32_t kept = win_prefix_warp(ktab[s].cap, wtab + base + s_first[q], s_w[q], lane, raw);
+    if (lane == 0) seg_kept[s] = kept;             /* known before any request has been decided */
+  }
+  if (!last_block_done(&hdr->win_done)) return;
+  kept_scan_block<kWinThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
 }
 
-/* E and Kp of the table entries of the short queues: one warp per queue runs over its windows,
- * 32 at a time. */
-__global__ void __launch_bounds__(256)
-k_win_prefix(const PlanHeader* __restrict__ hdr, uint32_t n_seg, const PardSegConst* __restrict__ ktab,
-             const uint32_t* __restrict__ seg_off, const uint32_t* __restrict__ win_off,
-             const uint32_t* __restrict__ win_cnt, WinEntry* __restrict__ wtab, uint32_t raw,
-             uint32_t* __restrict__ seg_kept) {
+/* The same for calls with very many short queues, where a warp per queue would mostly idle: a thread
+ * per queue (plain binary searches whose early probes coincide across the lanes; its few windows one
+ * after the other), 511 queues per block. */
+constexpr uint32_t kShortQueue = 128;              /* requests per queue on average below which this form is taken */
+__global__ void __launch_bounds__(kWinThreads)
+k_windows_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
+               uint32_t ibits, uint32_t n_seg, const PardSegConst* __restrict__ ktab, uint32_t* __restrict__ seg_off,
+               uint32_t* __restrict__ out_seg_off, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
+               WinEntry* __restrict__ wtab, uint32_t capacity, uint32_t force_scan, uint32_t tables, uint32_t raw,
+               uint32_t* __restrict__ seg_kept, uint32_t* __restrict__ kept_base, uint32_t* __restrict__ chunk_base,
+               uint32_t* __restrict__ out_seg_kept, unsigned long long* __restrict__ out_n_kept) {
   pdl_wait();
-  if (hdr->use_scan || hdr->wide || hdr->aborted) return;
-  const uint32_t s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (s >= n_seg) return;                          /* whole warps leave together */
-  if (seg_off[s + 1] - seg_off[s] > kWinLongQueue) return;   /* done by k_win_bounds */
-  const uint32_t kept = win_prefix_warp(s, ktab, win_off, win_cnt, wtab, threadIdx.x & 31, raw);
-  if ((threadIdx.x & 31) == 0 && kept != 0xffffffffu) seg_kept[s] = kept;     /* the queue's kept count, known before the decision */
+  __shared__ uint32_t s_lo[kWinThreads], s_warp[kWinThreads / 32], s_base, s_scan;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t s = blockIdx.x * (kWinThreads - 1u) + tid;          /* the last thread only finds the end of the one before */
+  const bool usable = hdr->wide == 0 && hdr->aborted == 0 && n > 0;
+  const uint32_t dbits = hdr->dbits, kshift = ibits + dbits;
+  const unsigned long long* src = (hdr->npass & 1) ? buf_b : buf_a;
+  const unsigned long long dmask = dbits >= 64 ? ~0ull : ((1ull << dbits) - 1);
+  auto first_with = [&](uint32_t a, uint32_t b, auto below) {        /* first position in [a, b) that is not below */
+    while (a < b) {
+      const uint32_t mid = a + (b - a) / 2;
+      if (below(mid, __ldg(src + mid))) a = mid + 1; else b = mid;
+    }
+    return a;
+  };
+  uint32_t lo = 0;
+  if (usable && s <= n_seg) lo = first_with(0u, n, [&](uint32_t, unsigned long long e) { return (uint32_t)(e >> kshift) < s; });
+  s_lo[tid] = lo;
+  if (tid == 0) s_scan = force_scan;
+  if (s <= n_seg && (tid + 1 < kWinThreads || s == n_seg)) {
+    seg_off[s] = lo;
+    if (out_seg_off) out_seg_off[s] = lo;
+  }
+  if (!tables) return;
+  __syncthreads();
+  const bool owner = tid + 1 < kWinThreads && s < n_seg;
+  const uint32_t end = owner ? s_lo[tid + 1] : lo;
+  uint32_t w = 0;
+  bool high_first = false;
+  if (owner && usable && end > lo) {
+    const PardSegConst K = ktab[s];
+    if (K.narrow & kSegNoStage) {
+      set_status(hdr, PARD_EDATA);
+    } else if (K.narrow & kSegHighFirst) {
+      high_first = true;
+      const uint32_t k = first_with(lo, end, [&](uint32_t p, unsigned long long e) { return p - lo < threshold_u(slack_of((e >> ibits) & dmask, K), K); }) - lo;
+      win_off[s] = k;
+      win_cnt[s] = 0;
+      seg_kept[s] = k;
+    } else {
+      const long long X = (long long)((src[end - 1] >> ibits) & dmask) - K.A_rel;
+      const unsigned long long nb = X < 0 ? 0 : win_of((unsigned long long)X, K) + 1;
+      if (nb >= kWinMaxPerSeg) s_scan = 1;
+      else w = (uint32_t)nb + 1;
+    }
+  }
+  uint32_t x = w;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= (uint32_t)o) x += y;
+  }
+  if (lane == 31) s_warp[warp] = x;
+  __syncthreads();
+  const uint32_t v = lane < kWinThreads / 32 ? s_warp[lane] : 0u;
+  const uint32_t total = __reduce_add_sync(0xffffffffu, v), before = x - w + __reduce_add_sync(0xffffffffu, lane < warp ? v : 0u);
+  if (tid == 0) {
+    const unsigned long long at = total && !s_scan ? atomicAdd(&hdr->win_total, (unsigned long long)total) : 0ull;
+    if (at + total > (unsigned long long)capacity) s_scan = 1;
+    s_base = (uint32_t)at;
+    if (s_scan) hdr->use_scan = 1;
+  }
+  __syncthreads();
+  if (owner && !high_first) {
+    const bool scan = s_scan != 0;
+    WinEntry* tab = wtab + s_base + before;
+    win_off[s] = s_base + before;
+    win_cnt[s] = scan ? 0u : w;
+    if (!scan && w) {
+      const PardSegConst K = ktab[s];
+      uint32_t P = lo, kept = 0;
+      int32_t E = kWinInf;
+      for (uint32_t b = 0; b < w; ++b) {           /* entry b from what window b - 1 (at first: deadline < A) holds */
+        const long long thr = K.A_rel + (long long)b * K.d;
+        const uint32_t next = first_with(P, end, [&](uint32_t, unsigned long long e) { return (long long)((e >> ibits) & dmask) < thr; });
+        const uint32_t p = P - lo, q = next - lo;
+        if (q > p) {
+          const uint32_t u = b ? win_u(b - 1, K.cap) : 0u;
+          E = min(E, (int32_t)u - (int32_t)(q - 1));
+          const uint32_t top = u < q ? u : q;
+          kept += top > p ? top - p : 0;
+        }
+        tab[b].P = q;
+        tab[b].E = E;
+        tab[b].Kp = kept;
+        P = next;
+      }
+      seg_kept[s] = raw ? kept : (uint32_t)((int32_t)(end - lo) - 1 + min(E, 1));
+    }
+  }
+  if (!last_block_done(&hdr->win_done)) return;
+  kept_scan_block<kWinThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
 }
 
 /* The window tables of a call with few queues, from the counts k_pack took: P is the running sum
@@ -2068,8 +2047,8 @@ k_win_from_counts(PlanHeader* hdr, uint32_t n_seg, const PardSegConst* __restric
     __threadfence_block();
     __syncwarp();
     /* P as the decision reads it: entry b = requests in windows below b, i.e. the sum up to entry b */
-    const uint32_t kept = win_prefix_warp(q, ktab, win_off, win_cnt, wtab, lane, raw);
-    if (lane == 0) s_kept[q] = kept == 0xffffffffu ? 0u : kept;      /* the queue's kept count, known before the sort */
+    const uint32_t kept = cnt ? win_prefix_warp(ktab[q].cap, wtab + off, cnt, lane, raw) : 0u;
+    if (lane == 0) s_kept[q] = kept;      /* the queue's kept count, known before the sort */
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -2576,9 +2555,6 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   uint32_t* win_off = (uint32_t*)(ws + L.win_off);
   WinEntry* wtab = (WinEntry*)(ws + L.wtab);
   uint32_t* win_cnt = (uint32_t*)(ws + L.win_cnt);
-  uint32_t* win_own = (uint32_t*)(ws + L.win_own);
-  uint32_t* win_big = (uint32_t*)(ws + L.win_big);
-  uint32_t* win_done = (uint32_t*)(ws + L.win_done);
   uint32_t* whist = (uint32_t*)(ws + L.whist);
   unsigned long long* buf_a = (unsigned long long*)(ws + L.buf_a);
   unsigned long long* buf_b = (unsigned long long*)(ws + L.buf_b);
@@ -2625,6 +2601,23 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     return launch_policy_emit(pa, stream);
   };
 
+  /* queue boundaries, and for the planner's own rule the window tables and output offsets; id_bits > 8:
+   * the boundaries are searched, never read off the digit counts */
+  auto launch_windows = [&](bool tables, uint32_t local_candidate, uint32_t id_bits = 64u) {
+    if (n / L.n_seg < kShortQueue && L.n_seg >= 4096)
+      launch_pdl(k_windows_many, L.n_seg / (kWinThreads - 1u) + 1, kWinThreads, 0, stream, hdr, (const unsigned long long*)buf_a,
+                 (const unsigned long long*)buf_b, n32, ibits, L.n_seg, (const PardSegConst*)ktab, seg_off, out->d_seg_offsets,
+                 win_off, win_cnt, wtab, L.win_capacity, (mode & PARD_MODE_SCAN) ? 1u : 0u, tables ? 1u : 0u,
+                 (mode & PARD_MODE_RAW) ? 1u : 0u, seg_kept, kept_base, chunk_base, out->d_seg_kept,
+                 (unsigned long long*)out->d_n_kept);
+    else
+      launch_pdl(k_windows, L.n_seg / kWinQueues + 1, kWinThreads, 0, stream, hdr, (const unsigned long long*)buf_a,
+               (const unsigned long long*)buf_b, n32, ibits, L.n_seg, (const PardSegConst*)ktab, seg_off, out->d_seg_offsets, win_off,
+               win_cnt, wtab, L.win_capacity, (mode & PARD_MODE_SCAN) ? 1u : 0u, (const uint32_t*)hist, id_bits, local_candidate,
+               tables ? 1u : 0u, (mode & PARD_MODE_RAW) ? 1u : 0u, seg_kept, kept_base, chunk_base, out->d_seg_kept,
+               (unsigned long long*)out->d_n_kept);
+  };
+
   /* ---- keys wider than one sort element: see k_wide_reset.  Run only when a finished call has
    * reported that width (the host cannot know the deadline span beforehand), hence not for
    * PARD_MODE_NOWAIT, whose caller gets PARD_ERANGE from pard_plan_status as before. ---- */
@@ -2663,12 +2656,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     }
     launch_pdl(k_wide_final, grid_n, 256, 0, stream, req4, n32, n_ctx, S, sbits, ibits, hdr, (const uint32_t*)order, buf_a);
     launch_pdl(k_wide_done, 1, 1, 0, stream, hdr, sbits);
-    if (L.n_seg >= kManyQueues)
-      launch_pdl(k_seg_win_many, ((L.n_seg + 31) / 31 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab,
-                 seg_off, out->d_seg_offsets, win_off, win_cnt, win_own, win_big, L.win_capacity, 0u, 0u, seg_kept);
-    else
-      launch_pdl(k_seg_win, (L.n_seg + 1 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab, seg_off,
-                 out->d_seg_offsets, win_off, win_cnt, win_own, win_big, L.win_capacity, 0u, (const uint32_t*)hist, sbits, 0u, 0u, seg_kept);
+    launch_windows(false, 0u, sbits);
     PolicyArgs pa = {};
     pa.hdr = hdr; pa.buf_a = buf_a; pa.buf_b = buf_b;
     pa.n = n32; pa.ibits = ibits; pa.n_seg = L.n_seg; pa.mode = mode;
@@ -2779,14 +2767,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   mark();
   if (win_hist) {
     /* boundaries and tables are there already */
-  } else if (L.n_seg >= kManyQueues)
-    launch_pdl(k_seg_win_many, ((L.n_seg + 31) / 31 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab,
-               seg_off, out->d_seg_offsets, win_off, win_cnt, win_own, win_big, L.win_capacity,
-               (mode & PARD_MODE_SCAN) ? 1u : 0u, rule_walk ? 0u : 1u, seg_kept);
-  else
-    launch_pdl(k_seg_win, (L.n_seg + 1 + 7) / 8, 256, 0, stream, hdr, buf_a, buf_b, n32, ibits, L.n_seg, ktab, seg_off,
-               out->d_seg_offsets, win_off, win_cnt, win_own, win_big, L.win_capacity,
-               (mode & PARD_MODE_SCAN) ? 1u : 0u, (const uint32_t*)hist, ctx_sort ? 64u : sbits, local_cand, rule_walk ? 0u : 1u, seg_kept);
+  } else {
+    launch_windows(!rule_walk, local_cand, ctx_sort ? 64u : sbits);
+  }
   if (n > 0 && rule_walk) {
     /* a rule without rising thresholds: every queue is walked in order (pard_policy.cu) */
     PolicyArgs pa = {};
@@ -2802,14 +2785,6 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     long long* est = (long long*)out->d_est_us;
     const bool raw = mode & PARD_MODE_RAW;
     /* window tables, and the decision from them */
-    if (!win_hist) {
-      launch_pdl(k_win_bounds, std::min<uint32_t>((L.win_capacity + 7) / 8, (uint32_t)sms * 8), 256, 0, stream,
-          hdr, buf_a, buf_b, ibits, L.n_seg, ktab, seg_off, win_off, win_cnt, win_own, win_big, win_done, wtab, raw ? 1u : 0u, seg_kept);
-      launch_pdl(k_win_prefix, (L.n_seg + 7) / 8, 256, 0, stream, hdr, L.n_seg, ktab, seg_off, win_off, win_cnt, wtab, raw ? 1u : 0u, seg_kept);
-      /* the tables give every queue's kept count: the output offsets are known before the decision */
-      launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
-                 (unsigned long long*)out->d_n_kept);
-    }
     mark();
     const uint32_t win_grid = (uint32_t)((n + (uint64_t)kDecTile - 1) / kDecTile);
     auto decide_win = raw ? (state->d_priority ? k_decide_win<true, true> : k_decide_win<true, false>)
@@ -2852,8 +2827,7 @@ extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t sta
    * most a sort tile: one kernel.  Else always clear and seg_const; with many queues also
    * key_width (and, when n > 0, ctx_span); when n > 0: prepass, pack, the radix passes, decide_win
    * and the scan path (one kernel that returns at once); with at most 64 queues the counted window
-   * tables (win_from_counts), else the queue boundaries, the searched tables and the output
-   * offsets that follow from them (seg_win, win_bounds, win_prefix, kept_scan). */
+   * tables (win_from_counts), else the queue boundaries and the searched ones (windows). */
   const uint64_t n_seg = (uint64_t)n_ctx * (uint64_t)stage_stride;
   const uint32_t width_kernels = n_seg <= kFoldSegs ? 0 : 1;   /* key_width (+ ctx_span when n > 0) */
   const bool local_cand = local_sort_candidate(n, n_ctx);
@@ -2866,10 +2840,9 @@ extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t sta
   }
   const uint32_t own = sort_own_passes(L.sort_tiles, L.max_passes, sms, local_cand ? 1u : 0u);
   const uint32_t passes = own + (own < L.max_passes ? 1 : 0);   /* and the kernel that does the rest */
-  const bool counted = n > 0 && n_seg <= kHistSegs && !local_cand;
   if (n_ctx == 1 && n > 0 && n <= (uint64_t)kSortTile) *launches = 1;
-  else if (n == 0) *launches = 4 + width_kernels;               /* clear, (key_width,) seg_const, seg_win, kept_scan */
-  else *launches = 2 + 2 * width_kernels + 2 + local_kernels + passes + 2 + (counted ? 1 : 4);
+  else if (n == 0) *launches = 4 + width_kernels;               /* clear, (key_width,) seg_const, windows, kept_scan */
+  else *launches = 2 + 2 * width_kernels + 2 + local_kernels + passes + 2 + 1;
   return PARD_OK;
 }
 

@@ -45,8 +45,7 @@ struct PlanHeader {
   uint32_t wide;              /* 1: segment, deadline and index bits exceed 64; nothing is sorted */
   uint32_t use_scan;          /* 1: too many batch windows for the window tables: decide by scanning */
   uint32_t aborted;           /* 1: a bounded wait ran out; the sort is incomplete and every later kernel returns */
-  uint32_t big_total;         /* window-table entries that belong to long queues */
-  uint32_t agg_done;          /* blocks of k_tile_agg that have stored their aggregates */
+  uint32_t win_done;          /* blocks of k_windows that have finished */
   uint32_t seg_done;          /* blocks of k_seg_const that have stored their constants */
   uint32_t unsorted;          /* 1: some request's ctx is smaller than its predecessor's */
   uint32_t ctx_too_big;       /* 1: some ctx holds more requests than one sort tile */
@@ -57,7 +56,7 @@ struct PlanHeader {
   uint32_t pair_steps_back;   /* 1: some request's (ctx, deadline) lies before its predecessor's */
   uint32_t lookup;            /* 1: the elements hold no deadline: it has to be looked up in the request array */
   uint32_t sort_bar[kMaxPasses]; /* blocks of k_sort_rest that have finished each of its passes */
-  uint32_t pad[64 - 25 - kMaxPasses - (kMaxPasses + 1)];
+  uint32_t pad[64 - 24 - kMaxPasses - (kMaxPasses + 1)];
 };
 static_assert(sizeof(PlanHeader) == 256, "header is 256 bytes");
 

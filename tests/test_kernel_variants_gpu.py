@@ -110,3 +110,15 @@ def test_estimate_w_shapes(M):
             rc, got = run_estimate_w(wl, s.astype(np.int32), num, den, seed, fill=0)
             assert rc == 0
             assert np.array_equal(got, np.asarray(want).reshape(got.shape))
+
+
+# ---- window tables of many queues: a warp or a thread per queue, block and table edges ------------
+@pytest.mark.parametrize("n_ctx,S,n", [(5, 15, 90_000), (5, 16, 90_000), (17, 16, 200_001), (1366, 3, 30_000), (4088, 1, 50_000),
+                                       (511, 9, 20_000), (2731, 3, 1_100_000)])
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW, pb.PARD_MODE_SCAN])
+def test_window_tables_of_many_queues(n_ctx, S, n, mode):
+    rng = np.random.default_rng(n)
+    wl = several_ctx(n_ctx, np.bincount(rng.integers(0, n_ctx, size=n), minlength=n_ctx), S=S, sort=False, mix=True, m=2)
+    check(wl, mode)
+    wl.state.priority = rng.integers(0, 2, size=(n_ctx, S)).astype(np.uint8)
+    check(wl, mode)
