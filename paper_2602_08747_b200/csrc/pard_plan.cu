@@ -126,6 +126,134 @@ k_clear(uint4* __restrict__ p, unsigned long long n16) {
     p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+/* Width of the sort key, once the widest deadline span is known, and the part of it that the
+ * passes have to sort.  key_sbits: the queue-id bits to sort (all of them, or the stage bits only
+ * when the passes stay inside the contexts' ranges).  The deadline field below them needs no pass
+ * when every queue's requests stand in the order it asks for: in arrival order the index alone
+ * orders a queue, and in budget order (low budget first everywhere) requests whose deadlines never
+ * step back along the array, or along every ctx of an array grouped by ctx, are ordered as they
+ * come.  (2^24 such requests in 256 contexts: one pass instead of four, 696 -> 408 us for the call.) */
+__device__ __forceinline__ void set_key_width(PlanHeader* hdr, unsigned long long span, uint32_t sbits, uint32_t ibits,
+                                              uint32_t key_sbits, uint32_t arrival_order, bool priority) {
+  uint32_t dbits = bit_width64(span);
+  if (arrival_order && sbits + dbits + ibits > 64) {    /* no room: the rule reads the deadlines from the requests */
+    dbits = 0;
+    hdr->lookup = 1;
+  }
+  const bool in_order = arrival_order || (!priority && !(hdr->time_steps_back && hdr->pair_steps_back));
+  const uint32_t skip = in_order ? dbits : 0u;
+  hdr->span_max = span;
+  hdr->dbits = dbits;
+  hdr->pshift = skip;
+  hdr->keybits = key_sbits + dbits - skip;
+  hdr->npass = (key_sbits + dbits - skip + 7) / 8;
+  if (sbits + dbits + ibits > 64) {
+    hdr->npass = 0;
+    hdr->wide = 1;
+    set_status(hdr, PARD_ERANGE);
+  }
+}
+
+/* What the constants of a call's queues are made from, and what follows from them and the deadline
+ * ranges before any request is packed. */
+struct ConstArgs {
+  PipeTable pipes;
+  pard_queue_state_t st;
+  uint32_t n_pipelines, n_ctx;
+  PardSegConst* ktab;
+  uint32_t sbits, ibits, key_sbits;
+  uint32_t with_key_width;         /* the block that finishes last also finds the key width (no launches for it) */
+  uint32_t arrival_order, win_hist, force_scan;
+  uint32_t* win_off;
+  uint32_t* win_cnt;
+};
+
+/* By one whole block, once every ctx's deadline range and every queue's constants are there: what
+ * hangs on both.  RANGES: the constants do not know the ranges yet. */
+template <bool RANGES>
+__device__ void finish_constants(const ConstArgs& a, const unsigned long long* ctx_dmin_inv, const unsigned long long* ctx_dmax,
+                                 PlanHeader* hdr) {
+  __shared__ unsigned long long s_span[8];
+  __shared__ uint32_t s_w[kHistSegs];
+  __shared__ uint32_t s_scan;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, S = (uint32_t)a.st.stage_stride, n_seg = a.n_ctx * S;
+  unsigned long long span = 0;
+  for (uint32_t c = tid; c < a.n_ctx; c += blockDim.x) {
+    const unsigned long long lo = ~__ldcg(&ctx_dmin_inv[c]), hi = __ldcg(&ctx_dmax[c]);
+    if (lo <= hi && hi - lo > span) span = hi - lo;
+  }
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, span, o);
+    span = x > span ? x : span;
+  }
+  if (lane == 0) s_span[tid >> 5] = span;
+  if (tid == 0) s_scan = a.force_scan;
+  __syncthreads();
+  if (tid == 0) {
+    for (uint32_t w = 1; w < blockDim.x / 32; ++w) span = s_span[w] > span ? s_span[w] : span;
+    set_key_width(hdr, span, a.sbits, a.ibits, a.key_sbits, a.arrival_order, a.st.d_priority != nullptr);
+  }
+  /* Few queues: their batch-window tables are COUNTED while the requests are packed (k_pack)
+   * instead of being searched for in the sorted elements afterwards.  That needs the tables'
+   * extents before any request has been looked at: a queue can have no window beyond that of its
+   * ctx's latest deadline.  Entry 0 of a queue counts its requests with deadline < A, entry b + 1
+   * those of window b; every queue has at least entry 0, so that the counts also give the queues'
+   * lengths. */
+  if (!RANGES && !a.win_hist) return;
+  for (uint32_t q = tid; q < n_seg; q += blockDim.x) {   /* all queues side by side */
+    const uint32_t c = q / S;
+    const unsigned long long lo = ~__ldcg(&ctx_dmin_inv[c]), hi = __ldcg(&ctx_dmax[c]);
+    PardSegConst* K = a.ktab + q;
+    const long long A = __ldcg(&K->A), d = __ldcg(&K->d);
+    uint32_t narrow = __ldcg(&K->narrow);
+    if (RANGES) {                                        /* as in ctx_constants */
+      const long long A_rel = (narrow & kSegHighFirst) ? (long long)hi - A : A - (long long)lo, lim = 1ll << 29;
+      const bool fits = __ldcg(&K->d_magic) != 0 && d < (1ll << 31) && A_rel > -lim && A_rel < lim && !(narrow & kSegNoStage);
+      narrow = (narrow & ~kSegNarrow) | (fits ? kSegNarrow : 0u);
+      K->A_rel = A_rel;
+      K->narrow = narrow;
+    }
+    if (a.win_hist) {
+      uint32_t w = 1;
+      if (!(narrow & kSegNoStage) && lo <= hi) {
+        const long long X = (long long)hi - A;
+        const unsigned long long nb = X < 0 ? 0ull : (unsigned long long)X / (unsigned long long)d + 1;
+        if (nb >= 4096) s_scan = 1;                      /* kWinMaxPerSeg: too many windows for a table */
+        else w = (uint32_t)nb + 1;
+      }
+      s_w[q] = w;
+    }
+  }
+  if (!a.win_hist) return;
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t total = 0;
+    bool scan = s_scan != 0;
+    for (uint32_t q = 0; q < n_seg; ++q) {
+      uint32_t w = s_w[q];
+      if (total + w > kHistCap) { scan = true; w = 1; }
+      a.win_off[q] = total;
+      a.win_cnt[q] = w;
+      total += w;
+    }
+    hdr->win_total = total;
+    if (scan) hdr->use_scan = 1;
+  }
+}
+
+/* Constants of all queues, a block per ctx, with a launch of their own: calls with many queues, whose
+ * blocks would hold up the prepass, and calls without requests. */
+__global__ void __launch_bounds__(kConstThreads)
+k_seg_const(const __grid_constant__ ConstArgs a, const unsigned long long* __restrict__ ctx_dmin_inv,
+            const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr) {
+  pdl_wait();
+  __shared__ CtxScratch scratch;
+  if (ctx_constants(a.pipes, a.n_pipelines, a.st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
+                    a.ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch))
+    set_status(hdr, PARD_EDATA);
+  if (a.with_key_width && last_block_done(&hdr->seg_done)) finish_constants<false>(a, ctx_dmin_inv, ctx_dmax, hdr);
+}
+
 /* ------------------------------------------------------------------------ */
 /* prepass: one coalesced 16-byte read per request                           */
 /* ------------------------------------------------------------------------ */
@@ -140,12 +268,31 @@ k_clear(uint4* __restrict__ p, unsigned long long n16) {
  * directly.  Bound by the read of the requests: four in flight per thread at 48 registers keep
  * five blocks on a multiprocessor. */
 constexpr int kPreUn = 4;
+
+__device__ __noinline__ void const_block(const ConstArgs& a, uint32_t c, PlanHeader* hdr) {
+  __shared__ CtxScratch scratch;
+  if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, 0, 0, a.ktab + (size_t)c * a.st.stage_stride, scratch)) set_status(hdr, PARD_EDATA);
+}
+__device__ __noinline__ void const_tail(const ConstArgs& a, const unsigned long long* ctx_dmin_inv, const unsigned long long* ctx_dmax,
+                                        PlanHeader* hdr) {
+  if (last_block_done(&hdr->seg_done)) finish_constants<true>(a, ctx_dmin_inv, ctx_dmax, hdr);
+}
+
+/* const_blocks: so many further blocks, the first ones of the grid, work out the queues' constants
+ * meanwhile -- a chain of dependent loads that needs no deadline --, and the block that finishes last
+ * completes them (one launch and its 8 us less for every call of up to 1,024 queues). */
 template <bool TABLE>
 __global__ void __launch_bounds__(256, 5)
 k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
           unsigned long long* __restrict__ ctx_dmin_inv, unsigned long long* __restrict__ ctx_dmax,
-          PlanHeader* hdr) {
+          PlanHeader* hdr, uint32_t const_blocks, const __grid_constant__ ConstArgs ca) {
   pdl_wait();
+  if (blockIdx.x < const_blocks) {
+    const_block(ca, blockIdx.x, hdr);
+    const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
+    return;
+  }
+  const uint32_t my_block = blockIdx.x - const_blocks, blocks = gridDim.x - const_blocks;
   extern __shared__ uint32_t s_range[];          /* TABLE: [n_ctx] complement of the smallest offset, [n_ctx] largest + 1, 0 = none */
   constexpr uint32_t kNone = 0xffffffffu;
   const uint32_t lane = threadIdx.x & 31;
@@ -192,7 +339,7 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     lmax = 0;
   };
   const uint64_t chunk = (uint64_t)blockDim.x * kPreUn;
-  for (uint64_t base = (uint64_t)blockIdx.x * chunk; base < n; base += (uint64_t)gridDim.x * chunk) {
+  for (uint64_t base = (uint64_t)my_block * chunk; base < n; base += (uint64_t)blocks * chunk) {
     uint4 r[kPreUn];
     const uint64_t first = base + (threadIdx.x >> 5) * (32 * kPreUn);   /* a warp's requests lie side by side */
 #pragma unroll
@@ -299,17 +446,19 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       if (__ldcg(&ctx_dmax[c]) < hi) atomicMax(&ctx_dmax[c], hi);
     }
   }
+  if (const_blocks) const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
 constexpr uint32_t kPreTableCtx = 4096;          /* 32 KB of table: five blocks still fit a multiprocessor */
 void launch_prepass(const uint4* req, uint32_t n, uint32_t n_ctx, uint32_t S, unsigned long long* ctx_dmin_inv,
-                    unsigned long long* ctx_dmax, PlanHeader* hdr, int sms, cudaStream_t stream) {
+                    unsigned long long* ctx_dmax, PlanHeader* hdr, uint32_t const_blocks, const ConstArgs& ca, int sms,
+                    cudaStream_t stream) {
   const uint32_t grid = std::min<uint32_t>((n + 256 * kPreUn - 1) / (256 * kPreUn), (uint32_t)sms * 5);
   /* the table pays once a block has more requests than the table has entries to clear and hand over */
   if (n_ctx > 1 && n_ctx <= kPreTableCtx && n / grid >= 2 * n_ctx)
-    launch_pdl(k_prepass<true>, grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr);
+    launch_pdl(k_prepass<true>, const_blocks + grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
   else
-    launch_pdl(k_prepass<false>, grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr);
+    launch_pdl(k_prepass<false>, const_blocks + grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
 }
 
 __global__ void k_ctx_span(const unsigned long long* __restrict__ ctx_dmin_inv,
@@ -326,116 +475,10 @@ __global__ void k_ctx_span(const unsigned long long* __restrict__ ctx_dmin_inv,
   if ((threadIdx.x & 31) == 0 && span) atomicMax(&hdr->span_max, span);
 }
 
-/* Width of the sort key, once the widest deadline span is known, and the part of it that the
- * passes have to sort.  key_sbits: the queue-id bits to sort (all of them, or the stage bits only
- * when the passes stay inside the contexts' ranges).  The deadline field below them needs no pass
- * when every queue's requests stand in the order it asks for: in arrival order the index alone
- * orders a queue, and in budget order (low budget first everywhere) requests whose deadlines never
- * step back along the array, or along every ctx of an array grouped by ctx, are ordered as they
- * come.  (2^24 such requests in 256 contexts: one pass instead of four, 696 -> 408 us for the call.) */
-__device__ __forceinline__ void set_key_width(PlanHeader* hdr, unsigned long long span, uint32_t sbits, uint32_t ibits,
-                                              uint32_t key_sbits, uint32_t arrival_order, bool priority) {
-  uint32_t dbits = bit_width64(span);
-  if (arrival_order && sbits + dbits + ibits > 64) {    /* no room: the rule reads the deadlines from the requests */
-    dbits = 0;
-    hdr->lookup = 1;
-  }
-  const bool in_order = arrival_order || (!priority && !(hdr->time_steps_back && hdr->pair_steps_back));
-  const uint32_t skip = in_order ? dbits : 0u;
-  hdr->span_max = span;
-  hdr->dbits = dbits;
-  hdr->pshift = skip;
-  hdr->keybits = key_sbits + dbits - skip;
-  hdr->npass = (key_sbits + dbits - skip + 7) / 8;
-  if (sbits + dbits + ibits > 64) {
-    hdr->npass = 0;
-    hdr->wide = 1;
-    set_status(hdr, PARD_ERANGE);
-  }
-}
-
 __global__ void k_key_width(uint32_t sbits, uint32_t ibits, PlanHeader* hdr, uint32_t arrival_order, uint32_t key_sbits,
                             uint32_t priority) {
   pdl_wait();
   set_key_width(hdr, hdr->span_max, sbits, ibits, key_sbits, arrival_order, priority != 0);
-}
-
-/* Per-segment constants; one block per ctx. */
-__global__ void __launch_bounds__(kConstThreads)
-k_seg_const(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
-            const __grid_constant__ pard_queue_state_t st, uint32_t n_ctx,
-            const unsigned long long* __restrict__ ctx_dmin_inv,
-            const unsigned long long* __restrict__ ctx_dmax, PardSegConst* __restrict__ ktab,
-            PlanHeader* hdr, uint32_t sbits, uint32_t ibits, uint32_t with_key_width, uint32_t arrival_order,
-            uint32_t win_hist, uint32_t force_scan, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
-            uint32_t key_sbits) {
-  pdl_wait();
-  __shared__ CtxScratch scratch;
-  const uint32_t S = (uint32_t)st.stage_stride;
-  const uint32_t lane = threadIdx.x & 31;
-  if (ctx_constants(pipes, n_pipelines, st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
-                    ktab + (size_t)blockIdx.x * S, scratch))
-    set_status(hdr, PARD_EDATA);
-  /* With few queues the block that finishes last also finds the widest deadline span and with
-   * it the width of the sort key (the work of k_ctx_span and k_key_width, without their launches). */
-  if (!with_key_width) return;
-  if (!last_block_done(&hdr->seg_done)) return;
-  __shared__ unsigned long long s_span[4];
-  unsigned long long span = 0;
-  for (uint32_t c = threadIdx.x; c < n_ctx; c += blockDim.x) {
-    const unsigned long long lo = ~ctx_dmin_inv[c], hi = ctx_dmax[c];
-    if (lo <= hi && hi - lo > span) span = hi - lo;
-  }
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long a = __shfl_xor_sync(0xffffffffu, span, o);
-    span = a > span ? a : span;
-  }
-  if (lane == 0) s_span[threadIdx.x >> 5] = span;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (uint32_t w = 1; w < blockDim.x / 32; ++w) span = s_span[w] > span ? s_span[w] : span;
-    set_key_width(hdr, span, sbits, ibits, key_sbits, arrival_order, st.d_priority != nullptr);
-  }
-  /* Few queues: their batch-window tables are COUNTED while the requests are packed (k_pack)
-   * instead of being searched for in the sorted elements afterwards.  That needs the tables'
-   * extents before any request has been looked at: a queue can have no window beyond that of its
-   * ctx's latest deadline.  Entry 0 of a queue counts its requests with deadline < A, entry b + 1
-   * those of window b; every queue has at least entry 0, so that the counts also give the queues'
-   * lengths. */
-  if (win_hist) {                                        /* still the last block, all its threads */
-    __shared__ uint32_t s_w[kHistSegs];
-    __shared__ uint32_t s_scan;
-    const uint32_t n_seg = n_ctx * S;
-    if (threadIdx.x == 0) s_scan = force_scan;
-    __syncthreads();
-    for (uint32_t q = threadIdx.x; q < n_seg; q += blockDim.x) {   /* every queue's number of entries, side by side */
-      const PardSegConst K = ktab[q];
-      const uint32_t c = q / S;
-      uint32_t w = 1;
-      const unsigned long long lo = ~ctx_dmin_inv[c], hi = ctx_dmax[c];
-      if (!(K.narrow & kSegNoStage) && lo <= hi) {
-        const long long X = (long long)hi - K.A;
-        const unsigned long long nb = X < 0 ? 0ull : (unsigned long long)X / (unsigned long long)K.d + 1;
-        if (nb >= 4096) s_scan = 1;                      /* kWinMaxPerSeg: too many windows for a table */
-        else w = (uint32_t)nb + 1;
-      }
-      s_w[q] = w;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t total = 0;
-      bool scan = s_scan != 0;
-      for (uint32_t q = 0; q < n_seg; ++q) {
-        uint32_t w = s_w[q];
-        if (total + w > kHistCap) { scan = true; w = 1; }
-        win_off[q] = total;
-        win_cnt[q] = w;
-        total += w;
-      }
-      hdr->win_total = total;
-      if (scan) hdr->use_scan = 1;
-    }
-  }
 }
 
 /* request -> sort element; digit histograms of every pass */
@@ -588,6 +631,162 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
 }
 
 /* ------------------------------------------------------------------------ */
+/* window tables: the decision pass without a scan                           */
+/* ------------------------------------------------------------------------ */
+/* Inside one queue the threshold u is a step function of the deadline: every
+ * request whose deadline falls into the same batch window
+ *     b = floor((D - A) / d)
+ * has u = cap * (b + 1) (requests with D < A have u = 0).  The running minimum
+ * of u_t - t that fixes the admitted position therefore only changes at the
+ * window boundaries: with P[b] = number of requests of the queue whose window
+ * is below b, the minimum over a complete window b is u(b) - (P[b+1] - 1), and
+ *     E[b] = minimum over all complete runs before window b
+ * is a prefix minimum over at most a few thousand windows per queue.  A request
+ * at queue position r in window b then has
+ *     min_{t<r}(u_t - t) = min(E[b], u(b) - (r - 1) if r > P[b])
+ * with no reference to any other request.  P comes from a search in the sorted
+ * elements (one warp per window), E and the raw-mode kept counts Kp from a
+ * per-queue prefix pass over the windows.  Queues with more than kWinMaxPerSeg
+ * windows, or more windows in total than the table holds, make the call fall
+ * back to the scan kernels (same results). */
+struct __align__(16) WinEntry {
+  uint32_t P;      /* requests of the queue in earlier windows (or expired)       */
+  int32_t E;       /* min of u_t - t over those requests, kWinInf if there is none */
+  uint32_t Kp;     /* raw mode: kept requests among them                          */
+  uint32_t pad;
+};
+constexpr uint32_t kWinMaxPerSeg = 4096;
+/* window of a non-negative X = D - A */
+__device__ __forceinline__ unsigned long long win_of(unsigned long long X, const PardSegConst& K) {
+  if ((X >> 32) == 0 && K.d_magic) return div_magic32((uint32_t)X, K.d_magic);
+  return X / (unsigned long long)K.d;
+}
+
+/* E and Kp of the table of one queue (cnt >= 1 entries): the warp runs over the queue's windows, 32 at a
+ * time. */
+__device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __restrict__ tab, uint32_t cnt, uint32_t lane, uint32_t raw) {
+  const uint32_t P0 = __ldcg(&tab[0].P);
+  int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;     /* the expired run: u = 0 */
+  uint32_t k_carry = 0;
+  if (lane == 0) { tab[0].E = e_carry; tab[0].Kp = 0; }
+  for (uint32_t b0 = 0; b0 + 1 < cnt; b0 += 32) {              /* windows b0..b0+31 -> entries b0+1.. */
+    const uint32_t b = b0 + lane;
+    int32_t val = kWinInf;
+    uint32_t kept = 0;
+    if (b + 1 < cnt) {
+      const uint32_t p = __ldcg(&tab[b].P), q = __ldcg(&tab[b + 1].P);
+      if (q > p) {
+        const uint32_t u = win_u(b, cap);
+        val = (int32_t)u - (int32_t)(q - 1);
+        const uint32_t top = u < q ? u : q;
+        kept = top > p ? top - p : 0;
+      }
+    }
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t v2 = __shfl_up_sync(0xffffffffu, val, o);
+      const uint32_t k2 = __shfl_up_sync(0xffffffffu, kept, o);
+      if (lane >= (uint32_t)o) { val = min(val, v2); kept += k2; }
+    }
+    const int32_t e_inc = min(e_carry, val);
+    const uint32_t k_inc = k_carry + kept;
+    if (b + 1 < cnt) { tab[b + 1].E = e_inc; tab[b + 1].Kp = k_inc; }
+    e_carry = __shfl_sync(0xffffffffu, e_inc, 31);
+    k_carry = __shfl_sync(0xffffffffu, k_inc, 31);
+  }
+  /* With the table complete the queue's number of kept requests is known before any request has
+   * been decided: the last entry closes the queue (P = its length n), the running Kp counts the
+   * kept requests under raw positions, and the running E is the minimum of u_t - t over the whole
+   * queue, so that the admitted count behind the last request is n - 1 + min(E, 1). */
+  const uint32_t n_q = __ldcg(&tab[cnt - 1].P);
+  return n_q == 0 ? 0u : (raw ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1)));
+}
+
+/* The window tables of a call with few queues, from the counts k_pack took: P is the running sum
+ * of a queue's counts, E and Kp follow as in the searched tables, and the queues' first positions
+ * are the running sum of their lengths.  By one block, a warp per queue: a block of the first sort
+ * kernel's launch, beside the sort (the counts do not depend on the order of the elements; as a launch
+ * of its own it held the sort up by 6 us). */
+struct WinCountArgs {
+  uint32_t on, n_seg, raw, sbits;
+  const PardSegConst* ktab;
+  const uint32_t* whist;
+  const uint32_t* win_off;
+  const uint32_t* win_cnt;
+  WinEntry* wtab;
+  uint32_t* seg_off;
+  uint32_t* out_seg_off;
+  uint32_t* seg_kept;
+  uint32_t* out_seg_kept;
+  uint32_t* kept_base;
+  unsigned long long* out_n_kept;
+  const uint32_t* hist;
+};
+__device__ __noinline__ void win_from_counts(PlanHeader* hdr, const WinCountArgs& a) {
+  if (hdr->wide || hdr->aborted) return;
+  const uint32_t n_seg = a.n_seg;
+  __shared__ uint32_t s_len[kHistSegs], s_kept[kHistSegs];
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  /* entry 0 left uncounted by k_pack (same condition there): the queue's length, from the last
+   * pass's digit counts, minus its other entries */
+  const uint32_t npass = hdr->npass;
+  const uint32_t top_bits = npass ? hdr->keybits - 8 * (npass - 1) : 0;
+  const bool derive = npass > 0 && a.sbits <= top_bits;
+  for (uint32_t q = warp; q < n_seg; q += blockDim.x / 32) {
+    const uint32_t off = a.win_off[q], cnt = a.win_cnt[q];
+    uint32_t entry0 = 0;
+    if (derive) {
+      const uint32_t* h = a.hist + (npass - 1) * kBins;
+      const uint32_t d0 = min(q << (top_bits - a.sbits), (uint32_t)kBins), d1 = min((q + 1) << (top_bits - a.sbits), (uint32_t)kBins);
+      uint32_t len = 0, others = 0;
+      for (uint32_t d = d0 + lane; d < d1; d += 32) len += h[d];
+      for (uint32_t b = 1 + lane; b < cnt; b += 32) others += a.whist[off + b];
+      for (int o = 16; o; o >>= 1) {
+        len += __shfl_xor_sync(0xffffffffu, len, o);
+        others += __shfl_xor_sync(0xffffffffu, others, o);
+      }
+      entry0 = len - others;
+    }
+    uint32_t run = 0;
+    for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
+      const uint32_t b = b0 + lane;
+      uint32_t x = b < cnt ? a.whist[off + b] : 0u;
+      if (derive && b == 0) x = entry0;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+      }
+      if (b < cnt) a.wtab[off + b].P = run + x;        /* requests of the queue up to and including entry b's */
+      run += __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) s_len[q] = run;
+    __threadfence_block();
+    __syncwarp();
+    /* P as the decision reads it: entry b = requests in windows below b, i.e. the sum up to entry b */
+    const uint32_t kept = cnt ? win_prefix_warp(a.ktab[q].cap, a.wtab + off, cnt, lane, a.raw) : 0u;
+    if (lane == 0) s_kept[q] = kept;      /* the queue's kept count, known before the sort */
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const bool scan = hdr->use_scan != 0;                /* then the scan path counts and packs */
+    uint32_t first = 0, kept = 0;
+    for (uint32_t q = 0; q < n_seg; ++q) {
+      a.seg_off[q] = first;
+      if (a.out_seg_off) a.out_seg_off[q] = first;
+      first += s_len[q];
+      if (!scan) {
+        a.kept_base[q] = kept;
+        a.seg_kept[q] = s_kept[q];
+        if (a.out_seg_kept) a.out_seg_kept[q] = s_kept[q];
+        kept += s_kept[q];
+      }
+    }
+    a.seg_off[n_seg] = first;
+    if (a.out_seg_off) a.out_seg_off[n_seg] = first;
+    if (!scan && a.out_n_kept) *a.out_n_kept = kept;
+  }
+}
+
+/* ------------------------------------------------------------------------ */
 /* one LSD radix pass (8 bits), stable, tile prefixes by decoupled look-back */
 /* ------------------------------------------------------------------------ */
 /* Tile = kSortTile elements; every warp owns a run of consecutive elements
@@ -606,10 +805,10 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
  *   5. the buffer is written out, run by run, to the digit's global range.
  * Large tiles keep the number of tiles in flight, and with it the depth of the
  * look-back, small. */
-/* The grid (resident as a whole) meets: every block's writes before are visible to every block
+/* The grid's `members` blocks (resident as a whole) meet: every block's writes before are visible to every block
  * after.  `bar` counts arrivals from zero.  Bounded: about half a second, then PARD_ETIMEOUT and false
  * in every block. */
-__device__ bool grid_barrier(PlanHeader* hdr, uint32_t* bar, bool withhold = false) {
+__device__ bool grid_barrier(PlanHeader* hdr, uint32_t* bar, uint32_t members, bool withhold = false) {
   __shared__ uint32_t s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -617,7 +816,7 @@ __device__ bool grid_barrier(PlanHeader* hdr, uint32_t* bar, bool withhold = fal
     if (!withhold) atomicAdd(bar, 1u);      /* (testing aid: a block that never arrives) */
     uint32_t spins = 0;
     bool ok = true;
-    while (ld_relaxed(bar) < gridDim.x) {     /* up to about half a second: other work may hold multiprocessors for a while */
+    while (ld_relaxed(bar) < members) {     /* up to about half a second: other work may hold multiprocessors for a while */
       if (++spins > 8 * kSpinLimit || hdr->aborted) { ok = false; break; }
       __nanosleep(200);
     }
@@ -920,15 +1119,24 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   }
 }
 
+/* (a call: inlined into the loop over the passes it would spill) */
+template <bool CTX>
+__device__ __noinline__ bool sort_tiles_resident(SortSmem& S, uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a,
+                                                 unsigned long long* buf_b, const uint32_t* hist, uint32_t* lookback,
+                                                 uint32_t* lookback_next, uint32_t n, uint32_t ibits, uint32_t stall, const CtxTiles& ct) {
+  return sort_tiles<true, CTX>(S, pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits, stall, ct);
+}
+
 /* One pass, one tile per block. */
 template <bool CTX>
 __global__ void __launch_bounds__(kSortThreads, 2)
 k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf_a,
             unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ hist,
             uint32_t* __restrict__ lookback, uint32_t* __restrict__ lookback_next, uint32_t n,
-            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct) {
+            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct, const __grid_constant__ WinCountArgs wc) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
   if (pass >= hdr->npass || hdr->aborted || sort_is_local(hdr, local_candidate)) return;
   sort_tiles<false, CTX>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
                          stall, ct);
@@ -944,16 +1152,18 @@ template <bool CTX>
 __global__ void __launch_bounds__(kSortThreads, 2)
 k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned long long* buf_b,
             const uint32_t* __restrict__ hist, uint32_t* lookback, size_t lb_words, uint32_t n,
-            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct) {
+            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct, const __grid_constant__ WinCountArgs wc) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
+  const uint32_t members = gridDim.x - (wc.on ? 1u : 0u);
   if (hdr->aborted || sort_is_local(hdr, local_candidate)) return;
   const uint32_t npass = hdr->npass;
   for (uint32_t p = pass; p < npass; ++p) {
-    if (!sort_tiles<true, CTX>(*reinterpret_cast<SortSmem*>(smem_raw), p, hdr, buf_a, buf_b, hist, lookback + (p & 1) * lb_words,
+    if (!sort_tiles_resident<CTX>(*reinterpret_cast<SortSmem*>(smem_raw), p, hdr, buf_a, buf_b, hist, lookback + (p & 1) * lb_words,
                                lookback + ((p + 1) & 1) * lb_words, n, ibits, p == 0 ? stall : 0u, ct))
       return;
-    if (p + 1 < npass && !grid_barrier(hdr, &hdr->sort_bar[p])) return;
+    if (p + 1 < npass && !grid_barrier(hdr, &hdr->sort_bar[p], members)) return;
   }
 }
 
@@ -1652,77 +1862,6 @@ k_kept_scan(const uint32_t* __restrict__ seg_kept, uint32_t n_seg, uint32_t* __r
   kept_scan_block<1024>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
 }
 
-/* ------------------------------------------------------------------------ */
-/* window tables: the decision pass without a scan                           */
-/* ------------------------------------------------------------------------ */
-/* Inside one queue the threshold u is a step function of the deadline: every
- * request whose deadline falls into the same batch window
- *     b = floor((D - A) / d)
- * has u = cap * (b + 1) (requests with D < A have u = 0).  The running minimum
- * of u_t - t that fixes the admitted position therefore only changes at the
- * window boundaries: with P[b] = number of requests of the queue whose window
- * is below b, the minimum over a complete window b is u(b) - (P[b+1] - 1), and
- *     E[b] = minimum over all complete runs before window b
- * is a prefix minimum over at most a few thousand windows per queue.  A request
- * at queue position r in window b then has
- *     min_{t<r}(u_t - t) = min(E[b], u(b) - (r - 1) if r > P[b])
- * with no reference to any other request.  P comes from a search in the sorted
- * elements (one warp per window), E and the raw-mode kept counts Kp from a
- * per-queue prefix pass over the windows.  Queues with more than kWinMaxPerSeg
- * windows, or more windows in total than the table holds, make the call fall
- * back to the scan kernels (same results). */
-struct __align__(16) WinEntry {
-  uint32_t P;      /* requests of the queue in earlier windows (or expired)       */
-  int32_t E;       /* min of u_t - t over those requests, kWinInf if there is none */
-  uint32_t Kp;     /* raw mode: kept requests among them                          */
-  uint32_t pad;
-};
-constexpr uint32_t kWinMaxPerSeg = 4096;
-/* window of a non-negative X = D - A */
-__device__ __forceinline__ unsigned long long win_of(unsigned long long X, const PardSegConst& K) {
-  if ((X >> 32) == 0 && K.d_magic) return div_magic32((uint32_t)X, K.d_magic);
-  return X / (unsigned long long)K.d;
-}
-
-/* E and Kp of the table of one queue (cnt >= 1 entries): the warp runs over the queue's windows, 32 at a
- * time. */
-__device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __restrict__ tab, uint32_t cnt, uint32_t lane, uint32_t raw) {
-  const uint32_t P0 = __ldcg(&tab[0].P);
-  int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;     /* the expired run: u = 0 */
-  uint32_t k_carry = 0;
-  if (lane == 0) { tab[0].E = e_carry; tab[0].Kp = 0; }
-  for (uint32_t b0 = 0; b0 + 1 < cnt; b0 += 32) {              /* windows b0..b0+31 -> entries b0+1.. */
-    const uint32_t b = b0 + lane;
-    int32_t val = kWinInf;
-    uint32_t kept = 0;
-    if (b + 1 < cnt) {
-      const uint32_t p = __ldcg(&tab[b].P), q = __ldcg(&tab[b + 1].P);
-      if (q > p) {
-        const uint32_t u = win_u(b, cap);
-        val = (int32_t)u - (int32_t)(q - 1);
-        const uint32_t top = u < q ? u : q;
-        kept = top > p ? top - p : 0;
-      }
-    }
-    for (int o = 1; o < 32; o <<= 1) {
-      const int32_t v2 = __shfl_up_sync(0xffffffffu, val, o);
-      const uint32_t k2 = __shfl_up_sync(0xffffffffu, kept, o);
-      if (lane >= (uint32_t)o) { val = min(val, v2); kept += k2; }
-    }
-    const int32_t e_inc = min(e_carry, val);
-    const uint32_t k_inc = k_carry + kept;
-    if (b + 1 < cnt) { tab[b + 1].E = e_inc; tab[b + 1].Kp = k_inc; }
-    e_carry = __shfl_sync(0xffffffffu, e_inc, 31);
-    k_carry = __shfl_sync(0xffffffffu, k_inc, 31);
-  }
-  /* With the table complete the queue's number of kept requests is known before any request has
-   * been decided: the last entry closes the queue (P = its length n), the running Kp counts the
-   * kept requests under raw positions, and the running E is the minimum of u_t - t over the whole
-   * queue, so that the admitted count behind the last request is n - 1 + min(E, 1). */
-  const uint32_t n_q = __ldcg(&tab[cnt - 1].P);
-  return n_q == 0 ? 0u : (raw ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1)));
-}
-
 /* Queue boundaries, window tables and output offsets of kWinQueues queues per block, from the sorted
  * elements:
  *   - every queue's first position: read off the last pass's digit counts when the queue id lies inside
@@ -1996,81 +2135,6 @@ k_windows_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, co
   kept_scan_block<kWinThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
 }
 
-/* The window tables of a call with few queues, from the counts k_pack took: P is the running sum
- * of a queue's counts, E and Kp follow as in the searched tables, and the queues' first positions
- * are the running sum of their lengths.  One block; a warp per queue.  Runs before the sort: the
- * counts do not depend on the order of the elements. */
-__global__ void __launch_bounds__(1024)
-k_win_from_counts(PlanHeader* hdr, uint32_t n_seg, const PardSegConst* __restrict__ ktab,
-                  const uint32_t* __restrict__ whist, const uint32_t* __restrict__ win_off,
-                  const uint32_t* __restrict__ win_cnt, WinEntry* __restrict__ wtab,
-                  uint32_t* __restrict__ seg_off, uint32_t* __restrict__ out_seg_off, uint32_t raw,
-                  uint32_t* __restrict__ seg_kept, uint32_t* __restrict__ out_seg_kept,
-                  uint32_t* __restrict__ kept_base, unsigned long long* __restrict__ out_n_kept,
-                  const uint32_t* __restrict__ hist, uint32_t sbits) {
-  pdl_wait();
-  __shared__ uint32_t s_len[kHistSegs], s_kept[kHistSegs];
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  /* entry 0 left uncounted by k_pack (same condition there): the queue's length, from the last
-   * pass's digit counts, minus its other entries */
-  const uint32_t npass = hdr->npass;
-  const uint32_t top_bits = npass ? hdr->keybits - 8 * (npass - 1) : 0;
-  const bool derive = npass > 0 && sbits <= top_bits;
-  for (uint32_t q = warp; q < n_seg; q += blockDim.x / 32) {
-    const uint32_t off = win_off[q], cnt = win_cnt[q];
-    uint32_t entry0 = 0;
-    if (derive) {
-      const uint32_t* h = hist + (npass - 1) * kBins;
-      const uint32_t d0 = min(q << (top_bits - sbits), (uint32_t)kBins), d1 = min((q + 1) << (top_bits - sbits), (uint32_t)kBins);
-      uint32_t len = 0, others = 0;
-      for (uint32_t d = d0 + lane; d < d1; d += 32) len += h[d];
-      for (uint32_t b = 1 + lane; b < cnt; b += 32) others += whist[off + b];
-      for (int o = 16; o; o >>= 1) {
-        len += __shfl_xor_sync(0xffffffffu, len, o);
-        others += __shfl_xor_sync(0xffffffffu, others, o);
-      }
-      entry0 = len - others;
-    }
-    uint32_t run = 0;
-    for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
-      const uint32_t b = b0 + lane;
-      uint32_t x = b < cnt ? whist[off + b] : 0u;
-      if (derive && b == 0) x = entry0;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= (uint32_t)o) x += y;
-      }
-      if (b < cnt) wtab[off + b].P = run + x;        /* requests of the queue up to and including entry b's */
-      run += __shfl_sync(0xffffffffu, x, 31);
-    }
-    if (lane == 0) s_len[q] = run;
-    __threadfence_block();
-    __syncwarp();
-    /* P as the decision reads it: entry b = requests in windows below b, i.e. the sum up to entry b */
-    const uint32_t kept = cnt ? win_prefix_warp(ktab[q].cap, wtab + off, cnt, lane, raw) : 0u;
-    if (lane == 0) s_kept[q] = kept;      /* the queue's kept count, known before the sort */
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const bool scan = hdr->use_scan != 0;                /* then the scan path counts and packs */
-    uint32_t first = 0, kept = 0;
-    for (uint32_t q = 0; q < n_seg; ++q) {
-      seg_off[q] = first;
-      if (out_seg_off) out_seg_off[q] = first;
-      first += s_len[q];
-      if (!scan) {
-        kept_base[q] = kept;
-        seg_kept[q] = s_kept[q];
-        if (out_seg_kept) out_seg_kept[q] = s_kept[q];
-        kept += s_kept[q];
-      }
-    }
-    seg_off[n_seg] = first;
-    if (out_seg_off) out_seg_off[n_seg] = first;
-    if (!scan && out_n_kept) *out_n_kept = kept;
-  }
-}
-
 /* Decision pass from the window tables: every request on its own.  HF: some
  * queue may be served high budget first (the caller gave priorities). */
 template <bool RAW, bool HF>
@@ -2255,13 +2319,13 @@ k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
   if (hdr->wide || hdr->aborted || !hdr->use_scan) return;
   const uint32_t n_tiles = (n + kDecTile - 1) / kDecTile;
   tile_agg_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, tile_agg);
-  if (!grid_barrier(hdr, &hdr->bar[0], stall && blockIdx.x == 0)) return;
+  if (!grid_barrier(hdr, &hdr->bar[0], gridDim.x, stall && blockIdx.x == 0)) return;
   if (blockIdx.x == 0) tile_scan_block<RAW, kDecThreads>(tile_agg, n_tiles, carry);
-  if (!grid_barrier(hdr, &hdr->bar[1])) return;
+  if (!grid_barrier(hdr, &hdr->bar[1], gridDim.x)) return;
   decide_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, carry, out_keep, out_est, out_perm, kept_tmp, seg_kept);
-  if (!grid_barrier(hdr, &hdr->bar[2])) return;
+  if (!grid_barrier(hdr, &hdr->bar[2], gridDim.x)) return;
   if (blockIdx.x == 0) kept_scan_block<kDecThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
-  if (!grid_barrier(hdr, &hdr->bar[3])) return;
+  if (!grid_barrier(hdr, &hdr->bar[3], gridDim.x)) return;
   if (out_kept_idx) kept_move_jobs(kept_tmp, seg_off, seg_kept, kept_base, chunk_base, n_seg, out_kept_idx);
 }
 
@@ -2618,6 +2682,13 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                (unsigned long long*)out->d_n_kept);
   };
 
+  auto const_args = [&]() {
+    ConstArgs ca = {};
+    ca.pipes = pipe_table; ca.st = *state; ca.n_pipelines = n_pipelines; ca.n_ctx = n_ctx; ca.ktab = ktab;
+    ca.sbits = sbits; ca.ibits = ibits; ca.key_sbits = sbits; ca.win_off = win_off; ca.win_cnt = win_cnt;
+    return ca;
+  };
+
   /* ---- keys wider than one sort element: see k_wide_reset.  Run only when a finished call has
    * reported that width (the host cannot know the deadline span beforehand), hence not for
    * PARD_MODE_NOWAIT, whose caller gets PARD_ERANGE from pard_plan_status as before. ---- */
@@ -2632,11 +2703,11 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
       launch_pdl(k_clear, (uint32_t)std::min<unsigned long long>((n16 + 255) / 256, (unsigned long long)sms * 4), 256, 0,
                  stream, (uint4*)(ws + L.hdr), n16);
     }
-    launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, sms, stream);
+    ConstArgs ca = const_args();
+    launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, 0u, ca, sms, stream);
     launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
     launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, 0u, sbits, 1u);
-    launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
-               hdr, sbits, ibits, 0u, 0u, 0u, 0u, win_off, win_cnt, sbits);
+    launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
     const uint32_t cw = 64 - ibits;                         /* key bits per super-pass */
     const uint32_t supers = (sbits + 60 + cw - 1) / cw;     /* for the widest legal span; chunks beyond the key are empty */
     const uint32_t chunk_passes = std::min<uint32_t>(kMaxPasses, (cw + 7) / 8);
@@ -2648,7 +2719,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  sp, (const PlanHeader*)hdr, (const uint32_t*)order, buf_a, hist);
       for (uint32_t p = 0; p < chunk_passes; ++p)
         launch_pdl(k_sort_pass<false>, L.sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
-                   lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, CtxTiles{});
+                   lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, CtxTiles{}, WinCountArgs{});
       launch_pdl(k_wide_chase, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a, buf_b, n32,
                  ibits, sp, (const uint32_t*)order);
       launch_pdl(k_wide_keep, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a,
@@ -2703,9 +2774,6 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                stream, (uint4*)(ws + L.hdr), n16);
   }
 
-  mark();
-  if (n > 0) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, sms, stream);
-  mark();
   /* Requests grouped by ctx (the caller's word) with contexts of more than a tile on average: the
    * radix passes stay inside every ctx's range -- tiles cut at ctx boundaries, digit counts per
    * ctx, look-back up to the ctx's first tile -- and sort the stage and deadline bits only; the
@@ -2714,17 +2782,23 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
   const uint32_t key_sbits = ctx_sort ? ceil_log2(S) : sbits;
   const CtxTiles ctx_tiles = {ctx_start, (const uint32_t*)(ws + L.tile_first), (const uint32_t*)(ws + L.hist_ctx), n_ctx};
-  const bool fold_width = L.n_seg <= kFoldSegs;          /* few queues: k_seg_const's last block finds the key width */
-  if (!fold_width) {
-    if (n > 0) launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
-    launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, arrival_order ? 1u : 0u, key_sbits, state->d_priority ? 1u : 0u);
-  }
   /* few queues, decided by the planner's own rule in budget order from the start of every queue:
    * the window tables are counted while the requests are packed */
   const bool win_hist = n > 0 && L.n_seg <= kHistSegs && !rule_walk && !state->d_priority && !local_cand && !ctx_sort;
-  launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, pipe_table, n_pipelines, *state, n_ctx, ctx_dmin, ctx_dmax, ktab,
-             hdr, sbits, ibits, fold_width ? 1u : 0u, arrival_order ? 1u : 0u, win_hist ? 1u : 0u,
-             (mode & PARD_MODE_SCAN) ? 1u : 0u, win_off, win_cnt, key_sbits);
+  ConstArgs ca = const_args();
+  ca.key_sbits = key_sbits;
+  ca.with_key_width = n_ctx <= kFoldCtx ? 1u : 0u;       /* few contexts: the last block to finish finds the key width */
+  ca.arrival_order = arrival_order ? 1u : 0u; ca.win_hist = win_hist ? 1u : 0u; ca.force_scan = (mode & PARD_MODE_SCAN) ? 1u : 0u;
+  const uint32_t const_blocks = n > 0 && L.n_seg <= kFoldSegs && ca.with_key_width ? n_ctx : 0u;
+  mark();
+  if (n > 0) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_blocks, ca, sms, stream);
+  mark();
+  if (!ca.with_key_width) {
+    if (n > 0) launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
+    launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, arrival_order ? 1u : 0u, key_sbits, state->d_priority ? 1u : 0u);
+  }
+  if (!const_blocks)
+    launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
   if ((local_cand && !local_sure) || ctx_sort)
     launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr);
   if (ctx_sort) launch_pdl(k_tile_table, 1, 1024, 0, stream, (const uint32_t*)ctx_start, n_ctx, (uint32_t*)(ws + L.tile_first));
@@ -2741,11 +2815,6 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     launch_pdl(win_hist ? k_pack<true> : k_pack<false>, grid, 256, 0, stream, req4, n32, n_ctx, S, ctx_dmin, ctx_dmax,
                state->d_priority, ibits, hdr, buf_a, hist, local_cand, (const PardSegConst*)ktab, (const uint32_t*)win_off,
                (const uint32_t*)win_cnt, whist);
-    if (win_hist)
-      launch_pdl(k_win_from_counts, 1, 1024, 0, stream, hdr, L.n_seg, (const PardSegConst*)ktab, (const uint32_t*)whist,
-                 (const uint32_t*)win_off, (const uint32_t*)win_cnt, wtab, seg_off, out->d_seg_offsets,
-                 (mode & PARD_MODE_RAW) ? 1u : 0u, seg_kept, out->d_seg_kept, kept_base, (unsigned long long*)out->d_n_kept,
-                 (const uint32_t*)hist, sbits);
   }
   /* passes with a launch of their own, then the rest in one kernel (see k_sort_rest) */
   const uint32_t sort_tiles = ctx_sort ? L.lb_tiles : L.sort_tiles;
@@ -2753,16 +2822,22 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   const uint32_t own_passes = sort_own_passes(sort_tiles, max_passes, sms, local_cand);
   const uint32_t rest_grid = std::min<uint32_t>(sort_tiles, 2u * (uint32_t)sms);
   const uint32_t stall = (mode & PARD_MODE_TEST_STALL) && !ctx_sort ? 1u : 0u;
+  WinCountArgs wc = {};
+  wc.on = win_hist ? 1u : 0u; wc.n_seg = L.n_seg; wc.raw = (mode & PARD_MODE_RAW) ? 1u : 0u; wc.sbits = sbits;
+  wc.ktab = ktab; wc.whist = whist; wc.win_off = win_off; wc.win_cnt = win_cnt; wc.wtab = wtab;
+  wc.seg_off = seg_off; wc.out_seg_off = out->d_seg_offsets; wc.seg_kept = seg_kept; wc.out_seg_kept = out->d_seg_kept;
+  wc.kept_base = kept_base; wc.out_n_kept = (unsigned long long*)out->d_n_kept; wc.hist = hist;
   for (uint32_t p = 0; p < (uint32_t)kMaxPasses; ++p) {
     mark();
     if (n == 0 || local_sure || p >= max_passes) continue;
     if (p < own_passes)
-      launch_pdl(ctx_sort ? k_sort_pass<true> : k_sort_pass<false>, sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
+      launch_pdl(ctx_sort ? k_sort_pass<true> : k_sort_pass<false>, sort_tiles + wc.on, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
                  buf_b, hist, lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, p == 0 ? stall : 0u,
-                 local_cand, ctx_tiles);
+                 local_cand, ctx_tiles, wc);
     else if (p == own_passes)
-      launch_pdl(ctx_sort ? k_sort_rest<true> : k_sort_rest<false>, rest_grid, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
-                 buf_b, hist, lookback, lb_words, n32, ibits, stall, local_cand, ctx_tiles);
+      launch_pdl(ctx_sort ? k_sort_rest<true> : k_sort_rest<false>, rest_grid + wc.on, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
+                 buf_b, hist, lookback, lb_words, n32, ibits, stall, local_cand, ctx_tiles, wc);
+    wc.on = 0;                                             /* the first launch has done it */
   }
   mark();
   if (win_hist) {
@@ -2824,12 +2899,13 @@ extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t sta
   int rc = pard_plan_workspace_bytes(n, n_ctx, stage_stride, &bytes);
   if (rc != PARD_OK) return rc;
   /* For the planner's own rule without priorities and without PARD_MODE_GROUPED.  One ctx of at
-   * most a sort tile: one kernel.  Else always clear and seg_const; with many queues also
-   * key_width (and, when n > 0, ctx_span); when n > 0: prepass, pack, the radix passes, decide_win
-   * and the scan path (one kernel that returns at once); with at most 64 queues the counted window
-   * tables (win_from_counts), else the queue boundaries and the searched ones (windows). */
+   * most a sort tile: one kernel.  Else always clear, and seg_const (few queues: inside the
+   * prepass); with many contexts also key_width (and, when n > 0, ctx_span); when n > 0: prepass, pack, the radix passes, decide_win
+   * and the scan path (one kernel that returns at once); with more than 64 queues also the
+   * queue boundaries and the searched window tables (windows). */
   const uint64_t n_seg = (uint64_t)n_ctx * (uint64_t)stage_stride;
-  const uint32_t width_kernels = n_seg <= kFoldSegs ? 0 : 1;   /* key_width (+ ctx_span when n > 0) */
+  const uint32_t width_kernels = n_ctx <= kFoldCtx ? 0 : 1;     /* key_width (+ ctx_span when n > 0) */
+  const uint32_t const_kernels = n > 0 && n_seg <= kFoldSegs ? 0 : 1;   /* seg_const, unless the prepass does its work */
   const bool local_cand = local_sort_candidate(n, n_ctx);
   const uint32_t local_kernels = local_cand ? 2 : 0;            /* ctx_ranges, sort_local */
   const Layout L = make_layout(n, n_ctx, stage_stride);
@@ -2842,7 +2918,7 @@ extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t sta
   const uint32_t passes = own + (own < L.max_passes ? 1 : 0);   /* and the kernel that does the rest */
   if (n_ctx == 1 && n > 0 && n <= (uint64_t)kSortTile) *launches = 1;
   else if (n == 0) *launches = 4 + width_kernels;               /* clear, (key_width,) seg_const, windows, kept_scan */
-  else *launches = 2 + 2 * width_kernels + 2 + local_kernels + passes + 2 + 1;
+  else *launches = 1 + const_kernels + 2 * width_kernels + 2 + local_kernels + passes + 2 + (n_seg <= kHistSegs && !local_cand ? 0 : 1);
   return PARD_OK;
 }
 

@@ -14,7 +14,8 @@ constexpr uint32_t kMaxPipelinesPerCall = 65536;
 constexpr uint32_t kSegNarrow = 1u;                /* bits of PardSegConst::narrow */
 constexpr uint32_t kSegNoStage = 2u;
 constexpr uint32_t kSegHighFirst = 4u;
-constexpr uint32_t kFoldSegs = 1024;              /* up to this many queues the key width is found inside k_seg_const */
+constexpr uint32_t kFoldSegs = 1024;              /* up to this many queues the constants are worked out beside the prepass */
+constexpr uint32_t kFoldCtx = 1024;               /* up to this many contexts the key width is found by the last block of another kernel */
 constexpr uint32_t kHistSegs = 64;                /* up to this many queues the batch-window tables are counted, not searched */
 constexpr uint32_t kHistCap = 8192;               /* window-table entries a counted table may have in all */
 constexpr uint32_t kSpinLimit = 1u << 18;          /* polling rounds (about a microsecond each) before giving up */
@@ -46,7 +47,7 @@ struct PlanHeader {
   uint32_t use_scan;          /* 1: too many batch windows for the window tables: decide by scanning */
   uint32_t aborted;           /* 1: a bounded wait ran out; the sort is incomplete and every later kernel returns */
   uint32_t win_done;          /* blocks of k_windows that have finished */
-  uint32_t seg_done;          /* blocks of k_seg_const that have stored their constants */
+  uint32_t seg_done;          /* blocks of k_seg_const (k_prepass) that have finished */
   uint32_t unsorted;          /* 1: some request's ctx is smaller than its predecessor's */
   uint32_t ctx_too_big;       /* 1: some ctx holds more requests than one sort tile */
   uint32_t bad_input;         /* 1: PARD_EDATA was found (kept apart from `status`, which holds the first error only) */
