@@ -303,7 +303,7 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     for (uint32_t i = threadIdx.x; i < 2 * n_ctx; i += blockDim.x) s_range[i] = 0;
     __syncthreads();
   }
-  bool time_back = false, pair_back = false, pair_seen = false;   /* see PlanHeader; looked for until both have been met */
+  bool time_back = false, pair_back = false;     /* see PlanHeader; looked for until both have been met */
   uint32_t run_ctx = kNone;
   unsigned long long lmin = ~0ull, lmax = 0;
   bool bad_seen = false;
@@ -348,30 +348,63 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       r[i] = j < n ? __ldg(&req[j]) : make_uint4(0u, 0u, kNone, 0u);
     }
     /* Are the requests in deadline order already?  Queues filled in arrival order with one
-     * objective are; then the key's deadline field needs no radix pass. */
+     * objective are; then the key's deadline field needs no radix pass.  Mostly a warp's 128 requests are
+     * of one ctx and share the deadlines' high word: then low words are compared, one shuffle per row. */
+    bool ordered = false;                        /* all 128 there, in range, of one ctx and in order: their range is that of the ends */
     if (!(time_back && pair_back)) {
       uint4 p = make_uint4(0u, 0u, 0u, 0u);      /* the request before the warp's first one */
       if (first > 0 && first < n) p = __ldg(&req[first - 1]);
-      /* one shuffle per row and word: lane 31 hands out the row before, whose last request precedes
-       * lane 0's (rows beyond the array compare as in order) */
+      const uint32_t c0 = __shfl_sync(0xffffffffu, r[0].z, 0), h0 = __shfl_sync(0xffffffffu, r[0].y, 0);
+      uint32_t other = first + 32 * kPreUn <= n && c0 < n_ctx && h0 < (uint32_t)(PARD_TIME_LIMIT_US >> 32) ? 0u : 1u, top = 0;
+      uint32_t last = 0;                         /* lane 31: the row before */
+      bool back = false;
 #pragma unroll
       for (int i = 0; i < kPreUn; ++i) {
-        const uint4 q = i == 0 ? p : r[i > 0 ? i - 1 : 0];
-        const bool give = lane == 31;
-        const unsigned long long D = ((unsigned long long)r[i].y << 32) | r[i].x, qD = ((unsigned long long)q.y << 32) | q.x;
-        const unsigned long long pD = __shfl_sync(0xffffffffu, give ? qD : D, (lane - 1) & 31);
-        const bool in = first + i * 32 + lane < n;
-        time_back |= in && D < pD;
-        if (!pair_back) {                        /* (uniform) */
+        const uint32_t px = __shfl_sync(0xffffffffu, lane == 31 ? last : r[i].x, (lane - 1) & 31);
+        last = r[i].x;
+        back |= r[i].x < px;                     /* (lane 0 of the first row compares with 0) */
+        other |= (r[i].z ^ c0) | (r[i].y ^ h0);
+        top = max(top, r[i].w & 0xffffu);
+      }
+      if (__all_sync(0xffffffffu, other == 0)) { /* what is left: the warp's first request against the one before */
+        ordered = __all_sync(0xffffffffu, !back && top < S);
+        const unsigned long long D = ((unsigned long long)r[0].y << 32) | r[0].x, pD = ((unsigned long long)p.y << 32) | p.x;
+        const bool tb = back || (lane == 0 && D < pD), pb = back || (lane == 0 && (r[0].z < p.z || (r[0].z == p.z && D < pD)));
+        time_back = time_back || __any_sync(0xffffffffu, tb);
+        pair_back = pair_back || __any_sync(0xffffffffu, pb);
+      } else {
+        /* one shuffle per row and word: lane 31 hands out the row before, whose last request precedes
+         * lane 0's (rows beyond the array compare as in order) */
+        bool time_seen = false, pair_seen = false;
+#pragma unroll
+        for (int i = 0; i < kPreUn; ++i) {
+          const uint4 q = i == 0 ? p : r[i > 0 ? i - 1 : 0];
+          const bool give = lane == 31;
+          const unsigned long long D = ((unsigned long long)r[i].y << 32) | r[i].x, qD = ((unsigned long long)q.y << 32) | q.x;
+          const unsigned long long pD = __shfl_sync(0xffffffffu, give ? qD : D, (lane - 1) & 31);
           const uint32_t pc = __shfl_sync(0xffffffffu, give ? q.z : r[i].z, (lane - 1) & 31);
+          const bool in = first + i * 32 + lane < n;
+          time_seen |= in && D < pD;
           pair_seen |= in && (r[i].z < pc || (r[i].z == pc && D < pD));
         }
+        time_back = time_back || __any_sync(0xffffffffu, time_seen);
+        pair_back = pair_back || __any_sync(0xffffffffu, pair_seen);
       }
-      time_back = __any_sync(0xffffffffu, time_back);
-      pair_back = pair_back || __any_sync(0xffffffffu, pair_seen);
     }
     /* a new chunk usually lies in another ctx than the last one: hand the old one over together */
     if (__any_sync(0xffffffffu, run_ctx != kNone && r[0].z != run_ctx)) warp_flush();
+    if (ordered) {
+      if (r[0].z != run_ctx) {                   /* (uniform) */
+        flush();
+        run_ctx = r[0].z;
+        lmin = ~0ull;
+        lmax = 0;
+      }
+      const unsigned long long D0 = ((unsigned long long)r[0].y << 32) | r[0].x, D1 = ((unsigned long long)r[kPreUn - 1].y << 32) | r[kPreUn - 1].x;
+      lmin = D0 < lmin ? D0 : lmin;
+      lmax = D1 > lmax ? D1 : lmax;
+      continue;
+    }
 #pragma unroll
     for (int i = 0; i < kPreUn; ++i) {
       if (first + i * 32 + lane >= n) continue;

@@ -24,6 +24,10 @@ constexpr int kSortThreads = 512;
 constexpr int kLoWarps = 8;                        /* warps 0..7 also do the look-back (one thread per digit) */
 constexpr int kItemsLo = 10, kItemsHi = 22;        /* rounds of 32 elements per warp: look-back warps / others (measured best) */
 constexpr int kSortTile = 32 * (kLoWarps * kItemsLo + (kSortThreads / 32 - kLoWarps) * kItemsHi);
+constexpr int kSmallLo = 6, kSmallHi = 12;         /* the same for the tiles of calls that do not fill the device: at most */
+constexpr uint32_t kSmallTile = 256 * (kSmallLo + kSmallHi), kSmallLeast = 8;    /* 4,608 elements, at least 2,048 */
+constexpr uint32_t kResidentTiles = 296;           /* tiles in flight on the full chip: two blocks per multiprocessor */
+constexpr int kLookGroup = 16;                     /* tiles whose counts are added up before the walk back */
 constexpr int kDecThreads = 128;                   /* small blocks: a short tail when the grid drains (measured against 64 and 256) */
 constexpr int kDecItems = 8;
 constexpr int kDecTile = kDecThreads * kDecItems;
