@@ -29,7 +29,9 @@ struct Layout {
       ctx_start, pipes, ktab, kept_base, chunk_base, tile_agg, tile_carry, win_off, win_cnt, wtab, kept_tmp,
       buf_a, buf_b, total;
   uint32_t n_seg, sort_tiles, dec_tiles, max_passes, win_capacity;
-  uint32_t lb_tiles;          /* tiles the look-back arrays are sized for */
+  uint32_t lb_rows;           /* rows of 256 words of a look-back array: tiles, and groups of tiles */
+  uint32_t ctx_tiles;         /* most tiles of passes inside the contexts' ranges */
+  uint32_t small_tiles, tile_size, geometry;   /* see make_layout, k_sort_rest */
   uint32_t ctx_passes;        /* 1: the call may sort inside the contexts' ranges (contexts of more than a tile on average) */
 };
 
@@ -45,11 +47,33 @@ inline uint32_t ceil_log2(uint64_t x) {          /* smallest b with 2^b >= x */
   return b;
 }
 
+/* Passes of the sort of a large call that get a launch of their own: the 24 bits that a queue id and
+ * the deadlines of about a second take. */
+constexpr uint32_t kOwnPasses = 3;
+
+bool local_sort_candidate(uint64_t n, uint32_t n_ctx) {
+  if (n_ctx == 1) return n > 0 && n <= (uint64_t)kSortTile;         /* certain: one ctx inside one tile */
+  return n >= (uint64_t)n_ctx * (kSortTile / 4) && n <= (uint64_t)n_ctx * kSortTile;
+}
+
 Layout make_layout(uint64_t n, uint32_t n_ctx, int32_t stage_stride) {
   Layout L;
   auto al = [](uint64_t x) { return (x + 255) & ~(uint64_t)255; };
   L.n_seg = n_ctx * (uint32_t)stage_stride;
-  L.sort_tiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
+  /* the sort's tiles: kSortTile elements, or, where one or two rounds of smaller ones do, as many as the
+   * device holds at a time (see k_sort_rest; three rounds of smaller ones lose to two of kSortTile) */
+  L.small_tiles = n <= 2ull * kResidentTiles * kSmallTile ? 1u : 0u;
+  L.tile_size = kSortTile;
+  L.geometry = 0;
+  if (L.small_tiles) {
+    const uint64_t rounds = std::max<uint64_t>(1, (n + (uint64_t)kResidentTiles * kSmallTile - 1) / ((uint64_t)kResidentTiles * kSmallTile));
+    const uint64_t size = (n + kResidentTiles * rounds - 1) / (kResidentTiles * rounds);
+    const uint32_t both = (uint32_t)std::min<uint64_t>(kSmallLo + kSmallHi, std::max<uint64_t>(kSmallLeast, (size + 255) / 256));
+    const uint32_t lo = std::max(1u, (both * kSmallLo + (kSmallLo + kSmallHi) / 2) / (kSmallLo + kSmallHi));
+    L.geometry = lo | (both - lo) << 8;
+    L.tile_size = 256 * both;
+  }
+  L.sort_tiles = (uint32_t)((n + L.tile_size - 1) / L.tile_size);
   L.dec_tiles = (uint32_t)((n + kDecTile - 1) / kDecTile);
   uint32_t ibits = std::max(1u, ceil_log2(n));
   uint32_t sbits = ceil_log2(L.n_seg);
@@ -65,10 +89,11 @@ Layout make_layout(uint64_t n, uint32_t n_ctx, int32_t stage_stride) {
   /* passes kept inside the contexts' ranges cut the tiles at ctx boundaries: at most one more
    * tile per ctx; they keep digit counts per ctx */
   L.ctx_passes = (n_ctx > 1 && (uint64_t)n_ctx * kSortTile < n) ? 1u : 0u;
-  L.lb_tiles = L.sort_tiles + (L.ctx_passes ? n_ctx : 0u);
+  L.ctx_tiles = (uint32_t)((n + kSortTile - 1) / kSortTile) + (L.ctx_passes ? n_ctx : 0u);
+  L.lb_rows = std::max(L.ctx_passes ? L.ctx_tiles : 0u, L.sort_tiles + L.sort_tiles / kLookGroup + 1);
   L.hist_ctx = o;  o = al(o + (L.ctx_passes ? 4ull * kMaxPasses * kBins * (uint64_t)n_ctx : 0ull));
-  L.lookback = o;  L.zero_end = al(o + 4ull * kBins * (uint64_t)L.lb_tiles);
-  o = al(o + 2 * 4ull * kBins * (uint64_t)L.lb_tiles);                      /* two arrays, used in turn */
+  L.lookback = o;  L.zero_end = al(o + 4ull * kBins * (uint64_t)L.lb_rows);
+  o = al(o + 2 * 4ull * kBins * (uint64_t)L.lb_rows);                      /* two arrays, used in turn */
   L.tile_first = o; o = al(o + (L.ctx_passes ? 4ull * ((uint64_t)n_ctx + 1) : 0ull));
   L.ctx_start = o; o = al(o + 4ull * ((uint64_t)n_ctx + 1));
   L.pipes = o;     o = al(o + 8ull * kMaxPipelinesPerCall);
@@ -874,17 +899,21 @@ struct SortSmem {
 };
 
 /* one warp's share of step 1: ITEMS rounds of 32 consecutive elements */
-template <int ITEMS, bool L2>
-__device__ __forceinline__ void sort_load_count(unsigned long long (&key)[kItemsHi], const unsigned long long* src,
+template <int ITEMS, bool L2, int CAP>
+__device__ __forceinline__ void sort_load_count(unsigned long long (&key)[CAP], const unsigned long long* src,
                                                 uint64_t first, uint32_t n, uint32_t shift, uint32_t* slot_row,
-                                                uint32_t lane, uint32_t dig_mask = 255u) {
+                                                uint32_t lane, uint32_t dig_mask, int items) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
+    if (i >= items) break;                             /* the same for the whole warp */
     const uint64_t j = first + i * 32 + lane;
     key[i] = j < n ? (L2 ? __ldcg(src + j) : src[j]) : ~0ull;
   }
 #pragma unroll
-  for (int i = 0; i < ITEMS; ++i) atomicAdd(&slot_row[(uint32_t)(key[i] >> shift) & dig_mask], 1u);
+  for (int i = 0; i < ITEMS; ++i) {
+    if (i >= items) break;
+    atomicAdd(&slot_row[(uint32_t)(key[i] >> shift) & dig_mask], 1u);
+  }
 }
 
 /* one warp's share of step 4 */
@@ -928,14 +957,16 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, const uint32_t (&bal
   return m;
 }
 
-template <int ITEMS, int BITS, bool L2>
-__device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[kItemsHi], const unsigned long long* src,
-                                                    uint64_t first, uint32_t shift, uint32_t* slot_row, uint32_t lane) {
+template <int ITEMS, int BITS, bool L2, int CAP>
+__device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[CAP], const unsigned long long* src,
+                                                    uint64_t first, uint32_t shift, uint32_t* slot_row, uint32_t lane, int items) {
 #pragma unroll
-  for (int i = 0; i < ITEMS; ++i) key[i] = L2 ? __ldcg(src + first + i * 32 + lane) : src[first + i * 32 + lane];
+  for (int i = 0; i < ITEMS; ++i)
+    if (i < items) key[i] = L2 ? __ldcg(src + first + i * 32 + lane) : src[first + i * 32 + lane];
   uint32_t mine = 0;                                     /* lane j: keys of this warp with digit j */
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
+    if (i >= items) break;
     const uint32_t d = (uint32_t)(key[i] >> shift);
     uint32_t bal[BITS];
 #pragma unroll
@@ -947,11 +978,12 @@ __device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[kI
 
 template <int ITEMS, int CAP, int BITS>
 __device__ __forceinline__ void sort_rank_drop_few(const unsigned long long (&key)[CAP], uint32_t shift,
-                                                   const uint32_t* slot_row, unsigned long long* keys, uint32_t lane) {
+                                                   const uint32_t* slot_row, unsigned long long* keys, uint32_t lane, int items) {
   uint32_t next = lane < (1u << BITS) ? slot_row[lane] : 0u;   /* lane j: next free slot of digit j for this warp */
   const uint32_t below = (1u << lane) - 1;
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
+    if (i >= items) break;
     const uint32_t d = (uint32_t)(key[i] >> shift) & ((1u << BITS) - 1);
     uint32_t bal[BITS];
 #pragma unroll
@@ -964,22 +996,18 @@ __device__ __forceinline__ void sort_rank_drop_few(const unsigned long long (&ke
 }
 
 /* digit width known at run time only: one instantiation per width */
-template <int ITEMS, bool L2>
-__device__ __forceinline__ void sort_load_count_few_n(unsigned long long (&key)[kItemsHi], const unsigned long long* src,
+template <int ITEMS, bool L2, int CAP>
+__device__ __forceinline__ void sort_load_count_few_n(unsigned long long (&key)[CAP], const unsigned long long* src,
                                                       uint64_t first, uint32_t shift, uint32_t bits, uint32_t* slot_row,
-                                                      uint32_t lane) {
-  switch (bits) {
-    case 1: sort_load_count_few<ITEMS, 1, L2>(key, src, first, shift, slot_row, lane); break;
-    default: sort_load_count_few<ITEMS, 2, L2>(key, src, first, shift, slot_row, lane); break;
-  }
+                                                      uint32_t lane, int items) {
+  if (bits == 1) sort_load_count_few<ITEMS, 1, L2>(key, src, first, shift, slot_row, lane, items);
+  else sort_load_count_few<ITEMS, 2, L2>(key, src, first, shift, slot_row, lane, items);
 }
 template <int ITEMS, int CAP>
 __device__ __forceinline__ void sort_rank_drop_few_n(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t bits,
-                                                     const uint32_t* slot_row, unsigned long long* keys, uint32_t lane) {
-  switch (bits) {
-    case 1: sort_rank_drop_few<ITEMS, CAP, 1>(key, shift, slot_row, keys, lane); break;
-    default: sort_rank_drop_few<ITEMS, CAP, 2>(key, shift, slot_row, keys, lane); break;
-  }
+                                                     const uint32_t* slot_row, unsigned long long* keys, uint32_t lane, int items) {
+  if (bits == 1) sort_rank_drop_few<ITEMS, CAP, 1>(key, shift, slot_row, keys, lane, items);
+  else sort_rank_drop_few<ITEMS, CAP, 2>(key, shift, slot_row, keys, lane, items);
 }
 
 /* CTX: the pass stays inside every ctx's range of the array (requests grouped by ctx, contexts of
@@ -995,19 +1023,22 @@ struct CtxTiles {
 
 /* PERSIST: the block takes tile after tile, and the elements may have been written by other blocks
  * of the same kernel (they are read from L2).  False: given up, a bounded wait ran out. */
-template <bool PERSIST, bool CTX>
+template <bool PERSIST, bool CTX, bool SMALL>
 __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf_a,
             unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ hist,
             uint32_t* __restrict__ lookback, uint32_t* __restrict__ lookback_next, uint32_t n,
-            uint32_t ibits, uint32_t stall, const CtxTiles& ct) {
+            uint32_t ibits, uint32_t stall, const CtxTiles& ct, uint32_t geometry) {
   constexpr int WARPS = kSortThreads / 32;
+  constexpr int kLo = SMALL ? kSmallLo : kItemsLo, kHi = SMALL ? kSmallHi : kItemsHi;     /* at most so many rounds per warp */
+  const int items_lo = SMALL ? (int)(geometry & 255u) : kLo, items_hi = SMALL ? (int)(geometry >> 8) : kHi;
+  const uint32_t tile_size = 256u * (uint32_t)(items_lo + items_hi);
   static_assert(kLoWarps * 32 == kBins, "one look-back thread per digit");
   const unsigned long long* src = (pass & 1) ? buf_b : buf_a;
   unsigned long long* dst = (pass & 1) ? buf_a : buf_b;
   hist += pass * kBins;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t lanebit = 1u << lane;
-  const uint32_t n_tiles = (uint32_t)(((uint64_t)n + kSortTile - 1) / kSortTile);
+  const uint32_t n_tiles = (uint32_t)(((uint64_t)n + tile_size - 1) / tile_size);
   for (;;) {
   if (tid == 0) {
     const uint32_t t = atomicAdd(&hdr->ticket[pass], 1u);
@@ -1036,7 +1067,7 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   if (!CTX && PERSIST && tile >= n_tiles) return true;
   if (CTX && S.ctx == 0xffffffffu) return true;
   if (CTX && tid < kBins) gh = ct.hist[((size_t)S.ctx * kMaxPasses + pass) * kBins + tid];
-  const uint64_t base = CTX ? (uint64_t)S.base : (uint64_t)tile * kSortTile;
+  const uint64_t base = CTX ? (uint64_t)S.base : (uint64_t)tile * tile_size;
   const uint32_t limit = CTX ? S.limit : n;            /* end of the range the tile belongs to */
   const int64_t lo_tile = CTX ? (int64_t)S.lo_tile : 0;
   const uint32_t shift = ibits + hdr->pshift + 8 * pass;
@@ -1044,21 +1075,20 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   /* 1. load and count.  The warps that will do the look-back own fewer
    * elements than the others, so that both groups finish at about the same
    * time and the look-back has registers for a wide batch. */
-  unsigned long long key[kItemsHi];
+  unsigned long long key[kHi];
   const bool lo_warp = warp < kLoWarps;
-  const uint32_t wfirst = lo_warp ? warp * (32 * kItemsLo)
-                                  : kLoWarps * 32 * kItemsLo + (warp - kLoWarps) * (32 * kItemsHi);
+  const uint32_t wfirst = lo_warp ? warp * (32 * items_lo) : kLoWarps * 32 * items_lo + (warp - kLoWarps) * (32 * items_hi);
   /* a digit of one or two bits on a full tile: counted and ranked by ballots */
   const uint32_t dig_bits = min(8u, hdr->keybits - 8 * pass);
   /* inside a ctx the bits above the key (the ctx's part of the queue id) are the same everywhere
    * and take no part in the digit */
   const uint32_t dig_mask = CTX ? (1u << dig_bits) - 1 : 255u;
-  const bool few = dig_bits <= 2 && base + kSortTile <= (uint64_t)limit;
+  const bool few = dig_bits <= 2 && base + tile_size <= (uint64_t)limit;
   if (few) {
-    if (lo_warp) sort_load_count_few_n<kItemsLo, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane);
-    else sort_load_count_few_n<kItemsHi, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane);
-  } else if (lo_warp) sort_load_count<kItemsLo, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask);
-  else sort_load_count<kItemsHi, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask);
+    if (lo_warp) sort_load_count_few_n<kLo, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane, items_lo);
+    else sort_load_count_few_n<kHi, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane, items_hi);
+  } else if (lo_warp) sort_load_count<kLo, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask, items_lo);
+  else sort_load_count<kHi, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask, items_hi);
   __syncthreads();
 
   /* 2. thread d owns digit d */
@@ -1081,6 +1111,7 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
     /* the tile's count is all that later tiles need from this one for now */
     if (!(stall && tile == 0)) st_relaxed(lookback + (size_t)tile * kBins + tid, cnt | kLbAgg);
     lookback_next[(size_t)tile * kBins + tid] = 0;     /* the array of the pass after this one */
+    if (SMALL && (tile % kLookGroup) == 0) lookback_next[((size_t)n_tiles + tile / kLookGroup) * kBins + tid] = 0;
   }
   __syncthreads();
   uint32_t dstart = 0, gstart = 0;
@@ -1097,17 +1128,53 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   }
   __syncthreads();
 
-  /* 3. look-back by the lower part of the block; the other warps go on */
+  /* 3. look-back by the lower part of the block; the other warps go on.  When all tiles
+   * start together (SMALL) no running sum is there to be found, and the walk back over single tiles took
+   * a round trip for every eight of them.  There the tiles form groups of kLookGroup: a tile adds up the
+   * counts of its own group's earlier tiles, the group's last tile publishes the group's, and the walk
+   * back goes over groups.  (At 2,048 wide tiles groups make it slower, 554 -> 573 us for a plan of
+   * 2^24: there a running sum is mostly one round trip away.) */
   if (tid < kBins) {
-    const uint32_t* lb = lookback;
     uint32_t excl = 0, spins = 0;
-    int64_t t = (int64_t)tile - 1;
-    bool done = t < lo_tile;
+    const uint32_t* lb = lookback;                       /* rows to walk back over, from row t down to row lowest */
+    uint32_t* own = lookback + (size_t)tile * kBins + tid;
+    int64_t t = (int64_t)tile - 1, lowest = lo_tile;
+    bool publish = true;
+    uint32_t mine = cnt;
+    if (SMALL) {
+      const uint32_t in_group = tile % kLookGroup;
+      uint32_t missing = in_group;                       /* earlier tiles of the group whose counts are still to come */
+      while (missing) {
+        uint32_t v[kLookGroup - 1];
+#pragma unroll
+        for (int k = 0; k < kLookGroup - 1; ++k) v[k] = k < (int)missing ? ld_relaxed(lb + (size_t)(tile - in_group + k) * kBins + tid) : 0u;
+        bool all = true;
+#pragma unroll
+        for (int k = kLookGroup - 2; k >= 0; --k) {      /* from the latest down: the row that is not there yet is usually a late one */
+          if (k < (int)missing && all) {
+            if (v[k] >> 30) { excl += v[k] & kLbMask; missing = (uint32_t)k; }
+            else all = false;
+          }
+        }
+        if (missing) {
+          if (++spins > kSpinLimit) { S.abort = 1; break; }
+          __nanosleep(40);
+        }
+      }
+      mine = excl + cnt;                                 /* the group up to this tile */
+      publish = in_group == kLookGroup - 1;
+      lb = lookback + (size_t)n_tiles * kBins;
+      own = lookback + ((size_t)n_tiles + tile / kLookGroup) * kBins + tid;
+      t = (int64_t)(tile / kLookGroup) - 1;
+      lowest = 0;
+      if (publish && !S.abort) st_relaxed(own, mine | kLbAgg);
+    }
+    bool done = t < lowest;
     while (!done) {
       uint32_t v[kLookBatch];
 #pragma unroll
       for (int k = 0; k < kLookBatch; ++k)
-        v[k] = (t - k >= lo_tile) ? ld_relaxed(lb + (size_t)(t - k) * kBins + tid) : +kLbIncl;   /* before the first tile: nothing */
+        v[k] = (t - k >= lowest) ? ld_relaxed(lb + (size_t)(t - k) * kBins + tid) : +kLbIncl;   /* before the first row: nothing */
       int used = 0;
 #pragma unroll
       for (int k = 0; k < kLookBatch; ++k) {
@@ -1118,21 +1185,21 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
         }
       }
       t -= used;
-      if (!done && used < kLookBatch) {                /* met a tile that has not published yet */
+      if (!done && used < kLookBatch) {                /* met a row that has not been published yet */
         if (++spins > kSpinLimit) { S.abort = 1; break; }
         __nanosleep(40);
       }
     }
-    if (!(stall && tile == 0)) st_relaxed(lookback + (size_t)tile * kBins + tid, ((excl + cnt) & kLbMask) | kLbIncl);
+    if (publish && !S.abort && !(stall && tile == 0)) st_relaxed(own, ((excl + cnt) & kLbMask) | kLbIncl);
     S.gofs[tid] = gstart + excl - dstart;
   }
 
   /* 4. rank and drop into the tile buffer */
   if (few) {
-    if (lo_warp) sort_rank_drop_few_n<kItemsLo, kItemsHi>(key, shift, dig_bits, S.slot[warp], S.keys, lane);
-    else sort_rank_drop_few_n<kItemsHi, kItemsHi>(key, shift, dig_bits, S.slot[warp], S.keys, lane);
-  } else if (lo_warp) sort_rank_drop<kItemsLo, kItemsHi>(key, shift, S.slot[warp], S.match[warp], S.keys, lanebit, kItemsLo, dig_mask);
-  else sort_rank_drop<kItemsHi, kItemsHi>(key, shift, S.slot[warp], S.match[warp], S.keys, lanebit, kItemsHi, dig_mask);
+    if (lo_warp) sort_rank_drop_few_n<kLo, kHi>(key, shift, dig_bits, S.slot[warp], S.keys, lane, items_lo);
+    else sort_rank_drop_few_n<kHi, kHi>(key, shift, dig_bits, S.slot[warp], S.keys, lane, items_hi);
+  } else if (lo_warp) sort_rank_drop<kLo, kHi>(key, shift, S.slot[warp], S.match[warp], S.keys, lanebit, items_lo, dig_mask);
+  else sort_rank_drop<kHi, kHi>(key, shift, S.slot[warp], S.match[warp], S.keys, lanebit, items_hi, dig_mask);
   __syncthreads();
   if (S.abort) {
     if (tid == 0) set_aborted(hdr);
@@ -1140,7 +1207,7 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   }
 
   /* 5. write out */
-  const uint32_t nvalid = (uint32_t)min((uint64_t)kSortTile, (uint64_t)limit - base);
+  const uint32_t nvalid = (uint32_t)min((uint64_t)tile_size, (uint64_t)limit - base);
 #pragma unroll 4
   for (uint32_t pos = tid; pos < nvalid; pos += kSortThreads) {
     const unsigned long long k = S.keys[pos];
@@ -1152,12 +1219,12 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   }
 }
 
-/* (a call: inlined into the loop over the passes it would spill) */
+/* (a call: inlined into the loop over the passes the wide tiles would spill more) */
 template <bool CTX>
 __device__ __noinline__ bool sort_tiles_resident(SortSmem& S, uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a,
-                                                 unsigned long long* buf_b, const uint32_t* hist, uint32_t* lookback,
-                                                 uint32_t* lookback_next, uint32_t n, uint32_t ibits, uint32_t stall, const CtxTiles& ct) {
-  return sort_tiles<true, CTX>(S, pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits, stall, ct);
+            unsigned long long* buf_b, const uint32_t* hist, uint32_t* lookback, uint32_t* lookback_next, uint32_t n,
+            uint32_t ibits, uint32_t stall, const CtxTiles& ct) {
+  return sort_tiles<true, CTX, false>(S, pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits, stall, ct, 0u);
 }
 
 /* One pass, one tile per block. */
@@ -1171,8 +1238,8 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
   if (pass >= hdr->npass || hdr->aborted || sort_is_local(hdr, local_candidate)) return;
-  sort_tiles<false, CTX>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
-                         stall, ct);
+  sort_tiles<false, CTX, false>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
+                                stall, ct, 0u);
 }
 
 /* All passes from `pass` on, by a grid that is resident as a whole and meets between them (bounded
@@ -1180,12 +1247,14 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
  * that finds nothing to do still costs a launch: 2.5 to 4.5 us each, up to seven per call.  At
  * 2^24 elements a resident grid takes 9 us more per pass than one block per tile (the blocks' loads
  * no longer start under the write-out of others), so the passes that large calls usually need keep
- * launches of their own; calls whose tiles are all resident at once do all passes here. */
-template <bool CTX>
+ * launches of their own.  Calls of one or two rounds of small tiles (SMALL) do all passes here,
+ * with tiles sized so that every block takes the same number of them. */
+template <bool CTX, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads, 2)
 k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned long long* buf_b,
             const uint32_t* __restrict__ hist, uint32_t* lookback, size_t lb_words, uint32_t n,
-            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct, const __grid_constant__ WinCountArgs wc) {
+            uint32_t ibits, uint32_t stall, uint32_t local_candidate, const CtxTiles ct, const __grid_constant__ WinCountArgs wc,
+            uint32_t geometry) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
@@ -1193,9 +1262,13 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
   if (hdr->aborted || sort_is_local(hdr, local_candidate)) return;
   const uint32_t npass = hdr->npass;
   for (uint32_t p = pass; p < npass; ++p) {
-    if (!sort_tiles_resident<CTX>(*reinterpret_cast<SortSmem*>(smem_raw), p, hdr, buf_a, buf_b, hist, lookback + (p & 1) * lb_words,
-                               lookback + ((p + 1) & 1) * lb_words, n, ibits, p == 0 ? stall : 0u, ct))
-      return;
+    SortSmem& S = *reinterpret_cast<SortSmem*>(smem_raw);
+    uint32_t* now = lookback + (p & 1) * lb_words;
+    uint32_t* next = lookback + ((p + 1) & 1) * lb_words;
+    bool go;
+    if constexpr (SMALL) go = sort_tiles<true, CTX, true>(S, p, hdr, buf_a, buf_b, hist, now, next, n, ibits, p == 0 ? stall : 0u, ct, geometry);
+    else go = sort_tiles_resident<CTX>(S, p, hdr, buf_a, buf_b, hist, now, next, n, ibits, p == 0 ? stall : 0u, ct);
+    if (!go) return;
     if (p + 1 < npass && !grid_barrier(hdr, &hdr->sort_bar[p], members)) return;
   }
 }
@@ -2387,6 +2460,7 @@ k_wide_reset(PlanHeader* hdr, uint32_t* __restrict__ hist, uint32_t* __restrict_
     hdr->keybits = wide_chunk_bits(hdr, sbits, ibits, super);   /* what the passes of this super-pass sort */
     hdr->pshift = 0;
     for (int i = 0; i <= kMaxPasses; ++i) hdr->ticket[i] = 0;
+    for (int i = 0; i < kMaxPasses; ++i) hdr->sort_bar[i] = 0;
     if (super == 0) {
       hdr->wide = 2;                                      /* the chunked sort is under way */
       hdr->status = hdr->bad_input ? (uint32_t)(-PARD_EDATA) : 0u;   /* the width was not an error after all */
@@ -2523,8 +2597,9 @@ int allow_sort_smem(int dev) {
   if (!done[dev].load(std::memory_order_relaxed)) {
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_pass<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
-    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(SortSmem)));
     const int rc = allow_local_smem();
@@ -2534,18 +2609,6 @@ int allow_sort_smem(int dev) {
   return PARD_OK;
 }
 
-/* Passes of the sort that get a launch of their own: none when all tiles are resident at once (or
- * the sort is only there in case the block-local one does not apply), else three, the 24 bits that
- * a queue id and the deadlines of about a second take. */
-uint32_t sort_own_passes(uint32_t tiles, uint32_t max_passes, int sms, uint32_t local_cand) {
-  if (local_cand || tiles <= 2u * (uint32_t)sms) return 0;
-  return std::min(3u, max_passes);
-}
-
-bool local_sort_candidate(uint64_t n, uint32_t n_ctx) {
-  if (n_ctx == 1) return n > 0 && n <= (uint64_t)kSortTile;         /* certain: one ctx inside one tile */
-  return n >= (uint64_t)n_ctx * (kSortTile / 4) && n <= (uint64_t)n_ctx * kSortTile;
-}
 
 int check_state(const pard_queue_state_t* st, uint32_t n_ctx) {
   if (!st) return PARD_EINVAL;
@@ -2642,7 +2705,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   PardSegConst* ktab = (PardSegConst*)(ws + L.ktab);
   uint32_t* hist = (uint32_t*)(ws + L.hist);
   uint32_t* lookback = (uint32_t*)(ws + L.lookback);
-  const size_t lb_words = (size_t)L.lb_tiles * kBins;
+  const size_t lb_words = (size_t)L.lb_rows * kBins;
   unsigned long long* tile_agg = (unsigned long long*)(ws + L.tile_agg);
   int32_t* tile_carry = (int32_t*)(ws + L.tile_carry);
   uint32_t* seg_kept = (uint32_t*)(ws + L.seg_kept);
@@ -2750,9 +2813,13 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  0, stream, hdr, hist, lookback, (unsigned long long)lb_words, sbits, ibits, sp);
       launch_pdl(k_wide_pack, grid_n, 256, 0, stream, req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, state->d_priority, sbits, ibits,
                  sp, (const PlanHeader*)hdr, (const uint32_t*)order, buf_a, hist);
-      for (uint32_t p = 0; p < chunk_passes; ++p)
-        launch_pdl(k_sort_pass<false>, L.sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
-                   lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, CtxTiles{}, WinCountArgs{});
+      if (L.small_tiles)
+        launch_pdl(k_sort_rest<false, true>, std::min<uint32_t>(L.sort_tiles, 2u * (uint32_t)sms), kSortThreads, sizeof(SortSmem), stream, 0u,
+                   hdr, buf_a, buf_b, (const uint32_t*)hist, lookback, lb_words, n32, ibits, 0u, 0u, CtxTiles{}, WinCountArgs{}, L.geometry);
+      else
+        for (uint32_t p = 0; p < chunk_passes; ++p)
+          launch_pdl(k_sort_pass<false>, L.sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
+                     lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, CtxTiles{}, WinCountArgs{});
       launch_pdl(k_wide_chase, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a, buf_b, n32,
                  ibits, sp, (const uint32_t*)order);
       launch_pdl(k_wide_keep, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a,
@@ -2841,7 +2908,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                state->d_priority, buf_a, buf_b, local_sure ? (const uint32_t*)nullptr : (const uint32_t*)ctx_start, n32, S,
                ceil_log2(S), ibits);
   if (ctx_sort) {
-    launch_pdl(k_pack_ctx, L.lb_tiles, 256, 0, stream, req4, S, ctx_dmin, ctx_dmax, state->d_priority, ibits, hdr, buf_a,
+    launch_pdl(k_pack_ctx, L.ctx_tiles, 256, 0, stream, req4, S, ctx_dmin, ctx_dmax, state->d_priority, ibits, hdr, buf_a,
                (uint32_t*)(ws + L.hist_ctx), ctx_tiles);
   } else if (n > 0 && !local_sure) {             /* returns at once when the blocks above did the work */
     uint32_t grid = (uint32_t)std::min<uint64_t>((n + 255) / 256, (uint64_t)sms * 8);
@@ -2850,9 +2917,10 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                (const uint32_t*)win_cnt, whist);
   }
   /* passes with a launch of their own, then the rest in one kernel (see k_sort_rest) */
-  const uint32_t sort_tiles = ctx_sort ? L.lb_tiles : L.sort_tiles;
+  const uint32_t sort_tiles = ctx_sort ? L.ctx_tiles : L.sort_tiles;
   const uint32_t max_passes = ctx_sort ? std::min<uint32_t>(kMaxPasses, (key_sbits + 60 + 7) / 8) : L.max_passes;
-  const uint32_t own_passes = sort_own_passes(sort_tiles, max_passes, sms, local_cand);
+  const bool small = L.small_tiles && !ctx_sort;
+  const uint32_t own_passes = small || local_cand ? 0u : std::min(kOwnPasses, max_passes);
   const uint32_t rest_grid = std::min<uint32_t>(sort_tiles, 2u * (uint32_t)sms);
   const uint32_t stall = (mode & PARD_MODE_TEST_STALL) && !ctx_sort ? 1u : 0u;
   WinCountArgs wc = {};
@@ -2868,8 +2936,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  buf_b, hist, lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, p == 0 ? stall : 0u,
                  local_cand, ctx_tiles, wc);
     else if (p == own_passes)
-      launch_pdl(ctx_sort ? k_sort_rest<true> : k_sort_rest<false>, rest_grid + wc.on, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
-                 buf_b, hist, lookback, lb_words, n32, ibits, stall, local_cand, ctx_tiles, wc);
+      launch_pdl(ctx_sort ? k_sort_rest<true, false> : small ? k_sort_rest<false, true> : k_sort_rest<false, false>, rest_grid + wc.on, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
+                 buf_b, hist, lookback, lb_words, n32, ibits, stall, local_cand, ctx_tiles, wc, L.geometry);
     wc.on = 0;                                             /* the first launch has done it */
   }
   mark();
@@ -2942,12 +3010,7 @@ extern "C" int pard_plan_kernel_launches(uint64_t n, uint32_t n_ctx, int32_t sta
   const bool local_cand = local_sort_candidate(n, n_ctx);
   const uint32_t local_kernels = local_cand ? 2 : 0;            /* ctx_ranges, sort_local */
   const Layout L = make_layout(n, n_ctx, stage_stride);
-  int dev = 0, sms = 148;                                       /* without a device: as on the full chip */
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    sms = 148;
-  }
-  const uint32_t own = sort_own_passes(L.sort_tiles, L.max_passes, sms, local_cand ? 1u : 0u);
+  const uint32_t own = L.small_tiles || local_sort_candidate(n, n_ctx) ? 0u : std::min(kOwnPasses, L.max_passes);
   const uint32_t passes = own + (own < L.max_passes ? 1 : 0);   /* and the kernel that does the rest */
   if (n_ctx == 1 && n > 0 && n <= (uint64_t)kSortTile) *launches = 1;
   else if (n == 0) *launches = 4 + width_kernels;               /* clear, (key_width,) seg_const, windows, kept_scan */
