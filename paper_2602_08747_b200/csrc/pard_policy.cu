@@ -131,16 +131,22 @@ __device__ __noinline__ long long masked_lsub(const PolicyArgs& a, const StagedP
 }
 
 /* number of batch rounds b for which a request still fits, b < v: Nexus tests "base + b*d + d <= D" */
-__device__ __forceinline__ uint32_t rounds_fit(long long X, const PardSegConst& K) {
+__device__ __forceinline__ uint32_t rounds_fit(long long X, unsigned long long magic, const PardSegConst& K) {
   if (X < 0) return 0;
   unsigned long long q;
-  if (((unsigned long long)X >> 32) == 0 && K.d_magic) q = div_magic32((uint32_t)X, K.d_magic);
+  if (((unsigned long long)X >> 32) == 0 && magic) q = div_magic32((uint32_t)X, magic);
   else q = (unsigned long long)X / (unsigned long long)K.d;
   return q >= kUClamp ? kUClamp : (uint32_t)q + 1;
 }
 
-/* One request's rounds and, for PARD_MODE_PATH_MASK, its own downstream estimate. */
-__global__ void __launch_bounds__(kPolThreads)
+/* One request's rounds and, for PARD_MODE_PATH_MASK, its own downstream estimate.  What it takes from
+ * the queue's constants stays in registers while a thread's requests are of one queue, which they
+ * mostly are: bound by instructions otherwise (2^24 requests under the window scan: 111 us with the
+ * table entry read for every request). */
+/* (Without masks the kernels of this file are kept to 64 registers: 32 warps per multiprocessor; the
+ * masked estimate is a call that costs more.) */
+template <bool MASK>
+__global__ void __launch_bounds__(kPolThreads, MASK ? 5 : 8)
 k_policy_terms(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   __shared__ StagedPaths sp;
@@ -148,8 +154,12 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
   const SortedView v = sorted_view(a);
   const bool lookup = a.hdr->lookup != 0;
   const uint64_t tile0 = (uint64_t)blockIdx.x * kPolTile;
-  if (a.mode & PARD_MODE_PATH_MASK) stage_paths(a, v, tile0, sp);
+  if (MASK) stage_paths(a, v, tile0, sp);
   constexpr int kUn = 4;                           /* elements, then their records, requested together */
+  uint32_t cur = 0xffffffffu;
+  long long from = 0;                              /* deadline - A = offset (or deadline) - from, or from - offset */
+  unsigned long long magic = 0;
+  bool none = false, falls = false;
 #pragma unroll 1
   for (int i0 = 0; i0 < kPolItems; i0 += kUn) {
     unsigned long long e[kUn], D[kUn];
@@ -167,7 +177,7 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
       flags[u] = 0;
       if (j >= a.n) continue;
       if (lookup) D[u] = __ldg(reinterpret_cast<const unsigned long long*>(&a.req[idx]));
-      if (a.mode & PARD_MODE_PATH_MASK) flags[u] = __ldg(&reinterpret_cast<const uint32_t*>(&a.req[idx])[3]) >> 16;
+      if (MASK) flags[u] = __ldg(&reinterpret_cast<const uint32_t*>(&a.req[idx])[3]) >> 16;
     }
 #pragma unroll
     for (int u = 0; u < kUn; ++u) {
@@ -175,9 +185,17 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
       if (j >= a.n) continue;
       const uint32_t seg = (uint32_t)(e[u] >> v.kshift), idx = (uint32_t)e[u] & v.imask;
       const PardSegConst& K = a.ktab[seg];
-      if (K.narrow & kSegNoStage) { set_status(a.hdr, PARD_EDATA); v.T[j] = 0; continue; }
-      long long X = lookup ? (long long)D[u] - K.A : slack_of((e[u] >> a.ibits) & v.dmask, K);   /* deadline - A */
-      if (a.mode & PARD_MODE_NEXUS) X += K.lsub;   /* the current module only: base + d */
+      if (seg != cur) {
+        cur = seg;
+        from = lookup ? K.A : K.A_rel;
+        if (a.mode & PARD_MODE_NEXUS) from -= K.lsub;           /* the current module only: base + d */
+        falls = !lookup && (K.narrow & kSegHighFirst);          /* offsets counted down from the ctx's largest deadline */
+        magic = K.d_magic;
+        none = K.narrow & kSegNoStage;
+      }
+      if (none) { set_status(a.hdr, PARD_EDATA); v.T[j] = 0; continue; }
+      long long X = (long long)(lookup ? D[u] : (e[u] >> a.ibits) & v.dmask) - from;
+      if (falls) X = -X;
       if (a.mode & PARD_MODE_CLIPPER) {
         /* the module's share of the request's objective, counted from its arrival at the module; the
          * request is kept iff its batch starts within the share: start <= arrive + share, i.e.
@@ -192,8 +210,8 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
           X = ar.arrive_us + share + K.d - (K.A - K.lsub);
         }
       }
-      if (flags[u]) X += K.lsub - masked_lsub(a, sp, seg, flags[u], K);
-      v.T[j] = rounds_fit(X, K);
+      if (MASK && flags[u]) X += K.lsub - masked_lsub(a, sp, seg, flags[u], K);
+      v.T[j] = rounds_fit(X, magic, K);
     }
   }
 }
@@ -535,10 +553,14 @@ k_policy_walk(const __grid_constant__ PolicyArgs a) {
 }
 
 /* Estimates, decisions and survivors.  A request's round is the number of rounds of its queue that
- * ended at or before it (a search in the ends, starting at the round of the thread's request
- * before); its place among the survivors is, for Nexus, given by its window, else the kept requests
+ * ended at or before it, found by a search in the ends: a warp's 32-ary search for the warp's first
+ * request, and from a round known to be close for all others -- a round takes at least a batch of
+ * requests, so p positions on it is at most p / cap rounds on.  (A binary search over all of the
+ * queue's rounds for every 128th request was a chain of up to 120 dependent loads: 2^24 requests in
+ * queues of 2^15 rounds, 130 us.)  Its place among the survivors is, for Nexus, given by its window, else the kept requests
  * ahead of it: those ahead of the tile (a.tile_x) and, by ballots, those inside it. */
-__global__ void __launch_bounds__(kPolThreads)
+template <bool MASK>
+__global__ void __launch_bounds__(kPolThreads, MASK ? 5 : 8)
 k_policy_emit(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   constexpr int kWarps = kPolThreads / 32, kRows = kPolItems * kWarps;
@@ -549,8 +571,8 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   const SortedView v = sorted_view(a);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile0 = blockIdx.x * kPolTile;
-  const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW, mask = a.mode & PARD_MODE_PATH_MASK;
-  if (mask) stage_paths(a, v, tile0, sp);
+  const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
+  if (MASK) stage_paths(a, v, tile0, sp);
   unsigned long long e[kPolItems];
   uint32_t t[kPolItems], round[kPolItems], flags[kPolItems];
 #pragma unroll
@@ -559,15 +581,33 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
     e[i] = j < a.n ? v.src[j] : 0ull;
     t[i] = j < a.n && !nexus ? v.T[j] : 0u;
   }
-  if (mask) {
+  if (MASK) {
 #pragma unroll
     for (int i = 0; i < kPolItems; ++i) {
       const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
       flags[i] = j < a.n ? __ldg(&reinterpret_cast<const uint32_t*>(&a.req[(uint32_t)e[i] & v.imask])[3]) >> 16 : 0u;
     }
   }
-  uint32_t cur = 0xffffffffu, lo = 0, hi = 0, nb = 0, b = 0, end = 0, cap = 0, tail = 0, keepbits = 0;
+  uint32_t cur = 0xffffffffu, lo = 0, hi = 0, nb = 0, b = 0, end = 0, cap = 0, tail = 0, keepbits = 0, at_once = 0;
   bool none = false;
+  /* the round of the warp's first request, for a warp whose first 32 requests are of one queue */
+  const uint32_t p0 = tile0 + warp * 32;
+  const uint32_t seg_first = __shfl_sync(0xffffffffu, (uint32_t)(e[0] >> v.kshift), 0);
+  const bool together = !raw && __all_sync(0xffffffffu, p0 + lane < a.n && (uint32_t)(e[0] >> v.kshift) == seg_first);
+  uint32_t b0 = 0;
+  if (together) {
+    const uint32_t* ends = v.C + a.seg_off[seg_first];
+    uint32_t z = a.rounds[seg_first];
+    while (b0 < z) {                               /* uniform across the warp */
+      const uint32_t span = z - b0;
+      const uint32_t p = b0 + (uint32_t)(((unsigned long long)(lane + 1) * span) / 33u);   /* b0 <= p < z */
+      const uint32_t c = __popc(__ballot_sync(0xffffffffu, ends[p] <= p0));                /* the lanes before lane c */
+      const uint32_t p_below = __shfl_sync(0xffffffffu, p, c > 0 ? c - 1 : 0);
+      const uint32_t p_at = __shfl_sync(0xffffffffu, p, c < 32 ? c : 31);
+      if (c > 0) b0 = p_below + 1;
+      if (c < 32) z = p_at;
+    }
+  }
 #pragma unroll
   for (int i = 0; i < kPolItems; ++i) {
     const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
@@ -585,6 +625,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
         none = a.ktab[seg].narrow & kSegNoStage;
         tail = nexus ? a.tail[seg] : 0u;
         b = 0;
+        at_once = cap ? kPolThreads / cap + 1 : kPolThreads;
         look = true;
       }
       if (raw) {
@@ -592,6 +633,8 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
         b = magic ? div_magic32(j - lo, magic) : j - lo;
       } else if (look || j >= end) {               /* (b < nb and the round goes on: nothing to search) */
         uint32_t z = nb;                           /* ends b .. nb-1: how many are <= j */
+        if (!look) z = min(nb, b + at_once);       /* kPolThreads positions on from a request of round b */
+        else if (i == 0 && together) { b = b0; z = min(nb, b0 + 31u / max(cap, 1u) + 1); }
         while (b < z) {
           const uint32_t mid = b + (z - b) / 2;
           if (v.C[lo + mid] <= j) b = mid + 1; else z = mid;
@@ -640,7 +683,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
     }
     const uint32_t keep = (keepbits >> i) & 1u;
     long long A = A0;
-    if (mask && flags[i] && d) A += masked_lsub(a, sp, seg, flags[i], a.ktab[seg]) - a.ktab[seg].lsub;
+    if (MASK && flags[i] && d) A += masked_lsub(a, sp, seg, flags[i], a.ktab[seg]) - a.ktab[seg].lsub;
     if (a.out_keep) a.out_keep[j] = (uint8_t)keep;
     if (a.out_est) a.out_est[j] = A + (long long)round[i] * d;
     if (a.out_perm) a.out_perm[j] = idx;
@@ -661,7 +704,7 @@ namespace pard_plan_detail {
 int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
   static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
-  launch_pdl(k_policy_terms, tiles, kPolThreads, 0, stream, a);
+  launch_pdl(a.mode & PARD_MODE_PATH_MASK ? k_policy_terms<true> : k_policy_terms<false>, tiles, kPolThreads, 0, stream, a);
   if (a.n / a.n_seg >= kWalkLong)
     launch_pdl(k_policy_walk<kWalkWarps>, a.n_seg, kWalkWarps * 32, 0, stream, a);
   else
@@ -671,7 +714,7 @@ int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
 
 int launch_policy_emit(const PolicyArgs& a, cudaStream_t stream) {
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
-  launch_pdl(k_policy_emit, tiles, kPolThreads, 0, stream, a);
+  launch_pdl(a.mode & PARD_MODE_PATH_MASK ? k_policy_emit<true> : k_policy_emit<false>, tiles, kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
 }
 
