@@ -122,3 +122,40 @@ def test_window_tables_of_many_queues(n_ctx, S, n, mode):
     check(wl, mode)
     wl.state.priority = rng.integers(0, 2, size=(n_ctx, S)).astype(np.uint8)
     check(wl, mode)
+
+
+# ---- tiles of a small call: least size, last group of tiles, one and two rounds, beyond ----------------
+@pytest.mark.parametrize("n", [8193, 2048 * 16, 2048 * 16 + 1, 2048 * 296, 2048 * 296 + 1, 296 * 4608, 296 * 4608 + 1,
+                               2 * 296 * 4608, 2 * 296 * 4608 + 1])
+def test_sort_tiles_at_the_edges_of_their_sizes(n):
+    sizes = [n // 3, n // 7, n - n // 3 - n // 7]
+    check(several_ctx(3, sizes, seed=n, sort=False, mix=True, span=3_000_000))
+
+
+# ---- order check on low words: high words, contexts and single steps inside and between warps ----------
+@pytest.mark.parametrize("at", [1, 31, 32, 33, 127, 128, 129, 5000, 19_999])
+@pytest.mark.parametrize("kind", ["step back", "high word", "new ctx", "bad stage"])
+def test_order_check_finds_the_single_step(at, kind):
+    wl = several_ctx(2, [20_000, 0], span=10**6)
+    if kind == "step back":
+        wl.requests["deadline_us"][at] = wl.requests["deadline_us"][at - 1] - 1
+    elif kind == "high word":                      # in order, low words stepping back
+        wl.requests["deadline_us"][at:] += (1 << 32) - 10**6
+    elif kind == "new ctx":
+        wl.requests["ctx"][at:] = 1
+        wl.requests["deadline_us"][at:] -= 900
+    else:
+        wl.requests["stage"][at] = 3
+        assert run_library(wl, 0, check=False)[0] == pb.PARD_EDATA
+        return
+    check(wl)
+
+
+# ---- packing with and without single words, queues' constants and counters of 32 bits ------------------
+@pytest.mark.parametrize("span", [1 << 28, (1 << 29) - 1, 1 << 29, 1 << 31])
+@pytest.mark.parametrize("n_ctx", [1, 3])
+def test_packing_at_the_widths_of_its_words(span, n_ctx):
+    wl = several_ctx(n_ctx, [40_000 // n_ctx] * n_ctx, sort=False, span=span)
+    wl.requests["deadline_us"][:2] = 1000, 1000 + span
+    for mode in (0, pb.PARD_MODE_GROUPED):
+        check(wl, mode)
