@@ -270,8 +270,8 @@ def kernel_table(prof, n, keep_frac, peak, prof_coarse=None):
     events the library records on its own stream.  "k_decide_win" is the decision
     kernel (threshold, estimate, keep, survivor lists; the phase also holds the
     three fallback launches that return at once); "decision_pass" is everything
-    after the sort: k_seg_win, k_win_bounds, k_win_prefix, the decision, k_kept_scan
-    and k_kept_move, timed as one phase (no events between its kernels) in a
+    after the sort: the searched window tables where a call has them and the decision,
+    timed as one phase (no events between its kernels) in a
     second, shorter run when prof_coarse is given."""
     k = prof["n_samples"]
     ms = prof["ms"]
@@ -508,7 +508,7 @@ def run_aux(dev, peak, kernels_only=False):
         sec, _ = timed_steps(plan, 10, 3, None)
         rules[label] = {"ms": 1e3 * sec / 10, "requests_per_s": w2.n * 10 / sec, "keep_fraction": kf}
         del plan
-    out["comparison_rules"] = {"workload": WORKLOAD + "b (16 queues of about 2^20 requests: one warp walks each queue)", **rules}
+    out["comparison_rules"] = {"workload": WORKLOAD + "b (16 queues of about 2^20 requests, each walked round by round)", **rules}
 
     # closed-loop replay: 16 instances, 64 epochs of 65,536 requests
     job_rng = np.random.default_rng(11)

@@ -191,19 +191,14 @@ typedef struct pard_plan_out {
                                    sizes:
                                    - contexts of at most 8,192 requests on average: the
                                      promise then includes that NO ctx holds more than
-                                     8,192.  Up to a few hundred contexts one thread block
-                                     plans each ctx from start to end in shared memory --
-                                     constants, sort, positions, decisions -- in six
-                                     kernel launches instead of about twenty, two to three
-                                     times faster on small and medium calls; beyond that a
-                                     block per ctx reads, checks and sorts its ctx and the
-                                     rest is the general path, minus its pass over all
-                                     requests for the deadline ranges and minus the
-                                     kernels it launches in reserve for ungrouped input;
+                                     8,192.  One thread block plans each ctx from start to
+                                     end in shared memory -- constants, sort, window
+                                     tables, decisions -- in a few kernel launches, two to
+                                     three times faster than without the promise;
                                    - larger contexts (and stage_stride a power of two):
                                      the radix passes stay inside every ctx's range and
-                                     sort the stage and deadline bits only -- one pass
-                                     fewer whenever the ctx bits of the key cost one.
+                                     sort the stage and deadline bits only (the stage
+                                     bits alone where deadlines come in order).
                                    The device checks the claim: a call that breaks it
                                    returns PARD_EDATA (as does, in the block-per-ctx
                                    forms, any request out of range) with unspecified
@@ -214,9 +209,9 @@ typedef struct pard_plan_out {
 
 /* Other decision orders and rules on the same queues, for comparison with the
  * planner's own (which stays the default).  Their thresholds do not rise along
- * a queue, so each queue is walked in order by one warp (32 requests per step)
- * instead of being decided request by request; they cost a few times the
- * default rule on long queues.  None combines with PARD_MODE_RAW.
+ * a queue, so each queue is walked round by round (a batch of every worker) by a
+ * group of warps instead of being decided request by request; they cost about
+ * what the default rule does.  None combines with PARD_MODE_RAW.
  *   PARD_MODE_PATH_MASK  requests whose downstream path is known (Sec. 5.2,
  *       dynamic-path DAGs, where a request takes one of several branches):
  *       pard_request_t.flags is a mask over the downstream paths of the
