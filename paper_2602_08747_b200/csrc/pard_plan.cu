@@ -191,7 +191,12 @@ struct ConstArgs {
   uint32_t arrival_order, win_hist, force_scan;
   uint32_t* win_off;
   uint32_t* win_cnt;
+  long long* path_sums;            /* see PolicyArgs; or null */
 };
+
+__device__ __forceinline__ long long* sums_of(const ConstArgs& a, uint32_t c) {
+  return a.path_sums ? a.path_sums + (size_t)c * a.st.stage_stride * kMaskPaths : nullptr;
+}
 
 /* By one whole block, once every ctx's deadline range and every queue's constants are there: what
  * hangs on both.  RANGES: the constants do not know the ranges yet. */
@@ -274,7 +279,7 @@ k_seg_const(const __grid_constant__ ConstArgs a, const unsigned long long* __res
   pdl_wait();
   __shared__ CtxScratch scratch;
   if (ctx_constants(a.pipes, a.n_pipelines, a.st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
-                    a.ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch))
+                    a.ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch, sums_of(a, blockIdx.x)))
     set_status(hdr, PARD_EDATA);
   if (a.with_key_width && last_block_done(&hdr->seg_done)) finish_constants<false>(a, ctx_dmin_inv, ctx_dmax, hdr);
 }
@@ -296,7 +301,8 @@ constexpr int kPreUn = 4;
 
 __device__ __noinline__ void const_block(const ConstArgs& a, uint32_t c, PlanHeader* hdr) {
   __shared__ CtxScratch scratch;
-  if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, 0, 0, a.ktab + (size_t)c * a.st.stage_stride, scratch)) set_status(hdr, PARD_EDATA);
+  if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, 0, 0, a.ktab + (size_t)c * a.st.stage_stride, scratch, sums_of(a, c)))
+    set_status(hdr, PARD_EDATA);
 }
 __device__ __noinline__ void const_tail(const ConstArgs& a, const unsigned long long* ctx_dmin_inv, const unsigned long long* ctx_dmax,
                                         PlanHeader* hdr) {
@@ -2958,6 +2964,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   ca.key_sbits = key_sbits;
   ca.with_key_width = n_ctx <= kFoldCtx ? 1u : 0u;       /* few contexts: the last block to finish finds the key width */
   ca.arrival_order = arrival_order ? 1u : 0u; ca.win_hist = win_hist ? 1u : 0u; ca.force_scan = (mode & PARD_MODE_SCAN) ? 1u : 0u;
+  /* known paths: the paths' sums are written down beside the constants, in the survivors' scratch, where
+   * they fit (queues of 32 requests on average); else blocks work them out again (stage_paths) */
+  ca.path_sums = (mode & PARD_MODE_PATH_MASK) && n >= 2ull * kMaskPaths * L.n_seg ? (long long*)kept_tmp : nullptr;
   const uint32_t const_blocks = n > 0 && L.n_seg <= kFoldSegs && ca.with_key_width ? n_ctx : 0u;
   mark();
   if (n > 0) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_blocks, ca, sms, stream);
@@ -3021,7 +3030,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     pa.hdr = hdr; pa.buf_a = buf_a; pa.buf_b = buf_b;
     pa.n = n32; pa.ibits = ibits; pa.n_seg = L.n_seg; pa.mode = mode;
     pa.ktab = ktab; pa.seg_off = seg_off; pa.req = req4; pa.arrivals = d_arrivals;
-    pa.pipes = pipe_table; pa.n_pipelines = n_pipelines; pa.st = *state;
+    pa.pipes = pipe_table; pa.n_pipelines = n_pipelines; pa.st = *state; pa.path_sums = ca.path_sums;
     mark();
     rc = decide_by_walk(pa);
     if (rc != PARD_OK) return rc;

@@ -108,7 +108,8 @@ __device__ __forceinline__ unsigned long long magic64(unsigned long long d) {
  * of range.  Bound by dependent loads (pipeline -> profile offsets -> durations; slot -> path ->
  * durations): with the durations of all stages fetched side by side first, a path costs one load
  * per stage instead of a chain of three.  One warp per queue that walked its paths on its own took
- * 10 us for 16 queues and 37 us for 32,768. */
+ * 10 us for 16 queues and 37 us for 32,768.  sums: the ctx's rows of PolicyArgs::path_sums, or null. */
+constexpr int kMaskPaths = 16;                     /* bits of pard_request_t.flags: paths of a stage that a request can name */
 constexpr int kConstThreads = 64;                  /* k_seg_const's blocks; any number of threads will do */
 struct CtxScratch {
   long long delay[PARD_MAX_STAGES];                /* q_i + d_i(B_i), -1: out of range */
@@ -120,7 +121,7 @@ __device__ __forceinline__ unsigned long long magic64(unsigned long long d);
 
 __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n_pipelines, const pard_queue_state_t& st, uint32_t c,
                                               unsigned long long dmin, unsigned long long dmax, PardSegConst* K_out,
-                                              CtxScratch& sc) {
+                                              CtxScratch& sc, long long* sums = nullptr) {
   const uint32_t S = (uint32_t)st.stage_stride, tid = threadIdx.x, nt = blockDim.x;
   const int32_t pi = st.d_pipeline_of_ctx ? st.d_pipeline_of_ctx[c] : 0;
   const PardPipeDev* p = nullptr;
@@ -155,12 +156,16 @@ __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n
       if (sc.slot_off[mid] <= s) lo = mid; else hi = mid;
     }
     atomicMax(&sc.lsub[lo], (unsigned long long)acc);      /* maximum over the stage's paths; a sink has none: 0 */
+    const int32_t j = s - sc.slot_off[lo];
+    if (sums && j < kMaskPaths) sums[lo * kMaskPaths + j] = acc;
   }
   __syncthreads();
   for (uint32_t k = tid; k < S; k += nt) {
     PardSegConst out;
     out.A = 0; out.A_rel = 0; out.d = 1; out.cap = 1; out.d_magic = 0; out.cap_magic = 0;
     out.narrow = 0; out.lsub = 0; out.dsum = 1;
+    if (sums && k < stages)                        /* paths the stage does not have */
+      for (int32_t j = (k + 1 < stages ? sc.slot_off[k + 1] : n_slots) - sc.slot_off[k]; j < kMaskPaths; ++j) sums[k * kMaskPaths + j] = -1;
     if (p && k >= stages) {
       out.narrow = kSegNoStage;                    /* no such stage: a request found in this queue is an input error */
     } else if (p) {
@@ -368,6 +373,7 @@ struct PolicyArgs {
   long long* out_est;
   uint32_t* out_perm;
   uint32_t* out_kept_idx;
+  const long long* path_sums;     /* [n_seg][kMaskPaths] Eq. 3 along every path a request can name, -1: no such path; or null */
   const uint32_t* kept_base;      /* [n_seg] output offset of every queue's survivors, known after the walk */
   uint32_t* seg_kept;
 };

@@ -32,7 +32,6 @@ constexpr int kPolThreads = 128;
 constexpr int kPolItems = 8;
 constexpr int kPolTile = kPolThreads * kPolItems;
 constexpr int kStageSegs = 16;           /* queues whose path sums a block keeps in shared memory */
-constexpr int kMaskPaths = 16;           /* bits of pard_request_t.flags */
 
 struct SortedView {
   const unsigned long long* src;
@@ -130,6 +129,24 @@ __device__ __noinline__ long long masked_lsub(const PolicyArgs& a, const StagedP
   return best;
 }
 
+/* The same from the sums written down beside the queue's constants. */
+__device__ __forceinline__ long long masked_lsub_at_hand(const PolicyArgs& a, uint32_t seg, uint32_t flags, long long lsub) {
+  const long long* t = a.path_sums + (size_t)seg * kMaskPaths;
+  long long best = -1;
+  for (uint32_t m = flags; m; m &= m - 1) {
+    const long long v = __ldg(t + __ffs((int)m) - 1);
+    best = v > best ? v : best;
+  }
+  if (best >= 0) return best;
+  if (__ldg(t) >= 0) set_status(a.hdr, PARD_EDATA);      /* the mask names no path of this stage (a sink has none) */
+  return lsub;
+}
+
+/* How the kernels of one request each get at its downstream estimate: all paths, as in the constants;
+ * by its mask, path sums worked out by the block; by its mask, path sums at hand.  (Working them out is
+ * a chain of dependent loads per path and block: a million requests with known paths, 27 -> 14 us for the rounds and 32 -> 19 us for the estimates.) */
+enum { kAllPaths, kMaskStaged, kMaskAtHand };
+
 /* number of batch rounds b for which a request still fits, b < v: Nexus tests "base + b*d + d <= D" */
 __device__ __forceinline__ uint32_t rounds_fit(long long X, unsigned long long magic, const PardSegConst& K) {
   if (X < 0) return 0;
@@ -143,18 +160,19 @@ __device__ __forceinline__ uint32_t rounds_fit(long long X, unsigned long long m
  * the queue's constants stays in registers while a thread's requests are of one queue, which they
  * mostly are: bound by instructions otherwise (2^24 requests under the window scan: 111 us with the
  * table entry read for every request). */
-/* (Without masks the kernels of this file are kept to 64 registers: 32 warps per multiprocessor; the
- * masked estimate is a call that costs more.) */
-template <bool MASK>
-__global__ void __launch_bounds__(kPolThreads, MASK ? 5 : 8)
+/* (The kernels of this file are kept to 64 registers, 32 warps per multiprocessor, but for those that
+ * work out path sums.) */
+template <int MASK>
+__global__ void __launch_bounds__(kPolThreads, MASK == kMaskStaged ? 5 : 8)
 k_policy_terms(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
-  __shared__ StagedPaths sp;
+  __shared__ __align__(16) unsigned char sp_raw[MASK == kMaskStaged ? sizeof(StagedPaths) : 16];
+  StagedPaths& sp = *reinterpret_cast<StagedPaths*>(sp_raw);
   if (a.hdr->wide || a.hdr->aborted) return;
   const SortedView v = sorted_view(a);
   const bool lookup = a.hdr->lookup != 0;
   const uint64_t tile0 = (uint64_t)blockIdx.x * kPolTile;
-  if (MASK) stage_paths(a, v, tile0, sp);
+  if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
   constexpr int kUn = 4;                           /* elements, then their records, requested together */
   uint32_t cur = 0xffffffffu;
   long long from = 0;                              /* deadline - A = offset (or deadline) - from, or from - offset */
@@ -210,7 +228,7 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
           X = ar.arrive_us + share + K.d - (K.A - K.lsub);
         }
       }
-      if (MASK && flags[u]) X += K.lsub - masked_lsub(a, sp, seg, flags[u], K);
+      if (MASK && flags[u]) X += K.lsub - (MASK == kMaskAtHand ? masked_lsub_at_hand(a, seg, flags[u], K.lsub) : masked_lsub(a, sp, seg, flags[u], K));
       v.T[j] = rounds_fit(X, magic, K);
     }
   }
@@ -559,20 +577,21 @@ k_policy_walk(const __grid_constant__ PolicyArgs a) {
  * queue's rounds for every 128th request was a chain of up to 120 dependent loads: 2^24 requests in
  * queues of 2^15 rounds, 130 us.)  Its place among the survivors is, for Nexus, given by its window, else the kept requests
  * ahead of it: those ahead of the tile (a.tile_x) and, by ballots, those inside it. */
-template <bool MASK>
-__global__ void __launch_bounds__(kPolThreads, MASK ? 5 : 8)
+template <int MASK>
+__global__ void __launch_bounds__(kPolThreads, MASK == kMaskStaged ? 5 : 8)
 k_policy_emit(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   constexpr int kWarps = kPolThreads / 32, kRows = kPolItems * kWarps;
   static_assert(kRows == 32, "one warp scans the rows");
-  __shared__ StagedPaths sp;
+  __shared__ __align__(16) unsigned char sp_raw[MASK == kMaskStaged ? sizeof(StagedPaths) : 16];
+  StagedPaths& sp = *reinterpret_cast<StagedPaths*>(sp_raw);
   __shared__ uint32_t s_keep[kRows], s_before[kRows + 1];
   if (a.hdr->wide || a.hdr->aborted) return;
   const SortedView v = sorted_view(a);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile0 = blockIdx.x * kPolTile;
   const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
-  if (MASK) stage_paths(a, v, tile0, sp);
+  if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
   unsigned long long e[kPolItems];
   uint32_t t[kPolItems], round[kPolItems], flags[kPolItems];
 #pragma unroll
@@ -683,7 +702,10 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
     }
     const uint32_t keep = (keepbits >> i) & 1u;
     long long A = A0;
-    if (MASK && flags[i] && d) A += masked_lsub(a, sp, seg, flags[i], a.ktab[seg]) - a.ktab[seg].lsub;
+    if (MASK && flags[i] && d) {
+      const PardSegConst& K = a.ktab[seg];
+      A += (MASK == kMaskAtHand ? masked_lsub_at_hand(a, seg, flags[i], K.lsub) : masked_lsub(a, sp, seg, flags[i], K)) - K.lsub;
+    }
     if (a.out_keep) a.out_keep[j] = (uint8_t)keep;
     if (a.out_est) a.out_est[j] = A + (long long)round[i] * d;
     if (a.out_perm) a.out_perm[j] = idx;
@@ -704,7 +726,8 @@ namespace pard_plan_detail {
 int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
   static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
-  launch_pdl(a.mode & PARD_MODE_PATH_MASK ? k_policy_terms<true> : k_policy_terms<false>, tiles, kPolThreads, 0, stream, a);
+  launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
+             tiles, kPolThreads, 0, stream, a);
   if (a.n / a.n_seg >= kWalkLong)
     launch_pdl(k_policy_walk<kWalkWarps>, a.n_seg, kWalkWarps * 32, 0, stream, a);
   else
@@ -714,7 +737,8 @@ int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
 
 int launch_policy_emit(const PolicyArgs& a, cudaStream_t stream) {
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
-  launch_pdl(a.mode & PARD_MODE_PATH_MASK ? k_policy_emit<true> : k_policy_emit<false>, tiles, kPolThreads, 0, stream, a);
+  launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_emit<kAllPaths> : a.path_sums ? k_policy_emit<kMaskAtHand> : k_policy_emit<kMaskStaged>,
+             tiles, kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
 }
 

@@ -159,3 +159,19 @@ def test_packing_at_the_widths_of_its_words(span, n_ctx):
     wl.requests["deadline_us"][:2] = 1000, 1000 + span
     for mode in (0, pb.PARD_MODE_GROUPED):
         check(wl, mode)
+
+
+# ---- known paths: path sums at hand from 32 requests per queue on average on, else worked out by blocks ---
+@pytest.mark.parametrize("off", [-1, 0, 1, 30_000])
+@pytest.mark.parametrize("n_ctx", [1, 40])
+def test_known_paths_with_sums_at_hand_and_without(off, n_ctx):
+    from tests.test_policy_parity_gpu import draw_masks
+    rng = np.random.default_rng(n_ctx)
+    edges = [(0, 1), (0, 2), (1, 3), (2, 3), (3, 4), (3, 5)]      # the first stage has four paths
+    p = util.pipeline(edges, 6, list(rng.integers(5, 40, size=6)), bmax=4)
+    n = 32 * 6 * n_ctx + off
+    st = util.state(n_ctx, 6, inputs.n_slots(p), 1000, 2, w=rng.integers(0, 50, size=(n_ctx, inputs.n_slots(p))))
+    r = util.requests(1000 + rng.integers(0, 3000, size=n), rng.integers(0, 6, size=n), rng.integers(0, n_ctx, size=n))
+    wl = inputs.Workload("paths", [p], r, st, n_ctx)
+    draw_masks(wl, rng)
+    check(wl, pb.PARD_MODE_PATH_MASK)
