@@ -2999,7 +2999,10 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   }
   /* passes with a launch of their own, then the rest in one kernel (see k_sort_rest) */
   const uint32_t sort_tiles = ctx_sort ? L.ctx_tiles : L.sort_tiles;
-  const uint32_t max_passes = ctx_sort ? std::min<uint32_t>(kMaxPasses, (key_sbits + 60 + 7) / 8) : L.max_passes;
+  /* the passes that the widest possible key needs; in arrival order the key is the queue id alone (see
+   * set_key_width), so that no launch turns out empty (three of them, 11 us a call at 2^24) */
+  const uint32_t max_passes = arrival_order ? (key_sbits + 7) / 8
+                            : ctx_sort ? std::min<uint32_t>(kMaxPasses, (key_sbits + 60 + 7) / 8) : L.max_passes;
   const bool small = L.small_tiles && !ctx_sort;
   const uint32_t own_passes = small || local_cand ? 0u : std::min(kOwnPasses, max_passes);
   const uint32_t rest_grid = std::min<uint32_t>(sort_tiles, 2u * (uint32_t)sms);
