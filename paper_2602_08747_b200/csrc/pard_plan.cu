@@ -754,7 +754,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
  * at queue position r in window b then has
  *     min_{t<r}(u_t - t) = min(E[b], u(b) - (r - 1) if r > P[b])
  * with no reference to any other request.  P comes from a search in the sorted
- * elements (one warp per window), E and the raw-mode kept counts Kp from a
+ * elements (k_windows) or a count while they are packed, E and the raw-mode kept counts Kp from a
  * per-queue prefix pass over the windows.  Queues with more than kWinMaxPerSeg
  * windows, or more windows in total than the table holds, make the call fall
  * back to the scan kernels (same results). */
@@ -1888,7 +1888,7 @@ __device__ void kept_scan_block(const uint32_t* seg_kept, uint32_t n_seg, uint32
  * queue are counted by a segmented exclusive prefix-sum.  Either way the
  * number k_r of kept requests ahead in the own queue is known per request, and
  * a kept request's index goes to kept_tmp[first position of its queue + k_r]:
- * every queue's survivors end up contiguous, k_kept_move packs the queues. */
+ * every queue's survivors end up contiguous, kept_move_jobs packs the queues. */
 template <bool RAW>
 __device__ void decide_tiles(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a,
          const unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t ibits,
@@ -2990,8 +2990,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                (uint32_t*)(ws + L.hist_ctx), ctx_tiles);
   } else if (n > 0 && !local_sure) {             /* returns at once when the blocks above did the work */
     /* every block adds its digit counts to the call's, up to 256 additions per pass: the fewer blocks the
-     * better, down to two per multiprocessor (a million requests with 1,184 blocks: 7 us more) */
-    const uint64_t blocks = std::min<uint64_t>(std::max<uint64_t>(n / 4096, 2ull * sms), 8ull * sms);
+     * better, down to two per multiprocessor and up to the four that are resident (a million requests with 1,184
+     * blocks: 7 us more; 2^24: 3 us more) */
+    const uint64_t blocks = std::min<uint64_t>(std::max<uint64_t>(n / 4096, 2ull * sms), 4ull * sms);
     const uint32_t grid = (uint32_t)std::min<uint64_t>((n + 255) / 256, blocks);
     launch_pdl(win_hist ? k_pack<true> : k_pack<false>, grid, 256, 0, stream, req4, n32, n_ctx, S, ctx_dmin, ctx_dmax,
                state->d_priority, ibits, hdr, buf_a, hist, local_cand, (const PardSegConst*)ktab, (const uint32_t*)win_off,

@@ -31,7 +31,7 @@ constexpr int kLookGroup = 16;                     /* tiles whose counts are add
 constexpr int kDecThreads = 128;                   /* small blocks: a short tail when the grid drains (measured against 64 and 256) */
 constexpr int kDecItems = 8;
 constexpr int kDecTile = kDecThreads * kDecItems;
-constexpr int kCompactChunk = 1024;                /* indices moved by one warp of k_kept_move */
+constexpr int kCompactChunk = 1024;                /* indices moved by one warp of kept_move_jobs */
 constexpr int kLookBatch = 8;                      /* earlier tiles inspected per round trip in the sort */
 
 /* look-back word of the sort: [31:30] state, [29:0] count */
