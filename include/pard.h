@@ -177,7 +177,8 @@ typedef struct pard_plan_out {
                                    for that long makes the call return PARD_ETIMEOUT   */
 #define PARD_MODE_TEST_STALL 8u /* testing aid for the bounded device-side waits: the
                                    first tile of the first sort pass withholds the word
-                                   later tiles wait for, and the first block of the scan
+                                   later tiles wait for (and is never counted as finished,
+                                   which the next pass waits for), and the first block of the scan
                                    path (PARD_MODE_SCAN) never arrives at the first of its
                                    grid-wide meeting points; the waits run out (after a
                                    fraction of a second) and the call returns

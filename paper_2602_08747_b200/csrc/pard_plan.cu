@@ -937,6 +937,33 @@ __device__ bool grid_barrier(PlanHeader* hdr, uint32_t* bar, uint32_t members, b
   return s_ok != 0;
 }
 
+/* Hands in the `mine` pieces of work that this block has finished and waits until all `target` of them have
+ * been handed in to `word` (from zero); what their blocks wrote before is visible to this block afterwards.
+ * A block comes here when it has found nothing left to take, so the pieces outstanding are with blocks that
+ * run already: the wait needs no block that has yet to be placed.  Bounded all the same: about half a
+ * second, then PARD_ETIMEOUT and false in every block. */
+__device__ bool finish_pieces(PlanHeader* hdr, uint32_t* word, uint32_t mine, uint32_t target) {
+  __shared__ uint32_t s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (mine) {
+      __threadfence();
+      atomicAdd(word, mine);
+    }
+    uint32_t spins = 0;
+    bool ok = true;
+    while (ld_relaxed(word) < target) {     /* up to about half a second: other work may hold multiprocessors for a while */
+      if (++spins > 8 * kSpinLimit || ((spins & 15) == 0 && ld_relaxed(&hdr->aborted))) { ok = false; break; }
+      __nanosleep(200);
+    }
+    if (!ok) set_aborted(hdr);
+    __threadfence();
+    s_ok = ok ? 1u : 0u;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
 struct SortSmem {
   unsigned long long keys[kSortTile];
   uint32_t slot[kSortThreads / 32][kBins];    /* counts, then next free tile-local slot per (warp, digit) */
@@ -946,6 +973,7 @@ struct SortSmem {
   uint32_t scan[2][kSortThreads / 32];
   uint32_t tile;
   uint32_t abort;
+  uint32_t done;                              /* tiles of the pass at hand that this block has finished */
   uint32_t ctx, lo_tile, base, limit, first;   /* the tile's ctx and range when passes stay inside the contexts */
 };
 
@@ -1267,6 +1295,7 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   }
   if (!PERSIST) return true;
   __syncthreads();                                     /* the tile buffer and the tables are reused */
+  if (tid == 0 && !(stall && tile == 0)) ++S.done;
   }
 }
 
@@ -1293,10 +1322,13 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
                                 stall, ct, 0u);
 }
 
-/* All passes from `pass` on, by a grid that is resident as a whole and meets between them (bounded
- * waits as in grid_barrier).  How many passes a key needs is only known on the device, and a pass
- * that finds nothing to do still costs a launch: 2.5 to 4.5 us each, up to seven per call.  At
- * 2^24 elements a resident grid takes 9 us more per pass than one block per tile (the blocks' loads
+/* All passes from `pass` on, by one grid.  How many passes a key needs is only known on the device, and a
+ * pass that finds nothing to do still costs a launch: 2.5 to 4.5 us each, up to seven per call.  A block
+ * takes tiles by ticket until the pass has none left, hands in how many it has finished, and begins the
+ * next pass when all tiles have been handed in.  It never waits for a block
+ * that has not been placed: however few of the grid's blocks run at a time -- other streams may hold the
+ * multiprocessors, another call's grid of this kind among them -- those that run finish the pass.
+ * At 2^24 elements such a grid takes 9 us more per pass than one block per tile (the blocks' loads
  * no longer start under the write-out of others), so the passes that large calls usually need keep
  * launches of their own.  Calls of one or two rounds of small tiles (SMALL) do all passes here,
  * with tiles sized so that every block takes the same number of them. */
@@ -1309,18 +1341,20 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  const uint32_t members = gridDim.x - (wc.on ? 1u : 0u);
   if (hdr->aborted || sort_is_local(hdr, local_candidate)) return;
   const uint32_t npass = hdr->npass;
+  const uint32_t tile_size = SMALL ? 256u * ((geometry & 255u) + (geometry >> 8)) : (uint32_t)kSortTile;
+  const uint32_t tiles = CTX ? ct.tile_first[ct.n_ctx] : (uint32_t)(((uint64_t)n + tile_size - 1) / tile_size);
   for (uint32_t p = pass; p < npass; ++p) {
     SortSmem& S = *reinterpret_cast<SortSmem*>(smem_raw);
+    if (threadIdx.x == 0) S.done = 0;
     uint32_t* now = lookback + (p & 1) * lb_words;
     uint32_t* next = lookback + ((p + 1) & 1) * lb_words;
     bool go;
     if constexpr (SMALL) go = sort_tiles<true, CTX, true>(S, p, hdr, buf_a, buf_b, hist, now, next, n, ibits, p == 0 ? stall : 0u, ct, geometry);
     else go = sort_tiles_resident<CTX>(S, p, hdr, buf_a, buf_b, hist, now, next, n, ibits, p == 0 ? stall : 0u, ct);
     if (!go) return;
-    if (p + 1 < npass && !grid_barrier(hdr, &hdr->sort_bar[p], members)) return;
+    if (p + 1 < npass && !finish_pieces(hdr, &hdr->sort_bar[p], S.done, tiles)) return;
   }
 }
 

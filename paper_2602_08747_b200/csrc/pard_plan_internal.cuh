@@ -60,7 +60,7 @@ struct PlanHeader {
   uint32_t time_steps_back;   /* 1: some request's deadline lies before its predecessor's */
   uint32_t pair_steps_back;   /* 1: some request's (ctx, deadline) lies before its predecessor's */
   uint32_t lookup;            /* 1: the elements hold no deadline: it has to be looked up in the request array */
-  uint32_t sort_bar[kMaxPasses]; /* blocks of k_sort_rest that have finished each of its passes */
+  uint32_t sort_bar[kMaxPasses]; /* tiles of each of k_sort_rest's passes that are finished */
   uint32_t pad[64 - 24 - kMaxPasses - (kMaxPasses + 1)];
 };
 static_assert(sizeof(PlanHeader) == 256, "header is 256 bytes");

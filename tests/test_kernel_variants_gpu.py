@@ -175,3 +175,36 @@ def test_known_paths_with_sums_at_hand_and_without(off, n_ctx):
     wl = inputs.Workload("paths", [p], r, st, n_ctx)
     draw_masks(wl, rng)
     check(wl, pb.PARD_MODE_PATH_MASK)
+
+
+# ---- calls that run at the same time: every block waits for work in flight only, never for a block to be placed ---
+@pytest.mark.parametrize("mode", [0])
+def test_calls_at_the_same_time(mode):
+    import torch
+    works = [several_ctx(3, [450_000] * 3, seed=1, sort=False, mix=True, span=3_000_000),      # tiles fill the device: every pass in one kernel
+             several_ctx(3, [430_001] * 3, seed=2, sort=False, mix=True, span=3_000_000),
+             several_ctx(2, [1_400_000] * 2, seed=3, sort=False, mix=True, span=1 << 27),       # passes of their own, then the rest
+             several_ctx(2, [700, 300], seed=4, sort=False, mix=True, span=1 << 20)]            # one tile
+    calls = []
+    for k, wl in enumerate(works):
+        S = wl.state.stage_stride
+        calls.append((wl, [pb.pard_load_pipeline(p) for p in wl.pipelines], pb.device_requests(wl.requests, "cuda:0"),
+                      pb.device_state(wl.state, "cuda:0"), pb.alloc_out(wl.n, wl.n_ctx * S, "cuda:0"),
+                      pb.alloc_workspace(pb.pard_plan_workspace_bytes(wl.n, wl.n_ctx, S), "cuda:0"),
+                      torch.cuda.Stream(priority=-(k & 1))))
+    torch.cuda.synchronize()
+    for _ in range(8):
+        for wl, pipes, req, state, out, ws, stream in calls:
+            pb.pard_plan(pipes, req, wl.n, state, wl.n_ctx, mode | pb.PARD_MODE_NOWAIT, out, ws, stream=stream.cuda_stream)
+    for wl, pipes, req, state, out, ws, stream in calls:
+        assert pb.pard_plan_status(ws, stream=stream.cuda_stream) == 0
+        got, want = pb.out_to_numpy(out, wl.n), oracle.plan(wl.pipelines, wl.requests, wl.state, wl.n_ctx)
+        for key in ("seg_offsets", "perm", "keep", "est_us", "n_kept", "kept_idx", "seg_kept"):
+            assert np.array_equal(got[key], want[key]), (wl.n, key)
+
+
+def test_wait_between_the_passes_runs_out_and_is_reported():
+    wl = several_ctx(2, [700, 300], sort=False, mix=True, span=1 << 20)      # one tile, several passes: no look-back to run out first
+    rc, _ = run_library(wl, pb.PARD_MODE_TEST_STALL, check=False)
+    assert rc == pb.PARD_ETIMEOUT
+    check(wl)
