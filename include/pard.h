@@ -171,17 +171,16 @@ typedef struct pard_plan_out {
                                    batch-window tables would do (same results; the scan
                                    is otherwise the fallback for queues with thousands
                                    of batch windows).  The scan path is one kernel whose
-                                   blocks (two per multiprocessor) wait for each other
-                                   between its steps, each wait bounded at about half a
-                                   second: a GPU that other streams keep completely full
-                                   for that long makes the call return PARD_ETIMEOUT   */
+                                   blocks wait between its steps for the work of other
+                                   running blocks, each wait bounded at about half a
+                                   second                                             */
 #define PARD_MODE_TEST_STALL 8u /* testing aid for the bounded device-side waits: the
                                    first tile of the first sort pass withholds the word
                                    later tiles wait for (and is never counted as finished,
-                                   which the next pass waits for), and the first block of the scan
-                                   path (PARD_MODE_SCAN) never arrives at the first of its
-                                   grid-wide meeting points; the waits run out (after a
-                                   fraction of a second) and the call returns
+                                   which the next pass waits for), and the first tiles of the scan
+                                   path's first step (PARD_MODE_SCAN) are never counted as
+                                   finished, which its next step waits for; the waits run
+                                   out (after a fraction of a second) and the call returns
                                    PARD_ETIMEOUT with unspecified outputs; the CUDA
                                    context stays usable.  Calls that the library sorts
                                    block by block (requests grouped by ctx, no ctx above

@@ -127,18 +127,19 @@ __device__ __forceinline__ bool sort_is_local(const PlanHeader* hdr, uint32_t ca
   return candidate && !hdr->unsorted && !hdr->ctx_too_big && !hdr->wide;
 }
 
-/* True in every thread of exactly one block: the one whose arrival at `counter` is the last of
- * the grid.  Every thread's earlier global writes are visible to that block afterwards. */
-__device__ __forceinline__ bool last_block_done(uint32_t* counter) {
+/* True in every thread of exactly one block: the one whose `mine` arrivals at `counter` complete `all`.
+ * Every thread's earlier global writes are visible to that block afterwards. */
+__device__ __forceinline__ bool last_arrival(uint32_t* counter, uint32_t mine, uint32_t all) {
   __shared__ uint32_t s_last;
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1 ? 1u : 0u;
+  if (threadIdx.x == 0) s_last = mine && atomicAdd(counter, mine) + mine == all ? 1u : 0u;
   __syncthreads();
   const bool last = s_last != 0;
   if (last) __threadfence();
   return last;
 }
+__device__ __forceinline__ bool last_block_done(uint32_t* counter) { return last_arrival(counter, 1u, gridDim.x); }
 
 /* Clears the part of the scratch that must start at zero.  A kernel rather than a memset: it is
  * launched like every other kernel of the call, so its blocks are placed while the previous
@@ -914,32 +915,9 @@ __device__ __noinline__ void win_from_counts(PlanHeader* hdr, const WinCountArgs
  *   5. the buffer is written out, run by run, to the digit's global range.
  * Large tiles keep the number of tiles in flight, and with it the depth of the
  * look-back, small. */
-/* The grid's `members` blocks (resident as a whole) meet: every block's writes before are visible to every block
- * after.  `bar` counts arrivals from zero.  Bounded: about half a second, then PARD_ETIMEOUT and false
- * in every block. */
-__device__ bool grid_barrier(PlanHeader* hdr, uint32_t* bar, uint32_t members, bool withhold = false) {
-  __shared__ uint32_t s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (!withhold) atomicAdd(bar, 1u);      /* (testing aid: a block that never arrives) */
-    uint32_t spins = 0;
-    bool ok = true;
-    while (ld_relaxed(bar) < members) {     /* up to about half a second: other work may hold multiprocessors for a while */
-      if (++spins > 8 * kSpinLimit || hdr->aborted) { ok = false; break; }
-      __nanosleep(200);
-    }
-    if (!ok) set_aborted(hdr);
-    __threadfence();
-    s_ok = ok ? 1u : 0u;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
 /* Hands in the `mine` pieces of work that this block has finished and waits until all `target` of them have
- * been handed in to `word` (from zero); what their blocks wrote before is visible to this block afterwards.
- * A block comes here when it has found nothing left to take, so the pieces outstanding are with blocks that
+ * been handed in to `word` (from zero; k_scan_path: until a flag is set); what their blocks wrote before is
+ * visible to this block afterwards.  A block comes here when it has found nothing left to take, so the pieces outstanding are with blocks that
  * run already: the wait needs no block that has yet to be placed.  Bounded all the same: about half a
  * second, then PARD_ETIMEOUT and false in every block. */
 __device__ bool finish_pieces(PlanHeader* hdr, uint32_t* word, uint32_t mine, uint32_t target) {
@@ -1793,21 +1771,18 @@ __device__ void tile_scan_block(const unsigned long long* tile_agg, uint32_t n_t
 }
 
 /* Tile aggregates: the segmented reduction over each tile of kDecTile sorted
- * elements.  Tiles are independent; the block that finishes last scans the
- * aggregates into the value carried into every tile, so that the decision
- * kernel never waits on another block. */
+ * elements, for tiles [first, end).  Tiles are independent. */
 template <bool RAW>
 __device__ void tile_agg_tiles(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a,
                                const unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t ibits,
                                const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off,
-                               unsigned long long* __restrict__ tile_agg) {
+                               unsigned long long* __restrict__ tile_agg, uint32_t first, uint32_t end) {
   constexpr int WARPS = kDecThreads / 32;
   __shared__ int32_t s_wm[WARPS];
   __shared__ uint32_t s_wh[WARPS];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const TileCtx T = make_tile_ctx(hdr, buf_a, buf_b, n, ibits, ktab, seg_off);
-  const uint32_t n_tiles = (n + kDecTile - 1) / kDecTile;
-  for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+  for (uint32_t tile = first; tile < end; ++tile) {
     const uint64_t base = (uint64_t)tile * kDecTile + (uint64_t)tid * kDecItems;
     unsigned long long e[kDecItems];
     uint32_t idx[kDecItems], u[kDecItems], r[kDecItems], lheadbits, sstart, seg_first;
@@ -1914,8 +1889,8 @@ __device__ void kept_scan_block(const uint32_t* seg_kept, uint32_t n_seg, uint32
   if (threadIdx.x == 0 && out_n_kept) *out_n_kept = s_ca;
 }
 
-/* Decision pass; one tile of kDecTile sorted elements per block, a thread owns
- * kDecItems consecutive elements.
+/* Decision pass over tiles [first, end) of kDecTile sorted elements; a thread owns kDecItems consecutive
+ * elements of a tile.
  *
  * Admitted mode: c_r = min(r, r-1 + min_{t<r}(u_t - t)) by a segmented
  * exclusive prefix-min; raw mode: c_r = r, and the kept requests ahead in the
@@ -1929,14 +1904,13 @@ __device__ void decide_tiles(const PlanHeader* __restrict__ hdr, const unsigned 
          const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off,
          const uint32_t* __restrict__ win_off, const int32_t* __restrict__ carry,
          uint8_t* __restrict__ out_keep, long long* __restrict__ out_est, uint32_t* __restrict__ out_perm,
-         uint32_t* __restrict__ kept_tmp, uint32_t* __restrict__ seg_kept) {
+         uint32_t* __restrict__ kept_tmp, uint32_t* __restrict__ seg_kept, uint32_t first, uint32_t end) {
   constexpr int WARPS = kDecThreads / 32;
   __shared__ int32_t s_wm[WARPS];
   __shared__ uint32_t s_wh[WARPS];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const TileCtx T = make_tile_ctx(hdr, buf_a, buf_b, n, ibits, ktab, seg_off);
-  const uint32_t n_tiles = (n + kDecTile - 1) / kDecTile;
-  for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+  for (uint32_t tile = first; tile < end; ++tile) {
   const uint64_t base = (uint64_t)tile * kDecTile + (uint64_t)tid * kDecItems;
   const bool full = base + kDecItems <= n;
   const int32_t tile_carry = __ldcg(&carry[tile]);       /* written by another block of this kernel */
@@ -2514,12 +2488,39 @@ __device__ __forceinline__ void kept_move_jobs(const uint32_t* __restrict__ kept
 /* The decision by scanning, from the sorted elements to the packed survivors, as ONE kernel: the
  * fallback for calls whose queues have too many batch windows for the tables (and what
  * PARD_MODE_SCAN asks for).  Launched on every call; returns at once when the tables did the
- * work.  Its five steps -- tile aggregates, their scan (block 0), the decision, the queues' kept
- * counts into output offsets (block 0), the packing of the survivors -- need the whole grid to
- * have finished the step before: the grid is small enough to be resident as a whole (at most two
- * blocks of 128 threads per multiprocessor), and its blocks meet at counters in the workspace
- * header, each wait bounded like the sort's (PARD_ETIMEOUT, every block gives up, nothing hangs;
- * the bound only bites when other streams keep the multiprocessors full for that long). */
+ * work.  Five steps: tile aggregates, their scan, the decision, the queues' kept counts into output
+ * offsets, the packing of the survivors.  The tiles of a step are taken by ticket, a run of them at a
+ * time, and every block hands in how many runs it has done; the block that completes the step also does
+ * the one-block step behind it and then sets a flag, which the others wait for before they go on.  So a wait
+ * is only ever for blocks that run already, and those that run finish the call, however few of the grid
+ * are placed at a time; each wait is bounded all the same (PARD_ETIMEOUT, every block gives up, nothing
+ * hangs). */
+constexpr uint32_t kScanRuns = 4;                /* runs of tiles per block of the grid: blocks that start late find less to do */
+/* The block's share of a step: work(first tile, end) for every run it gets hold of, the next ticket fetched
+ * while a run is worked on.  True in the block that completes the step.  stall: testing aid, the first run
+ * is never handed in. */
+template <typename Work>
+__device__ __forceinline__ bool scan_step(uint32_t* ticket, uint32_t* done, uint32_t n_tiles, bool stall, Work work) {
+  __shared__ uint32_t s_next;
+  const uint32_t per = (n_tiles + kScanRuns * gridDim.x - 1) / (kScanRuns * gridDim.x), runs = (n_tiles + per - 1) / per;
+  uint32_t mine = 0, next = 0;
+  if (threadIdx.x == 0) s_next = atomicAdd(ticket, 1u);
+  __syncthreads();
+  for (uint32_t t = s_next; t < runs; t = s_next) {
+    if (threadIdx.x == 0) next = atomicAdd(ticket, 1u);
+    work(t * per, min((t + 1) * per, n_tiles));
+    mine += stall && t == 0 ? 0u : 1u;
+    __syncthreads();
+    if (threadIdx.x == 0) s_next = next;
+    __syncthreads();
+  }
+  return last_arrival(done, mine, runs);
+}
+__device__ __forceinline__ void set_flag(uint32_t* word) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) atomicExch(word, 1u);
+}
 template <bool RAW>
 __global__ void __launch_bounds__(kDecThreads, 3)
 k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
@@ -2533,14 +2534,20 @@ k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
   pdl_wait();
   if (hdr->wide || hdr->aborted || !hdr->use_scan) return;
   const uint32_t n_tiles = (n + kDecTile - 1) / kDecTile;
-  tile_agg_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, tile_agg);
-  if (!grid_barrier(hdr, &hdr->bar[0], gridDim.x, stall && blockIdx.x == 0)) return;
-  if (blockIdx.x == 0) tile_scan_block<RAW, kDecThreads>(tile_agg, n_tiles, carry);
-  if (!grid_barrier(hdr, &hdr->bar[1], gridDim.x)) return;
-  decide_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, carry, out_keep, out_est, out_perm, kept_tmp, seg_kept);
-  if (!grid_barrier(hdr, &hdr->bar[2], gridDim.x)) return;
-  if (blockIdx.x == 0) kept_scan_block<kDecThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
-  if (!grid_barrier(hdr, &hdr->bar[3], gridDim.x)) return;
+  if (scan_step(&hdr->scan_ticket[0], &hdr->scan_done[0], n_tiles, stall != 0, [&](uint32_t first, uint32_t end) {
+        tile_agg_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, tile_agg, first, end);
+      })) {
+    tile_scan_block<RAW, kDecThreads>(tile_agg, n_tiles, carry);
+    set_flag(&hdr->scan_flag[0]);
+  }
+  if (!finish_pieces(hdr, &hdr->scan_flag[0], 0u, 1u)) return;
+  if (scan_step(&hdr->scan_ticket[1], &hdr->scan_done[1], n_tiles, false, [&](uint32_t first, uint32_t end) {
+        decide_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, carry, out_keep, out_est, out_perm, kept_tmp, seg_kept, first, end);
+      })) {
+    kept_scan_block<kDecThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
+    set_flag(&hdr->scan_flag[1]);
+  }
+  if (!finish_pieces(hdr, &hdr->scan_flag[1], 0u, 1u)) return;
   if (out_kept_idx) kept_move_jobs(kept_tmp, seg_off, seg_kept, kept_base, chunk_base, n_seg, out_kept_idx);
 }
 

@@ -55,13 +55,15 @@ struct PlanHeader {
   uint32_t unsorted;          /* 1: some request's ctx is smaller than its predecessor's */
   uint32_t ctx_too_big;       /* 1: some ctx holds more requests than one sort tile */
   uint32_t bad_input;         /* 1: PARD_EDATA was found (kept apart from `status`, which holds the first error only) */
-  uint32_t bar[4];            /* blocks of k_scan_path that have reached each of its grid-wide barriers */
+  uint32_t scan_ticket[2];    /* k_scan_path: runs of tiles taken, in the aggregates' step and in the decision's */
+  uint32_t scan_done[2];      /* runs finished */
+  uint32_t scan_flag[2];      /* 1: the one-block step behind it is done */
   uint32_t pshift;            /* low bits of the key that need no pass: the deadline field, when the requests come in its order */
   uint32_t time_steps_back;   /* 1: some request's deadline lies before its predecessor's */
   uint32_t pair_steps_back;   /* 1: some request's (ctx, deadline) lies before its predecessor's */
   uint32_t lookup;            /* 1: the elements hold no deadline: it has to be looked up in the request array */
   uint32_t sort_bar[kMaxPasses]; /* tiles of each of k_sort_rest's passes that are finished */
-  uint32_t pad[64 - 24 - kMaxPasses - (kMaxPasses + 1)];
+  uint32_t pad[64 - 26 - kMaxPasses - (kMaxPasses + 1)];
 };
 static_assert(sizeof(PlanHeader) == 256, "header is 256 bytes");
 

@@ -178,7 +178,7 @@ def test_known_paths_with_sums_at_hand_and_without(off, n_ctx):
 
 
 # ---- calls that run at the same time: every block waits for work in flight only, never for a block to be placed ---
-@pytest.mark.parametrize("mode", [0])
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_SCAN])
 def test_calls_at_the_same_time(mode):
     import torch
     works = [several_ctx(3, [450_000] * 3, seed=1, sort=False, mix=True, span=3_000_000),      # tiles fill the device: every pass in one kernel
