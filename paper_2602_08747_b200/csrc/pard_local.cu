@@ -36,6 +36,7 @@ constexpr int kLocItems = kLocalTile / kLocThreads;      /* rounds of 32 consecu
 static_assert(kLocItems == 16 && kLocItems * kLocThreads == kLocalTile, "16 items per thread");
 constexpr uint32_t kTabEntries = 2048;                   /* window-table entries of one ctx */
 constexpr uint32_t kNoWindow = 0xffffu;                  /* window of a request with deadline < A */
+constexpr uint32_t kNoCtx = 0xffffffffu;
 
 struct Tables {                                          /* 4. to 6., in the room of the sort's counters */
   uint32_t P[kTabEntries];                               /* requests of the queue in earlier windows */
@@ -765,13 +766,15 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   if (single) {                                          /* the only kernel of the call: the header starts here */
     if (tid < sizeof(PlanHeader) / 4) reinterpret_cast<uint32_t*>(hdr)[tid] = 0;
     if (tid == 0) { Sm.ctx = 0; Sm.first = 0; Sm.cnt = a.n; }
-  } else {
-    if (hdr->unsorted || hdr->ctx_too_big) {             /* k_ctx_prep found the promised grouping broken */
-      if (tid == 0 && blockIdx.x == 0) { set_status(hdr, PARD_EDATA); hdr->aborted = 1; }
-      return;
-    }
-    if (tid == 0) {
-      const uint32_t t = atomicAdd(&hdr->ticket[0], 1u);
+  } else if (tid == 0) {
+    /* The promised grouping is broken: found by k_ctx_prep, or (`unsorted`) by a block of this kernel, so
+     * that one thread has to look for the whole block.  (It takes its ticket meanwhile; that nobody will
+     * plan that ctx then does not matter, the waits behind it end with `aborted`.) */
+    const uint32_t broken = ld_relaxed(&hdr->unsorted) | ld_relaxed(&hdr->ctx_too_big), t = atomicAdd(&hdr->ticket[0], 1u);
+    Sm.ctx = kNoCtx;
+    if (broken) {
+      if (blockIdx.x == 0) { set_status(hdr, PARD_EDATA); hdr->aborted = 1; }
+    } else {
       Sm.ctx = t;
       Sm.first = a.ctx_start[t];
       Sm.cnt = a.ctx_start[t + 1] - Sm.first;
@@ -779,6 +782,7 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   }
   if (tid == 0) { Sm.flags = a.st.d_priority ? 4u : 0u; Sm.use_scan = 0; Sm.abort = 0; }
   __syncthreads();
+  if (Sm.ctx == kNoCtx) return;
   const uint32_t c = Sm.ctx, first = Sm.first, cnt = Sm.cnt;
   /* every warp owns `items` rounds of 32 consecutive requests: as few as the ctx needs */
   const int items = (int)((cnt + kLocThreads - 1) / kLocThreads);

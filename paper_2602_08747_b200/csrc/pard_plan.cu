@@ -127,6 +127,13 @@ __device__ __forceinline__ bool sort_is_local(const PlanHeader* hdr, uint32_t ca
   return candidate && !hdr->unsorted && !hdr->ctx_too_big && !hdr->wide;
 }
 
+/* Words of the header that blocks of the running kernel may set (a wait has run out, a ctx is not grouped)
+ * are read by one thread for its whole block: threads that read for themselves could see it change, and a
+ * block whose first warp has left would go on with what that warp was to fetch. */
+__device__ __forceinline__ bool gave_up(const PlanHeader* hdr) {
+  return __syncthreads_or(threadIdx.x == 0 && ld_relaxed(&hdr->aborted)) != 0;
+}
+
 /* True in every thread of exactly one block: the one whose `mine` arrivals at `counter` complete `all`.
  * Every thread's earlier global writes are visible to that block afterwards. */
 __device__ __forceinline__ bool last_arrival(uint32_t* counter, uint32_t mine, uint32_t all) {
@@ -832,7 +839,7 @@ struct WinCountArgs {
   const uint32_t* hist;
 };
 __device__ __noinline__ void win_from_counts(PlanHeader* hdr, const WinCountArgs& a) {
-  if (hdr->wide || hdr->aborted) return;
+  if (hdr->wide) return;
   const uint32_t n_seg = a.n_seg;
   __shared__ uint32_t s_len[kHistSegs], s_kept[kHistSegs];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1098,7 +1105,9 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   const uint32_t n_tiles = (uint32_t)(((uint64_t)n + tile_size - 1) / tile_size);
   for (;;) {
   if (tid == 0) {
-    const uint32_t t = atomicAdd(&hdr->ticket[pass], 1u);
+    const uint32_t given_up = PERSIST ? 0u : __ldcg(&hdr->aborted);     /* (see gave_up; in flight beside the ticket) */
+    uint32_t t = atomicAdd(&hdr->ticket[pass], 1u);
+    if (given_up) t = 0xffffffffu;                       /* behind all tiles */
     S.tile = t;
     S.abort = 0;
     if (CTX) {                                           /* the ctx of the tile: last c with tile_first[c] <= t */
@@ -1121,7 +1130,7 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   uint32_t gh = (!CTX && tid < kBins) ? hist[tid] : 0; /* count of digit tid in the whole array (in the ctx), needed in step 2 */
   __syncthreads();
   const uint32_t tile = S.tile;
-  if (!CTX && PERSIST && tile >= n_tiles) return true;
+  if (!CTX && tile >= n_tiles) return true;
   if (CTX && S.ctx == 0xffffffffu) return true;
   if (CTX && tid < kBins) gh = ct.hist[((size_t)S.ctx * kMaxPasses + pass) * kBins + tid];
   const uint64_t base = CTX ? (uint64_t)S.base : (uint64_t)tile * tile_size;
@@ -1295,7 +1304,7 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  if (pass >= hdr->npass || hdr->aborted || sort_is_local(hdr, local_candidate)) return;
+  if (pass >= hdr->npass || sort_is_local(hdr, local_candidate)) return;
   sort_tiles<false, CTX, false>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
                                 stall, ct, 0u);
 }
@@ -1319,7 +1328,7 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  if (hdr->aborted || sort_is_local(hdr, local_candidate)) return;
+  if (sort_is_local(hdr, local_candidate) || gave_up(hdr)) return;
   const uint32_t npass = hdr->npass;
   const uint32_t tile_size = SMALL ? 256u * ((geometry & 255u) + (geometry >> 8)) : (uint32_t)kSortTile;
   const uint32_t tiles = CTX ? ct.tile_first[ct.n_ctx] : (uint32_t)(((uint64_t)n + tile_size - 1) / tile_size);
@@ -1384,13 +1393,15 @@ k_pack_ctx(const uint4* __restrict__ req, uint32_t S, const unsigned long long* 
            const CtxTiles ct) {
   pdl_wait();
   __shared__ uint32_t s_hist[kMaxPasses * kBins];
-  __shared__ uint32_t s_c, s_base, s_limit;
-  if (hdr->unsorted) {                                   /* k_ctx_ranges found the requests out of ctx order */
-    if (blockIdx.x == 0 && threadIdx.x == 0) { hdr->aborted = 1; set_status(hdr, PARD_EDATA); }
-    return;
-  }
-  if (hdr->wide || hdr->aborted) return;
+  __shared__ uint32_t s_c, s_base, s_limit, s_skip;
   const uint32_t tile = blockIdx.x;
+  if (threadIdx.x == 0) {
+    const bool unsorted = ld_relaxed(&hdr->unsorted) != 0;       /* found out of ctx order, by k_ctx_ranges or a block of this kernel (see gave_up) */
+    if (unsorted && tile == 0) { hdr->aborted = 1; set_status(hdr, PARD_EDATA); }
+    s_skip = unsorted || hdr->wide || ld_relaxed(&hdr->aborted) ? 1u : 0u;
+  }
+  __syncthreads();
+  if (s_skip) return;
   if (threadIdx.x == 0) {
     uint32_t lo = 0, hi = ct.n_ctx;
     while (hi - lo > 1) {
@@ -1497,7 +1508,7 @@ k_sort_local(PlanHeader* __restrict__ hdr, uint32_t candidate, const uint4* __re
   constexpr int WARPS = kSortThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SortSmem& Sm = *reinterpret_cast<SortSmem*>(smem_raw);
-  if (!sort_is_local(hdr, candidate) || hdr->aborted) return;
+  if (!__syncthreads_or(threadIdx.x == 0 && sort_is_local(hdr, candidate))) return;     /* (see gave_up: `unsorted` is set below) */
   const uint32_t c = blockIdx.x;
   const uint32_t first = ctx_start ? ctx_start[c] : 0u;              /* no table: the call has one ctx */
   const uint32_t cnt = ctx_start ? ctx_start[c + 1] - first : n;
@@ -2532,7 +2543,7 @@ k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
             uint32_t* __restrict__ chunk_base, uint32_t* __restrict__ out_seg_kept,
             unsigned long long* __restrict__ out_n_kept, uint32_t* __restrict__ out_kept_idx, uint32_t stall) {
   pdl_wait();
-  if (hdr->wide || hdr->aborted || !hdr->use_scan) return;
+  if (hdr->wide || !hdr->use_scan || gave_up(hdr)) return;
   const uint32_t n_tiles = (n + kDecTile - 1) / kDecTile;
   if (scan_step(&hdr->scan_ticket[0], &hdr->scan_done[0], n_tiles, stall != 0, [&](uint32_t first, uint32_t end) {
         tile_agg_tiles<RAW>(hdr, buf_a, buf_b, n, ibits, ktab, seg_off, tile_agg, first, end);

@@ -208,3 +208,17 @@ def test_wait_between_the_passes_runs_out_and_is_reported():
     rc, _ = run_library(wl, pb.PARD_MODE_TEST_STALL, check=False)
     assert rc == pb.PARD_ETIMEOUT
     check(wl)
+
+
+# ---- requests found out of place by a block of a kernel whose other blocks are still starting ---------------------
+@pytest.mark.parametrize("n_ctx,per", [(900, 2100), (40, 9000)])          # a block per ctx; passes inside the contexts' ranges
+@pytest.mark.parametrize("at", [0, 0.3, 0.9])
+def test_requests_out_of_place_while_blocks_start(n_ctx, per, at):
+    wl = several_ctx(n_ctx, [per] * n_ctx, S=4, m=3)
+    i, j = int(at * n_ctx) * per + per // 2 + 1, n_ctx * per - per // 2           # inside their contexts: the ranges look grouped
+    wl.requests[[i, j]] = wl.requests[[j, i]]
+    for _ in range(5):
+        assert run_library(wl, pb.PARD_MODE_GROUPED, check=False)[0] == pb.PARD_EDATA
+    check(wl)                                                             # legal without the promise
+    wl.requests[[i, j]] = wl.requests[[j, i]]
+    check(wl, pb.PARD_MODE_GROUPED)
