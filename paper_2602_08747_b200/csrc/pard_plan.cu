@@ -2572,7 +2572,9 @@ k_scan_path(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a,
  * order by one more chunk, and the positions it yields are chased back to request indices.
  * The last super-pass leaves the order of the requests; the elements are then rewritten as
  * segment | index (no deadline bits) and the decision is taken by the queue walk, which looks
- * the deadlines up in the request array.  A slow path for legal but extreme inputs. */
+ * the deadlines up in the request array.  A slow path for legal but extreme inputs.
+ * Once a wait of the passes has run out (`aborted`) the elements are no longer positions, and none of
+ * these kernels may follow them. */
 __device__ __forceinline__ uint32_t wide_chunk_bits(const PlanHeader* hdr, uint32_t sbits, uint32_t ibits, uint32_t super) {
   const uint32_t kb = sbits + hdr->dbits, cw = 64 - ibits, lo = super * cw;
   return lo < kb ? min(cw, kb - lo) : 0u;
@@ -2608,6 +2610,7 @@ k_wide_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t 
             unsigned long long* __restrict__ dst, uint32_t* __restrict__ hist) {
   pdl_wait();
   __shared__ uint32_t s_hist[kMaxPasses * kBins];
+  if (hdr->aborted) return;
   const uint32_t bits = wide_chunk_bits(hdr, sbits, ibits, super), npass = (bits + 7) / 8;
   const uint32_t dbits = hdr->dbits, lo = super * (64 - ibits);
   for (uint32_t i = threadIdx.x; i < npass * kBins; i += blockDim.x) s_hist[i] = 0;
@@ -2640,6 +2643,7 @@ k_wide_chase(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
              unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t ibits, uint32_t super,
              const uint32_t* __restrict__ order) {
   pdl_wait();
+  if (hdr->aborted) return;
   const bool odd = hdr->npass & 1;
   const unsigned long long* sorted = odd ? buf_b : buf_a;
   uint32_t* tmp = reinterpret_cast<uint32_t*>(odd ? const_cast<unsigned long long*>(buf_a) : buf_b);
@@ -2655,6 +2659,7 @@ __global__ void __launch_bounds__(256)
 k_wide_keep(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a,
             const unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t* __restrict__ order) {
   pdl_wait();
+  if (hdr->aborted) return;
   const uint32_t* tmp = reinterpret_cast<const uint32_t*>((hdr->npass & 1) ? buf_a : buf_b);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += stride) order[q] = tmp[q];
@@ -2665,6 +2670,7 @@ __global__ void __launch_bounds__(256)
 k_wide_final(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S, uint32_t sbits, uint32_t ibits,
              PlanHeader* hdr, const uint32_t* __restrict__ order, unsigned long long* __restrict__ buf_a) {
   pdl_wait();
+  if (hdr->aborted) return;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += stride) {
     const uint32_t orig = order[q];
@@ -2935,6 +2941,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     const uint32_t supers = (sbits + 60 + cw - 1) / cw;     /* for the widest legal span; chunks beyond the key are empty */
     const uint32_t chunk_passes = std::min<uint32_t>(kMaxPasses, (cw + 7) / 8);
     uint32_t* order = kept_tmp;
+    const uint32_t stall = (mode & PARD_MODE_TEST_STALL) ? 1u : 0u;
     for (uint32_t sp = 0; sp < supers; ++sp) {
       launch_pdl(k_wide_reset, (uint32_t)std::min<uint64_t>((lb_words + kMaxPasses * kBins + 255) / 256, (uint64_t)sms * 4), 256,
                  0, stream, hdr, hist, lookback, (unsigned long long)lb_words, sbits, ibits, sp);
@@ -2942,11 +2949,11 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  sp, (const PlanHeader*)hdr, (const uint32_t*)order, buf_a, hist);
       if (L.small_tiles)
         launch_pdl(k_sort_rest<false, true>, std::min<uint32_t>(L.sort_tiles, 2u * (uint32_t)sms), kSortThreads, sizeof(SortSmem), stream, 0u,
-                   hdr, buf_a, buf_b, (const uint32_t*)hist, lookback, lb_words, n32, ibits, 0u, 0u, CtxTiles{}, WinCountArgs{}, L.geometry);
+                   hdr, buf_a, buf_b, (const uint32_t*)hist, lookback, lb_words, n32, ibits, stall, 0u, CtxTiles{}, WinCountArgs{}, L.geometry);
       else
         for (uint32_t p = 0; p < chunk_passes; ++p)
           launch_pdl(k_sort_pass<false>, L.sort_tiles, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a, buf_b, hist,
-                     lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, 0u, 0u, CtxTiles{}, WinCountArgs{});
+                     lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, p == 0 ? stall : 0u, 0u, CtxTiles{}, WinCountArgs{});
       launch_pdl(k_wide_chase, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a, buf_b, n32,
                  ibits, sp, (const uint32_t*)order);
       launch_pdl(k_wide_keep, grid_n, 256, 0, stream, (const PlanHeader*)hdr, (const unsigned long long*)buf_a,

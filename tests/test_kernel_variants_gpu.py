@@ -222,3 +222,13 @@ def test_requests_out_of_place_while_blocks_start(n_ctx, per, at):
     check(wl)                                                             # legal without the promise
     wl.requests[[i, j]] = wl.requests[[j, i]]
     check(wl, pb.PARD_MODE_GROUPED)
+
+
+# ---- keys beyond 64 bits: a wait of the chunks' passes runs out, and nothing follows the half-sorted positions ------
+@pytest.mark.parametrize("n", [1500, 10_000])                            # one tile, several
+def test_wide_key_stops_behind_a_wait_that_ran_out(n):
+    rng = np.random.default_rng(n)
+    wl = several_ctx(300, np.bincount(rng.integers(0, 300, size=n), minlength=300), S=3, sort=False, mix=True)
+    wl.requests["deadline_us"][:2] = 5, 1 << 59
+    assert run_library(wl, pb.PARD_MODE_TEST_STALL, check=False)[0] == pb.PARD_ETIMEOUT
+    check(wl)
