@@ -137,8 +137,8 @@ extern "C" int pard_plan_host(const pard_pipeline_t* const* pipelines, uint32_t 
   rc = pard_report_enqueue(t, d_status, d_n_kept, stream);
   if (rc == PARD_OK) rc = fixed_outputs();                           /* garbage if the status says so: unspecified then */
   if (rc != PARD_OK) return rc;
-  rc = pard_report_wait(t, d_status, stream);
-  bool counted = t.word != nullptr;
+  bool counted = false;                                              /* the number of survivors came with the answer */
+  rc = pard_report_wait(t, d_status, stream, &counted);
   if (rc == PARD_ERANGE && n > 0) {                                   /* keys wider than 64 bits: the waiting call has a second stage for them */
     rc = pard_plan(pipelines, n_pipelines, d_req, n, &d, n_ctx, mode & ~PARD_MODE_NOWAIT, &dout, ws + L.plan, L.plan_bytes, cuda_stream);
     if (rc == PARD_OK) rc = fixed_outputs();

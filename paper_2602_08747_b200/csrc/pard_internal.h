@@ -87,8 +87,10 @@ void pard_report_init();
 PardTicket pard_report_ticket();
 /* zeroes the status header (256 bytes) of a call, by a kernel that the next one need not wait for to be placed */
 cudaError_t pard_clear_status(void* hdr, cudaStream_t stream);
-/* waits for the answer to `t` (given by the work already enqueued on `stream`); the call's status */
-int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream);
+/* waits for the answer to `t` (given by the work already enqueued on `stream`); the call's status.
+ * *answered (may be NULL): whether the answer came; if not, the status was copied and t.word[1] holds
+ * what an earlier call left there */
+int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream, bool* answered);
 /* enqueues the answer to `t`, and *d_count (may be NULL) beside it in t.word[1] */
 int pard_report_enqueue(const PardTicket& t, const uint32_t* d_status, const unsigned long long* d_count, cudaStream_t stream);
 /* kStagingBytes of pinned memory of the calling thread's own, or NULL; free again when the call that

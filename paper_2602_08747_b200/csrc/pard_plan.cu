@@ -2997,7 +2997,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     while (phase <= PARD_N_PHASES) mark();             /* the phases are those of the other path: all of this counts as the first */
     PARD_CUDA_OK(cudaGetLastError());
     if (mode & PARD_MODE_NOWAIT) return PARD_OK;
-    rc = answered ? pard_report_wait(la.answer, &hdr->status, stream) : pard_plan_status(d_workspace, cuda_stream);
+    rc = answered ? pard_report_wait(la.answer, &hdr->status, stream, nullptr) : pard_plan_status(d_workspace, cuda_stream);
     return rc == PARD_ERANGE ? plan_wide() : rc;
   }
 

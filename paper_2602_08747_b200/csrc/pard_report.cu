@@ -90,11 +90,15 @@ PardTicket pard_report_ticket() {
   return t;
 }
 
-int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream) {
+int pard_report_wait(const PardTicket& t, const uint32_t* d_status, cudaStream_t stream, bool* answered) {
+  if (answered) *answered = false;
   if (t.word) {
     for (uint32_t spins = 1;; ++spins) {
       const unsigned long long w = __atomic_load_n(t.word, __ATOMIC_ACQUIRE);
-      if ((uint32_t)(w >> 32) == t.ticket) return (uint32_t)w ? -(int)(uint32_t)w : PARD_OK;
+      if ((uint32_t)(w >> 32) == t.ticket) {
+        if (answered) *answered = true;
+        return (uint32_t)w ? -(int)(uint32_t)w : PARD_OK;
+      }
 #if defined(__x86_64__)
       __builtin_ia32_pause();
 #endif
@@ -120,7 +124,7 @@ int pard_report_enqueue(const PardTicket& t, const uint32_t* d_status, const uns
 int pard_wait_status(const uint32_t* d_status, cudaStream_t stream) {
   const PardTicket t = pard_report_ticket();
   const int rc = pard_report_enqueue(t, d_status, nullptr, stream);
-  return rc != PARD_OK ? rc : pard_report_wait(t, d_status, stream);
+  return rc != PARD_OK ? rc : pard_report_wait(t, d_status, stream, nullptr);
 }
 
 char* pard_staging() {

@@ -284,3 +284,62 @@ def test_advance_state_argument_checks_happen_before_any_launch():
     assert call(S=65) == pb.PARD_ERANGE
     assert call(M=pb.PARD_MAX_DELAY_SAMPLES + 1, slot=0) == pb.PARD_ERANGE
     h.free()
+
+
+HARNESS = r"""
+#include <cstdio>
+#include <cstring>
+#include <cstdlib>
+#include "pard_internal.h"
+static unsigned long long answer[2];
+static bool answers;
+extern "C" cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { memcpy(d, s, n); return cudaSuccess; }
+extern "C" cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+extern "C" int pard_plan_workspace_bytes(uint64_t, uint32_t, int32_t, uint64_t* b) { *b = 256; return PARD_OK; }
+extern "C" int pard_plan(const pard_pipeline_t* const*, uint32_t, const pard_request_t*, uint64_t n, const pard_queue_state_t*, uint32_t, uint32_t,
+                         const pard_plan_out_t* o, void* ws, uint64_t, void*) {
+  memset(ws, 0, 4);
+  for (uint64_t i = 0; i < n; ++i) o->d_kept_idx[i] = (uint32_t)(100 + i);
+  *o->d_n_kept = 3;
+  return PARD_OK;
+}
+PardTicket pard_report_ticket() { return {answer, 7}; }
+int pard_report_enqueue(const PardTicket&, const uint32_t*, const unsigned long long* count, cudaStream_t) { if (answers) answer[1] = *count; return PARD_OK; }
+int pard_report_wait(const PardTicket&, const uint32_t*, cudaStream_t, bool* answered) { if (answered) *answered = answers; return PARD_OK; }
+char* pard_staging() { return nullptr; }
+int main() {
+  const uint64_t n = 8;
+  static pard_request_t req[8];
+  static int64_t now[1], fa[1], q[1];
+  static int32_t batch[1] = {1};
+  pard_queue_state_t st = {};
+  st.stage_stride = 1; st.d_now_us = now; st.d_batch = batch; st.d_free_at_us = fa; st.d_q_us = q;
+  uint64_t bytes;
+  pard_plan_host_workspace_bytes(n, 1, 1, 0, &bytes);
+  void* ws = aligned_alloc(256, (bytes + 255) / 256 * 256);
+  for (int k = 0; k < 2; ++k) {
+    answers = k == 1;
+    answer[1] = 6;                                        /* an older call's */
+    uint32_t kept[8] = {};
+    uint64_t n_kept = 0;
+    pard_plan_out_t out = {};
+    out.d_kept_idx = kept; out.d_n_kept = &n_kept;
+    const int rc = pard_plan_host(nullptr, 1, req, n, &st, 1, 0, &out, ws, bytes, nullptr);
+    printf("%d %d %u %u\n", rc, (int)n_kept, kept[2], kept[3]);
+  }
+}
+"""
+
+
+def test_host_call_takes_the_count_only_from_an_answer_that_came(tmp_path):
+    """When a waiting call finds the stream finished and no answer in its pinned word, the number of survivors is
+    copied from the device: the word beside the answer holds an older call's.  (The runtime and the planner are
+    stand-ins here; the host-buffer call is the library's.)"""
+    import subprocess
+    src = tmp_path / "harness.cpp"
+    src.write_text(HARNESS)
+    exe = str(tmp_path / "harness")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", pbuild.CSRC, "-I", os.path.join(cuda, "include"),
+                           "-o", exe, "-x", "c++", str(src), os.path.join(pbuild.CSRC, "pard_host.cu")])
+    assert subprocess.check_output([exe], text=True).split("\n")[:2] == ["0 3 102 0"] * 2
