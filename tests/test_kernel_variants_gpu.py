@@ -232,3 +232,39 @@ def test_wide_key_stops_behind_a_wait_that_ran_out(n):
     wl.requests["deadline_us"][:2] = 5, 1 << 59
     assert run_library(wl, pb.PARD_MODE_TEST_STALL, check=False)[0] == pb.PARD_ETIMEOUT
     check(wl)
+
+
+# ---- queues booked far ahead (backlog) or long idle: 32-bit copies of A against the ctx's deadlines ------------------
+def booked(targets, span, d, n=700, seed=0, grouped=True):
+    """One ctx per target; in the last stage of each, A lies `target` us behind the ctx's smallest deadline."""
+    rng = np.random.default_rng(seed)
+    S, first = 3, 1 << 41
+    p = util.pipeline(inputs.chain_edges(S), S, [11, 5, d], bmax=4)
+    n_ctx = len(targets)
+    ctx = np.repeat(np.arange(n_ctx), n)
+    dl = first + rng.integers(0, span + 1, size=ctx.size)
+    dl[::n], dl[n - 1::n] = first, first + span
+    dl = dl[np.lexsort((dl, ctx))]
+    if not grouped:
+        k = rng.permutation(ctx.size)
+        ctx, dl = ctx[k], dl[k]
+    now = [min(first - 300, first + t - d) for t in targets]
+    fa = np.zeros((n_ctx, S), np.int64)
+    fa[:, S - 1] = [first + t - d for t in targets]
+    st = util.state(n_ctx, S, inputs.n_slots(p), now, 2, free_at=fa, workers=3)
+    return inputs.Workload("booked", [p], util.requests(dl, rng.integers(0, S, size=ctx.size), ctx), st, n_ctx)
+
+
+@pytest.mark.parametrize("span", [0, 3000, (1 << 31) - 2, (1 << 31) - 1, 1 << 31])
+@pytest.mark.parametrize("d", [7, 1 << 24])
+def test_block_per_ctx_with_queues_booked_far_ahead(span, d):
+    targets = [0, 1, span - 1, span, span + 1, span + 2, (1 << 31) - 2, (1 << 31) - 1, 1 << 31, (1 << 31) + 1, (1 << 32) + 5, 1 << 40,
+               -1, -(1 << 31) + 1, -(1 << 31), -(1 << 31) - 1]
+    for step_back in (False, True):                       # in deadline order, and sorted by the block
+        wl = booked(targets, span, d)
+        if step_back:
+            wl.requests["deadline_us"][5::700] = wl.requests["deadline_us"][::700]
+        for mode in (pb.PARD_MODE_GROUPED, pb.PARD_MODE_GROUPED | pb.PARD_MODE_RAW):
+            check(wl, mode)
+    for t in targets:
+        check(booked([t], span, d))                       # a single ctx
