@@ -245,8 +245,8 @@ __device__ void finish_constants(const ConstArgs& a, const unsigned long long* c
     const long long A = __ldcg(&K->A), d = __ldcg(&K->d);
     uint32_t narrow = __ldcg(&K->narrow);
     if (RANGES) {                                        /* as in ctx_constants */
-      const long long A_rel = (narrow & kSegHighFirst) ? (long long)hi - A : A - (long long)lo, lim = 1ll << 29;
-      const bool fits = __ldcg(&K->d_magic) != 0 && d < (1ll << 31) && A_rel > -lim && A_rel < lim && !(narrow & kSegNoStage);
+      const long long A_rel = (narrow & kSegHighFirst) ? (long long)hi - A : A - (long long)lo;
+      const bool fits = fits_narrow(__ldcg(&K->d_magic), d, A_rel, (narrow & kSegHighFirst) != 0) && !(narrow & kSegNoStage);
       narrow = (narrow & ~kSegNarrow) | (fits ? kSegNarrow : 0u);
       K->A_rel = A_rel;
       K->narrow = narrow;
@@ -606,7 +606,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       const PardSegConst K = ktab[q];
       s_A[q] = K.A; s_d[q] = K.d; s_magic[q] = K.d_magic;
       all_narrow = all_narrow && (K.narrow & (kSegNarrow | kSegNoStage)) == kSegNarrow;
-      s_wcon[q] = make_uint4((uint32_t)(int32_t)K.A_rel, win_off[q], win_cnt[q], (K.narrow & (kSegNarrow | kSegNoStage)) == kSegNarrow ? 1u : 0u);
+      s_wcon[q] = make_uint4((uint32_t)narrow_A(K), win_off[q], win_cnt[q], (K.narrow & (kSegNarrow | kSegNoStage)) == kSegNarrow ? 1u : 0u);
     }
   }
   bool plain = !hdr->bad_input && !priority && hdr->keybits + pshift <= 32 && dbits <= 29;
@@ -1660,12 +1660,13 @@ __device__ __forceinline__ void tile_first_half(const TileCtx& T, uint64_t base,
     /* one queue, and every quantity fits 32 bits: the common case */
     const uint32_t r0 = (uint32_t)base - sstart;
     const bool high_first = K.narrow & kSegHighFirst;
+    const int32_t A = narrow_A(K);
 #pragma unroll
     for (int i = 0; i < kDecItems; ++i) {
       const uint32_t lo = (uint32_t)e[i], hi = (uint32_t)(e[i] >> 32);
       idx[i] = lo & T.imask;
       const uint32_t off = __funnelshift_r(lo, hi, T.ibits) & (uint32_t)T.dmask;
-      const int32_t X = high_first ? (int32_t)K.A_rel - (int32_t)off : (int32_t)off - (int32_t)K.A_rel;
+      const int32_t X = high_first ? A - (int32_t)off : (int32_t)off - A;
       const unsigned long long uu = (unsigned long long)(div_magic32((uint32_t)X, K.d_magic) + 1u) * K.cap;
       u[i] = X < 0 ? 0u : (uu > kUClamp ? kUClamp : (uint32_t)uu);
       r[i] = r0 + i;
@@ -2371,6 +2372,7 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
   uint32_t koff = kept_dst ? kept_off[cur_seg] : 0u;
   const bool narrow = T.narrow && (K.narrow & (kSegNarrow | kSegNoStage)) == kSegNarrow && full &&
                       cur_seg == (uint32_t)(e[kDecItems - 1] >> T.kshift);
+  const int32_t A32 = narrow_A(K);
 
   uint32_t keepbits = 0, idx[kDecItems];
   long long est[kDecItems];
@@ -2384,7 +2386,7 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
       long long X;
       if (narrow) {
         const int32_t off = (int32_t)(__funnelshift_r((uint32_t)e[i], (uint32_t)(e[i] >> 32), T.ibits) & (uint32_t)T.dmask);
-        X = (HF && (K.narrow & kSegHighFirst)) ? (int32_t)K.A_rel - off : off - (int32_t)K.A_rel;
+        X = (HF && (K.narrow & kSegHighFirst)) ? A32 - off : off - A32;
       } else {
         const uint32_t sg = (uint32_t)(e[i] >> T.kshift);
         if (sg != cur_seg) {

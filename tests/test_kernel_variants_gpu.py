@@ -268,3 +268,19 @@ def test_block_per_ctx_with_queues_booked_far_ahead(span, d):
             check(wl, mode)
     for t in targets:
         check(booked([t], span, d))                       # a single ctx
+
+
+@pytest.mark.parametrize("span", [3000, (1 << 29) - 1, 1 << 29, 1 << 31])
+@pytest.mark.parametrize("d", [7, 1 << 24])
+def test_single_words_with_queues_booked_far_ahead(span, d):
+    targets = [0, span, span + 1, (1 << 29) - 1, 1 << 29, (1 << 29) + 1, (1 << 31) + 1, (1 << 32) + 5, 1 << 40,
+               -1, -(1 << 29) + 1, -(1 << 29), -(1 << 29) - 1, -(1 << 31) - 1, -(1 << 32) - 5, -(1 << 40)]
+    for grouped in (True, False):                        # one queue or several per thread of the decision
+        wl = booked(targets, span, d, grouped=grouped)
+        for mode in (0, pb.PARD_MODE_RAW, pb.PARD_MODE_SCAN):
+            check(wl, mode)
+        wl.state.priority = np.ones((wl.n_ctx, 3), np.uint8)              # A against the latest deadline
+        for mode in (0, pb.PARD_MODE_RAW, pb.PARD_MODE_SCAN):
+            check(wl, mode)
+    for t in targets:                                    # few queues: tables counted while packing
+        check(booked([t], span, d, n=9000))
