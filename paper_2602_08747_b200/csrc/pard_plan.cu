@@ -1,15 +1,21 @@
 /* The planner of libpard: kernels and their orchestration.
  *
  * Steps (paper passages in pard.h):
- *   prepass   per-ctx deadline range, per-segment queue length, input checks
- *   segscan   queue lengths -> first position of every segment
+ *   prepass   per-ctx deadline range, input checks, whether deadlines come in order; with few queues
+ *             also their constants
  *   segconst  per-segment constants of Eq. 3: d_k(B_k), base, L_sub (max over
  *             downstream paths), folded into A = base + d + L_sub
- *   pack      request -> one 64-bit sort element (segment | deadline | index)
+ *   pack      request -> one 64-bit sort element (segment | deadline | index), digit counts of the
+ *             passes; with few queues also the counts behind the window tables
  *   sort      LSD radix sort, 8 bits per pass, one read and one write of the
  *             elements per pass (tile prefixes by decoupled look-back)
- *   decide    threshold u per request, segmented prefix-min scan -> admitted
- *             position c, estimate, keep flag, compaction, per-segment counts
+ *   windows   queue boundaries, batch-window tables, kept counts and output offsets (with few queues
+ *             from the counts, beside the sort)
+ *   decide    every request on its own from its queue's table: admitted position c, estimate, keep
+ *             flag, survivors to their final place; too many windows: the same by a segmented
+ *             prefix-min scan (k_scan_path)
+ * Calls grouped by ctx in small contexts are planned by a block per ctx (pard_local.cu), the comparison
+ * rules by a walk of every queue behind the sort (pard_policy.cu).
  */
 #include <algorithm>
 #include <atomic>
@@ -2346,12 +2352,9 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
              const uint32_t* __restrict__ win_off, const uint32_t* __restrict__ win_cnt,
              const WinEntry* __restrict__ wtab,
              uint8_t* __restrict__ out_keep, long long* __restrict__ out_est,
-             uint32_t* __restrict__ out_perm, uint32_t* __restrict__ kept_dst, const uint32_t* __restrict__ kept_off,
-             uint32_t* __restrict__ seg_kept) {
-  /* kept_dst / kept_off: where the survivors of a queue go.  Normally the queue's own range of a
-   * scratch array (kept_off = the queues' first positions), packed afterwards; with counted
-   * tables the queues' kept counts are known beforehand and the survivors go straight to their
-   * final place (kept_dst = the output, kept_off = the queues' output offsets, seg_kept = NULL). */
+             uint32_t* __restrict__ out_perm, uint32_t* __restrict__ out_kept_idx, const uint32_t* __restrict__ kept_base) {
+  /* The queues' kept counts followed from their tables, so the survivors go straight to their final
+   * place: kept_base holds the queues' output offsets. */
   pdl_wait();
   if (hdr->use_scan || hdr->wide || hdr->aborted) return;
   const TileCtx T = make_tile_ctx(hdr, buf_a, buf_b, n, ibits, ktab, seg_off);
@@ -2368,8 +2371,8 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
   }
   uint32_t cur_seg = (uint32_t)(e[0] >> T.kshift);
   PardSegConst K = ktab[cur_seg];
-  uint32_t sstart = seg_off[cur_seg], send = seg_off[cur_seg + 1], woff = win_off[cur_seg], wcnt = win_cnt[cur_seg];
-  uint32_t koff = kept_dst ? kept_off[cur_seg] : 0u;
+  uint32_t sstart = seg_off[cur_seg], woff = win_off[cur_seg], wcnt = win_cnt[cur_seg];
+  uint32_t koff = out_kept_idx ? kept_base[cur_seg] : 0u;
   const bool narrow = T.narrow && (K.narrow & (kSegNarrow | kSegNoStage)) == kSegNarrow && full &&
                       cur_seg == (uint32_t)(e[kDecItems - 1] >> T.kshift);
   const int32_t A32 = narrow_A(K);
@@ -2393,8 +2396,7 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
           cur_seg = sg;
           K = ktab[sg];
           sstart = seg_off[sg];
-          koff = kept_dst ? kept_off[sg] : 0u;
-          send = seg_off[sg + 1];
+          koff = out_kept_idx ? kept_base[sg] : 0u;
           woff = win_off[sg];
           wcnt = win_cnt[sg];
         }
@@ -2414,7 +2416,6 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
         if (b64 >= (unsigned long long)wcnt) {
           set_status(T.hdr, PARD_EDATA);
           est[i] = K.A;
-          if (seg_kept && (uint32_t)j + 1 == send) seg_kept[cur_seg] = 0;
           continue;
         }
         const uint32_t b = (uint32_t)b64;
@@ -2437,8 +2438,7 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
       kept = c < u ? 1u : 0u;
       const uint32_t round = K.cap_magic ? div_magic32(c, K.cap_magic) : c;
       est[i] = K.A + (long long)((unsigned long long)round * (unsigned long long)K.d);
-      if (kept && kept_dst) kept_dst[koff + ahead] = idx[i];
-      if (seg_kept && (uint32_t)j + 1 == send) seg_kept[cur_seg] = ahead + kept;   /* the last request knows the queue's count */
+      if (kept && out_kept_idx) out_kept_idx[koff + ahead] = idx[i];
     }
     keepbits |= kept << i;
   }
@@ -2812,14 +2812,12 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   if ((uintptr_t)d_requests & 15) return PARD_EINVAL;
   int dev = -1;
   PARD_CUDA_OK(cudaGetDevice(&dev));
-  std::vector<const PardPipeDev*> h_pipes(n_pipelines);
   int32_t max_slots = 0;
   for (uint32_t i = 0; i < n_pipelines; ++i) {
     const pard_pipeline_t* p = pipelines[i];
     if (!p || !p->d_blob || p->device != dev) return PARD_EINVAL;
     if (p->n_stages > state->stage_stride) return PARD_EINVAL;
     max_slots = std::max(max_slots, p->n_slots);
-    h_pipes[i] = (const PardPipeDev*)p->d_blob;
   }
   if (state->d_w_us && state->slot_stride < max_slots) return PARD_EINVAL;
   if (!d_workspace || ((uintptr_t)d_workspace & 255)) return PARD_EINVAL;
@@ -2833,7 +2831,6 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   char* ws = (char*)d_workspace;
   PlanHeader* hdr = (PlanHeader*)(ws + L.hdr);
-  const PardPipeDev** d_pipes = (const PardPipeDev**)(ws + L.pipes);
   unsigned long long* ctx_dmin = (unsigned long long*)(ws + L.ctx_dmin);
   unsigned long long* ctx_dmax = (unsigned long long*)(ws + L.ctx_dmax);
   uint32_t* seg_off = (uint32_t*)(ws + L.seg_off);
@@ -2874,12 +2871,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   mark();
   int sms = 148;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  PipeTable pipe_table = {};
-  pipe_table.many = d_pipes;
-  if (n_pipelines <= (uint32_t)kFewPipelines)
-    for (uint32_t i = 0; i < n_pipelines; ++i) pipe_table.few[i] = h_pipes[i];
-  else
-    PARD_CUDA_OK(cudaMemcpyAsync(d_pipes, h_pipes.data(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
+  PipeTable pipe_table;
+  rc = pard_pipe_table(pipelines, n_pipelines, ws + L.pipes, stream, &pipe_table);
+  if (rc != PARD_OK) return rc;
   rc = allow_sort_smem(dev);
   if (rc != PARD_OK) return rc;
   const uint4* req4 = (const uint4*)d_requests;
@@ -3113,7 +3107,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                           : (state->d_priority ? k_decide_win<false, true> : k_decide_win<false, false>);
     /* the survivors go straight to their place in the output */
     launch_pdl(decide_win, win_grid, kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off, win_off, win_cnt, wtab,
-               out->d_keep, est, out->d_perm, out->d_kept_idx, (const uint32_t*)kept_base, (uint32_t*)nullptr);
+               out->d_keep, est, out->d_perm, out->d_kept_idx, (const uint32_t*)kept_base);
     /* fallback when a queue has too many batch windows: the same decision by scanning, one kernel
      * that returns at once otherwise */
     const uint32_t scan_grid = std::min<uint32_t>(L.dec_tiles, (uint32_t)sms * 2);

@@ -133,8 +133,6 @@ struct CtxScratch {
   unsigned long long lsub[PARD_MAX_STAGES];
   int32_t slot_off[PARD_MAX_STAGES + 1];
 };
-__device__ __forceinline__ unsigned long long magic64(unsigned long long d);
-
 __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n_pipelines, const pard_queue_state_t& st, uint32_t c,
                                               unsigned long long dmin, unsigned long long dmax, PardSegConst* K_out,
                                               CtxScratch& sc, long long* sums = nullptr) {
