@@ -2238,10 +2238,19 @@ k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const u
   kept_scan_block<kWinThreads>(seg_kept, n_seg, kept_base, chunk_base, out_seg_kept, out_n_kept);
 }
 
-/* The same for calls with very many short queues, where a warp per queue would mostly idle: a thread
- * per queue (plain binary searches whose early probes coincide across the lanes; its few windows one
- * after the other), 511 queues per block. */
-constexpr uint32_t kShortQueue = 128;              /* requests per queue on average below which this form is taken */
+/* The same for calls with very many short queues: a thread per queue (plain binary searches whose early
+ * probes coincide across the lanes; its windows one after the other), 511 queues per block.  A thread's
+ * chain of dependent loads is longer than a warp's, and the longer the more requests a queue has; but
+ * k_windows keeps 4,736 queues in flight on 148 multiprocessors, so it walks its chain once per so many.
+ * Whole calls, interleaved contexts, a warp / a thread per queue:
+ *   queues              8,192      16,384     20,480     32,768     65,536
+ *     32 requests each  113 / 123  185 / 181  177 / 165  235 / 200  415 / 290 us
+ *    128                141 / 165  227 / 229  253 / 251  362 / 324  671 / 540
+ *    256                197 / 224  315 / 323  364 / 370  549 / 523  1109 / 988
+ *    512                279 / 316  487 / 512  634 / 687  967 / 963
+ * so: from 16,384 queues on, with more than 128 queues per request of the average queue. */
+constexpr uint32_t kManyQueues = 16384, kManyPerRequest = 128;
+inline bool many_short_queues(uint64_t n, uint64_t n_seg) { return n_seg >= kManyQueues && n_seg * n_seg > kManyPerRequest * n; }
 __global__ void __launch_bounds__(kWinThreads)
 k_windows_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
                uint32_t ibits, uint32_t n_seg, const PardSegConst* __restrict__ ktab, uint32_t* __restrict__ seg_off,
@@ -2893,7 +2902,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   /* queue boundaries, and for the planner's own rule the window tables and output offsets; id_bits > 8:
    * the boundaries are searched, never read off the digit counts */
   auto launch_windows = [&](bool tables, uint32_t local_candidate, uint32_t id_bits = 64u) {
-    if (n / L.n_seg < kShortQueue && L.n_seg >= 4096)
+    if (many_short_queues(n, L.n_seg))
       launch_pdl(k_windows_many, L.n_seg / (kWinThreads - 1u) + 1, kWinThreads, 0, stream, hdr, (const unsigned long long*)buf_a,
                  (const unsigned long long*)buf_b, n32, ibits, L.n_seg, (const PardSegConst*)ktab, seg_off, out->d_seg_offsets,
                  win_off, win_cnt, wtab, L.win_capacity, (mode & PARD_MODE_SCAN) ? 1u : 0u, tables ? 1u : 0u,

@@ -284,3 +284,16 @@ def test_single_words_with_queues_booked_far_ahead(span, d):
             check(wl, mode)
     for t in targets:                                    # few queues: tables counted while packing
         check(booked([t], span, d, n=9000))
+
+
+# ---- a thread per queue: from 16,384 queues on, more than 128 of them per request of the average queue; 511 to a block ----
+@pytest.mark.parametrize("n_ctx,S,n", [(16_383, 1, 60_000), (16_384, 1, 60_000), (16_384, 1, 2_097_151), (16_384, 1, 2_097_152),
+                                       (511, 33, 30_000), (5462, 3, 1_100_000), (8193, 2, 9_000)])
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW, pb.PARD_MODE_SCAN, FCFS])
+def test_window_tables_of_very_many_queues(n_ctx, S, n, mode):
+    rng = np.random.default_rng(n + S)
+    wl = several_ctx(n_ctx, np.bincount(rng.integers(0, n_ctx, size=n), minlength=n_ctx), S=S, sort=False, mix=True, m=2)
+    check(wl, mode)
+    if mode != FCFS:
+        wl.state.priority = rng.integers(0, 2, size=(n_ctx, S)).astype(np.uint8)
+        check(wl, mode)
