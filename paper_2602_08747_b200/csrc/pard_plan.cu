@@ -1320,7 +1320,9 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
  * takes tiles by ticket until the pass has none left, hands in how many it has finished, and begins the
  * next pass when all tiles have been handed in.  It never waits for a block
  * that has not been placed: however few of the grid's blocks run at a time -- other streams may hold the
- * multiprocessors, another call's grid of this kind among them -- those that run finish the pass.
+ * multiprocessors, another call's grid of this kind among them -- those that run finish the pass.  (Every
+ * tile handed in by itself: 214.0 against 211.2 us for 2.5 M requests of 512 contexts; a block's tiles
+ * together: 212.4, as when the grid's blocks were counted.)
  * At 2^24 elements such a grid takes 9 us more per pass than one block per tile (the blocks' loads
  * no longer start under the write-out of others), so the passes that large calls usually need keep
  * launches of their own.  Calls of one or two rounds of small tiles (SMALL) do all passes here,
@@ -2516,7 +2518,9 @@ __device__ __forceinline__ void kept_move_jobs(const uint32_t* __restrict__ kept
  * the one-block step behind it and then sets a flag, which the others wait for before they go on.  So a wait
  * is only ever for blocks that run already, and those that run finish the call, however few of the grid
  * are placed at a time; each wait is bounded all the same (PARD_ETIMEOUT, every block gives up, nothing
- * hangs). */
+ * hangs).  Bound by the two reads of the elements and by the one-block steps: forced for 2^24 requests the
+ * call takes 726 us, for a million 62.0 (713 and 58.9 when a wait was for every block of the grid; every run
+ * handed in by itself: 733 and 66). */
 constexpr uint32_t kScanRuns = 4;                /* runs of tiles per block of the grid: blocks that start late find less to do */
 /* The block's share of a step: work(first tile, end) for every run it gets hold of, the next ticket fetched
  * while a run is worked on.  True in the block that completes the step.  stall: testing aid, the first run

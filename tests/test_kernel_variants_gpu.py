@@ -112,7 +112,7 @@ def test_estimate_w_shapes(M):
             assert np.array_equal(got, np.asarray(want).reshape(got.shape))
 
 
-# ---- window tables of many queues: a warp or a thread per queue, block and table edges ------------
+# ---- window tables of many queues, a warp for each: block and table edges ------------
 @pytest.mark.parametrize("n_ctx,S,n", [(5, 15, 90_000), (5, 16, 90_000), (17, 16, 200_001), (1366, 3, 30_000), (4088, 1, 50_000),
                                        (511, 9, 20_000), (2731, 3, 1_100_000)])
 @pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW, pb.PARD_MODE_SCAN])

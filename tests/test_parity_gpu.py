@@ -25,8 +25,8 @@ def both(wl, mode=0):
     return got
 
 
-# sizes chosen to span several tiles of both the sort (4096) and the decision
-# pass (2048) and to leave a ragged tail
+# sizes chosen to span several tiles of both the sort (2,048 to 8,192 elements) and the decision
+# pass (1,024) and to leave a ragged tail
 @pytest.mark.parametrize("name,kw", [
     ("C1", {}), ("C1b", {}),
     ("C1", {"n": 1}), ("C1", {"n": 2047}), ("C1", {"n": 2049}), ("C1b", {"n": 12345}),
@@ -34,7 +34,7 @@ def both(wl, mode=0):
     ("C3", {"n": 70_001}), ("C3b", {"n": 300_007}),
     ("C4", {"n_epochs": 37, "per_epoch": 1000}), ("C4b", {"n_epochs": 64, "per_epoch": 8192}),
     ("C5", {"n_inst": 9, "per_inst": 5001}), ("C5b", {"n_inst": 16, "per_inst": 65536}),
-    # thousands of queues: the lane-per-queue form of the segment search
+    # thousands of queues: several rounds of the kernel that has a warp for each
     ("C4b", {"n_epochs": 1100, "per_epoch": 200}), ("C5b", {"n_inst": 600, "per_inst": 301}),
 ])
 @pytest.mark.parametrize("mode", [0, 1])
@@ -194,8 +194,9 @@ def test_bounded_wait_runs_out_and_is_reported():
 
 
 def test_bounded_grid_barrier_runs_out_and_is_reported():
-    """The scan path's blocks meet at counters; a block that never arrives (stall aid) makes every
-    other block's bounded wait run out: PARD_ETIMEOUT, nothing hangs, the next call is correct.
+    """The scan path's steps wait for all tiles of the step before; tiles that are never counted as
+    finished (stall aid) make every block's bounded wait run out: PARD_ETIMEOUT, nothing hangs, the next
+    call is correct.
     The call is sorted block by block, so the sort itself has no wait to run out first."""
     wl, _ = _grouped(n_epochs=40, seed=7)
     rc, _ = run_library(wl, mode=pb.PARD_MODE_SCAN | pb.PARD_MODE_TEST_STALL, check=False)
