@@ -18,7 +18,7 @@
  * Queues with more windows than the block's tables hold are decided by the segmented prefix-min
  * scan over the elements instead.
  * Bound by the chain of steps between barriers, two blocks per multiprocessor covering for each other:
- * of 400 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the copy bandwidth) 120 go to the
+ * of 385 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the copy bandwidth) 120 go to the
  * requests, 75 to the counting sort, 50 to the tables and 110 to the outputs.  The form before,
  * two segmented scans instead of tables, took 762 us there, three radix passes without a look at the
  * order 865. */

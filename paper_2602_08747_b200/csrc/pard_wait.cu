@@ -9,10 +9,10 @@
  * histogram over the top 11 of the bits that occur, a scan of it, then the few sums of the one bin
  * that holds the rank are compared with each other (or, if they are many, split again).
  * Bound by the integer pipes (multiplications and logic both near 60 % of their cycles, issue slots
- * at 69 %): of some 35 instructions per draw two thirds are splitmix64.  M = 10,000 on the
+ * at 68 %): of some 35 instructions per draw two thirds are splitmix64.  M = 10,000 on the
  * 4,500 slots of 256 pipelines (262 M draws): 635 us with a block of its own for every slot of the
  * stride -- most of them padding, each paying five dependent loads to find its path --, the sums
- * in shared memory and four rounds of selection over all of them; 425 us like this. */
+ * in shared memory and four rounds of selection over all of them; 437 us like this. */
 #include <algorithm>
 #include <mutex>
 
