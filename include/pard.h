@@ -50,7 +50,9 @@ typedef enum pard_status {
   PARD_ECYCLE      = -2,  /* the stage graph has a cycle                             */
   PARD_ERANGE      = -3,  /* a host-visible value is outside the limits above; with
                              PARD_MODE_NOWAIT also: the sort key exceeds 64 bits     */
-  PARD_ENOMEM      = -4,  /* host or device allocation failed (load time only)       */
+  PARD_ENOMEM      = -4,  /* host or device allocation failed (at load time,
+                             pard_profile_begin, or the host's table of the pipelines
+                             of a call with more than 256)                           */
   PARD_EWORKSPACE  = -5,  /* caller's workspace is smaller than required             */
   PARD_ETIMEOUT    = -6,  /* a bounded device-side wait ran out; outputs unspecified */
   PARD_ECUDA       = -7,  /* a CUDA runtime call failed                              */

@@ -3,6 +3,7 @@
  * and upload of the tables to the device. */
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <new>
 
 #include "pard_internal.h"
@@ -80,10 +81,8 @@ struct Enumerator {
   }
 };
 
-}  // namespace
-
-extern "C" int pard_load_pipeline(const pard_dag_t* dag, const pard_profile_t* prof,
-                                  uint32_t flags, pard_pipeline_t** out) {
+/* May throw std::bad_alloc (host tables). */
+int load_pipeline(const pard_dag_t* dag, const pard_profile_t* prof, uint32_t flags, pard_pipeline_t** out) {
   if (!out) return PARD_EINVAL;
   *out = nullptr;
   if (flags & ~PARD_LOAD_HOST_ONLY) return PARD_EINVAL;
@@ -123,28 +122,22 @@ extern "C" int pard_load_pipeline(const pard_dag_t* dag, const pard_profile_t* p
     }
   if (slots > PARD_MAX_PATH_SLOTS || total_len > PARD_MAX_PATH_LEN_SUM) return PARD_ERANGE;
 
-  pard_pipeline* p = new (std::nothrow) pard_pipeline();
-  if (!p) return PARD_ENOMEM;
-  try {
-    p->n_stages = S;
-    p->bmax.assign(prof->bmax, prof->bmax + S);
-    p->lat_offsets.assign(prof->lat_offsets, prof->lat_offsets + S + 1);
-    p->lat_us.assign(prof->lat_us, prof->lat_us + prof->lat_offsets[S]);
-    p->stage_slot_off.assign(S + 1, 0);
-    p->path_off.push_back(0);
-    p->local_off.resize(S);
-    Enumerator en{succ, p->path_off, p->path_stage, {}};
-    for (int32_t k = 0; k < S; ++k) {
-      for (int32_t j : succ[k]) en.extend(j);
-      p->stage_slot_off[k + 1] = (int32_t)p->path_off.size() - 1;
-      int32_t b = p->stage_slot_off[k], e = p->stage_slot_off[k + 1];
-      for (int32_t s = b; s <= e; ++s) p->local_off[k].push_back(p->path_off[s] - p->path_off[b]);
-    }
-    p->n_slots = (int32_t)p->path_off.size() - 1;
-  } catch (const std::bad_alloc&) {
-    delete p;
-    return PARD_ENOMEM;
+  std::unique_ptr<pard_pipeline> p(new pard_pipeline());
+  p->n_stages = S;
+  p->bmax.assign(prof->bmax, prof->bmax + S);
+  p->lat_offsets.assign(prof->lat_offsets, prof->lat_offsets + S + 1);
+  p->lat_us.assign(prof->lat_us, prof->lat_us + prof->lat_offsets[S]);
+  p->stage_slot_off.assign(S + 1, 0);
+  p->path_off.push_back(0);
+  p->local_off.resize(S);
+  Enumerator en{succ, p->path_off, p->path_stage, {}};
+  for (int32_t k = 0; k < S; ++k) {
+    for (int32_t j : succ[k]) en.extend(j);
+    p->stage_slot_off[k + 1] = (int32_t)p->path_off.size() - 1;
+    int32_t b = p->stage_slot_off[k], e = p->stage_slot_off[k + 1];
+    for (int32_t s = b; s <= e; ++s) p->local_off[k].push_back(p->path_off[s] - p->path_off[b]);
   }
+  p->n_slots = (int32_t)p->path_off.size() - 1;
 
   if (!(flags & PARD_LOAD_HOST_ONLY)) {
     /* one blob: header, then the tables, each 16-byte aligned */
@@ -158,14 +151,13 @@ extern "C" int pard_load_pipeline(const pard_dag_t* dag, const pard_profile_t* p
     size_t total = align16(off_ps + sizeof(int32_t) * std::max<size_t>(1, p->path_stage.size()));
     int dev = -1;
     char* d = nullptr;
-    if (cudaGetDevice(&dev) != cudaSuccess) { delete p; return PARD_ECUDA; }
+    std::vector<char> h(total, 0);                 /* ahead of the device's: nothing below throws */
+    if (cudaGetDevice(&dev) != cudaSuccess) return PARD_ECUDA;
     pard_report_init();
     if (cudaMalloc((void**)&d, total) != cudaSuccess) {
       cudaGetLastError();
-      delete p;
       return PARD_ENOMEM;
     }
-    std::vector<char> h(total, 0);
     PardPipeDev hdr;
     hdr.n_stages = S;
     hdr.n_slots = p->n_slots;
@@ -185,14 +177,24 @@ extern "C" int pard_load_pipeline(const pard_dag_t* dag, const pard_profile_t* p
       memcpy(h.data() + off_ps, p->path_stage.data(), sizeof(int32_t) * p->path_stage.size());
     if (cudaMemcpy(d, h.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) {
       cudaFree(d);
-      delete p;
       return PARD_ECUDA;
     }
     p->device = dev;
     p->d_blob = d;
   }
-  *out = p;
+  *out = p.release();
   return PARD_OK;
+}
+
+}  // namespace
+
+extern "C" int pard_load_pipeline(const pard_dag_t* dag, const pard_profile_t* prof,
+                                  uint32_t flags, pard_pipeline_t** out) {
+  try {
+    return load_pipeline(dag, prof, flags, out);
+  } catch (const std::bad_alloc&) {
+    return PARD_ENOMEM;
+  }
 }
 
 extern "C" int pard_free_pipeline(pard_pipeline_t* p) {

@@ -3177,7 +3177,11 @@ extern "C" int pard_profile_begin(uint32_t every, uint32_t max_samples) {
   if (every < 1 || max_samples < 1 || max_samples > 65536) return PARD_EINVAL;
   std::lock_guard<std::mutex> lock(g_prof.mu);
   if (g_prof.on.load()) return PARD_EINVAL;
-  g_prof.ev.assign((size_t)max_samples * kEventsPerSample, nullptr);
+  try {
+    g_prof.ev.assign((size_t)max_samples * kEventsPerSample, nullptr);
+  } catch (const std::bad_alloc&) {
+    return PARD_ENOMEM;
+  }
   for (auto& e : g_prof.ev)
     if (cudaEventCreate(&e) != cudaSuccess) {
       for (auto& f : g_prof.ev) if (f) cudaEventDestroy(f);

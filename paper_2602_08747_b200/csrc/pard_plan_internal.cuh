@@ -3,6 +3,9 @@
 #ifndef PARD_PLAN_INTERNAL_CUH_
 #define PARD_PLAN_INTERNAL_CUH_
 
+#include <memory>
+#include <new>
+
 #include "pard_internal.h"
 
 namespace pard_plan_detail {
@@ -94,9 +97,10 @@ inline int pard_pipe_table(const pard_pipeline_t* const* pipelines, uint32_t n_p
       out->few[i] = i < n_pipelines ? (const PardPipeDev*)pipelines[i]->d_blob : nullptr;
     return PARD_OK;
   }
-  std::vector<const PardPipeDev*> h(n_pipelines);
+  std::unique_ptr<const PardPipeDev*[]> h(new (std::nothrow) const PardPipeDev*[n_pipelines]);
+  if (!h) return PARD_ENOMEM;
   for (uint32_t i = 0; i < n_pipelines; ++i) h[i] = (const PardPipeDev*)pipelines[i]->d_blob;
-  PARD_CUDA_OK(cudaMemcpyAsync(d_many, h.data(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
+  PARD_CUDA_OK(cudaMemcpyAsync(d_many, h.get(), 8ull * n_pipelines, cudaMemcpyHostToDevice, stream));
   return PARD_OK;
 }
 

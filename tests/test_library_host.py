@@ -343,3 +343,49 @@ def test_host_call_takes_the_count_only_from_an_answer_that_came(tmp_path):
     subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", pbuild.CSRC, "-I", os.path.join(cuda, "include"),
                            "-o", exe, "-x", "c++", str(src), os.path.join(pbuild.CSRC, "pard_host.cu")])
     assert subprocess.check_output([exe], text=True).split("\n")[:2] == ["0 3 102 0"] * 2
+
+
+ALLOCATIONS = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <new>
+#include "pard.h"
+static long left = -1;                                   /* allocations until one fails; < 0: none does */
+void* operator new(size_t n) {
+  if (left >= 0 && left-- == 0) throw std::bad_alloc();
+  void* p = malloc(n);
+  if (!p) throw std::bad_alloc();
+  return p;
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+int main() {
+  const int32_t off[4] = {0, 2, 3, 3}, ids[3] = {1, 2, 2}, bmax[3] = {2, 2, 2};
+  const int64_t lo[4] = {0, 2, 4, 6}, lat[6] = {1, 2, 1, 2, 1, 2};
+  const pard_dag_t dag = {3, off, ids};
+  const pard_profile_t prof = {bmax, lo, lat};
+  int failed = 0;
+  for (long k = 0;; ++k) {
+    pard_pipeline_t* p = nullptr;
+    left = k;
+    const int rc = pard_load_pipeline(&dag, &prof, PARD_LOAD_HOST_ONLY, &p);
+    left = -1;
+    if (rc == PARD_OK) { pard_free_pipeline(p); break; }
+    if (rc != PARD_ENOMEM || p) return 1;
+    ++failed;
+  }
+  left = 0;
+  const int rc = pard_profile_begin(1, 16);
+  left = -1;
+  printf("%d %d\n", failed > 10, rc);
+}
+"""
+
+
+def test_no_exception_leaves_the_library_when_an_allocation_fails(tmp_path):
+    import subprocess
+    src, exe = tmp_path / "alloc.cpp", str(tmp_path / "alloc")
+    src.write_text(ALLOCATIONS)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-rdynamic", "-I", os.path.join(ROOT, "include"), "-o", exe, str(src), pbuild.LIB,
+                           "-Wl,-rpath," + os.path.dirname(pbuild.LIB)])
+    assert subprocess.check_output([exe], text=True).split() == ["1", str(pb.PARD_ENOMEM)]
