@@ -24,6 +24,7 @@ def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
     files.append(os.path.join(CSRC, "pard_internal.h"))
     files.append(os.path.join(CSRC, "pard_plan_internal.cuh"))
+    files.append(os.path.join(CSRC, "pard_direct.cuh"))
     files.append(os.path.join(ROOT, "include", "pard.h"))
     return files
 

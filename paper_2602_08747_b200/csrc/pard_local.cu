@@ -904,7 +904,7 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
    * from the table filled for all queues at once (a chain of dependent loads that every block
    * would otherwise wait for) and completed with what hangs on the ctx's deadline range */
   if (single) {
-    if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, dmin, dmax, Sm.K, *reinterpret_cast<CtxScratch*>(Sm.keys))) set_status(hdr, PARD_EDATA);
+    if (ctx_constants<false>(a.pipes, a.n_pipelines, a.st, c, dmin, dmax, Sm.K, *reinterpret_cast<CtxScratch*>(Sm.keys))) set_status(hdr, PARD_EDATA);
     for (uint32_t k = tid; k < S; k += kLocThreads)      /* (the thread that wrote it) */
       if (!(Sm.K[k].narrow & kSegHighFirst)) Sm.K[k].A_rel = booked_within(Sm.K[k].A_rel, span);
   } else {
@@ -1034,7 +1034,7 @@ k_ctx_prep(const __grid_constant__ LocalArgs a, PardSegConst* __restrict__ ktab,
   pdl_wait();
   __shared__ CtxScratch scratch;
   if (blockIdx.x < a.n_ctx) {
-    if (ctx_constants(a.pipes, a.n_pipelines, a.st, blockIdx.x, 0, 0, ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch))
+    if (ctx_constants<true>(a.pipes, a.n_pipelines, a.st, blockIdx.x, 0, 0, ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch))
       set_status(hdr, PARD_EDATA);
     return;
   }

@@ -212,6 +212,16 @@ __device__ __forceinline__ long long* sums_of(const ConstArgs& a, uint32_t c) {
   return a.path_sums ? a.path_sums + (size_t)c * a.st.stage_stride * kMaskPaths : nullptr;
 }
 
+/* What the constants of a queue take from the deadline range [lo, hi] of its ctx, as in ctx_constants; the new `narrow`. */
+__device__ __forceinline__ uint32_t range_constants(PardSegConst* K, long long A, long long d, uint32_t narrow, unsigned long long lo, unsigned long long hi) {
+  const long long A_rel = (narrow & kSegHighFirst) ? (long long)hi - A : A - (long long)lo;
+  const bool fits = fits_narrow(__ldcg(&K->d_magic), d, A_rel, (narrow & kSegHighFirst) != 0) && !(narrow & kSegNoStage);
+  narrow = (narrow & ~kSegNarrow) | (fits ? kSegNarrow : 0u);
+  K->A_rel = A_rel;
+  K->narrow = narrow;
+  return narrow;
+}
+
 /* By one whole block, once every ctx's deadline range and every queue's constants are there: what
  * hangs on both.  RANGES: the constants do not know the ranges yet. */
 template <bool RANGES>
@@ -250,13 +260,7 @@ __device__ void finish_constants(const ConstArgs& a, const unsigned long long* c
     PardSegConst* K = a.ktab + q;
     const long long A = __ldcg(&K->A), d = __ldcg(&K->d);
     uint32_t narrow = __ldcg(&K->narrow);
-    if (RANGES) {                                        /* as in ctx_constants */
-      const long long A_rel = (narrow & kSegHighFirst) ? (long long)hi - A : A - (long long)lo;
-      const bool fits = fits_narrow(__ldcg(&K->d_magic), d, A_rel, (narrow & kSegHighFirst) != 0) && !(narrow & kSegNoStage);
-      narrow = (narrow & ~kSegNarrow) | (fits ? kSegNarrow : 0u);
-      K->A_rel = A_rel;
-      K->narrow = narrow;
-    }
+    if (RANGES) narrow = range_constants(K, A, d, narrow, lo, hi);
     if (a.win_hist) {
       uint32_t w = 1;
       if (!(narrow & kSegNoStage) && lo <= hi) {
@@ -285,16 +289,125 @@ __device__ void finish_constants(const ConstArgs& a, const unsigned long long* c
   }
 }
 
+/* Kept requests per queue -> first output slot of every queue, the number of
+ * kCompactChunk-sized copy jobs before every queue, and the total.  One block,
+ * eight queues per thread and round. */
+template <int THREADS>
+__device__ void kept_scan_block(const uint32_t* seg_kept, uint32_t n_seg, uint32_t* kept_base,
+                                uint32_t* chunk_base, uint32_t* out_seg_kept, unsigned long long* out_n_kept) {
+  constexpr int PER = 8, WARPS = THREADS / 32;
+  __shared__ uint32_t s_a[32], s_b[32];
+  __shared__ uint32_t s_ca, s_cb;
+  if (threadIdx.x == 0) { s_ca = 0; s_cb = 0; }
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  /* a thread's eight entries as two 16-byte accesses where the arrays allow it */
+  const bool vec_in = ((uintptr_t)seg_kept & 15) == 0;
+  const bool vec_out = (((uintptr_t)kept_base | (uintptr_t)chunk_base) & 15) == 0;
+  const bool vec_user = out_seg_kept && ((uintptr_t)out_seg_kept & 15) == 0;
+  for (uint32_t base = 0; base < n_seg + 1; base += THREADS * PER) {
+    const uint32_t i0 = base + threadIdx.x * PER;
+    uint32_t v[PER], c[PER], x = 0, y = 0;
+    if (vec_in && i0 + PER <= n_seg) {
+      /* (L2 loads here and in kept_move_jobs: inside k_scan_path other blocks of the same kernel wrote these) */
+      const uint4 a = __ldcg(reinterpret_cast<const uint4*>(seg_kept + i0)), b = __ldcg(reinterpret_cast<const uint4*>(seg_kept + i0 + 4));
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+      for (int k = 0; k < PER; ++k) v[k] = i0 + k < n_seg ? __ldcg(&seg_kept[i0 + k]) : 0;
+    }
+    if (vec_user && i0 + PER <= n_seg) {
+      *reinterpret_cast<uint4*>(out_seg_kept + i0) = make_uint4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<uint4*>(out_seg_kept + i0 + 4) = make_uint4(v[4], v[5], v[6], v[7]);
+    } else if (out_seg_kept) {
+#pragma unroll
+      for (int k = 0; k < PER; ++k) if (i0 + k < n_seg) out_seg_kept[i0 + k] = v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      c[k] = (v[k] + kCompactChunk - 1) / kCompactChunk;
+      x += v[k];
+      y += c[k];
+    }
+    const uint32_t tx = x, ty = y;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= (uint32_t)o) { x += p; y += q; }
+    }
+    if (lane == 31) { s_a[warp] = x; s_b[warp] = y; }
+    __syncthreads();
+    if (warp == 0) {
+      const uint32_t a = lane < WARPS ? s_a[lane] : 0u, b = lane < WARPS ? s_b[lane] : 0u;
+      uint32_t ta = a, tb = b;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t p = __shfl_up_sync(0xffffffffu, ta, o), q = __shfl_up_sync(0xffffffffu, tb, o);
+        if (lane >= (uint32_t)o) { ta += p; tb += q; }
+      }
+      s_a[lane] = ta - a;
+      s_b[lane] = tb - b;
+    }
+    __syncthreads();
+    uint32_t ea = s_ca + s_a[warp] + x - tx, eb = s_cb + s_b[warp] + y - ty;   /* exclusive, before this thread's queues */
+    uint32_t oa[PER], ob[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      oa[k] = ea; ob[k] = eb;
+      ea += v[k];
+      eb += c[k];
+    }
+    if (vec_out && i0 + PER <= n_seg + 1) {
+      *reinterpret_cast<uint4*>(kept_base + i0) = make_uint4(oa[0], oa[1], oa[2], oa[3]);
+      *reinterpret_cast<uint4*>(kept_base + i0 + 4) = make_uint4(oa[4], oa[5], oa[6], oa[7]);
+      *reinterpret_cast<uint4*>(chunk_base + i0) = make_uint4(ob[0], ob[1], ob[2], ob[3]);
+      *reinterpret_cast<uint4*>(chunk_base + i0 + 4) = make_uint4(ob[4], ob[5], ob[6], ob[7]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < PER; ++k) if (i0 + k <= n_seg) { kept_base[i0 + k] = oa[k]; chunk_base[i0 + k] = ob[k]; }
+    }
+    __syncthreads();
+    if (threadIdx.x == THREADS - 1) { s_ca = ea; s_cb = eb; }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0 && out_n_kept) *out_n_kept = s_ca;
+}
+
+/* the lanes whose digit is d, from one ballot per digit bit */
+template <int BITS>
+__device__ __forceinline__ uint32_t digit_peers(uint32_t d, const uint32_t (&bal)[BITS]) {
+  uint32_t m = 0xffffffffu;
+#pragma unroll
+  for (int k = 0; k < BITS; ++k) m &= ((d >> k) & 1u) ? bal[k] : ~bal[k];
+  return m;
+}
+
+#include "pard_direct.cuh"
+
 /* Constants of all queues, a block per ctx, with a launch of their own: calls with many queues, whose
  * blocks would hold up the prepass, and calls without requests. */
 __global__ void __launch_bounds__(kConstThreads)
 k_seg_const(const __grid_constant__ ConstArgs a, const unsigned long long* __restrict__ ctx_dmin_inv,
             const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr) {
   pdl_wait();
+  if (hdr->direct) return;
   __shared__ CtxScratch scratch;
-  if (ctx_constants(a.pipes, a.n_pipelines, a.st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
+  if (ctx_constants<true>(a.pipes, a.n_pipelines, a.st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
                     a.ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch, sums_of(a, blockIdx.x)))
     set_status(hdr, PARD_EDATA);
+  if (a.with_key_width && last_block_done(&hdr->seg_done)) finish_constants<false>(a, ctx_dmin_inv, ctx_dmax, hdr);
+}
+
+/* The constants are there but for what they take from the deadline ranges (k_dir_count worked them out): a thread per
+ * queue; the block that finishes last finds the key width.  (k_seg_const anew: 12 us more for 8,192 queues.) */
+__global__ void __launch_bounds__(256)
+k_seg_finish(const __grid_constant__ ConstArgs a, const unsigned long long* __restrict__ ctx_dmin_inv,
+             const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr) {
+  pdl_wait();
+  if (hdr->direct) return;
+  const uint32_t S = (uint32_t)a.st.stage_stride, q = blockIdx.x * 256 + threadIdx.x;
+  if (q < a.n_ctx * S) {
+    PardSegConst* K = a.ktab + q;
+    range_constants(K, K->A, K->d, K->narrow, ~ctx_dmin_inv[q / S], ctx_dmax[q / S]);
+  }
   if (a.with_key_width && last_block_done(&hdr->seg_done)) finish_constants<false>(a, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
@@ -315,7 +428,7 @@ constexpr int kPreUn = 4;
 
 __device__ __noinline__ void const_block(const ConstArgs& a, uint32_t c, PlanHeader* hdr) {
   __shared__ CtxScratch scratch;
-  if (ctx_constants(a.pipes, a.n_pipelines, a.st, c, 0, 0, a.ktab + (size_t)c * a.st.stage_stride, scratch, sums_of(a, c)))
+  if (ctx_constants<true>(a.pipes, a.n_pipelines, a.st, c, 0, 0, a.ktab + (size_t)c * a.st.stage_stride, scratch, sums_of(a, c)))
     set_status(hdr, PARD_EDATA);
 }
 __device__ __noinline__ void const_tail(const ConstArgs& a, const unsigned long long* ctx_dmin_inv, const unsigned long long* ctx_dmax,
@@ -323,15 +436,16 @@ __device__ __noinline__ void const_tail(const ConstArgs& a, const unsigned long 
   if (last_block_done(&hdr->seg_done)) finish_constants<true>(a, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
-/* const_blocks: so many further blocks, the first ones of the grid, work out the queues' constants
- * meanwhile -- a chain of dependent loads that needs no deadline --, and the block that finishes last
+/* const_blocks: so many further blocks, the first ones of the grid, work out the queues' constants (which may also be
+ * there already) meanwhile -- a chain of dependent loads that needs no deadline --, and with `tail` the block that finishes last
  * completes them (one launch and its 8 us less for every call of up to 1,024 queues). */
 template <bool TABLE>
 __global__ void __launch_bounds__(256, 5)
 k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
           unsigned long long* __restrict__ ctx_dmin_inv, unsigned long long* __restrict__ ctx_dmax,
-          PlanHeader* hdr, uint32_t const_blocks, const __grid_constant__ ConstArgs ca) {
+          PlanHeader* hdr, uint32_t const_blocks, uint32_t tail, const __grid_constant__ ConstArgs ca) {
   pdl_wait();
+  if (hdr->direct) return;
   if (blockIdx.x < const_blocks) {
     const_block(ca, blockIdx.x, hdr);
     const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
@@ -524,25 +638,26 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       if (__ldcg(&ctx_dmax[c]) < hi) atomicMax(&ctx_dmax[c], hi);
     }
   }
-  if (const_blocks) const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
+  if (tail) const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
 constexpr uint32_t kPreTableCtx = 4096;          /* 32 KB of table: five blocks still fit a multiprocessor */
 void launch_prepass(const uint4* req, uint32_t n, uint32_t n_ctx, uint32_t S, unsigned long long* ctx_dmin_inv,
-                    unsigned long long* ctx_dmax, PlanHeader* hdr, uint32_t const_blocks, const ConstArgs& ca, int sms,
+                    unsigned long long* ctx_dmax, PlanHeader* hdr, uint32_t const_blocks, bool tail, const ConstArgs& ca, int sms,
                     cudaStream_t stream) {
   const uint32_t grid = std::min<uint32_t>((n + 256 * kPreUn - 1) / (256 * kPreUn), (uint32_t)sms * 5);
   /* the table pays once a block has more requests than the table has entries to clear and hand over */
   if (n_ctx > 1 && n_ctx <= kPreTableCtx && n / grid >= 2 * n_ctx)
-    launch_pdl(k_prepass<true>, const_blocks + grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
+    launch_pdl(k_prepass<true>, const_blocks + grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, tail ? 1u : 0u, ca);
   else
-    launch_pdl(k_prepass<false>, const_blocks + grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
+    launch_pdl(k_prepass<false>, const_blocks + grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, tail ? 1u : 0u, ca);
 }
 
 __global__ void k_ctx_span(const unsigned long long* __restrict__ ctx_dmin_inv,
                            const unsigned long long* __restrict__ ctx_dmax, uint32_t n_ctx,
                            PlanHeader* hdr) {
   pdl_wait();
+  if (hdr->direct) return;
   uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long span = 0;
   if (c < n_ctx && ~ctx_dmin_inv[c] <= ctx_dmax[c]) span = ctx_dmax[c] - ~ctx_dmin_inv[c];
@@ -556,6 +671,7 @@ __global__ void k_ctx_span(const unsigned long long* __restrict__ ctx_dmin_inv,
 __global__ void k_key_width(uint32_t sbits, uint32_t ibits, PlanHeader* hdr, uint32_t arrival_order, uint32_t key_sbits,
                             uint32_t priority) {
   pdl_wait();
+  if (hdr->direct) return;
   set_key_width(hdr, hdr->span_max, sbits, ibits, key_sbits, arrival_order, priority != 0);
 }
 
@@ -588,7 +704,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
   __shared__ long long s_A[WIN ? kHistSegs : 1], s_d[WIN ? kHistSegs : 1];
   __shared__ unsigned long long s_magic[WIN ? kHistSegs : 1];
   __shared__ uint4 s_wcon[WIN ? kHistSegs : 1];            /* per queue: A_rel, first table entry, entries, A_rel and d fit 32 bits */
-  if (hdr->wide || sort_is_local(hdr, local_candidate)) return;   /* sorted block by block: k_sort_local read the requests itself */
+  if (hdr->direct || hdr->wide || sort_is_local(hdr, local_candidate)) return;   /* sorted block by block: k_sort_local read the requests itself */
   const uint32_t npass = hdr->npass, dbits = hdr->dbits, pshift = hdr->pshift;
   for (uint32_t i = threadIdx.x; i < npass * kBins; i += blockDim.x) s_hist[i] = 0;
   /* The counters are kept in as many copies as fit (a power of two, at most one per lane), lane l
@@ -845,7 +961,7 @@ struct WinCountArgs {
   const uint32_t* hist;
 };
 __device__ __noinline__ void win_from_counts(PlanHeader* hdr, const WinCountArgs& a) {
-  if (hdr->wide) return;
+  if (hdr->wide || hdr->direct) return;
   const uint32_t n_seg = a.n_seg;
   __shared__ uint32_t s_len[kHistSegs], s_kept[kHistSegs];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1019,14 +1135,6 @@ __device__ __forceinline__ void sort_rank_drop(const unsigned long long (&key)[C
  * traffic (16.2 us against 14.5 us at 2^20 elements), so wider digits stay on the generic code.
  * The 89 us are what a pass costs with ranking almost free: tile load, write-out, scans and
  * barriers.  Full tiles only (no padding keys). */
-template <int BITS>
-__device__ __forceinline__ uint32_t digit_peers(uint32_t d, const uint32_t (&bal)[BITS]) {
-  uint32_t m = 0xffffffffu;
-#pragma unroll
-  for (int k = 0; k < BITS; ++k) m &= ((d >> k) & 1u) ? bal[k] : ~bal[k];
-  return m;
-}
-
 template <int ITEMS, int BITS, bool L2, int CAP>
 __device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[CAP], const unsigned long long* src,
                                                     uint64_t first, uint32_t shift, uint32_t* slot_row, uint32_t lane, int items) {
@@ -1310,7 +1418,7 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  if (pass >= hdr->npass || sort_is_local(hdr, local_candidate)) return;
+  if (hdr->direct || pass >= hdr->npass || sort_is_local(hdr, local_candidate)) return;
   sort_tiles<false, CTX, false>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
                                 stall, ct, 0u);
 }
@@ -1336,7 +1444,7 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  if (sort_is_local(hdr, local_candidate) || gave_up(hdr)) return;
+  if (hdr->direct || sort_is_local(hdr, local_candidate) || gave_up(hdr)) return;
   const uint32_t npass = hdr->npass;
   const uint32_t tile_size = SMALL ? 256u * ((geometry & 255u) + (geometry >> 8)) : (uint32_t)kSortTile;
   const uint32_t tiles = CTX ? ct.tile_first[ct.n_ctx] : (uint32_t)(((uint64_t)n + tile_size - 1) / tile_size);
@@ -1357,8 +1465,9 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
 /* First tile of every ctx when the tiles are cut at ctx boundaries: the running sum of
  * ceil(requests of the ctx / kSortTile).  One block. */
 __global__ void __launch_bounds__(1024)
-k_tile_table(const uint32_t* __restrict__ ctx_start, uint32_t n_ctx, uint32_t* __restrict__ tile_first) {
+k_tile_table(const uint32_t* __restrict__ ctx_start, uint32_t n_ctx, uint32_t* __restrict__ tile_first, const PlanHeader* hdr) {
   pdl_wait();
+  if (hdr->direct) return;
   __shared__ uint32_t s_w[32];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t per = (n_ctx + 1023) / 1024;          /* contexts per thread, consecutive */
@@ -1406,7 +1515,7 @@ k_pack_ctx(const uint4* __restrict__ req, uint32_t S, const unsigned long long* 
   if (threadIdx.x == 0) {
     const bool unsorted = ld_relaxed(&hdr->unsorted) != 0;       /* found out of ctx order, by k_ctx_ranges or a block of this kernel (see gave_up) */
     if (unsorted && tile == 0) { hdr->aborted = 1; set_status(hdr, PARD_EDATA); }
-    s_skip = unsorted || hdr->wide || ld_relaxed(&hdr->aborted) ? 1u : 0u;
+    s_skip = unsorted || hdr->direct || hdr->wide || ld_relaxed(&hdr->aborted) ? 1u : 0u;
   }
   __syncthreads();
   if (s_skip) return;
@@ -1497,6 +1606,7 @@ __global__ void __launch_bounds__(256)
 k_ctx_ranges(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t* __restrict__ ctx_start,
              PlanHeader* hdr) {
   pdl_wait();
+  if (hdr->direct) return;
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (c <= n_ctx) ctx_range_search(req, n, n_ctx, c, ctx_start, hdr, (uint32_t)kSortTile);   /* whole warps stay together */
 }
@@ -1513,6 +1623,7 @@ k_sort_local(PlanHeader* __restrict__ hdr, uint32_t candidate, const uint4* __re
              unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ ctx_start, uint32_t n,
              uint32_t S, uint32_t stage_bits, uint32_t ibits) {
   pdl_wait();
+  if (hdr->direct) return;
   constexpr int WARPS = kSortThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SortSmem& Sm = *reinterpret_cast<SortSmem*>(smem_raw);
@@ -1827,88 +1938,6 @@ __device__ void tile_agg_tiles(const PlanHeader* __restrict__ hdr, const unsigne
   }
 }
 
-/* Kept requests per queue -> first output slot of every queue, the number of
- * kCompactChunk-sized copy jobs before every queue, and the total.  One block,
- * eight queues per thread and round. */
-template <int THREADS>
-__device__ void kept_scan_block(const uint32_t* seg_kept, uint32_t n_seg, uint32_t* kept_base,
-                                uint32_t* chunk_base, uint32_t* out_seg_kept, unsigned long long* out_n_kept) {
-  constexpr int PER = 8, WARPS = THREADS / 32;
-  __shared__ uint32_t s_a[32], s_b[32];
-  __shared__ uint32_t s_ca, s_cb;
-  if (threadIdx.x == 0) { s_ca = 0; s_cb = 0; }
-  __syncthreads();
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  /* a thread's eight entries as two 16-byte accesses where the arrays allow it */
-  const bool vec_in = ((uintptr_t)seg_kept & 15) == 0;
-  const bool vec_out = (((uintptr_t)kept_base | (uintptr_t)chunk_base) & 15) == 0;
-  const bool vec_user = out_seg_kept && ((uintptr_t)out_seg_kept & 15) == 0;
-  for (uint32_t base = 0; base < n_seg + 1; base += THREADS * PER) {
-    const uint32_t i0 = base + threadIdx.x * PER;
-    uint32_t v[PER], c[PER], x = 0, y = 0;
-    if (vec_in && i0 + PER <= n_seg) {
-      /* (L2 loads here and in kept_move_jobs: inside k_scan_path other blocks of the same kernel wrote these) */
-      const uint4 a = __ldcg(reinterpret_cast<const uint4*>(seg_kept + i0)), b = __ldcg(reinterpret_cast<const uint4*>(seg_kept + i0 + 4));
-      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    } else {
-#pragma unroll
-      for (int k = 0; k < PER; ++k) v[k] = i0 + k < n_seg ? __ldcg(&seg_kept[i0 + k]) : 0;
-    }
-    if (vec_user && i0 + PER <= n_seg) {
-      *reinterpret_cast<uint4*>(out_seg_kept + i0) = make_uint4(v[0], v[1], v[2], v[3]);
-      *reinterpret_cast<uint4*>(out_seg_kept + i0 + 4) = make_uint4(v[4], v[5], v[6], v[7]);
-    } else if (out_seg_kept) {
-#pragma unroll
-      for (int k = 0; k < PER; ++k) if (i0 + k < n_seg) out_seg_kept[i0 + k] = v[k];
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      c[k] = (v[k] + kCompactChunk - 1) / kCompactChunk;
-      x += v[k];
-      y += c[k];
-    }
-    const uint32_t tx = x, ty = y;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
-      if (lane >= (uint32_t)o) { x += p; y += q; }
-    }
-    if (lane == 31) { s_a[warp] = x; s_b[warp] = y; }
-    __syncthreads();
-    if (warp == 0) {
-      const uint32_t a = lane < WARPS ? s_a[lane] : 0u, b = lane < WARPS ? s_b[lane] : 0u;
-      uint32_t ta = a, tb = b;
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t p = __shfl_up_sync(0xffffffffu, ta, o), q = __shfl_up_sync(0xffffffffu, tb, o);
-        if (lane >= (uint32_t)o) { ta += p; tb += q; }
-      }
-      s_a[lane] = ta - a;
-      s_b[lane] = tb - b;
-    }
-    __syncthreads();
-    uint32_t ea = s_ca + s_a[warp] + x - tx, eb = s_cb + s_b[warp] + y - ty;   /* exclusive, before this thread's queues */
-    uint32_t oa[PER], ob[PER];
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      oa[k] = ea; ob[k] = eb;
-      ea += v[k];
-      eb += c[k];
-    }
-    if (vec_out && i0 + PER <= n_seg + 1) {
-      *reinterpret_cast<uint4*>(kept_base + i0) = make_uint4(oa[0], oa[1], oa[2], oa[3]);
-      *reinterpret_cast<uint4*>(kept_base + i0 + 4) = make_uint4(oa[4], oa[5], oa[6], oa[7]);
-      *reinterpret_cast<uint4*>(chunk_base + i0) = make_uint4(ob[0], ob[1], ob[2], ob[3]);
-      *reinterpret_cast<uint4*>(chunk_base + i0 + 4) = make_uint4(ob[4], ob[5], ob[6], ob[7]);
-    } else {
-#pragma unroll
-      for (int k = 0; k < PER; ++k) if (i0 + k <= n_seg) { kept_base[i0 + k] = oa[k]; chunk_base[i0 + k] = ob[k]; }
-    }
-    __syncthreads();
-    if (threadIdx.x == THREADS - 1) { s_ca = ea; s_cb = eb; }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && out_n_kept) *out_n_kept = s_ca;
-}
-
 /* Decision pass over tiles [first, end) of kDecTile sorted elements; a thread owns kDecItems consecutive
  * elements of a tile.
  *
@@ -2096,6 +2125,7 @@ k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const u
           uint32_t* __restrict__ kept_base, uint32_t* __restrict__ chunk_base, uint32_t* __restrict__ out_seg_kept,
           unsigned long long* __restrict__ out_n_kept) {
   pdl_wait();
+  if (hdr->direct) return;
   __shared__ uint32_t s_lo[kWinQueues + 1], s_w[kWinQueues], s_first[kWinQueues + 1];
   __shared__ long long s_A[kWinQueues], s_d[kWinQueues];
   __shared__ uint32_t s_base, s_scan;
@@ -2261,6 +2291,7 @@ k_windows_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, co
                uint32_t* __restrict__ seg_kept, uint32_t* __restrict__ kept_base, uint32_t* __restrict__ chunk_base,
                uint32_t* __restrict__ out_seg_kept, unsigned long long* __restrict__ out_n_kept) {
   pdl_wait();
+  if (hdr->direct) return;
   __shared__ uint32_t s_lo[kWinThreads], s_warp[kWinThreads / 32], s_base, s_scan;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t s = blockIdx.x * (kWinThreads - 1u) + tid;          /* the last thread only finds the end of the one before */
@@ -2367,7 +2398,7 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
   /* The queues' kept counts followed from their tables, so the survivors go straight to their final
    * place: kept_base holds the queues' output offsets. */
   pdl_wait();
-  if (hdr->use_scan || hdr->wide || hdr->aborted) return;
+  if (hdr->direct || hdr->use_scan || hdr->wide || hdr->aborted) return;
   const TileCtx T = make_tile_ctx(hdr, buf_a, buf_b, n, ibits, ktab, seg_off);
   const uint64_t base = ((uint64_t)blockIdx.x * kDecThreads + threadIdx.x) * kDecItems;
   if (base >= n) return;
@@ -2942,7 +2973,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  stream, (uint4*)(ws + L.hdr), n16);
     }
     ConstArgs ca = const_args();
-    launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, 0u, ca, sms, stream);
+    launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, 0u, false, ca, sms, stream);
     launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
     launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, 0u, sbits, 1u);
     launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
@@ -3010,8 +3041,18 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     return rc == PARD_ERANGE ? plan_wide() : rc;
   }
 
+  /* ---- requests grouped by ctx (the caller's word, contexts of more than a tile on average) may stand in order
+   * already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
+   * 288 k of 24 contexts 71 -> 51; out of order they pay for the try, 567 -> 575 and 117 -> 118.  Without the caller's
+   * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
+  DirectArgs da = {};
+  const bool direct = (mode & PARD_MODE_GROUPED) && L.ctx_passes && !rule_walk && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN | PARD_MODE_TEST_STALL)) &&
+                      !state->d_priority && dir_layout(n, n_ctx, S, (char*)buf_b, &da);
+  da.req = req4; da.n = n32; da.n_ctx = n_ctx; da.S = S; da.sbits = sbits; da.ibits = ibits;
+  da.ktab = ktab; da.ctx_start = ctx_start; da.const_bad = kept_tmp;
+
   /* ---- clear the scratch that must start at zero: one contiguous region ---- */
-  {
+  if (!direct) {
     const unsigned long long n16 = (n > 0 ? L.zero_end : L.lookback) / 16;   /* offsets are multiples of 256 */
     launch_pdl(k_clear, (uint32_t)std::min<unsigned long long>((n16 + 255) / 256, (unsigned long long)sms * 4), 256, 0,
                stream, (uint4*)(ws + L.hdr), n16);
@@ -3035,20 +3076,40 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   /* known paths: the paths' sums are written down beside the constants, in the survivors' scratch, where
    * they fit (queues of 32 requests on average); else blocks work them out again (stage_paths) */
   ca.path_sums = (mode & PARD_MODE_PATH_MASK) && n >= 2ull * kMaskPaths * L.n_seg ? (long long*)kept_tmp : nullptr;
-  const uint32_t const_blocks = n > 0 && L.n_seg <= kFoldSegs && ca.with_key_width ? n_ctx : 0u;
+  const bool const_fold = n > 0 && L.n_seg <= kFoldSegs && ca.with_key_width;
+  if (direct) {
+    const unsigned long long n16 = L.zero_end / 16;
+    const uint32_t range_blocks = (n_ctx + kDirWarps - 1) / kDirWarps;
+    launch_pdl(k_dir_begin, n_ctx + range_blocks + (uint32_t)std::min<unsigned long long>((n16 + 255) / 256, (unsigned long long)sms * 4), kDirThreads, 0,
+               stream, da, ca, (uint4*)(ws + L.hdr), n16, range_blocks);
+  }
   mark();
-  if (n > 0) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_blocks, ca, sms, stream);
+  /* on the caller's word that the requests come grouped k_dir_count finds what the prepass would */
+  const bool direct_ranges = direct && ctx_sort;
+  if (direct)
+    launch_pdl(S > 8 ? k_dir_count<4> : k_dir_count<3>, da.n_pieces, kDirThreads, 0, stream, da, ca, hdr, ctx_dmin, ctx_dmax,
+               direct_ranges ? 1u : 0u);
+  if (n > 0 && !direct_ranges) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_fold && !direct ? n_ctx : 0u, const_fold, ca, sms, stream);
   mark();
   if (!ca.with_key_width) {
     if (n > 0) launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
     launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, arrival_order ? 1u : 0u, key_sbits, state->d_priority ? 1u : 0u);
   }
-  if (!const_blocks)
+  if (!const_fold && direct)
+    launch_pdl(k_seg_finish, (L.n_seg + 255) / 256, 256, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
+  else if (!const_fold)
     launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
-  if ((local_cand && !local_sure) || ctx_sort)
+  if ((local_cand && !local_sure) || (ctx_sort && !direct))
     launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr);
-  if (ctx_sort) launch_pdl(k_tile_table, 1, 1024, 0, stream, (const uint32_t*)ctx_start, n_ctx, (uint32_t*)(ws + L.tile_first));
+  if (ctx_sort) launch_pdl(k_tile_table, 1, 1024, 0, stream, (const uint32_t*)ctx_start, n_ctx, (uint32_t*)(ws + L.tile_first), (const PlanHeader*)hdr);
   mark();
+  if (direct) {
+    const DirScanOut scan_out = {seg_off, out->d_seg_offsets, seg_kept, kept_base, chunk_base, out->d_seg_kept, (unsigned long long*)out->d_n_kept};
+    launch_pdl(k_dir_scan, n_ctx, kDirScanThreads, 0, stream, da, hdr, scan_out);
+    launch_pdl(S > 8 ? k_dir_emit<4> : k_dir_emit<3>, std::min<uint32_t>(da.n_pieces, (uint32_t)sms * 4), kDirThreads, sizeof(EmitSmem), stream,
+               da, hdr, (const uint32_t*)seg_off, (const uint32_t*)kept_base, out->d_keep, (long long*)out->d_est_us, out->d_perm,
+               out->d_kept_idx);
+  }
   if (local_cand)                                /* every ctx inside one tile: sorted block by block, straight from the requests */
     launch_pdl(k_sort_local, n_ctx, kSortThreads, sizeof(SortSmem), stream, hdr, local_cand, req4, ctx_dmin, ctx_dmax,
                state->d_priority, buf_a, buf_b, local_sure ? (const uint32_t*)nullptr : (const uint32_t*)ctx_start, n32, S,

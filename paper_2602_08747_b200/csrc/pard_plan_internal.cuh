@@ -66,7 +66,11 @@ struct PlanHeader {
   uint32_t pair_steps_back;   /* 1: some request's (ctx, deadline) lies before its predecessor's */
   uint32_t lookup;            /* 1: the elements hold no deadline: it has to be looked up in the request array */
   uint32_t sort_bar[kMaxPasses]; /* tiles of each of k_sort_rest's passes that are finished */
-  uint32_t pad[64 - 26 - kMaxPasses - (kMaxPasses + 1)];
+  uint32_t direct;            /* 1: the requests came in order, the plan is made without a sort (pard_direct.cuh) */
+  uint32_t direct_off;        /* 1: they did not, or something else that path does not take */
+  uint32_t direct_done;       /* blocks of k_dir_count that have finished */
+  uint32_t direct_ticket;     /* pieces taken by k_dir_emit */
+  uint32_t pad[64 - 30 - kMaxPasses - (kMaxPasses + 1)];
 };
 static_assert(sizeof(PlanHeader) == 256, "header is 256 bytes");
 
@@ -131,7 +135,9 @@ __device__ __forceinline__ int32_t narrow_A(const PardSegConst& K) {
  * of range.  Bound by dependent loads (pipeline -> profile offsets -> durations; slot -> path ->
  * durations): with the durations of all stages fetched side by side first, a path costs one load
  * per stage instead of a chain of three.  One warp per queue that walked its paths on its own took
- * 10 us for 16 queues and 37 us for 32,768.  sums: the ctx's rows of PolicyArgs::path_sums, or null. */
+ * 10 us for 16 queues and 37 us for 32,768.  AHEAD: a thread requests what belongs to its own stage and slot at once
+ * (9.0 -> 7.0 us for the constants of one ctx; not in k_plan_local, which has no registers left for it: 4,096 epochs
+ * 391 -> 395 us).  sums: the ctx's rows of PolicyArgs::path_sums, or null. */
 constexpr int kMaskPaths = 16;                     /* bits of pard_request_t.flags: paths of a stage that a request can name */
 constexpr int kConstThreads = 64;                  /* k_seg_const's blocks; any number of threads will do */
 struct CtxScratch {
@@ -140,34 +146,58 @@ struct CtxScratch {
   unsigned long long lsub[PARD_MAX_STAGES];
   int32_t slot_off[PARD_MAX_STAGES + 1];
 };
+template <bool AHEAD>
 __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n_pipelines, const pard_queue_state_t& st, uint32_t c,
                                               unsigned long long dmin, unsigned long long dmax, PardSegConst* K_out,
                                               CtxScratch& sc, long long* sums = nullptr) {
   const uint32_t S = (uint32_t)st.stage_stride, tid = threadIdx.x, nt = blockDim.x;
   const int32_t pi = st.d_pipeline_of_ctx ? st.d_pipeline_of_ctx[c] : 0;
+  /* a thread's own stage and slot: all that does not hang on the pipeline, requested at once */
+  int32_t B_own = 1, m_own = 1;
+  int64_t q_own = 0, fa_own = 0, w_own = 0, now_own = 0;
+  bool high_own = false;
+  if (AHEAD) {
+    now_own = st.d_now_us[c];
+    if (tid < S) {
+      const size_t at = (size_t)c * S + tid;
+      B_own = st.d_batch[at];
+      q_own = st.d_q_us[at];
+      fa_own = st.d_free_at_us[at];
+      if (st.d_workers) m_own = st.d_workers[at];
+      if (st.d_priority) high_own = st.d_priority[at] != 0;
+    }
+    if (st.d_w_us && tid < (uint32_t)st.slot_stride) w_own = st.d_w_us[(size_t)c * st.slot_stride + tid];
+  }
   const PardPipeDev* p = nullptr;
   if (pi >= 0 && (uint32_t)pi < n_pipelines) p = n_pipelines <= (uint32_t)kFewPipelines ? pipes.few[pi] : pipes.many[pi];
   bool bad = p == nullptr;
-  const uint32_t stages = p ? (uint32_t)p->n_stages : 0u;   /* <= S: checked on the host */
-  const int32_t n_slots = p ? p->n_slots : 0;
+  PardPipeDev head = {};
+  if (AHEAD && p) head = *p;
+  const PardPipeDev* const P = AHEAD ? &head : p;
+  const uint32_t stages = p ? (uint32_t)P->n_stages : 0u;   /* <= S: checked on the host */
+  const int32_t n_slots = p ? P->n_slots : 0;
   const size_t row = (size_t)c * S;
+  int32_t e0_own = 0, e1_own = 0;
+  if (AHEAD && (int32_t)tid < n_slots) { e0_own = P->path_off[tid]; e1_own = P->path_off[tid + 1]; }
   for (uint32_t k = tid; k < stages; k += nt) {
-    const int32_t B = st.d_batch[row + k];
-    const int64_t q = st.d_q_us[row + k];
-    const bool ok = B >= 1 && B <= p->bmax[k];
-    const long long d = p->lat_us[p->lat_offsets[k] + (ok ? B : 1) - 1];
+    const bool own = AHEAD && k == tid;
+    const int32_t B = own ? B_own : st.d_batch[row + k];
+    const int64_t q = own ? q_own : st.d_q_us[row + k];
+    const bool ok = B >= 1 && B <= P->bmax[k];
+    const long long d = P->lat_us[P->lat_offsets[k] + (ok ? B : 1) - 1];
     sc.dur[k] = d;
     sc.delay[k] = ok && q >= 0 && q < PARD_TIME_LIMIT_US ? q + d : -1;
     sc.lsub[k] = 0;
-    sc.slot_off[k] = p->stage_slot_off[k];
+    sc.slot_off[k] = P->stage_slot_off[k];
   }
   __syncthreads();
   for (int32_t s = (int32_t)tid; s < n_slots; s += (int32_t)nt) {
-    int64_t acc = st.d_w_us ? st.d_w_us[(size_t)c * st.slot_stride + s] : 0;
+    const bool own = AHEAD && s == (int32_t)tid;
+    int64_t acc = own ? w_own : st.d_w_us ? st.d_w_us[(size_t)c * st.slot_stride + s] : 0;
     if (acc < 0 || acc >= PARD_TIME_LIMIT_US) { bad = true; acc = 0; }
-    const int32_t e1 = p->path_off[s + 1];
-    for (int32_t e = p->path_off[s]; e < e1; ++e) {
-      const long long t = sc.delay[p->path_stage[e]];
+    const int32_t e1 = own ? e1_own : P->path_off[s + 1];
+    for (int32_t e = own ? e0_own : P->path_off[s]; e < e1; ++e) {
+      const long long t = sc.delay[P->path_stage[e]];
       if (t < 0) bad = true;
       else acc += t;
     }
@@ -190,10 +220,12 @@ __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n
     if (p && k >= stages) {
       out.narrow = kSegNoStage;                    /* no such stage: a request found in this queue is an input error */
     } else if (p) {
-      const int32_t B = st.d_batch[row + k];
-      const int64_t m = st.d_workers ? st.d_workers[row + k] : 1;
-      const int64_t now = st.d_now_us[c], fa = st.d_free_at_us[row + k];
-      if (B < 1 || B > p->bmax[k] || m < 1 || now < 0 || now >= PARD_TIME_LIMIT_US || fa < 0 || fa >= PARD_TIME_LIMIT_US) {
+      const bool own = AHEAD && k == tid;
+      const int32_t B = own ? B_own : st.d_batch[row + k];
+      const int64_t now = AHEAD ? now_own : st.d_now_us[c];
+      const int64_t m = own ? m_own : st.d_workers ? st.d_workers[row + k] : 1;
+      const int64_t fa = own ? fa_own : st.d_free_at_us[row + k];
+      if (B < 1 || B > P->bmax[k] || m < 1 || now < 0 || now >= PARD_TIME_LIMIT_US || fa < 0 || fa >= PARD_TIME_LIMIT_US) {
         bad = true;
       } else {
         const int64_t d = sc.dur[k], lsub = (int64_t)sc.lsub[k], base = now > fa ? now : fa, cap = (int64_t)B * m;
@@ -202,7 +234,7 @@ __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n
         out.A = base + d + lsub;
         /* A against the origin of the queue's deadline offsets: offsets count up from the ctx's
          * smallest deadline, or, for a queue served high budget first, down from its largest */
-        const bool high_first = st.d_priority && st.d_priority[row + k] != 0;
+        const bool high_first = own ? high_own : st.d_priority && st.d_priority[row + k] != 0;
         out.A_rel = high_first ? (int64_t)dmax - out.A : out.A - (int64_t)dmin;
         out.d_magic = (d >= 2 && d < ((int64_t)1 << 32)) ? magic64((uint64_t)d) : 0;
         out.cap_magic = out.cap >= 2 ? magic64(out.cap) : 0;

@@ -1,0 +1,88 @@
+"""Grouped contexts whose requests come in order are planned without a sort: at the edges of its tiles (1,792 requests)
+and pieces (up to four tiles), with constants at the limits of its 32-bit arithmetic, and with the one request that
+sends the call to the general path, against the oracle (whole numbers: bit for bit)."""
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2602_08747_b200 import binding as pb
+from paper_2602_08747_b200 import inputs
+from tests import util
+from tests.gpu_util import assert_identical, run_library
+from tests.test_kernel_variants_gpu import booked, several_ctx
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [0, 1, 1791, 1792, 1793, 7167, 7168, 7169, 14_337, 40_000, 0, 30_000]
+
+
+def check(wl, mode=pb.PARD_MODE_GROUPED):
+    rc, got = run_library(wl, mode)
+    assert rc == 0
+    assert_identical(got, oracle.plan(wl.pipelines, wl.requests, wl.state, wl.n_ctx, 0))
+
+
+@pytest.mark.parametrize("S", [1, 3, 4, 8, 9, 16, 17])
+@pytest.mark.parametrize("span,B,m", [(3000, 2, 1), (40_000, 3, 7), (2_000_000_000, 4, 1), (10, 1, 1), (100_000, 2, 5000)])
+def test_sizes_at_the_edges_of_tiles_and_pieces(S, span, B, m):
+    check(several_ctx(len(EDGES), EDGES, seed=S, S=S, span=span, B=B, m=m))
+    big = [16_384, 16_385, 65_536, 200_000]               # pieces of more than one tile from a million requests on
+    if S == 8:
+        check(several_ctx(20, big * 5, seed=7, S=S, span=span, B=B, m=m))
+
+
+@pytest.mark.parametrize("S", [4, 16])
+def test_one_queue_holds_nearly_all(S):
+    wl = several_ctx(3, [20_000, 9_000, 30_000], S=S, span=50_000, m=30)
+    wl.requests["stage"] = np.where(np.arange(wl.n) % 997 == 0, wl.requests["stage"], S - 1)
+    check(wl)
+    wl.requests["stage"] = 0
+    check(wl)
+
+
+@pytest.mark.parametrize("at", [1, 1791, 1792, 20_000, 38_999])
+def test_one_deadline_steps_back(at):
+    for S in (3, 8):
+        wl = several_ctx(4, [20_000, 0, 9_000, 10_000], S=S)
+        wl.requests["deadline_us"][at] = 0
+        check(wl)
+
+
+@pytest.mark.parametrize("span", [3000, (1 << 31) - 3, (1 << 31) - 2, (1 << 31) - 1, 1 << 31, 1 << 33])
+@pytest.mark.parametrize("d", [1, 7, (1 << 31) + 9, (1 << 32) + 9])
+def test_constants_at_the_limits(span, d):
+    targets = [0, 1, span, span + 2, (1 << 31) - 2, (1 << 31) - 1, 1 << 31, 1 << 40, -1, -(1 << 31), -(1 << 31) - 1]
+    wl = booked(targets, span, d, n=8300)
+    check(wl)
+    for t in targets:                                     # without a ctx that the path does not take
+        check(booked([t, t], span, d, n=8300))
+
+
+def test_errors_are_still_reported():
+    def rc(wl):
+        return run_library(wl, pb.PARD_MODE_GROUPED, check=False)[0]
+
+    for S in (4, 3):                                      # with passes inside the contexts, and without
+        wl = several_ctx(3, [20_000, 9_000, 10_000], S=S)
+        for field, value in (("stage", S), ("ctx", 3), ("deadline_us", -1), ("deadline_us", 1 << 60)):
+            for at in (0, 25_000, wl.n - 1):
+                bad = inputs.Workload("bad", wl.pipelines, wl.requests.copy(), wl.state, wl.n_ctx)
+                bad.requests[field][at] = value
+                assert rc(bad) == pb.PARD_EDATA, (field, at)
+        check(wl)
+    wl = several_ctx(3, [20_000, 9_000, 10_000], S=4)
+    wl.requests["ctx"][100] = 1                           # not grouped
+    assert rc(wl) == pb.PARD_EDATA
+    wl = several_ctx(3, [20_000, 9_000, 10_000], S=4)
+    wl.state.batch[1, 2] = 0                              # constants out of range, of an empty ctx and of one with requests
+    for sizes in ([20_000, 0, 10_000], [20_000, 9_000, 10_000]):
+        for sort in (True, False):
+            assert rc(inputs.Workload("bad", wl.pipelines, several_ctx(3, sizes, S=4, sort=sort).requests, wl.state, 3)) == pb.PARD_EDATA
+    wl = several_ctx(3, [20_000, 9_000, 10_000], S=4)
+    short = util.pipeline(inputs.chain_edges(2), 2, [10, 20], bmax=4)     # a queue its pipeline lacks
+    wl.pipelines = [wl.pipelines[0], short]
+    wl.state.pipeline_of_ctx = np.array([0, 1, 0], np.int32)
+    assert rc(wl) == pb.PARD_EDATA
+    keep = ~((wl.requests["ctx"] == 1) & (wl.requests["stage"] >= 2))
+    wl.requests = np.ascontiguousarray(wl.requests[keep])
+    check(wl)
