@@ -7,8 +7,8 @@
  * u_t - t over them.  Both combine over consecutive spans, so the plan takes two reads of the requests and
  * nothing else:
  *   k_dir_begin   the queues' constants; the pieces, runs of tiles of one ctx; the scratch cleared
- *   k_dir_count   (count, minimum) of every queue, per piece; checks the order; where the sort that comes else needs
- *                 it, also what k_prepass finds, so that nothing is read twice when the order is not there
+ *   k_dir_count   (count, minimum) of every queue, per piece; checks the order; also finds what k_prepass would, so
+ *                 that nothing is read twice when the order is not there
  *   k_dir_scan    their running values over the pieces of every ctx, queue boundaries, kept counts, offsets
  *   k_dir_emit    every tile's requests ordered by stage in shared memory, decided, written to their place
  * What the path does not take -- deadlines that step back, requests not grouped, input errors, constants
@@ -203,7 +203,7 @@ k_dir_scan(const __grid_constant__ DirectArgs a, PlanHeader* hdr, const __grid_c
 template <int BITS>
 __global__ void __launch_bounds__(kDirThreads, 4)
 k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstArgs ca, PlanHeader* hdr,
-            unsigned long long* __restrict__ ctx_dmin_inv, unsigned long long* __restrict__ ctx_dmax, uint32_t ranges) {
+            unsigned long long* __restrict__ ctx_dmin_inv, unsigned long long* __restrict__ ctx_dmax) {
   pdl_wait();
   constexpr int kUn = 4;
   __shared__ DirConst s_K[kDirWarps][kDirStages];
@@ -241,7 +241,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   }
   if (gaps) {
     off = true;
-    if (ranges) hdr->unsorted = 1;                /* not grouped as the caller said: reported by k_pack_ctx */
+    hdr->unsorted = 1;                            /* not grouped as the caller said: reported by k_pack_ctx */
   }
   auto deadline = [&](uint32_t j) { return __ldg(reinterpret_cast<const unsigned long long*>(&a.req[j])); };
   const unsigned long long D0 = !off && begin < end ? deadline(begin) : 0ull;
@@ -319,7 +319,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
       lmax = deadline(wend - 1);
     }
   }
-  if (off && ranges) {                            /* what k_prepass would find: the deadlines' range, input errors */
+  if (off) {                            /* what k_prepass would find: the deadlines' range, input errors */
     bool bad = false, foreign = nonsense;
     lmin = ~0ull;
     lmax = 0;
@@ -355,7 +355,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   if (lane < kDirStages) s_warp[warp][lane] = figures();
   if (lane == 0) { s_min[warp] = lmin; s_max[warp] = lmax; }
   const bool block_off = __syncthreads_or(off);
-  if (ranges && tid == 0) {
+  if (tid == 0) {
     for (int w = 1; w < kDirWarps; ++w) {
       lmin = s_min[w] < lmin ? s_min[w] : lmin;
       lmax = s_max[w] > lmax ? s_max[w] : lmax;
@@ -367,10 +367,9 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   }
   if (block_off) {
     if (tid == 0 && !ld_relaxed(&hdr->direct_off)) {
-      if (ranges) hdr->time_steps_back = hdr->pair_steps_back = 1;   /* (or something else the path does not take: the sort then does more than it must) */
+      hdr->time_steps_back = hdr->pair_steps_back = 1;   /* (or something else the path does not take: the sort then does more than it must) */
       st_relaxed(&hdr->direct_off, 1u);
     }
-    if (!ranges) return;
   } else if (tid < kDirStages) {
     uint2 sum = make_uint2(0u, (uint32_t)kDirInf);
     for (int w = 0; w < kDirWarps; ++w) sum = dir_then(sum, s_warp[w][tid]);
@@ -379,7 +378,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   if (!last_block_done(&hdr->direct_done)) return;
   if (!ld_relaxed(&hdr->direct_off)) {
     if (tid == 0) hdr->direct = 1;
-  } else if (ranges && ca.with_key_width && a.n_ctx * a.S <= kFoldSegs) {
+  } else if (ca.with_key_width && a.n_ctx * a.S <= kFoldSegs) {
     finish_constants<true>(ca, ctx_dmin_inv, ctx_dmax, hdr);
   }
 }

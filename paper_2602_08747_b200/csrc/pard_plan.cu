@@ -388,7 +388,6 @@ __global__ void __launch_bounds__(kConstThreads)
 k_seg_const(const __grid_constant__ ConstArgs a, const unsigned long long* __restrict__ ctx_dmin_inv,
             const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr) {
   pdl_wait();
-  if (hdr->direct) return;
   __shared__ CtxScratch scratch;
   if (ctx_constants<true>(a.pipes, a.n_pipelines, a.st, blockIdx.x, ~ctx_dmin_inv[blockIdx.x], ctx_dmax[blockIdx.x],
                     a.ktab + (size_t)blockIdx.x * a.st.stage_stride, scratch, sums_of(a, blockIdx.x)))
@@ -436,16 +435,15 @@ __device__ __noinline__ void const_tail(const ConstArgs& a, const unsigned long 
   if (last_block_done(&hdr->seg_done)) finish_constants<true>(a, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
-/* const_blocks: so many further blocks, the first ones of the grid, work out the queues' constants (which may also be
- * there already) meanwhile -- a chain of dependent loads that needs no deadline --, and with `tail` the block that finishes last
+/* const_blocks: so many further blocks, the first ones of the grid, work out the queues' constants
+ * meanwhile -- a chain of dependent loads that needs no deadline --, and the block that finishes last
  * completes them (one launch and its 8 us less for every call of up to 1,024 queues). */
 template <bool TABLE>
 __global__ void __launch_bounds__(256, 5)
 k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
           unsigned long long* __restrict__ ctx_dmin_inv, unsigned long long* __restrict__ ctx_dmax,
-          PlanHeader* hdr, uint32_t const_blocks, uint32_t tail, const __grid_constant__ ConstArgs ca) {
+          PlanHeader* hdr, uint32_t const_blocks, const __grid_constant__ ConstArgs ca) {
   pdl_wait();
-  if (hdr->direct) return;
   if (blockIdx.x < const_blocks) {
     const_block(ca, blockIdx.x, hdr);
     const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
@@ -638,19 +636,19 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       if (__ldcg(&ctx_dmax[c]) < hi) atomicMax(&ctx_dmax[c], hi);
     }
   }
-  if (tail) const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
+  if (const_blocks) const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
 constexpr uint32_t kPreTableCtx = 4096;          /* 32 KB of table: five blocks still fit a multiprocessor */
 void launch_prepass(const uint4* req, uint32_t n, uint32_t n_ctx, uint32_t S, unsigned long long* ctx_dmin_inv,
-                    unsigned long long* ctx_dmax, PlanHeader* hdr, uint32_t const_blocks, bool tail, const ConstArgs& ca, int sms,
+                    unsigned long long* ctx_dmax, PlanHeader* hdr, uint32_t const_blocks, const ConstArgs& ca, int sms,
                     cudaStream_t stream) {
   const uint32_t grid = std::min<uint32_t>((n + 256 * kPreUn - 1) / (256 * kPreUn), (uint32_t)sms * 5);
   /* the table pays once a block has more requests than the table has entries to clear and hand over */
   if (n_ctx > 1 && n_ctx <= kPreTableCtx && n / grid >= 2 * n_ctx)
-    launch_pdl(k_prepass<true>, const_blocks + grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, tail ? 1u : 0u, ca);
+    launch_pdl(k_prepass<true>, const_blocks + grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
   else
-    launch_pdl(k_prepass<false>, const_blocks + grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, tail ? 1u : 0u, ca);
+    launch_pdl(k_prepass<false>, const_blocks + grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
 }
 
 __global__ void k_ctx_span(const unsigned long long* __restrict__ ctx_dmin_inv,
@@ -704,7 +702,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
   __shared__ long long s_A[WIN ? kHistSegs : 1], s_d[WIN ? kHistSegs : 1];
   __shared__ unsigned long long s_magic[WIN ? kHistSegs : 1];
   __shared__ uint4 s_wcon[WIN ? kHistSegs : 1];            /* per queue: A_rel, first table entry, entries, A_rel and d fit 32 bits */
-  if (hdr->direct || hdr->wide || sort_is_local(hdr, local_candidate)) return;   /* sorted block by block: k_sort_local read the requests itself */
+  if (hdr->wide || sort_is_local(hdr, local_candidate)) return;   /* sorted block by block: k_sort_local read the requests itself */
   const uint32_t npass = hdr->npass, dbits = hdr->dbits, pshift = hdr->pshift;
   for (uint32_t i = threadIdx.x; i < npass * kBins; i += blockDim.x) s_hist[i] = 0;
   /* The counters are kept in as many copies as fit (a power of two, at most one per lane), lane l
@@ -746,6 +744,8 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     const uint32_t up = 1u << ibits;
     uint32_t low = 0;                          /* low word of the ctx's smallest deadline */
     for (uint32_t j0 = blockIdx.x * blockDim.x + threadIdx.x; j0 < n; j0 += stride * kUn) {
+      if (threadIdx.x < kUn && n / 4 > stride * kUn)   /* the next round's requests, 256 in a row each (2^24: 5 us less; of three rounds: 1 us more) */
+        l2_ahead(reinterpret_cast<const unsigned long long*>(req), 2ull * (j0 - threadIdx.x), 2ull * stride * (kUn + threadIdx.x), 512, 2ull * n);
       uint4 rr[kUn];
 #pragma unroll
       for (int u = 0; u < kUn; ++u) {
@@ -961,7 +961,7 @@ struct WinCountArgs {
   const uint32_t* hist;
 };
 __device__ __noinline__ void win_from_counts(PlanHeader* hdr, const WinCountArgs& a) {
-  if (hdr->wide || hdr->direct) return;
+  if (hdr->wide) return;
   const uint32_t n_seg = a.n_seg;
   __shared__ uint32_t s_len[kHistSegs], s_kept[kHistSegs];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1248,6 +1248,7 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   if (CTX && S.ctx == 0xffffffffu) return true;
   if (CTX && tid < kBins) gh = ct.hist[((size_t)S.ctx * kMaxPasses + pass) * kBins + tid];
   const uint64_t base = CTX ? (uint64_t)S.base : (uint64_t)tile * tile_size;
+  if (!PERSIST && !CTX && tid == 0) l2_ahead(src, base, (uint64_t)kSortAhead * tile_size, tile_size, n);
   const uint32_t limit = CTX ? S.limit : n;            /* end of the range the tile belongs to */
   const int64_t lo_tile = CTX ? (int64_t)S.lo_tile : 0;
   const uint32_t shift = ibits + hdr->pshift + 8 * pass;
@@ -1418,7 +1419,7 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  if (hdr->direct || pass >= hdr->npass || sort_is_local(hdr, local_candidate)) return;
+  if ((CTX && hdr->direct) || pass >= hdr->npass || sort_is_local(hdr, local_candidate)) return;
   sort_tiles<false, CTX, false>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
                                 stall, ct, 0u);
 }
@@ -1444,7 +1445,7 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (wc.on && blockIdx.x == gridDim.x - 1) { win_from_counts(hdr, wc); return; }
-  if (hdr->direct || sort_is_local(hdr, local_candidate) || gave_up(hdr)) return;
+  if ((CTX && hdr->direct) || sort_is_local(hdr, local_candidate) || gave_up(hdr)) return;
   const uint32_t npass = hdr->npass;
   const uint32_t tile_size = SMALL ? 256u * ((geometry & 255u) + (geometry >> 8)) : (uint32_t)kSortTile;
   const uint32_t tiles = CTX ? ct.tile_first[ct.n_ctx] : (uint32_t)(((uint64_t)n + tile_size - 1) / tile_size);
@@ -1606,7 +1607,6 @@ __global__ void __launch_bounds__(256)
 k_ctx_ranges(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t* __restrict__ ctx_start,
              PlanHeader* hdr) {
   pdl_wait();
-  if (hdr->direct) return;
   const uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (c <= n_ctx) ctx_range_search(req, n, n_ctx, c, ctx_start, hdr, (uint32_t)kSortTile);   /* whole warps stay together */
 }
@@ -1623,7 +1623,6 @@ k_sort_local(PlanHeader* __restrict__ hdr, uint32_t candidate, const uint4* __re
              unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ ctx_start, uint32_t n,
              uint32_t S, uint32_t stage_bits, uint32_t ibits) {
   pdl_wait();
-  if (hdr->direct) return;
   constexpr int WARPS = kSortThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SortSmem& Sm = *reinterpret_cast<SortSmem*>(smem_raw);
@@ -2123,9 +2122,9 @@ k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const u
           WinEntry* __restrict__ wtab, uint32_t capacity, uint32_t force_scan, const uint32_t* __restrict__ hist, uint32_t sbits,
           uint32_t local_candidate, uint32_t tables, uint32_t raw, uint32_t* __restrict__ seg_kept,
           uint32_t* __restrict__ kept_base, uint32_t* __restrict__ chunk_base, uint32_t* __restrict__ out_seg_kept,
-          unsigned long long* __restrict__ out_n_kept) {
+          unsigned long long* __restrict__ out_n_kept, uint32_t direct) {
   pdl_wait();
-  if (hdr->direct) return;
+  if (direct && hdr->direct) return;               /* (direct: the call may have its plan already) */
   __shared__ uint32_t s_lo[kWinQueues + 1], s_w[kWinQueues], s_first[kWinQueues + 1];
   __shared__ long long s_A[kWinQueues], s_d[kWinQueues];
   __shared__ uint32_t s_base, s_scan;
@@ -2289,9 +2288,9 @@ k_windows_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, co
                uint32_t* __restrict__ out_seg_off, uint32_t* __restrict__ win_off, uint32_t* __restrict__ win_cnt,
                WinEntry* __restrict__ wtab, uint32_t capacity, uint32_t force_scan, uint32_t tables, uint32_t raw,
                uint32_t* __restrict__ seg_kept, uint32_t* __restrict__ kept_base, uint32_t* __restrict__ chunk_base,
-               uint32_t* __restrict__ out_seg_kept, unsigned long long* __restrict__ out_n_kept) {
+               uint32_t* __restrict__ out_seg_kept, unsigned long long* __restrict__ out_n_kept, uint32_t direct) {
   pdl_wait();
-  if (hdr->direct) return;
+  if (direct && hdr->direct) return;               /* (direct: the call may have its plan already) */
   __shared__ uint32_t s_lo[kWinThreads], s_warp[kWinThreads / 32], s_base, s_scan;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t s = blockIdx.x * (kWinThreads - 1u) + tid;          /* the last thread only finds the end of the one before */
@@ -2398,9 +2397,10 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
   /* The queues' kept counts followed from their tables, so the survivors go straight to their final
    * place: kept_base holds the queues' output offsets. */
   pdl_wait();
-  if (hdr->direct || hdr->use_scan || hdr->wide || hdr->aborted) return;
+  if (hdr->direct | hdr->use_scan | hdr->wide | hdr->aborted) return;
   const TileCtx T = make_tile_ctx(hdr, buf_a, buf_b, n, ibits, ktab, seg_off);
   const uint64_t base = ((uint64_t)blockIdx.x * kDecThreads + threadIdx.x) * kDecItems;
+  if (threadIdx.x == 0) l2_ahead(T.src, base, (uint64_t)kDecAhead * kDecTile, kDecTile, n);
   if (base >= n) return;
   const bool full = base + kDecItems <= n;
   unsigned long long e[kDecItems];
@@ -2936,19 +2936,19 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
 
   /* queue boundaries, and for the planner's own rule the window tables and output offsets; id_bits > 8:
    * the boundaries are searched, never read off the digit counts */
-  auto launch_windows = [&](bool tables, uint32_t local_candidate, uint32_t id_bits = 64u) {
+  auto launch_windows = [&](bool tables, uint32_t local_candidate, uint32_t id_bits = 64u, bool direct = false) {
     if (many_short_queues(n, L.n_seg))
       launch_pdl(k_windows_many, L.n_seg / (kWinThreads - 1u) + 1, kWinThreads, 0, stream, hdr, (const unsigned long long*)buf_a,
                  (const unsigned long long*)buf_b, n32, ibits, L.n_seg, (const PardSegConst*)ktab, seg_off, out->d_seg_offsets,
                  win_off, win_cnt, wtab, L.win_capacity, (mode & PARD_MODE_SCAN) ? 1u : 0u, tables ? 1u : 0u,
                  (mode & PARD_MODE_RAW) ? 1u : 0u, seg_kept, kept_base, chunk_base, out->d_seg_kept,
-                 (unsigned long long*)out->d_n_kept);
+                 (unsigned long long*)out->d_n_kept, direct ? 1u : 0u);
     else
       launch_pdl(k_windows, L.n_seg / kWinQueues + 1, kWinThreads, 0, stream, hdr, (const unsigned long long*)buf_a,
                (const unsigned long long*)buf_b, n32, ibits, L.n_seg, (const PardSegConst*)ktab, seg_off, out->d_seg_offsets, win_off,
                win_cnt, wtab, L.win_capacity, (mode & PARD_MODE_SCAN) ? 1u : 0u, (const uint32_t*)hist, id_bits, local_candidate,
                tables ? 1u : 0u, (mode & PARD_MODE_RAW) ? 1u : 0u, seg_kept, kept_base, chunk_base, out->d_seg_kept,
-               (unsigned long long*)out->d_n_kept);
+               (unsigned long long*)out->d_n_kept, direct ? 1u : 0u);
   };
 
   auto const_args = [&]() {
@@ -2973,7 +2973,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                  stream, (uint4*)(ws + L.hdr), n16);
     }
     ConstArgs ca = const_args();
-    launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, 0u, false, ca, sms, stream);
+    launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, 0u, ca, sms, stream);
     launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
     launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, 0u, sbits, 1u);
     launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
@@ -3041,12 +3041,18 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     return rc == PARD_ERANGE ? plan_wide() : rc;
   }
 
-  /* ---- requests grouped by ctx (the caller's word, contexts of more than a tile on average) may stand in order
-   * already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
+  /* Requests grouped by ctx (the caller's word) with contexts of more than a tile on average: the
+   * radix passes stay inside every ctx's range -- tiles cut at ctx boundaries, digit counts per
+   * ctx, look-back up to the ctx's first tile -- and sort the stage and deadline bits only; the
+   * ctx bits of the key need no pass (C5: four passes instead of five).  Needs the stage in the low
+   * bits of the queue id: stage_stride a power of two. */
+  const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
+
+  /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
    * 288 k of 24 contexts 71 -> 51; out of order they pay for the try, 567 -> 575 and 117 -> 118.  Without the caller's
    * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
   DirectArgs da = {};
-  const bool direct = (mode & PARD_MODE_GROUPED) && L.ctx_passes && !rule_walk && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN | PARD_MODE_TEST_STALL)) &&
+  const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN | PARD_MODE_TEST_STALL)) &&
                       !state->d_priority && dir_layout(n, n_ctx, S, (char*)buf_b, &da);
   da.req = req4; da.n = n32; da.n_ctx = n_ctx; da.S = S; da.sbits = sbits; da.ibits = ibits;
   da.ktab = ktab; da.ctx_start = ctx_start; da.const_bad = kept_tmp;
@@ -3058,12 +3064,6 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                stream, (uint4*)(ws + L.hdr), n16);
   }
 
-  /* Requests grouped by ctx (the caller's word) with contexts of more than a tile on average: the
-   * radix passes stay inside every ctx's range -- tiles cut at ctx boundaries, digit counts per
-   * ctx, look-back up to the ctx's first tile -- and sort the stage and deadline bits only; the
-   * ctx bits of the key need no pass (C5: four passes instead of five).  Needs the stage in the low
-   * bits of the queue id: stage_stride a power of two. */
-  const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
   const uint32_t key_sbits = ctx_sort ? ceil_log2(S) : sbits;
   const CtxTiles ctx_tiles = {ctx_start, (const uint32_t*)(ws + L.tile_first), (const uint32_t*)(ws + L.hist_ctx), n_ctx};
   /* few queues, decided by the planner's own rule in budget order from the start of every queue:
@@ -3084,12 +3084,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                stream, da, ca, (uint4*)(ws + L.hdr), n16, range_blocks);
   }
   mark();
-  /* on the caller's word that the requests come grouped k_dir_count finds what the prepass would */
-  const bool direct_ranges = direct && ctx_sort;
   if (direct)
-    launch_pdl(S > 8 ? k_dir_count<4> : k_dir_count<3>, da.n_pieces, kDirThreads, 0, stream, da, ca, hdr, ctx_dmin, ctx_dmax,
-               direct_ranges ? 1u : 0u);
-  if (n > 0 && !direct_ranges) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_fold && !direct ? n_ctx : 0u, const_fold, ca, sms, stream);
+    launch_pdl(S > 8 ? k_dir_count<4> : k_dir_count<3>, da.n_pieces, kDirThreads, 0, stream, da, ca, hdr, ctx_dmin, ctx_dmax);
+  if (n > 0 && !direct) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_fold ? n_ctx : 0u, ca, sms, stream);
   mark();
   if (!ca.with_key_width) {
     if (n > 0) launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
@@ -3158,7 +3155,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   if (win_hist) {
     /* boundaries and tables are there already */
   } else {
-    launch_windows(!rule_walk, local_cand, ctx_sort ? 64u : sbits);
+    launch_windows(!rule_walk, local_cand, ctx_sort ? 64u : sbits, direct);
   }
   if (n > 0 && rule_walk) {
     /* a rule without rising thresholds: every queue is walked in order (pard_policy.cu) */

@@ -172,6 +172,7 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
   const SortedView v = sorted_view(a);
   const bool lookup = a.hdr->lookup != 0;
   const uint64_t tile0 = (uint64_t)blockIdx.x * kPolTile;
+  if (threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);
   if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
   constexpr int kUn = 4;                           /* elements, then their records, requested together */
   uint32_t cur = 0xffffffffu;
@@ -591,6 +592,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile0 = blockIdx.x * kPolTile;
   const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
+  if (threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);
   if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
   unsigned long long e[kPolItems];
   uint32_t t[kPolItems], round[kPolItems], flags[kPolItems];
