@@ -427,24 +427,8 @@ struct EmitSmem {
 
 static_assert(sizeof(EmitSmem) <= 48 * 1024, "four blocks per multiprocessor, no opt-in");
 
-/* a tile's requests into shared memory, by one thread; the copy reports to `bar` */
-__device__ __forceinline__ void emit_fetch(EmitSmem& Sm, const uint4* src, uint32_t count) {
-  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&Sm.full), dst = (uint32_t)__cvta_generic_to_shared(Sm.raw), bytes = count * 16;
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               :: "r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-/* false: the copy has not arrived within about a second */
-__device__ __forceinline__ bool emit_arrived(EmitSmem& Sm, uint32_t parity) {
-  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&Sm.full);
-  for (uint32_t spins = 0; spins < 1u << 20; ++spins) {
-    uint32_t done;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (done) return true;
-  }
-  return false;
-}
+/* a tile's requests into shared memory, by one thread */
+__device__ __forceinline__ void emit_fetch(EmitSmem& Sm, const uint4* src, uint32_t count) { bulk_fetch(&Sm.full, Sm.raw, src, count * 16); }
 
 template <int BITS>
 __global__ void __launch_bounds__(kDirThreads, 4)
@@ -459,8 +443,7 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
   const bool est32 = ((uintptr_t)out_est & 31) == 0;
   uint32_t phase = 0;
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"((uint32_t)__cvta_generic_to_shared(&Sm.full)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    bulk_init(&Sm.full);
     uint32_t p = atomicAdd(&hdr->direct_ticket, 1u);
     uint4 info = make_uint4(0u, 0u, 0u, 0u);
     while (p < a.n_pieces) {                      /* (a piece may be empty) */
@@ -502,7 +485,7 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
       const uint32_t cnt = min(kDirTile, info.z - base);
       const bool final = base + kDirTile >= info.z;
       /* 1. the tile's requests, row by row; their ranks within the warp's share */
-      bool late = !emit_arrived(Sm, phase);
+      bool late = !bulk_arrived(&Sm.full, phase);
       phase ^= 1;
       uint32_t x[kDirRows], meta[kDirRows], run = 0;     /* run: lane j: the warp's requests of stage j so far */
       const uint32_t wfirst = warp * (kDirRows * 32);
@@ -519,7 +502,7 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
       }
       if (lane < kDirStages) Sm.cnt[warp][lane] = run;
       if (__syncthreads_or(late)) {
-        emit_arrived(Sm, phase ^ 1);              /* no copy is under way when the block ends */
+        bulk_arrived(&Sm.full, phase ^ 1);              /* no copy is under way when the block ends */
         if (tid == 0) set_aborted(hdr);
         return;
       }

@@ -120,14 +120,6 @@ Layout make_layout(uint64_t n, uint32_t n_ctx, int32_t stage_stride) {
   return L;
 }
 
-/* A bounded wait ran out: the elements are only partly sorted from here on, so nothing after
- * this may use them as indices. */
-__device__ __forceinline__ void set_aborted(PlanHeader* hdr) {
-  hdr->aborted = 1;
-  __threadfence();
-  atomicExch(&hdr->status, (uint32_t)(-PARD_ETIMEOUT));
-}
-
 /* See k_sort_local: the call's requests come grouped by ctx and no ctx exceeds a tile. */
 __device__ __forceinline__ bool sort_is_local(const PlanHeader* hdr, uint32_t candidate) {
   return candidate && !hdr->unsorted && !hdr->ctx_too_big && !hdr->wide;
@@ -2781,7 +2773,8 @@ int allow_sort_smem(int dev) {
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(SortSmem)));
-    const int rc = allow_local_smem();
+    int rc = allow_local_smem();
+    if (rc == PARD_OK) rc = allow_walk_smem();
     if (rc != PARD_OK) return rc;
     done[dev].store(true, std::memory_order_release);
   }

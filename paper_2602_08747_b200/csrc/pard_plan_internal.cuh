@@ -70,13 +70,22 @@ struct PlanHeader {
   uint32_t direct_off;        /* 1: they did not, or something else that path does not take */
   uint32_t direct_done;       /* blocks of k_dir_count that have finished */
   uint32_t direct_ticket;     /* pieces taken by k_dir_emit */
-  uint32_t pad[64 - 30 - kMaxPasses - (kMaxPasses + 1)];
+  uint32_t walk_late;         /* 1: a wait of the rules' walk ran out: `aborted` for the kernels behind it (its own blocks go on together) */
+  uint32_t pad[64 - 31 - kMaxPasses - (kMaxPasses + 1)];
 };
 static_assert(sizeof(PlanHeader) == 256, "header is 256 bytes");
 
 __device__ __forceinline__ void set_status(PlanHeader* hdr, int status) {
   if (status == PARD_EDATA) hdr->bad_input = 1;
   atomicCAS(&hdr->status, 0u, (uint32_t)(-status));
+}
+
+/* A bounded wait ran out: the elements are only partly sorted from here on, so nothing after
+ * this may use them as indices. */
+__device__ __forceinline__ void set_aborted(PlanHeader* hdr) {
+  hdr->aborted = 1;
+  __threadfence();
+  atomicExch(&hdr->status, (uint32_t)(-PARD_ETIMEOUT));
 }
 
 /* The device tables of the call's pipelines: handed over inside the kernel arguments when there are few
@@ -314,6 +323,30 @@ __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" :: "l"(p), "r"(v) : "memory");
 }
 
+/* Copies into shared memory that report to an mbarrier (one arrival per phase).  All 16-byte aligned, the size a
+ * multiple of 16. */
+__device__ __forceinline__ void bulk_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"((uint32_t)__cvta_generic_to_shared(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_fetch(unsigned long long* bar, void* dst, const void* src, uint32_t bytes) {
+  const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar), d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(b), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               :: "r"(d), "l"(src), "r"(bytes), "r"(b) : "memory");
+}
+/* false: the copy has not arrived within about a second */
+__device__ __forceinline__ bool bulk_arrived(unsigned long long* bar, uint32_t parity) {
+  const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
+  for (uint32_t spins = 0; spins < 1u << 20; ++spins) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(b), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
 struct SegVal {            /* value of a segmented running reduction */
   int32_t m;               /* admitted mode: minimum of u_t - t; raw mode: number of kept requests;
                               over the elements since the last queue head (or since the span's start) */
@@ -440,6 +473,7 @@ struct PolicyArgs {
   const uint32_t* kept_base;      /* [n_seg] output offset of every queue's survivors, known after the walk */
   uint32_t* seg_kept;
 };
+int allow_walk_smem();             /* once per device, by the planner's set-up */
 /* thresholds and walk: every queue's rounds and kept count (seg_kept) */
 int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream);
 /* estimates, flags, order and survivors, once the output offsets are known */

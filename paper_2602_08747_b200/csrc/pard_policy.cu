@@ -20,8 +20,11 @@
  *   k_policy_emit    every request on its own again: its round by a search in the ends, estimate,
  *                    decision, survivors straight to their final place
  * T and C live in the sort buffer that does not hold the elements.
- * Nexus on 16 queues of 2^20 requests: the walk takes 0.094 ms where one warp per queue, 32 requests
- * per step, took 23.8 ms. */
+ * Nexus on 16 queues of 2^20 requests: the walk takes 0.053 ms by clusters of eight blocks (0.080 by one block,
+ * 0.093 without copies ahead) where one warp per queue, 32 requests per step, took 23.8 ms; a call of 2^24
+ * requests 453 -> 396 us. */
+#include <type_traits>
+
 #include "pard_plan_internal.cuh"
 
 using namespace pard_plan_detail;
@@ -235,22 +238,59 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
   }
 }
 
-/* What a group of WARPS warps that walks one queue together exchanges: running sums and maxima
- * over its threads, in thread order.  One barrier each; the slots are used in turn. */
-template <int WARPS>
+/* The blocks of a cluster: this one's rank, a word stored in block `to`'s shared memory, all of them brought
+ * together. */
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_store(uint32_t* p, uint32_t to, uint32_t v) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(to));
+  asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(remote), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+/* What a group of WARPS warps in each of CTAS blocks that walks one queue together exchanges: running sums and maxima
+ * over its threads, in thread order.  One barrier each, of the block or of the cluster; the slots are used in turn. */
+template <int WARPS, int CTAS>
 struct WalkGroup {
+  static constexpr int kAll = WARPS * CTAS, kPer = kAll > 32 ? kAll / 32 : 1;   /* warps of the group; figures that a lane adds up */
   struct Shared {
-    uint32_t sum[2][WARPS];
-    int32_t top[2][WARPS];
-    uint32_t first[2][WARPS];
+    __align__(16) uint32_t of_warp[2][2][kAll];    /* every block has all of them */
     uint32_t pos;
   };
   Shared& sh;
-  uint32_t lane, warp;
+  uint32_t lane, warp, rank;
   uint32_t turn;
+  __device__ uint32_t thread() const { return (rank * WARPS + warp) * 32 + lane; }
   __device__ void sync() const {
-    if (WARPS > 1) __syncthreads();
+    if (CTAS > 1) cluster_sync();
+    else if (WARPS > 1) __syncthreads();
     else __syncwarp();
+  }
+  /* the warps' figures x (and y), the same in all lanes of a warp, to everybody: op(index, x, y) for this lane's share of them */
+  template <bool TWO, typename Op>
+  __device__ void exchange(uint32_t x, uint32_t y, Op op) {
+    const uint32_t me = rank * WARPS + warp;
+    turn ^= 1;
+    if (CTAS > 1) {
+      if (lane < CTAS) {
+        cluster_store(&sh.of_warp[turn][0][me], lane, x);
+        if (TWO) cluster_store(&sh.of_warp[turn][1][me], lane, y);
+      }
+    } else if (lane == 0) {
+      sh.of_warp[turn][0][me] = x;
+      if (TWO) sh.of_warp[turn][1][me] = y;
+    }
+    sync();
+    if (lane * kPer < kAll)
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) op(lane * kPer + k, sh.of_warp[turn][0][lane * kPer + k], TWO ? sh.of_warp[turn][1][lane * kPer + k] : 0u);
   }
   /* sum over the earlier threads; *total: over all */
   __device__ uint32_t sum_before(uint32_t x, uint32_t* total) {
@@ -260,16 +300,15 @@ struct WalkGroup {
       const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= (uint32_t)o) incl += y;
     }
-    if (WARPS == 1) {
-      *total = __shfl_sync(0xffffffffu, incl, 31);
+    const uint32_t mine = __shfl_sync(0xffffffffu, incl, 31), me = rank * WARPS + warp;
+    if (kAll == 1) {
+      *total = mine;
       return incl - x;
     }
-    turn ^= 1;
-    if (lane == 31) sh.sum[turn][warp] = incl;
-    sync();
-    const uint32_t w = lane < (uint32_t)WARPS ? sh.sum[turn][lane] : 0u;
-    *total = __reduce_add_sync(0xffffffffu, w);
-    return incl - x + __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u);
+    uint32_t all = 0, before = 0;
+    exchange<false>(mine, 0u, [&](uint32_t k, uint32_t v, uint32_t) { all += v; before += k < me ? v : 0u; });
+    *total = __reduce_add_sync(0xffffffffu, all);
+    return incl - x + __reduce_add_sync(0xffffffffu, before);
   }
   /* maximum over the earlier threads (at least `floor`); *total: over all */
   __device__ int32_t max_before(int32_t x, int32_t floor, int32_t* total) {
@@ -281,36 +320,47 @@ struct WalkGroup {
     }
     int32_t before = __shfl_up_sync(0xffffffffu, incl, 1);
     if (lane == 0) before = floor;
-    if (WARPS == 1) {
-      *total = max(floor, __shfl_sync(0xffffffffu, incl, 31));
+    const int32_t mine = __shfl_sync(0xffffffffu, incl, 31);
+    if (kAll == 1) {
+      *total = max(floor, mine);
       return max(floor, before);
     }
-    turn ^= 1;
-    if (lane == 31) sh.top[turn][warp] = incl;
-    sync();
-    const int32_t w = lane < (uint32_t)WARPS ? sh.top[turn][lane] : floor;
-    *total = max(floor, __reduce_max_sync(0xffffffffu, w));
-    return max(max(floor, before), __reduce_max_sync(0xffffffffu, lane < warp ? w : floor));
+    const uint32_t me = rank * WARPS + warp;
+    int32_t all = floor, ahead = floor;
+    exchange<false>((uint32_t)mine, 0u, [&](uint32_t k, uint32_t v, uint32_t) { all = max(all, (int32_t)v); ahead = k < me ? max(ahead, (int32_t)v) : ahead; });
+    *total = __reduce_max_sync(0xffffffffu, all);
+    return max(max(floor, before), __reduce_max_sync(0xffffffffu, ahead));
   }
-  /* smallest and largest x of the group, one barrier */
+  /* smallest and largest x of the group */
   __device__ void range_all(uint32_t lo, int32_t hi, uint32_t* least, int32_t* most) {
-    const uint32_t m = __reduce_min_sync(0xffffffffu, lo);
-    const int32_t t = __reduce_max_sync(0xffffffffu, hi);
-    if (WARPS == 1) { *least = m; *most = t; return; }
-    turn ^= 1;
-    if (lane == 0) { sh.first[turn][warp] = m; sh.top[turn][warp] = t; }
-    sync();
-    *least = __reduce_min_sync(0xffffffffu, lane < (uint32_t)WARPS ? sh.first[turn][lane] : 0xffffffffu);
-    *most = __reduce_max_sync(0xffffffffu, lane < (uint32_t)WARPS ? sh.top[turn][lane] : -1);
+    uint32_t m = __reduce_min_sync(0xffffffffu, lo);
+    int32_t t = __reduce_max_sync(0xffffffffu, hi);
+    if (kAll > 1) {
+      uint32_t ms = 0xffffffffu;
+      int32_t ts = -1;
+      exchange<true>(m, (uint32_t)t, [&](uint32_t, uint32_t x, uint32_t y) { ms = min(ms, x); ts = max(ts, (int32_t)y); });
+      m = __reduce_min_sync(0xffffffffu, ms);
+      t = __reduce_max_sync(0xffffffffu, ts);
+    }
+    *least = m;
+    *most = t;
   }
   /* smallest x of the group */
   __device__ uint32_t min_all(uint32_t x) {
-    const uint32_t m = __reduce_min_sync(0xffffffffu, x);
-    if (WARPS == 1) return m;
-    turn ^= 1;
-    if (lane == 0) sh.first[turn][warp] = m;
-    sync();
-    return __reduce_min_sync(0xffffffffu, lane < (uint32_t)WARPS ? sh.first[turn][lane] : 0xffffffffu);
+    uint32_t m = __reduce_min_sync(0xffffffffu, x);
+    if (kAll > 1) {
+      uint32_t ms = 0xffffffffu;
+      exchange<false>(m, 0u, [&](uint32_t, uint32_t v, uint32_t) { ms = min(ms, v); });
+      m = __reduce_min_sync(0xffffffffu, ms);
+    }
+    return m;
+  }
+  /* by one thread: a position for all, who see it behind the next sync() */
+  __device__ void tell(uint32_t pos) {
+    if (CTAS > 1)
+      for (int k = 0; k < CTAS; ++k) cluster_store(&sh.pos, (uint32_t)k, pos);
+    else
+      sh.pos = pos;
   }
 };
 
@@ -318,24 +368,126 @@ constexpr int kWalkItems = 16;                     /* consecutive requests per t
 constexpr uint32_t kWalkWarps = 32;                /* warps of a group that walks a long queue (16: 123 us instead of 94 at 16 x 2^20) */
 constexpr uint32_t kWalkLong = 2048;               /* requests per queue on average from which a block, not a warp, walks one:
                                                       an eighth of the 16,384 requests a block takes in one step */
+constexpr int kWalkCtas = 8;                       /* blocks of a cluster that walks a queue */
+constexpr uint32_t kWalkShare = kWalkWarps * 32 * kWalkItems;           /* requests a block takes in one step */
+constexpr uint32_t kWalkClusterLong = 4 * kWalkCtas * kWalkShare;       /* shorter queues, and ... */
+constexpr uint32_t kWalkClusterCap = 4 * kWalkShare;                    /* ... queues of smaller rounds are walked by one block: a round costs */
+constexpr uint32_t kWalkClusterWindow = kWalkShare;                     /* two of the cluster's barriers; windows of Nexus seldom fill */
+constexpr uint32_t kWalkClusterQueues = 37;        /* most queues: as many clusters as two rounds of the device's blocks */
 constexpr uint32_t kWalkSmallRound = 64;           /* rounds below this size are walked by one warp, 32 requests per step: a step
                                                       closes several of them, where a group needs a barrier for each */
 
-/* this thread's 16 thresholds; the array may be read up to the next multiple of 16 (workspace) */
-__device__ __forceinline__ void walk_load(const uint32_t* __restrict__ T, uint32_t at, uint32_t hi, uint32_t (&v)[kWalkItems]) {
+/* The thresholds of step after step, 16 consecutive ones per thread; the array may be read up to the next multiple
+ * of 16 (workspace).
+ * A block (WARPS > 1) has them copied into shared memory, kFeedDepth steps ahead, and reads them there four at a
+ * time, the four vectors of a thread in an order that starts a place further with every second thread: as loads of
+ * 64 bytes per lane from global memory they took 16 wavefronts an instruction, and a step 1.45 us of which the rest
+ * of the work needs 0.5 (16 queues of 2^20, Nexus: the walk 93 us). */
+constexpr int kFeedDepth = 3;
+template <int WARPS, int CTAS>
+struct WalkFeed {
+  static constexpr uint32_t kStep = WARPS * 32 * kWalkItems;
+  const uint32_t* T;
+  uint32_t at, hi, next[kWalkItems];
+  static constexpr uint32_t rot = 0;
+  __device__ void load() {
 #pragma unroll
-  for (int q = 0; q < kWalkItems / 4; ++q) {
-    uint4 x = make_uint4(0u, 0u, 0u, 0u);
-    if (at + 4 * q < hi) x = *reinterpret_cast<const uint4*>(T + at + 4 * q);
-    v[4 * q] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+    for (int q = 0; q < kWalkItems / 4; ++q) {
+      uint4 x = make_uint4(0u, 0u, 0u, 0u);
+      if (at + 4 * q < hi) x = *reinterpret_cast<const uint4*>(T + at + 4 * q);
+      next[4 * q] = x.x; next[4 * q + 1] = x.y; next[4 * q + 2] = x.z; next[4 * q + 3] = x.w;
+    }
+    at += kStep;
   }
+  __device__ WalkFeed(const PolicyArgs&, const uint32_t* T_, uint32_t first, uint32_t hi_, uint32_t t, uint32_t) : T(T_), at(first + t * kWalkItems), hi(hi_) { load(); }
+  /* this step's, and the next one's on their way */
+  __device__ void step(uint32_t (&u)[kWalkItems]) {
+#pragma unroll
+    for (int i = 0; i < kWalkItems; ++i) u[i] = next[i];
+    load();
+  }
+  __device__ uint32_t in_order(uint32_t bits) const { return bits; }
+};
+struct FeedSmem {
+  uint32_t ring[kFeedDepth][kWalkWarps * 32 * kWalkItems];
+  unsigned long long full[kFeedDepth];             /* mbarriers */
+};
+__device__ __forceinline__ FeedSmem* feed_smem() {
+  extern __shared__ __align__(16) unsigned char walk_raw[];
+  return reinterpret_cast<FeedSmem*>(walk_raw);
 }
-
-/* bits of this thread's requests that fit round b */
+template <int CTAS>
+struct WalkFeed<(int)kWalkWarps, CTAS> {
+  static constexpr uint32_t kShare = kWalkWarps * 32 * kWalkItems;      /* of a block; the step's are the blocks' shares in order of rank */
+  FeedSmem& Sm;
+  const PolicyArgs& a;
+  const uint32_t* T;
+  uint32_t from, hi, t, slot, parity, rot;         /* from: first of the next share to fetch; rot: the vector a thread begins with */
+  uint32_t left;                                   /* steps for which this block has a share */
+  uint32_t begin;
+  bool alone;                                      /* one step in all: read as it stands (with copies 160 queues of 3,125 took 2 us more) */
+  __device__ void fetch(uint32_t to) {             /* by thread 0 */
+    if (from >= hi) return;
+    bulk_fetch(&Sm.full[to], Sm.ring[to], T + from, ((min(hi - from, kShare) + 3) & ~3u) * 4);
+    from += CTAS * kShare;
+  }
+  __device__ WalkFeed(const PolicyArgs& a_, const uint32_t* T_, uint32_t first, uint32_t hi_, uint32_t t_, uint32_t rank)
+      : Sm(*feed_smem()), a(a_), T(T_), from(first + rank * kShare), hi(hi_), t(t_), slot(0), parity(0), rot((t_ >> 1) & 3u),
+        left(from < hi_ ? (hi_ - from + CTAS * kShare - 1) / (CTAS * kShare) : 0u), begin(first), alone(CTAS == 1 && hi_ - first <= kShare) {
+    if (alone) {
+      rot = 0;
+      return;
+    }
+    if (t == 0) {
+      for (int k = 0; k < kFeedDepth; ++k) bulk_init(&Sm.full[k]);
+      for (int k = 0; k < kFeedDepth; ++k) fetch(k);
+    }
+    __syncthreads();
+  }
+  /* A wait that runs out does not end the walk here: blocks of a cluster store into each other's shared memory, so
+   * they go on together, this one without requests that fit. */
+  __device__ void step(uint32_t (&u)[kWalkItems]) {
+#pragma unroll
+    for (int i = 0; i < kWalkItems; ++i) u[i] = 0;
+    if (!left) return;
+    --left;
+    if (alone) {
+      const uint4* mine = reinterpret_cast<const uint4*>(T + begin) + t * (kWalkItems / 4);
+#pragma unroll
+      for (uint32_t q = 0; q < kWalkItems / 4; ++q)
+        if (begin + t * kWalkItems + 4 * q < hi) {
+          const uint4 x = mine[q];
+          u[4 * q] = x.x; u[4 * q + 1] = x.y; u[4 * q + 2] = x.z; u[4 * q + 3] = x.w;
+        }
+      return;
+    }
+    const bool late = !bulk_arrived(&Sm.full[slot], parity);
+    const uint4* mine = reinterpret_cast<const uint4*>(Sm.ring[slot]) + t * (kWalkItems / 4);
+#pragma unroll
+    for (uint32_t q = 0; q < kWalkItems / 4; ++q) {
+      const uint4 x = mine[(q + rot) & 3u];
+      u[4 * q] = x.x; u[4 * q + 1] = x.y; u[4 * q + 2] = x.z; u[4 * q + 3] = x.w;
+    }
+    if (__syncthreads_or(late)) {                  /* (also: everybody has read the slot) */
+      left = 0;
+      if (t == 0) {
+        for (int k = 0; k < kFeedDepth; ++k) bulk_arrived(&Sm.full[k], k < (int)slot ? parity ^ 1 : parity);   /* no copy is under way when the block ends */
+        a.hdr->walk_late = 1;
+        set_status(a.hdr, PARD_ETIMEOUT);
+      }
+      return;
+    }
+    if (t == 0) fetch(slot);
+    if (++slot == kFeedDepth) { slot = 0; parity ^= 1; }
+  }
+  /* bit i of `bits`: the i-th value as read; of the result: the i-th in the array */
+  __device__ uint32_t in_order(uint32_t bits) const { return ((bits << (4 * rot)) | (bits >> (16 - 4 * rot))) & 0xffffu; }
+};
+/* bits of this thread's requests that fit round b (in the order of u) */
 __device__ __forceinline__ uint32_t walk_fit(const uint32_t (&v)[kWalkItems], uint32_t b) {
   uint32_t g = 0;
 #pragma unroll
-  for (int i = 0; i < kWalkItems; ++i) g |= (v[i] > b ? 1u : 0u) << i;
+  for (int i = kWalkItems - 1; i >= 0; --i) g = __funnelshift_l(b - v[i], g, 1);      /* both at most 2^30: the sign says it */
   return g;
 }
 
@@ -349,20 +501,17 @@ __device__ __forceinline__ uint32_t walk_range(uint32_t at, uint32_t from, uint3
 
 /* The general rule in rounds of at least kWalkSmallRound.  RAW: every request ahead takes a slot,
  * so a request's round is its position's and no round has to be waited for. */
-template <int WARPS, bool RAW>
-__device__ void walk_admit(WalkGroup<WARPS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
+template <int WARPS, int CTAS, bool RAW>
+__device__ void walk_admit(WalkGroup<WARPS, CTAS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
                            uint32_t hi, const PardSegConst& K) {
-  constexpr uint32_t kStep = WARPS * 32 * kWalkItems;
-  const uint32_t cap = K.cap, t = G.warp * 32 + G.lane;
+  constexpr uint32_t kStep = CTAS * WARPS * 32 * kWalkItems;
+  const uint32_t cap = K.cap, t = G.thread();
   uint32_t x = 0, b = 0, left = cap;
-  uint32_t next[kWalkItems];
   uint32_t at = (lo & ~(uint32_t)(kWalkItems - 1)) + t * kWalkItems;
-  walk_load(v.T, at, hi, next);
+  WalkFeed<WARPS, CTAS> feed(a, v.T, lo & ~(uint32_t)(kWalkItems - 1), hi, G.warp * 32 + G.lane, G.rank);
   for (uint32_t step = lo & ~(uint32_t)(kWalkItems - 1); step < hi; step += kStep, at += kStep) {
     uint32_t u[kWalkItems];
-#pragma unroll
-    for (int i = 0; i < kWalkItems; ++i) u[i] = next[i];
-    walk_load(v.T, at + kStep, hi, next);          /* the next step's, while this one is decided */
+    feed.step(u);
     uint32_t open = walk_range(at, lo, hi), kept = 0, before = 0, total = 0;
     const uint32_t x0 = x;
     bool several = false;
@@ -371,13 +520,13 @@ __device__ void walk_admit(WalkGroup<WARPS>& G, const PolicyArgs& a, const Sorte
       if (RAW) {
 #pragma unroll
         for (int i = 0; i < kWalkItems; ++i) {
-          const uint32_t r = at + i - lo, round = K.cap_magic ? div_magic32(r, K.cap_magic) : r;
+          const uint32_t r = at + ((i + 4 * feed.rot) & (kWalkItems - 1)) - lo, round = K.cap_magic ? div_magic32(r, K.cap_magic) : r;
           fit |= (u[i] > round ? 1u : 0u) << i;
         }
       } else {
         fit = walk_fit(u, b);
       }
-      fit &= open;
+      fit = feed.in_order(fit) & open;
       const uint32_t mine = __popc(fit);
       before = G.sum_before(mine, &total);
       if (RAW || total < left) {                   /* the round does not close in this step */
@@ -393,7 +542,7 @@ __device__ void walk_admit(WalkGroup<WARPS>& G, const PolicyArgs& a, const Sorte
         const uint32_t end = at + __ffs(m);        /* position behind it */
         kept |= fit & (0xffffu >> (at + 16 - end));
         v.C[lo + b] = end;
-        G.sh.pos = end;
+        G.tell(end);
       } else if (before + mine < left) {
         kept |= fit;
       }
@@ -444,26 +593,23 @@ __device__ void walk_admit_small(const PolicyArgs& a, const SortedView& v, uint3
  * (b < v_r), everything before it is dropped, b advances, the scan goes on behind it.  With `bad`
  * the last position that does not fit (or that ends the window before), a window closes at
  * bad + W, the first time that lies before the next misfit. */
-template <int WARPS>
-__device__ void walk_nexus(WalkGroup<WARPS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
+template <int WARPS, int CTAS>
+__device__ void walk_nexus(WalkGroup<WARPS, CTAS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
                            uint32_t hi, uint32_t W) {
-  constexpr uint32_t kStep = WARPS * 32 * kWalkItems;
+  constexpr uint32_t kStep = CTAS * WARPS * 32 * kWalkItems;
   constexpr uint32_t kNone = 0xffffffffu;
-  const uint32_t t = G.warp * 32 + G.lane;
+  const uint32_t t = G.thread();
   uint32_t b = 0;
   int32_t bad = (int32_t)lo - 1;
-  uint32_t next[kWalkItems];
   uint32_t at = (lo & ~(uint32_t)(kWalkItems - 1)) + t * kWalkItems;
-  walk_load(v.T, at, hi, next);
+  WalkFeed<WARPS, CTAS> feed(a, v.T, lo & ~(uint32_t)(kWalkItems - 1), hi, G.warp * 32 + G.lane, G.rank);
   for (uint32_t step = lo & ~(uint32_t)(kWalkItems - 1); step < hi; step += kStep, at += kStep) {
     uint32_t u[kWalkItems];
-#pragma unroll
-    for (int i = 0; i < kWalkItems; ++i) u[i] = next[i];
-    walk_load(v.T, at + kStep, hi, next);
+    feed.step(u);
     uint32_t from = lo;
     for (;;) {
       const uint32_t open = walk_range(at, from, hi);
-      const uint32_t miss = ~walk_fit(u, b) & open;
+      const uint32_t miss = ~feed.in_order(walk_fit(u, b)) & open;
       if (W >= kStep) {                            /* a window cannot begin and end in one step: only the running one can close */
         uint32_t least;
         int32_t most;
@@ -481,15 +627,12 @@ __device__ void walk_nexus(WalkGroup<WARPS>& G, const PolicyArgs& a, const Sorte
         break;
       }
       int32_t top;
-      int32_t last = G.max_before(miss ? (int32_t)at + 31 - __clz(miss) : -1, bad, &top);
+      const int32_t last = G.max_before(miss ? (int32_t)at + 31 - __clz(miss) : -1, bad, &top);
       uint32_t found = kNone;
-      for (uint32_t m = miss; open;) {             /* stretches of fitting requests between this thread's misfits */
-        const uint32_t end = m ? at + __ffs(m) - 1 : min(at + 16, hi);     /* where the stretch ends */
+      if (open) {                                  /* a window can only close ahead of the thread's first misfit: it is longer than a thread's share */
+        const uint32_t end = miss ? at + __ffs(miss) - 1 : min(at + 16, hi);
         const unsigned long long full = (unsigned long long)((long long)last + W);   /* where a window would close */
-        if (full < end && full >= max(at, from)) { found = (uint32_t)full; break; }
-        if (!m) break;
-        last = (int32_t)end;
-        m &= m - 1;
+        if (full < end && full >= max(at, from)) found = (uint32_t)full;
       }
       found = G.min_all(found);
       if (found == kNone) { bad = top; break; }
@@ -541,34 +684,46 @@ __device__ void walk_nexus_small(const PolicyArgs& a, const SortedView& v, uint3
   if (lane == 0) { a.rounds[s] = b; a.tail[s] = run; a.seg_kept[s] = b * W + run; }
 }
 
-template <int WARPS>
+/* CTAS > 1: a cluster per queue, for the queues where its barriers are worth it: many steps, few rounds.  The first
+ * block of the cluster walks the others by itself.  (A step of one block 1.2 us, of a cluster some 1.5 for eight times
+ * the requests, a round 0.6 and 1.5; 2^23 requests with known paths in 32 queues of 2^18: 612 by blocks, 621 by clusters.) */
+template <int WARPS, int CTAS>
 __global__ void __launch_bounds__(WARPS == 1 ? kPolThreads : WARPS * 32)
 k_policy_walk(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
   constexpr int kGroups = WARPS == 1 ? kPolThreads / 32 : 1;
-  __shared__ typename WalkGroup<WARPS>::Shared sh[kGroups];
-  if (a.hdr->wide || a.hdr->aborted) return;
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t s = WARPS == 1 ? blockIdx.x * kGroups + warp : blockIdx.x;
+  __shared__ typename WalkGroup<WARPS, CTAS>::Shared sh[kGroups];
+  if (a.hdr->wide || a.hdr->aborted) return;       /* (nothing sets them while this kernel runs) */
+  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rank = CTAS > 1 ? cluster_rank() : 0u;
+  const uint32_t s = WARPS == 1 ? blockIdx.x * kGroups + warp : blockIdx.x / CTAS;
   if (s >= a.n_seg) return;                        /* whole groups leave together */
   const SortedView v = sorted_view(a);
   const uint32_t lo = a.seg_off[s], hi = a.seg_off[s + 1];
   if (hi <= lo) {
-    if (lane == 0 && (WARPS == 1 || warp == 0)) { a.rounds[s] = 0; a.tail[s] = 0; a.seg_kept[s] = 0; }
+    if (rank == 0 && lane == 0 && (WARPS == 1 || warp == 0)) { a.rounds[s] = 0; a.tail[s] = 0; a.seg_kept[s] = 0; }
     return;
   }
   const PardSegConst K = a.ktab[s];
   const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
   if (K.cap < kWalkSmallRound && !raw) {
-    if (WARPS > 1 && warp != 0) return;
+    if (rank || (WARPS > 1 && warp != 0)) return;
     if (nexus) walk_nexus_small(a, v, s, lo, hi, K.cap, lane);
     else walk_admit_small(a, v, s, lo, hi, K, lane);
     return;
   }
-  WalkGroup<WARPS> G{sh[WARPS == 1 ? warp : 0], lane, WARPS == 1 ? 0u : warp, 0u};
-  if (nexus) walk_nexus<WARPS>(G, a, v, s, lo, hi, K.cap);
-  else if (raw) walk_admit<WARPS, true>(G, a, v, s, lo, hi, K);
-  else walk_admit<WARPS, false>(G, a, v, s, lo, hi, K);
+  auto walk = [&](auto ctas) {
+    constexpr int N = decltype(ctas)::value;
+    WalkGroup<WARPS, N> G{reinterpret_cast<typename WalkGroup<WARPS, N>::Shared&>(sh[WARPS == 1 ? warp : 0]), lane, WARPS == 1 ? 0u : warp, N > 1 ? rank : 0u, 0u};
+    if (nexus) walk_nexus<WARPS, N>(G, a, v, s, lo, hi, K.cap);
+    else if (raw) walk_admit<WARPS, N, true>(G, a, v, s, lo, hi, K);
+    else walk_admit<WARPS, N, false>(G, a, v, s, lo, hi, K);
+  };
+  if (CTAS > 1 && (raw || K.cap < (nexus ? kWalkClusterWindow : kWalkClusterCap) || hi - lo < kWalkClusterLong)) {
+    if (rank == 0) walk(std::integral_constant<int, 1>());
+  } else {
+    if (CTAS > 1) cluster_sync();                  /* every block's shared memory is there before another stores into it */
+    walk(std::integral_constant<int, CTAS>());
+  }
 }
 
 /* Estimates, decisions and survivors.  A request's round is the number of rounds of its queue that
@@ -587,7 +742,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   __shared__ __align__(16) unsigned char sp_raw[MASK == kMaskStaged ? sizeof(StagedPaths) : 16];
   StagedPaths& sp = *reinterpret_cast<StagedPaths*>(sp_raw);
   __shared__ uint32_t s_keep[kRows], s_before[kRows + 1];
-  if (a.hdr->wide || a.hdr->aborted) return;
+  if (a.hdr->wide | a.hdr->aborted | a.hdr->walk_late) return;
   const SortedView v = sorted_view(a);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile0 = blockIdx.x * kPolTile;
@@ -725,15 +880,24 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
 
 namespace pard_plan_detail {
 
+int allow_walk_smem() {
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_policy_walk<kWalkWarps, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FeedSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_policy_walk<kWalkWarps, kWalkCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FeedSmem)));
+  return PARD_OK;
+}
+
 int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
+  static_assert(kWalkItems < (int)kWalkSmallRound, "a window is longer than a thread's share of a step");
   static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
   launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
              tiles, kPolThreads, 0, stream, a);
-  if (a.n / a.n_seg >= kWalkLong)
-    launch_pdl(k_policy_walk<kWalkWarps>, a.n_seg, kWalkWarps * 32, 0, stream, a);
+  if (a.n / a.n_seg >= kWalkClusterLong / 2 && a.n_seg <= kWalkClusterQueues)
+    PARD_CUDA_OK(launch_pdl_cluster(k_policy_walk<kWalkWarps, kWalkCtas>, a.n_seg * kWalkCtas, kWalkWarps * 32, sizeof(FeedSmem), kWalkCtas, stream, a));
+  else if (a.n / a.n_seg >= kWalkLong)
+    launch_pdl(k_policy_walk<kWalkWarps, 1>, a.n_seg, kWalkWarps * 32, sizeof(FeedSmem), stream, a);
   else
-    launch_pdl(k_policy_walk<1>, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
+    launch_pdl(k_policy_walk<1, 1>, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
 }
 

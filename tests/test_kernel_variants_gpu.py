@@ -297,3 +297,20 @@ def test_window_tables_of_very_many_queues(n_ctx, S, n, mode):
     if mode != FCFS:
         wl.state.priority = rng.integers(0, 2, size=(n_ctx, S)).astype(np.uint8)
         check(wl, mode)
+
+
+# ---- long queues walked by a cluster of eight blocks (131,072 requests a step), their rounds and their neighbours ------
+@pytest.mark.parametrize("rule", [FCFS, NEXUS])
+@pytest.mark.parametrize("cap", [16_383, 16_384, 65_535, 65_536, 131_072, 150_001])
+@pytest.mark.parametrize("sizes", [[524_287], [524_288], [524_289, 5], [900_000, 0, 540_000, 560_000], [1_000_003]])
+def test_walk_by_clusters(rule, cap, sizes):
+    rng = np.random.default_rng(cap + len(sizes))
+    p = util.pipeline([], 1, [13], bmax=4096)
+    B = next(b for b in range(4096, 0, -1) if cap % b == 0)
+    for share in (0.0, 0.00001, 0.3):                      # of late requests
+        wl = several_ctx(len(sizes), sizes, S=1, sort=False)
+        wl.pipelines = [p]
+        wl.state = util.state(len(sizes), 1, 0, 0, B, workers=cap // B)
+        late = rng.random(wl.n) < share
+        wl.requests["deadline_us"] = np.where(late, rng.integers(0, 60, size=wl.n), 10**6)
+        check(wl, rule)
