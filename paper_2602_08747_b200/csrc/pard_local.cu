@@ -787,6 +787,9 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
       Sm.ctx = t;
       Sm.first = a.ctx_start[t];
       Sm.cnt = a.ctx_start[t + 1] - Sm.first;
+      /* As many requests behind this ctx on their way into L2 for the block that takes the next one: 4,096 x 8,192
+       * requests 391 -> 361 us (two contexts on 362, eight 398; by each thread's own prefetches 470 -> 506). */
+      l2_ahead(reinterpret_cast<const unsigned long long*>(a.req), 2ull * Sm.first, 2ull * Sm.cnt, 2 * Sm.cnt, 2ull * a.n);
     }
   }
   if (tid == 0) { Sm.flags = a.st.d_priority ? 4u : 0u; Sm.use_scan = 0; Sm.abort = 0; }

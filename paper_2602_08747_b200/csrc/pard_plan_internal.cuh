@@ -308,7 +308,7 @@ __device__ __forceinline__ void store4(void* p, unsigned long long a, unsigned l
  * the meantime.  At 2^24 requests (us per call; before: 528): sort passes 16 tiles ahead (of 296 in flight) 512,
  * 32 ahead 513, 120 ahead 516, 296 ahead 521; the decision 600 tiles ahead another 4 (300 and 2,400: 2). */
 __device__ __forceinline__ void l2_ahead(const unsigned long long* src, uint64_t from, uint64_t ahead, uint32_t count, uint64_t n) {
-  if (from + ahead + count <= n)
+  if (count && from + ahead + count <= n)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(src + from + ahead), "r"(count * 8) : "memory");
 }
 constexpr uint32_t kSortAhead = 16, kDecAhead = 600;    /* tiles of kSortTile and of kDecTile */
