@@ -767,12 +767,14 @@ __device__ __noinline__ void finish_ctx(PlanHeader* __restrict__ hdr, const Loca
     }
 }
 
-template <bool RAW>
+template <bool RAW, bool SINGLE>
 __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t S = (uint32_t)a.st.stage_stride;
-  const bool single = a.ctx_start == nullptr;
-  if (single) {                                          /* the only kernel of the call: the header starts here */
+  /* SINGLE: the call's one ctx; the last warps work out its constants, a chain of dependent loads, while the others read
+   * the requests (3,001 requests of three stages 36.0 -> 33.5 us a call, 8,000 50.5 -> 47.5). */
+  constexpr uint32_t kReaders = SINGLE ? kLocWarps - 4 : kLocWarps;
+  if (SINGLE) {                                          /* the only kernel of the call: the header starts here */
     if (tid < sizeof(PlanHeader) / 4) reinterpret_cast<uint32_t*>(hdr)[tid] = 0;
     if (tid == 0) { Sm.ctx = 0; Sm.first = 0; Sm.cnt = a.n; }
   } else if (tid == 0) {
@@ -807,15 +809,16 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   const bool few = S <= 16 && !a.st.d_priority;          /* (queues served high budget first want descending deadlines) */
   unsigned long long lmin = ~0ull, lmax = 0;
   uint32_t seen = few ? 0u : 4u;                         /* 1: a request of another ctx, 2: out of range, 4: not in order */
-  if (wfirst < cnt) {
+  const uint32_t ritems = SINGLE ? (cnt + 32 * kReaders - 1) / (32 * kReaders) : (uint32_t)items, rfirst = warp * 32 * ritems;   /* rounds per warp in this step */
+  if (rfirst < cnt && warp < kReaders) {
     const uint4* req = a.req + first;
-    const uint4 p = __ldg(&req[wfirst > 0 ? wfirst - 1 : 0]);
+    const uint4 p = __ldg(&req[rfirst > 0 ? rfirst - 1 : 0]);
     const uint32_t high = p.y;
     uint32_t last = p.x;                                 /* low words of the row before this one, first the request before the warp's */
     constexpr int kUn = 4;                               /* requests in flight per thread */
-    const uint32_t wend = min(cnt, wfirst + 32 * (uint32_t)items);
+    const uint32_t wend = min(cnt, rfirst + 32 * ritems);
 #pragma unroll 1
-    for (uint32_t p0 = wfirst + lane; p0 - lane < wend; p0 += 32 * kUn) {
+    for (uint32_t p0 = rfirst + lane; p0 - lane < wend; p0 += 32 * kUn) {
       uint4 r[kUn];
       const bool full = p0 - lane + 32 * kUn <= wend;    /* uniform */
 #pragma unroll
@@ -867,6 +870,10 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
       }
     }
   }
+  if (SINGLE && warp >= kReaders) {
+    __shared__ CtxScratch s_scratch;
+    if (ctx_constants<true, 1>(a.pipes, a.n_pipelines, a.st, c, 0, 0, Sm.K, s_scratch, nullptr, 32 * kReaders)) set_status(hdr, PARD_EDATA);
+  }
   for (int o = 16; o; o >>= 1) {
     const unsigned long long x = __shfl_xor_sync(0xffffffffu, lmin, o), y = __shfl_xor_sync(0xffffffffu, lmax, o);
     lmin = x < lmin ? x : lmin;
@@ -903,19 +910,13 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   const uint32_t sb = 32u - __clz(flagged ? S : S - 1);  /* bit width of the largest value; __clz(0) = 32 */
   if (flagged && tid == 0) set_status(hdr, PARD_EDATA);
 
-  /* 2. constants of the ctx's queues: worked out here when the call is this one block; else taken
+  /* 2. constants of the ctx's queues: worked out beside the first step when the call is this one block; else taken
    * from the table filled for all queues at once (a chain of dependent loads that every block
-   * would otherwise wait for) and completed with what hangs on the ctx's deadline range */
-  if (single) {
-    if (ctx_constants<false>(a.pipes, a.n_pipelines, a.st, c, dmin, dmax, Sm.K, *reinterpret_cast<CtxScratch*>(Sm.keys))) set_status(hdr, PARD_EDATA);
-    for (uint32_t k = tid; k < S; k += kLocThreads)      /* (the thread that wrote it) */
-      if (!(Sm.K[k].narrow & kSegHighFirst)) Sm.K[k].A_rel = booked_within(Sm.K[k].A_rel, span);
-  } else {
-    for (uint32_t k = tid; k < S; k += kLocThreads) {
-      PardSegConst K = a.ktab[(size_t)c * S + k];
-      K.A_rel = (K.narrow & kSegHighFirst) ? (int64_t)dmax - K.A : booked_within(K.A - (int64_t)dmin, span);
-      Sm.K[k] = K;
-    }
+   * would otherwise wait for); completed with what hangs on the ctx's deadline range */
+  for (uint32_t k = tid; k < S; k += kLocThreads) {
+    PardSegConst K = SINGLE ? Sm.K[k] : a.ktab[(size_t)c * S + k];
+    K.A_rel = (K.narrow & kSegHighFirst) ? (int64_t)dmax - K.A : booked_within(K.A - (int64_t)dmin, span);
+    Sm.K[k] = K;
   }
 
   /* 3. elements, sorted */
@@ -1014,12 +1015,12 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   finish_ctx<RAW>(hdr, a, Sm, f, c, first, cnt, items);
 }
 
-template <bool RAW>
-__global__ void __launch_bounds__(kLocThreads, 2)
+template <bool RAW, bool SINGLE>
+__global__ void __launch_bounds__(kLocThreads, SINGLE ? 1 : 2)
 k_plan_local(PlanHeader* __restrict__ hdr, const __grid_constant__ LocalArgs a) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  plan_ctx<RAW>(hdr, a, *reinterpret_cast<LocalSmem*>(smem_raw));
+  plan_ctx<RAW, SINGLE>(hdr, a, *reinterpret_cast<LocalSmem*>(smem_raw));
   if (a.answer.word) {
     __syncthreads();
     if (threadIdx.x == 0) pard_report(&hdr->status, a.answer.word, a.answer.ticket);
@@ -1050,8 +1051,10 @@ k_ctx_prep(const __grid_constant__ LocalArgs a, PardSegConst* __restrict__ ktab,
 namespace pard_plan_detail {
 
 int allow_local_smem() {
-  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
-  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_plan_local<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(LocalSmem)));
   return PARD_OK;
 }
 
@@ -1062,8 +1065,9 @@ int launch_ctx_prep(const LocalArgs& a, PardSegConst* ktab, uint32_t* ctx_start,
 }
 
 int launch_plan_local(const LocalArgs& a, PlanHeader* hdr, bool raw, cudaStream_t stream) {
-  PARD_CUDA_OK(launch_pdl(raw ? k_plan_local<true> : k_plan_local<false>, a.ctx_start ? a.n_ctx : 1u, kLocThreads, sizeof(LocalSmem),
-                          stream, hdr, a));
+  auto kernel = a.ctx_start ? (raw ? k_plan_local<true, false> : k_plan_local<false, false>)
+                            : (raw ? k_plan_local<true, true> : k_plan_local<false, true>);
+  PARD_CUDA_OK(launch_pdl(kernel, a.ctx_start ? a.n_ctx : 1u, kLocThreads, sizeof(LocalSmem), stream, hdr, a));
   return PARD_OK;
 }
 

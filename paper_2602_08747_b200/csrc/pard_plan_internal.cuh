@@ -146,7 +146,7 @@ __device__ __forceinline__ int32_t narrow_A(const PardSegConst& K) {
  * per stage instead of a chain of three.  One warp per queue that walked its paths on its own took
  * 10 us for 16 queues and 37 us for 32,768.  AHEAD: a thread requests what belongs to its own stage and slot at once
  * (9.0 -> 7.0 us for the constants of one ctx; not in k_plan_local, which has no registers left for it: 4,096 epochs
- * 391 -> 395 us).  sums: the ctx's rows of PolicyArgs::path_sums, or null. */
+ * 391 -> 395 us).  BAR: by the threads from first_thread on, with a barrier of their own.  sums: the ctx's rows of PolicyArgs::path_sums, or null. */
 constexpr int kMaskPaths = 16;                     /* bits of pard_request_t.flags: paths of a stage that a request can name */
 constexpr int kConstThreads = 64;                  /* k_seg_const's blocks; any number of threads will do */
 struct CtxScratch {
@@ -155,11 +155,15 @@ struct CtxScratch {
   unsigned long long lsub[PARD_MAX_STAGES];
   int32_t slot_off[PARD_MAX_STAGES + 1];
 };
-template <bool AHEAD>
+template <bool AHEAD, int BAR = 0>
 __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n_pipelines, const pard_queue_state_t& st, uint32_t c,
                                               unsigned long long dmin, unsigned long long dmax, PardSegConst* K_out,
-                                              CtxScratch& sc, long long* sums = nullptr) {
-  const uint32_t S = (uint32_t)st.stage_stride, tid = threadIdx.x, nt = blockDim.x;
+                                              CtxScratch& sc, long long* sums = nullptr, uint32_t first_thread = 0) {
+  const uint32_t S = (uint32_t)st.stage_stride, tid = threadIdx.x - first_thread, nt = blockDim.x - first_thread;
+  auto sync = [&]() {
+    if (BAR) asm volatile("bar.sync %0, %1;" :: "n"(BAR), "r"(nt) : "memory");
+    else __syncthreads();
+  };
   const int32_t pi = st.d_pipeline_of_ctx ? st.d_pipeline_of_ctx[c] : 0;
   /* a thread's own stage and slot: all that does not hang on the pipeline, requested at once */
   int32_t B_own = 1, m_own = 1;
@@ -199,7 +203,7 @@ __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n
     sc.lsub[k] = 0;
     sc.slot_off[k] = P->stage_slot_off[k];
   }
-  __syncthreads();
+  sync();
   for (int32_t s = (int32_t)tid; s < n_slots; s += (int32_t)nt) {
     const bool own = AHEAD && s == (int32_t)tid;
     int64_t acc = own ? w_own : st.d_w_us ? st.d_w_us[(size_t)c * st.slot_stride + s] : 0;
@@ -219,7 +223,7 @@ __device__ __forceinline__ bool ctx_constants(const PipeTable& pipes, uint32_t n
     const int32_t j = s - sc.slot_off[lo];
     if (sums && j < kMaskPaths) sums[lo * kMaskPaths + j] = acc;
   }
-  __syncthreads();
+  sync();
   for (uint32_t k = tid; k < S; k += nt) {
     PardSegConst out;
     out.A = 0; out.A_rel = 0; out.d = 1; out.cap = 1; out.d_magic = 0; out.cap_magic = 0;
