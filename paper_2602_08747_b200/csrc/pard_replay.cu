@@ -2,7 +2,8 @@
  * replay): what pard_plan admitted is what the workers run.  Follows the
  * planner's own reading of paper Sec. 4.2 (t_e, the expected end of the
  * previous batch; batches run back to back) and records the queueing-delay
- * sample that pard_update_queue_delay averages.  One thread per (ctx, stage). */
+ * sample that pard_update_queue_delay averages.  One thread per (ctx, stage); up to kOneBlock of them are
+ * one block, which then also clears the status: a launch and its 2 us less per epoch. */
 #include "pard_plan_internal.cuh"
 
 using namespace pard_plan_detail;
@@ -15,7 +16,8 @@ struct AdvHeader {
 };
 static_assert(sizeof(AdvHeader) == 256, "header is 256 bytes");
 
-__global__ void __launch_bounds__(256)
+constexpr uint32_t kOneBlock = 1024;
+__global__ void __launch_bounds__(kOneBlock)
 k_advance_state(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
                 const int32_t* __restrict__ pipeline_of_ctx, uint32_t n_ctx, uint32_t S,
                 const long long* __restrict__ now_us, const int32_t* __restrict__ batch,
@@ -23,6 +25,10 @@ k_advance_state(const __grid_constant__ PipeTable pipes, uint32_t n_pipelines,
                 long long* __restrict__ free_at, long long* __restrict__ sample_time,
                 int32_t* __restrict__ sample_delay, uint32_t M, uint32_t slot, AdvHeader* __restrict__ hdr) {
   pdl_wait();
+  if (gridDim.x == 1) {
+    if (threadIdx.x < sizeof(AdvHeader) / 4) reinterpret_cast<uint32_t*>(hdr)[threadIdx.x] = 0;
+    __syncthreads();
+  }
   const uint32_t seg = blockIdx.x * blockDim.x + threadIdx.x;
   if (seg >= n_ctx * S) return;
   const uint32_t c = seg / S, k = seg % S;
@@ -99,9 +105,10 @@ extern "C" int pard_advance_state(const pard_pipeline_t* const* pipelines, uint3
   PipeTable table;
   const int trc = pard_pipe_table(pipelines, n_pipelines, (char*)d_workspace + sizeof(AdvHeader), stream, &table);
   if (trc != PARD_OK) return trc;
-  PARD_CUDA_OK(pard_clear_status(hdr, stream));
   const uint32_t n_seg = n_ctx * (uint32_t)stage_stride;
-  PARD_CUDA_OK(launch_pdl(k_advance_state, (n_seg + 255) / 256, 256, 0, stream,
+  const uint32_t threads = n_seg > kOneBlock ? 256u : n_seg <= 64 ? 64u : (n_seg + 31) & ~31u;
+  if (n_seg > kOneBlock) PARD_CUDA_OK(pard_clear_status(hdr, stream));
+  PARD_CUDA_OK(launch_pdl(k_advance_state, (n_seg + threads - 1) / threads, threads, 0, stream,
                           table, n_pipelines, d_pipeline_of_ctx, n_ctx,
                           (uint32_t)stage_stride, (const long long*)d_now_us, d_batch, d_workers, d_seg_kept,
                           (long long*)d_free_at_us, (long long*)d_sample_time_us, d_sample_delay_us, n_samples,
