@@ -440,7 +440,6 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
   extern __shared__ __align__(16) unsigned char emit_raw[];
   EmitSmem& Sm = *reinterpret_cast<EmitSmem*>(emit_raw);
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, below = (1u << lane) - 1, kl = lane & (kDirStages - 1);
-  const bool est32 = ((uintptr_t)out_est & 31) == 0;
   uint32_t phase = 0;
   if (tid == 0) {
     bulk_init(&Sm.full);
@@ -650,13 +649,7 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
           }
         }
         if (mask == 0xfu) {
-          if (out_est) {
-            if (est32) store4(out_est + o, e[0], e[1], e[2], e[3]);
-            else {
-              *reinterpret_cast<longlong2*>(out_est + o) = make_longlong2(e[0], e[1]);
-              *reinterpret_cast<longlong2*>(out_est + o + 2) = make_longlong2(e[2], e[3]);
-            }
-          }
+          if (out_est) store4(out_est + o, e[0], e[1], e[2], e[3]);
           if (out_perm) *reinterpret_cast<uint4*>(out_perm + o) = make_uint4(idx[0], idx[1], idx[2], idx[3]);
           if (out_keep) *reinterpret_cast<uint32_t*>(out_keep + o) = keeps;
         } else {

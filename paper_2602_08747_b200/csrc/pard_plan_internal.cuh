@@ -295,16 +295,21 @@ __device__ __forceinline__ long long slack_of(unsigned long long off, const Pard
   return (K.narrow & kSegHighFirst) ? K.A_rel - (long long)off : (long long)off - K.A_rel;
 }
 
-/* 32 bytes with one access; p is 32-byte aligned */
+/* 32 bytes with one access, from the scratch (p 32-byte aligned) */
 __device__ __forceinline__ void load4(const unsigned long long* p, unsigned long long* v) {
   asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];"
                : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3]) : "l"(p));
 }
+/* 32 bytes of an output, which the caller may have put on a 16-byte boundary: with one access, or with two */
 __device__ __forceinline__ void store4(void* p, unsigned long long a, unsigned long long b,
                                        unsigned long long c, unsigned long long d) {
-  asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" :: "l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+  if (((uintptr_t)p & 31) == 0) {
+    asm volatile("st.global.v4.u64 [%0], {%1, %2, %3, %4};" :: "l"(p), "l"(a), "l"(b), "l"(c), "l"(d) : "memory");
+  } else {
+    asm volatile("st.global.v2.u64 [%0], {%1, %2};" :: "l"(p), "l"(a), "l"(b) : "memory");
+    asm volatile("st.global.v2.u64 [%0+16], {%1, %2};" :: "l"(p), "l"(c), "l"(d) : "memory");
+  }
 }
-
 
 /* `count` elements of 8 bytes, `ahead` of them behind `from` in an array of n, on their way into L2 before the block
  * that will work on them asks for them, by one thread: a block's loads then wait for L2 instead of memory.  Blocks

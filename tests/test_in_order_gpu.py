@@ -86,3 +86,28 @@ def test_errors_are_still_reported():
     keep = ~((wl.requests["ctx"] == 1) & (wl.requests["stage"] >= 2))
     wl.requests = np.ascontiguousarray(wl.requests[keep])
     check(wl)
+
+
+@pytest.mark.parametrize("shift", [0, 16])
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_GROUPED, pb.PARD_MODE_SCAN, pb.PARD_MODE_RAW, pb.PARD_MODE_FCFS])
+@pytest.mark.parametrize("sizes", [[5000], [30_011], [3000, 7001], [20_000, 9_001]])
+def test_outputs_on_16_byte_boundaries(shift, mode, sizes):
+    """What the entry points ask of d_est_us and d_perm; the kernels' widest stores are of 32 bytes."""
+    import torch
+
+    for sort in (True, False):
+        wl = several_ctx(len(sizes), sizes, S=4, m=9, sort=sort)
+        want = oracle.plan(wl.pipelines, wl.requests, wl.state, wl.n_ctx, mode & (pb.PARD_MODE_RAW | pb.PARD_MODE_FCFS))
+        pipes = [pb.pard_load_pipeline(p) for p in wl.pipelines]
+        out = pb.alloc_out(wl.n, wl.n_ctx * 4, "cuda")
+        out.est_us = torch.empty(wl.n + 4, dtype=torch.int64, device="cuda")[shift // 8:]
+        out.perm = torch.empty(wl.n + 8, dtype=torch.int32, device="cuda")[shift // 4:]
+        assert out.est_us.data_ptr() % 32 == shift and out.perm.data_ptr() % 32 == shift
+        ws = pb.alloc_workspace(pb.pard_plan_workspace_bytes(wl.n, wl.n_ctx, 4), "cuda")
+        pb.pard_plan_policy(pipes, pb.device_requests(wl.requests, "cuda"), None, wl.n, pb.device_state(wl.state, "cuda"), wl.n_ctx,
+                            mode, out, ws, stream=torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.est_us[:wl.n].cpu().numpy(), want["est_us"])
+        assert np.array_equal(out.perm[:wl.n].cpu().numpy().view(np.uint32), want["perm"])
+        for p in pipes:
+            p.free()
