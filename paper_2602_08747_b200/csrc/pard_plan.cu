@@ -736,7 +736,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     const uint32_t up = 1u << ibits;
     uint32_t low = 0;                          /* low word of the ctx's smallest deadline */
     for (uint32_t j0 = blockIdx.x * blockDim.x + threadIdx.x; j0 < n; j0 += stride * kUn) {
-      if (threadIdx.x < kUn && n / 4 > stride * kUn)   /* the next round's requests, 256 in a row each (2^24: 5 us less; of three rounds: 1 us more) */
+      if (threadIdx.x < kUn)                   /* the next round's requests, 256 in a row each (2^24: 5 us less) */
         l2_ahead(reinterpret_cast<const unsigned long long*>(req), 2ull * (j0 - threadIdx.x), 2ull * stride * (kUn + threadIdx.x), 512, 2ull * n);
       uint4 rr[kUn];
 #pragma unroll

@@ -315,9 +315,11 @@ __device__ __forceinline__ void store4(void* p, unsigned long long a, unsigned l
  * that will work on them asks for them, by one thread: a block's loads then wait for L2 instead of memory.  Blocks
  * are placed in the order of their tiles, so a tile's load phase comes about as many tiles later as are placed in
  * the meantime.  At 2^24 requests (us per call; before: 528): sort passes 16 tiles ahead (of 296 in flight) 512,
- * 32 ahead 513, 120 ahead 516, 296 ahead 521; the decision 600 tiles ahead another 4 (300 and 2,400: 2). */
+ * 32 ahead 513, 120 ahead 516, 296 ahead 521; the decision 600 tiles ahead another 4 (300 and 2,400: 2).  Not for
+ * arrays that are in L2 as they were written or read before: 9 M elements 332 -> 320 us a call, 4 M 311 -> 313. */
+constexpr uint64_t kAheadFrom = (48ull << 20) / 8;
 __device__ __forceinline__ void l2_ahead(const unsigned long long* src, uint64_t from, uint64_t ahead, uint32_t count, uint64_t n) {
-  if (count && from + ahead + count <= n)
+  if (n > kAheadFrom && count && from + ahead + count <= n)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(src + from + ahead), "r"(count * 8) : "memory");
 }
 constexpr uint32_t kSortAhead = 16, kDecAhead = 600;    /* tiles of kSortTile and of kDecTile */

@@ -175,7 +175,7 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
   const SortedView v = sorted_view(a);
   const bool lookup = a.hdr->lookup != 0;
   const uint64_t tile0 = (uint64_t)blockIdx.x * kPolTile;
-  if (threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);
+  if (MASK == kAllPaths && threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);   /* (the others have no registers left for it) */
   if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
   constexpr int kUn = 4;                           /* elements, then their records, requested together */
   uint32_t cur = 0xffffffffu;
@@ -374,17 +374,19 @@ constexpr uint32_t kWalkClusterLong = 4 * kWalkCtas * kWalkShare;       /* short
 constexpr uint32_t kWalkClusterCap = 4 * kWalkShare;                    /* ... queues of smaller rounds are walked by one block: a round costs */
 constexpr uint32_t kWalkClusterWindow = kWalkShare;                     /* two of the cluster's barriers; windows of Nexus seldom fill */
 constexpr uint32_t kWalkClusterQueues = 37;        /* most queues: as many clusters as two rounds of the device's blocks */
+constexpr uint32_t kWalkCopiesLong = 4 * kWalkShare;   /* from so many requests per queue on, and up to so many queues, one block's */
+constexpr uint32_t kWalkCopiesQueues = 148;        /* thresholds are copied ahead: the room leaves one block per multiprocessor instead of two */
 constexpr uint32_t kWalkSmallRound = 64;           /* rounds below this size are walked by one warp, 32 requests per step: a step
                                                       closes several of them, where a group needs a barrier for each */
 
 /* The thresholds of step after step, 16 consecutive ones per thread; the array may be read up to the next multiple
  * of 16 (workspace).
- * A block (WARPS > 1) has them copied into shared memory, kFeedDepth steps ahead, and reads them there four at a
+ * COPIES: a block has them copied into shared memory, kFeedDepth steps ahead, and reads them there four at a
  * time, the four vectors of a thread in an order that starts a place further with every second thread: as loads of
  * 64 bytes per lane from global memory they took 16 wavefronts an instruction, and a step 1.45 us of which the rest
  * of the work needs 0.5 (16 queues of 2^20, Nexus: the walk 93 us). */
 constexpr int kFeedDepth = 3;
-template <int WARPS, int CTAS>
+template <int WARPS, int CTAS, bool COPIES>
 struct WalkFeed {
   static constexpr uint32_t kStep = WARPS * 32 * kWalkItems;
   const uint32_t* T;
@@ -417,15 +419,13 @@ __device__ __forceinline__ FeedSmem* feed_smem() {
   return reinterpret_cast<FeedSmem*>(walk_raw);
 }
 template <int CTAS>
-struct WalkFeed<(int)kWalkWarps, CTAS> {
+struct WalkFeed<(int)kWalkWarps, CTAS, true> {
   static constexpr uint32_t kShare = kWalkWarps * 32 * kWalkItems;      /* of a block; the step's are the blocks' shares in order of rank */
   FeedSmem& Sm;
   const PolicyArgs& a;
   const uint32_t* T;
   uint32_t from, hi, t, slot, parity, rot;         /* from: first of the next share to fetch; rot: the vector a thread begins with */
   uint32_t left;                                   /* steps for which this block has a share */
-  uint32_t begin;
-  bool alone;                                      /* one step in all: read as it stands (with copies 160 queues of 3,125 took 2 us more) */
   __device__ void fetch(uint32_t to) {             /* by thread 0 */
     if (from >= hi) return;
     bulk_fetch(&Sm.full[to], Sm.ring[to], T + from, ((min(hi - from, kShare) + 3) & ~3u) * 4);
@@ -433,11 +433,7 @@ struct WalkFeed<(int)kWalkWarps, CTAS> {
   }
   __device__ WalkFeed(const PolicyArgs& a_, const uint32_t* T_, uint32_t first, uint32_t hi_, uint32_t t_, uint32_t rank)
       : Sm(*feed_smem()), a(a_), T(T_), from(first + rank * kShare), hi(hi_), t(t_), slot(0), parity(0), rot((t_ >> 1) & 3u),
-        left(from < hi_ ? (hi_ - from + CTAS * kShare - 1) / (CTAS * kShare) : 0u), begin(first), alone(CTAS == 1 && hi_ - first <= kShare) {
-    if (alone) {
-      rot = 0;
-      return;
-    }
+        left(from < hi_ ? (hi_ - from + CTAS * kShare - 1) / (CTAS * kShare) : 0u) {
     if (t == 0) {
       for (int k = 0; k < kFeedDepth; ++k) bulk_init(&Sm.full[k]);
       for (int k = 0; k < kFeedDepth; ++k) fetch(k);
@@ -451,16 +447,6 @@ struct WalkFeed<(int)kWalkWarps, CTAS> {
     for (int i = 0; i < kWalkItems; ++i) u[i] = 0;
     if (!left) return;
     --left;
-    if (alone) {
-      const uint4* mine = reinterpret_cast<const uint4*>(T + begin) + t * (kWalkItems / 4);
-#pragma unroll
-      for (uint32_t q = 0; q < kWalkItems / 4; ++q)
-        if (begin + t * kWalkItems + 4 * q < hi) {
-          const uint4 x = mine[q];
-          u[4 * q] = x.x; u[4 * q + 1] = x.y; u[4 * q + 2] = x.z; u[4 * q + 3] = x.w;
-        }
-      return;
-    }
     const bool late = !bulk_arrived(&Sm.full[slot], parity);
     const uint4* mine = reinterpret_cast<const uint4*>(Sm.ring[slot]) + t * (kWalkItems / 4);
 #pragma unroll
@@ -501,14 +487,14 @@ __device__ __forceinline__ uint32_t walk_range(uint32_t at, uint32_t from, uint3
 
 /* The general rule in rounds of at least kWalkSmallRound.  RAW: every request ahead takes a slot,
  * so a request's round is its position's and no round has to be waited for. */
-template <int WARPS, int CTAS, bool RAW>
+template <int WARPS, int CTAS, bool COPIES, bool RAW>
 __device__ void walk_admit(WalkGroup<WARPS, CTAS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
                            uint32_t hi, const PardSegConst& K) {
   constexpr uint32_t kStep = CTAS * WARPS * 32 * kWalkItems;
   const uint32_t cap = K.cap, t = G.thread();
   uint32_t x = 0, b = 0, left = cap;
   uint32_t at = (lo & ~(uint32_t)(kWalkItems - 1)) + t * kWalkItems;
-  WalkFeed<WARPS, CTAS> feed(a, v.T, lo & ~(uint32_t)(kWalkItems - 1), hi, G.warp * 32 + G.lane, G.rank);
+  WalkFeed<WARPS, CTAS, COPIES> feed(a, v.T, lo & ~(uint32_t)(kWalkItems - 1), hi, G.warp * 32 + G.lane, G.rank);
   for (uint32_t step = lo & ~(uint32_t)(kWalkItems - 1); step < hi; step += kStep, at += kStep) {
     uint32_t u[kWalkItems];
     feed.step(u);
@@ -593,7 +579,7 @@ __device__ void walk_admit_small(const PolicyArgs& a, const SortedView& v, uint3
  * (b < v_r), everything before it is dropped, b advances, the scan goes on behind it.  With `bad`
  * the last position that does not fit (or that ends the window before), a window closes at
  * bad + W, the first time that lies before the next misfit. */
-template <int WARPS, int CTAS>
+template <int WARPS, int CTAS, bool COPIES>
 __device__ void walk_nexus(WalkGroup<WARPS, CTAS>& G, const PolicyArgs& a, const SortedView& v, uint32_t s, uint32_t lo,
                            uint32_t hi, uint32_t W) {
   constexpr uint32_t kStep = CTAS * WARPS * 32 * kWalkItems;
@@ -602,7 +588,7 @@ __device__ void walk_nexus(WalkGroup<WARPS, CTAS>& G, const PolicyArgs& a, const
   uint32_t b = 0;
   int32_t bad = (int32_t)lo - 1;
   uint32_t at = (lo & ~(uint32_t)(kWalkItems - 1)) + t * kWalkItems;
-  WalkFeed<WARPS, CTAS> feed(a, v.T, lo & ~(uint32_t)(kWalkItems - 1), hi, G.warp * 32 + G.lane, G.rank);
+  WalkFeed<WARPS, CTAS, COPIES> feed(a, v.T, lo & ~(uint32_t)(kWalkItems - 1), hi, G.warp * 32 + G.lane, G.rank);
   for (uint32_t step = lo & ~(uint32_t)(kWalkItems - 1); step < hi; step += kStep, at += kStep) {
     uint32_t u[kWalkItems];
     feed.step(u);
@@ -687,7 +673,7 @@ __device__ void walk_nexus_small(const PolicyArgs& a, const SortedView& v, uint3
 /* CTAS > 1: a cluster per queue, for the queues where its barriers are worth it: many steps, few rounds.  The first
  * block of the cluster walks the others by itself.  (A step of one block 1.2 us, of a cluster some 1.5 for eight times
  * the requests, a round 0.6 and 1.5; 2^23 requests with known paths in 32 queues of 2^18: 612 by blocks, 621 by clusters.) */
-template <int WARPS, int CTAS>
+template <int WARPS, int CTAS, bool COPIES>
 __global__ void __launch_bounds__(WARPS == 1 ? kPolThreads : WARPS * 32)
 k_policy_walk(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
@@ -714,9 +700,9 @@ k_policy_walk(const __grid_constant__ PolicyArgs a) {
   auto walk = [&](auto ctas) {
     constexpr int N = decltype(ctas)::value;
     WalkGroup<WARPS, N> G{reinterpret_cast<typename WalkGroup<WARPS, N>::Shared&>(sh[WARPS == 1 ? warp : 0]), lane, WARPS == 1 ? 0u : warp, N > 1 ? rank : 0u, 0u};
-    if (nexus) walk_nexus<WARPS, N>(G, a, v, s, lo, hi, K.cap);
-    else if (raw) walk_admit<WARPS, N, true>(G, a, v, s, lo, hi, K);
-    else walk_admit<WARPS, N, false>(G, a, v, s, lo, hi, K);
+    if (nexus) walk_nexus<WARPS, N, COPIES>(G, a, v, s, lo, hi, K.cap);
+    else if (raw) walk_admit<WARPS, N, COPIES, true>(G, a, v, s, lo, hi, K);
+    else walk_admit<WARPS, N, COPIES, false>(G, a, v, s, lo, hi, K);
   };
   if (CTAS > 1 && (raw || K.cap < (nexus ? kWalkClusterWindow : kWalkClusterCap) || hi - lo < kWalkClusterLong)) {
     if (rank == 0) walk(std::integral_constant<int, 1>());
@@ -747,7 +733,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile0 = blockIdx.x * kPolTile;
   const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
-  if (threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);
+  if (MASK == kAllPaths && threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);   /* (the others have no registers left for it) */
   if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
   unsigned long long e[kPolItems];
   uint32_t t[kPolItems], round[kPolItems], flags[kPolItems];
@@ -881,8 +867,8 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
 namespace pard_plan_detail {
 
 int allow_walk_smem() {
-  PARD_CUDA_OK(cudaFuncSetAttribute(k_policy_walk<kWalkWarps, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FeedSmem)));
-  PARD_CUDA_OK(cudaFuncSetAttribute(k_policy_walk<kWalkWarps, kWalkCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FeedSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_policy_walk<kWalkWarps, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FeedSmem)));
+  PARD_CUDA_OK(cudaFuncSetAttribute(k_policy_walk<kWalkWarps, kWalkCtas, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FeedSmem)));
   return PARD_OK;
 }
 
@@ -893,11 +879,12 @@ int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
   launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
              tiles, kPolThreads, 0, stream, a);
   if (a.n / a.n_seg >= kWalkClusterLong / 2 && a.n_seg <= kWalkClusterQueues)
-    PARD_CUDA_OK(launch_pdl_cluster(k_policy_walk<kWalkWarps, kWalkCtas>, a.n_seg * kWalkCtas, kWalkWarps * 32, sizeof(FeedSmem), kWalkCtas, stream, a));
+    PARD_CUDA_OK(launch_pdl_cluster(k_policy_walk<kWalkWarps, kWalkCtas, true>, a.n_seg * kWalkCtas, kWalkWarps * 32, sizeof(FeedSmem), kWalkCtas, stream, a));
   else if (a.n / a.n_seg >= kWalkLong)
-    launch_pdl(k_policy_walk<kWalkWarps, 1>, a.n_seg, kWalkWarps * 32, sizeof(FeedSmem), stream, a);
+    launch_pdl(a.n / a.n_seg >= kWalkCopiesLong && a.n_seg <= kWalkCopiesQueues ? k_policy_walk<kWalkWarps, 1, true> : k_policy_walk<kWalkWarps, 1, false>,
+               a.n_seg, kWalkWarps * 32, a.n / a.n_seg >= kWalkCopiesLong && a.n_seg <= kWalkCopiesQueues ? sizeof(FeedSmem) : 0, stream, a);
   else
-    launch_pdl(k_policy_walk<1, 1>, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
+    launch_pdl(k_policy_walk<1, 1, false>, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
 }
 
