@@ -392,7 +392,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
  * it by more than their number, so the running minimum over the slots is a running maximum of (stage, amount) in one
  * word, which never leaks from one queue into the next.  The next tile is copied into shared memory meanwhile.
  * Pieces are taken by ticket.  Bound by shared memory (two thirds of its wavefronts) and instructions: 127 us for 2^24
- * requests of 16 stages, 82 by its bytes (16 in, 13 + 4f out).  On the way there: a lane per request 151, groups of
+ * requests of 16 stages, 75 by its bytes (16 in, 13 + 4f out, 8 % kept).  On the way there: a lane per request 151, groups of
  * 8 slots 147, with copies ahead and what does not fill a group left for the next tile 131; a warp per tile without
  * block barriers 156; ranks from four-bit counters per thread instead of ballots the same 127. */
 constexpr int kEmitRounds = 2;                    /* groups per thread */

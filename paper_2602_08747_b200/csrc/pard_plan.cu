@@ -14,8 +14,8 @@
  *   decide    every request on its own from its queue's table: admitted position c, estimate, keep
  *             flag, survivors to their final place; too many windows: the same by a segmented
  *             prefix-min scan (k_scan_path)
- * Calls grouped by ctx in small contexts are planned by a block per ctx (pard_local.cu), the comparison
- * rules by a walk of every queue behind the sort (pard_policy.cu).
+ * Calls grouped by ctx in small contexts are planned by a block per ctx (pard_local.cu), in large ones that come in
+ * order without a sort (pard_direct.cuh), the comparison rules by a walk of every queue behind the sort (pard_policy.cu).
  */
 #include <algorithm>
 #include <atomic>
@@ -388,7 +388,7 @@ k_seg_const(const __grid_constant__ ConstArgs a, const unsigned long long* __res
 }
 
 /* The constants are there but for what they take from the deadline ranges (k_dir_count worked them out): a thread per
- * queue; the block that finishes last finds the key width.  (k_seg_const anew: 12 us more for 8,192 queues.) */
+ * queue; the block that finishes last finds the key width.  (k_seg_const, which would do it all again, takes 13 us for 8,192 queues.) */
 __global__ void __launch_bounds__(256)
 k_seg_finish(const __grid_constant__ ConstArgs a, const unsigned long long* __restrict__ ctx_dmin_inv,
              const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr) {
@@ -3042,7 +3042,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
 
   /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
-   * 288 k of 24 contexts 71 -> 51; out of order they pay for the try, 567 -> 575 and 117 -> 118.  Without the caller's
+   * 288 k of 24 contexts 71 -> 51; out of order they pay for the try, 567 -> 574 and 117 -> 118.  Without the caller's
    * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
   DirectArgs da = {};
   const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN | PARD_MODE_TEST_STALL)) &&
