@@ -1227,6 +1227,8 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
       S.base = ct.ctx_start[lo] + (t - ct.tile_first[lo]) * (uint32_t)kSortTile;
       S.limit = ct.ctx_start[lo + 1];
       S.first = ct.ctx_start[lo];
+      /* (tiles of one ctx after the other: about that far on, from a 16-byte boundary) */
+      if (!PERSIST) l2_ahead(src, S.base & ~1u, (uint64_t)kSortAhead * kSortTile, kSortTile, n);
     }
   }
   for (uint32_t i = tid; i < WARPS * kBins; i += kSortThreads) {
@@ -3042,7 +3044,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
 
   /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
-   * 288 k of 24 contexts 71 -> 51; out of order they pay for the try, 567 -> 574 and 117 -> 118.  Without the caller's
+   * 288 k of 24 contexts 71 -> 51; out of order the try costs 7 of 567 us, 1 of 117
+   * (the passes behind it, their tiles on the way into L2 ahead of them, made up for it: 542 and 118).  Without the caller's
    * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
   DirectArgs da = {};
   const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN | PARD_MODE_TEST_STALL)) &&
