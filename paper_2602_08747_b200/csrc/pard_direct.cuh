@@ -254,11 +254,12 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
       if (g.narrow & kSegNoStage) mineK.A = -1;   /* no such stage: its requests are input errors */
       else off |= !dir_const(g, D0, mineK);
     }
+    off |= D0 >= (unsigned long long)PARD_TIME_LIMIT_US - (1ull << 31);      /* in every warp: whichever holds a deadline beyond the limit looks for it */
     if (tid == 0) {
       /* the ctx's deadlines must leave room for the key that a sort would need */
       const uint32_t first = __ldcg(&a.ctx_start[c]), stop = __ldcg(&a.ctx_start[c + 1]);
       const unsigned long long Df = deadline(min(first, a.n - 1)), Dl = deadline(min(max(stop, 1u), a.n) - 1), Dp = deadline(begin > first ? begin - 1 : begin);
-      off |= Dl < Df || D0 < Dp || D0 >= (unsigned long long)PARD_TIME_LIMIT_US - (1ull << 31) || a.sbits + a.ibits + bit_width64(Dl - Df) > 64;
+      off |= Dl < Df || D0 < Dp || a.sbits + a.ibits + bit_width64(Dl - Df) > 64;
     }
   }
   if (lane < kDirStages) { s_K[warp][lane] = mineK; s_low[warp][lane] = kDirInf; }

@@ -88,6 +88,22 @@ def test_errors_are_still_reported():
     check(wl)
 
 
+@pytest.mark.parametrize("ctx", [0, 1])
+@pytest.mark.parametrize("crossing", [0, 1, 255, 256, 257, 600, 1039, 1040])
+def test_deadlines_that_cross_the_limit_inside_the_last_piece(ctx, crossing):
+    """Deadlines of a ctx one microsecond apart, the first one outside [0, 2^60) so many requests behind the beginning
+    of the ctx's last piece (8,960: five tiles; 256 requests to a warp); 1,040: behind its last request."""
+    wl = several_ctx(2, [10_000, 10_000], S=4, m=20)
+    wl.state.now_us[ctx] = (1 << 60) - 20_000
+    wl.requests["deadline_us"][10_000 * ctx:][:10_000] = (1 << 60) - 8_960 - crossing + np.arange(10_000)
+    if crossing == 1040:
+        check(wl)
+        check(wl, 0)
+    else:
+        for mode in (pb.PARD_MODE_GROUPED, 0):
+            assert run_library(wl, mode, check=False)[0] == pb.PARD_EDATA
+
+
 @pytest.mark.parametrize("shift", [0, 16])
 @pytest.mark.parametrize("mode", [0, pb.PARD_MODE_GROUPED, pb.PARD_MODE_SCAN, pb.PARD_MODE_RAW, pb.PARD_MODE_FCFS])
 @pytest.mark.parametrize("sizes", [[5000], [30_011], [3000, 7001], [20_000, 9_001]])
