@@ -13,7 +13,8 @@
  *   k_dir_emit    every tile's requests ordered by stage in shared memory, decided, written to their place
  * What the path does not take -- deadlines that step back, requests not grouped, input errors, constants
  * beyond 32 bits -- is found out by k_dir_count (direct_off); the kernels of the general path, launched behind
- * these in any case, then do the work, and return at once otherwise. */
+ * these in any case, then do the work, and return at once otherwise.  Whether a deadline stepped back goes to
+ * them too (pair_steps_back): without one their passes take the stage bits alone. */
 
 constexpr int kDirThreads = 256;
 constexpr int kDirWarps = kDirThreads / 32;
@@ -33,6 +34,8 @@ struct DirectArgs {
   uint4* piece_info;                              /* [n_pieces] ctx, first request, end, 0 */
   uint2* piece_rows;                              /* [n_pieces][kDirStages] count, minimum; from k_dir_scan on: of all earlier pieces of the ctx */
 };
+
+constexpr uint32_t kDirOff = 1u, kDirSteps = 2u;  /* bits of PlanHeader::direct_off; the second: a step back has been seen, nobody needs to look for more */
 
 /* {count, minimum} of a span followed by another */
 __device__ __forceinline__ uint2 dir_then(uint2 a, uint2 b) { return make_uint2(a.x + b.x, (uint32_t)min((int32_t)a.y, (int32_t)b.y - (int32_t)a.x)); }
@@ -210,6 +213,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   __shared__ uint2 s_warp[kDirWarps][kDirStages];
   __shared__ int32_t s_low[kDirWarps][kDirStages];
   __shared__ unsigned long long s_min[kDirWarps], s_max[kDirWarps];
+  __shared__ bool s_back[kDirWarps];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t piece = blockIdx.x;
   uint4 info = __ldcg(&a.piece_info[piece]);
@@ -228,7 +232,8 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
       if (pos + i * 32 + lane < wend) r[i] = __ldg(&a.req[pos + i * 32 + lane]);
     }
   };
-  bool off = nonsense || ld_relaxed(&hdr->direct_off) != 0;
+  const uint32_t off_word = ld_relaxed(&hdr->direct_off);
+  bool off = nonsense || off_word != 0;
   if (!off) fetch(wbegin);
   /* the boundaries found must ascend from 0 to n (the requests' own ctxs are compared below: both together prove the grouping) */
   bool gaps = false, bad_const = false;
@@ -245,7 +250,11 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   }
   auto deadline = [&](uint32_t j) { return __ldg(reinterpret_cast<const unsigned long long*>(&a.req[j])); };
   const unsigned long long D0 = !off && begin < end ? deadline(begin) : 0ull;
-  uint32_t last = !off && wbegin < wend && wbegin > begin ? (uint32_t)(deadline(wbegin - 1) - D0) : 0u;
+  uint32_t last = 0;                              /* offset of the request before; in 32 bits or not one that may come before any */
+  if (!off && wbegin < wend && wbegin > begin) {
+    const unsigned long long before = deadline(wbegin - 1) - D0;
+    last = before >> 32 ? 0xffffffffu : (uint32_t)before;
+  }
   DirConst mineK = {0, 1u, 1u, 0ull};             /* every warp keeps the constants for itself: no barrier before the end */
   if (!off && begin < end) {
     const uint32_t k = lane & (kDirStages - 1);
@@ -267,6 +276,7 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   uint32_t run = 0, ucur = 0;
   int32_t low = kDirInf, next = mineK.A;
   unsigned long long lmin = ~0ull, lmax = 0;
+  bool stepped = false;
   /* the figures of the requests so far, as {count, minimum} */
   auto figures = [&]() {
     const int32_t m = min(low, s_low[warp][lane & (kDirStages - 1)]);
@@ -320,32 +330,49 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
       lmax = deadline(wend - 1);
     }
   }
-  if (off) {                            /* what k_prepass would find: the deadlines' range, input errors */
+  /* What k_prepass would find: the deadlines' range, input errors, steps back (the warps that stay out of this have
+   * found none, the request ahead of their first one included).  The path may be off for another reason: requests in
+   * order then need no more passes than if it had not been tried.  (With steps back taken for granted, ordered requests
+   * of 256 contexts, 2^24 with one stage of 1 us: 812 us a call, now 609; 288 k of 24 in two halves 2^32 us apart:
+   * 128 and 85.  The general path by itself: 608 and 84.)  The next rows are asked for ahead (unordered 2^24 547 -> 543). */
+  if (off) {
     bool bad = false, foreign = nonsense;
     lmin = ~0ull;
     lmax = 0;
-    for (uint32_t pos = wbegin + lane; pos - lane < wend; pos += 32 * kUn) {
-      uint4 v[kUn];
+    auto look = [&](auto steps) {
+      constexpr bool STEPS = decltype(steps)::value;
+      unsigned long long prev = 0;                /* lane 31: of the row before */
+      if (STEPS && wbegin < wend && (wbegin > begin || begin > __ldcg(&a.ctx_start[c]))) prev = deadline(wbegin - 1);
+      fetch(wbegin);
+      for (uint32_t pos = wbegin; pos < wend; pos += 32 * kUn) {
+        uint4 v[kUn];
 #pragma unroll
-      for (int i = 0; i < kUn; ++i) {
-        v[i] = make_uint4(0u, 0xffffffffu, c, 0u);
-        if (pos + i * 32 < wend) v[i] = __ldg(&a.req[pos + i * 32]);
-      }
+        for (int i = 0; i < kUn; ++i) v[i] = r[i];
+        fetch(pos + 32 * kUn);
 #pragma unroll
-      for (int i = 0; i < kUn; ++i) {
-        const unsigned long long D = ((unsigned long long)v[i].y << 32) | v[i].x;
-        const bool there = pos + i * 32 < wend;
-        foreign |= there && v[i].z != c;
-        if (D >= (unsigned long long)PARD_TIME_LIMIT_US || v[i].z != c || (v[i].w & 0xffffu) >= a.S) {
-          bad |= there && v[i].z == c;
-          continue;
+        for (int i = 0; i < kUn; ++i) {
+          const bool there = pos + i * 32 + lane < wend;
+          const unsigned long long D = there ? ((unsigned long long)v[i].y << 32) | v[i].x : ~0ull;
+          if (STEPS) {                            /* (rows beyond the share compare as in order) */
+            const unsigned long long pD = __shfl_sync(0xffffffffu, lane == 31 ? prev : D, (lane - 1) & 31);
+            prev = D;
+            stepped |= D < pD;
+          }
+          foreign |= there && v[i].z != c;
+          if (D >= (unsigned long long)PARD_TIME_LIMIT_US || v[i].z != c || (v[i].w & 0xffffu) >= a.S) {
+            bad |= there && v[i].z == c;
+            continue;
+          }
+          lmin = D < lmin ? D : lmin;
+          lmax = D > lmax ? D : lmax;
         }
-        lmin = D < lmin ? D : lmin;
-        lmax = D > lmax ? D : lmax;
       }
-    }
+    };
+    if (__any_sync(0xffffffffu, off_word & kDirSteps)) look(std::false_type());
+    else look(std::true_type());
     if (bad) set_status(hdr, PARD_EDATA);
     if (foreign) hdr->unsorted = 1;
+    stepped = __any_sync(0xffffffffu, stepped);
     for (int o = 16; o; o >>= 1) {
       const unsigned long long p = __shfl_xor_sync(0xffffffffu, lmin, o), q = __shfl_xor_sync(0xffffffffu, lmax, o);
       lmin = p < lmin ? p : lmin;
@@ -354,12 +381,13 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
   }
   __syncwarp();
   if (lane < kDirStages) s_warp[warp][lane] = figures();
-  if (lane == 0) { s_min[warp] = lmin; s_max[warp] = lmax; }
+  if (lane == 0) { s_min[warp] = lmin; s_max[warp] = lmax; s_back[warp] = stepped; }
   const bool block_off = __syncthreads_or(off);
   if (tid == 0) {
     for (int w = 1; w < kDirWarps; ++w) {
       lmin = s_min[w] < lmin ? s_min[w] : lmin;
       lmax = s_max[w] > lmax ? s_max[w] : lmax;
+      stepped |= s_back[w];
     }
     if (lmin <= lmax) {
       if (__ldcg(&ctx_dmin_inv[c]) < ~lmin) atomicMax(&ctx_dmin_inv[c], ~lmin);
@@ -367,9 +395,12 @@ k_dir_count(const __grid_constant__ DirectArgs a, const __grid_constant__ ConstA
     }
   }
   if (block_off) {
-    if (tid == 0 && !ld_relaxed(&hdr->direct_off)) {
-      hdr->time_steps_back = hdr->pair_steps_back = 1;   /* (or something else the path does not take: the sort then does more than it must) */
-      st_relaxed(&hdr->direct_off, 1u);
+    if (tid == 0) {
+      const uint32_t word = stepped ? kDirOff | kDirSteps : kDirOff;
+      if (word & ~ld_relaxed(&hdr->direct_off)) {
+        if (stepped) hdr->time_steps_back = hdr->pair_steps_back = 1;    /* inside a ctx: both */
+        atomicOr(&hdr->direct_off, word);
+      }
     }
   } else if (tid < kDirStages) {
     uint2 sum = make_uint2(0u, (uint32_t)kDirInf);

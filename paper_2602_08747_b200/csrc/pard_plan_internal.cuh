@@ -67,7 +67,7 @@ struct PlanHeader {
   uint32_t lookup;            /* 1: the elements hold no deadline: it has to be looked up in the request array */
   uint32_t sort_bar[kMaxPasses]; /* tiles of each of k_sort_rest's passes that are finished */
   uint32_t direct;            /* 1: the requests came in order, the plan is made without a sort (pard_direct.cuh) */
-  uint32_t direct_off;        /* 1: they did not, or something else that path does not take */
+  uint32_t direct_off;        /* not 0: they did not, or something else that path does not take (kDirOff, kDirSteps) */
   uint32_t direct_done;       /* blocks of k_dir_count that have finished */
   uint32_t direct_ticket;     /* pieces taken by k_dir_emit */
   uint32_t walk_late;         /* 1: a wait of the rules' walk ran out: `aborted` for the kernels behind it (its own blocks go on together) */

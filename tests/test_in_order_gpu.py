@@ -48,6 +48,65 @@ def test_one_deadline_steps_back(at):
         check(wl)
 
 
+# ---- in order, but not for this path: the passes behind it then sort the stage bits alone ----------------------------
+def radix_passes(wl):
+    """The passes that a call's sort needed: word 3 of its workspace."""
+    import torch
+
+    pipes = [pb.pard_load_pipeline(p) for p in wl.pipelines]
+    S = wl.state.stage_stride
+    ws = pb.alloc_workspace(pb.pard_plan_workspace_bytes(wl.n, wl.n_ctx, S), "cuda")
+    pb.pard_plan(pipes, pb.device_requests(wl.requests, "cuda"), wl.n, pb.device_state(wl.state, "cuda"), wl.n_ctx, pb.PARD_MODE_GROUPED,
+                 pb.alloc_out(wl.n, wl.n_ctx * S, "cuda"), ws, stream=torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    for p in pipes:
+        p.free()
+    return int(ws[12:16].view(torch.int32).item())
+
+
+def off_the_path(reason, n_ctx=3, per=20_000, **kw):
+    wl = several_ctx(n_ctx, [per] * n_ctx, S=8, m=20, **kw)
+    d = wl.requests["deadline_us"].reshape(n_ctx, per)
+    if reason == "stage of 1 us":
+        wl.pipelines = [util.pipeline(inputs.chain_edges(8), 8, [9, 30, 1, 7, 12, 5, 17, 8], bmax=4)]
+    elif reason == "piece beyond 32 bits":
+        d[1, per // 2:] += 1 << 32
+    elif reason == "piece beyond 31 bits":
+        d[n_ctx - 1, per // 3:] += 1 << 31
+    elif reason == "booked long ago":
+        d[0] += (1 << 31) + 5000
+    return wl
+
+
+@pytest.mark.parametrize("reason,n_ctx,per", [(r, c, k) for r in ("stage of 1 us", "piece beyond 32 bits", "piece beyond 31 bits", "booked long ago")
+                                              for c, k in ((3, 20_000), (70, 16_384))] + [("stage of 1 us", 1025, 8_193)])
+def test_in_order_for_the_passes_alone(reason, n_ctx, per):
+    wl = off_the_path(reason, n_ctx, per)
+    check(wl)
+    assert radix_passes(wl) == 1
+    for at in (per + 1, 2 * per - 1)[:1 if n_ctx > 1000 else 2]:                    # one step back, in the second ctx
+        wl = off_the_path(reason, n_ctx, per)
+        wl.requests["deadline_us"][at] = wl.requests["deadline_us"][at - 1] - 1
+        check(wl)
+        assert radix_passes(wl) > 1
+
+
+@pytest.mark.parametrize("reason", ["", "stage of 1 us", "piece beyond 32 bits"])
+@pytest.mark.parametrize("at", [1, 31, 32, 255, 256, 257, 1791, 1792, 1793, 2048, 20_001, 21_792, 39_999])
+def test_no_step_back_is_missed(reason, at):
+    """By one microsecond; behind a deadline too far ahead for 32-bit offsets, its low word small; and over several requests."""
+    for far, until in ((0, at), (1 << 31, at), (1 << 32, at), ((1 << 32) - 5, at), (0, at + 300), (1 << 33, at + 300)):
+        wl = off_the_path(reason)
+        d = wl.requests["deadline_us"]
+        if far:
+            d[max(until - 300, at - 1):until] += far      # a step back at `until`
+        elif until > at:
+            d[at:until] -= 900                            # at `at` (and none behind)
+        else:
+            d[at] = d[at - 1] - 1
+        check(wl)
+
+
 @pytest.mark.parametrize("span", [3000, (1 << 31) - 3, (1 << 31) - 2, (1 << 31) - 1, 1 << 31, 1 << 33])
 @pytest.mark.parametrize("d", [1, 7, (1 << 31) + 9, (1 << 32) + 9])
 def test_constants_at_the_limits(span, d):
