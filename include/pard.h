@@ -172,7 +172,9 @@ typedef struct pard_plan_out {
 #define PARD_MODE_SCAN     4u   /* take the decision by the scan path even when the
                                    batch-window tables would do (same results; the scan
                                    is otherwise the fallback for queues with thousands
-                                   of batch windows).  The scan path is one kernel whose
+                                   of batch windows); under the rules below, whose queues
+                                   are walked, by one block each also where clusters of
+                                   blocks would do.  The scan path is one kernel whose
                                    blocks wait between its steps for the work of other
                                    running blocks, each wait bounded at about half a
                                    second                                             */

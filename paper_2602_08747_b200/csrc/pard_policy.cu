@@ -872,13 +872,34 @@ int allow_walk_smem() {
   return PARD_OK;
 }
 
+/* A cluster's blocks are placed together.  Whether the device, or the share of it that this context may use, has room
+ * for one at all is asked for every such call, not once: the share may change.  (The host's 25 us per call of 2^24
+ * requests stay what they were; by one block each the 16 queues take 22 us more, 420 against 398.) */
+static bool cluster_walk_fits() {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = kWalkCtas;
+  cfg.blockDim = kWalkWarps * 32;
+  cfg.dynamicSmemBytes = sizeof(FeedSmem);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kWalkCtas;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, k_policy_walk<kWalkWarps, kWalkCtas, true>, &cfg) == cudaSuccess) return clusters > 0;
+  cudaGetLastError();                              /* an answer like any other: nothing of the call has failed */
+  return false;
+}
+
 int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
   static_assert(kWalkItems < (int)kWalkSmallRound, "a window is longer than a thread's share of a step");
   static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
   launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
              tiles, kPolThreads, 0, stream, a);
-  if (a.n / a.n_seg >= kWalkClusterLong / 2 && a.n_seg <= kWalkClusterQueues)
+  PARD_CUDA_OK(cudaGetLastError());
+  if (a.n / a.n_seg >= kWalkClusterLong / 2 && a.n_seg <= kWalkClusterQueues && !(a.mode & PARD_MODE_SCAN) && cluster_walk_fits())
     PARD_CUDA_OK(launch_pdl_cluster(k_policy_walk<kWalkWarps, kWalkCtas, true>, a.n_seg * kWalkCtas, kWalkWarps * 32, sizeof(FeedSmem), kWalkCtas, stream, a));
   else if (a.n / a.n_seg >= kWalkLong)
     launch_pdl(a.n / a.n_seg >= kWalkCopiesLong && a.n_seg <= kWalkCopiesQueues ? k_policy_walk<kWalkWarps, 1, true> : k_policy_walk<kWalkWarps, 1, false>,

@@ -314,3 +314,18 @@ def test_walk_by_clusters(rule, cap, sizes):
         late = rng.random(wl.n) < share
         wl.requests["deadline_us"] = np.where(late, rng.integers(0, 60, size=wl.n), 10**6)
         check(wl, rule)
+
+
+# ---- the same where a cluster cannot be placed: by one block each (PARD_MODE_SCAN asks for it) -------------------------
+@pytest.mark.parametrize("rule", [FCFS, NEXUS, pb.PARD_MODE_PATH_MASK])
+@pytest.mark.parametrize("cap", [16_384, 65_536, 150_001])
+@pytest.mark.parametrize("sizes", [[524_288], [900_000, 0, 540_000, 560_000]])
+def test_walk_of_long_queues_without_clusters(rule, cap, sizes):
+    B = next(b for b in range(4096, 0, -1) if cap % b == 0)
+    wl = several_ctx(len(sizes), sizes, S=1, sort=False)
+    rng = np.random.default_rng(cap)
+    wl.pipelines = [util.pipeline([], 1, [13], bmax=4096)]
+    wl.state = util.state(len(sizes), 1, 0, 0, B, workers=cap // B)
+    wl.requests["deadline_us"] = np.where(rng.random(wl.n) < 0.001, rng.integers(0, 60, size=wl.n), 10**6)
+    got = check(wl, rule | pb.PARD_MODE_SCAN)
+    assert_identical(got, check(wl, rule))
