@@ -183,7 +183,9 @@ typedef struct pard_plan_out {
                                    later tiles wait for (and is never counted as finished,
                                    which the next pass waits for), and the first tiles of the scan
                                    path's first step (PARD_MODE_SCAN) are never counted as
-                                   finished, which its next step waits for; the waits run
+                                   finished, which its next step waits for; a block of the path without
+                                   a sort (PARD_MODE_GROUPED, in order) and of the rules' walk of a
+                                   long queue never asks for the first copy it waits for; the waits run
                                    out (after a fraction of a second) and the call returns
                                    PARD_ETIMEOUT with unspecified outputs; the CUDA
                                    context stays usable.  Calls that the library sorts

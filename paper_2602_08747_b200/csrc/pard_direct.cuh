@@ -31,6 +31,7 @@ struct DirectArgs {
   uint32_t* ctx_start;                            /* [n_ctx + 1] */
   uint32_t* const_bad;                            /* [n_ctx] 1: an input of the constants out of range */
   uint32_t piece, n_pieces;                       /* requests per piece, a multiple of the tile; pieces (some may be empty) */
+  uint32_t stall;                                 /* testing aid: k_dir_emit's first block never asks for its first tile */
   uint4* piece_info;                              /* [n_pieces] ctx, first request, end, 0 */
   uint2* piece_rows;                              /* [n_pieces][kDirStages] count, minimum; from k_dir_scan on: of all earlier pieces of the ctx */
 };
@@ -484,7 +485,7 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
     }
     Sm.next = p;
     Sm.info = info;
-    if (p < a.n_pieces) emit_fetch(Sm, a.req + info.y, min(kDirTile, info.z - info.y));
+    if (p < a.n_pieces && !(a.stall && blockIdx.x == 0)) emit_fetch(Sm, a.req + info.y, min(kDirTile, info.z - info.y));
   }
   __syncthreads();
   for (;;) {

@@ -3048,10 +3048,10 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
    * (the passes behind it, their tiles on the way into L2 ahead of them, made up for it: 542 and 118).  Without the caller's
    * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
   DirectArgs da = {};
-  const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN | PARD_MODE_TEST_STALL)) &&
+  const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN)) &&
                       !state->d_priority && dir_layout(n, n_ctx, S, (char*)buf_b, &da);
   da.req = req4; da.n = n32; da.n_ctx = n_ctx; da.S = S; da.sbits = sbits; da.ibits = ibits;
-  da.ktab = ktab; da.ctx_start = ctx_start; da.const_bad = kept_tmp;
+  da.ktab = ktab; da.ctx_start = ctx_start; da.const_bad = kept_tmp; da.stall = (mode & PARD_MODE_TEST_STALL) ? 1u : 0u;
 
   /* ---- clear the scratch that must start at zero: one contiguous region ---- */
   if (!direct) {

@@ -349,7 +349,7 @@ __device__ __forceinline__ void bulk_fetch(unsigned long long* bar, void* dst, c
 /* false: the copy has not arrived within about a second */
 __device__ __forceinline__ bool bulk_arrived(unsigned long long* bar, uint32_t parity) {
   const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
-  for (uint32_t spins = 0; spins < 1u << 20; ++spins) {
+  for (uint32_t spins = 0; spins < 1u << 18; ++spins) {
     uint32_t done;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(done) : "r"(b), "r"(parity) : "memory");

@@ -436,7 +436,10 @@ struct WalkFeed<(int)kWalkWarps, CTAS, true> {
         left(from < hi_ ? (hi_ - from + CTAS * kShare - 1) / (CTAS * kShare) : 0u) {
     if (t == 0) {
       for (int k = 0; k < kFeedDepth; ++k) bulk_init(&Sm.full[k]);
-      for (int k = 0; k < kFeedDepth; ++k) fetch(k);
+      for (int k = 0; k < kFeedDepth; ++k) {
+        if (k == 0 && (a.mode & PARD_MODE_TEST_STALL) && blockIdx.x == 0) from += CTAS * kShare;     /* testing aid: a share never asked for */
+        else fetch(k);
+      }
     }
     __syncthreads();
   }
@@ -455,6 +458,8 @@ struct WalkFeed<(int)kWalkWarps, CTAS, true> {
       u[4 * q] = x.x; u[4 * q + 1] = x.y; u[4 * q + 2] = x.z; u[4 * q + 3] = x.w;
     }
     if (__syncthreads_or(late)) {                  /* (also: everybody has read the slot) */
+#pragma unroll
+      for (int i = 0; i < kWalkItems; ++i) u[i] = 0;
       left = 0;
       if (t == 0) {
         for (int k = 0; k < kFeedDepth; ++k) bulk_arrived(&Sm.full[k], k < (int)slot ? parity ^ 1 : parity);   /* no copy is under way when the block ends */

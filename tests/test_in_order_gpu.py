@@ -163,6 +163,13 @@ def test_deadlines_that_cross_the_limit_inside_the_last_piece(ctx, crossing):
             assert run_library(wl, mode, check=False)[0] == pb.PARD_EDATA
 
 
+@pytest.mark.parametrize("sizes", [[9000, 9000], [20_000, 0, 30_000], [65_536] * 20])
+def test_wait_for_a_tile_runs_out_and_is_reported(sizes):
+    wl = several_ctx(len(sizes), sizes, S=8, m=20)
+    assert run_library(wl, pb.PARD_MODE_GROUPED | pb.PARD_MODE_TEST_STALL, check=False)[0] == pb.PARD_ETIMEOUT
+    check(wl)
+
+
 @pytest.mark.parametrize("shift", [0, 16])
 @pytest.mark.parametrize("mode", [0, pb.PARD_MODE_GROUPED, pb.PARD_MODE_SCAN, pb.PARD_MODE_RAW, pb.PARD_MODE_FCFS])
 @pytest.mark.parametrize("sizes", [[5000], [30_011], [3000, 7001], [20_000, 9_001]])

@@ -316,6 +316,16 @@ def test_walk_by_clusters(rule, cap, sizes):
         check(wl, rule)
 
 
+@pytest.mark.parametrize("rule", [FCFS, NEXUS])
+@pytest.mark.parametrize("walk", [0, pb.PARD_MODE_SCAN])   # by a cluster, by one block
+def test_wait_for_copied_thresholds_runs_out_and_is_reported(rule, walk):
+    wl = several_ctx(1, [600_001], S=1, sort=False)        # one queue in arrival order: no radix pass whose wait would run out first
+    wl.pipelines = [util.pipeline([], 1, [13], bmax=4096)]
+    wl.state = util.state(1, 1, 0, 0, 4096, workers=16)
+    assert run_library(wl, rule | walk | pb.PARD_MODE_TEST_STALL, check=False)[0] == pb.PARD_ETIMEOUT
+    check(wl, rule | walk)
+
+
 # ---- the same where a cluster cannot be placed: by one block each (PARD_MODE_SCAN asks for it) -------------------------
 @pytest.mark.parametrize("rule", [FCFS, NEXUS, pb.PARD_MODE_PATH_MASK])
 @pytest.mark.parametrize("cap", [16_384, 65_536, 150_001])
