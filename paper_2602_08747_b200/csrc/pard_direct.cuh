@@ -724,9 +724,9 @@ k_dir_emit(const __grid_constant__ DirectArgs a, PlanHeader* __restrict__ hdr, c
  * of at most four tiles, so that the blocks of long and of short contexts end together.  (One ctx: its constants would
  * have to be there before the requests are read, where k_prepass works them out meanwhile; a million requests in
  * order gained 2 us, as many out of order lost 3.) */
-inline bool dir_layout(uint64_t n, uint32_t n_ctx, uint32_t S, char* buf, DirectArgs* a) {
+inline bool dir_layout(uint64_t n, uint32_t n_ctx, uint32_t S, int sms, char* buf, DirectArgs* a) {
   if (S > (uint32_t)kDirStages) return false;
-  const uint64_t tiles = (n + kDirTile - 1) / kDirTile, blocks = 148 * 4;
+  const uint64_t tiles = (n + kDirTile - 1) / kDirTile, blocks = 4ull * sms;
   a->piece = kDirTile * (uint32_t)std::min<uint64_t>(kDirMaxTiles, (tiles + blocks - 1) / blocks);
   a->n_pieces = (uint32_t)(n / a->piece) + n_ctx;     /* (contexts of more than 8,192 requests on average: 16 + 128 bytes for 1,792 of them) */
   a->piece_info = (uint4*)buf;

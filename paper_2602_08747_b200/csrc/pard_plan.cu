@@ -2922,7 +2922,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     pa.rounds = win_cnt; pa.tail = win_off; pa.tile_x = (uint32_t*)tile_carry;
     pa.out_keep = out->d_keep; pa.out_est = (long long*)out->d_est_us; pa.out_perm = out->d_perm;
     pa.out_kept_idx = out->d_kept_idx; pa.kept_base = kept_base; pa.seg_kept = seg_kept;
-    int wrc = launch_policy_walk(pa, stream);
+    int wrc = launch_policy_walk(pa, sms, stream);
     if (wrc != PARD_OK) return wrc;
     launch_pdl(k_kept_scan, 1, 1024, 0, stream, seg_kept, L.n_seg, kept_base, chunk_base, out->d_seg_kept,
                (unsigned long long*)out->d_n_kept);
@@ -3049,7 +3049,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
    * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
   DirectArgs da = {};
   const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN)) &&
-                      !state->d_priority && dir_layout(n, n_ctx, S, (char*)buf_b, &da);
+                      !state->d_priority && dir_layout(n, n_ctx, S, sms, (char*)buf_b, &da);
   da.req = req4; da.n = n32; da.n_ctx = n_ctx; da.S = S; da.sbits = sbits; da.ibits = ibits;
   da.ktab = ktab; da.ctx_start = ctx_start; da.const_bad = kept_tmp; da.stall = (mode & PARD_MODE_TEST_STALL) ? 1u : 0u;
 

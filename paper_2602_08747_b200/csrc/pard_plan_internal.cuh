@@ -486,7 +486,7 @@ struct PolicyArgs {
 };
 int allow_walk_smem();             /* once per device, by the planner's set-up */
 /* thresholds and walk: every queue's rounds and kept count (seg_kept) */
-int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream);
+int launch_policy_walk(const PolicyArgs& a, int sms, cudaStream_t stream);
 /* estimates, flags, order and survivors, once the output offsets are known */
 int launch_policy_emit(const PolicyArgs& a, cudaStream_t stream);
 

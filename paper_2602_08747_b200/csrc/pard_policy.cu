@@ -373,9 +373,9 @@ constexpr uint32_t kWalkShare = kWalkWarps * 32 * kWalkItems;           /* reque
 constexpr uint32_t kWalkClusterLong = 4 * kWalkCtas * kWalkShare;       /* shorter queues, and ... */
 constexpr uint32_t kWalkClusterCap = 4 * kWalkShare;                    /* ... queues of smaller rounds are walked by one block: a round costs */
 constexpr uint32_t kWalkClusterWindow = kWalkShare;                     /* two of the cluster's barriers; windows of Nexus seldom fill */
-constexpr uint32_t kWalkClusterQueues = 37;        /* most queues: as many clusters as two rounds of the device's blocks */
-constexpr uint32_t kWalkCopiesLong = 4 * kWalkShare;   /* from so many requests per queue on, and up to so many queues, one block's */
-constexpr uint32_t kWalkCopiesQueues = 148;        /* thresholds are copied ahead: the room leaves one block per multiprocessor instead of two */
+constexpr int kWalkClusterRounds = 2;              /* most queues: as many clusters as two rounds of the device's blocks (37) */
+constexpr uint32_t kWalkCopiesLong = 4 * kWalkShare;   /* from so many requests per queue on, and up to a queue per multiprocessor, one block's
+                                                      thresholds are copied ahead: the room leaves one block there instead of two */
 constexpr uint32_t kWalkSmallRound = 64;           /* rounds below this size are walked by one warp, 32 requests per step: a step
                                                       closes several of them, where a group needs a barrier for each */
 
@@ -897,18 +897,19 @@ static bool cluster_walk_fits() {
   return false;
 }
 
-int launch_policy_walk(const PolicyArgs& a, cudaStream_t stream) {
+int launch_policy_walk(const PolicyArgs& a, int sms, cudaStream_t stream) {
   static_assert(kWalkItems < (int)kWalkSmallRound, "a window is longer than a thread's share of a step");
   static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
   launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
              tiles, kPolThreads, 0, stream, a);
   PARD_CUDA_OK(cudaGetLastError());
-  if (a.n / a.n_seg >= kWalkClusterLong / 2 && a.n_seg <= kWalkClusterQueues && !(a.mode & PARD_MODE_SCAN) && cluster_walk_fits())
+  const uint32_t per = a.n / a.n_seg;
+  const bool copies = per >= kWalkCopiesLong && a.n_seg <= (uint32_t)sms;
+  if (per >= kWalkClusterLong / 2 && a.n_seg <= (uint32_t)(kWalkClusterRounds * sms / kWalkCtas) && !(a.mode & PARD_MODE_SCAN) && cluster_walk_fits())
     PARD_CUDA_OK(launch_pdl_cluster(k_policy_walk<kWalkWarps, kWalkCtas, true>, a.n_seg * kWalkCtas, kWalkWarps * 32, sizeof(FeedSmem), kWalkCtas, stream, a));
-  else if (a.n / a.n_seg >= kWalkLong)
-    launch_pdl(a.n / a.n_seg >= kWalkCopiesLong && a.n_seg <= kWalkCopiesQueues ? k_policy_walk<kWalkWarps, 1, true> : k_policy_walk<kWalkWarps, 1, false>,
-               a.n_seg, kWalkWarps * 32, a.n / a.n_seg >= kWalkCopiesLong && a.n_seg <= kWalkCopiesQueues ? sizeof(FeedSmem) : 0, stream, a);
+  else if (per >= kWalkLong)
+    launch_pdl(copies ? k_policy_walk<kWalkWarps, 1, true> : k_policy_walk<kWalkWarps, 1, false>, a.n_seg, kWalkWarps * 32, copies ? sizeof(FeedSmem) : 0, stream, a);
   else
     launch_pdl(k_policy_walk<1, 1, false>, (a.n_seg + kPolThreads / 32 - 1) / (kPolThreads / 32), kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
