@@ -36,13 +36,25 @@ def measured_peaks():
         return 6650.0, "fallback"
 
 
+#: everything that pard_plan.cu, whose kernels C3 runs, is compiled from
+TRAFFIC_SOURCES = ["include/pard.h"] + ["paper_2602_08747_b200/csrc/" + f for f in
+                                        ("pard_direct.cuh", "pard_internal.h", "pard_plan.cu", "pard_plan_internal.cuh")]
+
+
+def traffic_sha256():
+    import hashlib
+    h = hashlib.sha256()
+    for f in TRAFFIC_SOURCES:
+        with open(os.path.join(ROOT, f), "rb") as src:
+            h.update(src.read())
+    return h.hexdigest()
+
+
 def ncu_traffic(kernel):
     """DRAM bytes per launch of `kernel` from the committed ncu summary, or None
     when the kernel source has changed since the counters were taken."""
-    import hashlib
     try:
-        src = os.path.join(ROOT, "paper_2602_08747_b200", "csrc", "pard_plan.cu")
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()
+        sha = traffic_sha256()
         vals = {}
         for line in open(os.path.join(ROOT, "profiles", "dram_traffic_C3.txt")):
             if line.startswith("#") or not line.strip():
