@@ -186,7 +186,7 @@ typedef struct pard_plan_out {
                                    finished, which its next step waits for; a block of the path without
                                    a sort (PARD_MODE_GROUPED, in order) and of the rules' walk of a
                                    long queue never asks for the first copy it waits for; the waits run
-                                   out (after a fraction of a second) and the call returns
+                                   out (after about a second) and the call returns
                                    PARD_ETIMEOUT with unspecified outputs; the CUDA
                                    context stays usable.  Calls that the library sorts
                                    block by block (requests grouped by ctx, no ctx above

@@ -3044,9 +3044,11 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
 
   /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
-   * 288 k of 24 contexts 71 -> 51; out of order the try costs 7 of 567 us, 1 of 117
-   * (the passes behind it, their tiles on the way into L2 ahead of them, made up for it: 542 and 118).  Without the caller's
-   * word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
+   * 288 k of 24 contexts 71 -> 51.  Out of order the try costs 7 of 568 us, 2 of 71 (575 and 73; the tiles of the passes
+   * behind it on their way into L2 make that 544 and 74).  In order, but with a constant that the path does not take, 608 -> 609 and 70 -> 74.
+   * The path itself would take any stride up to 16 (12 stages: 243 us, by the general sort 434); but the kernels of that sort would have to look,
+   * ahead of their first loads, whether the plan is made, and every other call of theirs paid 0.7 us for it.  Without the
+   * caller's word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
   DirectArgs da = {};
   const bool direct = ctx_sort && !(mode & (PARD_MODE_RAW | PARD_MODE_SCAN)) &&
                       !state->d_priority && dir_layout(n, n_ctx, S, sms, (char*)buf_b, &da);
