@@ -416,6 +416,7 @@ k_seg_finish(const __grid_constant__ ConstArgs a, const unsigned long long* __re
  * directly.  Bound by the read of the requests: four in flight per thread at 48 registers keep
  * five blocks on a multiprocessor. */
 constexpr int kPreUn = 4;
+constexpr uint32_t kCountSegs = 256;             /* COUNT: most queues, one digit */
 
 __device__ __noinline__ void const_block(const ConstArgs& a, uint32_t c, PlanHeader* hdr) {
   __shared__ CtxScratch scratch;
@@ -429,12 +430,14 @@ __device__ __noinline__ void const_tail(const ConstArgs& a, const unsigned long 
 
 /* const_blocks: so many further blocks, the first ones of the grid, work out the queues' constants
  * meanwhile -- a chain of dependent loads that needs no deadline --, and the block that finishes last
- * completes them (one launch and its 8 us less for every call of up to 1,024 queues). */
-template <bool TABLE>
+ * completes them (one launch and its 8 us less for every call of up to 1,024 queues).
+ * COUNT: calls in arrival order, sorted by the queue id alone.  Their order needs no look at the deadlines, and the
+ * queues' lengths are all that the one pass wants, so they are counted here and k_pack is left out (k_sort_requests). */
+template <bool TABLE, bool COUNT>
 __global__ void __launch_bounds__(256, 5)
 k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
           unsigned long long* __restrict__ ctx_dmin_inv, unsigned long long* __restrict__ ctx_dmax,
-          PlanHeader* hdr, uint32_t const_blocks, const __grid_constant__ ConstArgs ca) {
+          PlanHeader* hdr, uint32_t const_blocks, const __grid_constant__ ConstArgs ca, uint32_t* __restrict__ hist) {
   pdl_wait();
   if (blockIdx.x < const_blocks) {
     const_block(ca, blockIdx.x, hdr);
@@ -452,7 +455,13 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
     for (uint32_t i = threadIdx.x; i < 2 * n_ctx; i += blockDim.x) s_range[i] = 0;
     __syncthreads();
   }
-  bool time_back = false, pair_back = false;     /* see PlanHeader; looked for until both have been met */
+  __shared__ uint32_t s_count[COUNT ? 8 : 1][COUNT ? kCountSegs : 1];
+  uint32_t* const count = s_count[COUNT ? threadIdx.x >> 5 : 0];
+  if (COUNT) {
+    for (uint32_t q = lane; q < kCountSegs; q += 32) count[q] = 0;
+    __syncwarp();
+  }
+  bool time_back = COUNT, pair_back = COUNT;     /* see PlanHeader; looked for until both have been met */
   uint32_t run_ctx = kNone;
   unsigned long long lmin = ~0ull, lmax = 0;
   bool bad_seen = false;
@@ -561,8 +570,10 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       const uint32_t ctx = r[i].z, stage = r[i].w & 0xffffu;
       if (D >= (unsigned long long)PARD_TIME_LIMIT_US || ctx >= n_ctx || stage >= S) {
         bad_seen = true;
+        if (COUNT) atomicAdd(&count[ctx < n_ctx && stage < S ? ctx * S + stage : 0u], 1u);   /* (request_element sorts it there) */
         continue;
       }
+      if (COUNT) atomicAdd(&count[ctx * S + stage], 1u);
       if (ctx != run_ctx) {
         flush();
         run_ctx = ctx;
@@ -616,8 +627,8 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       if (x < ~a) atomicMax(&ctx_dmin_inv[c], ~a);
       if (y < b) atomicMax(&ctx_dmax[c], b);
     }
-    if (lane == 30 && (back & 1u) && __ldcg(&hdr->time_steps_back) == 0) hdr->time_steps_back = 1;
-    if (lane == 31 && (back & 2u) && __ldcg(&hdr->pair_steps_back) == 0) hdr->pair_steps_back = 1;
+    if (!COUNT && lane == 30 && (back & 1u) && __ldcg(&hdr->time_steps_back) == 0) hdr->time_steps_back = 1;
+    if (!COUNT && lane == 31 && (back & 2u) && __ldcg(&hdr->pair_steps_back) == 0) hdr->pair_steps_back = 1;
   }
   if (TABLE) {
     __syncthreads();
@@ -628,19 +639,25 @@ k_prepass(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       if (__ldcg(&ctx_dmax[c]) < hi) atomicMax(&ctx_dmax[c], hi);
     }
   }
+  if (COUNT)
+    for (uint32_t q = threadIdx.x; q < n_ctx * S; q += 256) {
+      uint32_t sum = 0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) sum += s_count[COUNT ? w : 0][q];
+      if (sum) atomicAdd(&hist[q], sum);
+    }
   if (const_blocks) const_tail(ca, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
 constexpr uint32_t kPreTableCtx = 4096;          /* 32 KB of table: five blocks still fit a multiprocessor */
 void launch_prepass(const uint4* req, uint32_t n, uint32_t n_ctx, uint32_t S, unsigned long long* ctx_dmin_inv,
                     unsigned long long* ctx_dmax, PlanHeader* hdr, uint32_t const_blocks, const ConstArgs& ca, int sms,
-                    cudaStream_t stream) {
+                    cudaStream_t stream, uint32_t* count = nullptr) {
   const uint32_t grid = std::min<uint32_t>((n + 256 * kPreUn - 1) / (256 * kPreUn), (uint32_t)sms * 5);
   /* the table pays once a block has more requests than the table has entries to clear and hand over */
-  if (n_ctx > 1 && n_ctx <= kPreTableCtx && n / grid >= 2 * n_ctx)
-    launch_pdl(k_prepass<true>, const_blocks + grid, 256, 8ull * n_ctx, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
-  else
-    launch_pdl(k_prepass<false>, const_blocks + grid, 256, 0, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca);
+  const bool table = n_ctx > 1 && n_ctx <= kPreTableCtx && n / grid >= 2 * n_ctx;
+  launch_pdl(table ? (count ? k_prepass<true, true> : k_prepass<true, false>) : (count ? k_prepass<false, true> : k_prepass<false, false>),
+             const_blocks + grid, 256, table ? 8ull * n_ctx : 0ull, stream, req, n, n_ctx, S, ctx_dmin_inv, ctx_dmax, hdr, const_blocks, ca, count);
 }
 
 __global__ void k_ctx_span(const unsigned long long* __restrict__ ctx_dmin_inv,
@@ -1063,6 +1080,8 @@ __device__ bool finish_pieces(PlanHeader* hdr, uint32_t* word, uint32_t mine, ui
   return s_ok != 0;
 }
 
+constexpr int kItemsReq = (kItemsLo + kItemsHi) / 2;     /* k_sort_requests: its loads take the registers of the longer shares (10 and 22: 200 bytes spilled) */
+
 struct SortSmem {
   unsigned long long keys[kSortTile];
   uint32_t slot[kSortThreads / 32][kBins];    /* counts, then next free tile-local slot per (warp, digit) */
@@ -1076,17 +1095,64 @@ struct SortSmem {
   uint32_t ctx, lo_tile, base, limit, first;   /* the tile's ctx and range when passes stay inside the contexts */
 };
 
+/* A pass that takes the requests themselves instead of elements (k_sort_requests), and, for the rules that look no
+ * further than the deadline, what k_policy_terms would write beside them. */
+struct RequestPass {
+  const uint4* req;
+  const unsigned long long* ctx_dmin_inv;
+  uint32_t n_ctx, S, nexus;
+  const PardSegConst* ktab;
+  uint32_t* rounds;                                    /* [n] rounds that a request still fits, or null */
+};
+/* k_pack's element of a request, low budget first; cmin: its ctx's smallest deadline */
+__device__ __forceinline__ unsigned long long request_element(const RequestPass& rp, const uint4& r, uint32_t j, uint32_t dbits, uint32_t ibits,
+                                                              unsigned long long cmin, bool plain) {
+  const uint32_t ctx = r.z, stage = r.w & 0xffffu;
+  if (plain) {                                         /* the key fits one word, deadline offsets 31 bits */
+    const uint32_t key = (ctx * rp.S + stage) << dbits | ((r.x - (uint32_t)cmin) & ((1u << dbits) - 1));
+    return (unsigned long long)(ctx < rp.n_ctx && stage < rp.S ? key : 0u) * (1u << ibits) + j;
+  }
+  const unsigned long long off = ((((unsigned long long)r.y << 32) | r.x) - cmin) & ((1ull << dbits) - 1);   /* dbits < 64: see set_key_width */
+  const unsigned long long e = ((unsigned long long)(ctx * rp.S + stage) << dbits | off) << ibits;
+  return (ctx < rp.n_ctx && stage < rp.S ? e : 0ull) | j;
+}
+
 /* one warp's share of step 1: ITEMS rounds of 32 consecutive elements */
 template <int ITEMS, bool L2, int CAP>
-__device__ __forceinline__ void sort_load_count(unsigned long long (&key)[CAP], const unsigned long long* src,
-                                                uint64_t first, uint32_t n, uint32_t shift, uint32_t* slot_row,
-                                                uint32_t lane, uint32_t dig_mask, int items) {
+__device__ __forceinline__ void sort_load(unsigned long long (&key)[CAP], const unsigned long long* src, uint64_t first, uint32_t n,
+                                          uint32_t lane, int items) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     if (i >= items) break;                             /* the same for the whole warp */
     const uint64_t j = first + i * 32 + lane;
     key[i] = j < n ? (L2 ? __ldcg(src + j) : src[j]) : ~0ull;
   }
+}
+template <int ITEMS, int CAP>
+__device__ __forceinline__ void sort_load_requests(unsigned long long (&key)[CAP], const RequestPass& rp, uint64_t first, uint32_t n,
+                                                   uint32_t dbits, uint32_t ibits, uint32_t lane, int items, bool plain) {
+  constexpr int kUn = 4;                               /* requests under way together */
+  const bool one = rp.n_ctx == 1;
+  const unsigned long long only = ~__ldg(&rp.ctx_dmin_inv[0]);
+#pragma unroll
+  for (int i0 = 0; i0 < ITEMS; i0 += kUn) {
+    if (i0 >= items) break;                            /* the same for the whole warp */
+    uint4 r[kUn];
+    unsigned long long cmin[kUn];
+#pragma unroll
+    for (int u = 0; u < kUn; ++u) r[u] = __ldg(&rp.req[min(first + (i0 + u) * 32 + lane, (uint64_t)n - 1)]);
+#pragma unroll
+    for (int u = 0; u < kUn; ++u) cmin[u] = one ? only : ~__ldg(&rp.ctx_dmin_inv[min(r[u].z, rp.n_ctx - 1)]);
+#pragma unroll
+    for (int u = 0; u < kUn; ++u) {
+      if (i0 + u >= ITEMS) break;
+      const uint64_t j = first + (i0 + u) * 32 + lane;
+      key[i0 + u] = j < n ? request_element(rp, r[u], (uint32_t)j, dbits, ibits, cmin[u], plain) : ~0ull;
+    }
+  }
+}
+template <int ITEMS, int CAP>
+__device__ __forceinline__ void sort_count(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t* slot_row, uint32_t dig_mask, int items) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     if (i >= items) break;
@@ -1127,12 +1193,8 @@ __device__ __forceinline__ void sort_rank_drop(const unsigned long long (&key)[C
  * traffic (16.2 us against 14.5 us at 2^20 elements), so wider digits stay on the generic code.
  * The 89 us are what a pass costs with ranking almost free: tile load, write-out, scans and
  * barriers.  Full tiles only (no padding keys). */
-template <int ITEMS, int BITS, bool L2, int CAP>
-__device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[CAP], const unsigned long long* src,
-                                                    uint64_t first, uint32_t shift, uint32_t* slot_row, uint32_t lane, int items) {
-#pragma unroll
-  for (int i = 0; i < ITEMS; ++i)
-    if (i < items) key[i] = L2 ? __ldcg(src + first + i * 32 + lane) : src[first + i * 32 + lane];
+template <int ITEMS, int BITS, int CAP>
+__device__ __forceinline__ void sort_count_few(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t* slot_row, uint32_t lane, int items) {
   uint32_t mine = 0;                                     /* lane j: keys of this warp with digit j */
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
@@ -1166,12 +1228,11 @@ __device__ __forceinline__ void sort_rank_drop_few(const unsigned long long (&ke
 }
 
 /* digit width known at run time only: one instantiation per width */
-template <int ITEMS, bool L2, int CAP>
-__device__ __forceinline__ void sort_load_count_few_n(unsigned long long (&key)[CAP], const unsigned long long* src,
-                                                      uint64_t first, uint32_t shift, uint32_t bits, uint32_t* slot_row,
-                                                      uint32_t lane, int items) {
-  if (bits == 1) sort_load_count_few<ITEMS, 1, L2>(key, src, first, shift, slot_row, lane, items);
-  else sort_load_count_few<ITEMS, 2, L2>(key, src, first, shift, slot_row, lane, items);
+template <int ITEMS, int CAP>
+__device__ __forceinline__ void sort_count_few_n(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t bits, uint32_t* slot_row,
+                                                 uint32_t lane, int items) {
+  if (bits == 1) sort_count_few<ITEMS, 1>(key, shift, slot_row, lane, items);
+  else sort_count_few<ITEMS, 2>(key, shift, slot_row, lane, items);
 }
 template <int ITEMS, int CAP>
 __device__ __forceinline__ void sort_rank_drop_few_n(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t bits,
@@ -1193,13 +1254,13 @@ struct CtxTiles {
 
 /* PERSIST: the block takes tile after tile, and the elements may have been written by other blocks
  * of the same kernel (they are read from L2).  False: given up, a bounded wait ran out. */
-template <bool PERSIST, bool CTX, bool SMALL>
+template <bool PERSIST, bool CTX, bool SMALL, bool REQ = false>
 __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf_a,
             unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ hist,
             uint32_t* __restrict__ lookback, uint32_t* __restrict__ lookback_next, uint32_t n,
-            uint32_t ibits, uint32_t stall, const CtxTiles& ct, uint32_t geometry) {
+            uint32_t ibits, uint32_t stall, const CtxTiles& ct, uint32_t geometry, const RequestPass& rp = RequestPass{}) {
   constexpr int WARPS = kSortThreads / 32;
-  constexpr int kLo = SMALL ? kSmallLo : kItemsLo, kHi = SMALL ? kSmallHi : kItemsHi;     /* at most so many rounds per warp */
+  constexpr int kLo = SMALL ? kSmallLo : REQ ? kItemsReq : kItemsLo, kHi = SMALL ? kSmallHi : REQ ? kItemsReq : kItemsHi;     /* at most so many rounds per warp */
   const int items_lo = SMALL ? (int)(geometry & 255u) : kLo, items_hi = SMALL ? (int)(geometry >> 8) : kHi;
   const uint32_t tile_size = 256u * (uint32_t)(items_lo + items_hi);
   static_assert(kLoWarps * 32 == kBins, "one look-back thread per digit");
@@ -1242,7 +1303,9 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
   if (CTX && S.ctx == 0xffffffffu) return true;
   if (CTX && tid < kBins) gh = ct.hist[((size_t)S.ctx * kMaxPasses + pass) * kBins + tid];
   const uint64_t base = CTX ? (uint64_t)S.base : (uint64_t)tile * tile_size;
-  if (!PERSIST && !CTX && tid == 0) l2_ahead(src, base, (uint64_t)kSortAhead * tile_size, tile_size, n);
+  if (REQ && !PERSIST && tid == 0)
+    l2_ahead(reinterpret_cast<const unsigned long long*>(rp.req), 2 * base, 2ull * kSortAhead * tile_size, 2 * tile_size, 2ull * n);
+  if (!REQ && !PERSIST && !CTX && tid == 0) l2_ahead(src, base, (uint64_t)kSortAhead * tile_size, tile_size, n);
   const uint32_t limit = CTX ? S.limit : n;            /* end of the range the tile belongs to */
   const int64_t lo_tile = CTX ? (int64_t)S.lo_tile : 0;
   const uint32_t shift = ibits + hdr->pshift + 8 * pass;
@@ -1259,11 +1322,20 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
    * and take no part in the digit */
   const uint32_t dig_mask = CTX ? (1u << dig_bits) - 1 : 255u;
   const bool few = dig_bits <= 2 && base + tile_size <= (uint64_t)limit;
+  if constexpr (REQ) {
+    const uint32_t dbits = hdr->dbits;
+    const bool plain = dbits < 32 && hdr->keybits + hdr->pshift <= 32;
+    if (lo_warp) sort_load_requests<kLo>(key, rp, base + wfirst, limit, dbits, ibits, lane, items_lo, plain);
+    else sort_load_requests<kHi>(key, rp, base + wfirst, limit, dbits, ibits, lane, items_hi, plain);
+  } else {
+    if (lo_warp) sort_load<kLo, PERSIST>(key, src, base + wfirst, limit, lane, items_lo);
+    else sort_load<kHi, PERSIST>(key, src, base + wfirst, limit, lane, items_hi);
+  }
   if (few) {
-    if (lo_warp) sort_load_count_few_n<kLo, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane, items_lo);
-    else sort_load_count_few_n<kHi, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane, items_hi);
-  } else if (lo_warp) sort_load_count<kLo, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask, items_lo);
-  else sort_load_count<kHi, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask, items_hi);
+    if (lo_warp) sort_count_few_n<kLo>(key, shift, dig_bits, S.slot[warp], lane, items_lo);
+    else sort_count_few_n<kHi>(key, shift, dig_bits, S.slot[warp], lane, items_hi);
+  } else if (lo_warp) sort_count<kLo>(key, shift, S.slot[warp], dig_mask, items_lo);
+  else sort_count<kHi>(key, shift, S.slot[warp], dig_mask, items_hi);
   __syncthreads();
 
   /* 2. thread d owns digit d */
@@ -1383,6 +1455,43 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
 
   /* 5. write out */
   const uint32_t nvalid = (uint32_t)min((uint64_t)tile_size, (uint64_t)limit - base);
+  if (REQ && rp.rounds) {
+    const uint32_t dbits = hdr->dbits, imask = (1u << ibits) - 1;
+    const unsigned long long dmask = (1ull << dbits) - 1;
+    const bool lookup = hdr->lookup != 0;
+    uint32_t* const out = reinterpret_cast<uint32_t*>(dst);
+    longlong2* con = reinterpret_cast<longlong2*>(&S.match[0][0]);   /* per queue, which is the digit: what its deadlines are compared with, 1 / d */
+    bool easy = dbits <= 29 && !lookup;                /* 32-bit arithmetic will do */
+    for (uint32_t q = tid; q < rp.n_ctx * rp.S; q += kSortThreads) {
+      const PardSegConst& K = rp.ktab[q];
+      const bool none = K.narrow & kSegNoStage;
+      const long long from = none ? 1ll << 62 : (lookup ? K.A : K.A_rel) - (rp.nexus ? K.lsub : 0ll);   /* Nexus: the current module only, base + d */
+      if (none && (q + 1 < kBins ? S.dstart[q + 1] : nvalid) > S.dstart[q]) set_status(hdr, PARD_EDATA);   /* (the tile has requests of the queue) */
+      con[q] = make_longlong2(from, (long long)K.d_magic);
+      easy = easy && (none || (K.d_magic != 0 && from > -(1ll << 30)));
+    }
+    if (__syncthreads_and(easy)) {
+#pragma unroll 4
+      for (uint32_t pos = tid; pos < nvalid; pos += kSortThreads) {
+        const unsigned long long k = S.keys[pos];
+        const uint32_t d = (uint32_t)(k >> shift) & 255u, at = S.gofs[d] + pos;
+        const longlong2 c = con[d];
+        const int32_t X = (int32_t)(__funnelshift_r((uint32_t)k, (uint32_t)(k >> 32), ibits) & (uint32_t)dmask) - (int32_t)min(c.x, 1ll << 30);
+        out[at] = (uint32_t)k & imask;
+        rp.rounds[at] = X < 0 ? 0u : div_magic32((uint32_t)X, (unsigned long long)c.y) + 1;   /* < 2^30: d >= 2 */
+      }
+    } else {
+      for (uint32_t pos = tid; pos < nvalid; pos += kSortThreads) {
+        const unsigned long long k = S.keys[pos];
+        const uint32_t d = (uint32_t)(k >> shift) & 255u, at = S.gofs[d] + pos, idx = (uint32_t)k & imask;
+        const longlong2 c = con[d];
+        const long long X = (long long)(lookup ? __ldg(reinterpret_cast<const unsigned long long*>(&rp.req[idx])) : (k >> ibits) & dmask) - c.x;
+        out[at] = idx;
+        rp.rounds[at] = rounds_fit(X, (unsigned long long)c.y, (unsigned long long)rp.ktab[d].d);
+      }
+    }
+    return true;
+  }
 #pragma unroll 4
   for (uint32_t pos = tid; pos < nvalid; pos += kSortThreads) {
     const unsigned long long k = S.keys[pos];
@@ -1416,6 +1525,23 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
   if ((CTX && hdr->direct) || pass >= hdr->npass || sort_is_local(hdr, local_candidate)) return;
   sort_tiles<false, CTX, false>(*reinterpret_cast<SortSmem*>(smem_raw), pass, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
                                 stall, ct, 0u);
+}
+
+/* The one pass of a call in arrival order with up to 256 queues, from the requests: their elements need not be written
+ * and read back first, and for the rules that compare the deadline alone (rp.rounds) the pass leaves what the walk and
+ * the outputs want, the index and the rounds, 8 bytes per request.  2^24 requests of 16 queues under the window scan:
+ * k_pack, the pass and k_policy_terms took 57 + 81 + 57 us, this takes 122 (470 MB: 72 by bytes), the call 402 -> 309.
+ * Bound by instructions (half of the issue slots, 150 per 32 requests) and by the pass's shared-memory atomics.
+ * Requests are loaded four at a time, ahead of any use: one by one 201 us. */
+template <bool SMALL>
+__global__ void __launch_bounds__(kSortThreads, 2)
+k_sort_requests(PlanHeader* hdr, unsigned long long* __restrict__ buf_a, unsigned long long* __restrict__ buf_b, const uint32_t* __restrict__ hist,
+                uint32_t* __restrict__ lookback, uint32_t* __restrict__ lookback_next, uint32_t n, uint32_t ibits, uint32_t stall,
+                uint32_t geometry, const __grid_constant__ RequestPass rp) {
+  pdl_wait();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  sort_tiles<false, false, SMALL, true>(*reinterpret_cast<SortSmem*>(smem_raw), 0u, hdr, buf_a, buf_b, hist, lookback, lookback_next, n, ibits,
+                                        stall, CtxTiles{}, geometry, rp);
 }
 
 /* All passes from `pass` on, by one grid.  How many passes a key needs is only known on the device, and a
@@ -2775,6 +2901,8 @@ int allow_sort_smem(int dev) {
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_rest<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_local, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_requests<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
+    PARD_CUDA_OK(cudaFuncSetAttribute(k_sort_requests<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortSmem)));
     int rc = allow_local_smem();
     if (rc == PARD_OK) rc = allow_walk_smem();
     if (rc != PARD_OK) return rc;
@@ -3075,6 +3203,9 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
    * they fit (queues of 32 requests on average); else blocks work them out again (stage_paths) */
   ca.path_sums = (mode & PARD_MODE_PATH_MASK) && n >= 2ull * kMaskPaths * L.n_seg ? (long long*)kept_tmp : nullptr;
   const bool const_fold = n > 0 && L.n_seg <= kFoldSegs && ca.with_key_width;
+  /* arrival order, a queue id of one digit: sorted straight from the requests (k_sort_requests) */
+  const bool from_requests = arrival_order && L.n_seg > 1 && L.n_seg <= kCountSegs && !local_cand && n > 0;
+  const bool with_rounds = from_requests && !(mode & (PARD_MODE_CLIPPER | PARD_MODE_PATH_MASK));
   if (direct) {
     const unsigned long long n16 = L.zero_end / 16;
     const uint32_t range_blocks = (n_ctx + kDirWarps - 1) / kDirWarps;
@@ -3084,7 +3215,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   mark();
   if (direct)
     launch_pdl(S > 8 ? k_dir_count<4> : k_dir_count<3>, da.n_pieces, kDirThreads, 0, stream, da, ca, hdr, ctx_dmin, ctx_dmax);
-  if (n > 0 && !direct) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_fold ? n_ctx : 0u, ca, sms, stream);
+  if (n > 0 && !direct) launch_prepass(req4, n32, n_ctx, S, ctx_dmin, ctx_dmax, hdr, const_fold ? n_ctx : 0u, ca, sms, stream, from_requests ? hist : nullptr);
   mark();
   if (!ca.with_key_width) {
     if (n > 0) launch_pdl(k_ctx_span, (n_ctx + 255) / 256, 256, 0, stream, ctx_dmin, ctx_dmax, n_ctx, hdr);
@@ -3112,6 +3243,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   if (ctx_sort) {
     launch_pdl(k_pack_ctx, L.ctx_tiles, 256, 0, stream, req4, S, ctx_dmin, ctx_dmax, state->d_priority, ibits, hdr, buf_a,
                (uint32_t*)(ws + L.hist_ctx), ctx_tiles);
+  } else if (from_requests) {
+    /* (by the sort below) */
   } else if (n > 0 && !local_sure) {             /* returns at once when the blocks above did the work */
     /* every block adds its digit counts to the call's, up to 256 additions per pass: the fewer blocks the
      * better, down to two per multiprocessor and up to the four that are resident (a million requests with 1,184
@@ -3140,7 +3273,11 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   for (uint32_t p = 0; p < (uint32_t)kMaxPasses; ++p) {
     mark();
     if (n == 0 || local_sure || p >= max_passes) continue;
-    if (p < own_passes)
+    if (from_requests) {                                   /* (one pass: max_passes is 1) */
+      const RequestPass rp = {req4, ctx_dmin, n_ctx, S, (mode & PARD_MODE_NEXUS) ? 1u : 0u, ktab, with_rounds ? (uint32_t*)buf_a : nullptr};
+      launch_pdl(small ? k_sort_requests<true> : k_sort_requests<false>, sort_tiles, kSortThreads, sizeof(SortSmem), stream, hdr, buf_a, buf_b,
+                 (const uint32_t*)hist, lookback, lookback + lb_words, n32, ibits, stall, L.geometry, rp);
+    } else if (p < own_passes)
       launch_pdl(ctx_sort ? k_sort_pass<true> : k_sort_pass<false>, sort_tiles + wc.on, kSortThreads, sizeof(SortSmem), stream, p, hdr, buf_a,
                  buf_b, hist, lookback + (p & 1) * lb_words, lookback + ((p + 1) & 1) * lb_words, n32, ibits, p == 0 ? stall : 0u,
                  local_cand, ctx_tiles, wc);
@@ -3162,6 +3299,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     pa.n = n32; pa.ibits = ibits; pa.n_seg = L.n_seg; pa.mode = mode;
     pa.ktab = ktab; pa.seg_off = seg_off; pa.req = req4; pa.arrivals = d_arrivals;
     pa.pipes = pipe_table; pa.n_pipelines = n_pipelines; pa.st = *state; pa.path_sums = ca.path_sums;
+    pa.rounds_there = with_rounds ? 1u : 0u;
     mark();
     rc = decide_by_walk(pa);
     if (rc != PARD_OK) return rc;

@@ -289,6 +289,15 @@ __device__ __forceinline__ uint32_t threshold_u(int64_t X, const PardSegConst& K
   return u > kUClamp ? kUClamp : (uint32_t)u;
 }
 
+/* number of batch rounds b for which a request still fits, b < v: Nexus tests "base + b*d + d <= D" */
+__device__ __forceinline__ uint32_t rounds_fit(long long X, unsigned long long magic, unsigned long long d) {
+  if (X < 0) return 0;
+  unsigned long long q;
+  if (((unsigned long long)X >> 32) == 0 && magic) q = div_magic32((uint32_t)X, magic);
+  else q = (unsigned long long)X / d;
+  return q >= kUClamp ? kUClamp : (uint32_t)q + 1;
+}
+
 /* X = deadline - A of a request from its deadline offset: offsets of a queue served high
  * budget first count down from the ctx's largest deadline, and A_rel is that deadline - A */
 __device__ __forceinline__ long long slack_of(unsigned long long off, const PardSegConst& K) {
@@ -474,6 +483,7 @@ struct PolicyArgs {
   uint32_t n_pipelines;
   pard_queue_state_t st;
   uint32_t* rounds;               /* [n_seg] batch rounds the walk has closed */
+  uint32_t rounds_there;          /* the sort has written every request's rounds (k_sort_requests) */
   uint32_t* tail;                 /* [n_seg] Nexus: requests of the last, partly filled window */
   uint32_t* tile_x;               /* [tiles of kDecTile] kept requests ahead of the tile's first one, in its queue */
   uint8_t* out_keep;

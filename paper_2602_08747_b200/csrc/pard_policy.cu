@@ -14,7 +14,8 @@
  * is therefore a chain of rounds, not of requests: in round b, count the requests with v_r > b
  * until there are cap of them, which any number of threads can do side by side.  Nexus' scan has
  * the same shape (find the first cap consecutive requests with v_r > b).
- *   k_policy_terms   every request on its own: v_r                                -> T[n]
+ *   k_policy_terms   every request on its own: v_r                                -> T[n]; calls in arrival order
+ *                    that look no further than the deadline have it from their sort (k_sort_requests)
  *   k_policy_walk    a group of threads per queue (16 requests each and step) closes round after
  *                    round; round b's end goes to C[first position of the queue + b]
  *   k_policy_emit    every request on its own again: its round by a search in the ends, estimate,
@@ -22,7 +23,7 @@
  * T and C live in the sort buffer that does not hold the elements.
  * Nexus on 16 queues of 2^20 requests: the walk takes 0.053 ms by clusters of eight blocks (0.080 by one block,
  * 0.093 without copies ahead) where one warp per queue, 32 requests per step, took 23.8 ms; a call of 2^24
- * requests 452 -> 402 us. */
+ * requests 452 -> 402 us, 309 since the sort takes the requests themselves and k_policy_emit eight in a row. */
 #include <type_traits>
 
 #include "pard_plan_internal.cuh"
@@ -132,11 +133,14 @@ __device__ __noinline__ long long masked_lsub(const PolicyArgs& a, const StagedP
   return best;
 }
 
-/* The same from the sums written down beside the queue's constants. */
+/* The same from the sums written down beside the queue's constants.  (A request mostly names one path or two: their
+ * loads do not wait for each other, nor those of several requests.) */
 __device__ __forceinline__ long long masked_lsub_at_hand(const PolicyArgs& a, uint32_t seg, uint32_t flags, long long lsub) {
   const long long* t = a.path_sums + (size_t)seg * kMaskPaths;
-  long long best = -1;
-  for (uint32_t m = flags; m; m &= m - 1) {
+  const uint32_t rest = flags & (flags - 1);
+  const long long one = __ldg(t + __ffs((int)flags) - 1), two = rest ? __ldg(t + __ffs((int)rest) - 1) : -1ll;
+  long long best = one > two ? one : two;
+  for (uint32_t m = rest & (rest - 1); m; m &= m - 1) {
     const long long v = __ldg(t + __ffs((int)m) - 1);
     best = v > best ? v : best;
   }
@@ -149,15 +153,6 @@ __device__ __forceinline__ long long masked_lsub_at_hand(const PolicyArgs& a, ui
  * by its mask, path sums worked out by the block; by its mask, path sums at hand.  (Working them out is
  * a chain of dependent loads per path and block: a million requests with known paths, 27 -> 14 us for the rounds and 32 -> 19 us for the estimates.) */
 enum { kAllPaths, kMaskStaged, kMaskAtHand };
-
-/* number of batch rounds b for which a request still fits, b < v: Nexus tests "base + b*d + d <= D" */
-__device__ __forceinline__ uint32_t rounds_fit(long long X, unsigned long long magic, const PardSegConst& K) {
-  if (X < 0) return 0;
-  unsigned long long q;
-  if (((unsigned long long)X >> 32) == 0 && magic) q = div_magic32((uint32_t)X, magic);
-  else q = (unsigned long long)X / (unsigned long long)K.d;
-  return q >= kUClamp ? kUClamp : (uint32_t)q + 1;
-}
 
 /* One request's rounds and, for PARD_MODE_PATH_MASK, its own downstream estimate.  What it takes from
  * the queue's constants stays in registers while a thread's requests are of one queue, which they
@@ -233,7 +228,7 @@ k_policy_terms(const __grid_constant__ PolicyArgs a) {
         }
       }
       if (MASK && flags[u]) X += K.lsub - (MASK == kMaskAtHand ? masked_lsub_at_hand(a, seg, flags[u], K.lsub) : masked_lsub(a, sp, seg, flags[u], K));
-      v.T[j] = rounds_fit(X, magic, K);
+      v.T[j] = rounds_fit(X, magic, (unsigned long long)K.d);
     }
   }
 }
@@ -717,52 +712,105 @@ k_policy_walk(const __grid_constant__ PolicyArgs a) {
   }
 }
 
-/* Estimates, decisions and survivors.  A request's round is the number of rounds of its queue that
- * ended at or before it, found by a search in the ends: a warp's 32-ary search for the warp's first
- * request, and from a round known to be close for all others -- a round takes at least a batch of
- * requests, so p positions on it is at most p / cap rounds on.  (A binary search over all of the
+/* Estimates, decisions and survivors, eight consecutive requests per thread.  A request's round is the number of rounds
+ * of its queue that ended at or before it, found by a search in the ends: a warp's 32-ary search for the warp's first
+ * request, from there a few steps for a thread's first one -- a round takes at least a batch of requests, so p positions
+ * on it is at most p / cap rounds on --, and one round after the other behind that.  (A binary search over all of the
  * queue's rounds for every 128th request was a chain of up to 120 dependent loads: 2^24 requests in
  * queues of 2^15 rounds, 130 us.)  Its place among the survivors is, for Nexus, given by its window, else the kept requests
- * ahead of it: those ahead of the tile (a.tile_x) and, by ballots, those inside it. */
-template <int MASK>
+ * ahead of it: those ahead of the tile (a.tile_x) and those inside it.  Survivors of a warp that sees one queue only
+ * follow one another and go out from shared memory, side by side.
+ * Bound by instructions: 2^24 requests under the window scan 90 us with every 128th request to a thread (119 instructions
+ * per request), 64 like this; 17 + 4f bytes each would take 45.
+ * INDEX: the sort left the requests' indexes alone (k_sort_requests); a queue is known by its positions. */
+template <int MASK, bool INDEX = false>
 __global__ void __launch_bounds__(kPolThreads, MASK == kMaskStaged ? 5 : 8)
 k_policy_emit(const __grid_constant__ PolicyArgs a) {
   pdl_wait();
-  constexpr int kWarps = kPolThreads / 32, kRows = kPolItems * kWarps;
-  static_assert(kRows == 32, "one warp scans the rows");
+  constexpr int kRows = kPolTile / 32;
+  static_assert(kRows == 32 && kPolItems == 8, "one warp scans the rows of 32; a thread's flags are one byte");
   __shared__ __align__(16) unsigned char sp_raw[MASK == kMaskStaged ? sizeof(StagedPaths) : 16];
   StagedPaths& sp = *reinterpret_cast<StagedPaths*>(sp_raw);
-  __shared__ uint32_t s_keep[kRows], s_before[kRows + 1];
+  __shared__ uint32_t s_keep[kRows], s_before[kRows];
   if (a.hdr->wide | a.hdr->aborted | a.hdr->walk_late) return;
   const SortedView v = sorted_view(a);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t tile0 = blockIdx.x * kPolTile;
-  const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW;
-  if (MASK == kAllPaths && threadIdx.x == 0) l2_ahead(v.src, tile0, (uint64_t)kDecAhead * kPolTile, kPolTile, a.n);   /* (the others have no registers left for it) */
+  const uint32_t tile0 = blockIdx.x * kPolTile, j0 = tile0 + threadIdx.x * kPolItems;
+  const bool nexus = a.mode & PARD_MODE_NEXUS, raw = a.mode & PARD_MODE_RAW, full = j0 + kPolItems <= a.n;
+  __shared__ uint32_t s_out[kPolThreads / 32][32 * kPolItems];
+  if (MASK == kAllPaths && threadIdx.x == 0)       /* (the others have no registers left for it) */
+    l2_ahead(v.src, INDEX ? tile0 / 2 : tile0, (uint64_t)kDecAhead * kPolTile / (INDEX ? 2 : 1), INDEX ? kPolTile / 2 : kPolTile, INDEX ? a.n / 2 : a.n);
   if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
-  unsigned long long e[kPolItems];
-  uint32_t t[kPolItems], round[kPolItems], flags[kPolItems];
+  uint32_t idx[kPolItems], t[kPolItems], my_seg = 0, last_seg = 0;
+  long long est[kPolItems];                        /* at first: by how much the paths that a request names take it from the queue's estimate */
 #pragma unroll
-  for (int i = 0; i < kPolItems; ++i) {
-    const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
-    e[i] = j < a.n ? v.src[j] : 0ull;
-    t[i] = j < a.n && !nexus ? v.T[j] : 0u;
-  }
-  if (MASK) {
+  for (int k = 0; k < kPolItems; ++k) est[k] = 0;
+  if (INDEX) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(v.src);
+    if (full) {
+      const uint4 x = *reinterpret_cast<const uint4*>(src + j0), y = *reinterpret_cast<const uint4*>(src + j0 + 4);
+      idx[0] = x.x; idx[1] = x.y; idx[2] = x.z; idx[3] = x.w; idx[4] = y.x; idx[5] = y.y; idx[6] = y.z; idx[7] = y.w;
+    } else {
 #pragma unroll
-    for (int i = 0; i < kPolItems; ++i) {
-      const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
-      flags[i] = j < a.n ? __ldg(&reinterpret_cast<const uint32_t*>(&a.req[(uint32_t)e[i] & v.imask])[3]) >> 16 : 0u;
+      for (int i = 0; i < kPolItems; ++i) idx[i] = j0 + i < a.n ? src[j0 + i] : 0u;
+    }
+  } else {
+    unsigned long long e[kPolItems];
+    if (full) {
+      load4(v.src + j0, e);
+      load4(v.src + j0 + 4, e + 4);
+    } else {
+#pragma unroll
+      for (int i = 0; i < kPolItems; ++i) e[i] = j0 + i < a.n ? v.src[j0 + i] : 0ull;
+    }
+#pragma unroll
+    for (int i = 0; i < kPolItems; ++i) idx[i] = (uint32_t)e[i] & v.imask;
+    my_seg = (uint32_t)(e[0] >> v.kshift);
+    last_seg = (uint32_t)(e[kPolItems - 1] >> v.kshift);
+    if (MASK) {
+      uint32_t flags[kPolItems];
+#pragma unroll
+      for (int k = 0; k < kPolItems; ++k) flags[k] = j0 + k < a.n ? __ldg(&reinterpret_cast<const uint32_t*>(&a.req[idx[k]])[3]) >> 16 : 0u;
+#pragma unroll
+      for (int k = 0; k < kPolItems; ++k)
+        if (flags[k]) {
+          const uint32_t seg = (uint32_t)(e[k] >> v.kshift);
+          const PardSegConst& K = a.ktab[seg];
+          if (!(K.narrow & kSegNoStage)) est[k] = (MASK == kMaskAtHand ? masked_lsub_at_hand(a, seg, flags[k], K.lsub) : masked_lsub(a, sp, seg, flags[k], K)) - K.lsub;
+        }
     }
   }
-  uint32_t cur = 0xffffffffu, lo = 0, hi = 0, nb = 0, b = 0, end = 0, cap = 0, tail = 0, keepbits = 0, at_once = 0;
-  bool none = false;
-  /* the round of the warp's first request, for a warp whose first 32 requests are of one queue */
-  const uint32_t p0 = tile0 + warp * 32;
-  const uint32_t seg_first = __shfl_sync(0xffffffffu, (uint32_t)(e[0] >> v.kshift), 0);
-  const bool together = !raw && __all_sync(0xffffffffu, p0 + lane < a.n && (uint32_t)(e[0] >> v.kshift) == seg_first);
+  if (full && !nexus) {
+    const uint4 x = *reinterpret_cast<const uint4*>(v.T + j0), y = *reinterpret_cast<const uint4*>(v.T + j0 + 4);
+    t[0] = x.x; t[1] = x.y; t[2] = x.z; t[3] = x.w; t[4] = y.x; t[5] = y.y; t[6] = y.z; t[7] = y.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPolItems; ++i) t[i] = j0 + i < a.n && !nexus ? v.T[j0 + i] : 0u;
+  }
+  /* the round of the warp's first request */
+  const uint32_t p0 = tile0 + warp * (32 * kPolItems);
+  uint32_t seg_first = 0;
+  bool one_queue;                                  /* all of the warp's requests are there and of one queue */
+  if (INDEX) {                                     /* the queues that end at or before p0 come before it */
+    uint32_t before = 0;
+    for (uint32_t q = lane; q < a.n_seg; q += 32) before += a.seg_off[q + 1] <= p0 ? 1u : 0u;
+    seg_first = min(__reduce_add_sync(0xffffffffu, before), a.n_seg - 1);
+    one_queue = p0 + 32 * kPolItems <= min(a.seg_off[seg_first + 1], a.n);
+  } else {
+    seg_first = __shfl_sync(0xffffffffu, my_seg, 0);
+    one_queue = __all_sync(0xffffffffu, full && my_seg == seg_first && last_seg == seg_first);
+  }
+  /* the queue of position j, which is not before queue `from`: the last that begins at or before j */
+  auto queue_at = [&](uint32_t j, uint32_t from) {
+    uint32_t z = a.n_seg;
+    while (z - from > 1) {
+      const uint32_t mid = from + (z - from) / 2;
+      if (a.seg_off[mid] <= j) from = mid; else z = mid;
+    }
+    return from;
+  };
   uint32_t b0 = 0;
-  if (together) {
+  if (!raw && p0 < a.n) {
     const uint32_t* ends = v.C + a.seg_off[seg_first];
     uint32_t z = a.rounds[seg_first];
     while (b0 < z) {                               /* uniform across the warp */
@@ -775,48 +823,112 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
       if (c < 32) z = p_at;
     }
   }
-#pragma unroll
-  for (int i = 0; i < kPolItems; ++i) {
-    const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
-    bool keep = false;
-    round[i] = 0;
-    if (j < a.n) {
-      const uint32_t seg = (uint32_t)(e[i] >> v.kshift);
-      bool look = false;
-      if (seg != cur) {
-        cur = seg;
-        lo = a.seg_off[seg];
-        hi = a.seg_off[seg + 1];
-        nb = raw ? 0u : a.rounds[seg];
-        cap = a.ktab[seg].cap;
-        none = a.ktab[seg].narrow & kSegNoStage;
-        tail = nexus ? a.tail[seg] : 0u;
-        b = 0;
-        at_once = cap ? kPolThreads / cap + 1 : kPolThreads;
-        look = true;
-      }
-      if (raw) {
-        const unsigned long long magic = a.ktab[seg].cap_magic;
-        b = magic ? div_magic32(j - lo, magic) : j - lo;
-      } else if (look || j >= end) {               /* (b < nb and the round goes on: nothing to search) */
-        uint32_t z = nb;                           /* ends b .. nb-1: how many are <= j */
-        if (!look) z = min(nb, b + at_once);       /* kPolThreads positions on from a request of round b */
-        else if (i == 0 && together) { b = b0; z = min(nb, b0 + 31u / max(cap, 1u) + 1); }
+  /* span after span of requests of one queue and round: mostly the thread's eight are one */
+  uint32_t lo = 0, hi = 0, nb = 0, b = 0, cap = 0, tail = 0, place = 0, keepbits = 0, at = 0;
+  long long A0 = 0, d = 0;
+  bool none = false;
+  const uint32_t count = j0 < a.n ? min(a.n - j0, (uint32_t)kPolItems) : 0u;
+  for (uint32_t i = 0; i < count;) {
+    const uint32_t j = j0 + i;
+    if (j >= hi) {                                 /* a queue begins, or the thread's share does */
+      if (INDEX || i > 0) my_seg = one_queue ? seg_first : queue_at(j, i > 0 ? my_seg : seg_first);
+      const PardSegConst& K = a.ktab[my_seg];
+      lo = a.seg_off[my_seg];
+      hi = a.seg_off[my_seg + 1];
+      nb = raw ? 0u : a.rounds[my_seg];
+      cap = K.cap;
+      none = K.narrow & kSegNoStage;
+      tail = nexus ? a.tail[my_seg] : 0u;
+      A0 = K.A;
+      d = none ? 0 : K.d;
+      if (!none && (a.mode & (PARD_MODE_NEXUS | PARD_MODE_CLIPPER))) A0 -= K.lsub;     /* the current module only */
+      if (nexus && a.out_kept_idx) place = a.kept_base[my_seg];
+      b = 0;                                       /* (a queue that begins inside the thread's share: its first round) */
+      if (i == 0 && !raw) {
+        uint32_t z = nb;                           /* ends b .. z-1: how many are <= j */
+        if (my_seg == seg_first) { b = b0; z = min(nb, b0 + (j - p0) / max(cap, 1u) + 1); }
         while (b < z) {
           const uint32_t mid = b + (z - b) / 2;
           if (v.C[lo + mid] <= j) b = mid + 1; else z = mid;
         }
-        end = b < nb ? v.C[lo + b] : 0xffffffffu;
       }
-      if (nexus) keep = b < nb ? j + cap >= end : j + tail >= hi;
-      else keep = t[i] > b;
-      keep = keep && !none;
-      round[i] = b;
+    } else {
+      ++b;                                         /* (no round is empty) */
     }
-    const uint32_t m = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) s_keep[i * kWarps + warp] = m;
-    keepbits |= (keep ? 1u : 0u) << i;
+    uint32_t end = b < nb ? v.C[lo + b] : 0xffffffffu, stop = min(min(end, hi) - j0, count);
+    if (raw) {
+      const unsigned long long magic = a.ktab[my_seg].cap_magic;
+      b = magic ? div_magic32(j - lo, magic) : j - lo;
+      stop = i + 1;
+    }
+    const long long now = A0 + (long long)b * d;
+    const uint32_t from = b < nb ? end - cap : hi - tail;      /* Nexus: the window's first request */
+    uint32_t kept = 0;
+    if (!nexus) {
+#pragma unroll
+      for (int k = 0; k < kPolItems; ++k) kept |= (t[k] > b ? 1u : 0u) << k;
+    } else {
+      kept = from <= j0 ? 255u : 255u << min(from - j0, 8u);
+    }
+    const uint32_t span = (1u << stop) - (1u << i);
+    kept = none ? 0u : kept & span;
+#pragma unroll
+    for (int k = 0; k < kPolItems; ++k) est[k] += (span >> k) & 1u ? now : 0ll;
+    if (nexus && kept && a.out_kept_idx) {
+      const uint32_t to = place + b * cap + (j0 - from);       /* of the thread's request 0, were it of this window */
+      if (!one_queue) {
+#pragma unroll
+        for (int k = 0; k < kPolItems; ++k)
+          if ((kept >> k) & 1u) a.out_kept_idx[to + k] = idx[k];
+      } else if (!keepbits) {
+        at = to + (uint32_t)__ffs((int)kept) - 1;  /* the thread's first */
+      }
+    }
+    keepbits |= kept;
+    i = stop;
   }
+  if (full) {
+    if (a.out_keep) *reinterpret_cast<uint2*>(a.out_keep + j0) = make_uint2(((keepbits & 15u) * 0x00204081u) & 0x01010101u, ((keepbits >> 4) * 0x00204081u) & 0x01010101u);
+    if (a.out_est) {
+      store4(a.out_est + j0, est[0], est[1], est[2], est[3]);
+      store4(a.out_est + j0 + 4, est[4], est[5], est[6], est[7]);
+    }
+    if (a.out_perm) {
+      auto two = [&](int i) { return idx[i] | (unsigned long long)idx[i + 1] << 32; };
+      store4(a.out_perm + j0, two(0), two(2), two(4), two(6));
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPolItems; ++i)
+      if (j0 + i < a.n) {
+        if (a.out_keep) a.out_keep[j0 + i] = (keepbits >> i) & 1u;
+        if (a.out_est) a.out_est[j0 + i] = est[i];
+        if (a.out_perm) a.out_perm[j0 + i] = idx[i];
+      }
+  }
+  if (!a.out_kept_idx) return;
+  /* a warp's survivors, to be written from position `to` of the output on */
+  auto write_out = [&](uint32_t rank, uint32_t total, uint32_t to) {
+    uint32_t* out = s_out[warp];
+#pragma unroll
+    for (int i = 0; i < kPolItems; ++i)
+      if ((keepbits >> i) & 1u) out[rank + __popc(keepbits & ((1u << i) - 1))] = idx[i];
+    __syncwarp();
+    for (uint32_t k = lane; k < total; k += 32) a.out_kept_idx[to + k] = out[k];
+  };
+  if (nexus) {
+    if (!one_queue) return;
+    uint32_t rank = __popc(keepbits);
+    const uint32_t mine = rank, any = __ballot_sync(0xffffffffu, mine != 0);
+    if (!any) return;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, rank, o);
+      if (lane >= (uint32_t)o) rank += y;
+    }
+    write_out(rank - mine, __shfl_sync(0xffffffffu, rank, 31), __shfl_sync(0xffffffffu, at, __ffs((int)any) - 1));
+    return;
+  }
+  reinterpret_cast<uint8_t*>(s_keep)[threadIdx.x] = (uint8_t)keepbits;
   __syncthreads();
   if (warp == 0) {
     const uint32_t x = __popc(s_keep[lane]);
@@ -830,40 +942,28 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   __syncthreads();
   /* kept requests of the tile ahead of its position p */
   auto kept_before = [&](uint32_t p) { return s_before[p >> 5] + __popc(s_keep[p >> 5] & ((1u << (p & 31)) - 1)); };
-  uint32_t last = 0xffffffffu, first = 0, place = 0, window = 0;
-  long long A0 = 0, d = 0;
+  uint32_t c = kept_before(threadIdx.x * kPolItems);
+  /* output position of the queue's survivors, less those of the tile ahead of its first */
+  auto place_of = [&](uint32_t seg) {
+    const uint32_t first = a.seg_off[seg];
+    return a.kept_base[seg] + (first <= tile0 ? a.tile_x[blockIdx.x] : 0u - kept_before(first - tile0));
+  };
+  if (one_queue) {
+    const uint32_t c0 = __shfl_sync(0xffffffffu, c, 0);
+    write_out(c - c0, __shfl_sync(0xffffffffu, c + __popc(keepbits), 31) - c0, place_of(seg_first) + c0);
+    return;
+  }
+  uint32_t behind = 0;                             /* end of the queue at hand */
 #pragma unroll
   for (int i = 0; i < kPolItems; ++i) {
-    const uint32_t j = tile0 + i * kPolThreads + threadIdx.x;
-    if (j >= a.n) break;
-    const uint32_t seg = (uint32_t)(e[i] >> v.kshift), idx = (uint32_t)e[i] & v.imask;
-    if (seg != last) {
-      last = seg;
-      const PardSegConst& K = a.ktab[seg];
-      first = a.seg_off[seg];
-      A0 = K.A;
-      d = K.d;
-      window = K.cap;
-      if (a.mode & (PARD_MODE_NEXUS | PARD_MODE_CLIPPER)) A0 -= K.lsub;     /* the current module only */
-      if (K.narrow & kSegNoStage) { A0 = K.A; d = 0; }
-      if (a.out_kept_idx) place = a.kept_base[seg];
+    if (!((keepbits >> i) & 1u)) continue;         /* (requests beyond the array are not kept) */
+    if (j0 + i >= behind) {
+      const uint32_t seg = queue_at(j0 + i, seg_first);
+      at = place_of(seg);
+      behind = a.seg_off[seg + 1];
     }
-    const uint32_t keep = (keepbits >> i) & 1u;
-    long long A = A0;
-    if (MASK && flags[i] && d) {
-      const PardSegConst& K = a.ktab[seg];
-      A += (MASK == kMaskAtHand ? masked_lsub_at_hand(a, seg, flags[i], K.lsub) : masked_lsub(a, sp, seg, flags[i], K)) - K.lsub;
-    }
-    if (a.out_keep) a.out_keep[j] = (uint8_t)keep;
-    if (a.out_est) a.out_est[j] = A + (long long)round[i] * d;
-    if (a.out_perm) a.out_perm[j] = idx;
-    if (keep && a.out_kept_idx) {
-      uint32_t c;
-      if (nexus) c = round[i] * window + (round[i] < a.rounds[seg] ? j + window - v.C[first + round[i]] : j + a.tail[seg] - a.seg_off[seg + 1]);
-      else if (first <= tile0) c = a.tile_x[blockIdx.x] + kept_before(j - tile0);
-      else c = kept_before(j - tile0) - kept_before(first - tile0);
-      a.out_kept_idx[place + c] = idx;
-    }
+    a.out_kept_idx[at + c] = idx[i];
+    ++c;
   }
 }
 
@@ -901,7 +1001,8 @@ int launch_policy_walk(const PolicyArgs& a, int sms, cudaStream_t stream) {
   static_assert(kWalkItems < (int)kWalkSmallRound, "a window is longer than a thread's share of a step");
   static_assert(kPolTile == kDecTile, "tile_x is indexed by the planner's decision tiles");
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
-  launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
+  if (!a.rounds_there)
+    launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_terms<kAllPaths> : a.path_sums ? k_policy_terms<kMaskAtHand> : k_policy_terms<kMaskStaged>,
              tiles, kPolThreads, 0, stream, a);
   PARD_CUDA_OK(cudaGetLastError());
   const uint32_t per = a.n / a.n_seg;
@@ -917,7 +1018,7 @@ int launch_policy_walk(const PolicyArgs& a, int sms, cudaStream_t stream) {
 
 int launch_policy_emit(const PolicyArgs& a, cudaStream_t stream) {
   const uint32_t tiles = (uint32_t)(((uint64_t)a.n + kPolTile - 1) / kPolTile);
-  launch_pdl(!(a.mode & PARD_MODE_PATH_MASK) ? k_policy_emit<kAllPaths> : a.path_sums ? k_policy_emit<kMaskAtHand> : k_policy_emit<kMaskStaged>,
+  launch_pdl(a.rounds_there ? k_policy_emit<kAllPaths, true> : !(a.mode & PARD_MODE_PATH_MASK) ? k_policy_emit<kAllPaths> : a.path_sums ? k_policy_emit<kMaskAtHand> : k_policy_emit<kMaskStaged>,
              tiles, kPolThreads, 0, stream, a);
   return cudaGetLastError() == cudaSuccess ? PARD_OK : PARD_ECUDA;
 }

@@ -53,6 +53,24 @@ def test_walk_rounds_against_steps_and_queue_lengths(rule, cap, n):
         check(inputs.Workload("edge", [p], util.requests(dl), st, 1), rule)
 
 
+# ---- arrival order, one pass straight from the requests: up to 256 queues -------------------------
+@pytest.mark.parametrize("rule", [FCFS, NEXUS, FCFS | pb.PARD_MODE_PATH_MASK])
+@pytest.mark.parametrize("queues", [2, 4, 5, 255, 256, 257])
+@pytest.mark.parametrize("n", [8193, 24_575, 24_576, 60_001])
+def test_arrival_order_from_the_requests(rule, queues, n):
+    sizes = np.bincount(np.random.default_rng(n).integers(0, queues, size=n), minlength=queues)
+    for S, far in ((1, 0), (1, 1 << 57)):                  # the last: offsets beyond the elements, looked up
+        wl = several_ctx(queues, sizes, S=S, sort=False, mix=True, m=1 + n % 3)
+        wl.requests["deadline_us"][::7] += far
+        check(wl, rule)
+
+
+@pytest.mark.parametrize("rule", [FCFS, NEXUS])
+@pytest.mark.parametrize("n", [2_727_936, 2_727_937])      # the last size of the small tiles, the first of the wide ones
+def test_arrival_order_from_the_requests_tiles(rule, n):
+    check(several_ctx(2, [n // 3, n - n // 3], sort=False, mix=True, m=700, span=60_000), rule)
+
+
 @pytest.mark.parametrize("sizes", [[5000, 0, 1, 4099], [200] * 40, [2100, 2048, 1]])
 @pytest.mark.parametrize("mode", [FCFS, NEXUS, pb.PARD_MODE_PATH_MASK])
 def test_walk_of_several_queues_with_heads_inside_tiles(sizes, mode):
