@@ -1119,15 +1119,22 @@ __device__ __forceinline__ unsigned long long request_element(const RequestPass&
 
 /* one warp's share of step 1: ITEMS rounds of 32 consecutive elements */
 template <int ITEMS, bool L2, int CAP>
-__device__ __forceinline__ void sort_load(unsigned long long (&key)[CAP], const unsigned long long* src, uint64_t first, uint32_t n,
-                                          uint32_t lane, int items) {
+__device__ __forceinline__ void sort_load_count(unsigned long long (&key)[CAP], const unsigned long long* src,
+                                                uint64_t first, uint32_t n, uint32_t shift, uint32_t* slot_row,
+                                                uint32_t lane, uint32_t dig_mask, int items) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     if (i >= items) break;                             /* the same for the whole warp */
     const uint64_t j = first + i * 32 + lane;
     key[i] = j < n ? (L2 ? __ldcg(src + j) : src[j]) : ~0ull;
   }
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    if (i >= items) break;
+    atomicAdd(&slot_row[(uint32_t)(key[i] >> shift) & dig_mask], 1u);
+  }
 }
+/* the same in two steps, from the requests */
 template <int ITEMS, int CAP>
 __device__ __forceinline__ void sort_load_requests(unsigned long long (&key)[CAP], const RequestPass& rp, uint64_t first, uint32_t n,
                                                    uint32_t dbits, uint32_t ibits, uint32_t lane, int items, bool plain) {
@@ -1193,6 +1200,25 @@ __device__ __forceinline__ void sort_rank_drop(const unsigned long long (&key)[C
  * traffic (16.2 us against 14.5 us at 2^20 elements), so wider digits stay on the generic code.
  * The 89 us are what a pass costs with ranking almost free: tile load, write-out, scans and
  * barriers.  Full tiles only (no padding keys). */
+template <int ITEMS, int BITS, bool L2, int CAP>
+__device__ __forceinline__ void sort_load_count_few(unsigned long long (&key)[CAP], const unsigned long long* src,
+                                                    uint64_t first, uint32_t shift, uint32_t* slot_row, uint32_t lane, int items) {
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i)
+    if (i < items) key[i] = L2 ? __ldcg(src + first + i * 32 + lane) : src[first + i * 32 + lane];
+  uint32_t mine = 0;                                     /* lane j: keys of this warp with digit j */
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    if (i >= items) break;
+    const uint32_t d = (uint32_t)(key[i] >> shift);
+    uint32_t bal[BITS];
+#pragma unroll
+    for (int k = 0; k < BITS; ++k) bal[k] = __ballot_sync(0xffffffffu, (d >> k) & 1u);
+    mine += __popc(digit_peers<BITS>(lane, bal));
+  }
+  if (lane < (1u << BITS)) slot_row[lane] = mine;
+}
+
 template <int ITEMS, int BITS, int CAP>
 __device__ __forceinline__ void sort_count_few(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t* slot_row, uint32_t lane, int items) {
   uint32_t mine = 0;                                     /* lane j: keys of this warp with digit j */
@@ -1228,6 +1254,13 @@ __device__ __forceinline__ void sort_rank_drop_few(const unsigned long long (&ke
 }
 
 /* digit width known at run time only: one instantiation per width */
+template <int ITEMS, bool L2, int CAP>
+__device__ __forceinline__ void sort_load_count_few_n(unsigned long long (&key)[CAP], const unsigned long long* src,
+                                                      uint64_t first, uint32_t shift, uint32_t bits, uint32_t* slot_row,
+                                                      uint32_t lane, int items) {
+  if (bits == 1) sort_load_count_few<ITEMS, 1, L2>(key, src, first, shift, slot_row, lane, items);
+  else sort_load_count_few<ITEMS, 2, L2>(key, src, first, shift, slot_row, lane, items);
+}
 template <int ITEMS, int CAP>
 __device__ __forceinline__ void sort_count_few_n(const unsigned long long (&key)[CAP], uint32_t shift, uint32_t bits, uint32_t* slot_row,
                                                  uint32_t lane, int items) {
@@ -1327,15 +1360,16 @@ __device__ __forceinline__ bool sort_tiles(SortSmem& S, uint32_t pass, PlanHeade
     const bool plain = dbits < 32 && hdr->keybits + hdr->pshift <= 32;
     if (lo_warp) sort_load_requests<kLo>(key, rp, base + wfirst, limit, dbits, ibits, lane, items_lo, plain);
     else sort_load_requests<kHi>(key, rp, base + wfirst, limit, dbits, ibits, lane, items_hi, plain);
-  } else {
-    if (lo_warp) sort_load<kLo, PERSIST>(key, src, base + wfirst, limit, lane, items_lo);
-    else sort_load<kHi, PERSIST>(key, src, base + wfirst, limit, lane, items_hi);
-  }
-  if (few) {
-    if (lo_warp) sort_count_few_n<kLo>(key, shift, dig_bits, S.slot[warp], lane, items_lo);
-    else sort_count_few_n<kHi>(key, shift, dig_bits, S.slot[warp], lane, items_hi);
-  } else if (lo_warp) sort_count<kLo>(key, shift, S.slot[warp], dig_mask, items_lo);
-  else sort_count<kHi>(key, shift, S.slot[warp], dig_mask, items_hi);
+    if (few) {
+      if (lo_warp) sort_count_few_n<kLo>(key, shift, dig_bits, S.slot[warp], lane, items_lo);
+      else sort_count_few_n<kHi>(key, shift, dig_bits, S.slot[warp], lane, items_hi);
+    } else if (lo_warp) sort_count<kLo>(key, shift, S.slot[warp], dig_mask, items_lo);
+    else sort_count<kHi>(key, shift, S.slot[warp], dig_mask, items_hi);
+  } else if (few) {
+    if (lo_warp) sort_load_count_few_n<kLo, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane, items_lo);
+    else sort_load_count_few_n<kHi, PERSIST>(key, src, base + wfirst, shift, dig_bits, S.slot[warp], lane, items_hi);
+  } else if (lo_warp) sort_load_count<kLo, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask, items_lo);
+  else sort_load_count<kHi, PERSIST>(key, src, base + wfirst, limit, shift, S.slot[warp], lane, dig_mask, items_hi);
   __syncthreads();
 
   /* 2. thread d owns digit d */
