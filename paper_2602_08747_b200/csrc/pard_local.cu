@@ -17,11 +17,11 @@
  * 16 bytes are read and 13 + 4f written per request and nothing else touches global memory.
  * Queues with more windows than the block's tables hold are decided by the segmented prefix-min
  * scan over the elements instead.
- * Bound by the chain of steps between barriers, two blocks per multiprocessor covering for each other:
- * of 385 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the copy bandwidth) 120 go to the
- * requests, 75 to the counting sort, 50 to the tables and 110 to the outputs.  The form before,
- * two segmented scans instead of tables, took 762 us there, three radix passes without a look at the
- * order 865. */
+ * Bound by instructions (half of the issue slots, integer ones at half rate) and the chain of steps between barriers, two
+ * blocks per multiprocessor covering for each other: of 303 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the
+ * copy bandwidth) 86 go to the requests, 74 to the counting sort, 30 to the tables, 90 to the outputs and 20 to the
+ * survivors.  Every request's window and position on its own, 32 in a row to a warp: 345; two segmented scans instead of
+ * tables took 762, three radix passes without a look at the order 865. */
 #include <cstddef>
 
 #include "pard_plan_internal.cuh"
@@ -46,23 +46,24 @@ struct Tables {                                          /* 4. to 6., in the roo
 };
 
 /* The usual ctx after its sort: nothing served high budget first, offsets and A within 31 bits, at most
- * 32 stages.  The elements fall apart into arrays, queue after queue. */
+ * 32 stages.  The elements fall apart into arrays, queue after queue; position p stands at p + lead, lead = the ctx's first
+ * request modulo 8, so that a thread's groups of eight are those of the output. */
+constexpr int kLocGroup = 8;
+constexpr uint32_t kLocOneByOne = 768;                   /* see finish_split */
 struct Split {
-  uint32_t off[kLocalTile];                              /* deadline offsets */
-  uint16_t idx[kLocalTile];                              /* index inside the ctx */
-  uint16_t win[kLocalTile];                              /* window */
+  uint32_t off[kLocalTile + kLocGroup];                  /* deadline offsets */
+  uint16_t idx[kLocalTile + kLocGroup];                  /* index inside the ctx */
   uint32_t P[kTabEntries];
-  int32_t EK[kTabEntries];                               /* E, or Kp for raw positions */
-  uint32_t U[kTabEntries];                               /* u of the window */
+  int2 QU[kTabEntries];                                  /* of a window: min(E, 1) - 1, or Kp for raw positions; u */
   uint16_t kept[kLocalTile];                             /* survivors, queue after queue */
 };
 
 /* Requests that come in order, on their way into the Split form: beside its off and idx. */
 struct Ordered {
-  uint32_t off[kLocalTile];                              /* Split's */
-  uint16_t idx[kLocalTile];
+  uint32_t off[kLocalTile + kLocGroup];                  /* Split's */
+  uint16_t idx[kLocalTile + kLocGroup];
   uint32_t D[kLocalTile];                                /* low words of the deadlines */
-  uint8_t code[kLocalTile];                              /* stage, then stage | rank << 4 among the 16 requests of one thread */
+  uint8_t code[kLocalTile];                              /* four times the stage */
   uint16_t place[16][kLocThreads];                       /* [stage][thread]: first place of the thread's requests */
 };
 
@@ -74,6 +75,7 @@ struct LocalSmem {
       uint32_t match[kLocWarps][kBins];                  /* lanes currently holding the digit */
     };
     Tables tab;
+    unsigned char room[sizeof(Ordered) - sizeof(unsigned long long) * kLocalTile];
   };
   PardSegConst K[PARD_MAX_STAGES];
   uint32_t stage_first[PARD_MAX_STAGES + 2];
@@ -81,7 +83,6 @@ struct LocalSmem {
   uint32_t kept_base[PARD_MAX_STAGES];
   uint32_t hb_kept[PARD_MAX_STAGES];                     /* high budget first: length of the kept prefix */
   uint32_t win_off[PARD_MAX_STAGES], win_cnt[PARD_MAX_STAGES];
-  uint32_t row_first[PARD_MAX_STAGES + 1];               /* Split: first row of 32 positions of every queue */
   uint32_t scan[kLocWarps];
   uint32_t few[8][kLocWarps];
   unsigned long long red_min[kLocWarps], red_max[kLocWarps];
@@ -91,6 +92,12 @@ struct LocalSmem {
 };
 
 static_assert(sizeof(Ordered) <= offsetof(LocalSmem, K) && sizeof(Split) <= offsetof(LocalSmem, K), "inside keys and counters");
+
+/* smallest of the warp's values, by the words */
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long x) {
+  const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(x >> 32));
+  return (unsigned long long)hi << 32 | __reduce_min_sync(0xffffffffu, (uint32_t)(x >> 32) == hi ? (uint32_t)x : 0xffffffffu);
+}
 
 /* a thread's sorted element, decoded */
 struct Elem {
@@ -194,72 +201,103 @@ __device__ __forceinline__ void pass_byte(unsigned long long (&key)[kLocItems], 
   }
 }
 
-/* A stable counting sort by stage of requests that come in order: a thread owns 16 consecutive
- * requests and counts its stages in the bytes of registers, which also yields every request's rank
- * among them; the counts, two to a word, are scanned over the block.  HALVES: 8 stages each.  (By
- * ballots, row after row, the same took three times the instructions.)  Leaves the queues' first
- * positions in Sm.stage_first. */
-template <int HALVES>
-__device__ __forceinline__ void order_few(LocalSmem& Sm, Ordered& T, uint32_t cnt, uint32_t S) {
+/* the codes of a thread's PER consecutive requests: 16, or 4 in contexts of up to 2,048 requests, so that every warp has
+ * some (one of 141: 26.2 -> 22.5 us) */
+template <int PER>
+__device__ __forceinline__ uint4 load_codes(const Ordered& T, uint32_t tid) {
+  if (PER == 16) return *reinterpret_cast<const uint4*>(&T.code[tid * 16]);
+  return make_uint4(*reinterpret_cast<const uint32_t*>(&T.code[tid * 4]), 0u, 0u, 0u);
+}
+
+/* A stable counting sort by stage of requests that come in order: a thread owns 16 (in small contexts 4) consecutive
+ * requests and counts its stages in half bytes of a register (of two, from nine stages on), which also yields every
+ * request's rank among them (returned, four bits each); the counts, two to a word, are scanned over the block.  Bound by
+ * instructions: with whole bytes 17 per request where this takes 7.  (By ballots, row after row, with ranks and deadlines
+ * kept in registers: no fewer, and spilled.)  Leaves the queues' first positions in Sm.stage_first and the
+ * thread's places in T.place. */
+template <int HALVES, int PER>
+__device__ __forceinline__ uint2 order_few(LocalSmem& Sm, Ordered& T, uint32_t cnt, uint32_t S) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kWords = 2 * HALVES;                     /* 4 stages each */
-  uint32_t n[kWords];
+  uint32_t n[HALVES], ranks[2] = {0, 0};                 /* n: stages 0 to 7, 8 to 15; of the first 15 requests */
 #pragma unroll
-  for (int h = 0; h < kWords; ++h) n[h] = 0;
-  const uint32_t mine = cnt > tid * 16 ? min(cnt - tid * 16, 16u) : 0u;
+  for (int h = 0; h < HALVES; ++h) n[h] = 0;
+  const uint32_t mine = cnt > tid * PER ? min(cnt - tid * PER, (uint32_t)PER) : 0u;
+  uint32_t last[HALVES];                                 /* the sixteenth, apart: a count of 16 takes five bits */
+#pragma unroll
+  for (int h = 0; h < HALVES; ++h) last[h] = 0;
   if (mine) {
-    uint4* codes = reinterpret_cast<uint4*>(&T.code[tid * 16]);
-    const uint4 s = *codes;
-    uint32_t out[4];
+    const uint4 s = load_codes<PER>(T, tid);
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
+    for (int i = 0; i < PER; ++i) {
+      if (i >= (int)mine) break;
       const uint32_t w = i < 4 ? s.x : i < 8 ? s.y : i < 12 ? s.z : s.w;
-      const uint32_t k = (w >> (8 * (i & 3))) & 15u, sh = (k & 3u) * 8, inc = (i < (int)mine ? 1u : 0u) << sh;
-      uint32_t have = n[0];
-#pragma unroll
-      for (int h = 1; h < kWords; ++h) have = (k >> 2) == (uint32_t)h ? n[h] : have;
-      const uint32_t r = (have >> sh) & 0xffu;
-#pragma unroll
-      for (int h = 0; h < kWords; ++h) n[h] += (k >> 2) == (uint32_t)h ? inc : 0u;
-      out[i / 4] = (i & 3) ? out[i / 4] | ((k | r << 4) << (8 * (i & 3))) : (k | r << 4);
+      const uint32_t k4 = (w >> (8 * (i & 3))) & 63u;     /* four times the stage */
+      const uint32_t sh = HALVES == 2 ? k4 & 31u : k4, inc = 1u << sh;
+      const bool up = HALVES == 2 && k4 >= 32;
+      ranks[i / 8] |= (((up ? n[HALVES - 1] : n[0]) >> sh) & 15u) << (4 * (i & 7));
+      uint32_t* to = i < 15 ? n : last;
+      if (HALVES == 1) to[0] += inc;
+      else { to[0] += up ? 0u : inc; to[HALVES - 1] += up ? inc : 0u; }
     }
-    *codes = make_uint4(out[0], out[1], out[2], out[3]);
   }
-  /* stages 4h, 4h+2 in c[2h], 4h+1, 4h+3 in c[2h+1]; counts of at most 8,192 in 16 bits */
-  uint32_t c[2 * kWords], own[2 * kWords];
+  /* stages 8h + q and 8h + q + 4 in c[4h + q]; counts of at most 8,192 in 16 bits */
+  uint32_t c[4 * HALVES], own[4 * HALVES];
 #pragma unroll
-  for (int h = 0; h < kWords; ++h) {
-    own[2 * h] = c[2 * h] = n[h] & 0x00ff00ffu;
-    own[2 * h + 1] = c[2 * h + 1] = (n[h] >> 8) & 0x00ff00ffu;
-  }
+  for (int h = 0; h < HALVES; ++h)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) own[4 * h + q] = c[4 * h + q] = ((n[h] >> (4 * q)) & 0x000f000fu) + ((last[h] >> (4 * q)) & 0x000f000fu);
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1)
 #pragma unroll
-    for (int q = 0; q < 2 * kWords; ++q) {
+    for (int q = 0; q < 4 * HALVES; ++q) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, c[q], o);
       if (lane >= (uint32_t)o) c[q] += y;
     }
   if (lane == 31)
 #pragma unroll
-    for (int q = 0; q < 2 * kWords; ++q) Sm.few[q][warp] = c[q];
+    for (int q = 0; q < 4 * HALVES; ++q) Sm.few[q][warp] = c[q];
   __syncthreads();
   uint32_t run = 0;                                      /* first position of the stage at hand */
-  uint32_t total[2 * kWords];
+  uint32_t total[4 * HALVES];
 #pragma unroll
-  for (int q = 0; q < 2 * kWords; ++q) {
+  for (int q = 0; q < 4 * HALVES; ++q) {
     const uint32_t w = lane < (uint32_t)kLocWarps ? Sm.few[q][lane] : 0u;
     total[q] = __reduce_add_sync(0xffffffffu, w);
     c[q] += __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) - own[q];     /* before this thread */
   }
 #pragma unroll
   for (int k = 0; k < 8 * HALVES; ++k) {
-    const int q = 2 * (k / 4) + (k & 1), sh = (k & 2) ? 16 : 0;
+    const int q = 4 * (k / 8) + (k & 3), sh = (k & 4) ? 16 : 0;
     T.place[k][tid] = (uint16_t)(run + ((c[q] >> sh) & 0xffffu));
     if (tid == 0 && k < (int)S) Sm.stage_first[k] = run;
     run += (total[q] >> sh) & 0xffffu;
   }
   if (tid == 0) Sm.stage_first[S] = cnt;
   __syncthreads();
+  return make_uint2(ranks[0], ranks[1]);
+}
+
+/* the thread's own requests to their places */
+template <int PER>
+__device__ __forceinline__ void place_few(Ordered& T, uint32_t cnt, uint2 ranks, uint32_t lead, uint32_t dmin) {
+  const uint32_t tid = threadIdx.x, p0 = tid * PER;
+  if (p0 >= cnt) return;
+  const bool whole = p0 + PER <= cnt;
+  const uint4 s = load_codes<PER>(T, tid);
+#pragma unroll
+  for (int q = 0; q < PER / 4; ++q) {
+    const uint4 x = *reinterpret_cast<const uint4*>(&T.D[p0 + 4 * q]);
+    const uint32_t w = q == 0 ? s.x : q == 1 ? s.y : q == 2 ? s.z : s.w;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t pos = p0 + 4 * q + u, low = u == 0 ? x.x : u == 1 ? x.y : u == 2 ? x.z : x.w;
+      const uint32_t at = lead + (&T.place[0][tid])[((w >> (8 * u)) & 63u) * (kLocThreads / 4)] + (((q < 2 ? ranks.x : ranks.y) >> (4 * ((4 * q + u) & 7))) & 15u);
+      if (whole || pos < cnt) {
+        T.off[at] = low - dmin;
+        T.idx[at] = (uint16_t)pos;
+      }
+    }
+  }
 }
 
 /* E and, for raw positions, Kp of one queue's table, by one warp; returns the queue's kept count,
@@ -394,98 +432,131 @@ __device__ __forceinline__ bool split_fits(const LocalArgs& a, const LocalSmem& 
   return __syncthreads_and(ok) != 0;
 }
 
-/* 4. to 6. in the Split form.  Work is dealt out in rows of 32 positions of one queue, so that the
- * queue's constants are the same for a whole row.  False: more windows than the tables hold,
- * nothing has been written. */
+/* 4. to 6. in the Split form.  A thread takes groups of eight positions.  Windows only rise along a queue, so a group
+ * whose neighbour ahead and whose last request are in one window is done with two divisions; along a window the
+ * admitted position rises by one per request up to u, c = min(r + q, u) with q = min(E, 1) - 1 (at the window's first
+ * request too: E is at most the u before less the requests ahead), so its survivors are the window's first ones and a
+ * group's estimates are at most two when a batch round takes eight.  (Every request on its own, 32 in a row to a warp: 218
+ * instructions per request for 4,096 contexts of 8,192, 175 like this with the sort below; calls 354 -> 314 us, 2,000 of 4,000
+ * 155 -> 138, one of 7,800 31.5 -> 28.5.)  Up to kLocOneByOne requests a group per thread would leave most warps idle, and
+ * every request goes on its own: by groups ten contexts of 730 took 31.8 us and 600 of 256 34.7, like this 29.4 and 30.4
+ * (as before: 29.4 and 32.4); 1,000 of 1,000 are faster by groups, 54.4 -> 48.9.  False: more windows than the tables
+ * hold, nothing has been written. */
 template <bool RAW>
-__device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, uint32_t c, uint32_t first) {
+__device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, uint32_t c, uint32_t first, uint32_t cnt) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t S = (uint32_t)a.st.stage_stride;
+  const uint32_t S = (uint32_t)a.st.stage_stride, lead = first % kLocGroup;
   Split& T = *reinterpret_cast<Split*>(Sm.keys);
-  if (warp == 0) {                                       /* extents: windows up to every queue's last request, rows */
-    uint32_t w = 0, rows = 0;
+  if (warp == 0) {                                       /* extents: windows up to every queue's last request */
+    uint32_t w = 0;
     if (lane < S) {
       const uint32_t lo = Sm.stage_first[lane], hi = Sm.stage_first[lane + 1];
       const PardSegConst& K = Sm.K[lane];
       if (hi > lo) {
-        const long long X = (long long)T.off[hi - 1] - K.A_rel;
+        const long long X = (long long)T.off[lead + hi - 1] - K.A_rel;
         w = X < 0 ? 1u : min(div_magic32((uint32_t)X, K.d_magic), kTabEntries) + 2u;
-        rows = (hi - lo + 31) / 32;
       }
     }
-    uint32_t x = w, y = rows;
+    uint32_t x = w;
     for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
-      if (lane >= (uint32_t)o) { x += p; y += q; }
+      const uint32_t p = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (uint32_t)o) x += p;
     }
     if (lane < S) {
       Sm.win_off[lane] = x - w;
       Sm.win_cnt[lane] = w;
-      Sm.row_first[lane] = y - rows;
       if (w && x <= kTabEntries) T.P[x - 1] = Sm.stage_first[lane + 1] - Sm.stage_first[lane];   /* the end marker */
     }
-    if (lane == 31) {
-      Sm.row_first[S] = y;
-      Sm.use_scan = x > kTabEntries ? 1u : 0u;
-    }
+    if (lane == 31) Sm.use_scan = x > kTabEntries ? 1u : 0u;
   }
   __syncthreads();
   if (Sm.use_scan) return false;
-  /* a warp takes consecutive rows; lane j holds queue j's first row */
-  const uint32_t n_rows = Sm.row_first[S], my_row_first = lane < S ? Sm.row_first[lane] : 0xffffffffu;
-  const uint32_t per = (n_rows + kLocWarps - 1) / kLocWarps, row0 = min(warp * per, n_rows), row1 = min(row0 + per, n_rows);
-  for (uint32_t row = row0; row < row1;) {
-    const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, my_row_first <= row));   /* the queue of the row */
-    const uint32_t lo = Sm.stage_first[k], n = Sm.stage_first[k + 1] - lo, rf = Sm.row_first[k];
-    const uint32_t rows = min(row1, Sm.row_first[k + 1]);
-    const int32_t A = (int32_t)Sm.K[k].A_rel;
-    const unsigned long long magic = Sm.K[k].d_magic;
-    uint32_t* P = T.P + Sm.win_off[k];
-    uint32_t r = (row - rf) * 32 + lane;
-    uint32_t before = kNoWindow;                         /* window of the request ahead of the row */
-    if (row > rf) {
-      const int32_t off = (int32_t)T.off[lo + r - lane - 1];
-      before = off < A ? kNoWindow : div_magic32((uint32_t)off - (uint32_t)A, magic);
+  /* the queue of position p, the last that begins at or before it */
+  auto queue_at = [&](uint32_t p) {
+    uint32_t k = 0, z = S;
+    while (z - k > 1) {
+      const uint32_t mid = (k + z) / 2;
+      if (Sm.stage_first[mid] <= p) k = mid; else z = mid;
     }
-#pragma unroll 2
-    for (; row < rows; ++row, r += 32) {
-      const bool in = r < n;
-      const int32_t off = in ? (int32_t)T.off[lo + r] : A;
-      const uint32_t b = off < A ? kNoWindow : div_magic32((uint32_t)off - (uint32_t)A, magic);
-      const uint32_t pb = __shfl_sync(0xffffffffu, lane == 31 ? before : b, (lane - 1) & 31);
-      before = b;
-      if (in) {
-        T.win[lo + r] = (uint16_t)b;
-        if (b != pb || r == 0) {                         /* (b == kNoWindow: no entry begins here) */
-          if (b != kNoWindow)
-            for (uint32_t e = r == 0 || pb == kNoWindow ? 0u : pb + 1; e <= b; ++e) P[e] = r;
+    return k;
+  };
+  const uint32_t end = lead + cnt, groups = cnt ? (end + kLocGroup - 1) / kLocGroup : 0u;   /* (an empty ctx: none) */
+  const bool one_by_one = cnt <= kLocOneByOne;
+  if (one_by_one)
+    for (uint32_t p = tid; p < cnt; p += kLocThreads) {
+      const uint32_t k = queue_at(p), r = p - Sm.stage_first[k];
+      const int32_t off = (int32_t)T.off[lead + p], A = (int32_t)Sm.K[k].A_rel;
+      const unsigned long long magic = Sm.K[k].d_magic;
+      const int32_t b = off < A ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)A, magic);
+      int32_t e = -1;
+      if (r) {
+        const int32_t before = (int32_t)T.off[lead + p - 1];
+        e = before < A ? -1 : (int32_t)div_magic32((uint32_t)before - (uint32_t)A, magic);
+      }
+      while (e < b) T.P[Sm.win_off[k] + (uint32_t)++e] = r;
+    }
+  else
+  for (uint32_t g = tid; g < groups; g += kLocThreads) {
+    const uint32_t x0 = g * kLocGroup;
+    uint32_t x = max(x0, lead);                          /* span after span of requests of one queue: mostly one */
+    const uint32_t xe = min(x0 + kLocGroup, end);
+    while (x < xe) {
+      const uint32_t k = queue_at(x - lead), lo = Sm.stage_first[k], stop = min(xe, lead + Sm.stage_first[k + 1]), r = x - lead - lo;
+      const int32_t A = (int32_t)Sm.K[k].A_rel;
+      const unsigned long long magic = Sm.K[k].d_magic;
+      auto window = [&](uint32_t at) {                   /* -1: deadline before A */
+        const int32_t off = (int32_t)T.off[at];
+        return off < A ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)A, magic);
+      };
+      const int32_t ahead = r ? window(x - 1) : -1, last = window(stop - 1);
+      if (ahead < last) {                                /* windows begin here: their P, the requests before them */
+        const uint32_t d = (uint32_t)Sm.K[k].d;
+        uint32_t X[kLocGroup];                           /* deadline - A, expired: 0 (window 0 begins at the first that is not) */
+        uint32_t expired = 0;
+        const uint4 u = *reinterpret_cast<const uint4*>(&T.off[x0]), v = *reinterpret_cast<const uint4*>(&T.off[x0 + 4]);
+        const uint32_t off[kLocGroup] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < kLocGroup; ++i) {
+          const bool in = x0 + i >= x && x0 + i < stop;
+          const bool late = (int32_t)off[i] < A;
+          X[i] = !in ? 0xffffffffu : late ? 0u : off[i] - (uint32_t)A;
+          expired += in && late ? 1u : 0u;
+        }
+        uint32_t* P = T.P + Sm.win_off[k];
+        for (int32_t e = ahead + 1; e <= last; ++e) {
+          const uint32_t from = (uint32_t)e * d;         /* <= the last request's deadline - A */
+          uint32_t below = 0;
+#pragma unroll
+          for (int i = 0; i < kLocGroup; ++i) below += X[i] < from ? 1u : 0u;
+          P[e] = r + (e ? below : expired);
         }
       }
+      x = stop;
     }
   }
   __syncthreads();
   /* E (Kp), u and every queue's kept count */
   for (uint32_t k = warp; k < S; k += kLocWarps) {
     uint32_t kept = 0;
-    const uint32_t at = Sm.win_off[k], cnt = Sm.win_cnt[k], cap = Sm.K[k].cap;
-    if (cnt) {
+    const uint32_t at = Sm.win_off[k], wins = Sm.win_cnt[k], cap = Sm.K[k].cap;
+    if (wins) {
       const uint32_t P0 = T.P[at];
       int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;       /* the requests with deadline < A: u = 0 */
       uint32_t k_carry = 0;
-      if (lane == 0) T.EK[at] = RAW ? 0 : e_carry;
-      for (uint32_t b0 = 0; b0 + 1 < cnt; b0 += 32) {                /* windows b0.. -> entries b0+1.. */
+      for (uint32_t b0 = 0; b0 + 1 < wins; b0 += 32) {               /* windows b0.. */
         const uint32_t b = b0 + lane;
         int32_t val = kWinInf;
-        uint32_t more = 0;
-        if (b + 1 < cnt) {
-          const uint32_t p = T.P[at + b], q = T.P[at + b + 1], u = win_u(b, cap);
-          T.U[at + b] = u;
+        uint32_t more = 0, u = 0;
+        if (b + 1 < wins) {
+          const uint32_t p = T.P[at + b], q = T.P[at + b + 1];
+          u = win_u(b, cap);
           if (q > p) {
             val = (int32_t)u - (int32_t)(q - 1);
             const uint32_t top = u < q ? u : q;
             more = top > p ? top - p : 0;
           }
         }
+        const uint32_t own_more = more;
         for (int o = 1; o < 32; o <<= 1) {
           if (RAW) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, more, o);
@@ -495,12 +566,14 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
             if (lane >= (uint32_t)o) val = min(val, y);
           }
         }
-        const int32_t out = RAW ? (int32_t)(k_carry + more) : min(e_carry, val);
-        if (b + 1 < cnt) T.EK[at + b + 1] = out;
-        const int32_t last = __shfl_sync(0xffffffffu, out, 31);
-        if (RAW) k_carry = (uint32_t)last; else e_carry = last;
+        /* of the windows before this lane's */
+        int32_t before = __shfl_up_sync(0xffffffffu, val, 1);
+        before = min(e_carry, lane ? before : kWinInf);
+        if (b + 1 < wins) T.QU[at + b] = make_int2(RAW ? (int32_t)(k_carry + more - own_more) : min(before, 1) - 1, (int32_t)u);
+        if (RAW) k_carry += __shfl_sync(0xffffffffu, more, 31);
+        else e_carry = min(e_carry, __shfl_sync(0xffffffffu, val, 31));
       }
-      const uint32_t n_q = T.P[at + cnt - 1];
+      const uint32_t n_q = T.P[at + wins - 1];
       kept = RAW ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1));
     }
     if (lane == 0) {
@@ -512,43 +585,103 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
   __syncthreads();
   if (warp == 0) publish_kept(a, Sm, c, lane);
   __syncthreads();
-  for (uint32_t row = row0; row < row1;) {
-    const uint32_t k = 31 - __clz(__ballot_sync(0xffffffffu, my_row_first <= row));
-    const uint32_t lo = Sm.stage_first[k], n = Sm.stage_first[k + 1] - lo, rf = Sm.row_first[k];
-    const uint32_t rows = min(row1, Sm.row_first[k + 1]);
-    const PardSegConst& K = Sm.K[k];
-    const long long A = K.A;
-    const unsigned long long cap_magic = K.cap_magic;
-    const uint32_t d = (uint32_t)K.d, woff = Sm.win_off[k];          /* d fits 32 bits: it has a magic number */
-    uint16_t* kept_out = T.kept + Sm.kept_base[k];
-    uint32_t r = (row - rf) * 32 + lane;
-    const size_t g0 = (size_t)first + lo + r;
-    uint8_t* keep_p = a.out_keep + g0;
-    long long* est_p = a.out_est + g0;
-    uint32_t* perm_p = a.out_perm + g0;
-#pragma unroll 2
-    for (; row < rows; ++row, r += 32, keep_p += 32, est_p += 32, perm_p += 32) {
-      if (r >= n) continue;
-      const uint32_t b = T.win[lo + r], local = T.idx[lo + r];
+  if (one_by_one)
+    for (uint32_t p = tid; p < cnt; p += kLocThreads) {
+      const uint32_t k = queue_at(p), r = p - Sm.stage_first[k], local = T.idx[lead + p];
+      const PardSegConst& K = Sm.K[k];
+      const int32_t off = (int32_t)T.off[lead + p], A = (int32_t)K.A_rel;
       uint32_t cpos = RAW ? r : 0u, ahead = 0, u = 0;    /* batch-slot position; kept requests ahead in the queue */
-      if (b != kNoWindow) {
-        const uint32_t P = T.P[woff + b];
-        u = T.U[woff + b];
+      if (off >= A) {
+        const uint32_t at = Sm.win_off[k] + div_magic32((uint32_t)off - (uint32_t)A, K.d_magic);
+        const int2 w = T.QU[at];
+        u = (uint32_t)w.y;
         if (RAW) {
-          const uint32_t top = r < u ? r : u;
-          ahead = (uint32_t)T.EK[woff + b] + (top > P ? top - P : 0);
+          const uint32_t top = r < u ? r : u, P = T.P[at];
+          ahead = (uint32_t)w.x + (top > P ? top - P : 0);
         } else {
-          int32_t m = T.EK[woff + b];                    /* min over t < r of (u_t - t); values above 1 cannot lower the position */
-          if (r > P) m = min(m, (int32_t)u - (int32_t)(r - 1));
-          cpos = ahead = r == 0 ? 0u : r - 1 + (uint32_t)min(m, 1);
+          cpos = ahead = min((uint32_t)((int32_t)r + w.x), u);
         }
       }
       const bool keep = cpos < u;
-      const uint32_t round = cap_magic ? div_magic32(cpos, cap_magic) : cpos;
-      if (keep) kept_out[ahead] = (uint16_t)local;
-      if (a.out_keep) *keep_p = keep ? 1 : 0;
-      if (a.out_est) *est_p = A + (long long)((unsigned long long)round * d);
-      if (a.out_perm) *perm_p = first + local;
+      const uint32_t round = K.cap_magic ? div_magic32(cpos, K.cap_magic) : cpos;
+      if (keep) T.kept[Sm.kept_base[k] + ahead] = (uint16_t)local;
+      const size_t at = (size_t)first + p;
+      if (a.out_keep) a.out_keep[at] = keep ? 1 : 0;
+      if (a.out_est) a.out_est[at] = K.A + (long long)((unsigned long long)round * (uint32_t)K.d);
+      if (a.out_perm) a.out_perm[at] = first + local;
+    }
+  else
+  for (uint32_t g = tid; g < groups; g += kLocThreads) {
+    const uint32_t x0 = g * kLocGroup, xa = max(x0, lead), xe = min(x0 + kLocGroup, end);
+    const size_t out = (size_t)(first - lead) + x0;
+    const uint4 ix = *reinterpret_cast<const uint4*>(&T.idx[x0]);
+    const uint32_t pair[4] = {ix.x, ix.y, ix.z, ix.w};
+    uint32_t keepbits = 0, list = 0, k = 0, r_less = 0, rest = 0;  /* position in the queue less that in the group; the queue's end in the group */
+    long long est[kLocGroup];
+#pragma unroll
+    for (int q = 0; q < kLocGroup; ++q) est[q] = 0;
+    int32_t b = 0;
+    for (uint32_t i = xa - x0; i < xe - x0;) {           /* span after span of one queue and window: mostly one */
+      if (i >= rest) {                                   /* a queue begins, or the group does */
+        k = queue_at(x0 + i - lead);
+        r_less = x0 - lead - Sm.stage_first[k];
+        rest = min(lead + Sm.stage_first[k + 1], xe) - x0;
+        const int32_t off = (int32_t)T.off[x0 + i], A = (int32_t)Sm.K[k].A_rel;
+        b = off < A ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)A, Sm.K[k].d_magic);
+      }
+      const PardSegConst& K = Sm.K[k];
+      const uint32_t r = r_less + i, cap = K.cap;
+      uint32_t at = Sm.win_off[k] + (uint32_t)b;
+      for (; T.P[at + 1] <= r; ++at) ++b;                /* the window of request r */
+      uint32_t stop = min(T.P[at + 1] - r_less, rest);
+      int2 w = make_int2(0, 0);
+      if (b >= 0) w = T.QU[at];
+      uint32_t c0 = 0, left = 0, into = 0;               /* batch-slot position, kept ones of the span from here on, their place among the queue's */
+      if (RAW) {
+        stop = i + 1;
+        c0 = r;
+        left = b >= 0 && r < (uint32_t)w.y ? 1u : 0u;
+        into = left ? (uint32_t)w.x + r - T.P[at] : 0u;
+      } else if (b >= 0) {
+        c0 = into = min((uint32_t)((int32_t)r + w.x), (uint32_t)w.y);
+        left = (uint32_t)w.y - c0;
+      }
+      const uint32_t round = cap > 1 ? div_magic32(c0, K.cap_magic) : c0, fresh = cap - (c0 - round * cap);   /* requests up to the next round */
+      if (cap < kLocGroup && left) stop = min(stop, i + fresh);       /* small rounds: one at a time */
+      const uint32_t next = fresh <= left ? i + fresh : (uint32_t)kLocGroup;
+      const long long e0 = K.A + (long long)((unsigned long long)round * (uint32_t)K.d), e1 = e0 + K.d;      /* d fits 32 bits: it has a magic number */
+#pragma unroll
+      for (int q = 0; q < kLocGroup; ++q) {              /* (what lies behind the span is made good by the next one) */
+        if (q >= (int)i) est[q] = e0;
+        if (q >= (int)next) est[q] = e1;
+      }
+      const uint32_t n_kept = min(stop - i, left);
+      if (!keepbits) list = Sm.kept_base[k] + into;
+      keepbits |= ((1u << n_kept) - 1) << i;
+      i = stop;
+    }
+    /* the thread's survivors follow one another, across queues too */
+#pragma unroll
+    for (int q = 0; q < kLocGroup; ++q)
+      if ((keepbits >> q) & 1u) T.kept[list++] = (uint16_t)((q & 1) ? pair[q / 2] >> 16 : pair[q / 2] & 0xffffu);
+    if (xe - xa == kLocGroup) {
+      if (a.out_keep) *reinterpret_cast<uint2*>(a.out_keep + out) = make_uint2(((keepbits & 15u) * 0x00204081u) & 0x01010101u, ((keepbits >> 4) * 0x00204081u) & 0x01010101u);
+      if (a.out_est) {
+        store4(a.out_est + out, est[0], est[1], est[2], est[3]);
+        store4(a.out_est + out + 4, est[4], est[5], est[6], est[7]);
+      }
+      if (a.out_perm) {
+        auto two = [&](uint32_t v) { return (first + (v & 0xffffu)) | (unsigned long long)(first + (v >> 16)) << 32; };
+        store4(a.out_perm + out, two(pair[0]), two(pair[1]), two(pair[2]), two(pair[3]));
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < kLocGroup; ++q)
+        if (x0 + q >= xa && x0 + q < xe) {
+          if (a.out_keep) a.out_keep[out + q] = (keepbits >> q) & 1u;
+          if (a.out_est) a.out_est[out + q] = est[q];
+          if (a.out_perm) a.out_perm[out + q] = first + ((q & 1) ? pair[q / 2] >> 16 : pair[q / 2] & 0xffffu);
+        }
     }
   }
   if (!place_survivors(hdr, a, Sm, c)) return true;      /* (its barrier also completes the list) */
@@ -813,72 +946,74 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   if (rfirst < cnt && warp < kReaders) {
     const uint4* req = a.req + first;
     const uint4 p = __ldg(&req[rfirst > 0 ? rfirst - 1 : 0]);
-    const uint32_t high = p.y;
+    const uint32_t wend = min(cnt, rfirst + 32 * ritems);
+    const uint32_t high = p.y, x_first = __ldg(&req[rfirst]).x, x_last = __ldg(&req[wend - 1]).x;
     uint32_t last = p.x;                                 /* low words of the row before this one, first the request before the warp's */
     constexpr int kUn = 4;                               /* requests in flight per thread */
-    const uint32_t wend = min(cnt, rfirst + 32 * ritems);
+    bool ordered = few;                                  /* (uniform) */
 #pragma unroll 1
     for (uint32_t p0 = rfirst + lane; p0 - lane < wend; p0 += 32 * kUn) {
       uint4 r[kUn];
       const bool full = p0 - lane + 32 * kUn <= wend;    /* uniform */
+      if (full) {
 #pragma unroll
-      for (int u = 0; u < kUn; ++u) {
-        r[u] = make_uint4(0xffffffffu, high, c, 0u);     /* behind every request */
-        if (full || p0 + u * 32 < wend) r[u] = __ldg(&req[p0 + u * 32]);
-      }
-      uint32_t other = 0, top = 0, hi = 0;
-      bool back = false;
-#pragma unroll
-      for (int u = 0; u < kUn; ++u) {
-        const uint32_t px = __shfl_sync(0xffffffffu, lane == 31 ? last : r[u].x, (lane - 1) & 31);
-        last = r[u].x;
-        back |= r[u].x < px;
-        other |= r[u].z ^ c;
-        hi |= r[u].y ^ high;
-        top = max(top, r[u].w & 0xffffu);
-        if (full || p0 + u * 32 < wend) {
-          O.D[p0 + u * 32] = r[u].x;
-          O.code[p0 + u * 32] = (uint8_t)(r[u].w & 15u);
-        }
-      }
-      const bool fine = !back && (other | hi) == 0 && top < S && high < (uint32_t)(PARD_TIME_LIMIT_US >> 32);
-      if (__all_sync(0xffffffffu, fine) && !(seen & 4u)) {
-        /* in order: the lane's range is that of its first and its last request */
-        uint32_t x1 = r[0].x;
-#pragma unroll
-        for (int u = 1; u < kUn; ++u)
-          if (full || p0 + u * 32 < wend) x1 = r[u].x;
-        if (p0 < wend) {
-          const unsigned long long D0 = ((unsigned long long)high << 32) | r[0].x, D1 = ((unsigned long long)high << 32) | x1;
-          lmin = D0 < lmin ? D0 : lmin;
-          lmax = D1 > lmax ? D1 : lmax;
-        }
+        for (int u = 0; u < kUn; ++u) r[u] = __ldg(&req[p0 + u * 32]);
       } else {
-        seen |= 4u;
 #pragma unroll
         for (int u = 0; u < kUn; ++u) {
-          const unsigned long long D = ((unsigned long long)r[u].y << 32) | r[u].x;
-          if (p0 + u * 32 < wend) {
-            if (r[u].z == c && (r[u].w & 0xffffu) < S && D < (unsigned long long)PARD_TIME_LIMIT_US) {
-              lmin = D < lmin ? D : lmin;
-              lmax = D > lmax ? D : lmax;
-            } else {
-              seen |= r[u].z != c ? 3u : 2u;
-            }
+          r[u] = make_uint4(0xffffffffu, high, c, 0u);   /* behind every request */
+          if (p0 + u * 32 < wend) r[u] = __ldg(&req[p0 + u * 32]);
+        }
+      }
+      if (ordered) {
+        uint32_t other = 0, top = 0;
+        bool back = false;
+        const uint32_t behind = __shfl_sync(0xffffffffu, last, 31);
+#pragma unroll
+        for (int u = 0; u < kUn; ++u) {
+          const uint32_t px = __shfl_sync(0xffffffffu, lane == 31 ? last : r[u].x, (lane - 1) & 31);
+          last = r[u].x;
+          back |= r[u].x < px;
+          other |= (r[u].z ^ c) | (r[u].y ^ high);
+          top = max(top, r[u].w & 0xffffu);
+          if (full || p0 + u * 32 < wend) {
+            O.D[p0 + u * 32] = r[u].x;
+            O.code[p0 + u * 32] = (uint8_t)(4 * (r[u].w & 15u));
+          }
+        }
+        if (__all_sync(0xffffffffu, !back && other == 0 && top < S && high < (uint32_t)(PARD_TIME_LIMIT_US >> 32))) continue;
+        ordered = false;
+        if (p0 - lane > rfirst) {                        /* the rows so far were in order */
+          lmin = ((unsigned long long)high << 32) | x_first;
+          lmax = ((unsigned long long)high << 32) | behind;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kUn; ++u) {
+        const unsigned long long D = ((unsigned long long)r[u].y << 32) | r[u].x;
+        if (p0 + u * 32 < wend) {
+          if (r[u].z == c && (r[u].w & 0xffffu) < S && D < (unsigned long long)PARD_TIME_LIMIT_US) {
+            lmin = D < lmin ? D : lmin;
+            lmax = D > lmax ? D : lmax;
+          } else {
+            seen |= r[u].z != c ? 3u : 2u;
           }
         }
       }
+    }
+    if (ordered) {                                       /* the warp's range is that of its first and its last request */
+      lmin = ((unsigned long long)high << 32) | x_first;
+      lmax = ((unsigned long long)high << 32) | x_last;
+    } else {
+      seen |= 4u;
     }
   }
   if (SINGLE && warp >= kReaders) {
     __shared__ CtxScratch s_scratch;
     if (ctx_constants<true, 1>(a.pipes, a.n_pipelines, a.st, c, 0, 0, Sm.K, s_scratch, nullptr, 32 * kReaders)) set_status(hdr, PARD_EDATA);
   }
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long x = __shfl_xor_sync(0xffffffffu, lmin, o), y = __shfl_xor_sync(0xffffffffu, lmax, o);
-    lmin = x < lmin ? x : lmin;
-    lmax = y > lmax ? y : lmax;
-  }
+  lmin = warp_min(lmin);
+  lmax = ~warp_min(~lmax);
   seen = __reduce_or_sync(0xffffffffu, seen);
   if (lane == 0) {
     Sm.red_min[warp] = lmin;
@@ -891,12 +1026,7 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
     if (tid == 0) { hdr->unsorted = 1; set_status(hdr, PARD_EDATA); hdr->aborted = 1; }
     return;
   }
-  unsigned long long dmin = ~0ull, dmax = 0;
-#pragma unroll
-  for (int w = 0; w < kLocWarps; ++w) {
-    dmin = Sm.red_min[w] < dmin ? Sm.red_min[w] : dmin;
-    dmax = Sm.red_max[w] > dmax ? Sm.red_max[w] : dmax;
-  }
+  const unsigned long long dmin = warp_min(Sm.red_min[lane % kLocWarps]), dmax = ~warp_min(~Sm.red_max[lane % kLocWarps]);
   const bool flagged = flags & 2u;
   const unsigned long long span = dmin <= dmax ? dmax - dmin : 0ull;
   const bool in_order = cnt > 0 && !(flags & 6u) && (span >> 31) == 0;
@@ -920,21 +1050,16 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
   }
 
   /* 3. elements, sorted */
+  const uint32_t lead = first % kLocGroup;
   if (in_order) {
-    if (S <= 8) order_few<1>(Sm, O, cnt, S);
-    else order_few<2>(Sm, O, cnt, S);
+    const bool small = cnt <= 4 * kLocThreads;
+    const uint2 ranks = small ? (S <= 8 ? order_few<1, 4>(Sm, O, cnt, S) : order_few<2, 4>(Sm, O, cnt, S))
+                              : (S <= 8 ? order_few<1, 16>(Sm, O, cnt, S) : order_few<2, 16>(Sm, O, cnt, S));
     if (split_fits(a, Sm, span)) {
-#pragma unroll 4
-      for (int i = 0; i < items; ++i) {
-        const uint32_t pos = wfirst + i * 32 + lane;
-        if (pos < cnt) {
-          const uint32_t code = O.code[pos], at = O.place[code & 15u][pos >> 4] + (code >> 4);
-          O.off[at] = O.D[pos] - (uint32_t)dmin;
-          O.idx[at] = (uint16_t)pos;
-        }
-      }
+      if (small) place_few<4>(O, cnt, ranks, lead, (uint32_t)dmin);
+      else place_few<16>(O, cnt, ranks, lead, (uint32_t)dmin);
       __syncthreads();
-      if (finish_split<RAW>(hdr, a, Sm, c, first)) return;
+      if (finish_split<RAW>(hdr, a, Sm, c, first, cnt)) return;
     }
   }
   if (sb + f.dbits + f.ibits > 64) {         /* the element does not fit 64 bits */
@@ -1001,12 +1126,12 @@ __device__ __forceinline__ void plan_ctx(PlanHeader* __restrict__ hdr, const Loc
       if (i >= items) break;
       const uint32_t pos = wfirst + i * 32 + lane;
       if (pos < cnt) {
-        T.off[pos] = (uint32_t)((e[i] >> f.ibits) & f.dmask);
-        T.idx[pos] = (uint16_t)(((uint32_t)e[i] & f.imask) - first);
+        T.off[lead + pos] = (uint32_t)((e[i] >> f.ibits) & f.dmask);
+        T.idx[lead + pos] = (uint16_t)(((uint32_t)e[i] & f.imask) - first);
       }
     }
     __syncthreads();
-    if (finish_split<RAW>(hdr, a, Sm, c, first)) return;
+    if (finish_split<RAW>(hdr, a, Sm, c, first, cnt)) return;
 #pragma unroll
     for (int i = 0; i < kLocItems; ++i)                  /* too many windows: as they were */
       if (i < items) Sm.keys[wfirst + i * 32 + lane] = e[i];

@@ -53,6 +53,16 @@ def test_walk_rounds_against_steps_and_queue_lengths(rule, cap, n):
         check(inputs.Workload("edge", [p], util.requests(dl), st, 1), rule)
 
 
+# ---- a block per ctx, groups of eight positions against requests one by one --------------------------
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
+@pytest.mark.parametrize("m", [1, 2, 4, 40])                                  # batch rounds of 2, 4, 8 and 80
+@pytest.mark.parametrize("sizes", [[767, 769, 5, 768, 0, 770], [2047, 2049, 3, 2048, 2051], [8191, 0, 1, 8192, 4100], [3001, 6, 0, 0, 7990]])
+def test_groups_of_positions(sizes, m, mode):
+    for S, sort, span in ((3, True, 40_000), (9, True, 3000), (16, False, 3000)):
+        check(several_ctx(len(sizes), sizes, seed=m, S=S, sort=sort, m=m, span=span), mode | pb.PARD_MODE_GROUPED)
+    check(several_ctx(1, [sizes[0]], seed=m, S=5, m=m, span=100), mode)       # one ctx, many equal deadlines
+
+
 # ---- arrival order, one pass straight from the requests: up to 256 queues -------------------------
 @pytest.mark.parametrize("rule", [FCFS, NEXUS, FCFS | pb.PARD_MODE_PATH_MASK])
 @pytest.mark.parametrize("queues", [2, 4, 5, 255, 256, 257])
