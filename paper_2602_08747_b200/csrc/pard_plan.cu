@@ -219,7 +219,7 @@ __device__ __forceinline__ uint32_t range_constants(PardSegConst* K, long long A
 template <bool RANGES>
 __device__ void finish_constants(const ConstArgs& a, const unsigned long long* ctx_dmin_inv, const unsigned long long* ctx_dmax,
                                  PlanHeader* hdr) {
-  __shared__ unsigned long long s_span[8];
+  __shared__ unsigned long long s_span[32];
   __shared__ uint32_t s_w[kHistSegs];
   __shared__ uint32_t s_scan;
   const uint32_t tid = threadIdx.x, lane = tid & 31, S = (uint32_t)a.st.stage_stride, n_seg = a.n_ctx * S;
@@ -387,15 +387,53 @@ k_seg_const(const __grid_constant__ ConstArgs a, const unsigned long long* __res
   if (a.with_key_width && last_block_done(&hdr->seg_done)) finish_constants<false>(a, ctx_dmin_inv, ctx_dmax, hdr);
 }
 
+/* First tile of every ctx when the tiles are cut at ctx boundaries: the running sum of
+ * ceil(requests of the ctx / kSortTile).  One block of 1,024 threads. */
+__device__ __forceinline__ void tile_table(const uint32_t* __restrict__ ctx_start, uint32_t n_ctx, uint32_t* __restrict__ tile_first) {
+  __shared__ uint32_t s_w[32];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t per = (n_ctx + 1023) / 1024;          /* contexts per thread, consecutive */
+  const uint32_t c0 = tid * per, c1 = min(n_ctx, c0 + per);
+  uint32_t sum = 0;
+  for (uint32_t c = c0; c < c1; ++c) sum += (ctx_start[c + 1] - ctx_start[c] + kSortTile - 1) / kSortTile;
+  uint32_t incl = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= (uint32_t)o) incl += y;
+  }
+  if (lane == 31) s_w[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t w = s_w[lane];
+    uint32_t x = w;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= (uint32_t)o) x += y;
+    }
+    s_w[lane] = x - w;
+  }
+  __syncthreads();
+  uint32_t run = s_w[warp] + incl - sum;
+  for (uint32_t c = c0; c < c1; ++c) {
+    tile_first[c] = run;
+    run += (ctx_start[c + 1] - ctx_start[c] + kSortTile - 1) / kSortTile;
+  }
+  if (c1 == n_ctx && c0 < n_ctx) tile_first[n_ctx] = run;
+  if (n_ctx == 0 && tid == 0) tile_first[0] = 0;
+}
+
 /* The constants are there but for what they take from the deadline ranges (k_dir_count worked them out): a thread per
- * queue; the block that finishes last finds the key width.  (k_seg_const, which would do it all again, takes 13 us for 8,192 queues.) */
-__global__ void __launch_bounds__(256)
+ * queue; the block that finishes last finds the key width.  (k_seg_const, which would do it all again, takes 13 us for 8,192 queues.)
+ * The grid's last block lays out the tiles of the passes behind (k_tile_table). */
+__global__ void __launch_bounds__(1024)
 k_seg_finish(const __grid_constant__ ConstArgs a, const unsigned long long* __restrict__ ctx_dmin_inv,
-             const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr) {
+             const unsigned long long* __restrict__ ctx_dmax, PlanHeader* hdr, const uint32_t* __restrict__ ctx_start, uint32_t* __restrict__ tile_first) {
   pdl_wait();
   if (hdr->direct) return;
-  const uint32_t S = (uint32_t)a.st.stage_stride, q = blockIdx.x * 256 + threadIdx.x;
-  if (q < a.n_ctx * S) {
+  const uint32_t S = (uint32_t)a.st.stage_stride, q = blockIdx.x * 1024 + threadIdx.x;
+  if (blockIdx.x == gridDim.x - 1) {
+    tile_table(ctx_start, a.n_ctx, tile_first);
+  } else if (q < a.n_ctx * S) {
     PardSegConst* K = a.ktab + q;
     range_constants(K, K->A, K->d, K->narrow, ~ctx_dmin_inv[q / S], ctx_dmax[q / S]);
   }
@@ -1617,42 +1655,10 @@ k_sort_rest(uint32_t pass, PlanHeader* hdr, unsigned long long* buf_a, unsigned 
 }
 
 
-/* First tile of every ctx when the tiles are cut at ctx boundaries: the running sum of
- * ceil(requests of the ctx / kSortTile).  One block. */
 __global__ void __launch_bounds__(1024)
 k_tile_table(const uint32_t* __restrict__ ctx_start, uint32_t n_ctx, uint32_t* __restrict__ tile_first, const PlanHeader* hdr) {
   pdl_wait();
-  if (hdr->direct) return;
-  __shared__ uint32_t s_w[32];
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t per = (n_ctx + 1023) / 1024;          /* contexts per thread, consecutive */
-  const uint32_t c0 = tid * per, c1 = min(n_ctx, c0 + per);
-  uint32_t sum = 0;
-  for (uint32_t c = c0; c < c1; ++c) sum += (ctx_start[c + 1] - ctx_start[c] + kSortTile - 1) / kSortTile;
-  uint32_t incl = sum;
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= (uint32_t)o) incl += y;
-  }
-  if (lane == 31) s_w[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t w = s_w[lane];
-    uint32_t x = w;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= (uint32_t)o) x += y;
-    }
-    s_w[lane] = x - w;
-  }
-  __syncthreads();
-  uint32_t run = s_w[warp] + incl - sum;
-  for (uint32_t c = c0; c < c1; ++c) {
-    tile_first[c] = run;
-    run += (ctx_start[c + 1] - ctx_start[c] + kSortTile - 1) / kSortTile;
-  }
-  if (c1 == n_ctx && c0 < n_ctx) tile_first[n_ctx] = run;
-  if (n_ctx == 0 && tid == 0) tile_first[0] = 0;
+  if (!hdr->direct) tile_table(ctx_start, n_ctx, tile_first);
 }
 
 /* k_pack for passes that stay inside the contexts: a block packs one tile (all of one ctx) and
@@ -2540,8 +2546,7 @@ k_windows_many(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, co
 /* Decision pass from the window tables: every request on its own.  HF: some
  * queue may be served high budget first (the caller gave priorities). */
 template <bool RAW, bool HF>
-__global__ void __launch_bounds__(kDecThreads, 8)
-k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a,
+__device__ __forceinline__ void decide_tile(uint32_t tile, const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a,
              const unsigned long long* __restrict__ buf_b, uint32_t n, uint32_t ibits,
              const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off,
              const uint32_t* __restrict__ win_off, const uint32_t* __restrict__ win_cnt,
@@ -2550,10 +2555,8 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
              uint32_t* __restrict__ out_perm, uint32_t* __restrict__ out_kept_idx, const uint32_t* __restrict__ kept_base) {
   /* The queues' kept counts followed from their tables, so the survivors go straight to their final
    * place: kept_base holds the queues' output offsets. */
-  pdl_wait();
-  if (hdr->direct | hdr->use_scan | hdr->wide | hdr->aborted) return;
   const TileCtx T = make_tile_ctx(hdr, buf_a, buf_b, n, ibits, ktab, seg_off);
-  const uint64_t base = ((uint64_t)blockIdx.x * kDecThreads + threadIdx.x) * kDecItems;
+  const uint64_t base = ((uint64_t)tile * kDecThreads + threadIdx.x) * kDecItems;
   if (threadIdx.x == 0) l2_ahead(T.src, base, (uint64_t)kDecAhead * kDecTile, kDecTile, n);
   if (base >= n) return;
   const bool full = base + kDecItems <= n;
@@ -2661,6 +2664,33 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
         if (out_perm) out_perm[base + i] = idx[i];
       }
   }
+}
+
+/* A tile per block. */
+template <bool RAW, bool HF>
+__global__ void __launch_bounds__(kDecThreads, 8)
+k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
+             uint32_t ibits, const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off, const uint32_t* __restrict__ win_off,
+             const uint32_t* __restrict__ win_cnt, const WinEntry* __restrict__ wtab, uint8_t* __restrict__ out_keep,
+             long long* __restrict__ out_est, uint32_t* __restrict__ out_perm, uint32_t* __restrict__ out_kept_idx,
+             const uint32_t* __restrict__ kept_base) {
+  pdl_wait();
+  if (hdr->direct | hdr->use_scan | hdr->wide | hdr->aborted) return;
+  decide_tile<RAW, HF>(blockIdx.x, hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, win_cnt, wtab, out_keep, out_est, out_perm, out_kept_idx, kept_base);
+}
+/* For calls that mostly have their plan by then (pard_direct.cuh): a few blocks that take one tile after the other.  A
+ * block per tile, 16,384 at 2^24 requests, took 11 us to find that there is nothing to do. */
+__global__ void __launch_bounds__(kDecThreads, 7)
+k_decide_rest(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
+              uint32_t ibits, const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off, const uint32_t* __restrict__ win_off,
+              const uint32_t* __restrict__ win_cnt, const WinEntry* __restrict__ wtab, uint8_t* __restrict__ out_keep,
+              long long* __restrict__ out_est, uint32_t* __restrict__ out_perm, uint32_t* __restrict__ out_kept_idx,
+              const uint32_t* __restrict__ kept_base) {
+  pdl_wait();
+  if (hdr->direct | hdr->use_scan | hdr->wide | hdr->aborted) return;
+  const uint32_t tiles = (uint32_t)(((uint64_t)n + kDecTile - 1) / kDecTile);
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x)
+    decide_tile<false, false>(tile, hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, win_cnt, wtab, out_keep, out_est, out_perm, out_kept_idx, kept_base);
 }
 
 /* Packs the queues' survivors: copy job j moves up to kCompactChunk indices of one queue; a
@@ -3256,12 +3286,13 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     launch_pdl(k_key_width, 1, 1, 0, stream, sbits, ibits, hdr, arrival_order ? 1u : 0u, key_sbits, state->d_priority ? 1u : 0u);
   }
   if (!const_fold && direct)
-    launch_pdl(k_seg_finish, (L.n_seg + 255) / 256, 256, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
+    launch_pdl(k_seg_finish, (L.n_seg + 1023) / 1024 + 1, 1024, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr,
+               (const uint32_t*)ctx_start, (uint32_t*)(ws + L.tile_first));
   else if (!const_fold)
     launch_pdl(k_seg_const, n_ctx, kConstThreads, 0, stream, ca, (const unsigned long long*)ctx_dmin, (const unsigned long long*)ctx_dmax, hdr);
   if ((local_cand && !local_sure) || (ctx_sort && !direct))
     launch_pdl(k_ctx_ranges, (n_ctx + 1 + 7) / 8, 256, 0, stream, req4, n32, n_ctx, ctx_start, hdr);
-  if (ctx_sort) launch_pdl(k_tile_table, 1, 1024, 0, stream, (const uint32_t*)ctx_start, n_ctx, (uint32_t*)(ws + L.tile_first), (const PlanHeader*)hdr);
+  if (ctx_sort && (const_fold || !direct)) launch_pdl(k_tile_table, 1, 1024, 0, stream, (const uint32_t*)ctx_start, n_ctx, (uint32_t*)(ws + L.tile_first), (const PlanHeader*)hdr);
   mark();
   if (direct) {
     const DirScanOut scan_out = {seg_off, out->d_seg_offsets, seg_kept, kept_base, chunk_base, out->d_seg_kept, (unsigned long long*)out->d_n_kept};
@@ -3338,17 +3369,21 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
     rc = decide_by_walk(pa);
     if (rc != PARD_OK) return rc;
   } else if (n > 0) {
-    uint32_t* tmp = out->d_kept_idx ? kept_tmp : nullptr;
     long long* est = (long long*)out->d_est_us;
     const bool raw = mode & PARD_MODE_RAW;
+    uint32_t* tmp = out->d_kept_idx ? kept_tmp : nullptr;
     /* window tables, and the decision from them */
     mark();
     const uint32_t win_grid = (uint32_t)((n + (uint64_t)kDecTile - 1) / kDecTile);
     auto decide_win = raw ? (state->d_priority ? k_decide_win<true, true> : k_decide_win<true, false>)
                           : (state->d_priority ? k_decide_win<false, true> : k_decide_win<false, false>);
     /* the survivors go straight to their place in the output */
-    launch_pdl(decide_win, win_grid, kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off, win_off, win_cnt, wtab,
-               out->d_keep, est, out->d_perm, out->d_kept_idx, (const uint32_t*)kept_base);
+    if (direct)
+      launch_pdl(k_decide_rest, std::min<uint32_t>(win_grid, 28u * (uint32_t)sms), kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off,
+                 win_off, win_cnt, wtab, out->d_keep, est, out->d_perm, out->d_kept_idx, (const uint32_t*)kept_base);
+    else
+      launch_pdl(decide_win, win_grid, kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off, win_off, win_cnt, wtab,
+                 out->d_keep, est, out->d_perm, out->d_kept_idx, (const uint32_t*)kept_base);
     /* fallback when a queue has too many batch windows: the same decision by scanning, one kernel
      * that returns at once otherwise */
     const uint32_t scan_grid = std::min<uint32_t>(L.dec_tiles, (uint32_t)sms * 2);
