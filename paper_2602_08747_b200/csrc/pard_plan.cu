@@ -949,18 +949,26 @@ __device__ __forceinline__ unsigned long long win_of(unsigned long long X, const
 }
 
 /* E and Kp of the table of one queue (cnt >= 1 entries): the warp runs over the queue's windows, 32 at a
- * time. */
-__device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __restrict__ tab, uint32_t cnt, uint32_t lane, uint32_t raw) {
-  const uint32_t P0 = __ldcg(&tab[0].P);
+ * time.  SHARED: the P are in shared memory, s_P, and go out with the rest of their entries. */
+template <bool SHARED = false>
+__device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __restrict__ tab, uint32_t cnt, uint32_t lane, uint32_t raw,
+                                                    const uint32_t* s_P = nullptr) {
+  auto P_of = [&](uint32_t b) { return SHARED ? s_P[b] : __ldcg(&tab[b].P); };
+  auto put = [&](uint32_t b, uint32_t P, int32_t E, uint32_t Kp) {
+    if (SHARED) *reinterpret_cast<uint4*>(&tab[b]) = make_uint4(P, (uint32_t)E, Kp, 0u);
+    else { tab[b].E = E; tab[b].Kp = Kp; }
+  };
+  const uint32_t P0 = P_of(0);
   int32_t e_carry = P0 > 0 ? -(int32_t)(P0 - 1) : kWinInf;     /* the expired run: u = 0 */
   uint32_t k_carry = 0;
-  if (lane == 0) { tab[0].E = e_carry; tab[0].Kp = 0; }
+  if (lane == 0) put(0, P0, e_carry, 0);
   for (uint32_t b0 = 0; b0 + 1 < cnt; b0 += 32) {              /* windows b0..b0+31 -> entries b0+1.. */
     const uint32_t b = b0 + lane;
     int32_t val = kWinInf;
-    uint32_t kept = 0;
+    uint32_t kept = 0, q = 0;
     if (b + 1 < cnt) {
-      const uint32_t p = __ldcg(&tab[b].P), q = __ldcg(&tab[b + 1].P);
+      const uint32_t p = P_of(b);
+      q = P_of(b + 1);
       if (q > p) {
         const uint32_t u = win_u(b, cap);
         val = (int32_t)u - (int32_t)(q - 1);
@@ -975,7 +983,7 @@ __device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __re
     }
     const int32_t e_inc = min(e_carry, val);
     const uint32_t k_inc = k_carry + kept;
-    if (b + 1 < cnt) { tab[b + 1].E = e_inc; tab[b + 1].Kp = k_inc; }
+    if (b + 1 < cnt) put(b + 1, q, e_inc, k_inc);
     e_carry = __shfl_sync(0xffffffffu, e_inc, 31);
     k_carry = __shfl_sync(0xffffffffu, k_inc, 31);
   }
@@ -983,7 +991,7 @@ __device__ __forceinline__ uint32_t win_prefix_warp(uint32_t cap, WinEntry* __re
    * been decided: the last entry closes the queue (P = its length n), the running Kp counts the
    * kept requests under raw positions, and the running E is the minimum of u_t - t over the whole
    * queue, so that the admitted count behind the last request is n - 1 + min(E, 1). */
-  const uint32_t n_q = __ldcg(&tab[cnt - 1].P);
+  const uint32_t n_q = P_of(cnt - 1);
   return n_q == 0 ? 0u : (raw ? k_carry : (uint32_t)((int32_t)n_q - 1 + min(e_carry, 1)));
 }
 
@@ -2270,11 +2278,14 @@ k_kept_scan(const uint32_t* __restrict__ seg_kept, uint32_t n_seg, uint32_t* __r
  *     length of its kept prefix instead (win_off), by a warp's 32-ary search: its thresholds fall along
  *     the queue while the positions rise;
  *   - in the last block to finish, the output offsets of all queues' survivors.
- * Bound by dependent loads.  As four launches (boundaries, entries of short queues by a lane and of long
+ * Bound by dependent loads: the queue's constants are requested beside the boundaries, and P stays in shared memory until
+ * E and Kp are there (8,192 queues of 305 requests 36.3 -> 29.2 us, 256 of 4,096 16.5 -> 15.0; seven probes per step of the
+ * search instead of three: no gain).  As four launches (boundaries, entries of short queues by a lane and of long
  * ones by a warp each, prefixes, offsets) the same took 9 us more for 256 queues of 4,096 requests (a
  * replay epoch: 73 -> 64 us) and 12 more for 4,096 of them. */
 constexpr int kWinQueues = 16;
 constexpr int kWinThreads = 32 * kWinQueues;
+constexpr uint32_t kWinEntries = 4096;           /* entries of a block whose P stay in shared memory until E and Kp are there */
 __global__ void __launch_bounds__(kWinThreads, 2)
 k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
           uint32_t ibits, uint32_t n_seg, const PardSegConst* __restrict__ ktab, uint32_t* __restrict__ seg_off,
@@ -2287,9 +2298,10 @@ k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const u
   if (direct && hdr->direct) return;               /* (direct: the call may have its plan already) */
   __shared__ uint32_t s_lo[kWinQueues + 1], s_w[kWinQueues], s_first[kWinQueues + 1];
   __shared__ long long s_A[kWinQueues], s_d[kWinQueues];
-  __shared__ uint32_t s_base, s_scan;
+  __shared__ uint32_t s_base, s_scan, s_P[kWinEntries];
   const uint32_t tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
   const uint32_t s0 = blockIdx.x * kWinQueues, s = s0 + q;
+  const PardSegConst K = ktab[min(s, n_seg - 1)];  /* (requested beside the boundaries) */
   const bool usable = hdr->wide == 0 && hdr->aborted == 0 && n > 0;       /* else nothing was sorted */
   const uint32_t npass = hdr->npass, dbits = hdr->dbits;
   const unsigned long long* src = (npass & 1) ? buf_b : buf_a;
@@ -2351,7 +2363,6 @@ k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const u
   {
     uint32_t w = 0;
     if (mine) {                                    /* whole warps */
-      const PardSegConst K = ktab[s];
       if (K.narrow & kSegNoStage) {
         if (lane == 0) set_status(hdr, PARD_EDATA);   /* requests queued at a stage the pipeline lacks */
       } else if (K.narrow & kSegHighFirst) {
@@ -2418,11 +2429,14 @@ k_windows(PlanHeader* hdr, const unsigned long long* __restrict__ buf_a, const u
       else if (l1) { a = m1 + 1; b = m2; }
       else b = m1;
     }
-    wtab[base + e].P = a - first;
+    if (total <= kWinEntries) s_P[e] = a - first;
+    else wtab[base + e].P = a - first;
   }
   __syncthreads();
   if (total && mine && !high_first && s_w[q]) {
-    const uint32_t kept = win_prefix_warp(ktab[s].cap, wtab + base + s_first[q], s_w[q], lane, raw);
+    WinEntry* tab = wtab + base + s_first[q];
+    const uint32_t kept = total <= kWinEntries ? win_prefix_warp<true>(K.cap, tab, s_w[q], lane, raw, s_P + s_first[q])
+                                               : win_prefix_warp(K.cap, tab, s_w[q], lane, raw);
     if (lane == 0) seg_kept[s] = kept;             /* known before any request has been decided */
   }
   if (!last_block_done(&hdr->win_done)) return;

@@ -63,6 +63,26 @@ def test_groups_of_positions(sizes, m, mode):
     check(several_ctx(1, [sizes[0]], seed=m, S=5, m=m, span=100), mode)       # one ctx, many equal deadlines
 
 
+# ---- searched tables: entries of 16 queues in shared memory, or more than fit there --------------------
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
+@pytest.mark.parametrize("span", [2000, 5500, 9000, 40_000])                  # some 1,900 to 40,000 entries
+def test_searched_tables_of_sixteen_queues(span, mode):
+    for m in (1, 30):
+        check(several_ctx(5, [1900, 1700, 0, 3000, 2001], S=16, sort=False, mix=True, span=span, m=m), mode)
+
+
+# ---- mixed contexts: their ranges and orders in shared memory up to 1,024 of them ----------------------
+@pytest.mark.parametrize("n_ctx, S", [(2, 40), (1023, 3), (1024, 16), (1025, 3), (1024, 17)])
+def test_packing_of_mixed_contexts(n_ctx, S):
+    rng = np.random.default_rng(n_ctx + S)
+    sizes = np.bincount(rng.integers(0, n_ctx, size=30_001), minlength=n_ctx)
+    wl = several_ctx(n_ctx, sizes, S=S, sort=False, mix=True, m=3)
+    wl.requests["deadline_us"] += (wl.requests["ctx"].astype(np.int64) % 7) << 33     # far apart: low words alone tell contexts' origins
+    check(wl)
+    wl.state.priority = (rng.random((n_ctx, S)) < 0.4).astype(np.uint8)
+    check(wl)
+
+
 # ---- arrival order, one pass straight from the requests: up to 256 queues -------------------------
 @pytest.mark.parametrize("rule", [FCFS, NEXUS, FCFS | pb.PARD_MODE_PATH_MASK])
 @pytest.mark.parametrize("queues", [2, 4, 5, 255, 256, 257])
