@@ -732,6 +732,7 @@ __device__ __forceinline__ void count_digits(uint32_t* hist, uint32_t key, uint3
  * every request in range, low budget first, keys of one word, window tables within the shared counters
  * -- has a loop of its own that tests none of it per request (2^24 requests with window counts:
  * 98 -> 77 us). */
+constexpr uint32_t kPackCtx = 64;
 template <bool WIN>
 __global__ void __launch_bounds__(256)
 k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
@@ -749,6 +750,10 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
   __shared__ long long s_A[WIN ? kHistSegs : 1], s_d[WIN ? kHistSegs : 1];
   __shared__ unsigned long long s_magic[WIN ? kHistSegs : 1];
   __shared__ uint4 s_wcon[WIN ? kHistSegs : 1];            /* per queue: A_rel, first table entry, entries, A_rel and d fit 32 bits */
+  /* Few contexts: the low words of their smallest deadlines in shared memory (a replay's epochs, 16 contexts, 455 -> 451 us.
+   * 512 contexts with priorities, all in such tables: the kernel 20.7 -> 24.9). */
+  __shared__ uint32_t s_low[kPackCtx];
+  const bool table = n_ctx > 1 && n_ctx <= kPackCtx;
   if (hdr->wide || sort_is_local(hdr, local_candidate)) return;   /* sorted block by block: k_sort_local read the requests itself */
   const uint32_t npass = hdr->npass, dbits = hdr->dbits, pshift = hdr->pshift;
   for (uint32_t i = threadIdx.x; i < npass * kBins; i += blockDim.x) s_hist[i] = 0;
@@ -776,6 +781,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
       s_wcon[q] = make_uint4((uint32_t)narrow_A(K), win_off[q], win_cnt[q], (K.narrow & (kSegNarrow | kSegNoStage)) == kSegNarrow ? 1u : 0u);
     }
   }
+  if (table && threadIdx.x < n_ctx) s_low[threadIdx.x] = (uint32_t)~ctx_dmin_inv[threadIdx.x];
   bool plain = !hdr->bad_input && !priority && hdr->keybits + pshift <= 32 && dbits <= 29;
   if (WIN) plain = __syncthreads_and(plain && win_shared && all_narrow);
   else __syncthreads();
@@ -804,7 +810,9 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
         const uint32_t j = j0 + (uint32_t)u * stride;
         if (j >= n) break;
         const uint4 r = rr[u];
-        if (r.z != cur_ctx) {
+        if (table) {
+          low = s_low[r.z];
+        } else if (r.z != cur_ctx) {
           cur_ctx = r.z;
           low = (uint32_t)~ctx_dmin_inv[cur_ctx];
         }
