@@ -8,7 +8,8 @@
  *   pack      request -> one 64-bit sort element (segment | deadline | index), digit counts of the
  *             passes; with few queues also the counts behind the window tables
  *   sort      LSD radix sort, 8 bits per pass, one read and one write of the
- *             elements per pass (tile prefixes by decoupled look-back)
+ *             elements per pass (tile prefixes by decoupled look-back); in arrival order with up to 256
+ *             queues one pass straight from the requests, counted by the prepass (nothing is packed)
  *   windows   queue boundaries, batch-window tables, kept counts and output offsets (with few queues
  *             from the counts, beside the sort)
  *   decide    every request on its own from its queue's table: admitted position c, estimate, keep
@@ -3257,8 +3258,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
    * bits of the queue id: stage_stride a power of two. */
   const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
 
-  /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 239 us,
-   * 288 k of 24 contexts 71 -> 51.  Out of order the try costs 7 of 568 us, 2 of 71 (575 and 73; the tiles of the passes
+  /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 232 us,
+   * 288 k of 24 contexts 71 -> 51.  Out of order the try costs 12 of 568 us, 2 of 71 (575 and 73; the tiles of the passes
    * behind it on their way into L2 make that 544 and 74).  In order, but with a constant that the path does not take, 608 -> 609 and 70 -> 74.
    * The path itself would take any stride up to 16 (12 stages: 243 us, by the general sort 434); but the kernels of that sort would have to look,
    * ahead of their first loads, whether the plan is made, and every other call of theirs paid 0.7 us for it.  Without the
