@@ -49,13 +49,16 @@ constexpr unsigned long long kMixA = 0xBF58476D1CE4E5B9ull, kMixB = 0x94D049BB13
 __device__ __forceinline__ unsigned long long splitmix_fixed(uint32_t hi) {
   return (unsigned long long)((hi ^ (hi >> 30)) * (uint32_t)kMixA) << 32;
 }
-__device__ __forceinline__ uint32_t splitmix_hi(uint32_t lo, uint32_t hi, unsigned long long fixed) {
-  const uint32_t l = lo ^ __funnelshift_r(lo, hi, 30);
+/* the rest, from the low word after the first shift */
+__device__ __forceinline__ uint32_t splitmix_rest(uint32_t l, unsigned long long fixed) {
   unsigned long long z = (unsigned long long)l * (uint32_t)kMixA + fixed;
   z += (unsigned long long)(l * (uint32_t)(kMixA >> 32)) << 32;
   z = (z ^ (z >> 27)) * kMixB;
   const uint32_t h = (uint32_t)(z >> 32);
   return h ^ (h >> 31);
+}
+__device__ __forceinline__ uint32_t splitmix_hi(uint32_t lo, uint32_t hi, unsigned long long fixed) {
+  return splitmix_rest(lo ^ __funnelshift_r(lo, hi, 30), fixed);
 }
 
 __device__ __forceinline__ void copy_async_16(uint32_t smem, const void* g) {
@@ -131,6 +134,9 @@ k_estimate_w(const __grid_constant__ PipeTable pipes, const WaitArgs a) {
     uint32_t seen = 0;
     const unsigned long long x0 = a.seed + 0x9E3779B97F4A7C15ull + ((unsigned long long)c * a.R + slot) * M * 64ull;
     const bool same_hi = (uint32_t)x0 <= ~0u - (THREADS * PER + 1u) * 64u;       /* uniform */
+    /* nearly always the two top bits of the low words are the same too, all that the first shift takes from them: one shift
+     * per stage instead of one per draw (4,500 slots 450.5 -> 445.8 us) */
+    const bool same_top = same_hi && ((uint32_t)x0 >> 30) == (((uint32_t)x0 + (THREADS * PER + 1u) * 64u) >> 30);
     unsigned long long x = x0 + tid * 64ull;
 #pragma unroll 1
     for (uint32_t j = 0; j < len; ++j, ++x) {
@@ -148,6 +154,7 @@ k_estimate_w(const __grid_constant__ PipeTable pipes, const WaitArgs a) {
       const uint32_t* row = s_rows + (DOUBLE ? buf * row_words : 0u);
       const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
       const unsigned long long fixed = splitmix_fixed(hi);
+      const uint32_t shifted = __funnelshift_r(lo, hi, 30);
       auto draw = [&](int i) {
         const uint32_t step = (uint32_t)i * THREADS * 64u;
         if (same_hi) return row[__umulhi(splitmix_hi(lo + step, hi, fixed), M)];
@@ -157,10 +164,10 @@ k_estimate_w(const __grid_constant__ PipeTable pipes, const WaitArgs a) {
 #pragma unroll
       for (int i0 = 0; i0 < PER; i0 += kGroup) {
         if (i0 * THREADS >= (int)M) break;                   /* uniform */
-        if (same_hi && (i0 + kGroup) * THREADS <= (int)M) {  /* every lane has all of the group's samples */
+        if (same_top && (i0 + kGroup) * THREADS <= (int)M) {  /* every lane has all of the group's samples */
 #pragma unroll
           for (int i = i0; i < i0 + kGroup; ++i) {
-            const uint32_t v = row[__umulhi(splitmix_hi(lo + (uint32_t)i * THREADS * 64u, hi, fixed), M)];
+            const uint32_t v = row[__umulhi(splitmix_rest((lo + (uint32_t)i * THREADS * 64u) ^ shifted, fixed), M)];
             seen |= v;
             sum[i] += v;                                     /* < 64 * 2^24 = 2^30 when no value is bad */
           }

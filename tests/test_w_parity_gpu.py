@@ -45,6 +45,15 @@ def test_quantile_levels(num, den):
     compare(wl, samples, num, den, seed=2**64 - 5)
 
 
+@pytest.mark.parametrize("bit", [30, 31, 32])
+def test_counters_that_carry_inside_a_slot(bit):
+    """The draws' counters pass a multiple of 2^bit inside the first slot, just ahead of it, and behind it."""
+    wl = inputs.make("C5", n_inst=2, per_inst=16)
+    samples = inputs.draw_wait_samples(np.random.default_rng(bit), wl, 5000)
+    for before in (0, 1, 64 * 2500, 64 * 5000, 64 * 5200):
+        compare(wl, samples, 1, 10, seed=((1 << bit) - before - 0x9E3779B97F4A7C15) % 2**64)
+
+
 @pytest.mark.parametrize("M", [1, 2, 31, 255, 256, 257, 32768])
 def test_sample_counts(M):
     """Fewer samples than threads, exactly one round, and the largest allowed count."""
