@@ -201,7 +201,7 @@ typedef struct pard_plan_out {
                                      end in shared memory -- sort, window tables, decisions
                                      -- in three kernel launches, about twice as fast as
                                      without the promise (4,096 contexts of 8,192 requests:
-                                     0.36 ms against 0.70);
+                                     0.32 ms against 0.70);
                                    - larger contexts (and stage_stride a power of two):
                                      the radix passes stay inside every ctx's range and
                                      sort the stage and deadline bits only (the stage
