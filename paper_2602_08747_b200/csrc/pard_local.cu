@@ -471,6 +471,8 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
   }
   __syncthreads();
   if (Sm.use_scan) return false;
+  /* (The loops below move on by a request at least and look no further than a queue's table, so that they end whatever
+   * the arrays hold.) */
   /* the queue of position p, the last that begins at or before it */
   auto queue_at = [&](uint32_t p) {
     uint32_t k = 0, z = S;
@@ -501,7 +503,7 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
     uint32_t x = max(x0, lead);                          /* span after span of requests of one queue: mostly one */
     const uint32_t xe = min(x0 + kLocGroup, end);
     while (x < xe) {
-      const uint32_t k = queue_at(x - lead), lo = Sm.stage_first[k], stop = min(xe, lead + Sm.stage_first[k + 1]), r = x - lead - lo;
+      const uint32_t k = queue_at(x - lead), lo = Sm.stage_first[k], stop = max(min(xe, lead + Sm.stage_first[k + 1]), x + 1), r = x - lead - lo;
       const int32_t A = (int32_t)Sm.K[k].A_rel;
       const unsigned long long magic = Sm.K[k].d_magic;
       auto window = [&](uint32_t at) {                   /* -1: deadline before A */
@@ -632,8 +634,9 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
       const PardSegConst& K = Sm.K[k];
       const uint32_t r = r_less + i, cap = K.cap;
       uint32_t at = Sm.win_off[k] + (uint32_t)b;
-      for (; T.P[at + 1] <= r; ++at) ++b;                /* the window of request r */
-      uint32_t stop = min(T.P[at + 1] - r_less, rest);
+      const uint32_t end_mark = Sm.win_off[k] + Sm.win_cnt[k] - 1;
+      for (; at + 1 < end_mark && T.P[at + 1] <= r; ++at) ++b;       /* the window of request r */
+      uint32_t stop = max(min(T.P[at + 1] - r_less, rest), i + 1);
       int2 w = make_int2(0, 0);
       if (b >= 0) w = T.QU[at];
       uint32_t c0 = 0, left = 0, into = 0;               /* batch-slot position, kept ones of the span from here on, their place among the queue's */
