@@ -224,6 +224,25 @@ def test_errors_of_the_rules():
     check(inputs.make("C1"), FCFS)                              # the context still works
 
 
+# queues of every length side by side, most of them empty: a thread's eight requests cross several
+@pytest.mark.parametrize("mode", [FCFS, NEXUS, CLIPPER, MASK])
+@pytest.mark.parametrize("n_ctx", [64, 65, 700])                # of four stages: 256 queues (one digit), 260, 2,800
+@pytest.mark.parametrize("cap", [1, 3, 50])
+def test_outputs_across_short_and_empty_queues(n_ctx, mode, cap):
+    rng = np.random.default_rng(n_ctx + cap)
+    p = util.pipeline([(0, 1), (0, 2), (1, 3), (2, 3), (0, 3)], 4, [90, 150, 60, 40], bmax=64)
+    sizes = rng.choice([0, 0, 0, 1, 2, 5, 40, 900], size=n_ctx)
+    sizes[[1, n_ctx - 2]] = 9000, 1
+    ctx = rng.permutation(np.repeat(np.arange(n_ctx), sizes))
+    stage = np.where(rng.random(ctx.size) < 0.7, (ctx * 7) % 4, rng.integers(0, 4, size=ctx.size))
+    st = util.state(n_ctx, 4, inputs.n_slots(p), 1000, cap, q=rng.integers(0, 30, size=(n_ctx, 4)),
+                    w=rng.integers(0, 40, size=(n_ctx, inputs.n_slots(p))))
+    wl = inputs.Workload("short", [p], util.requests(900 + rng.integers(0, 4000, size=ctx.size), stage, ctx), st, n_ctx)
+    if mode == MASK:
+        draw_masks(wl, rng)
+    check(wl, mode, draw_arrivals(wl, rng) if mode == CLIPPER else None)
+
+
 # full sizes: one configuration per rule
 @pytest.mark.parametrize("name,mode", [("C3b", MASK), ("C3", FCFS), ("C4", NEXUS), ("C5", CLIPPER)])
 def test_rules_full_size(name, mode):
