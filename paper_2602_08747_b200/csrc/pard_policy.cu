@@ -740,11 +740,25 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   __shared__ uint32_t s_out[kPolThreads / 32][32 * kPolItems];
   if (MASK == kAllPaths && threadIdx.x == 0)       /* (the others have no registers left for it) */
     l2_ahead(v.src, INDEX ? tile0 / 2 : tile0, (uint64_t)kDecAhead * kPolTile / (INDEX ? 2 : 1), INDEX ? kPolTile / 2 : kPolTile, INDEX ? a.n / 2 : a.n);
-  if (MASK == kMaskStaged) stage_paths(a, v, tile0, sp);
+  /* Path sums worked out on the spot: 32 requests in a row to a warp for that, which mostly are of one queue or two.  (Only a
+   * tile's first queues are staged; eight in a row per thread leave all others to the last warps: a million requests in
+   * queues of 30 296 -> 314 us for the call.) */
+  __shared__ long long s_paths[MASK == kMaskStaged ? kPolTile : 1];
+  if (MASK == kMaskStaged) {
+    stage_paths(a, v, tile0, sp);
+#pragma unroll 1
+    for (uint32_t p = threadIdx.x; p < (uint32_t)kPolTile && tile0 + p < a.n; p += kPolThreads) {
+      const unsigned long long e = v.src[tile0 + p];
+      const uint32_t flags = __ldg(&reinterpret_cast<const uint32_t*>(&a.req[(uint32_t)e & v.imask])[3]) >> 16, seg = (uint32_t)(e >> v.kshift);
+      const PardSegConst& K = a.ktab[seg];
+      s_paths[p] = flags && !(K.narrow & kSegNoStage) ? masked_lsub(a, sp, seg, flags, K) - K.lsub : 0ll;
+    }
+    __syncthreads();
+  }
   uint32_t idx[kPolItems], t[kPolItems], my_seg = 0, last_seg = 0;
   long long est[kPolItems];                        /* at first: by how much the paths that a request names take it from the queue's estimate */
 #pragma unroll
-  for (int k = 0; k < kPolItems; ++k) est[k] = 0;
+  for (int k = 0; k < kPolItems; ++k) est[k] = MASK == kMaskStaged && j0 + k < a.n ? s_paths[threadIdx.x * kPolItems + k] : 0ll;
   if (INDEX) {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(v.src);
     if (full) {
@@ -767,7 +781,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
     for (int i = 0; i < kPolItems; ++i) idx[i] = (uint32_t)e[i] & v.imask;
     my_seg = (uint32_t)(e[0] >> v.kshift);
     last_seg = (uint32_t)(e[kPolItems - 1] >> v.kshift);
-    if (MASK) {
+    if (MASK == kMaskAtHand) {
       uint32_t flags[kPolItems];
 #pragma unroll
       for (int k = 0; k < kPolItems; ++k) flags[k] = j0 + k < a.n ? __ldg(&reinterpret_cast<const uint32_t*>(&a.req[idx[k]])[3]) >> 16 : 0u;
@@ -776,7 +790,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
         if (flags[k]) {
           const uint32_t seg = (uint32_t)(e[k] >> v.kshift);
           const PardSegConst& K = a.ktab[seg];
-          if (!(K.narrow & kSegNoStage)) est[k] = (MASK == kMaskAtHand ? masked_lsub_at_hand(a, seg, flags[k], K.lsub) : masked_lsub(a, sp, seg, flags[k], K)) - K.lsub;
+          if (!(K.narrow & kSegNoStage)) est[k] = masked_lsub_at_hand(a, seg, flags[k], K.lsub) - K.lsub;
         }
     }
   }

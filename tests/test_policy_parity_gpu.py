@@ -243,6 +243,23 @@ def test_outputs_across_short_and_empty_queues(n_ctx, mode, cap):
     check(wl, mode, draw_arrivals(wl, rng) if mode == CLIPPER else None)
 
 
+# known paths in queues too short for their path sums to be at hand: a block has those of its tile's first 16 queues
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 9000])
+@pytest.mark.parametrize("per", [1, 20, 31])                    # requests per queue on average
+def test_known_paths_in_short_queues(n, per):
+    rng = np.random.default_rng(n + per)
+    p = inputs.make_pipeline(inputs.DAG8_EDGES, 8, [4] * 8, [rng.integers(5, 60, size=4) for _ in range(8)])
+    n_ctx = max(1, n // (8 * per))
+    st = util.state(n_ctx, 9, inputs.n_slots(p), 1000, 2, q=rng.integers(0, 30, size=(n_ctx, 9)),       # (a stage that the pipeline lacks)
+                    w=rng.integers(0, 400, size=(n_ctx, inputs.n_slots(p))))
+    st.batch[:, 8] = 1
+    wl = inputs.Workload("paths", [p], util.requests(900 + rng.integers(0, 900, size=n), rng.integers(0, 8, size=n), rng.integers(0, n_ctx, size=n)),
+                         st, n_ctx)
+    draw_masks(wl, rng)
+    check(wl, MASK)
+    check(wl, MASK | FCFS)
+
+
 # full sizes: one configuration per rule
 @pytest.mark.parametrize("name,mode", [("C3b", MASK), ("C3", FCFS), ("C4", NEXUS), ("C5", CLIPPER)])
 def test_rules_full_size(name, mode):
