@@ -736,7 +736,9 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
   const SortedView v = sorted_view(a);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t tile0 = blockIdx.x * kPolTile, j0 = tile0 + threadIdx.x * kPolItems;
-  const bool nexus = !MASK && (a.mode & PARD_MODE_NEXUS), full = j0 + kPolItems <= a.n;     /* (known paths do not combine with it, raw positions with no rule) */
+  const bool nexus = !MASK && (a.mode & PARD_MODE_NEXUS), full = j0 + kPolItems <= a.n;     /* (known paths do not combine with it) */
+  /* raw positions: no rule takes them, but the planner's own comes here too when its key is wider than an element */
+  const bool raw = !MASK && !INDEX && (a.mode & PARD_MODE_RAW);
   __shared__ uint32_t s_out[kPolThreads / 32][32 * kPolItems];
   if (MASK == kAllPaths && threadIdx.x == 0)       /* (the others have no registers left for it) */
     l2_ahead(v.src, INDEX ? tile0 / 2 : tile0, (uint64_t)kDecAhead * kPolTile / (INDEX ? 2 : 1), INDEX ? kPolTile / 2 : kPolTile, INDEX ? a.n / 2 : a.n);
@@ -828,7 +830,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
     return from;
   };
   uint32_t b0 = 0;
-  if (p0 < a.n) {
+  if (!raw && p0 < a.n) {
     const uint32_t* ends = v.C + a.seg_off[seg_first];
     uint32_t z = a.rounds[seg_first];
     while (b0 < z) {                               /* uniform across the warp */
@@ -853,7 +855,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
       const PardSegConst& K = a.ktab[my_seg];
       lo = a.seg_off[my_seg];
       hi = a.seg_off[my_seg + 1];
-      nb = a.rounds[my_seg];
+      nb = raw ? 0u : a.rounds[my_seg];
       cap = K.cap;
       none = K.narrow & kSegNoStage;
       tail = nexus ? a.tail[my_seg] : 0u;
@@ -862,7 +864,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
       if (!MASK && !none && (a.mode & (PARD_MODE_NEXUS | PARD_MODE_CLIPPER))) A0 -= K.lsub;     /* the current module only */
       if (nexus && a.out_kept_idx) place = a.kept_base[my_seg];
       b = 0;                                       /* (a queue that begins inside the thread's share: its first round) */
-      if (i == 0) {
+      if (i == 0 && !raw) {
         if (my_seg == seg_first) b = b0;
         const uint32_t on = j - max(lo, p0);
         uint32_t z = min(nb, b + (K.cap_magic ? div_magic32(on, K.cap_magic) : on) + 1);     /* ends b .. z-1: how many are <= j */
@@ -875,7 +877,12 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
       ++b;                                         /* (no round is empty) */
     }
     const uint32_t end = b < nb ? v.C[lo + b] : 0xffffffffu;
-    const uint32_t stop = max(min(min(end, hi) - j0, count), i + 1);     /* (i + 1: the loop ends whatever the arrays hold) */
+    uint32_t stop = max(min(min(end, hi) - j0, count), i + 1);           /* (i + 1: the loop ends whatever the arrays hold) */
+    if (raw) {
+      const unsigned long long magic = a.ktab[my_seg].cap_magic;
+      b = magic ? div_magic32(j - lo, magic) : j - lo;
+      stop = i + 1;
+    }
     const long long now = A0 + (long long)b * d;
     const uint32_t from = b < nb ? end - cap : hi - tail;      /* Nexus: the window's first request */
     uint32_t kept = 0;
