@@ -483,7 +483,6 @@ struct PolicyArgs {
   uint32_t n_pipelines;
   pard_queue_state_t st;
   uint32_t* rounds;               /* [n_seg] batch rounds the walk has closed */
-  uint32_t rounds_there;          /* the sort has written every request's rounds (k_sort_requests) */
   uint32_t* tail;                 /* [n_seg] Nexus: requests of the last, partly filled window */
   uint32_t* tile_x;               /* [tiles of kDecTile] kept requests ahead of the tile's first one, in its queue */
   uint8_t* out_keep;
@@ -493,6 +492,7 @@ struct PolicyArgs {
   const long long* path_sums;     /* [n_seg][kMaskPaths] Eq. 3 along every path a request can name, -1: no such path; or null */
   const uint32_t* kept_base;      /* [n_seg] output offset of every queue's survivors, known after the walk */
   uint32_t* seg_kept;
+  uint32_t rounds_there;          /* the sort has written every request's rounds (k_sort_requests) */
 };
 int allow_walk_smem();             /* once per device, by the planner's set-up */
 /* thresholds and walk: every queue's rounds and kept count (seg_kept) */
