@@ -436,7 +436,7 @@ __device__ __forceinline__ bool split_fits(const LocalArgs& a, const LocalSmem& 
  * whose neighbour ahead and whose last request are in one window is done with two divisions; along a window the
  * admitted position rises by one per request up to u, c = min(r + q, u) with q = min(E, 1) - 1 (at the window's first
  * request too: E is at most the u before less the requests ahead), so its survivors are the window's first ones and a
- * group's estimates are at most two when a batch round takes eight.  (Every request on its own, 32 in a row to a warp: 218
+ * group's estimates are at most two when a batch round takes eight, for raw positions (c = r) too.  (Every request on its own, 32 in a row to a warp: 218
  * instructions per request for 4,096 contexts of 8,192, 175 like this with the sort below; calls 354 -> 314 us, 2,000 of 4,000
  * 155 -> 138, one of 7,800 31.5 -> 28.5.)  Up to kLocOneByOne requests a group per thread would leave most warps idle, and
  * every request goes on its own: by groups ten contexts of 730 took 31.8 us and 600 of 256 34.7, like this 29.4 and 30.4
@@ -641,22 +641,34 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
       if (b >= 0) w = T.QU[at];
       uint32_t c0 = 0, left = 0, into = 0;               /* batch-slot position, kept ones of the span from here on, their place among the queue's */
       if (RAW) {
-        stop = i + 1;
         c0 = r;
-        left = b >= 0 && r < (uint32_t)w.y ? 1u : 0u;
-        into = left ? (uint32_t)w.x + r - T.P[at] : 0u;
+        if (b >= 0 && r < (uint32_t)w.y) {
+          left = (uint32_t)w.y - r;
+          into = (uint32_t)w.x + r - T.P[at];
+        }
       } else if (b >= 0) {
         c0 = into = min((uint32_t)((int32_t)r + w.x), (uint32_t)w.y);
         left = (uint32_t)w.y - c0;
       }
-      const uint32_t round = cap > 1 ? div_magic32(c0, K.cap_magic) : c0, fresh = cap - (c0 - round * cap);   /* requests up to the next round */
-      if (cap < kLocGroup && left) stop = min(stop, i + fresh);       /* small rounds: one at a time */
-      const uint32_t next = fresh <= left ? i + fresh : (uint32_t)kLocGroup;
-      const long long e0 = K.A + (long long)((unsigned long long)round * (uint32_t)K.d), e1 = e0 + K.d;      /* d fits 32 bits: it has a magic number */
+      const long long A = K.A;
+      const uint32_t d = (uint32_t)K.d;                  /* d fits 32 bits: it has a magic number */
+      const unsigned long long magic = K.cap_magic;
+      if (cap >= kLocGroup) {
+        const uint32_t round = div_magic32(c0, magic), fresh = cap - (c0 - round * cap);     /* requests up to the next round */
+        const uint32_t next = RAW || fresh <= left ? i + fresh : (uint32_t)kLocGroup;
+        const long long e0 = A + (long long)((unsigned long long)round * d), e1 = e0 + d;
 #pragma unroll
-      for (int q = 0; q < kLocGroup; ++q) {              /* (what lies behind the span is made good by the next one) */
-        if (q >= (int)i) est[q] = e0;
-        if (q >= (int)next) est[q] = e1;
+        for (int q = 0; q < kLocGroup; ++q) {            /* (what lies behind the span is made good by the next one) */
+          if (q >= (int)i) est[q] = e0;
+          if (q >= (int)next) est[q] = e1;
+        }
+      } else {                                           /* small rounds */
+#pragma unroll
+        for (int q = 0; q < kLocGroup; ++q)
+          if (q >= (int)i) {
+            const uint32_t c = RAW ? c0 + (q - i) : min(c0 + (q - i), c0 + left);
+            est[q] = A + (long long)((unsigned long long)(cap > 1 ? div_magic32(c, magic) : c) * d);
+          }
       }
       const uint32_t n_kept = min(stop - i, left);
       if (!keepbits) list = Sm.kept_base[k] + into;

@@ -63,6 +63,14 @@ def test_groups_of_positions(sizes, m, mode):
     check(several_ctx(1, [sizes[0]], seed=m, S=5, m=m, span=100), mode)       # one ctx, many equal deadlines
 
 
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
+@pytest.mark.parametrize("cap", [1, 3, 7, 8, 9, 15, 16])                      # a group's estimates one by one, or two of them
+def test_groups_of_positions_across_batch_rounds(cap, mode):
+    for sizes, S, span in (([2500, 8192, 1, 4099, 2049], 3, 6000), ([8191, 3001], 10, 300), ([2053] * 9, 1, 40_000)):
+        for sort in (True, False):
+            check(several_ctx(len(sizes), sizes, seed=cap, S=S, sort=sort, span=span, B=cap), mode | pb.PARD_MODE_GROUPED)
+
+
 # ---- searched tables: entries of 16 queues in shared memory, or more than fit there --------------------
 @pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
 @pytest.mark.parametrize("span", [2000, 5500, 9000, 40_000])                  # some 1,900 to 40,000 entries
