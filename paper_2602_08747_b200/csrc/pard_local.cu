@@ -49,7 +49,8 @@ struct Tables {                                          /* 4. to 6., in the roo
  * 32 stages.  The elements fall apart into arrays, queue after queue; position p stands at p + lead, lead = the ctx's first
  * request modulo 8, so that a thread's groups of eight are those of the output. */
 constexpr int kLocGroup = 8;
-constexpr uint32_t kLocOneByOne = 768;                   /* see finish_split */
+constexpr int32_t kFewWindows = 4;                       /* of a group, by eight comparisons each; more: request after request */
+constexpr uint32_t kLocOneByOne = 1024;                  /* see finish_split */
 struct Split {
   uint32_t off[kLocalTile + kLocGroup];                  /* deadline offsets */
   uint16_t idx[kLocalTile + kLocGroup];                  /* index inside the ctx */
@@ -436,12 +437,17 @@ __device__ __forceinline__ bool split_fits(const LocalArgs& a, const LocalSmem& 
  * whose neighbour ahead and whose last request are in one window is done with two divisions; along a window the
  * admitted position rises by one per request up to u, c = min(r + q, u) with q = min(E, 1) - 1 (at the window's first
  * request too: E is at most the u before less the requests ahead), so its survivors are the window's first ones and a
- * group's estimates are at most two when a batch round takes eight, for raw positions (c = r) too.  (Every request on its own, 32 in a row to a warp: 218
- * instructions per request for 4,096 contexts of 8,192, 175 like this with the sort below; calls 354 -> 314 us, 2,000 of 4,000
- * 155 -> 138, one of 7,800 31.5 -> 28.5.)  Up to kLocOneByOne requests a group per thread would leave most warps idle, and
- * every request goes on its own: by groups ten contexts of 730 took 31.8 us and 600 of 256 34.7, like this 29.4 and 30.4
- * (as before: 29.4 and 32.4); 1,000 of 1,000 are faster by groups, 54.4 -> 48.9.  False: more windows than the tables
- * hold, nothing has been written. */
+ * group's estimates are at most two when a batch round takes eight, for raw positions (c = r) too.  (Every request on its
+ * own, 32 in a row to a warp: 218 instructions per request for 4,096 contexts of 8,192, 175 like this with the sort below;
+ * calls 362 -> 321 us, raw positions 360 -> 318, rounds of one request 385 -> 334.)
+ * The tables' P begin as zeros, written by all threads: a queue whose first request lies many windows on, as after a
+ * pause or with rounds of a few requests, has its first windows done.  (By the thread of that request, eight comparisons
+ * for each: 2,000 contexts of 1,000 requests in rounds of one 122 us, every request on its own 109, like this 94.)
+ * Every request goes on its own where groups would leave most warps idle: up to kLocOneByOne requests, and up to twice as
+ * many where a group meets more than a window on average (3,000 contexts of 800 in rounds of one, two objectives:
+ * groups 227 us, like this 214; 2,000 of 1,500 173 and 166, by default rounds 161 as groups, 163 one by one) or there is one
+ * ctx (less code to fetch when its caller's other work has taken the L2: 2,000 requests 39.9 -> 36.0 us; 4,000 would take
+ * 33.7 instead of 30.8 with the code at hand).  False: more windows than the tables hold, nothing has been written. */
 template <bool RAW>
 __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const LocalArgs& a, LocalSmem& Sm, uint32_t c, uint32_t first, uint32_t cnt) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -465,12 +471,14 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
     if (lane < S) {
       Sm.win_off[lane] = x - w;
       Sm.win_cnt[lane] = w;
-      if (w && x <= kTabEntries) T.P[x - 1] = Sm.stage_first[lane + 1] - Sm.stage_first[lane];   /* the end marker */
     }
     if (lane == 31) Sm.use_scan = x > kTabEntries ? 1u : 0u;
+  } else {                                               /* no request ahead of a window: what holds up to a queue's first one */
+    for (uint32_t e = tid - 32; e < kTabEntries / 4; e += kLocThreads - 32) reinterpret_cast<uint4*>(T.P)[e] = make_uint4(0u, 0u, 0u, 0u);
   }
   __syncthreads();
   if (Sm.use_scan) return false;
+  if (tid < S && Sm.win_cnt[tid]) T.P[Sm.win_off[tid] + Sm.win_cnt[tid] - 1] = Sm.stage_first[tid + 1] - Sm.stage_first[tid];   /* the end marker */
   /* (The loops below move on by a request at least and look no further than a queue's table, so that they end whatever
    * the arrays hold.) */
   /* the queue of position p, the last that begins at or before it */
@@ -483,14 +491,14 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
     return k;
   };
   const uint32_t end = lead + cnt, groups = cnt ? (end + kLocGroup - 1) / kLocGroup : 0u;   /* (an empty ctx: none) */
-  const bool one_by_one = cnt <= kLocOneByOne;
+  const bool one_by_one = cnt <= kLocOneByOne || (cnt <= 2 * kLocOneByOne && (a.n_ctx == 1 || Sm.win_off[S - 1] + Sm.win_cnt[S - 1] > groups));
   if (one_by_one)
     for (uint32_t p = tid; p < cnt; p += kLocThreads) {
       const uint32_t k = queue_at(p), r = p - Sm.stage_first[k];
       const int32_t off = (int32_t)T.off[lead + p], A = (int32_t)Sm.K[k].A_rel;
       const unsigned long long magic = Sm.K[k].d_magic;
       const int32_t b = off < A ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)A, magic);
-      int32_t e = -1;
+      int32_t e = b;                                     /* (up to a queue's first request: no request ahead) */
       if (r) {
         const int32_t before = (int32_t)T.off[lead + p - 1];
         e = before < A ? -1 : (int32_t)div_magic32((uint32_t)before - (uint32_t)A, magic);
@@ -506,12 +514,17 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
       const uint32_t k = queue_at(x - lead), lo = Sm.stage_first[k], stop = max(min(xe, lead + Sm.stage_first[k + 1]), x + 1), r = x - lead - lo;
       const int32_t A = (int32_t)Sm.K[k].A_rel;
       const unsigned long long magic = Sm.K[k].d_magic;
+      uint32_t* P = T.P + Sm.win_off[k];
       auto window = [&](uint32_t at) {                   /* -1: deadline before A */
         const int32_t off = (int32_t)T.off[at];
         return off < A ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)A, magic);
       };
-      const int32_t ahead = r ? window(x - 1) : -1, last = window(stop - 1);
-      if (ahead < last) {                                /* windows begin here: their P, the requests before them */
+      const int32_t ahead = window(r ? x - 1 : x), last = window(stop - 1);
+      if (last - ahead > kFewWindows) {                  /* windows begin here: their P, the requests before them */
+        int32_t e = ahead;
+        for (uint32_t y = x; y < stop; ++y)
+          for (const int32_t b = window(y); e < b;) P[++e] = y - lead - lo;
+      } else if (ahead < last) {
         const uint32_t d = (uint32_t)Sm.K[k].d;
         uint32_t X[kLocGroup];                           /* deadline - A, expired: 0 (window 0 begins at the first that is not) */
         uint32_t expired = 0;
@@ -524,7 +537,6 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
           X[i] = !in ? 0xffffffffu : late ? 0u : off[i] - (uint32_t)A;
           expired += in && late ? 1u : 0u;
         }
-        uint32_t* P = T.P + Sm.win_off[k];
         for (int32_t e = ahead + 1; e <= last; ++e) {
           const uint32_t from = (uint32_t)e * d;         /* <= the last request's deadline - A */
           uint32_t below = 0;
@@ -622,21 +634,18 @@ __device__ __forceinline__ bool finish_split(PlanHeader* __restrict__ hdr, const
     long long est[kLocGroup];
 #pragma unroll
     for (int q = 0; q < kLocGroup; ++q) est[q] = 0;
-    int32_t b = 0;
     for (uint32_t i = xa - x0; i < xe - x0;) {           /* span after span of one queue and window: mostly one */
       if (i >= rest) {                                   /* a queue begins, or the group does */
         k = queue_at(x0 + i - lead);
         r_less = x0 - lead - Sm.stage_first[k];
         rest = min(lead + Sm.stage_first[k + 1], xe) - x0;
-        const int32_t off = (int32_t)T.off[x0 + i], A = (int32_t)Sm.K[k].A_rel;
-        b = off < A ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)A, Sm.K[k].d_magic);
       }
       const PardSegConst& K = Sm.K[k];
       const uint32_t r = r_less + i, cap = K.cap;
-      uint32_t at = Sm.win_off[k] + (uint32_t)b;
-      const uint32_t end_mark = Sm.win_off[k] + Sm.win_cnt[k] - 1;
-      for (; at + 1 < end_mark && T.P[at + 1] <= r; ++at) ++b;       /* the window of request r */
-      uint32_t stop = max(min(T.P[at + 1] - r_less, rest), i + 1);
+      const int32_t off = (int32_t)T.off[x0 + i], first_off = (int32_t)K.A_rel;
+      const int32_t b = off < first_off ? -1 : (int32_t)div_magic32((uint32_t)off - (uint32_t)first_off, K.d_magic);
+      const uint32_t at = Sm.win_off[k] + (uint32_t)b;
+      const uint32_t stop = max(min(T.P[at + 1] - r_less, rest), i + 1);
       int2 w = make_int2(0, 0);
       if (b >= 0) w = T.QU[at];
       uint32_t c0 = 0, left = 0, into = 0;               /* batch-slot position, kept ones of the span from here on, their place among the queue's */

@@ -71,6 +71,19 @@ def test_groups_of_positions_across_batch_rounds(cap, mode):
             check(several_ctx(len(sizes), sizes, seed=cap, S=S, sort=sort, span=span, B=cap), mode | pb.PARD_MODE_GROUPED)
 
 
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
+@pytest.mark.parametrize("sizes", [[1023, 1024, 1025, 1], [2047, 2048, 2049, 0, 7], [1500] * 9, [8192, 8191, 3000], [1024], [1025], [2048], [2049]])
+def test_windows_without_requests(sizes, mode):
+    rng = np.random.default_rng(sum(sizes))
+    for S, gap, expired in ((3, 0, 0.2), (3, 900, 0.0), (3, 900, 0.2), (8, 1500, 0.01), (3, 20_000, 0.1)):     # the last: more windows than the tables hold
+        wl = several_ctx(len(sizes), sizes, seed=S, S=S, sort=False, span=3, m=2)
+        kind = rng.random(wl.n)
+        wl.requests["deadline_us"] += np.where(kind < expired, -900, np.where(kind < 0.6, gap, gap * 4 // 3 + 60))
+        check(wl, mode | pb.PARD_MODE_GROUPED)                                # sorted by the block
+        wl.requests = wl.requests[np.lexsort((wl.requests["deadline_us"], wl.requests["ctx"]))]
+        check(wl, mode | pb.PARD_MODE_GROUPED)                                # in order
+
+
 # ---- searched tables: entries of 16 queues in shared memory, or more than fit there --------------------
 @pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
 @pytest.mark.parametrize("span", [2000, 5500, 9000, 40_000])                  # some 1,900 to 40,000 entries
