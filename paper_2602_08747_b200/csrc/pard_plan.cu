@@ -2701,9 +2701,13 @@ k_decide_win(const PlanHeader* __restrict__ hdr, const unsigned long long* __res
   if (hdr->direct | hdr->use_scan | hdr->wide | hdr->aborted) return;
   decide_tile<RAW, HF>(blockIdx.x, hdr, buf_a, buf_b, n, ibits, ktab, seg_off, win_off, win_cnt, wtab, out_keep, out_est, out_perm, out_kept_idx, kept_base);
 }
-/* For calls that mostly have their plan by then (pard_direct.cuh): a few blocks that take one tile after the other.  A
- * block per tile, 16,384 at 2^24 requests, took 11 us to find that there is nothing to do. */
-__global__ void __launch_bounds__(kDecThreads, 7)
+/* For calls that mostly have their plan by then (pard_direct.cuh): fewer blocks, which take one tile after the other.  A
+ * block per tile, 16,384 at 2^24 requests, took 11 us to find that there is nothing to do; a block that goes on to a next
+ * tile decides a little slower than a new one.  Five rounds of the seven blocks that fit a multiprocessor: 2^24 requests of 64
+ * contexts out of order 537.6 us with a block per tile, 542.5 with four rounds, 539.7 like this, of 256 contexts 545.7, 545,
+ * 545; those in order 244.8, 233.2, 233.7. */
+constexpr uint32_t kRestBlocks = 7, kRestRounds = 5;
+__global__ void __launch_bounds__(kDecThreads, kRestBlocks)
 k_decide_rest(const PlanHeader* __restrict__ hdr, const unsigned long long* __restrict__ buf_a, const unsigned long long* __restrict__ buf_b, uint32_t n,
               uint32_t ibits, const PardSegConst* __restrict__ ktab, const uint32_t* __restrict__ seg_off, const uint32_t* __restrict__ win_off,
               const uint32_t* __restrict__ win_cnt, const WinEntry* __restrict__ wtab, uint8_t* __restrict__ out_keep,
@@ -3259,8 +3263,8 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
   const bool ctx_sort = (mode & PARD_MODE_GROUPED) && L.ctx_passes && (S & (S - 1)) == 0 && !rule_walk && n > 0;
 
   /* ---- such requests may stand in order already: planned without a sort if they do (pard_direct.cuh).  2^24 requests of 256 contexts in order 345 -> 232 us,
-   * 288 k of 24 contexts 71 -> 51.  Out of order the try costs 12 of 568 us, 2 of 71 (575 and 73; the tiles of the passes
-   * behind it on their way into L2 make that 544 and 74).  In order, but with a constant that the path does not take, 608 -> 609 and 70 -> 74.
+   * 288 k of 24 contexts 71 -> 51.  Out of order the try cost 7 of 568 us, 2 of 71; the tiles of the passes behind it on
+   * their way into L2 brought that to 544 and 74, at which it stands (k_decide_rest).  In order, but with a constant that the path does not take, 608 -> 609 and 70 -> 74.
    * The path itself would take any stride up to 16 (12 stages: 243 us, by the general sort 434); but the kernels of that sort would have to look,
    * ahead of their first loads, whether the plan is made, and every other call of theirs paid 0.7 us for it.  Without the
    * caller's word a call would pay 8 to 11 us, of 85 to 210, for finding out that its contexts come mixed. ---- */
@@ -3402,7 +3406,7 @@ extern "C" int pard_plan_policy(const pard_pipeline_t* const* pipelines, uint32_
                           : (state->d_priority ? k_decide_win<false, true> : k_decide_win<false, false>);
     /* the survivors go straight to their place in the output */
     if (direct)
-      launch_pdl(k_decide_rest, std::min<uint32_t>(win_grid, 28u * (uint32_t)sms), kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off,
+      launch_pdl(k_decide_rest, std::min<uint32_t>(win_grid, kRestRounds * kRestBlocks * (uint32_t)sms), kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off,
                  win_off, win_cnt, wtab, out->d_keep, est, out->d_perm, out->d_kept_idx, (const uint32_t*)kept_base);
     else
       launch_pdl(decide_win, win_grid, kDecThreads, 0, stream, hdr, buf_a, buf_b, n32, ibits, ktab, seg_off, win_off, win_cnt, wtab,

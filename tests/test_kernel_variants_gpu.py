@@ -293,6 +293,14 @@ def test_requests_out_of_place_while_blocks_start(n_ctx, per, at):
     check(wl, pb.PARD_MODE_GROUPED)
 
 
+# ---- out of order although grouped, decided by blocks that take one tile after the other: more tiles than blocks ------
+@pytest.mark.parametrize("n", [5_304_320, 5_304_321, 6_500_001])           # 5,180 tiles of 1,024 on 148 multiprocessors, and more
+def test_decision_behind_a_try_that_found_no_order(n):
+    sizes = np.full(24, n // 24)
+    sizes[7] += n - sizes.sum()
+    check(several_ctx(24, sizes, S=4, sort=False, span=60_000, m=300), pb.PARD_MODE_GROUPED)
+
+
 # ---- keys beyond 64 bits: a wait of the chunks' passes runs out, and nothing follows the half-sorted positions ------
 @pytest.mark.parametrize("n", [1500, 10_000])                            # one tile, several
 def test_wide_key_stops_behind_a_wait_that_ran_out(n):
