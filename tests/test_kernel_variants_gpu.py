@@ -92,6 +92,43 @@ def test_searched_tables_of_sixteen_queues(span, mode):
         check(several_ctx(5, [1900, 1700, 0, 3000, 2001], S=16, sort=False, mix=True, span=span, m=m), mode)
 
 
+def table_entries(wl, want):
+    """Window-table entries of every queue: an end marker, and a window up to the last request's.  A queue's first request
+    is estimated at A."""
+    d = np.array([wl.pipelines[0].lat_us[o] for o in wl.pipelines[0].lat_offsets[:wl.state.stage_stride]])
+    off, dl = want["seg_offsets"], wl.requests["deadline_us"][want["perm"]]
+    out = np.zeros(off.size - 1, np.int64)
+    for q in np.flatnonzero(np.diff(off)):
+        X = int(dl[off[q]:off[q + 1]].max()) - int(want["est_us"][off[q]])
+        out[q] = 1 if X < 0 else X // d[q % d.size] + 2
+    return out
+
+
+@pytest.mark.parametrize("mode", [0, pb.PARD_MODE_RAW])
+@pytest.mark.parametrize("lo, hi", [(1500, 2500), (3850, 4096), (4097, 4350), (5500, 6500)])      # entries of a block's 16 queues; 4,096 fit
+def test_searched_tables_within_the_workspace(lo, hi, mode):
+    n_ctx, S, n = 5, 16, 900_000
+    sizes = [200_000, 150_000, 0, 249_000, 301_000]
+    for m in (1, 300):
+        wl = several_ctx(n_ctx, sizes, S=S, sort=False, mix=True, span=1, m=m)
+        d = wl.pipelines[0].lat_us[wl.pipelines[0].lat_offsets[:S]]
+        want = oracle.plan(wl.pipelines, wl.requests, wl.state, n_ctx, mode)
+        start = want["est_us"][want["seg_offsets"][:S]]                       # A of the first ctx's queues
+        last = int(((lo + hi) / 2 - 1.5 * S + (start / d).sum()) / (1.0 / d).sum())
+        wl.requests["deadline_us"] = np.random.default_rng(m).integers(1000, last + 1, size=n)
+        want = oracle.plan(wl.pipelines, wl.requests, wl.state, n_ctx, mode)
+        entries = table_entries(wl, want)
+        blocks = entries.reshape(-1, 16).sum(axis=1)
+        assert entries.sum() <= n // 32 + 4 * n_ctx * S + 1024                # all fit: nothing is left to the scan
+        assert ((lo <= blocks[[0, 1, 3, 4]]) & (blocks[[0, 1, 3, 4]] <= hi)).all(), blocks
+        rc, got = run_library(wl, mode)
+        assert rc == 0
+        assert_identical(got, want)
+        wl.state.priority = np.zeros((n_ctx, S), np.uint8)                    # some queues without a table between the others
+        wl.state.priority[:, ::3] = 1
+        check(wl, mode)
+
+
 # ---- mixed contexts: the origins of up to 64 in shared memory ------------------------------------------
 @pytest.mark.parametrize("n_ctx, S", [(2, 20), (2, 40), (63, 1), (64, 1), (64, 3), (65, 3)])
 def test_packing_of_mixed_contexts(n_ctx, S):
