@@ -141,6 +141,19 @@ def test_packing_of_mixed_contexts(n_ctx, S):
     check(wl)
 
 
+@pytest.mark.parametrize("n_ctx, S", [(2, 20), (2, 40), (63, 1), (64, 1), (64, 3), (65, 3)])
+def test_packing_of_mixed_contexts_far_apart(n_ctx, S):
+    """Contexts whose clocks are far apart, each booked close to its own: every queue's constants stay short."""
+    rng = np.random.default_rng(n_ctx + S)
+    sizes = np.bincount(rng.integers(0, n_ctx, size=20_001 + 70 * n_ctx), minlength=n_ctx)
+    wl = several_ctx(n_ctx, sizes, S=S, sort=False, mix=True, m=3)
+    apart = ((np.arange(n_ctx, dtype=np.int64) * 5) % 7 << 33) + np.arange(n_ctx) * 1_000_003
+    wl.requests["deadline_us"] += apart[wl.requests["ctx"]]
+    wl.state.now_us += apart
+    for mode in (0, pb.PARD_MODE_RAW):
+        check(wl, mode)
+
+
 # ---- arrival order, one pass straight from the requests: up to 256 queues -------------------------
 @pytest.mark.parametrize("rule", [FCFS, NEXUS, FCFS | pb.PARD_MODE_PATH_MASK])
 @pytest.mark.parametrize("queues", [2, 4, 5, 255, 256, 257])
