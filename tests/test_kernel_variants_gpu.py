@@ -166,6 +166,56 @@ def test_arrival_order_from_the_requests(rule, queues, n):
         check(wl, rule)
 
 
+@pytest.mark.parametrize("rule", [FCFS, NEXUS, FCFS | pb.PARD_MODE_PATH_MASK])
+@pytest.mark.parametrize("n_ctx, S", [(1, 2), (85, 3), (64, 4), (32, 8), (8, 32), (4, 64)])       # 2, 255, 256 queues
+@pytest.mark.parametrize("n", [8193, 24_576, 60_001])
+def test_arrival_order_from_the_requests_of_several_stages(rule, n_ctx, S, n):
+    rng = np.random.default_rng(n + S)
+    sizes = np.bincount(rng.integers(0, n_ctx, size=n), minlength=n_ctx)
+    for far in (0, 1 << 57):                               # the last: offsets beyond the elements, looked up
+        wl = several_ctx(n_ctx, sizes, seed=n, S=S, sort=False, mix=True, m=1 + n % 3, span=40 * S + 3000)
+        wl.requests["deadline_us"][::7] += far
+        if rule & pb.PARD_MODE_PATH_MASK:                  # every stage but the last has one path
+            wl.requests["flags"] = np.where(wl.requests["stage"] + 1 < S, rng.integers(0, 2, size=n), 0)
+        check(wl, rule)
+
+
+@pytest.mark.parametrize("rule", [FCFS, NEXUS, FCFS | pb.PARD_MODE_PATH_MASK, pb.PARD_MODE_CLIPPER])
+@pytest.mark.parametrize("n, n_ctx", [(20_000, 2), (20_000, 64), (2_800_000, 64)])                # small tiles, wide ones
+def test_errors_found_while_sorting_in_arrival_order(rule, n, n_ctx):
+    """A request out of range is counted in the queue that its element is sorted into, and reported."""
+    wl = several_ctx(n_ctx, np.full(n_ctx, n // n_ctx), S=4, sort=False, mix=True, m=5)
+    wl.pipelines = [util.pipeline(inputs.chain_edges(3), 3, [20, 30, 7], bmax=4)]                 # (three of the row's four stages)
+    wl.requests["stage"] %= 3
+    wl.state.batch[:, 3] = 1
+    n = wl.n
+    good, arrivals = wl.requests.copy(), util.arrivals(np.full(n, 900), 500) if rule == pb.PARD_MODE_CLIPPER else None
+
+    def status(change):
+        wl.requests = good.copy()
+        change(wl.requests)
+        return run_library(wl, rule, check=False, arrivals=arrivals)[0]
+
+    def put(field, at, value):
+        def change(r):
+            r[field][at] = value
+        return change
+
+    for at in (0, n // 2, n - 1, slice(100, n, 301)):
+        for field, value in (("stage", 4), ("ctx", n_ctx), ("deadline_us", -5), ("deadline_us", 1 << 60)):
+            assert status(put(field, at, value)) == pb.PARD_EDATA, (field, at)
+    for ctx in (0, n_ctx // 2, n_ctx - 1):                 # a queue of a stage that the pipeline lacks; the last one is the last of all
+        assert status(put("stage", int(np.flatnonzero(good["ctx"] == ctx)[5]), 3)) == pb.PARD_EDATA, ctx
+    if n < 100_000:                                        # a wait between tiles runs out
+        wl.requests = good
+        assert run_library(wl, rule | pb.PARD_MODE_TEST_STALL, check=False, arrivals=arrivals)[0] == pb.PARD_ETIMEOUT
+    wl.requests = good
+    want = oracle.plan(wl.pipelines, good, wl.state, n_ctx, rule, arrivals)
+    rc, got = run_library(wl, rule, arrivals=arrivals)     # the context still works afterwards
+    assert rc == 0
+    assert_identical(got, want)
+
+
 @pytest.mark.parametrize("rule", [FCFS, NEXUS])
 @pytest.mark.parametrize("n", [2_727_936, 2_727_937])      # the last size of the small tiles, the first of the wide ones
 def test_arrival_order_from_the_requests_tiles(rule, n):
