@@ -18,8 +18,8 @@
  * Queues with more windows than the block's tables hold are decided by the segmented prefix-min
  * scan over the elements instead.
  * Bound by instructions (half of the issue slots, integer ones at half rate) and the chain of steps between barriers, two
- * blocks per multiprocessor covering for each other: of 303 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the
- * copy bandwidth) 86 go to the requests, 74 to the counting sort, 30 to the tables, 90 to the outputs and 20 to the
+ * blocks per multiprocessor covering for each other: of 297 us for 4,096 contexts of 8,192 requests (1.0 GB: 155 us at the
+ * copy bandwidth) 86 go to the requests, 74 to the counting sort, 30 to the tables, 87 to the outputs and 20 to the
  * survivors.  Every request's window and position on its own, 32 in a row to a warp: 345; two segmented scans instead of
  * tables took 762, three radix passes without a look at the order 865. */
 #include <cstddef>
@@ -438,7 +438,7 @@ __device__ __forceinline__ bool split_fits(const LocalArgs& a, const LocalSmem& 
  * admitted position rises by one per request up to u, c = min(r + q, u) with q = min(E, 1) - 1 (at the window's first
  * request too: E is at most the u before less the requests ahead), so its survivors are the window's first ones and a
  * group's estimates are at most two when a batch round takes eight, for raw positions (c = r) too.  (Every request on its
- * own, 32 in a row to a warp: 218 instructions per request for 4,096 contexts of 8,192, 175 like this with the sort below;
+ * own, 32 in a row to a warp: 218 instructions per request for 4,096 contexts of 8,192, 172 like this with the sort below;
  * calls 362 -> 321 us, raw positions 360 -> 318, rounds of one request 385 -> 334.)
  * The tables' P begin as zeros, written by all threads: a queue whose first request lies many windows on, as after a
  * pause or with rounds of a few requests, has its first windows done.  (By the thread of that request, eight comparisons

@@ -751,7 +751,7 @@ k_pack(const uint4* __restrict__ req, uint32_t n, uint32_t n_ctx, uint32_t S,
   __shared__ long long s_A[WIN ? kHistSegs : 1], s_d[WIN ? kHistSegs : 1];
   __shared__ unsigned long long s_magic[WIN ? kHistSegs : 1];
   __shared__ uint4 s_wcon[WIN ? kHistSegs : 1];            /* per queue: A_rel, first table entry, entries, A_rel and d fit 32 bits */
-  /* Few contexts: the low words of their smallest deadlines in shared memory (a replay's epochs, 16 contexts, 455 -> 451 us.
+  /* Few contexts: the low words of their smallest deadlines in shared memory (a replay's epochs, 16 contexts, 451.6 -> 449.7 us.
    * 512 contexts with priorities, all in such tables: the kernel 20.7 -> 24.9). */
   __shared__ uint32_t s_low[kPackCtx];
   const bool table = n_ctx > 1 && n_ctx <= kPackCtx;
@@ -1619,8 +1619,8 @@ k_sort_pass(uint32_t pass, PlanHeader* hdr, unsigned long long* __restrict__ buf
 /* The one pass of a call in arrival order with up to 256 queues, from the requests: their elements need not be written
  * and read back first, and for the rules that compare the deadline alone (rp.rounds) the pass leaves what the walk and
  * the outputs want, the index and the rounds, 8 bytes per request.  2^24 requests of 16 queues under the window scan:
- * k_pack, the pass and k_policy_terms took 57 + 81 + 57 us, this takes 122 (470 MB: 72 by bytes), the call 402 -> 309.
- * Bound by instructions (half of the issue slots, 150 per 32 requests) and by the pass's shared-memory atomics.
+ * k_pack, the pass and k_policy_terms took 57 + 81 + 57 us, this takes 122 (403 MB: 62 by bytes), the call 402 -> 309.
+ * Bound by instructions (half of the issue slots, 140 per 32 requests) and by the pass's shared-memory atomics.
  * Requests are loaded four at a time, ahead of any use: one by one 201 us. */
 template <bool SMALL>
 __global__ void __launch_bounds__(kSortThreads, 2)

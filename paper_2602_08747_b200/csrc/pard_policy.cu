@@ -744,7 +744,7 @@ k_policy_emit(const __grid_constant__ PolicyArgs a) {
     l2_ahead(v.src, INDEX ? tile0 / 2 : tile0, (uint64_t)kDecAhead * kPolTile / (INDEX ? 2 : 1), INDEX ? kPolTile / 2 : kPolTile, INDEX ? a.n / 2 : a.n);
   /* Path sums worked out on the spot: 32 requests in a row to a warp for that, which mostly are of one queue or two.  (Only a
    * tile's first queues are staged; eight in a row per thread leave all others to the last warps: a million requests in
-   * queues of 30 296 -> 314 us for the call.) */
+   * queues of 30 290 -> 326 us for the call.) */
   __shared__ long long s_paths[MASK == kMaskStaged ? kPolTile : 1];
   if (MASK == kMaskStaged) {
     stage_paths(a, v, tile0, sp);

@@ -12,7 +12,7 @@
  * at 68 %): of some 35 instructions per draw two thirds are splitmix64.  M = 10,000 on the
  * 4,500 slots of 256 pipelines (262 M draws): 635 us with a block of its own for every slot of the
  * stride -- most of them padding, each paying five dependent loads to find its path --, the sums
- * in shared memory and four rounds of selection over all of them; 437 us like this. */
+ * in shared memory and four rounds of selection over all of them; 430 us like this. */
 #include <algorithm>
 #include <mutex>
 
@@ -135,7 +135,7 @@ k_estimate_w(const __grid_constant__ PipeTable pipes, const WaitArgs a) {
     const unsigned long long x0 = a.seed + 0x9E3779B97F4A7C15ull + ((unsigned long long)c * a.R + slot) * M * 64ull;
     const bool same_hi = (uint32_t)x0 <= ~0u - (THREADS * PER + 1u) * 64u;       /* uniform */
     /* nearly always the two top bits of the low words are the same too, all that the first shift takes from them: one shift
-     * per stage instead of one per draw (4,500 slots 450.5 -> 445.8 us) */
+     * per stage instead of one per draw (the kernel, 4,500 slots: 435.5 -> 429.5 us) */
     const bool same_top = same_hi && ((uint32_t)x0 >> 30) == (((uint32_t)x0 + (THREADS * PER + 1u) * 64u) >> 30);
     unsigned long long x = x0 + tid * 64ull;
 #pragma unroll 1
